@@ -272,7 +272,8 @@ lq_status lq_selftest_wait_timeout(int device, void* cuda_stream);
  *   "store_qb"     1: lq_quantize_act also writes the branch activation codes to HBM so that lq_act_export can
  *                  return them (parity tests); 0 (default): they stay on chip
  *   "gemm_ctas"    CTAs of the GEMM kernels; 0 (default) = one per SM
- *   "quant_ctas", "quant_warps"   residency and consumer warps of the quantizer kernel; 0 = chosen by the library
+ *   "quant_warps", "quant_ctas"   how the quantizer kernel is cut: row groups of 8 per tile (at most 8 count) and 128-value
+ *                  stages of K per chunk; 0 = chosen by the library
  *   "overlap"      1 (default): kernels are launched with programmatic stream serialization - a kernel's CTAs may take
  *                  their SMs and set up while the previous kernel on the stream drains, and wait (in the kernel) for
  *                  that kernel's completion before touching global memory; 0: plain launches

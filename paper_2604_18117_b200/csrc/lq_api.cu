@@ -142,9 +142,9 @@ lq_layer* lq_layer_new(const lq_config* cfg) {
   L->has_bias = false;
   L->device = -1;
   L->main_kind = g_lq_main_kind;
-  L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1f = nullptr; L->d_L1h = nullptr; L->d_sL1 = nullptr;
+  L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1c = nullptr; L->d_sL1 = nullptr;
   L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfb = nullptr;
-  L->d_s1b = nullptr; L->d_sfl2 = nullptr;
+  L->d_sfl1 = nullptr; L->d_sfl2 = nullptr;
   return L;
 }
 
@@ -347,19 +347,6 @@ lq_status lq_make_tmap_bytes(CUtensorMap* tm, void* base, uint64_t rows, uint64_
   return r == CUDA_SUCCESS ? LQ_OK : LQ_ERR_CUDA;
 }
 
-lq_status lq_make_tmap_rows16(CUtensorMap* tm, const void* X, uint64_t M, uint64_t K) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return LQ_ERR_CUDA;
-  cuuint64_t dims[2] = {K, M};
-  cuuint64_t strides[1] = {K * 2};
-  cuuint32_t box[2] = {64, 16};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? LQ_OK : LQ_ERR_CUDA;
-}
-
 // ---- device status word ------------------------------------------------------------------
 static int32_t* g_status[64] = {nullptr};
 static std::mutex g_status_mu;
@@ -401,11 +388,11 @@ extern "C" lq_status lq_selftest_wait_timeout(int device, void* stream) {
 static void layer_free_device(lq_layer* L) {
   if (L->device < 0) return;
   cudaSetDevice(L->device);
-  cudaFree(L->d_Wq8); cudaFree(L->d_sw); cudaFree(L->d_L1f); cudaFree(L->d_L1h); cudaFree(L->d_sL1);
+  cudaFree(L->d_Wq8); cudaFree(L->d_sw); cudaFree(L->d_L1c); cudaFree(L->d_sL1);
   cudaFree(L->d_L2c); cudaFree(L->d_sL2); cudaFree(L->d_bias); cudaFree(L->d_sfb);
-  cudaFree(L->d_s1b); cudaFree(L->d_sfl2);
-  L->d_s1b = nullptr; L->d_sfl2 = nullptr;
-  L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1f = nullptr; L->d_L1h = nullptr; L->d_sL1 = nullptr;
+  cudaFree(L->d_sfl1); cudaFree(L->d_sfl2);
+  L->d_sfl1 = nullptr; L->d_sfl2 = nullptr;
+  L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1c = nullptr; L->d_sL1 = nullptr;
   L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfb = nullptr;
   L->device = -1;
 }
@@ -425,7 +412,7 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
   CUDA_OK(cudaSetDevice(device));
   L->device = device;
   L->main_kind = g_lq_main_kind;
-  const int K = L->K, N = L->N, r = L->r, G = L->G, Kpad = L->Kpad, Npad = L->Npad, Gpad = L->Gpad;
+  const int K = L->K, N = L->N, r = L->r, G = L->G, Kpad = L->Kpad, Npad = L->Npad, Gpad = L->Gpad, rn = lq_l1_rows(L);
   lq_status st;
   try {
     std::vector<uint8_t> w8((size_t)Npad * Kpad, lq_encode_code_host(0, L->main_kind));
@@ -455,43 +442,38 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
     std::vector<float> s1(LQ_MAX_RANK, 1.f), s2((size_t)Npad, 1.f);
     std::vector<uint8_t> l2c((size_t)Npad * LQ_RCONT, 0);
     if (L->integer_branch) {
-      // B fragments of mma.sync.m16n8k32 (s8) under the k order the quantizer's lanes hold their codes in: per box of
-      // 64 values and 8-column tile, lane 4 c + t carries k = 64 box + 16 t + 0..15 of column 8 tile + c
-      const int ntiles = lq_quant_rank_tiles(r, false), nbox = Kpad / 64;
-      std::vector<uint8_t> l1f((size_t)nbox * ntiles * 32 * 16, 0);
-      for (int b = 0; b < nbox; ++b)
-        for (int nt = 0; nt < ntiles; ++nt)
-          for (int lane = 0; lane < 32; ++lane) {
-            const int j = nt * 8 + (lane >> 2), kb = b * 64 + (lane & 3) * 16;
-            uint8_t* dst = &l1f[(((size_t)b * ntiles + nt) * 32 + lane) * 16];
-            for (int i = 0; i < 16; ++i) dst[i] = (j < r && kb + i < K) ? (uint8_t)L->L1q[(size_t)(kb + i) * r + j] : 0;
-          }
-      if ((st = upload(&L->d_L1f, l1f)) != LQ_OK) return st;
+      std::vector<uint8_t> l1c((size_t)rn * Kpad, 0);
+      for (int k = 0; k < K; ++k)
+        for (int j = 0; j < r; ++j) l1c[(size_t)j * Kpad + k] = (uint8_t)L->L1q[(size_t)k * r + j];
+      if ((st = upload(&L->d_L1c, l1c)) != LQ_OK) return st;
       for (int j = 0; j < r; ++j) s1[j] = L->sL1[j];
       for (int n = 0; n < N; ++n) s2[n] = L->sL2[n];
       for (int j = 0; j < r; ++j)
         for (int n = 0; n < N; ++n) l2c[(size_t)n * LQ_RCONT + j] = (uint8_t)L->L2q[(size_t)j * N + n];
     } else if ((L->mxfp || L->a8) && r > 0) {
-      // B fragments of mma.sync.m16n8k32 (e4m3) for the MXFP quantizer, whose lanes hold two runs of eight values per
-      // box (one per block of 32): lane 4 c + t carries k = 64 box + 32 j + 8 t + 0..7 of column 8 tile + c, j = 0, 1
-      const int ntiles = lq_quant_rank_tiles(r, false), nbox = Kpad / 64, rpad = ntiles * 8;
-      std::vector<uint8_t> l1f((size_t)nbox * ntiles * 32 * 16, 0);
-      for (int b = 0; b < nbox; ++b)
-        for (int nt = 0; nt < ntiles; ++nt)
-          for (int lane = 0; lane < 32; ++lane) {
-            const int j = nt * 8 + (lane >> 2);
-            uint8_t* dst = &l1f[(((size_t)b * ntiles + nt) * 32 + lane) * 16];
-            for (int blk = 0; blk < 2; ++blk)
-              for (int i = 0; i < 8; ++i) {
-                const int k = b * 64 + 32 * blk + 8 * (lane & 3) + i;
-                dst[8 * blk + i] = (j < r && k < K) ? (L->a8 ? (uint8_t)L->L1q[(size_t)k * r + j] : L->L1e[(size_t)k * r + j]) : 0;
-              }
-          }
-      if ((st = upload(&L->d_L1f, l1f)) != LQ_OK) return st;
-      std::vector<float> s1b((size_t)(Kpad / 32) * rpad, 0.f);
+      // The first factor's elements as E4M3 bytes (8-bit integer codes: a plane of hi digits, then one of lo digits) and its
+      // E8M0 scale bytes along K, one chunk of 128 columns x 4 blocks per stage and plane
+      const int planes = lq_l1_planes(L);
+      const size_t plane = (size_t)rn * Kpad, sf_plane = (size_t)(Kpad / 128) * 512;
+      std::vector<uint8_t> l1c(planes * plane, 0), sfl1(planes * sf_plane, 127);
+      for (int k = 0; k < K; ++k)
+        for (int j = 0; j < r; ++j) {
+          uint8_t* dst = &l1c[(size_t)j * Kpad + k];
+          if (!L->a8) { *dst = L->L1e[(size_t)k * r + j]; continue; }
+          int hi = 0, lo = L->L1q[(size_t)k * r + j];
+          if (planes == 2) { lq_split_digits(lo, &hi, &lo); dst[plane] = lq_digit_e4m3(lo); lo = hi; }
+          *dst = lq_digit_e4m3(lo);
+        }
       for (int b = 0; b < lq_ceil_div(K, 32); ++b)
-        for (int j = 0; j < r; ++j) s1b[(size_t)b * rpad + j] = L->s1b[(size_t)b * r + j];
-      if ((st = upload(&L->d_s1b, s1b)) != LQ_OK) return st;
+        for (int j = 0; j < r; ++j) {
+          int e = 0;
+          pow2_exponent(L->s1b[(size_t)b * r + j], &e);
+          const size_t at = lq_sf_offset(j, b, Kpad);
+          sfl1[at] = (uint8_t)(e + 127 + (planes == 2 ? 4 : 0));
+          if (planes == 2) sfl1[sf_plane + at] = (uint8_t)(e + 127);
+        }
+      if ((st = upload(&L->d_L1c, l1c)) != LQ_OK) return st;
+      if ((st = upload(&L->d_sfl1, sfl1)) != LQ_OK) return st;
       // E8M0 bytes of L2's block scales along the rank, one 128-byte-of-rank stage: [1][Npad/128][512]
       std::vector<uint8_t> sfl2((size_t)(Npad / 128) * 512, 127);
       if (L->a8 && L->cfg.branch == LQ_BRANCH_MXINT4) {
@@ -535,17 +517,11 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
       }
       if ((st = upload(&L->d_sfl2, sfl2)) != LQ_OK) return st;
     } else if (L->f16_branch) {
-      // the same fragment order with 16 halves per lane (mma.sync.m16n8k16, four k steps per box)
-      const int ntiles = lq_quant_rank_tiles(r, true), nbox = Kpad / 64;
-      std::vector<uint16_t> l1t((size_t)nbox * ntiles * 32 * 16, 0);
-      for (int b = 0; b < nbox; ++b)
-        for (int nt = 0; nt < ntiles; ++nt)
-          for (int lane = 0; lane < 32; ++lane) {
-            const int j = nt * 8 + (lane >> 2), kb = b * 64 + (lane & 3) * 16;
-            uint16_t* dst = &l1t[(((size_t)b * ntiles + nt) * 32 + lane) * 16];
-            for (int i = 0; i < 16; ++i) dst[i] = (j < r && kb + i < K) ? L->L1h[(size_t)(kb + i) * r + j] : 0;
-          }
-      if ((st = upload(&L->d_L1h, l1t)) != LQ_OK) return st;
+      std::vector<uint8_t> l1c((size_t)rn * Kpad * 2, 0);
+      uint16_t* h = (uint16_t*)l1c.data();
+      for (int k = 0; k < K; ++k)
+        for (int j = 0; j < r; ++j) h[(size_t)j * Kpad + k] = L->L1h[(size_t)k * r + j];
+      if ((st = upload(&L->d_L1c, l1c)) != LQ_OK) return st;
       uint16_t* c16 = (uint16_t*)l2c.data();
       for (int j = 0; j < r; ++j)
         for (int n = 0; n < N; ++n) c16[(size_t)n * (LQ_RCONT / 2) + j] = L->L2h[(size_t)j * N + n];
@@ -556,6 +532,8 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
   } catch (const std::bad_alloc&) { return LQ_ERR_ALLOC; }
   if ((st = lq_make_tmap_bytes(&L->tmB, L->d_Wq8, Npad, Kpad, LQ_BN)) != LQ_OK) return st;
   if ((st = lq_make_tmap_bytes(&L->tmB2, L->d_Wq8, Npad, Kpad, 2 * LQ_BN)) != LQ_OK) return st;
+  if (r > 0 && (st = lq_make_tmap_bytes(&L->tmL1, L->d_L1c, (uint64_t)rn * lq_l1_planes(L), (uint64_t)Kpad * (L->f16_branch ? 2 : 1),
+                                        (uint32_t)rn)) != LQ_OK) return st;
   if ((st = lq_make_tmap_bytes(&L->tmL2, L->d_L2c, Npad, LQ_RCONT, LQ_BN)) != LQ_OK) return st;
   if (!lq_device_status_ptr(device)) return LQ_ERR_CUDA;
   if ((st = lq_gemm_prepare(device)) != LQ_OK) return st;

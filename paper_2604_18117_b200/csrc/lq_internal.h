@@ -85,19 +85,19 @@ struct lq_layer {
   int main_kind;               // LQ_KIND_*: byte encoding of the 4-bit codes in the MMA operands
   uint8_t* d_Wq8;              // [Npad][Kpad] bytes, K contiguous (B operand, K-major)
   float* d_sw;                 // [Gpad][Npad] fp32 (exact images of the fp16 scales)
-  uint8_t* d_L1f;              // [Kpad/64][r tiles][32 lanes][16 bytes]: first factor in mma.sync B-fragment order (integer
-                               // branches): lane 4 c + t holds k = 64 box + 16 t + 0..15 of column 8 tile + c
-  uint16_t* d_L1h;             // the same order with 16 halves per lane (W16A16)
+  uint8_t* d_L1c;              // [planes * rn][Kpad] bytes (W16A16: [rn][Kpad] halves), K contiguous: first factor as the B operand of
+                               // the down-projection; rn = lq_l1_rows; MXINT8 factors: the hi digits' rows, then the lo digits'
+  uint8_t* d_sfl1;             // MX branches: E8M0 bytes of L1's block scales, [planes][Kpad/128][512] in the tensor-memory layout
   float* d_sL1;                // [LQ_MAX_RANK]
   uint8_t* d_L2c;              // [Npad][LQ_RCONT] bytes: int8 codes (or up to 64 halves) of column n, r contiguous
   float* d_sL2;                // [Npad]  (ones for W16A16)
   float* d_bias;               // [Npad]  (zeros without bias)
-  float* d_s1b;                // mxfp: 2^e1 [Kpad/32][rpad] (zero-padded columns)
   uint8_t* d_sfl2;             // mxfp: E8M0 bytes of L2's block scales, [1][Npad/128][512] in the tensor-memory layout
   uint8_t* d_sfb;              // MXINT4: E8M0 bytes of the weight scales, [Kpad/128][Npad/128][512] in the 32 x 16-byte
                                // layout tensor memory wants (byte 16*(n%32) + 4*((n%128)/32) + block%4)
   CUtensorMap tmB;             // over d_Wq8, box [LQ_BN][128B], 128B swizzle
   CUtensorMap tmB2;            // over d_Wq8, box [2 LQ_BN][128B]: both halves of a 256-column tile in one copy
+  CUtensorMap tmL1;            // over d_L1c, box [rn][128B], 128B swizzle
   CUtensorMap tmL2;            // over d_L2c, box [LQ_BN][128B], 128B swizzle
 };
 
@@ -140,13 +140,13 @@ lq_status lq_gemm_prepare(int device);
 lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_dtype dt, cudaStream_t st);
 lq_status lq_gemm_mx_prepare(int device);
 lq_status lq_launch_wait_probe(int device, cudaStream_t st);   // bounded-wait self-test kernel
-int lq_quant_rank_tiles(int r, bool f16);   // 8-column tiles of the rank the quantizer kernels are built for (2, 4, 8 or 16)
 
-// TMA descriptors (lq_api.cu).  lq_make_tmap_bytes: 2-D byte tensor [rows][row_bytes], box [box_rows][128 bytes],
-// 128-byte swizzle.  lq_make_tmap_rows16: fp16 activations [M][K], box 16 rows x 64 values, 128-byte swizzle,
-// zeros outside the tensor.
+// columns of the down-projection's MMA (the rank rounded up to 16) and digit planes of its first factor
+static inline int lq_l1_rows(const lq_layer* L) { return lq_round_up(L->r > 0 ? L->r : 16, 16); }
+static inline int lq_l1_planes(const lq_layer* L) { return L->a8 && L->cfg.branch == LQ_BRANCH_MXINT8 ? 2 : 1; }
+
+// TMA descriptor (lq_api.cu): 2-D byte tensor [rows][row_bytes], box [box_rows][128 bytes], 128-byte swizzle.
 lq_status lq_make_tmap_bytes(CUtensorMap* tm, void* base, uint64_t rows, uint64_t row_bytes, uint32_t box_rows);
-lq_status lq_make_tmap_rows16(CUtensorMap* tm, const void* X, uint64_t M, uint64_t K);
 
 // byte an MMA operand carries for a 4-bit code q in [-7, 7]
 static inline uint8_t lq_encode_code_host(int q, int kind) {
@@ -158,7 +158,7 @@ static inline uint8_t lq_encode_code_host(int q, int kind) {
 
 extern int g_lq_main_kind;   // option "main_kind"
 extern int g_lq_gemm_ctas;   // option "gemm_ctas" (0 = one per SM)
-extern int g_lq_quant_warps, g_lq_quant_ctas;   // options "quant_warps", "quant_ctas": 0 = chosen by the launcher
+extern int g_lq_quant_warps, g_lq_quant_ctas;   // options "quant_warps", "quant_ctas": the quantizer's row groups per tile and stages per chunk, 0 = chosen by the launcher
 extern int g_lq_overlap;     // option "overlap": launch kernels with programmatic stream serialization
 extern int g_lq_store_qb;    // option "store_qb": also write the branch activation codes to HBM (parity export)
 
@@ -170,13 +170,26 @@ extern int g_lq_store_qb;    // option "store_qb": also write the branch activat
 // quantizer -> GEMM -> next quantizer overlaps its launch gaps and tails.  All kernels here are persistent (the whole
 // grid is resident at once), so a waiting successor never holds an SM that a predecessor CTA still needs.
 template <typename... KArgs, typename... Args>
-static inline cudaError_t lq_launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args&&... args) {
+static inline cudaError_t lq_launch_cluster(void (*kernel)(KArgs...), int grid, int block, int cluster, size_t smem, cudaStream_t st,
+                                            Args&&... args) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)grid); lc.blockDim = dim3((unsigned)block); lc.dynamicSmemBytes = smem; lc.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = at; lc.numAttrs = g_lq_overlap ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (g_lq_overlap) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  lc.attrs = at; lc.numAttrs = (unsigned)n;
   return cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+static inline cudaError_t lq_launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args&&... args) {
+  return lq_launch_cluster(kernel, grid, block, 1, smem, st, std::forward<Args>(args)...);
 }
 #endif

@@ -69,6 +69,7 @@ extern "C" lq_status lq_linear_forward_static(const lq_layer* L, const void* X, 
   lq_act A;
   memset(&A, 0, sizeof(A));
   A.K = L->K; A.N = L->N; A.r = L->r; A.G = L->G; A.Kpad = L->Kpad; A.Gpad = L->Gpad;
+  A.planes = 1; A.tq_stride = LQ_RCONT;
   A.branch = L->cfg.branch; A.M_max = M; A.Mpad = (int)Mpad; A.device = L->device; A.main_kind = L->main_kind; A.M = M;
   A.d_qx8 = base + o_qx;
   A.d_qb = (int8_t*)(base + o_qb);

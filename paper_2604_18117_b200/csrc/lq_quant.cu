@@ -1,32 +1,48 @@
-// Activation side of the layer, ONE kernel and one read of X from HBM (Figure 1; Appendix A.2: both branches
+// Activation side of the layer, ONE kernel and one pass of X over HBM (Figure 1; Appendix A.2: both branches
 // consume quantized X, except the full-precision reference branch of Section 4.2 / Table 2):
-//   a1  4-bit codes + scales per token and group of 64 along K (SINT4, Appendix A.3) or block of 32 (MXINT4)
+//   a1  codes + scales per token and block along K (SINT4: 64, MX formats: 32; Appendix A.3)
 //   a2  per-token codes of the low-rank branch (needs the whole row's maximum first)
-//   a3  down-projection I1 = qb L1q, exact int32, on mma.sync (s8) - or T = X L1 in fp16 x fp16 -> fp32 for the
-//       fp16 reference branch - straight from the registers that hold the freshly made codes
-//   a4  t = fl32(fl32(I1) * fl32(sXb * sL1)), per-token re-quantization of the rank-r row
+//   a3  down-projection I1 = qb L1q on the tensor cores (tcgen05): exact int32 (integer branches), fp16 x fp16 -> fp32
+//       (fp16 reference branch), block-scaled (MX branches: the operand IS the main codes and their scale bytes)
+//   a4  the rank-r row, re-quantized (per token, or per block of 32 along the rank)
 //
-// Shape of the kernel: persistent CTAs walk 16-row tiles.  A tile arrives as TMA boxes of 16 rows x 64 values
-// (128-byte swizzle); W consumer warps each own the boxes g = w, w + W, ... of a tile, and each has a private ring
-// of D shared-memory slots with a full/empty mbarrier pair per slot, fed by one lane of the producer warp (lane w
-// serves warp w: a slot is always filled and drained by the same pair, strictly in order, so a one-bit phase
-// never aliases even though copies complete out of order).  A lane (gid, tig) of a consumer warp
-// holds 16 consecutive values of rows gid and gid + 8 - exactly one operand fragment of the m16 MMA under a
-// k order that A and B share (a sum over k does not care which k sits in which fragment slot), so the branch
-// codes never touch shared memory.  With an integer branch a tile is walked twice (row maxima, then codes);
-// when the ring holds a whole tile the second walk reads the same slots, otherwise the producer streams the
-// tile a second time (served by the L2: DRAM still sees X once).
+// Shape of the kernel (persistent, one CTA per SM, warp-specialised, 20 warps): tiles of TR = 8 RG rows, walked in chunks
+// of TR rows x SX stages of 128 values.
+//   warp 3      TMA producer of X: a box is TR rows x 64 values; a ring of up to twelve chunks is always in flight, across
+//               tiles too
+//   warps 4-19  quantizer: in a chunk each warp has one piece, 8 rows x one stage.  Eight lanes own 64 values of a row, a
+//               16-byte vector each, and every lane has vectors of two rows: a block of 32 is four lanes, its maximum two
+//               shuffles, and loads, stores and shared-memory accesses all move whole rows of a box.  (A first version
+//               loaded X into registers from global memory, half rows per instruction: the tag stage of the L1 was
+//               what bounded it, at 40 lookups a piece, and its unrolled ring cost a microsecond of instruction misses.)
+//               The branch's operand goes to shared memory in the layout the MMA reads (K-major, 128-byte swizzle)
+//   warp 2      owns tensor memory; fetches the first factor's slabs, one per stage, and issues the MMAs of a
+//               chunk once its slabs are complete.  The MMA is 128 rows high; the rows beyond TR read whatever follows in
+//               shared memory and their results are never looked at (rows are independent, and the tensor cores are
+//               idle here otherwise)
+//   warps 0-1   a4: lane = row; the rank-r row is read from tensor memory under the next tile's quantization (two
+//               accumulator sets alternate)
+// An integer branch needs the row's maximum before its first code: the tile is walked twice, the first time for the main
+// codes and the maximum, the second time for the branch codes - from the ring when it holds the whole tile, else
+// streamed again from the L2.
 //
 // Exactness contract: codes and scales equal the definition evaluated in IEEE binary32 with
 // round-to-nearest-even and true division.  The kernel is division free:
 //   scale     fp16(a / 7) == fp16(a * fl32(1/7)) for every finite fp16 a (checked exhaustively on the host),
 //             because a/7 never comes closer than 2^-15 (relative) to an fp16 midpoint.
-//   quotient  x / s from the correctly rounded reciprocal by one FMA correction step, which yields the correctly
-//             rounded binary32 quotient (div_rn_by below); rounding to the nearest even integer by adding
-//             1.5 * 2^23.  MXINT4: 1/s is a power of two, so x * (1/s) is already exact.
+//   SINT4     x and s are 11-bit numbers, so x / s is either exactly k + 1/2 or at least 2^-14 away from it.  The product
+//             x * fl32(1/s) is within 2^-20 of the quotient; adding 192 rounds it to a multiple of 2^-16, which restores
+//             exact ties and moves nothing else across one; a second addition then rounds to the integer, ties to even.
+//   branch    x / sb from the correctly rounded reciprocal by one FMA correction step, which yields the correctly
+//             rounded binary32 quotient; 1.5 * 2^23 rounds it to the nearest even integer.
+//   MX        x * 2^-e is exact, and the fp16 pipe does it two values at a time: one fma with 1.5 * 2^10 rounds x * 2^-e to
+//             the nearest even integer without an intermediate rounding; blocks so small that 2^-e is no fp16 number
+//             are scaled up (exactly) first, a rare branch.  MXFP8e4: products below 2^-14 may lose bits, far below half of e4m3's
+//             smallest step 2^-9.
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lq_device.cuh"
 
@@ -34,11 +50,12 @@ namespace {
 
 using namespace lqdev;
 
-constexpr int TR = 16;                 // rows per tile (one m16 MMA tile)
-constexpr int BOX_K = 64;              // values of K per box: one 128-byte swizzle row
-constexpr int BOX_BYTES = TR * BOX_K * 2;
+constexpr int QWARPS = 16;             // quantizer warps (at most; RG * SX of them have work)
+constexpr int FIRST_QWARP = 4;         // warps 0-1 a4, 2 MMA and first factor, 3 X
+constexpr int NTHREADS = (FIRST_QWARP + QWARPS) * 32;
+constexpr int MAX_SLOTS = 4;           // chunk slots of the branch's operands
+constexpr int MAX_XSLOTS = 12;         // chunk slots of X
 constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer (ties to even)
-constexpr int MAX_CONSUMER_WARPS = 9;
 enum { BR_NONE = 0, BR_INT = 1, BR_F16 = 2, BR_MXFP = 3, BR_MXINT = 4 };
 // MXFP: MXFP8e4 activation codes for an MXFP4 weight; MXINT8: MXINT8 activation codes for an MXINT4 weight, stored as
 // two E4M3 digit planes (code = 16 hi + lo)
@@ -46,75 +63,98 @@ enum { MAIN_SINT4 = 0, MAIN_MXINT4 = 1, MAIN_MXFP = 2, MAIN_MXINT8 = 3 };
 
 struct QuantParams {
   int M, K, Kpad, Mpad;
-  int G;                // scales per row that hold data: ceil(K / 64) (SINT4) or ceil(K / 32) (MXINT4)
-  int nbox;             // Kpad / 64 boxes per tile (trailing ones may be all padding: their codes are zeros)
-  int ntiles;           // ceil(M / 16)
-  int depth;            // D: ring slots per consumer warp
-  int refetch;          // 1: a warp's ring is smaller than its share of a tile, the producer streams every tile twice
+  int G;                // SINT4: groups of 64 that hold data
+  int nst;              // Kpad / 128 stages of K
+  int groups, stages;   // RG row groups of 8 per tile, SX stages of K per chunk
+  int ntiles, nchunks;  // tiles of the launch, chunks of a tile
+  int slots, xslots;    // chunk slots of the branch's operands and of X
+  int refetch;          // integer branch: the X ring is smaller than a tile, which is streamed twice
   uint8_t* qx8;         // [Mpad][Kpad] (MXINT8: [Mpad][2 Kpad], the hi digits' plane then the lo digits')
   float* sx;            // [Gpad][Mpad]
-  uint8_t* sfa;         // MXINT4: E8M0 scale bytes [Mpad/128][Kpad/128][512] (MXINT8: [Mpad/128][2 Kpad/128][512], by plane)
+  uint8_t* sfa;         // MX: E8M0 scale bytes [Mpad/128][Kpad/128][512] (MXINT8: [Mpad/128][2 Kpad/128][512], by plane)
   int8_t* qb;           // [Mpad][Kpad] or null (not stored)
   float* sXb;           // [Mpad]
-  const uint4* L1f;     // first factor in fragment order: [nbox][r tiles][32 lanes] x 16 bytes (int8) or 32 bytes (fp16)
   const float* sL1;     // [LQ_MAX_RANK]
-  const float* s1b;     // MXFP: block scales 2^e of the first factor, [Kpad/32][rpad]
-  uint8_t* sft;         // MXFP: E8M0 bytes of the rank-r intermediate's block scales, [Mpad/128][512]
-  uint8_t* tq;          // [Mpad][LQ_RCONT]
+  const uint8_t* sfl1;  // MX branches: E8M0 bytes of the first factor's block scales, [planes][Kpad/128][512]
+  uint8_t* sft;         // MX branches: E8M0 bytes of the rank-r intermediate's block scales, [Mpad/128][512 or 1024]
+  uint8_t* tq;          // [Mpad][tq_stride]
   float* sT;            // [Mpad]
-  int r, rpad;          // rank, rank rounded up to 8
+  int r, rn;            // rank, rank rounded up to 16 (columns of the MMA)
+  int bplanes;          // MXINT: digit planes of the first factor (2: 8-bit codes, 1: 4-bit codes)
   int tq_stride;        // bytes per row of tq: LQ_RCONT, or 2 LQ_RCONT when each digit plane of the intermediate has a container
+  int nacc;             // accumulators a tile's stages alternate over (floating-point branches: shorter chains of fp32 sums)
+  int tmem_cols;        // power of two
+  int smem;             // dynamic shared memory of the launch
   int act6;             // MXFP: the activations (X and the rank-r intermediate) are MXFP6e2 instead of MXFP8e4
   float qm;             // largest branch activation code
   int32_t* status;
 };
 
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+// Shared memory, from a 1024-byte aligned base; the same arithmetic on the host (size) and in the kernel.  First the X ring;
+// then the slots: a slot holds a
+// chunk: its operand slabs (128 bytes of K wide, a_ps and b_ps of them per stage) and scale bytes.
+struct QuantSmem {
+  int xslot, a_unit, a_ps, b_unit, b_ps;
+  int off_b, off_sfa, off_sfb, slot;            // within a slot
+  int off_slots, off_l1, off_max, off_sb, off_bar, total;
+};
+__host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, int bplanes, int slots, int xslots) {
+  QuantSmem s{};
+  const bool mx = br == BR_MXFP || br == BR_MXINT;
+  s.xslot = tr * 256 * st;                      // st: stages of K per chunk
+  s.a_unit = tr * 128; s.b_unit = rn * 128;
+  s.a_ps = br == BR_NONE ? 0 : (br == BR_F16 || br == BR_MXINT) ? 2 : 1;
+  s.b_ps = br == BR_NONE ? 0 : br == BR_F16 ? 2 : br == BR_MXINT ? bplanes : 1;
+  s.off_b = st * s.a_ps * s.a_unit;
+  s.off_sfa = s.off_b + st * s.b_ps * s.b_unit;
+  s.off_sfb = s.off_sfa + (mx ? st * s.a_ps * 512 : 0);
+  s.slot = s.off_sfb + (mx ? st * s.b_ps * 512 : 0);
+  s.slot = (s.slot + 1023) & ~1023;
+  s.off_slots = xslots * s.xslot;
+  s.off_l1 = s.off_slots + (br == BR_NONE ? 0 : slots) * s.slot;
+  s.off_max = s.off_l1 + LQ_MAX_RANK * 4;       // row maxima of three tiles in rotation, row scales of two
+  s.off_sb = s.off_max + 3 * 64 * 4;
+  s.off_bar = s.off_sb + 2 * 64 * 4;
+  s.total = s.off_bar + 128;
+  // the 128-row MMA reads past the last slab of a shorter tile
+  if (br != BR_NONE && s.total < s.off_l1 + 128 * 128) s.total = s.off_l1 + 128 * 128;
+  return s;
 }
 
-// two floats holding integers in [-7, 7] -> two E4M3 bytes (hi: first operand, lo: second)
+__device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
+__device__ __forceinline__ uint32_t as_u32(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+__device__ __forceinline__ float pow2f_n(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }   // -126 <= e <= 127
+
+// two floats -> two E4M3 bytes (hi: first operand, lo: second)
 __device__ __forceinline__ uint32_t f32x2_to_e4m3x2(float hi, float lo) {
   uint16_t r;
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
   return (uint32_t)r;
 }
-
-__device__ __forceinline__ void mma_s8_16832(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                             uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_e4m3_16832(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                               uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k32.row.col.f32.e4m3.e4m3.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_f16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                              uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+__device__ __forceinline__ uint32_t f16x4_to_e4m3x4(__half2 a, __half2 b) {
+  uint32_t w;
+  asm("{\n\t.reg .b16 lo, hi;\n\tcvt.rn.satfinite.e4m3x2.f16x2 lo, %1;\n\tcvt.rn.satfinite.e4m3x2.f16x2 hi, %2;\n\t"
+      "mov.b32 %0, {lo, hi};\n\t}" : "=r"(w) : "r"(as_u32(a)), "r"(as_u32(b)));
+  return w;
 }
 
-// largest magnitude of 16 halves (two 16-byte vectors), exact in fp16
-__device__ __forceinline__ __half absmax16(const uint4& a, const uint4& b) {
-  const __half2* p = reinterpret_cast<const __half2*>(&a);
-  const __half2* q = reinterpret_cast<const __half2*>(&b);
-  __half2 m = __hmax2(__hmax2(__habs2(p[0]), __habs2(p[1])), __hmax2(__habs2(p[2]), __habs2(p[3])));
-  m = __hmax2(m, __hmax2(__hmax2(__habs2(q[0]), __habs2(q[1])), __hmax2(__habs2(q[2]), __habs2(q[3]))));
-  return __hmax(__low2half(m), __high2half(m));
-}
-
+// largest magnitude of eight halves (one 16-byte vector), exact in fp16
 __device__ __forceinline__ __half absmax8(const uint4& a) {
-  const __half2* p = reinterpret_cast<const __half2*>(&a);
-  const __half2 m = __hmax2(__hmax2(__habs2(p[0]), __habs2(p[1])), __hmax2(__habs2(p[2]), __habs2(p[3])));
+  const __half2 m = __hmax2(__hmax2(__habs2(as_half2(a.x)), __habs2(as_half2(a.y))), __hmax2(__habs2(as_half2(a.z)), __habs2(as_half2(a.w))));
   return __hmax(__low2half(m), __high2half(m));
+}
+
+// 2^-e as an fp16 factor (1 for the all-zero block's -127).  Where that is out of fp16's range - the block's maximum is
+// below 2^-7 or less - the values are scaled up, exactly, and e follows.
+__device__ __forceinline__ __half2 half_scale(uint4& v, int e) {
+  if (e < -15 && e > -127) {
+    const __half2 up = __float2half2_rn(4096.f);
+    for (; e < -15; e += 12) {
+      v.x = as_u32(__hmul2(as_half2(v.x), up)); v.y = as_u32(__hmul2(as_half2(v.y), up));
+      v.z = as_u32(__hmul2(as_half2(v.z), up)); v.w = as_u32(__hmul2(as_half2(v.w), up));
+    }
+  }
+  return __half2half2(__ushort_as_half((unsigned short)((15 - (e == -127 ? 0 : e)) << 10)));
 }
 
 // MXFP8e4 / MXFP6e2 of eight values that share a block (Appendix A.3 "MX Formats"; conversion of the OCP specification
@@ -138,750 +178,692 @@ __device__ __forceinline__ uint32_t f32x2_to_e4m3x2_via_e2m3(float hi, float lo)
 __device__ __forceinline__ uint32_t mxfp_pair(float hi, float lo, bool six) {
   return six ? f32x2_to_e4m3x2_via_e2m3(hi, lo) : f32x2_to_e4m3x2(hi, lo);
 }
-__device__ __forceinline__ uint2 mxfp8_codes8(const uint4& v, int e, bool six = false) {
-  const __half2* h2 = reinterpret_cast<const __half2*>(&v);
-  const float inv = e == -127 ? 0.f : __uint_as_float((uint32_t)(127 - e) << 23);
-  float x[8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 f = __half22float2(h2[i]);
-    x[2 * i] = f.x * inv; x[2 * i + 1] = f.y * inv;
-  }
+__device__ __forceinline__ uint2 mxfp_codes8(uint4 v, int e, bool six) {
   uint2 w;
-  w.x = mxfp_pair(x[1], x[0], six) | (mxfp_pair(x[3], x[2], six) << 16);
-  w.y = mxfp_pair(x[5], x[4], six) | (mxfp_pair(x[7], x[6], six) << 16);
+  if (six) {
+    const float inv = e == -127 ? 0.f : pow2f_n(-e);
+    const float2 a = __half22float2(as_half2(v.x)), b = __half22float2(as_half2(v.y)), c = __half22float2(as_half2(v.z)),
+                 d = __half22float2(as_half2(v.w));
+    w.x = f32x2_to_e4m3x2_via_e2m3(a.y * inv, a.x * inv) | (f32x2_to_e4m3x2_via_e2m3(b.y * inv, b.x * inv) << 16);
+    w.y = f32x2_to_e4m3x2_via_e2m3(c.y * inv, c.x * inv) | (f32x2_to_e4m3x2_via_e2m3(d.y * inv, d.x * inv) << 16);
+    return w;
+  }
+  const __half2 inv = half_scale(v, e);  // e in [-32, 7]
+  auto q = [&](uint32_t h) { return __hmul2(as_half2(h), inv); };
+  w.x = f16x4_to_e4m3x4(q(v.x), q(v.y));
+  w.y = f16x4_to_e4m3x4(q(v.z), q(v.w));
   return w;
 }
-// 2^e as a float (0 for the all-zero block's -127: its codes are zeros anyway)
-__device__ __forceinline__ float pow2f(int e) { return e <= -127 ? 0.f : __uint_as_float((uint32_t)(e + 127) << 23); }
 
-// MXINT8 (Appendix A.3 "MX Formats": signed 8-bit codes, blocks of 32, power-of-two scale): the block's exponent is the
-// smallest e with 127 * 2^e >= a for the block maximum a = 1.f * 2^E: e = E - 6 if 1.f <= 127/64, else E - 5; at
-// least -127, and -127 for an all-zero block.
+// MXINT4 (Appendix A.3): 2^e with e the smallest integer such that 7 * 2^e >= a: a = 1.f * 2^E, e = E - 2 if 1.f <= 1.75
+// else E - 1; -127 for an all-zero block.  Codes rint_even(x / 2^e) as E4M3 bytes.
+__device__ __forceinline__ int mxint4_exponent(float a) {
+  const uint32_t ab = __float_as_uint(a);
+  return a > 0.f ? (int)(ab >> 23) - 127 - (((ab & 0x7FFFFFu) <= 0x600000u) ? 2 : 1) : -127;
+}
+__device__ __forceinline__ uint2 mxint4_codes8(uint4 v, int e) {
+  const __half2 magic = __float2half2_rn(1536.f), inv = half_scale(v, e);   // e in [-26, 14]
+  auto q = [&](uint32_t h) { return __hsub2(__hfma2(as_half2(h), inv, magic), magic); };
+  return make_uint2(f16x4_to_e4m3x4(q(v.x), q(v.y)), f16x4_to_e4m3x4(q(v.z), q(v.w)));
+}
+
+// MXINT8 (signed 8-bit codes, blocks of 32, power-of-two scale): the block's exponent is the smallest e with
+// 127 * 2^e >= a for the block maximum a = 1.f * 2^E: e = E - 6 if 1.f <= 127/64, else E - 5; at least -127, and -127
+// for an all-zero block.
 __device__ __forceinline__ int mxint8_exponent(float a) {
   const uint32_t ab = __float_as_uint(a);
   const int e = (int)(ab >> 23) - 127 - (((ab & 0x7FFFFFu) <= 0x7E0000u) ? 6 : 5);
   return a > 0.f ? max(e, -127) : -127;
 }
-// One value under the block's exponent: the code c = rint_even(x / 2^e) (the division is exact), as the int8 byte the
-// down-projection multiplies and as two digits c = 16 hi + lo, lo in [-8, 7], hi in [-8, 8], both exact E4M3 values.
-struct Code8 { float hi, lo; uint32_t byte; };
-__device__ __forceinline__ Code8 mxint8_code(float x, float inv) {
-  const float t = __fmaf_rn(x, inv, MAGIC);
-  const float c = __fadd_rn(t, -MAGIC);
-  Code8 r;
-  r.byte = __float_as_uint(t) & 0xFFu;                 // the low byte of (c + MAGIC)'s bit pattern is c
-  r.hi = floorf(__fmul_rn(__fadd_rn(c, 8.f), 0.0625f));
-  r.lo = __fmaf_rn(r.hi, -16.f, c);
-  return r;
-}
-// eight values of one block (one 16-byte vector of halves): the E4M3 bytes of the hi and lo digits and the int8 codes
-__device__ __forceinline__ void mxint8_codes8(const uint4& v, int e, uint2& hi, uint2& lo, uint2& s8) {
-  const __half2* h2 = reinterpret_cast<const __half2*>(&v);
-  const float inv = e == -127 ? 0.f : __uint_as_float((uint32_t)(127 - e) << 23);
-  Code8 c[8];
+// The code c = rint_even(x / 2^e) of eight values as two digits, c = 16 hi + lo, lo in [-8, 7], hi in [-8, 8], both exact
+// E4M3 values: hi = rint((c + 1/4) / 16), every step exact in fp16 (|c| <= 127).
+__device__ __forceinline__ void mxint8_codes8(uint4 v, int e, uint2& hi, uint2& lo) {
+  const __half2 inv = half_scale(v, e);  // e in [-30, 10]
+  const __half2 magic = __float2half2_rn(1536.f), sixteenth = __float2half2_rn(0.0625f), bias = __float2half2_rn(0.015625f),
+                m16 = __float2half2_rn(-16.f);
+  __half2 h[4], l[4];
+  const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float2 f = __half22float2(h2[i]);
-    c[2 * i] = mxint8_code(f.x, inv); c[2 * i + 1] = mxint8_code(f.y, inv);
+    const __half2 c = __hsub2(__hfma2(as_half2(x[i]), inv, magic), magic);
+    h[i] = __hsub2(__hadd2(__hfma2(c, sixteenth, bias), magic), magic);
+    l[i] = __hfma2(h[i], m16, c);
   }
-  hi.x = f32x2_to_e4m3x2(c[1].hi, c[0].hi) | (f32x2_to_e4m3x2(c[3].hi, c[2].hi) << 16);
-  hi.y = f32x2_to_e4m3x2(c[5].hi, c[4].hi) | (f32x2_to_e4m3x2(c[7].hi, c[6].hi) << 16);
-  lo.x = f32x2_to_e4m3x2(c[1].lo, c[0].lo) | (f32x2_to_e4m3x2(c[3].lo, c[2].lo) << 16);
-  lo.y = f32x2_to_e4m3x2(c[5].lo, c[4].lo) | (f32x2_to_e4m3x2(c[7].lo, c[6].lo) << 16);
-  s8.x = c[0].byte | (c[1].byte << 8) | (c[2].byte << 16) | (c[3].byte << 24);
-  s8.y = c[4].byte | (c[5].byte << 8) | (c[6].byte << 16) | (c[7].byte << 24);
+  hi = make_uint2(f16x4_to_e4m3x4(h[0], h[1]), f16x4_to_e4m3x4(h[2], h[3]));
+  lo = make_uint2(f16x4_to_e4m3x4(l[0], l[1]), f16x4_to_e4m3x4(l[2], l[3]));
+}
+// One fp32 value (the rank-r intermediate) under its block's exponent, the same digits.
+__device__ __forceinline__ void mxint8_digits(float x, float inv, float& hi, float& lo) {
+  const float c = __fadd_rn(__fmaf_rn(x, inv, MAGIC), -MAGIC);
+  hi = floorf(__fmul_rn(__fadd_rn(c, 8.f), 0.0625f));
+  lo = __fmaf_rn(hi, -16.f, c);
 }
 
-// Correctly rounded quotient a / b in binary32 from the correctly rounded reciprocal y = fl32(1/b), division free:
-// q0 = fl32(a y) is within one ulp of a / b, r = a - b q0 is exact in an FMA, and fl32(q0 + r y) is then the
-// correctly rounded quotient (Markstein's correction step).  Operands here are far from overflow and underflow.
-__device__ __forceinline__ float div_rn_by(float a, float b, float y) {
-  const float q0 = __fmul_rn(a, y);
-  const float r = __fmaf_rn(-q0, b, a);
-  return __fmaf_rn(r, y, q0);
-}
-
-// Scale of one group for a1.  `a` is the maximum magnitude of the whole group (SINT4: 64 values, MXINT4: 32),
-// already reduced over the lanes that share it.
-struct MainScale {
-  float s;       // SINT4: the fp16 scale as a float
-  float inv;     // fl32(1/s) (MXINT4: 2^-e, exact)
-  int e;         // MXINT4: block exponent
-  bool coarse;   // SINT4: subnormal scale, the quotient may exceed 7.5 and has to be clamped
+// SINT4 (Appendix A.3): fp16 scale a / 7 (at least 2^-24), codes rint_even(x / s) clamped to [-7, 7]; only a subnormal
+// scale can leave the quotient above 7.5.
+struct Sint4Scale {
+  float s, inv;
+  bool coarse;
 };
-template <bool MX>
-__device__ __forceinline__ MainScale main_scale(float a) {
-  MainScale m;
-  if constexpr (MX) {
-    // 2^e with e the smallest integer such that 7 * 2^e >= a: a = 1.f * 2^E, e = E - 2 if 1.f <= 1.75 else E - 1
-    const uint32_t ab = __float_as_uint(a);
-    m.e = -127;
-    if (a > 0.f) m.e = (int)(ab >> 23) - 127 - (((ab & 0x7FFFFFu) <= 0x600000u) ? 2 : 1);
-    m.inv = __uint_as_float((uint32_t)(127 - (a > 0.f ? m.e : 0)) << 23);
-    m.s = 0.f;
-    m.coarse = false;
-  } else {
-    __half s16 = __float2half_rn(__fmul_rn(a, 0.142857149243354797f));   // fl32(1/7)
-    const unsigned short sbits = __half_as_ushort(s16);
-    if (sbits == 0) s16 = __ushort_as_half((unsigned short)1);            // floor 2^-24
-    m.s = __half2float(s16);
-    m.inv = __frcp_rn(m.s);
-    m.coarse = sbits < 0x0400;
-    m.e = 0;
-  }
+__device__ __forceinline__ Sint4Scale sint4_scale(float a) {
+  Sint4Scale m;
+  __half s16 = __float2half_rn(__fmul_rn(a, 0.142857149243354797f));   // fl32(1/7)
+  const unsigned short bits = __half_as_ushort(s16);
+  if (bits == 0) s16 = __ushort_as_half((unsigned short)1);             // floor 2^-24
+  m.s = __half2float(s16);
+  m.inv = __frcp_rn(m.s);
+  m.coarse = bits < 0x0400;
   return m;
 }
+__device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
+__device__ __forceinline__ uint2 sint4_codes8(const uint4& v, const Sint4Scale& m) {
+  const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
+  const float2 inv = splat(m.inv), c0 = splat(192.f), c1 = splat(MAGIC - 192.f), c2 = splat(-MAGIC);
+  float2 q[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) q[i] = __fadd2_rn(__fadd2_rn(__ffma2_rn(x[i], inv, c0), c1), c2);
+  if (m.coarse) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q[i] = make_float2(fminf(fmaxf(q[i].x, -7.f), 7.f), fminf(fmaxf(q[i].y, -7.f), 7.f));
+  }
+  return make_uint2(f32x2_to_e4m3x2(q[0].y, q[0].x) | (f32x2_to_e4m3x2(q[1].y, q[1].x) << 16),
+                    f32x2_to_e4m3x2(q[2].y, q[2].x) | (f32x2_to_e4m3x2(q[3].y, q[3].x) << 16));
+}
 
-// a1 and a2 for eight consecutive values of one row (one 16-byte vector of halves).
-//   main    SINT4: the correctly rounded quotient x / s, then round-to-nearest-even by the magic constant - the
-//           definition itself; |x| / s <= 7 (1 + 2^-11) for a normal fp16 scale, so only a subnormal (coarse) scale
-//           needs the clamp.  MXINT4: 1/s is a power of two, x * (1/s) is exact.
-//   branch  int8 codes under the row's scale sb, invb = fl32(1/sb); |x| / sb <= qm (1 + 2^-23), so the rounded quotient
-//           never leaves [-qm, qm].  The low byte of (code + MAGIC)'s bit pattern is the code.
-// Returns the 8 operand bytes of the main codes (E4M3 images) and the 8 branch code bytes.
-template <bool MX, bool BRANCH>
-__device__ __forceinline__ void quant8(const uint4& v, const MainScale& ms, float sb, float invb, uint2& w, uint2& b) {
-  const __half2* h2 = reinterpret_cast<const __half2*>(&v);
-  float x[8], q[8];
+// Branch codes of eight values under the row's scale sb, invb = fl32(1/sb): q0 = fl32(x invb) is within one ulp of x / sb,
+// r = x - sb q0 is exact in an FMA, and fl32(q0 + r invb) is then the correctly rounded quotient (Markstein's correction
+// step); |x| / sb <= qm (1 + 2^-23), so it never leaves [-qm, qm].  The low byte of (code + MAGIC)'s bit pattern is the code.
+__device__ __forceinline__ uint2 branch_codes8(const uint4& v, float sb, float invb) {
+  const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
+  const float2 y = splat(invb), ns = splat(-sb), magic = splat(MAGIC);
+  uint32_t t[8];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float2 f = __half22float2(h2[i]);
-    x[2 * i] = f.x; x[2 * i + 1] = f.y;
+    const float2 q0 = __fmul2_rn(x[i], y);
+    const float2 q1 = __fadd2_rn(__ffma2_rn(__ffma2_rn(q0, ns, x[i]), y, q0), magic);
+    t[2 * i] = __float_as_uint(q1.x); t[2 * i + 1] = __float_as_uint(q1.y);
   }
-  if constexpr (MX) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) q[i] = __fadd_rn(__fmaf_rn(x[i], ms.inv, MAGIC), -MAGIC);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) q[i] = __fadd_rn(__fadd_rn(div_rn_by(x[i], ms.s, ms.inv), MAGIC), -MAGIC);
-    if (ms.coarse) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) q[i] = fminf(fmaxf(q[i], -7.f), 7.f);
-    }
-  }
-  w.x = f32x2_to_e4m3x2(q[1], q[0]) | (f32x2_to_e4m3x2(q[3], q[2]) << 16);
-  w.y = f32x2_to_e4m3x2(q[5], q[4]) | (f32x2_to_e4m3x2(q[7], q[6]) << 16);
-  if constexpr (BRANCH) {
-    uint32_t t[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) t[i] = __float_as_uint(__fadd_rn(div_rn_by(x[i], sb, invb), MAGIC));
-    b.x = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
-    b.y = __byte_perm(__byte_perm(t[4], t[5], 0x0040), __byte_perm(t[6], t[7], 0x0040), 0x5410);
-  }
+  uint2 b;
+  b.x = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
+  b.y = __byte_perm(__byte_perm(t[4], t[5], 0x0040), __byte_perm(t[6], t[7], 0x0040), 0x5410);
+  return b;
 }
 
-// CTA-wide rendezvous of the consumer warps on an mbarrier (count = number of consumer warps), bounded like every wait
-__device__ __forceinline__ bool consumers_sync(uint32_t bar, uint32_t parity, int lane, volatile int* abort_flag,
-                                               int32_t* status) {
-  __syncwarp();
-  if (lane == 0) mbar_arrive(bar);
-  return mbar_wait(bar, parity, abort_flag, status, LQ_STAGE_QUANT);
-}
-
-// Shared memory (dynamic), from a 1024-byte aligned base:
-//   ring      W x D boxes of 2 KB
-//   bars      full[W D], empty[W D], syncA, syncB, syncC
-//   red       BR_INT: int I1[2][16][rpad]; BR_F16: float part[W][16][rpad]
-//   rowmax    int[2][16] (bit patterns of non-negative floats)
-//   abort     int
-// Instances for rank > 32 (NTR >= 8) hold 32 or more accumulator and as many fragment registers per thread: compiled
-// for two CTAs per SM (96 registers) they spill, so they are compiled for one (measured: rank 64 10-33 % faster,
-// rank 128 10-20 %); the launch planner picks the residency from the register count it reads back.
-template <int MAIN, int BR, int NTR>   // NTR: 8-column tiles of the rank (rank <= 8 NTR)
-__global__ void __launch_bounds__((MAX_CONSUMER_WARPS + 1) * 32, NTR >= 8 ? 1 : 2) lq_quant_kernel(const __grid_constant__ CUtensorMap tmX,
-                                                                                 const QuantParams p) {
-  constexpr bool MX = MAIN == MAIN_MXINT4;
-  constexpr bool I8 = MAIN == MAIN_MXINT8;
-  constexpr bool FP = MAIN == MAIN_MXFP || I8;             // lanes hold eight values from each of a box's two blocks
-  constexpr bool FACC = BR == BR_F16 || BR == BR_MXFP || BR == BR_MXINT;     // fp32 partial sums of the down-projection
+template <int MAIN, int BR>
+__global__ void __launch_bounds__(NTHREADS, 1)
+lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmL1, const QuantParams p) {
+  constexpr bool SINT = MAIN == MAIN_SINT4;
+  constexpr bool MXB = BR == BR_MXFP || BR == BR_MXINT;      // the branch multiplies the main codes under their scale bytes
   extern __shared__ uint8_t qsm_raw[];
   const uint32_t base = (smem_u32(qsm_raw) + 1023u) & ~1023u;
   uint8_t* smem = qsm_raw + (base - smem_u32(qsm_raw));
-  const int W = (int)(blockDim.x >> 5) - 1;                 // consumer warps; warp W is the producer
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31;
-  const int gid = lane >> 2, tig = lane & 3;
-  const int nslot = W * p.depth;
-  const uint32_t ring = base;
-  const uint32_t bars = base + (uint32_t)nslot * BOX_BYTES;
-  auto bar_full = [&](int s) { return bars + 8u * (uint32_t)s; };
-  auto bar_empty = [&](int s) { return bars + 8u * (uint32_t)(nslot + s); };
-  const uint32_t bar_sync = bars + 16u * (uint32_t)nslot;   // three rendezvous barriers
-  uint8_t* red_ptr = smem + (size_t)nslot * BOX_BYTES + 16 * (size_t)nslot + 32;
-  int* I1_s = reinterpret_cast<int*>(red_ptr);
-  float* part_s = reinterpret_cast<float*>(red_ptr);
-  const size_t red_bytes = BR == BR_INT ? (size_t)2 * TR * p.rpad * 4 : FACC ? (size_t)W * TR * p.rpad * 4 : 0;
-  int* rowmax_s = reinterpret_cast<int*>(red_ptr + red_bytes);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(rowmax_s + 2 * TR);
+  const int RG = p.groups, spc = p.stages, TR = 8 * RG, nq = RG * spc;       // spc: stages of K per chunk
+  const QuantSmem sm = quant_smem(BR, TR, spc, p.rn, p.bplanes, p.slots, p.xslots);
+  auto bar_afull = [&](int s) { return base + (uint32_t)sm.off_bar + 8u * (uint32_t)s; };
+  auto bar_bfull = [&](int s) { return bar_afull(MAX_SLOTS + s); };
+  auto bar_empty = [&](int s) { return bar_afull(2 * MAX_SLOTS + s); };
+  auto bar_tfull = [&](int b) { return bar_afull(3 * MAX_SLOTS + b); };
+  auto bar_tempty = [&](int b) { return bar_afull(3 * MAX_SLOTS + 2 + b); };
+  const uint32_t bar_sync = bar_afull(3 * MAX_SLOTS + 4);
+  auto bar_xfull = [&](int s) { return bar_afull(3 * MAX_SLOTS + 5 + s); };
+  auto bar_xempty = [&](int s) { return bar_afull(3 * MAX_SLOTS + 5 + MAX_XSLOTS + s); };
+  int* rowmax = reinterpret_cast<int*>(smem + sm.off_max);                   // [3][64] fp16 bit patterns
+  float* row_sb = reinterpret_cast<float*>(smem + sm.off_sb);                // [2][64]
+  float* sl1 = reinterpret_cast<float*>(smem + sm.off_l1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + sm.off_bar + 8 * (3 * MAX_SLOTS + 5 + 2 * MAX_XSLOTS));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < nslot; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-    for (int b = 0; b < 3; ++b) mbar_init(bar_sync + 8u * b, (uint32_t)W);
+    for (int s = 0; s < p.xslots; ++s) { mbar_init(bar_xfull(s), 1); mbar_init(bar_xempty(s), (uint32_t)nq); }
+    if constexpr (BR != BR_NONE) {
+      for (int s = 0; s < p.slots; ++s) { mbar_init(bar_afull(s), (uint32_t)nq); mbar_init(bar_bfull(s), 1); mbar_init(bar_empty(s), 1); }
+      for (int b = 0; b < 2; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), 2); }
+      mbar_init(bar_sync, (uint32_t)nq);
+    }
     *abort_flag = 0;
     mbar_init_fence();
   }
   if constexpr (BR == BR_INT) {
-    for (int i = threadIdx.x; i < 2 * TR * p.rpad; i += blockDim.x) I1_s[i] = 0;
-    if (threadIdx.x < 2 * TR) rowmax_s[threadIdx.x] = 0;
+    if (threadIdx.x < 3 * 64) rowmax[threadIdx.x] = 0;
+    if (threadIdx.x >= 256 && threadIdx.x < 256 + LQ_MAX_RANK) sl1[threadIdx.x - 256] = p.sL1[threadIdx.x - 256];
   }
+  if (BR != BR_NONE && warp == 2) tmem_alloc(smem_u32(tmem_slot), (uint32_t)p.tmem_cols);
+  tc_fence_before();
   __syncthreads();
-  grid_dependency_sync();        // set-up done; from here on X is read and the activation record written
+  tc_fence_after();
+  // The tensor-memory columns are taken before a dependent kernel may start and want them.
+  grid_launch_dependents();
 
-  const int passes = (BR == BR_INT && p.refetch) ? 2 : 1;   // how often the producer streams a tile
-
-  if (warp == W) {
-    // ------------------------------------------------------------------ TMA producer: lane w feeds consumer warp w
-    if (lane < W) {
-      const int s0 = lane * p.depth;
-      int idx = 0;
-      uint32_t phase = 0, issued = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x) {
-        const int m0 = tile * TR;
-        for (int ps = 0; ps < passes && ok; ++ps) {
-          for (int g = lane; g < p.nbox; g += W) {
-            ok = mbar_wait(bar_empty(s0 + idx), phase ^ 1, abort_flag, p.status, LQ_STAGE_PRODUCER);
-            if (!ok) break;
-            mbar_expect_tx(bar_full(s0 + idx), BOX_BYTES);
-            tma_load_2d(ring + (uint32_t)(s0 + idx) * BOX_BYTES, &tmX, g * BOX_K, m0, bar_full(s0 + idx));
-            ++issued;
-            if (++idx == p.depth) { idx = 0; phase ^= 1; }
+  const int qw = warp - FIRST_QWARP;
+  if (warp == 3) {
+    // ------------------------------------------------------------------ TMA producer: X
+    grid_dependency_wait();
+    int xs = 0;
+    uint32_t par = 1, issued = 0;
+    bool ok = true;
+    const int walks = BR == BR_INT && p.refetch ? 2 : 1;
+    for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x)
+      for (int w = 0; w < walks && ok; ++w)
+        for (int c = 0; c < p.nchunks; ++c) {
+          ok = mbar_wait_warp(bar_xempty(xs), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
+          if (!ok) break;
+          if (elect_one()) {
+            const int nb = 2 * min(spc, p.nst - c * spc);
+            mbar_expect_tx(bar_xfull(xs), (uint32_t)(nb * TR * 128));
+            for (int b = 0; b < nb; ++b)
+              tma_load_2d(base + (uint32_t)(xs * sm.xslot + b * TR * 128), &tmX, (2 * c * spc + b) * 128, tile * TR, bar_xfull(xs));
           }
+          __syncwarp();
+          ++issued;
+          if (++xs == p.xslots) { xs = 0; par ^= 1; }
         }
+    if (!ok && lane == 0)      // aborting: the copies in flight get a bounded time to land
+      for (uint32_t i = min(issued, (uint32_t)p.xslots); i > 0; --i) {
+        if (--xs < 0) { xs = p.xslots - 1; par ^= 1; }
+        mbar_settle(bar_xfull(xs), par ^ 1);
       }
-      if (!ok) {
-        // aborting: let the copies already issued land before the CTA's shared memory goes away
-        const uint32_t n = issued < (uint32_t)p.depth ? issued : (uint32_t)p.depth;
-        for (uint32_t i = 0; i < n; ++i) {
-          if (--idx < 0) { idx = p.depth - 1; phase ^= 1; }
-          mbar_settle(bar_full(s0 + idx), phase);
+  } else if (BR != BR_NONE && warp == 2) {
+    // ------------------------------------------------------------------ first factor and MMA issuer
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    const uint32_t shape = idesc_shape(p.rn), tsf = tmem + (uint32_t)(2 * p.nacc * p.rn);
+    const int total = ((p.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * p.nchunks;   // chunks of this CTA
+    // the slabs of chunk number n (chunk `c` of its tile) into their slot: weights, so no earlier kernel is waited for
+    auto fetch_b = [&](int slot, int c) {
+      const int st0 = c * spc, ns = min(spc, p.nst - st0);
+      const uint32_t dst = base + (uint32_t)(sm.off_slots + slot * sm.slot), full = bar_bfull(slot);
+      if (elect_one()) {
+        mbar_expect_tx(full, (uint32_t)(ns * sm.b_ps * (sm.b_unit + (MXB ? 512 : 0))));
+        for (int s = 0; s < ns; ++s)
+          for (int u = 0; u < sm.b_ps; ++u) {
+            const int i = s * sm.b_ps + u;
+            // fp16: a stage's 256 bytes of K in two slabs; digit planes: rn rows further down
+            tma_load_2d(dst + sm.off_b + i * sm.b_unit, &tmL1, BR == BR_F16 ? (2 * (st0 + s) + u) * 128 : (st0 + s) * 128,
+                        BR == BR_F16 ? 0 : u * p.rn, full);
+            if constexpr (MXB) bulk_load(dst + sm.off_sfb + i * 512, p.sfl1 + (size_t)(u * p.nst + st0 + s) * 512, 512, full);
+          }
+      }
+      __syncwarp();
+    };
+    int fetched = 0, fslot = 0, fchunk = 0;
+    uint32_t fpar = 1;
+    bool ok = true;
+    // keeps the slabs of up to slots - 1 chunks ahead of the MMAs in flight; a slot's previous MMAs were issued a chunk ago
+    auto fetch_upto = [&](int n) {
+      for (; ok && fetched < n; ++fetched) {
+        ok = mbar_wait_warp(bar_empty(fslot), fpar, abort_flag, p.status, LQ_STAGE_MMA);
+        if (!ok) break;
+        fetch_b(fslot, fchunk);
+        if (++fslot == p.slots) { fslot = 0; fpar ^= 1; }
+        if (++fchunk == p.nchunks) fchunk = 0;
+      }
+    };
+    fetch_upto(min(p.slots, total));
+    uint32_t tc = 0, par = 0;
+    int slot = 0, done = 0;
+    for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x, ++tc) {
+      const uint32_t set = tmem + (uint32_t)((tc & 1) * p.nacc * p.rn);
+      ok = mbar_wait_warp(bar_tempty(tc & 1), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
+      for (int c = 0; c < p.nchunks && ok; ++c) {
+        const int ns = min(spc, p.nst - c * spc);
+        ok = mbar_wait_warp(bar_bfull(slot), par, abort_flag, p.status, LQ_STAGE_MMA) &&
+             mbar_wait_warp(bar_afull(slot), par, abort_flag, p.status, LQ_STAGE_MMA);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t at = base + (uint32_t)(sm.off_slots + slot * sm.slot);
+        if (elect_one()) {
+          for (int s = 0; s < ns; ++s) {
+            const int gs = c * spc + s;                          // stage of K: the accumulators take turns
+            const uint32_t d = set + (uint32_t)((gs & (p.nacc - 1)) * p.rn), more = gs >= p.nacc;
+            const uint32_t a = at + s * sm.a_ps * sm.a_unit, bw = at + sm.off_b + s * sm.b_ps * sm.b_unit;
+            if constexpr (BR == BR_INT) {
+              const uint64_t ad = make_smem_desc(a), bd = make_smem_desc(bw);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) tc_mma<TC_I8>(d, ad + 2 * j, bd + 2 * j, IDESC_I8 | shape, more | (uint32_t)j);
+            } else if constexpr (BR == BR_F16) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                tc_mma<TC_F16>(d, make_smem_desc(a + (j >> 2) * sm.a_unit) + 2 * (j & 3), make_smem_desc(bw + (j >> 2) * sm.b_unit) + 2 * (j & 3),
+                               IDESC_F16 | shape, more | (uint32_t)j);
+            } else {
+              // scale bytes into tensor memory (one slot: the tensor pipe executes these copies and MMAs in issue order),
+              // then every pair of digit planes
+              const int ap = BR == BR_MXINT ? 2 : 1, bp = BR == BR_MXINT ? p.bplanes : 1;
+              for (int u = 0; u < ap; ++u) tc_cp_sf(tsf + 4 * u, make_smem_desc_plain(at + sm.off_sfa + (s * ap + u) * 512, 16, 128));
+              for (int u = 0; u < bp; ++u) tc_cp_sf(tsf + 8 + 4 * u, make_smem_desc_plain(at + sm.off_sfb + (s * bp + u) * 512, 16, 128));
+              for (int ua = 0; ua < ap; ++ua)
+                for (int ub = 0; ub < bp; ++ub) {
+                  const uint64_t ad = make_smem_desc(a + ua * sm.a_unit), bd = make_smem_desc(bw + ub * sm.b_unit);
+#pragma unroll
+                  for (int j = 0; j < 4; ++j)
+                    tc_mma_mx(d, ad + 2 * j, bd + 2 * j, idesc_mx(p.rn, j), tsf + 4 * ua, tsf + 8 + 4 * ub, more | (uint32_t)(j | ua | ub));
+                }
+            }
+          }
+          tc_commit(bar_empty(slot));
+          if (c + 1 == p.nchunks) tc_commit(bar_tfull(tc & 1));
         }
+        __syncwarp();
+        if (++slot == p.slots) { slot = 0; par ^= 1; }
+        ++done;
+        fetch_upto(min(done + p.slots - 1, total));
       }
     }
-  } else {
-    // ------------------------------------------------------------------ consumers
-    // box sequence of this warp: boxes w, w + W, ... of every pass of every tile, through its own ring
-    const int s0 = warp * p.depth;
-    int idx = 0;
-    uint32_t phase = 0;
-    auto advance = [&]() {
-      if (++idx == p.depth) { idx = 0; phase ^= 1; }
-    };
-    // this lane's two 16-byte chunks of a swizzled 128-byte row; rows gid and gid + 8 share the swizzle phase
-    const uint32_t row_off = (uint32_t)gid * 128u;
-    // (MXFP: one 16-byte chunk from each of the box's two blocks of 32 instead: values 8 tig .. and 32 + 8 tig ..)
-    const uint32_t c0 = (uint32_t)((FP ? tig : 2 * tig) ^ (gid & 7)) << 4, c1 = (uint32_t)((FP ? 4 + tig : 2 * tig + 1) ^ (gid & 7)) << 4;
-    uint32_t sync_par = 0;
-    uint32_t tcount = 0;
-    bool ok = true;
-    for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x, ++tcount) {
-      const int m0 = tile * TR;
-      const int par = (int)(tcount & 1);
-      const int m_lo = m0 + gid, m_hi = m0 + gid + 8;
-      const bool v_lo = m_lo < p.M, v_hi = m_hi < p.M;
-      uint8_t* const qx_lo = p.qx8 + (size_t)m_lo * p.Kpad + 16 * tig;   // this lane's bytes of a row start here
-      uint8_t* const qx_hi = qx_lo + (size_t)8 * p.Kpad;
-      float sb_lo = 1.f, sb_hi = 1.f, invb_lo = 1.f, invb_hi = 1.f;
-      // ---- walk 1 (integer branch only): the rows' maxima
-      if constexpr (BR == BR_INT) {
-        const int idx0 = idx;
-        const uint32_t phase0 = phase;
-        __half2 hm = __float2half2_rn(0.f);                 // (row gid, row gid + 8)
-        for (int g = warp; g < p.nbox; g += W) {
-          ok = mbar_wait(bar_full(s0 + idx), phase, abort_flag, p.status, LQ_STAGE_QUANT);
-          if (!ok) break;
-          const uint8_t* bx = smem + (size_t)(s0 + idx) * BOX_BYTES + row_off;
-          const uint4 l0 = *reinterpret_cast<const uint4*>(bx + c0), l1 = *reinterpret_cast<const uint4*>(bx + c1);
-          const uint4 h0 = *reinterpret_cast<const uint4*>(bx + 1024 + c0), h1 = *reinterpret_cast<const uint4*>(bx + 1024 + c1);
-          hm = __hmax2(hm, __halves2half2(absmax16(l0, l1), absmax16(h0, h1)));
-          if (p.refetch) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_empty(s0 + idx));
-          }
-          advance();
-        }
-        if (!ok) break;
-        if (!p.refetch) { idx = idx0; phase = phase0; }     // the second walk reads the same slots
-        hm = __hmax2(hm, __shfl_xor_sync(0xffffffffu, hm, 1));
-        hm = __hmax2(hm, __shfl_xor_sync(0xffffffffu, hm, 2));
-        if (tig == 0) {
-          atomicMax(&rowmax_s[par * TR + gid], __float_as_int(__low2float(hm)));
-          atomicMax(&rowmax_s[par * TR + gid + 8], __float_as_int(__high2float(hm)));
-        }
-        ok = consumers_sync(bar_sync, sync_par, lane, abort_flag, p.status);
-        if (!ok) break;
-        if (threadIdx.x < TR) rowmax_s[(par ^ 1) * TR + threadIdx.x] = 0;     // the other buffer: next tile's
-        const float rm_lo = __int_as_float(rowmax_s[par * TR + gid]), rm_hi = __int_as_float(rowmax_s[par * TR + gid + 8]);
-        sb_lo = (rm_lo == 0.f) ? 1.0f : __fdiv_rn(rm_lo, p.qm);
-        sb_hi = (rm_hi == 0.f) ? 1.0f : __fdiv_rn(rm_hi, p.qm);
-        invb_lo = __frcp_rn(sb_lo); invb_hi = __frcp_rn(sb_hi);
-        if (warp == 0 && tig == 0) {
-          if (v_lo) p.sXb[m_lo] = sb_lo;
-          if (v_hi) p.sXb[m_hi] = sb_hi;
-        }
+    if (!ok && lane == 0) {    // aborting: the copies in flight get a bounded time to land
+      for (int i = min(fetched, p.slots); i > 0; --i) {
+        if (--fslot < 0) { fslot = p.slots - 1; fpar ^= 1; }
+        mbar_settle(bar_bfull(fslot), fpar ^ 1);
       }
-      // ---- walk 2: codes, scales, down-projection
-      int acci[BR == BR_INT ? NTR : 1][4];
-      float accf[FACC ? NTR : 1][4];
+    }
+  } else if (BR != BR_NONE && warp < 2) {
+    // ------------------------------------------------------------------ a4: lane = row of the tile, straight from tensor memory
+    grid_dependency_wait();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0) + ((uint32_t)(32 * warp) << 16);
+    const int nacc = min(p.nacc, p.nst), row = 32 * warp + lane;
+    uint32_t tc = 0;
+    for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++tc) {
+      const int m = tile * TR + row;
+      const bool valid = row < TR && m < p.M;
+      const uint32_t set = tmem + (uint32_t)((tc & 1) * p.nacc * p.rn);
+      if (!mbar_wait_warp(bar_tfull(tc & 1), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN)) break;
+      tc_fence_after();
+      uint8_t* const tqr = p.tq + (size_t)m * p.tq_stride;
+      if (32 * warp < TR) {
+        // 32 columns of the row from `col` on (zeros beyond the accumulator): the accumulators' sum
+        auto fetch = [&](int col, float (&t)[32]) {
+          const bool wide = col + 16 < p.rn;
+          for (int a = 0; a < nacc; ++a) {
+            uint32_t v[32];
+            tmem_ld_32x16(set + (uint32_t)(a * p.rn + col), reinterpret_cast<uint32_t(&)[16]>(v[0]));
+            if (wide) tmem_ld_32x16(set + (uint32_t)(a * p.rn + col + 16), reinterpret_cast<uint32_t(&)[16]>(v[16]));
+            tmem_ld_wait();
 #pragma unroll
-      for (int a = 0; a < NTR; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          if constexpr (BR == BR_INT) acci[a][b] = 0;
-          if constexpr (FACC) accf[a][b] = 0.f;
-        }
-      {
-        // First-factor fragments (read-only, shared by all CTAs, L2 resident) travel one box ahead of their use: the
-        // load of box g + W is in flight while box g is quantized.  FRAGV: 16-byte vectors per lane and column tile.
-        constexpr int FRAGV = BR == BR_F16 ? 2 : 1;
-        uint4 bfrag[BR == BR_NONE ? 1 : NTR * FRAGV];
-        auto load_frags = [&](int g) {
-          if constexpr (BR != BR_NONE) {
-            const uint4* src = p.L1f + ((size_t)g * NTR * 32 + lane) * FRAGV;
-#pragma unroll
-            for (int i = 0; i < NTR * FRAGV; ++i) bfrag[i] = __ldg(src + (size_t)(i / FRAGV) * 32 * FRAGV + (i % FRAGV));
+            for (int j = 0; j < 32; ++j) {
+              const float x = j >= 16 && !wide ? 0.f : BR == BR_INT ? __int2float_rn((int)v[j]) : __uint_as_float(v[j]);
+              t[j] = a == 0 ? x : t[j] + x;
+            }
           }
         };
-        if (warp < p.nbox) load_frags(warp);
-        for (int g = warp; g < p.nbox; g += W) {
-          ok = mbar_wait(bar_full(s0 + idx), phase, abort_flag, p.status, LQ_STAGE_QUANT);
-          if (!ok) break;
-          const uint8_t* bx = smem + (size_t)(s0 + idx) * BOX_BYTES + row_off;
-          const uint4 l0 = *reinterpret_cast<const uint4*>(bx + c0), l1 = *reinterpret_cast<const uint4*>(bx + c1);
-          const uint4 h0 = *reinterpret_cast<const uint4*>(bx + 1024 + c0), h1 = *reinterpret_cast<const uint4*>(bx + 1024 + c1);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_empty(s0 + idx));   // the values are in registers: the slot may be refilled
-          advance();
-          const size_t koff = (size_t)(g * BOX_K);             // this box's first value of a row
-          if constexpr (FP) {
-            // l0 / h0: eight values of block 2g, l1 / h1: of block 2g + 1; a block's maximum lives in four lanes
-            float a00 = __half2float(absmax8(l0)), a01 = __half2float(absmax8(l1));
-            float a10 = __half2float(absmax8(h0)), a11 = __half2float(absmax8(h1));
-#pragma unroll
-            for (int o = 1; o <= 2; o <<= 1) {
-              a00 = fmaxf(a00, __shfl_xor_sync(0xffffffffu, a00, o)); a01 = fmaxf(a01, __shfl_xor_sync(0xffffffffu, a01, o));
-              a10 = fmaxf(a10, __shfl_xor_sync(0xffffffffu, a10, o)); a11 = fmaxf(a11, __shfl_xor_sync(0xffffffffu, a11, o));
-            }
-            if constexpr (I8) {
-              const int e00 = mxint8_exponent(a00), e01 = mxint8_exponent(a01), e10 = mxint8_exponent(a10), e11 = mxint8_exponent(a11);
-              uint2 h00, h01, h10, h11, d00, d01, d10, d11, s00, s01, s10, s11;   // hi digits, lo digits, int8 codes
-              mxint8_codes8(l0, e00, h00, d00, s00); mxint8_codes8(l1, e01, h01, d01, s01);
-              mxint8_codes8(h0, e10, h10, d10, s10); mxint8_codes8(h1, e11, h11, d11, s11);
-              const size_t xs = (size_t)2 * p.Kpad;                // bytes per row: the hi plane, then the lo plane
-              uint8_t* q_lo = p.qx8 + (size_t)m_lo * xs + koff + 8 * tig;
-              uint8_t* q_hi = q_lo + (size_t)8 * xs;
-              if (v_lo) {
-                *reinterpret_cast<uint2*>(q_lo) = h00; *reinterpret_cast<uint2*>(q_lo + 32) = h01;
-                *reinterpret_cast<uint2*>(q_lo + p.Kpad) = d00; *reinterpret_cast<uint2*>(q_lo + p.Kpad + 32) = d01;
-              }
-              if (v_hi) {
-                *reinterpret_cast<uint2*>(q_hi) = h10; *reinterpret_cast<uint2*>(q_hi + 32) = h11;
-                *reinterpret_cast<uint2*>(q_hi + p.Kpad) = d10; *reinterpret_cast<uint2*>(q_hi + p.Kpad + 32) = d11;
-              }
-              if (tig == 0) {
-                const int kb = 2 * g;                            // blocks kb, kb + 1 share a 4-block scale chunk
-                const size_t ks = (size_t)(p.Kpad >> 7);         // K stages per plane
-                if (kb < p.G) {
-                  if (v_lo) {
-                    uint8_t* sf = p.sfa + ((size_t)(m_lo >> 7) * 2 * ks + (kb >> 2)) * 512 + 16 * (m_lo & 31) + 4 * ((m_lo & 127) >> 5) + (kb & 3);
-                    sf[0] = (uint8_t)(e00 + 4 + 127); sf[ks * 512] = (uint8_t)(e00 + 127);
-                    if (kb + 1 < p.G) { sf[1] = (uint8_t)(e01 + 4 + 127); sf[ks * 512 + 1] = (uint8_t)(e01 + 127); }
-                  }
-                  if (v_hi) {
-                    uint8_t* sf = p.sfa + ((size_t)(m_hi >> 7) * 2 * ks + (kb >> 2)) * 512 + 16 * (m_hi & 31) + 4 * ((m_hi & 127) >> 5) + (kb & 3);
-                    sf[0] = (uint8_t)(e10 + 4 + 127); sf[ks * 512] = (uint8_t)(e10 + 127);
-                    if (kb + 1 < p.G) { sf[1] = (uint8_t)(e11 + 4 + 127); sf[ks * 512 + 1] = (uint8_t)(e11 + 127); }
-                  }
-                }
-              }
-              if constexpr (BR == BR_MXINT) {
-                // a3: per block of 32 one exact integer MMA step on the codes just made, then the block's two power-of-two
-                // scales in fp32 (|partial| <= 32 * 127 * 127 < 2^24: the conversion is exact)
-                const float sa00 = pow2f(e00), sa01 = pow2f(e01), sa10 = pow2f(e10), sa11 = pow2f(e11);
-#pragma unroll
-                for (int nt = 0; nt < NTR; ++nt) {
-                  const float2 sb0 = __ldg(reinterpret_cast<const float2*>(p.s1b + (size_t)(2 * g) * p.rpad + nt * 8 + 2 * tig));
-                  const float2 sb1 = __ldg(reinterpret_cast<const float2*>(p.s1b + (size_t)(2 * g + 1) * p.rpad + nt * 8 + 2 * tig));
-                  int i0[4] = {0, 0, 0, 0}, i1[4] = {0, 0, 0, 0};
-                  mma_s8_16832(i0, s00.x, s10.x, s00.y, s10.y, bfrag[nt].x, bfrag[nt].y);
-                  mma_s8_16832(i1, s01.x, s11.x, s01.y, s11.y, bfrag[nt].z, bfrag[nt].w);
-                  accf[nt][0] = fmaf(__int2float_rn(i0[0]), sa00 * sb0.x, fmaf(__int2float_rn(i1[0]), sa01 * sb1.x, accf[nt][0]));
-                  accf[nt][1] = fmaf(__int2float_rn(i0[1]), sa00 * sb0.y, fmaf(__int2float_rn(i1[1]), sa01 * sb1.y, accf[nt][1]));
-                  accf[nt][2] = fmaf(__int2float_rn(i0[2]), sa10 * sb0.x, fmaf(__int2float_rn(i1[2]), sa11 * sb1.x, accf[nt][2]));
-                  accf[nt][3] = fmaf(__int2float_rn(i0[3]), sa10 * sb0.y, fmaf(__int2float_rn(i1[3]), sa11 * sb1.y, accf[nt][3]));
-                }
-              }
-              if (g + W < p.nbox) load_frags(g + W);
-              continue;
-            }
-            const bool six = p.act6 != 0;
-            const int e00 = mxfp8_exponent(a00, six), e01 = mxfp8_exponent(a01, six), e10 = mxfp8_exponent(a10, six), e11 = mxfp8_exponent(a11, six);
-            const uint2 w00 = mxfp8_codes8(l0, e00, six), w01 = mxfp8_codes8(l1, e01, six);
-            const uint2 w10 = mxfp8_codes8(h0, e10, six), w11 = mxfp8_codes8(h1, e11, six);
-            uint8_t* q_lo = p.qx8 + (size_t)m_lo * p.Kpad + koff + 8 * tig;
-            uint8_t* q_hi = q_lo + (size_t)8 * p.Kpad;
-            if (v_lo) { *reinterpret_cast<uint2*>(q_lo) = w00; *reinterpret_cast<uint2*>(q_lo + 32) = w01; }
-            if (v_hi) { *reinterpret_cast<uint2*>(q_hi) = w10; *reinterpret_cast<uint2*>(q_hi + 32) = w11; }
-            if (tig == 0) {
-              const int kb = 2 * g;                            // blocks kb, kb + 1 share a 4-block scale chunk
-              if (kb < p.G) {
-                if (v_lo) {
-                  uint8_t* sf = p.sfa + ((size_t)(m_lo >> 7) * (p.Kpad >> 7) + (kb >> 2)) * 512 + 16 * (m_lo & 31) + 4 * ((m_lo & 127) >> 5) + (kb & 3);
-                  sf[0] = (uint8_t)(e00 + 127);
-                  if (kb + 1 < p.G) sf[1] = (uint8_t)(e01 + 127);
-                }
-                if (v_hi) {
-                  uint8_t* sf = p.sfa + ((size_t)(m_hi >> 7) * (p.Kpad >> 7) + (kb >> 2)) * 512 + 16 * (m_hi & 31) + 4 * ((m_hi & 127) >> 5) + (kb & 3);
-                  sf[0] = (uint8_t)(e10 + 127);
-                  if (kb + 1 < p.G) sf[1] = (uint8_t)(e11 + 127);
-                }
-              }
-            }
-            if constexpr (BR == BR_MXFP) {
-              // a3: per block of 32 one MMA step on the codes just made (their bytes ARE the A fragments), the block's
-              // two power-of-two scales applied to its partial sums in fp32
-              const float sa00 = pow2f(e00), sa01 = pow2f(e01), sa10 = pow2f(e10), sa11 = pow2f(e11);
-#pragma unroll
-              for (int nt = 0; nt < NTR; ++nt) {
-                const float2 sb0 = __ldg(reinterpret_cast<const float2*>(p.s1b + (size_t)(2 * g) * p.rpad + nt * 8 + 2 * tig));
-                const float2 sb1 = __ldg(reinterpret_cast<const float2*>(p.s1b + (size_t)(2 * g + 1) * p.rpad + nt * 8 + 2 * tig));
-                float f0[4] = {0.f, 0.f, 0.f, 0.f}, f1[4] = {0.f, 0.f, 0.f, 0.f};
-                mma_e4m3_16832(f0, w00.x, w10.x, w00.y, w10.y, bfrag[nt].x, bfrag[nt].y);
-                mma_e4m3_16832(f1, w01.x, w11.x, w01.y, w11.y, bfrag[nt].z, bfrag[nt].w);
-                accf[nt][0] = fmaf(f0[0], sa00 * sb0.x, fmaf(f1[0], sa01 * sb1.x, accf[nt][0]));
-                accf[nt][1] = fmaf(f0[1], sa00 * sb0.y, fmaf(f1[1], sa01 * sb1.y, accf[nt][1]));
-                accf[nt][2] = fmaf(f0[2], sa10 * sb0.x, fmaf(f1[2], sa11 * sb1.x, accf[nt][2]));
-                accf[nt][3] = fmaf(f0[3], sa10 * sb0.y, fmaf(f1[3], sa11 * sb1.y, accf[nt][3]));
-              }
-            }
-            if (g + W < p.nbox) load_frags(g + W);
-            continue;
-          }
-          uint4 w_lo, w_hi, b_lo = make_uint4(0, 0, 0, 0), b_hi = make_uint4(0, 0, 0, 0);
-          // group maxima: 64 values = four lanes (SINT4), 32 values = two lanes (MXINT4)
-          float a_lo = __half2float(absmax16(l0, l1)), a_hi = __half2float(absmax16(h0, h1));
-          a_lo = fmaxf(a_lo, __shfl_xor_sync(0xffffffffu, a_lo, 1));
-          a_hi = fmaxf(a_hi, __shfl_xor_sync(0xffffffffu, a_hi, 1));
-          if constexpr (!MX) {
-            a_lo = fmaxf(a_lo, __shfl_xor_sync(0xffffffffu, a_lo, 2));
-            a_hi = fmaxf(a_hi, __shfl_xor_sync(0xffffffffu, a_hi, 2));
-          }
-          const MainScale ms_lo = main_scale<MX>(a_lo), ms_hi = main_scale<MX>(a_hi);
-          {
-            uint2 w, b;
-            quant8<MX, BR == BR_INT>(l0, ms_lo, sb_lo, invb_lo, w, b);
-            w_lo.x = w.x; w_lo.y = w.y; b_lo.x = b.x; b_lo.y = b.y;
-            quant8<MX, BR == BR_INT>(l1, ms_lo, sb_lo, invb_lo, w, b);
-            w_lo.z = w.x; w_lo.w = w.y; b_lo.z = b.x; b_lo.w = b.y;
-          }
-          {
-            uint2 w, b;
-            quant8<MX, BR == BR_INT>(h0, ms_hi, sb_hi, invb_hi, w, b);
-            w_hi.x = w.x; w_hi.y = w.y; b_hi.x = b.x; b_hi.y = b.y;
-            quant8<MX, BR == BR_INT>(h1, ms_hi, sb_hi, invb_hi, w, b);
-            w_hi.z = w.x; w_hi.w = w.y; b_hi.z = b.x; b_hi.w = b.y;
-          }
-          const float s_lo = ms_lo.s, s_hi = ms_hi.s;
-          const int e_lo = ms_lo.e, e_hi = ms_hi.e;
-          // stores: 16 operand bytes per row and lane (64 contiguous bytes per row and box)
-          if (v_lo) {
-            *reinterpret_cast<uint4*>(qx_lo + koff) = w_lo;
-            if (BR == BR_INT && p.qb != nullptr) *reinterpret_cast<uint4*>(p.qb + (qx_lo - p.qx8) + koff) = b_lo;
-          }
-          if (v_hi) {
-            *reinterpret_cast<uint4*>(qx_hi + koff) = w_hi;
-            if (BR == BR_INT && p.qb != nullptr) *reinterpret_cast<uint4*>(p.qb + (qx_hi - p.qx8) + koff) = b_hi;
-          }
-          if constexpr (MX) {
-            const int kb = 2 * g + (tig >> 1);               // block of 32 along K
-            if ((tig & 1) == 0 && kb < p.G) {
-              if (v_lo)
-                p.sfa[((size_t)(m_lo >> 7) * (p.Kpad >> 7) + (kb >> 2)) * 512 + 16 * (m_lo & 31) + 4 * ((m_lo & 127) >> 5) + (kb & 3)] =
-                    (uint8_t)(e_lo + 127);
-              if (v_hi)
-                p.sfa[((size_t)(m_hi >> 7) * (p.Kpad >> 7) + (kb >> 2)) * 512 + 16 * (m_hi & 31) + 4 * ((m_hi & 127) >> 5) + (kb & 3)] =
-                    (uint8_t)(e_hi + 127);
-            }
-          } else {
-            if (tig == 0 && g < p.G) {
-              if (v_lo) p.sx[(size_t)g * p.Mpad + m_lo] = s_lo;
-              if (v_hi) p.sx[(size_t)g * p.Mpad + m_hi] = s_hi;
-            }
-          }
-          // a3 on the fragments just made: bytes 8j .. 8j+7 of a lane's run feed MMA step j
-          if constexpr (BR == BR_INT) {
-#pragma unroll
-            for (int nt = 0; nt < NTR; ++nt) {
-              mma_s8_16832(acci[nt], b_lo.x, b_hi.x, b_lo.y, b_hi.y, bfrag[nt].x, bfrag[nt].y);
-              mma_s8_16832(acci[nt], b_lo.z, b_hi.z, b_lo.w, b_hi.w, bfrag[nt].z, bfrag[nt].w);
-            }
-          }
-          if constexpr (BR == BR_F16) {
-            // rows beyond M and values beyond K are zeros (TMA fill); fp16 x fp16 -> fp32, four k16 steps per box
-#pragma unroll
-            for (int nt = 0; nt < NTR; ++nt) {
-              const uint4 f0 = bfrag[2 * nt], f1 = bfrag[2 * nt + 1];
-              mma_f16_16816(accf[nt], l0.x, h0.x, l0.y, h0.y, f0.x, f0.y);
-              mma_f16_16816(accf[nt], l0.z, h0.z, l0.w, h0.w, f0.z, f0.w);
-              mma_f16_16816(accf[nt], l1.x, h1.x, l1.y, h1.y, f1.x, f1.y);
-              mma_f16_16816(accf[nt], l1.z, h1.z, l1.w, h1.w, f1.z, f1.w);
-            }
-          }
-          if (g + W < p.nbox) load_frags(g + W);
-        }
-        if (!ok) break;
-      }
-      if constexpr (BR == BR_NONE) continue;
-      // ---- the warps' partial products meet in shared memory
-      if constexpr (BR == BR_INT) {
-        int* I1 = I1_s + par * TR * p.rpad;
-#pragma unroll
-        for (int nt = 0; nt < NTR; ++nt) {
-          const int col = nt * 8 + tig * 2;
-          if (col < p.rpad) {
-            atomicAdd(&I1[gid * p.rpad + col], acci[nt][0]);
-            atomicAdd(&I1[gid * p.rpad + col + 1], acci[nt][1]);
-            atomicAdd(&I1[(gid + 8) * p.rpad + col], acci[nt][2]);
-            atomicAdd(&I1[(gid + 8) * p.rpad + col + 1], acci[nt][3]);
-          }
-        }
-      } else {
-        float* mine = part_s + (size_t)warp * TR * p.rpad;
-#pragma unroll
-        for (int nt = 0; nt < NTR; ++nt) {
-          const int col = nt * 8 + tig * 2;
-          if (col < p.rpad) {
-            *reinterpret_cast<float2*>(&mine[gid * p.rpad + col]) = make_float2(accf[nt][0], accf[nt][1]);
-            *reinterpret_cast<float2*>(&mine[(gid + 8) * p.rpad + col]) = make_float2(accf[nt][2], accf[nt][3]);
-          }
-        }
-      }
-      ok = consumers_sync(bar_sync + 8, sync_par, lane, abort_flag, p.status);
-      if (!ok) break;
-      // ---- a4: the rank-r rows of this tile, one warp per row
-      for (int rl = warp; rl < TR; rl += W) {
-        const int m = m0 + rl;
+        float t[32];
         if constexpr (BR == BR_INT) {
-          int* I1 = I1_s + par * TR * p.rpad + rl * p.rpad;
-          const float rm = __int_as_float(rowmax_s[par * TR + rl]);
-          const float sb = (rm == 0.f) ? 1.0f : __fdiv_rn(rm, p.qm);
-          float t[4], amax = 0.f;
+          const float sr = row_sb[(tc & 1) * 64 + row];
+          auto scaled = [&](int c) {                           // t = fl32(fl32(I1) fl32(sXb sL1))
+            fetch(c, t);
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            const int j = lane + 32 * jj;
-            t[jj] = 0.f;
-            if (j < p.rpad) {
-              const int v = I1[j];
-              I1[j] = 0;                                      // ready for the tile after next
-              if (j < p.r) {
-                t[jj] = __fmul_rn(__int2float_rn(v), __fmul_rn(sb, p.sL1[j]));
-                amax = fmaxf(amax, fabsf(t[jj]));
-              }
-            }
-          }
-          amax = warp_max(amax);
-          if (m < p.M) {
-            const float st = (amax == 0.f) ? 1.0f : __fdiv_rn(amax, p.qm);
-            if (lane == 0) p.sT[m] = st;
+            for (int j = 0; j < 32; ++j) t[j] = valid ? __fmul_rn(t[j], __fmul_rn(sr, sl1[c + j])) : 0.f;   // rows beyond the tile hold anything
+          };
+          float amax = 0.f;
+          for (int c = 0; c < p.rn; c += 32) {
+            scaled(c);
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-              const int j = lane + 32 * jj;
-              if (j < p.r) {
-                float q = rintf(__fdiv_rn(t[jj], st));
-                q = fminf(fmaxf(q, -p.qm), p.qm);
-                p.tq[(size_t)m * LQ_RCONT + j] = (uint8_t)(int8_t)(int)q;
+            for (int j = 0; j < 32; ++j) amax = fmaxf(amax, fabsf(t[j]));
+          }
+          const float st = amax == 0.f ? 1.f : __fdiv_rn(amax, p.qm), y = __frcp_rn(st);
+          const bool plain = st > 1e-27f && st < 1e27f;        // no step of the corrected quotient can leave binary32's normal range
+          if (valid) p.sT[m] = st;
+          for (int c = 0; c < p.rn; c += 32) {                 // whole blocks of 32: zeros where the up-projection's K is padded
+            if (p.rn > 32) scaled(c);
+            uint32_t w[8];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              float q;
+              if (plain) {
+                const float q0 = __fmul_rn(t[j], y);
+                q = __fmaf_rn(__fmaf_rn(-q0, st, t[j]), y, q0);
+              } else {
+                q = __fdiv_rn(t[j], st);
               }
+              const uint32_t code = __float_as_uint(__fadd_rn(fminf(fmaxf(q, -p.qm), p.qm), MAGIC)) & 0xFFu;
+              w[j >> 2] = (j & 3) == 0 ? code : w[j >> 2] | (code << (8 * (j & 3)));
+            }
+            if (valid) {
+              *reinterpret_cast<uint4*>(tqr + c) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(tqr + c + 16) = make_uint4(w[4], w[5], w[6], w[7]);
             }
           }
-        } else if constexpr (BR == BR_MXINT) {
-          // T in fp32 (the warps' partial sums added in warp order), then MXINT8 along the rank: one block of 32 per warp
-          // pass; the two digit planes of the codes share the row's container (hi at byte j, lo at byte 64 + j) and the
-          // scale chunk's four slots are (hi, block 0), (hi, block 1), (lo, block 0), (lo, block 1)
-          if (m < p.M) {
-            for (int c = 0; c * 32 < p.r; ++c) {
-              const int j = c * 32 + lane;
-              float v = 0.f;
-              if (j < p.rpad)
-                for (int w2 = 0; w2 < W; ++w2) v += part_s[((size_t)w2 * TR + rl) * p.rpad + j];
-              if (j >= p.r) v = 0.f;
-              const int e = mxint8_exponent(warp_max(fabsf(v)));
-              const float inv = e == -127 ? 0.f : __uint_as_float((uint32_t)(127 - e) << 23);
-              const Code8 cd = mxint8_code(v, inv);
-              // one container for both planes (rank <= 64): lo digits 64 bytes after the hi digits, scale slots c and
-              // 2 + c of one chunk; a container per plane (rank <= 128): lo digits 128 bytes on, slot c of the next chunk
-              const bool split = p.tq_stride != LQ_RCONT;
-              p.tq[(size_t)m * p.tq_stride + j] = (uint8_t)(f32x2_to_e4m3x2(0.f, cd.hi) & 0xFF);
-              p.tq[(size_t)m * p.tq_stride + (split ? 128 : 64) + j] = (uint8_t)(f32x2_to_e4m3x2(0.f, cd.lo) & 0xFF);
-              if (lane == 0) {
-                uint8_t* sf = p.sft + (size_t)(m >> 7) * (split ? 1024 : 512) + 16 * (m & 31) + 4 * ((m & 127) >> 5);
-                sf[c] = (uint8_t)(e + 4 + 127); sf[(split ? 512 : 2) + c] = (uint8_t)(e + 127);
-              }
-            }
-          }
-        } else if constexpr (BR == BR_MXFP) {
-          // T = deq(Q(X)) deq(Q2(L1)) in fp32 (the warps' partial sums added in warp order), then MXFP8e4 along the rank:
-          // one block of 32 per warp pass, its maximum by a warp reduction
-          if (m < p.M) {
-            for (int c = 0; c * 32 < p.r; ++c) {
-              const int j = c * 32 + lane;
-              float v = 0.f;
-              if (j < p.rpad)
-                for (int w2 = 0; w2 < W; ++w2) v += part_s[((size_t)w2 * TR + rl) * p.rpad + j];
-              if (j >= p.r) v = 0.f;
-              const int e = mxfp8_exponent(warp_max(fabsf(v)), p.act6 != 0);
-              const float inv = e == -127 ? 0.f : __uint_as_float((uint32_t)(127 - e) << 23);
-              p.tq[(size_t)m * LQ_RCONT + j] = (uint8_t)(mxfp_pair(0.f, v * inv, p.act6 != 0) & 0xFF);
-              if (lane == 0) p.sft[(size_t)(m >> 7) * 512 + 16 * (m & 31) + 4 * ((m & 127) >> 5) + c] = (uint8_t)(e + 127);
+        } else if constexpr (BR == BR_F16) {
+          if (valid) p.sT[m] = 1.f;
+          for (int c = 0; c < p.rn; c += 32) {
+            fetch(c, t);
+            uint32_t w[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) w[j] = as_u32(__floats2half2_rn(t[2 * j], t[2 * j + 1]));
+            if (valid) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(tqr + 2 * c + 16 * j) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
             }
           }
         } else {
-          // T = fp16(X L1): the warps' fp32 partial sums are added in warp order (the result does not depend on timing)
-          if (m < p.M) {
-            for (int j = lane; j < p.r; j += 32) {
-              float v = 0.f;
-              for (int w2 = 0; w2 < W; ++w2) v += part_s[((size_t)w2 * TR + rl) * p.rpad + j];
-              reinterpret_cast<__half*>(p.tq + (size_t)m * LQ_RCONT)[j] = __float2half_rn(v);
+          // blocks of 32 along the rank.  MXINT with one container for both planes (rank <= 64): lo digits 64 bytes after the
+          // hi digits, scale slots c and 2 + c of one chunk; a container per plane: 128 bytes on, slot c of the next chunk
+          const bool sep = p.tq_stride != LQ_RCONT;
+          uint8_t* const sf = p.sft + (size_t)(m >> 7) * (BR == BR_MXINT && sep ? 1024 : 512) + 16 * (m & 31) + 4 * ((m & 127) >> 5);
+          for (int b = 0; 32 * b < p.rn; ++b) {
+            fetch(32 * b, t);
+            float amax = 0.f;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) amax = fmaxf(amax, fabsf(t[j]));
+            const int e = BR == BR_MXINT ? mxint8_exponent(amax) : mxfp8_exponent(amax, p.act6 != 0);
+            const float inv = e == -127 ? 0.f : pow2f_n(-e);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              uint32_t w[4], d[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                if constexpr (BR == BR_MXINT) {
+                  float hi[4], lo[4];
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) mxint8_digits(t[16 * h + 4 * j + i], inv, hi[i], lo[i]);
+                  w[j] = f32x2_to_e4m3x2(hi[1], hi[0]) | (f32x2_to_e4m3x2(hi[3], hi[2]) << 16);
+                  d[j] = f32x2_to_e4m3x2(lo[1], lo[0]) | (f32x2_to_e4m3x2(lo[3], lo[2]) << 16);
+                } else {
+                  const bool six = p.act6 != 0;
+                  w[j] = mxfp_pair(t[16 * h + 4 * j + 1] * inv, t[16 * h + 4 * j] * inv, six) | (mxfp_pair(t[16 * h + 4 * j + 3] * inv, t[16 * h + 4 * j + 2] * inv, six) << 16);
+                  d[j] = 0;
+                }
+              }
+              if (valid) {
+                *reinterpret_cast<uint4*>(tqr + 32 * b + 16 * h) = make_uint4(w[0], w[1], w[2], w[3]);
+                if (BR == BR_MXINT) *reinterpret_cast<uint4*>(tqr + (sep ? 128 : 64) + 32 * b + 16 * h) = make_uint4(d[0], d[1], d[2], d[3]);
+              }
             }
-            if (lane == 0) p.sT[m] = 1.0f;
+            if (valid) {
+              sf[b] = (uint8_t)(e + 127 + (BR == BR_MXINT ? 4 : 0));
+              if (BR == BR_MXINT) sf[(sep ? 512 : 2) + b] = (uint8_t)(e + 127);
+            }
           }
         }
       }
-      if constexpr (FACC) {
-        ok = consumers_sync(bar_sync + 16, sync_par, lane, abort_flag, p.status);   // partial sums may be overwritten
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_tempty(tc & 1));
+    }
+  } else if (warp >= FIRST_QWARP && qw < nq) {
+    // ------------------------------------------------------------------ quantizer
+    // This lane: 16-byte vector lc of rows ra and ra + 2 of the tile, of both 64-value boxes of a stage.  The four rows of
+    // one access have both values of bit 2, so that the 64-byte halves they write to an operand slab do not meet in the
+    // same banks.
+    const int rg = qw % RG, sx = qw / RG, lr = lane >> 3, lc = lane & 7;
+    const int ra = 8 * rg + (lr & 1) + 2 * (lr & 2);
+    const uint32_t sw = (uint32_t)(ra & 7), hstep = (uint32_t)(TR * 128);               // from a box to the next
+    const uint32_t xo = base + (uint32_t)(sx * TR * 256 + ra * 128);                    // row ra of this warp's first box
+    const uint32_t xo_a = xo + ((lc ^ sw) << 4), xo_b = xo + 256 + ((lc ^ sw ^ 2) << 4);
+    // this lane's eight codes in an operand slab (rows of 128 bytes, 16-byte pieces exchanged by row mod 8); the second box's
+    // are at the address with bit 6 flipped
+    const uint32_t ao = base + (uint32_t)(sm.off_slots + sx * sm.a_ps * sm.a_unit + ra * 128 + 8 * (lc & 1));
+    const uint32_t ao_a = ao + (((lc >> 1) ^ sw) << 4), ao_b = ao + 256 + (((lc >> 1) ^ sw ^ 2) << 4);
+    const int sr = ra + 2 * (lc & 1);                                                   // lanes 0 and 1 of a row store its scale bytes
+    const uint32_t so = base + (uint32_t)(sm.off_slots + sm.off_sfa + sx * sm.a_ps * 512 + 16 * (sr & 31) + 4 * (sr >> 5));
+    const size_t qs = MAIN == MAIN_MXINT8 ? (size_t)2 * p.Kpad : (size_t)p.Kpad;        // bytes per row of qx8
+    grid_dependency_wait();        // from here on the activation record is written
+    int xs = 0, slot = 0;
+    uint32_t xpar = 0, epar = 1, tc = 0, buf = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x, ++tc) {
+      const int ma = tile * TR + ra, ms = tile * TR + sr;
+      const bool va = ma < p.M, vb = ma + 2 < p.M, vs = lc < 2 && ms < p.M;
+      uint8_t* const qa = p.qx8 + (size_t)ma * qs + sx * 128 + 8 * lc;
+      uint8_t* const sfr = SINT ? nullptr : p.sfa + ((size_t)(ms >> 7) * (qs >> 7) + sx) * 512 + 16 * (ms & 31) + 4 * ((ms & 127) >> 5);
+      float sb_a = 1.f, sb_b = 1.f, inv_a = 1.f, inv_b = 1.f;
+      __half2 hm = __float2half2_rn(0.f);                        // maxima of rows ra, ra + 2
+      // One walk over the tile.  MAINP: main codes and scales; BRP: the branch's operand; FREE: the X slots are handed back.
+      auto walk = [&](auto MAINP, auto BRP, const bool free_x) {
+        for (int c = 0, st = sx; c < p.nchunks; ++c, st += spc) {
+          const bool live = st < p.nst;
+          if (!mbar_wait_warp(bar_xfull(xs), xpar, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
+          uint4 a[2], b[2];
+          if (live) {
+            const uint32_t at = (uint32_t)(xs * sm.xslot);
+            a[0] = lds_v4(xo_a + at); b[0] = lds_v4(xo_b + at);
+            a[1] = lds_v4(xo_a + at + hstep); b[1] = lds_v4(xo_b + at + hstep);
+          }
+          uint2 wa[2], wb[2], da[2], db[2];                      // main codes of the two rows (MXINT8: hi digits; d: lo digits)
+          uint32_t four = 0;                                     // the stage's scale bytes of row sr (lanes 0 and 1 of a row)
+          if constexpr (decltype(MAINP)::value) {
+            if (live) {
+              [[maybe_unused]] uint32_t own = 0;
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                __half2 bm = __halves2half2(absmax8(a[h]), absmax8(b[h]));
+                bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
+                bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
+                if constexpr (SINT) bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 4));
+                if constexpr (BR == BR_INT) hm = __hmax2(hm, bm);
+                const float m0 = __low2float(bm), m1 = __high2float(bm);
+                if constexpr (SINT) {
+                  const Sint4Scale s0 = sint4_scale(m0), s1 = sint4_scale(m1);
+                  wa[h] = sint4_codes8(a[h], s0); wb[h] = sint4_codes8(b[h], s1);
+                  const int g = 2 * st + h;
+                  if (vs && g < p.G) p.sx[(size_t)g * p.Mpad + ms] = lc ? s1.s : s0.s;
+                } else {
+                  int e0, e1;
+                  if constexpr (MAIN == MAIN_MXINT4) {
+                    e0 = mxint4_exponent(m0); e1 = mxint4_exponent(m1);
+                    wa[h] = mxint4_codes8(a[h], e0); wb[h] = mxint4_codes8(b[h], e1);
+                  } else if constexpr (MAIN == MAIN_MXFP) {
+                    const bool six = p.act6 != 0;
+                    e0 = mxfp8_exponent(m0, six); e1 = mxfp8_exponent(m1, six);
+                    wa[h] = mxfp_codes8(a[h], e0, six); wb[h] = mxfp_codes8(b[h], e1, six);
+                  } else {
+                    e0 = mxint8_exponent(m0); e1 = mxint8_exponent(m1);
+                    mxint8_codes8(a[h], e0, wa[h], da[h]); mxint8_codes8(b[h], e1, wb[h], db[h]);
+                  }
+                  own |= ((uint32_t)(e0 + 127) | ((uint32_t)(e1 + 127) << 16)) << (8 * h);
+                }
+              }
+              if constexpr (!SINT) {
+                // a row's four bytes are with two lanes, a block pair apart: lane 0 collects row ra's, lane 1 row ra + 2's
+                const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 4);
+                four = __byte_perm(own, other, lc ? 0x7362 : 0x5140);
+                if (vs) {
+                  uint8_t* sf = sfr + (size_t)c * spc * 512;     // (the hi digits weigh 16 times as much)
+                  *reinterpret_cast<uint32_t*>(sf) = MAIN == MAIN_MXINT8 ? four + 0x04040404u : four;
+                  if (MAIN == MAIN_MXINT8) *reinterpret_cast<uint32_t*>(sf + (size_t)p.nst * 512) = four;
+                }
+              }
+              uint8_t* const q = qa + c * spc * 128;
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                if (va) {
+                  *reinterpret_cast<uint2*>(q + 64 * h) = wa[h];
+                  if (MAIN == MAIN_MXINT8) *reinterpret_cast<uint2*>(q + p.Kpad + 64 * h) = da[h];
+                }
+                if (vb) {
+                  *reinterpret_cast<uint2*>(q + 2 * qs + 64 * h) = wb[h];
+                  if (MAIN == MAIN_MXINT8) *reinterpret_cast<uint2*>(q + 2 * qs + p.Kpad + 64 * h) = db[h];
+                }
+              }
+            }
+          }
+          if constexpr (decltype(BRP)::value) {
+            [[maybe_unused]] uint2 ca[2], cb[2];
+            if constexpr (BR == BR_INT) {
+              if (live) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) { ca[h] = branch_codes8(a[h], sb_a, inv_a); cb[h] = branch_codes8(b[h], sb_b, inv_b); }
+              }
+            }
+            if (!mbar_wait_warp(bar_empty(slot), epar, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
+            const uint32_t at = (uint32_t)(slot * sm.slot);
+            if (live) {
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                if constexpr (BR == BR_INT) {
+                  sts_v2((ao_a + at) ^ (64 * h), ca[h]);
+                  sts_v2((ao_b + at) ^ (64 * h), cb[h]);
+                  if (p.qb != nullptr) {
+                    int8_t* o = p.qb + (qa - p.qx8) + c * spc * 128 + 64 * h;
+                    if (va) *reinterpret_cast<uint2*>(o) = ca[h];
+                    if (vb) *reinterpret_cast<uint2*>(o + 2 * qs) = cb[h];
+                  }
+                } else if constexpr (BR == BR_F16) {             // a slab per box: 64 halves, laid out as in the X ring
+                  sts_v4(xo_a + sm.off_slots + at + h * hstep, a[h]);
+                  sts_v4(xo_b + sm.off_slots + at + h * hstep, b[h]);
+                } else {
+                  sts_v2((ao_a + at) ^ (64 * h), wa[h]);
+                  sts_v2((ao_b + at) ^ (64 * h), wb[h]);
+                  if constexpr (BR == BR_MXINT) {
+                    sts_v2(((ao_a + at) ^ (64 * h)) + sm.a_unit, da[h]);
+                    sts_v2(((ao_b + at) ^ (64 * h)) + sm.a_unit, db[h]);
+                  }
+                }
+              }
+              if (MXB && lc < 2) {
+                sts_u32(so + at, BR == BR_MXINT ? four + 0x04040404u : four);
+                if (BR == BR_MXINT) sts_u32(so + at + 512, four);
+              }
+            }
+            fence_proxy_async();
+          }
+          // The X slot goes back only here: by now the stores above have been issued, and they needed every value that was
+          // loaded from it.  (An arrival right after the loads can overtake them: a load may still sit in its queue when the
+          // slot is refilled.)
+          __syncwarp();
+          if (lane == 0) {
+            if (decltype(BRP)::value) mbar_arrive(bar_afull(slot));
+            if (free_x) mbar_arrive(bar_xempty(xs));
+          }
+          if (++xs == p.xslots) { xs = 0; xpar ^= 1; }
+          if (decltype(BRP)::value && ++slot == p.slots) { slot = 0; epar ^= 1; }
+        }
+        return true;
+      };
+      using Yes = std::true_type;
+      using No = std::false_type;
+      if constexpr (BR == BR_INT) {
+        const int xs0 = xs;
+        const uint32_t xpar0 = xpar;
+        ok = walk(Yes(), No(), p.refetch != 0);
         if (!ok) break;
-      }
-      sync_par ^= 1;
-    }
-  }
-}
-
-struct LaunchPlan {
-  int W, depth, refetch, ctas_per_sm;
-  size_t smem;
-};
-
-// Picks the consumer-warp count, ring depth and residency for a row length.  Budget: 227 KB of shared memory and
-// 64 K registers per SM (allocated per warp in units of 8 registers per thread).  Measured on the PixArt shapes
-// (K = 1152, 4608; all branch kinds): two CTAs per SM with eight or nine consumer warps each is the fastest or within
-// a few percent of it, so that is the default; the options "quant_ctas" / "quant_warps" override it for tuning.
-LaunchPlan plan_launch(int nbox, int br, int rpad, int regs) {
-  const size_t SM_SMEM = 227 * 1024;
-  LaunchPlan best{};
-  double best_score = -1.0;
-  for (int ctas = 4; ctas >= 1; --ctas) {
-    if (g_lq_quant_ctas > 0 ? ctas != g_lq_quant_ctas : ctas > 2) continue;
-    for (int W = 4; W <= MAX_CONSUMER_WARPS; ++W) {
-      if (g_lq_quant_warps > 0 ? W != g_lq_quant_warps : W < 8) continue;
-      const int threads = (W + 1) * 32;
-      if (ctas * threads > 2048 || ctas * threads * ((regs + 7) / 8 * 8) > 65536) continue;
-      const size_t red = br == BR_INT ? (size_t)2 * TR * rpad * 4 : (br == BR_F16 || br == BR_MXFP || br == BR_MXINT) ? (size_t)W * TR * rpad * 4 : 0;
-      const size_t fixed = 1024 + 64 + red + 2 * TR * 4 + 64;
-      const size_t budget = std::min(SM_SMEM, SM_SMEM / ctas - 1024);
-      if (budget < fixed + (size_t)W * (BOX_BYTES + 16)) continue;
-      const int per = (nbox + W - 1) / W;                     // boxes of a tile per warp
-      int depth = (int)((budget - fixed) / (BOX_BYTES + 16)) / W;
-      int refetch = 0;
-      if (depth > 2 * per) depth = 2 * per;
-      if (depth < per && br == BR_INT) refetch = 1;
-      // score: resident consumer warps, discounted by the imbalance of boxes over warps; more CTAs and warps win ties
-      const double balance = (double)nbox / (double)(per * W);
-      const double score = ctas * W * balance + 0.01 * ctas + 0.001 * W;
-      if (score > best_score) {
-        best_score = score;
-        best = LaunchPlan{W, depth, refetch, ctas, fixed + (size_t)W * depth * (BOX_BYTES + 16)};
+        if (!p.refetch) { xs = xs0; xpar = xpar0; }              // the second walk reads the same slots
+        // ---- the rows' maxima and scales: non-negative halves order like their bit patterns
+        hm = __hmax2(hm, __shfl_xor_sync(0xffffffffu, hm, 4));
+        int* mx = rowmax + buf * 64;
+        if (lc < 2) atomicMax(&mx[sr], (int)__half_as_ushort(lc ? __high2half(hm) : __low2half(hm)));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_sync);
+        ok = mbar_wait_warp(bar_sync, tc & 1, abort_flag, p.status, LQ_STAGE_QUANT);
+        if (!ok) break;
+        const float rm_a = __half2float(__ushort_as_half((unsigned short)mx[ra]));
+        const float rm_b = __half2float(__ushort_as_half((unsigned short)mx[ra + 2]));
+        const uint32_t after = buf == 0 ? 2 : buf - 1;           // two tiles on: every warp is past its last use
+        if (sx == 0 && lc < 2) rowmax[after * 64 + sr] = 0;
+        buf = buf == 2 ? 0 : buf + 1;
+        sb_a = rm_a == 0.f ? 1.f : __fdiv_rn(rm_a, p.qm);
+        sb_b = rm_b == 0.f ? 1.f : __fdiv_rn(rm_b, p.qm);
+        inv_a = __frcp_rn(sb_a); inv_b = __frcp_rn(sb_b);
+        if (sx == 0) {                                           // a4 reads the scale: its previous tile of this parity must be done
+          ok = mbar_wait_warp(bar_tempty(tc & 1), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_QUANT);
+          if (!ok) break;
+          if (lc < 2) row_sb[(tc & 1) * 64 + sr] = lc ? sb_b : sb_a;
+          if (vs) p.sXb[ms] = lc ? sb_b : sb_a;
+        }
+        ok = walk(No(), Yes(), true);
+      } else {
+        ok = walk(Yes(), std::integral_constant<bool, BR != BR_NONE>(), true);
       }
     }
   }
-  return best;
+
+  tc_fence_before();
+  __syncthreads();
+  if (BR != BR_NONE && warp == 2) {
+    tc_fence_after();
+    tmem_dealloc(__shfl_sync(0xffffffffu, *tmem_slot, 0), (uint32_t)p.tmem_cols);
+  }
 }
 
-template <int MAIN, int BR, int NTR>
-cudaError_t launch_quant(const CUtensorMap& tm, QuantParams& p, int sms, cudaStream_t st) {
+// How a launch is cut.  Cost model in chunk times of a full complement of warps: a CTA's tiles times (its chunks, twice
+// where a tile is walked twice, plus what starting and finishing a tile costs); among equals the higher tile, which reads
+// the first factor less often.
+bool plan_cut(int br, QuantParams& p, int sms) {
+  const int walks = br == BR_INT ? 2 : 1, room = 227 * 1024 - 1024;
+  double best = 1e30;
+  QuantParams out = p;
+  for (int groups = 8; groups >= 1; --groups) {
+    if (g_lq_quant_warps > 0 && groups != std::min(8, g_lq_quant_warps)) continue;
+    for (int stages = std::min(QWARPS / groups, p.nst); stages >= 1; --stages) {
+      if (g_lq_quant_ctas > 0 && stages != g_lq_quant_ctas) continue;
+      QuantParams c = p;
+      c.groups = groups; c.stages = stages;
+      c.ntiles = lq_ceil_div(p.M, 8 * groups);
+      c.nchunks = lq_ceil_div(p.nst, stages);
+      c.xslots = 0;
+      // operand slots first, then as many chunks of X as fit; an integer branch would rather hold a whole tile of X
+      const int want = br == BR_INT ? c.nchunks : 4;
+      for (int slots = br == BR_NONE ? 1 : MAX_SLOTS; slots >= (br == BR_NONE ? 1 : 2) && c.xslots < want; --slots) {
+        const QuantSmem s = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, slots, 0);
+        const int fit = std::min(MAX_XSLOTS, (room - s.total) / s.xslot);
+        if (fit > c.xslots && fit >= 2) { c.xslots = fit; c.slots = slots; }
+      }
+      if (c.xslots < 2) continue;
+      c.xslots = std::min(c.xslots, 2 * c.nchunks);
+      c.refetch = br == BR_INT && c.xslots < c.nchunks;
+      c.smem = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, c.slots, c.xslots).total + 1024;
+      const double chunk = 0.4 + 0.6 * groups * stages / QWARPS;
+      const double cost = lq_ceil_div(c.ntiles, sms) * (c.nchunks * walks * chunk + 1.0) + 3.0;
+      if (cost < best) { best = cost; out = c; }
+    }
+  }
+  p = out;
+  return best < 1e30;
+}
+
+template <int MAIN, int BR>
+cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, int sms, cudaStream_t st) {
   static bool attr_set[64] = {false};
-  static int regs[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_set[dev & 63]) {
-    cudaError_t e = cudaFuncSetAttribute(lq_quant_kernel<MAIN, BR, NTR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    const cudaError_t e = cudaFuncSetAttribute(lq_quant_kernel<MAIN, BR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, lq_quant_kernel<MAIN, BR, NTR>)) != cudaSuccess) return e;
-    regs[dev & 63] = fa.numRegs;
     attr_set[dev & 63] = true;
   }
-  const LaunchPlan pl = plan_launch(p.nbox, BR, p.rpad, regs[dev & 63]);
-  if (pl.W == 0) return cudaErrorInvalidConfiguration;
-  p.depth = pl.depth; p.refetch = pl.refetch;
-  int grid = sms * pl.ctas_per_sm;
-  if (grid > p.ntiles) grid = p.ntiles;
-  const cudaError_t e = lq_launch(lq_quant_kernel<MAIN, BR, NTR>, grid, (pl.W + 1) * 32, pl.smem, st, tm, p);
+  if (!plan_cut(BR, p, sms)) return cudaErrorInvalidConfiguration;
+  CUtensorMap tmX;
+  if (lq_make_tmap_bytes(&tmX, const_cast<void*>(X), (uint64_t)p.M, (uint64_t)p.K * 2, (uint32_t)(8 * p.groups)) != LQ_OK)
+    return cudaErrorInvalidValue;
+  const cudaError_t e = lq_launch(lq_quant_kernel<MAIN, BR>, std::min(p.ntiles, sms), NTHREADS, (size_t)p.smem, st, tmX, tm, p);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int MAIN>
-cudaError_t dispatch_quant(int br, int ntr, const CUtensorMap& tm, QuantParams& p, int sms, cudaStream_t st) {
-  if (br == BR_NONE) return launch_quant<MAIN, BR_NONE, 1>(tm, p, sms, st);
-  if constexpr (MAIN == MAIN_MXINT8) {
-    if (ntr <= 2) return launch_quant<MAIN, BR_MXINT, 2>(tm, p, sms, st);
-    if (ntr <= 4) return launch_quant<MAIN, BR_MXINT, 4>(tm, p, sms, st);
-    if (ntr <= 8) return launch_quant<MAIN, BR_MXINT, 8>(tm, p, sms, st);
-    return launch_quant<MAIN, BR_MXINT, 16>(tm, p, sms, st);
-  } else if constexpr (MAIN == MAIN_MXFP) {
-    if (ntr <= 2) return launch_quant<MAIN, BR_MXFP, 2>(tm, p, sms, st);
-    if (ntr <= 4) return launch_quant<MAIN, BR_MXFP, 4>(tm, p, sms, st);
-    if (ntr <= 8) return launch_quant<MAIN, BR_MXFP, 8>(tm, p, sms, st);
-    return launch_quant<MAIN, BR_MXFP, 16>(tm, p, sms, st);
-  } else {
-    if (br == BR_INT) {
-      if (ntr <= 2) return launch_quant<MAIN, BR_INT, 2>(tm, p, sms, st);
-      if (ntr <= 4) return launch_quant<MAIN, BR_INT, 4>(tm, p, sms, st);
-      if (ntr <= 8) return launch_quant<MAIN, BR_INT, 8>(tm, p, sms, st);
-      return launch_quant<MAIN, BR_INT, 16>(tm, p, sms, st);
-    }
-    if (ntr <= 2) return launch_quant<MAIN, BR_F16, 2>(tm, p, sms, st);
-    if (ntr <= 4) return launch_quant<MAIN, BR_F16, 4>(tm, p, sms, st);
-    return launch_quant<MAIN, BR_F16, 8>(tm, p, sms, st);
-  }
-}
-
 }  // namespace
-
-// rank rounded up to the kernels' instantiated widths (8-column tiles: 2, 4, 8, 16)
-int lq_quant_rank_tiles(int r, bool f16) {
-  const int nt = lq_ceil_div(r > 0 ? r : 8, 8);
-  return nt <= 2 ? 2 : nt <= 4 ? 4 : (nt <= 8 || f16) ? 8 : 16;
-}
 
 lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A, cudaStream_t st) {
   if (cudaSetDevice(A->device) != cudaSuccess) return LQ_ERR_CUDA;
   if (A->main_kind != LQ_KIND_E4M3) return LQ_ERR_UNSUPPORTED;
   const int abits = lq_branch_abits(L->cfg.branch);
-  const int br = L->mxfp ? (L->r > 0 ? BR_MXFP : BR_NONE) : L->a8 ? (L->r > 0 ? BR_MXINT : BR_NONE) : L->f16_branch ? BR_F16 : (L->integer_branch && abits > 0) ? BR_INT : BR_NONE;
-  const int ntr = lq_quant_rank_tiles(L->r, L->f16_branch);
   QuantParams p;
   p.M = M; p.K = L->K; p.Kpad = L->Kpad; p.Mpad = A->Mpad; p.G = L->G;
-  p.nbox = L->Kpad / BOX_K;
-  p.ntiles = lq_ceil_div(M, TR);
+  p.nst = L->Kpad / LQ_KSTAGE;
   p.qx8 = A->d_qx8; p.sx = A->d_sx; p.sfa = A->d_sfa;
   p.qb = g_lq_store_qb ? A->d_qb : nullptr;
-  p.sXb = A->d_sXb;
-  p.L1f = reinterpret_cast<const uint4*>(L->f16_branch ? (const void*)L->d_L1h : (const void*)L->d_L1f);
-  p.sL1 = L->d_sL1; p.tq = A->d_tq; p.sT = A->d_sT;
-  p.s1b = L->d_s1b; p.sft = A->d_sft;
-  p.r = L->r; p.rpad = ntr * 8;
+  p.sXb = A->d_sXb; p.sL1 = L->d_sL1; p.sfl1 = L->d_sfl1;
+  p.sft = A->d_sft; p.tq = A->d_tq; p.sT = A->d_sT;
+  p.r = L->r; p.rn = lq_l1_rows(L);
+  p.bplanes = lq_l1_planes(L);
   p.tq_stride = A->tq_stride;
+  // Floating-point branches: a tile's stages alternate over two to four accumulators, which are added in fp32 at the end;
+  // tensor memory holds two such sets and the scale bytes' columns.
+  p.nacc = L->integer_branch ? 1 : p.rn <= 48 ? 4 : p.rn <= 112 ? 2 : 1;
+  if (L->f16_branch && p.rn > 48) p.nacc = 4;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < 2 * p.nacc * p.rn + ((L->mxfp || L->a8) ? 16 : 0)) p.tmem_cols *= 2;
   p.act6 = (L->mxfp && L->cfg.act_fmt == LQ_ACT_MXFP6) ? 1 : 0;
-  p.qm = br == BR_INT ? (float)((1 << (abits - 1)) - 1) : 0.f;
+  p.qm = abits > 0 ? (float)((1 << (abits - 1)) - 1) : 0.f;
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;
-  CUtensorMap tm;
-  lq_status s = lq_make_tmap_rows16(&tm, X, (uint64_t)M, (uint64_t)L->K);
-  if (s != LQ_OK) return s;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device) != cudaSuccess) return LQ_ERR_CUDA;
-  const cudaError_t e = L->mxfp ? dispatch_quant<MAIN_MXFP>(br, ntr, tm, p, sms, st)
-                        : L->a8 ? dispatch_quant<MAIN_MXINT8>(br, ntr, tm, p, sms, st)
-                        : L->mx ? dispatch_quant<MAIN_MXINT4>(br, ntr, tm, p, sms, st) : dispatch_quant<MAIN_SINT4>(br, ntr, tm, p, sms, st);
+  cudaError_t e;
+  if (L->mxfp) e = L->r > 0 ? launch_quant<MAIN_MXFP, BR_MXFP>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXFP, BR_NONE>(X, L->tmL1, p, sms, st);
+  else if (L->a8) e = L->r > 0 ? launch_quant<MAIN_MXINT8, BR_MXINT>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXINT8, BR_NONE>(X, L->tmL1, p, sms, st);
+  else if (L->mx)
+    e = L->f16_branch ? launch_quant<MAIN_MXINT4, BR_F16>(X, L->tmL1, p, sms, st)
+                      : L->integer_branch ? launch_quant<MAIN_MXINT4, BR_INT>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXINT4, BR_NONE>(X, L->tmL1, p, sms, st);
+  else
+    e = L->f16_branch ? launch_quant<MAIN_SINT4, BR_F16>(X, L->tmL1, p, sms, st)
+                      : L->integer_branch ? launch_quant<MAIN_SINT4, BR_INT>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_SINT4, BR_NONE>(X, L->tmL1, p, sms, st);
   return lq_note_cuda(e) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }
