@@ -452,10 +452,10 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
         for (int n = 0; n < N; ++n) l2c[(size_t)n * LQ_RCONT + j] = (uint8_t)L->L2q[(size_t)j * N + n];
     } else if ((L->mxfp || L->a8) && r > 0) {
       // The first factor's elements as E4M3 bytes (8-bit integer codes: a plane of hi digits, then one of lo digits) and its
-      // E8M0 scale bytes along K, one chunk of 128 columns x 4 blocks per stage and plane
+      // E8M0 scale bytes along K, one chunk of (at most) 128 rows x 4 blocks per stage
       const int planes = lq_l1_planes(L);
-      const size_t plane = (size_t)rn * Kpad, sf_plane = (size_t)(Kpad / 128) * 512;
-      std::vector<uint8_t> l1c(planes * plane, 0), sfl1(planes * sf_plane, 127);
+      const size_t plane = (size_t)rn * Kpad;
+      std::vector<uint8_t> l1c(planes * plane, 0), sfl1((size_t)(Kpad / 128) * 512, 127);
       for (int k = 0; k < K; ++k)
         for (int j = 0; j < r; ++j) {
           uint8_t* dst = &l1c[(size_t)j * Kpad + k];
@@ -468,9 +468,8 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
         for (int j = 0; j < r; ++j) {
           int e = 0;
           pow2_exponent(L->s1b[(size_t)b * r + j], &e);
-          const size_t at = lq_sf_offset(j, b, Kpad);
-          sfl1[at] = (uint8_t)(e + 127 + (planes == 2 ? 4 : 0));
-          if (planes == 2) sfl1[sf_plane + at] = (uint8_t)(e + 127);
+          sfl1[lq_sf_offset(j, b, Kpad)] = (uint8_t)(e + 127 + (planes == 2 ? 4 : 0));
+          if (planes == 2) sfl1[lq_sf_offset(rn + j, b, Kpad)] = (uint8_t)(e + 127);
         }
       if ((st = upload(&L->d_L1c, l1c)) != LQ_OK) return st;
       if ((st = upload(&L->d_sfl1, sfl1)) != LQ_OK) return st;
@@ -533,7 +532,7 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
   if ((st = lq_make_tmap_bytes(&L->tmB, L->d_Wq8, Npad, Kpad, LQ_BN)) != LQ_OK) return st;
   if ((st = lq_make_tmap_bytes(&L->tmB2, L->d_Wq8, Npad, Kpad, 2 * LQ_BN)) != LQ_OK) return st;
   if (r > 0 && (st = lq_make_tmap_bytes(&L->tmL1, L->d_L1c, (uint64_t)rn * lq_l1_planes(L), (uint64_t)Kpad * (L->f16_branch ? 2 : 1),
-                                        (uint32_t)rn)) != LQ_OK) return st;
+                                        (uint32_t)(rn * lq_l1_planes(L)))) != LQ_OK) return st;
   if ((st = lq_make_tmap_bytes(&L->tmL2, L->d_L2c, Npad, LQ_RCONT, LQ_BN)) != LQ_OK) return st;
   if (!lq_device_status_ptr(device)) return LQ_ERR_CUDA;
   if ((st = lq_gemm_prepare(device)) != LQ_OK) return st;

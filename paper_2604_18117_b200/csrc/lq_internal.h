@@ -87,7 +87,7 @@ struct lq_layer {
   float* d_sw;                 // [Gpad][Npad] fp32 (exact images of the fp16 scales)
   uint8_t* d_L1c;              // [planes * rn][Kpad] bytes (W16A16: [rn][Kpad] halves), K contiguous: first factor as the B operand of
                                // the down-projection; rn = lq_l1_rows; MXINT8 factors: the hi digits' rows, then the lo digits'
-  uint8_t* d_sfl1;             // MX branches: E8M0 bytes of L1's block scales, [planes][Kpad/128][512] in the tensor-memory layout
+  uint8_t* d_sfl1;             // MX branches: E8M0 bytes of L1's block scales, [Kpad/128][512] in the tensor-memory layout (row = row of d_L1c)
   float* d_sL1;                // [LQ_MAX_RANK]
   uint8_t* d_L2c;              // [Npad][LQ_RCONT] bytes: int8 codes (or up to 64 halves) of column n, r contiguous
   float* d_sL2;                // [Npad]  (ones for W16A16)
@@ -97,7 +97,7 @@ struct lq_layer {
                                // layout tensor memory wants (byte 16*(n%32) + 4*((n%128)/32) + block%4)
   CUtensorMap tmB;             // over d_Wq8, box [LQ_BN][128B], 128B swizzle
   CUtensorMap tmB2;            // over d_Wq8, box [2 LQ_BN][128B]: both halves of a 256-column tile in one copy
-  CUtensorMap tmL1;            // over d_L1c, box [rn][128B], 128B swizzle
+  CUtensorMap tmL1;            // over d_L1c, box [all rows][128B], 128B swizzle
   CUtensorMap tmL2;            // over d_L2c, box [LQ_BN][128B], 128B swizzle
 };
 

@@ -10,16 +10,19 @@
 // of TR rows x SX stages of 128 values.
 //   warp 3      TMA producer of X: a box is TR rows x 64 values; a ring of up to twelve chunks is always in flight, across
 //               tiles too
-//   warps 4-19  quantizer: in a chunk each warp has one piece, 8 rows x one stage.  Eight lanes own 64 values of a row, a
-//               16-byte vector each, and every lane has vectors of two rows: a block of 32 is four lanes, its maximum two
-//               shuffles, and loads, stores and shared-memory accesses all move whole rows of a box.  (A first version
-//               loaded X into registers from global memory, half rows per instruction: the tag stage of the L1 was
-//               what bounded it, at 40 lookups a piece, and its unrolled ring cost a microsecond of instruction misses.)
-//               The branch's operand goes to shared memory in the layout the MMA reads (K-major, 128-byte swizzle)
-//   warp 2      owns tensor memory; fetches the first factor's slabs, one per stage, and issues the MMAs of a
-//               chunk once its slabs are complete.  The MMA is 128 rows high; the rows beyond TR read whatever follows in
-//               shared memory and their results are never looked at (rows are independent, and the tensor cores are
-//               idle here otherwise)
+//   warps 5-19  quantizer: teams of RG x SX warps take the chunks in turn; in a chunk each warp has one piece, 8 rows x one
+//               stage.  Eight lanes own 64 values of a row, a 16-byte vector each, and every lane has vectors of two rows: a
+//               block of 32 is four lanes, its maximum two shuffles, and loads, stores and shared-memory accesses all move
+//               whole rows of a box.  (A first version loaded X into registers from global memory, half rows per
+//               instruction: the tag stage of the L1 was what bounded it, at 40 lookups a piece, and its unrolled ring
+//               cost a microsecond of instruction misses.)  The branch's operand goes to shared memory in the layout
+//               the MMA reads (K-major, 128-byte swizzle).  More warps (28 at 64 registers) were no faster, twelve were
+//               10-30 % slower
+//   warp 4      TMA producer of the first factor's slabs, one per stage, and their scale bytes.  (The MMA warp fetched them at
+//               first, after the chunk it had just issued: the slabs were late, 24 against 30 us at K = 4608)
+//   warp 2      owns tensor memory, issues the MMAs of a chunk once its slabs are complete.  The MMA is 128 rows high; the rows
+//               beyond TR read whatever follows in shared memory and their results are never looked at (rows are
+//               independent, and the tensor cores are idle here otherwise)
 //   warps 0-1   a4: lane = row; the rank-r row is read from tensor memory under the next tile's quantization (two
 //               accumulator sets alternate)
 // An integer branch needs the row's maximum before its first code: the tile is walked twice, the first time for the main
@@ -31,7 +34,7 @@
 //   scale     fp16(a / 7) == fp16(a * fl32(1/7)) for every finite fp16 a (checked exhaustively on the host),
 //             because a/7 never comes closer than 2^-15 (relative) to an fp16 midpoint.
 //   SINT4     x and s are 11-bit numbers, so x / s is either exactly k + 1/2 or at least 2^-14 away from it.  The product
-//             x * fl32(1/s) is within 2^-20 of the quotient; adding 192 rounds it to a multiple of 2^-16, which restores
+//             with a reciprocal that is an ulp or two off is within 2^-19 of the quotient; adding 192 rounds it to a multiple of 2^-16, which restores
 //             exact ties and moves nothing else across one; a second addition then rounds to the integer, ties to even.
 //   branch    x / sb from the correctly rounded reciprocal by one FMA correction step, which yields the correctly
 //             rounded binary32 quotient; 1.5 * 2^23 rounds it to the nearest even integer.
@@ -50,22 +53,24 @@ namespace {
 
 using namespace lqdev;
 
-constexpr int QWARPS = 16;             // quantizer warps (at most; RG * SX of them have work)
-constexpr int FIRST_QWARP = 4;         // warps 0-1 a4, 2 MMA and first factor, 3 X
+constexpr int QWARPS = 15;             // quantizer warps (at most; teams of RG * SX): 20 warps are the most that leave 96 registers each
+constexpr int FIRST_QWARP = 5;         // warps 0-1 a4, 2 MMA, 3 X, 4 first factor
 constexpr int NTHREADS = (FIRST_QWARP + QWARPS) * 32;
 constexpr int MAX_SLOTS = 4;           // chunk slots of the branch's operands
+constexpr int MAX_UNSETTLED = 32;      // list of a4's rows to look at again, per warp
 constexpr int MAX_XSLOTS = 12;         // chunk slots of X
 constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer (ties to even)
 enum { BR_NONE = 0, BR_INT = 1, BR_F16 = 2, BR_MXFP = 3, BR_MXINT = 4 };
 // MXFP: MXFP8e4 activation codes for an MXFP4 weight; MXINT8: MXINT8 activation codes for an MXINT4 weight, stored as
-// two E4M3 digit planes (code = 16 hi + lo)
-enum { MAIN_SINT4 = 0, MAIN_MXINT4 = 1, MAIN_MXFP = 2, MAIN_MXINT8 = 3 };
+// two E4M3 digit planes (code = 16 hi + lo); MXFP6: MXFP6e2 activation codes, stored as the E4M3 bytes of the same values
+enum { MAIN_SINT4 = 0, MAIN_MXINT4 = 1, MAIN_MXFP = 2, MAIN_MXINT8 = 3, MAIN_MXFP6 = 4 };
 
 struct QuantParams {
   int M, K, Kpad, Mpad;
   int G;                // SINT4: groups of 64 that hold data
   int nst;              // Kpad / 128 stages of K
   int groups, stages;   // RG row groups of 8 per tile, SX stages of K per chunk
+  int teams;            // teams of RG * SX quantizer warps: they take the chunks in turn
   int ntiles, nchunks;  // tiles of the launch, chunks of a tile
   int slots, xslots;    // chunk slots of the branch's operands and of X
   int refetch;          // integer branch: the X ring is smaller than a tile, which is streamed twice
@@ -75,24 +80,25 @@ struct QuantParams {
   int8_t* qb;           // [Mpad][Kpad] or null (not stored)
   float* sXb;           // [Mpad]
   const float* sL1;     // [LQ_MAX_RANK]
-  const uint8_t* sfl1;  // MX branches: E8M0 bytes of the first factor's block scales, [planes][Kpad/128][512]
+  const uint8_t* l1c;   // MXFP: the first factor's elements, [rn][Kpad] (the MMA reads them through tmL1)
+  const uint8_t* sfl1;  // MX branches: E8M0 bytes of the first factor's block scales, [Kpad/128][512]
   uint8_t* sft;         // MX branches: E8M0 bytes of the rank-r intermediate's block scales, [Mpad/128][512 or 1024]
   uint8_t* tq;          // [Mpad][tq_stride]
   float* sT;            // [Mpad]
   int r, rn;            // rank, rank rounded up to 16 (columns of the MMA)
-  int bplanes;          // MXINT: digit planes of the first factor (2: 8-bit codes, 1: 4-bit codes)
+  int bplanes;          // digit planes of the first factor, side by side in the MMA's columns (2: MXINT8 factors, else 1)
   int tq_stride;        // bytes per row of tq: LQ_RCONT, or 2 LQ_RCONT when each digit plane of the intermediate has a container
-  int nacc;             // accumulators a tile's stages alternate over (floating-point branches: shorter chains of fp32 sums)
+  int nacc, sets;       // accumulators a tile's stages alternate over (floating-point branches: shorter chains of fp32 sums),
+                        // sets of them (2: the next tile's MMAs run under a4)
   int tmem_cols;        // power of two
   int smem;             // dynamic shared memory of the launch
-  int act6;             // MXFP: the activations (X and the rank-r intermediate) are MXFP6e2 instead of MXFP8e4
+  float dev;            // MXFP: how far a sum of the tensor core may be from the one in defining order, over its block's maximum
   float qm;             // largest branch activation code
   int32_t* status;
 };
 
-// Shared memory, from a 1024-byte aligned base; the same arithmetic on the host (size) and in the kernel.  First the X ring;
-// then the slots: a slot holds a
-// chunk: its operand slabs (128 bytes of K wide, a_ps and b_ps of them per stage) and scale bytes.
+// Shared memory, from a 1024-byte aligned base; the same arithmetic on the host (size) and in the kernel.  First the X ring,
+// then the slots: a slot holds a chunk's operand slabs (128 bytes of K wide, a_ps and b_ps of them per stage) and scale bytes.
 struct QuantSmem {
   int xslot, a_unit, a_ps, b_unit, b_ps;
   int off_b, off_sfa, off_sfb, slot;            // within a slot
@@ -102,9 +108,9 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
   QuantSmem s{};
   const bool mx = br == BR_MXFP || br == BR_MXINT;
   s.xslot = tr * 256 * st;                      // st: stages of K per chunk
-  s.a_unit = tr * 128; s.b_unit = rn * 128;
+  s.a_unit = tr * 128; s.b_unit = rn * bplanes * 128;
   s.a_ps = br == BR_NONE ? 0 : (br == BR_F16 || br == BR_MXINT) ? 2 : 1;
-  s.b_ps = br == BR_NONE ? 0 : br == BR_F16 ? 2 : br == BR_MXINT ? bplanes : 1;
+  s.b_ps = br == BR_NONE ? 0 : br == BR_F16 ? 2 : 1;
   s.off_b = st * s.a_ps * s.a_unit;
   s.off_sfa = s.off_b + st * s.b_ps * s.b_unit;
   s.off_sfb = s.off_sfa + (mx ? st * s.a_ps * 512 : 0);
@@ -112,14 +118,24 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
   s.slot = (s.slot + 1023) & ~1023;
   s.off_slots = xslots * s.xslot;
   s.off_l1 = s.off_slots + (br == BR_NONE ? 0 : slots) * s.slot;
-  s.off_max = s.off_l1 + LQ_MAX_RANK * 4;       // row maxima of three tiles in rotation, row scales of two
+  s.off_max = s.off_l1 + (br == BR_MXFP ? 2 * MAX_UNSETTLED * 16 + 256 * 4 : LQ_MAX_RANK * 4);   // sL1; MXFP: list, scratch
+  // row maxima of three tiles in rotation, row scales of two
   s.off_sb = s.off_max + 3 * 64 * 4;
   s.off_bar = s.off_sb + 2 * 64 * 4;
-  s.total = s.off_bar + 128;
+  s.total = s.off_bar + 8 * (2 * MAX_XSLOTS + 3 * MAX_SLOTS + 5) + 16;
   // the 128-row MMA reads past the last slab of a shorter tile
   if (br != BR_NONE && s.total < s.off_l1 + 128 * 128) s.total = s.off_l1 + 128 * 128;
   return s;
 }
+
+// Position in a ring of n slots and the parity its barriers have there.
+struct Ring {
+  int at;
+  uint32_t par;
+  __device__ __forceinline__ void step(int by, int n) {
+    for (at += by; at >= n; at -= n) par ^= 1;
+  }
+};
 
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
 __device__ __forceinline__ uint32_t as_u32(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
@@ -144,10 +160,26 @@ __device__ __forceinline__ __half absmax8(const uint4& a) {
   return __hmax(__low2half(m), __high2half(m));
 }
 
-// 2^-e as an fp16 factor (1 for the all-zero block's -127).  Where that is out of fp16's range - the block's maximum is
-// below 2^-7 or less - the values are scaled up, exactly, and e follows.
+// Block exponents and factors 2^-e of two rows at once, from the fp16 bit patterns of their block maxima (the low half: the
+// first row).  e = E' - TOP, E' the maximum's binary exponent, one more where its mantissa is beyond 0x400 - UP.  The
+// exponent fields stay where they are in the halves: two integer instructions give both factors.  Where a factor would
+// not be a normal fp16 number - a maximum below 2^-7 or less, an all-zero block - `ok` is false.
+template <int TOP, int UP>
+struct PairScale {
+  uint32_t inv;          // the factors' bit patterns
+  uint32_t bytes;        // E8M0 bytes: first row in bits 0-7, second in bits 16-23
+  bool ok;
+  __device__ __forceinline__ explicit PairScale(uint32_t bm) {
+    const uint32_t m = (bm + (uint32_t)(UP * 0x10001)) & 0x7C007C00u;
+    inv = (uint32_t)((30 + TOP) << 10) * 0x10001u - m;
+    bytes = (m >> 10) + (uint32_t)(112 - TOP) * 0x10001u;
+    ok = (m & 0xFFFFu) >= (TOP << 10) && m >= ((uint32_t)TOP << 26);
+  }
+};
+// The same factor for one row and any exponent (1 for the all-zero block's -127).  Where 2^-e is out of fp16's range the
+// values are scaled up, exactly, and e follows.
 __device__ __forceinline__ __half2 half_scale(uint4& v, int e) {
-  if (e < -15 && e > -127) {
+  if (e > -127) {
     const __half2 up = __float2half2_rn(4096.f);
     for (; e < -15; e += 12) {
       v.x = as_u32(__hmul2(as_half2(v.x), up)); v.y = as_u32(__hmul2(as_half2(v.y), up));
@@ -163,8 +195,9 @@ __device__ __forceinline__ __half2 half_scale(uint4& v, int e) {
 // the hardware conversion (nearest even, magnitudes above the largest normal clamped).  Every e2m3 value is an e4m3
 // value, so both formats are stored, and multiplied, as e4m3 bytes: the 6-bit path rounds to e2m3 first and widens
 // the result (e2m3 -> f16 -> e4m3, both exact).
-__device__ __forceinline__ int mxfp8_exponent(float a, bool six = false) {
-  const int e = (int)(__float_as_uint(a) >> 23) - 127 - (six ? 2 : 8);
+template <bool SIX>
+__device__ __forceinline__ int mxfp_exponent(float a) {
+  const int e = (int)(__float_as_uint(a) >> 23) - 127 - (SIX ? 2 : 8);
   return (a > 0.f && e >= -126) ? e : -127;
 }
 __device__ __forceinline__ uint32_t f32x2_to_e4m3x2_via_e2m3(float hi, float lo) {
@@ -175,24 +208,20 @@ __device__ __forceinline__ uint32_t f32x2_to_e4m3x2_via_e2m3(float hi, float lo)
   asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(r8) : "r"(h2));
   return (uint32_t)r8;
 }
-__device__ __forceinline__ uint32_t mxfp_pair(float hi, float lo, bool six) {
-  return six ? f32x2_to_e4m3x2_via_e2m3(hi, lo) : f32x2_to_e4m3x2(hi, lo);
+template <bool SIX>
+__device__ __forceinline__ uint32_t mxfp_pair(float hi, float lo) {
+  return SIX ? f32x2_to_e4m3x2_via_e2m3(hi, lo) : f32x2_to_e4m3x2(hi, lo);
 }
-__device__ __forceinline__ uint2 mxfp_codes8(uint4 v, int e, bool six) {
-  uint2 w;
-  if (six) {
-    const float inv = e == -127 ? 0.f : pow2f_n(-e);
-    const float2 a = __half22float2(as_half2(v.x)), b = __half22float2(as_half2(v.y)), c = __half22float2(as_half2(v.z)),
-                 d = __half22float2(as_half2(v.w));
-    w.x = f32x2_to_e4m3x2_via_e2m3(a.y * inv, a.x * inv) | (f32x2_to_e4m3x2_via_e2m3(b.y * inv, b.x * inv) << 16);
-    w.y = f32x2_to_e4m3x2_via_e2m3(c.y * inv, c.x * inv) | (f32x2_to_e4m3x2_via_e2m3(d.y * inv, d.x * inv) << 16);
-    return w;
-  }
-  const __half2 inv = half_scale(v, e);  // e in [-32, 7]
+__device__ __forceinline__ uint2 mxfp6_codes8(const uint4& v, int e) {
+  const float inv = e == -127 ? 0.f : pow2f_n(-e);
+  const float2 a = __half22float2(as_half2(v.x)), b = __half22float2(as_half2(v.y)), c = __half22float2(as_half2(v.z)),
+               d = __half22float2(as_half2(v.w));
+  return make_uint2(f32x2_to_e4m3x2_via_e2m3(a.y * inv, a.x * inv) | (f32x2_to_e4m3x2_via_e2m3(b.y * inv, b.x * inv) << 16),
+                    f32x2_to_e4m3x2_via_e2m3(c.y * inv, c.x * inv) | (f32x2_to_e4m3x2_via_e2m3(d.y * inv, d.x * inv) << 16));
+}
+__device__ __forceinline__ uint2 mxfp8_codes8(const uint4& v, __half2 inv) {
   auto q = [&](uint32_t h) { return __hmul2(as_half2(h), inv); };
-  w.x = f16x4_to_e4m3x4(q(v.x), q(v.y));
-  w.y = f16x4_to_e4m3x4(q(v.z), q(v.w));
-  return w;
+  return make_uint2(f16x4_to_e4m3x4(q(v.x), q(v.y)), f16x4_to_e4m3x4(q(v.z), q(v.w)));
 }
 
 // MXINT4 (Appendix A.3): 2^e with e the smallest integer such that 7 * 2^e >= a: a = 1.f * 2^E, e = E - 2 if 1.f <= 1.75
@@ -201,8 +230,8 @@ __device__ __forceinline__ int mxint4_exponent(float a) {
   const uint32_t ab = __float_as_uint(a);
   return a > 0.f ? (int)(ab >> 23) - 127 - (((ab & 0x7FFFFFu) <= 0x600000u) ? 2 : 1) : -127;
 }
-__device__ __forceinline__ uint2 mxint4_codes8(uint4 v, int e) {
-  const __half2 magic = __float2half2_rn(1536.f), inv = half_scale(v, e);   // e in [-26, 14]
+__device__ __forceinline__ uint2 mxint4_codes8(const uint4& v, __half2 inv) {
+  const __half2 magic = __float2half2_rn(1536.f);
   auto q = [&](uint32_t h) { return __hsub2(__hfma2(as_half2(h), inv, magic), magic); };
   return make_uint2(f16x4_to_e4m3x4(q(v.x), q(v.y)), f16x4_to_e4m3x4(q(v.z), q(v.w)));
 }
@@ -217,8 +246,7 @@ __device__ __forceinline__ int mxint8_exponent(float a) {
 }
 // The code c = rint_even(x / 2^e) of eight values as two digits, c = 16 hi + lo, lo in [-8, 7], hi in [-8, 8], both exact
 // E4M3 values: hi = rint((c + 1/4) / 16), every step exact in fp16 (|c| <= 127).
-__device__ __forceinline__ void mxint8_codes8(uint4 v, int e, uint2& hi, uint2& lo) {
-  const __half2 inv = half_scale(v, e);  // e in [-30, 10]
+__device__ __forceinline__ void mxint8_codes8(const uint4& v, __half2 inv, uint2& hi, uint2& lo) {
   const __half2 magic = __float2half2_rn(1536.f), sixteenth = __float2half2_rn(0.0625f), bias = __float2half2_rn(0.015625f),
                 m16 = __float2half2_rn(-16.f);
   __half2 h[4], l[4];
@@ -239,30 +267,62 @@ __device__ __forceinline__ void mxint8_digits(float x, float inv, float& hi, flo
   lo = __fmaf_rn(hi, -16.f, c);
 }
 
-// SINT4 (Appendix A.3): fp16 scale a / 7 (at least 2^-24), codes rint_even(x / s) clamped to [-7, 7]; only a subnormal
-// scale can leave the quotient above 7.5.
-struct Sint4Scale {
-  float s, inv;
-  bool coarse;
+// Two rows' vectors whose block maxima are out of PairScale's range (MXFP6e2: any): kept out of the main loop's instructions.
+// The E8M0 bytes come as PairScale has them.
+struct RareCodes {
+  uint2 wa, wb, da, db;
+  uint32_t bytes;
 };
-__device__ __forceinline__ Sint4Scale sint4_scale(float a) {
-  Sint4Scale m;
-  __half s16 = __float2half_rn(__fmul_rn(a, 0.142857149243354797f));   // fl32(1/7)
-  const unsigned short bits = __half_as_ushort(s16);
-  if (bits == 0) s16 = __ushort_as_half((unsigned short)1);             // floor 2^-24
-  m.s = __half2float(s16);
-  m.inv = __frcp_rn(m.s);
-  m.coarse = bits < 0x0400;
-  return m;
+template <int MAIN>
+__device__ __noinline__ RareCodes rare_codes(uint4 a, uint4 b, __half2 bm) {
+  const float m0 = __low2float(bm), m1 = __high2float(bm);
+  RareCodes r;
+  r.da = r.db = make_uint2(0, 0);
+  int e0, e1;
+  if constexpr (MAIN == MAIN_MXFP6) {
+    e0 = mxfp_exponent<true>(m0); e1 = mxfp_exponent<true>(m1);
+    r.wa = mxfp6_codes8(a, e0); r.wb = mxfp6_codes8(b, e1);
+  } else if constexpr (MAIN == MAIN_MXFP) {
+    e0 = mxfp_exponent<false>(m0); e1 = mxfp_exponent<false>(m1);
+    const __half2 i0 = half_scale(a, e0), i1 = half_scale(b, e1);
+    r.wa = mxfp8_codes8(a, i0); r.wb = mxfp8_codes8(b, i1);
+  } else if constexpr (MAIN == MAIN_MXINT4) {
+    e0 = mxint4_exponent(m0); e1 = mxint4_exponent(m1);
+    const __half2 i0 = half_scale(a, e0), i1 = half_scale(b, e1);
+    r.wa = mxint4_codes8(a, i0); r.wb = mxint4_codes8(b, i1);
+  } else {
+    e0 = mxint8_exponent(m0); e1 = mxint8_exponent(m1);
+    const __half2 i0 = half_scale(a, e0), i1 = half_scale(b, e1);
+    mxint8_codes8(a, i0, r.wa, r.da); mxint8_codes8(b, i1, r.wb, r.db);
+  }
+  r.bytes = (uint32_t)(e0 + 127) | ((uint32_t)(e1 + 127) << 16);
+  return r;
 }
+
+// SINT4 (Appendix A.3): fp16 scales a / 7 (at least 2^-24) of two rows from their group maxima; the reciprocals may be an
+// ulp off (see the top).  Codes rint_even(x / s) clamped to [-7, 7]; only a subnormal scale can leave the quotient above 7.5.
+struct Sint4Scale {
+  float s[2], inv[2];
+  bool coarse;
+  __device__ __forceinline__ explicit Sint4Scale(__half2 a) {
+    const float2 f = __half22float2(a);
+    const __half2 s16 = __floats2half2_rn(__fmul_rn(f.x, 0.142857149243354797f), __fmul_rn(f.y, 0.142857149243354797f));   // fl32(1/7)
+    const uint32_t bits = __vmaxu2(as_u32(s16), 0x00010001u);           // floor 2^-24
+    const float2 g = __half22float2(as_half2(bits));
+    s[0] = g.x; s[1] = g.y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv[0]) : "f"(g.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv[1]) : "f"(g.y));
+    coarse = (bits & 0xFFFFu) < 0x0400u || bits < 0x04000000u;
+  }
+};
 __device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
-__device__ __forceinline__ uint2 sint4_codes8(const uint4& v, const Sint4Scale& m) {
+__device__ __forceinline__ uint2 sint4_codes8(const uint4& v, float rcp, bool coarse) {
   const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
-  const float2 inv = splat(m.inv), c0 = splat(192.f), c1 = splat(MAGIC - 192.f), c2 = splat(-MAGIC);
+  const float2 inv = splat(rcp), c0 = splat(192.f), c1 = splat(MAGIC - 192.f), c2 = splat(-MAGIC);
   float2 q[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) q[i] = __fadd2_rn(__fadd2_rn(__ffma2_rn(x[i], inv, c0), c1), c2);
-  if (m.coarse) {
+  if (coarse) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) q[i] = make_float2(fminf(fmaxf(q[i].x, -7.f), 7.f), fminf(fmaxf(q[i].y, -7.f), 7.f));
   }
@@ -289,9 +349,97 @@ __device__ __forceinline__ uint2 branch_codes8(const uint4& v, float sb, float i
   return b;
 }
 
+// One element of T = deq(Q(X)) deq(Q2(L1)) with the sum in its defining order (whole warp; every lane gets it): a partial sum
+// of 32 products per block on mma.sync, fp32 additions of the scaled partial sums in nine interleaved chains (box g of 64
+// values belongs to chain g mod 9, its second block first), the chains added in order.  The tensor core's own order differs
+// from it by less than 2^-22.2 of the block's maximum in 999 of 1000 elements at K = 1152, 2^-20.6 at K = 4608 with
+// one-sided inputs.  Eight blocks per MMA: row i of A and column i of B hold block i, so the products wanted are on the
+// diagonal.
+__device__ __forceinline__ void mma_e4m3_16832(float (&c)[4], uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k32.row.col.f32.e4m3.e4m3.f32 {%0,%1,%2,%3}, {%4,%5,%6,%5}, {%7,%8}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(0), "r"(a2), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint2 ld_volatile_v2(const uint8_t* p) {
+  uint2 v;
+  asm volatile("ld.volatile.global.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+  return v;
+}
+// The partial sums of one element, scaled, into `part`: warp w of the block takes blocks 8 w .. 8 w + 7 and so on.
+__device__ __noinline__ void canonical_parts(const uint8_t* qx, const uint8_t* sfx, const uint8_t* l1, const uint8_t* sfl, int blocks, float* part) {
+  const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+#pragma unroll 1
+  for (int b0 = 8 * (int)(threadIdx.x >> 5); b0 < blocks; b0 += 8 * (NTHREADS / 32)) {
+    const int b = b0 + gid;                                      // (blocks is a multiple of 4)
+    uint2 a = make_uint2(0, 0), w = a;
+    float s = 0.f;
+    if (b < blocks) {
+      a = ld_volatile_v2(qx + 32 * b + 8 * tig);
+      w = *reinterpret_cast<const uint2*>(l1 + 32 * b + 8 * tig);
+      const uint32_t ea = *reinterpret_cast<const volatile uint8_t*>(sfx + (b >> 2) * 512 + (b & 3)), el = sfl[(b >> 2) * 512 + (b & 3)];
+      s = __uint_as_float(ea << 23) * __uint_as_float(el << 23);
+    }
+    float c[4] = {0.f, 0.f, 0.f, 0.f};
+    mma_e4m3_16832(c, a.x, a.y, w.x, w.y);
+    if (tig == (gid >> 1) && b < blocks) part[b] = ((gid & 1) ? c[1] : c[0]) * s;
+  }
+}
+// Their sum (whole warp; every lane gets it).
+__device__ __forceinline__ float canonical_sum(const float* part, int blocks) {
+  const int lane = threadIdx.x & 31;
+  float chain = 0.f, v = 0.f;
+  if (lane < 9)
+    for (int b = 2 * lane; b < blocks; b += 18) chain = __fadd_rn(part[b], __fadd_rn(part[b + 1], chain));
+  for (int c = 0; c < 9; ++c) v += __shfl_sync(0xffffffffu, chain, c);
+  return v;
+}
+// Whether an element may change its code within the deviation: elements of the largest binade (steps of 32 in e4m3, 1/2 in
+// e2m3) whose distance to the nearest code is within the deviation of half a step.
+template <bool SIX>
+struct TieTest {
+  float k, limit;
+  __device__ __forceinline__ TieTest(float inv, float dev) : k(inv * (SIX ? 2.f : 0.03125f)), limit(0.5f - dev * k) {}
+  __device__ __forceinline__ bool operator()(float x) const {
+    const float u = fabsf(x) * k;
+    return u > 7.5f && fabsf(u - __fadd_rn(__fadd_rn(u, MAGIC), -MAGIC)) > limit;
+  }
+};
+// Elements `what.z` of block `what.y` of row `what.x` of the rank-r intermediate again, from the sums in defining order (all
+// threads of the CTA); with all of them asked for, the block's exponent too.
+template <bool SIX>
+__device__ __noinline__ void settle_block(const QuantParams& p, int4 what, float* part) {
+  const int lane = threadIdx.x & 31, m = what.x, b = what.y;
+  const uint32_t which = (uint32_t)what.z;
+  const size_t sf_row = 16 * (m & 31) + 4 * ((m & 127) >> 5);
+  float mine = 0.f;
+  for (uint32_t todo = which; todo != 0; todo &= todo - 1) {
+    const int j = __ffs(todo) - 1, col = 32 * b + j;
+    if (col >= p.r) break;
+    canonical_parts(p.qx8 + (size_t)m * p.Kpad, p.sfa + (size_t)(m >> 7) * (p.Kpad >> 7) * 512 + sf_row, p.l1c + (size_t)col * p.Kpad,
+                    p.sfl1 + 16 * (col & 31) + 4 * (col >> 5), p.Kpad / 32, part);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const float v = canonical_sum(part, p.Kpad / 32);
+      if (lane == j) mine = v;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x >= 32) return;
+  int e = what.w;
+  if (which == 0xFFFFFFFFu) {
+    float amax = fabsf(mine);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    e = mxfp_exponent<SIX>(amax);
+    if (lane == 0) p.sft[(size_t)(m >> 7) * 512 + sf_row + b] = (uint8_t)(e + 127);
+  }
+  const float inv = e == -127 ? 0.f : pow2f_n(-e);
+  if ((which >> lane) & 1) p.tq[(size_t)m * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, mine * inv);
+}
+
 template <int MAIN, int BR>
 __global__ void __launch_bounds__(NTHREADS, 1)
-lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmL1, const QuantParams p) {
+lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmL1,
+                const __grid_constant__ QuantParams p) {
   constexpr bool SINT = MAIN == MAIN_SINT4;
   constexpr bool MXB = BR == BR_MXFP || BR == BR_MXINT;      // the branch multiplies the main codes under their scale bytes
   extern __shared__ uint8_t qsm_raw[];
@@ -299,7 +447,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint8_t* smem = qsm_raw + (base - smem_u32(qsm_raw));
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31;
-  const int RG = p.groups, spc = p.stages, TR = 8 * RG, nq = RG * spc;       // spc: stages of K per chunk
+  const int RG = p.groups, spc = p.stages, TR = 8 * RG, nq = RG * spc;       // spc: stages of K per chunk, nq: warps of a team
   const QuantSmem sm = quant_smem(BR, TR, spc, p.rn, p.bplanes, p.slots, p.xslots);
   auto bar_afull = [&](int s) { return base + (uint32_t)sm.off_bar + 8u * (uint32_t)s; };
   auto bar_bfull = [&](int s) { return bar_afull(MAX_SLOTS + s); };
@@ -320,7 +468,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     if constexpr (BR != BR_NONE) {
       for (int s = 0; s < p.slots; ++s) { mbar_init(bar_afull(s), (uint32_t)nq); mbar_init(bar_bfull(s), 1); mbar_init(bar_empty(s), 1); }
       for (int b = 0; b < 2; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), 2); }
-      mbar_init(bar_sync, (uint32_t)nq);
+      mbar_init(bar_sync, (uint32_t)(nq * p.teams));
     }
     *abort_flag = 0;
     mbar_init_fence();
@@ -364,46 +512,46 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (--xs < 0) { xs = p.xslots - 1; par ^= 1; }
         mbar_settle(bar_xfull(xs), par ^ 1);
       }
-  } else if (BR != BR_NONE && warp == 2) {
-    // ------------------------------------------------------------------ first factor and MMA issuer
-    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    const uint32_t shape = idesc_shape(p.rn), tsf = tmem + (uint32_t)(2 * p.nacc * p.rn);
-    const int total = ((p.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * p.nchunks;   // chunks of this CTA
-    // the slabs of chunk number n (chunk `c` of its tile) into their slot: weights, so no earlier kernel is waited for
-    auto fetch_b = [&](int slot, int c) {
-      const int st0 = c * spc, ns = min(spc, p.nst - st0);
-      const uint32_t dst = base + (uint32_t)(sm.off_slots + slot * sm.slot), full = bar_bfull(slot);
-      if (elect_one()) {
-        mbar_expect_tx(full, (uint32_t)(ns * sm.b_ps * (sm.b_unit + (MXB ? 512 : 0))));
-        for (int s = 0; s < ns; ++s)
-          for (int u = 0; u < sm.b_ps; ++u) {
-            const int i = s * sm.b_ps + u;
-            // fp16: a stage's 256 bytes of K in two slabs; digit planes: rn rows further down
-            tma_load_2d(dst + sm.off_b + i * sm.b_unit, &tmL1, BR == BR_F16 ? (2 * (st0 + s) + u) * 128 : (st0 + s) * 128,
-                        BR == BR_F16 ? 0 : u * p.rn, full);
-            if constexpr (MXB) bulk_load(dst + sm.off_sfb + i * 512, p.sfl1 + (size_t)(u * p.nst + st0 + s) * 512, 512, full);
-          }
-      }
-      __syncwarp();
-    };
-    int fetched = 0, fslot = 0, fchunk = 0;
-    uint32_t fpar = 1;
+  } else if (BR != BR_NONE && warp == 4) {
+    // ------------------------------------------------------------------ TMA producer: the first factor (weights: no earlier
+    // kernel has to be waited for)
+    int slot = 0;
+    uint32_t par = 1, issued = 0;
     bool ok = true;
-    // keeps the slabs of up to slots - 1 chunks ahead of the MMAs in flight; a slot's previous MMAs were issued a chunk ago
-    auto fetch_upto = [&](int n) {
-      for (; ok && fetched < n; ++fetched) {
-        ok = mbar_wait_warp(bar_empty(fslot), fpar, abort_flag, p.status, LQ_STAGE_MMA);
+    for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x)
+      for (int c = 0; c < p.nchunks; ++c) {
+        ok = mbar_wait_warp(bar_empty(slot), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
         if (!ok) break;
-        fetch_b(fslot, fchunk);
-        if (++fslot == p.slots) { fslot = 0; fpar ^= 1; }
-        if (++fchunk == p.nchunks) fchunk = 0;
+        const int st0 = c * spc, ns = min(spc, p.nst - st0);
+        const uint32_t dst = base + (uint32_t)(sm.off_slots + slot * sm.slot), full = bar_bfull(slot);
+        if (elect_one()) {
+          mbar_expect_tx(full, (uint32_t)(ns * sm.b_ps * (sm.b_unit + (MXB ? 512 : 0))));
+          for (int s = 0; s < ns; ++s)
+            for (int u = 0; u < sm.b_ps; ++u) {
+              const int i = s * sm.b_ps + u;                     // fp16: a stage's 256 bytes of K in two slabs
+              tma_load_2d(dst + sm.off_b + i * sm.b_unit, &tmL1, (BR == BR_F16 ? 2 * (st0 + s) + u : st0 + s) * 128, 0, full);
+              if constexpr (MXB) bulk_load(dst + sm.off_sfb + i * 512, p.sfl1 + (size_t)(st0 + s) * 512, 512, full);
+            }
+        }
+        __syncwarp();
+        ++issued;
+        if (++slot == p.slots) { slot = 0; par ^= 1; }
       }
-    };
-    fetch_upto(min(p.slots, total));
+    if (!ok && lane == 0)      // aborting: the copies in flight get a bounded time to land
+      for (uint32_t i = min(issued, (uint32_t)p.slots); i > 0; --i) {
+        if (--slot < 0) { slot = p.slots - 1; par ^= 1; }
+        mbar_settle(bar_bfull(slot), par ^ 1);
+      }
+  } else if (BR != BR_NONE && warp == 2) {
+    // ------------------------------------------------------------------ MMA issuer
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    const int cols = p.rn * p.bplanes;
+    const uint32_t shape = idesc_shape(cols), tsf = tmem + (uint32_t)(p.sets * p.nacc * cols);
+    bool ok = true;
     uint32_t tc = 0, par = 0;
-    int slot = 0, done = 0;
+    int slot = 0;
     for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x, ++tc) {
-      const uint32_t set = tmem + (uint32_t)((tc & 1) * p.nacc * p.rn);
+      const uint32_t set = tmem + (uint32_t)((tc & (p.sets - 1)) * p.nacc * cols);
       ok = mbar_wait_warp(bar_tempty(tc & 1), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
       for (int c = 0; c < p.nchunks && ok; ++c) {
         const int ns = min(spc, p.nst - c * spc);
@@ -415,7 +563,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (elect_one()) {
           for (int s = 0; s < ns; ++s) {
             const int gs = c * spc + s;                          // stage of K: the accumulators take turns
-            const uint32_t d = set + (uint32_t)((gs & (p.nacc - 1)) * p.rn), more = gs >= p.nacc;
+            const uint32_t d = set + (uint32_t)((gs & (p.nacc - 1)) * cols), more = gs >= p.nacc;
             const uint32_t a = at + s * sm.a_ps * sm.a_unit, bw = at + sm.off_b + s * sm.b_ps * sm.b_unit;
             if constexpr (BR == BR_INT) {
               const uint64_t ad = make_smem_desc(a), bd = make_smem_desc(bw);
@@ -428,17 +576,16 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
                                IDESC_F16 | shape, more | (uint32_t)j);
             } else {
               // scale bytes into tensor memory (one slot: the tensor pipe executes these copies and MMAs in issue order),
-              // then every pair of digit planes
-              const int ap = BR == BR_MXINT ? 2 : 1, bp = BR == BR_MXINT ? p.bplanes : 1;
+              // then the activations' digit planes one after the other
+              const int ap = BR == BR_MXINT ? 2 : 1;
               for (int u = 0; u < ap; ++u) tc_cp_sf(tsf + 4 * u, make_smem_desc_plain(at + sm.off_sfa + (s * ap + u) * 512, 16, 128));
-              for (int u = 0; u < bp; ++u) tc_cp_sf(tsf + 8 + 4 * u, make_smem_desc_plain(at + sm.off_sfb + (s * bp + u) * 512, 16, 128));
-              for (int ua = 0; ua < ap; ++ua)
-                for (int ub = 0; ub < bp; ++ub) {
-                  const uint64_t ad = make_smem_desc(a + ua * sm.a_unit), bd = make_smem_desc(bw + ub * sm.b_unit);
+              tc_cp_sf(tsf + 8, make_smem_desc_plain(at + sm.off_sfb + s * 512, 16, 128));
+              for (int u = 0; u < ap; ++u) {
+                const uint64_t ad = make_smem_desc(a + u * sm.a_unit), bd = make_smem_desc(bw);
 #pragma unroll
-                  for (int j = 0; j < 4; ++j)
-                    tc_mma_mx(d, ad + 2 * j, bd + 2 * j, idesc_mx(p.rn, j), tsf + 4 * ua, tsf + 8 + 4 * ub, more | (uint32_t)(j | ua | ub));
-                }
+                for (int j = 0; j < 4; ++j)
+                  tc_mma_mx(d, ad + 2 * j, bd + 2 * j, idesc_mx(cols, j), tsf + 4 * u, tsf + 8, more | (uint32_t)(j | u));
+              }
             }
           }
           tc_commit(bar_empty(slot));
@@ -446,14 +593,6 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         }
         __syncwarp();
         if (++slot == p.slots) { slot = 0; par ^= 1; }
-        ++done;
-        fetch_upto(min(done + p.slots - 1, total));
-      }
-    }
-    if (!ok && lane == 0) {    // aborting: the copies in flight get a bounded time to land
-      for (int i = min(fetched, p.slots); i > 0; --i) {
-        if (--fslot < 0) { fslot = p.slots - 1; fpar ^= 1; }
-        mbar_settle(bar_bfull(fslot), fpar ^ 1);
       }
     }
   } else if (BR != BR_NONE && warp < 2) {
@@ -462,115 +601,144 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0) + ((uint32_t)(32 * warp) << 16);
     const int nacc = min(p.nacc, p.nst), row = 32 * warp + lane;
     uint32_t tc = 0;
+    int4* unsettled = reinterpret_cast<int4*>(smem + sm.off_l1) + warp * MAX_UNSETTLED;   // MXFP: (row, block, elements, exponent) from 1 on
+    if (BR == BR_MXFP && lane == 0) unsettled[0].x = 0;
+    __syncwarp();
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++tc) {
       const int m = tile * TR + row;
       const bool valid = row < TR && m < p.M;
-      const uint32_t set = tmem + (uint32_t)((tc & 1) * p.nacc * p.rn);
+      const uint32_t set = tmem + (uint32_t)((tc & (p.sets - 1)) * p.nacc * p.rn * p.bplanes);
       if (!mbar_wait_warp(bar_tfull(tc & 1), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN)) break;
       tc_fence_after();
       uint8_t* const tqr = p.tq + (size_t)m * p.tq_stride;
       if (32 * warp < TR) {
-        // 32 columns of the row from `col` on (zeros beyond the accumulator): the accumulators' sum
-        auto fetch = [&](int col, float (&t)[32]) {
-          const bool wide = col + 16 < p.rn;
-          for (int a = 0; a < nacc; ++a) {
-            uint32_t v[32];
-            tmem_ld_32x16(set + (uint32_t)(a * p.rn + col), reinterpret_cast<uint32_t(&)[16]>(v[0]));
-            if (wide) tmem_ld_32x16(set + (uint32_t)(a * p.rn + col + 16), reinterpret_cast<uint32_t(&)[16]>(v[16]));
+        // 16 columns of the row from `col` on: the sum over the accumulators (and the first factor's digit planes)
+        auto fetch = [&](int col, float (&t)[16]) {
+          uint32_t v[16];
+#pragma unroll 1
+          for (int a = 0; a < nacc * p.bplanes; ++a) {
+            tmem_ld_32x16(set + (uint32_t)(a * p.rn + col), v);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const float x = j >= 16 && !wide ? 0.f : BR == BR_INT ? __int2float_rn((int)v[j]) : __uint_as_float(v[j]);
+            for (int j = 0; j < 16; ++j) {
+              const float x = BR == BR_INT ? __int2float_rn((int)v[j]) : __uint_as_float(v[j]);
               t[j] = a == 0 ? x : t[j] + x;
             }
           }
         };
-        float t[32];
+        float t[16];
         if constexpr (BR == BR_INT) {
           const float sr = row_sb[(tc & 1) * 64 + row];
-          auto scaled = [&](int c) {                           // t = fl32(fl32(I1) fl32(sXb sL1))
+          auto scaled = [&](int c) {                           // t = fl32(fl32(I1) fl32(sXb sL1)); rows beyond the tile hold anything
             fetch(c, t);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) t[j] = valid ? __fmul_rn(t[j], __fmul_rn(sr, sl1[c + j])) : 0.f;   // rows beyond the tile hold anything
+            for (int j = 0; j < 16; ++j) t[j] = valid ? __fmul_rn(t[j], __fmul_rn(sr, sl1[c + j])) : 0.f;
           };
           float amax = 0.f;
-          for (int c = 0; c < p.rn; c += 32) {
+#pragma unroll 1
+          for (int c = 0; c < p.rn; c += 16) {
             scaled(c);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) amax = fmaxf(amax, fabsf(t[j]));
+            for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(t[j]));
           }
-          const float st = amax == 0.f ? 1.f : __fdiv_rn(amax, p.qm), y = __frcp_rn(st);
-          const bool plain = st > 1e-27f && st < 1e27f;        // no step of the corrected quotient can leave binary32's normal range
+          const float st = amax == 0.f ? 1.f : __fdiv_rn(amax, p.qm);
           if (valid) p.sT[m] = st;
-          for (int c = 0; c < p.rn; c += 32) {                 // whole blocks of 32: zeros where the up-projection's K is padded
-            if (p.rn > 32) scaled(c);
-            uint32_t w[8];
+          // The quotient t / st as in branch_codes8.  A power of two keeps its steps in binary32's normal range; the quotient
+          // stays what it is (what underflows is far below half a code).
+          const float k = st < 1e-20f ? 0x1p64f : st > 1e20f ? 0x1p-64f : 1.f, ns = -st * k, y = __frcp_rn(st * k);
+#pragma unroll 1
+          for (int c = 0; c < p.rn; c += 16) {
+            scaled(c);
+            uint32_t w[4];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              float q;
-              if (plain) {
-                const float q0 = __fmul_rn(t[j], y);
-                q = __fmaf_rn(__fmaf_rn(-q0, st, t[j]), y, q0);
-              } else {
-                q = __fdiv_rn(t[j], st);
-              }
-              const uint32_t code = __float_as_uint(__fadd_rn(fminf(fmaxf(q, -p.qm), p.qm), MAGIC)) & 0xFFu;
+            for (int j = 0; j < 16; ++j) {
+              const float x = t[j] * k, q0 = __fmul_rn(x, y), q = __fmaf_rn(__fmaf_rn(q0, ns, x), y, q0);
+              const uint32_t code = __float_as_uint(__fadd_rn(q, MAGIC)) & 0xFFu;
               w[j >> 2] = (j & 3) == 0 ? code : w[j >> 2] | (code << (8 * (j & 3)));
             }
-            if (valid) {
-              *reinterpret_cast<uint4*>(tqr + c) = make_uint4(w[0], w[1], w[2], w[3]);
-              *reinterpret_cast<uint4*>(tqr + c + 16) = make_uint4(w[4], w[5], w[6], w[7]);
-            }
+            if (valid) *reinterpret_cast<uint4*>(tqr + c) = make_uint4(w[0], w[1], w[2], w[3]);
           }
+          // zeros up to the next multiple of 32, where the up-projection's K ends
+          if ((p.rn & 16) && valid) *reinterpret_cast<uint4*>(tqr + p.rn) = make_uint4(0, 0, 0, 0);
         } else if constexpr (BR == BR_F16) {
           if (valid) p.sT[m] = 1.f;
-          for (int c = 0; c < p.rn; c += 32) {
+#pragma unroll 1
+          for (int c = 0; c < p.rn; c += 16) {
             fetch(c, t);
-            uint32_t w[16];
+            uint32_t w[8];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) w[j] = as_u32(__floats2half2_rn(t[2 * j], t[2 * j + 1]));
+            for (int j = 0; j < 8; ++j) w[j] = as_u32(__floats2half2_rn(t[2 * j], t[2 * j + 1]));
             if (valid) {
-#pragma unroll
-              for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(tqr + 2 * c + 16 * j) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+              *reinterpret_cast<uint4*>(tqr + 2 * c) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(tqr + 2 * c + 16) = make_uint4(w[4], w[5], w[6], w[7]);
             }
           }
         } else {
-          // blocks of 32 along the rank.  MXINT with one container for both planes (rank <= 64): lo digits 64 bytes after the
-          // hi digits, scale slots c and 2 + c of one chunk; a container per plane: 128 bytes on, slot c of the next chunk
+          // blocks of 32 along the rank
+          constexpr bool FPB = BR == BR_MXFP, SIX = MAIN == MAIN_MXFP6;
+          // MXINT with one container for both planes (rank <= 64): lo digits 64 bytes after the hi digits, scale slots c and
+          // 2 + c of one chunk; a container per plane: 128 bytes on, slot c of the next chunk
           const bool sep = p.tq_stride != LQ_RCONT;
-          uint8_t* const sf = p.sft + (size_t)(m >> 7) * (BR == BR_MXINT && sep ? 1024 : 512) + 16 * (m & 31) + 4 * ((m & 127) >> 5);
+          uint8_t* const sf = p.sft + (size_t)(m >> 7) * (!FPB && sep ? 1024 : 512) + 16 * (m & 31) + 4 * ((m & 127) >> 5);
+#pragma unroll 1
           for (int b = 0; 32 * b < p.rn; ++b) {
+            float t2[16];
             fetch(32 * b, t);
+            if (32 * b + 16 < p.rn) fetch(32 * b + 16, t2);
+            else {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) t2[j] = 0.f;
+            }
             float amax = 0.f;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) amax = fmaxf(amax, fabsf(t[j]));
-            const int e = BR == BR_MXINT ? mxint8_exponent(amax) : mxfp8_exponent(amax, p.act6 != 0);
+            for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fmaxf(fabsf(t[j]), fabsf(t2[j])));
+            const int e = FPB ? mxfp_exponent<SIX>(amax) : mxint8_exponent(amax);
             const float inv = e == -127 ? 0.f : pow2f_n(-e);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
+              const float (&x)[16] = h ? t2 : t;
               uint32_t w[4], d[4];
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                if constexpr (BR == BR_MXINT) {
+                if constexpr (!FPB) {
                   float hi[4], lo[4];
 #pragma unroll
-                  for (int i = 0; i < 4; ++i) mxint8_digits(t[16 * h + 4 * j + i], inv, hi[i], lo[i]);
+                  for (int i = 0; i < 4; ++i) mxint8_digits(x[4 * j + i], inv, hi[i], lo[i]);
                   w[j] = f32x2_to_e4m3x2(hi[1], hi[0]) | (f32x2_to_e4m3x2(hi[3], hi[2]) << 16);
                   d[j] = f32x2_to_e4m3x2(lo[1], lo[0]) | (f32x2_to_e4m3x2(lo[3], lo[2]) << 16);
                 } else {
-                  const bool six = p.act6 != 0;
-                  w[j] = mxfp_pair(t[16 * h + 4 * j + 1] * inv, t[16 * h + 4 * j] * inv, six) | (mxfp_pair(t[16 * h + 4 * j + 3] * inv, t[16 * h + 4 * j + 2] * inv, six) << 16);
+                  w[j] = mxfp_pair<SIX>(x[4 * j + 1] * inv, x[4 * j] * inv) | (mxfp_pair<SIX>(x[4 * j + 3] * inv, x[4 * j + 2] * inv) << 16);
                   d[j] = 0;
                 }
               }
               if (valid) {
                 *reinterpret_cast<uint4*>(tqr + 32 * b + 16 * h) = make_uint4(w[0], w[1], w[2], w[3]);
-                if (BR == BR_MXINT) *reinterpret_cast<uint4*>(tqr + (sep ? 128 : 64) + 32 * b + 16 * h) = make_uint4(d[0], d[1], d[2], d[3]);
+                if (!FPB) *reinterpret_cast<uint4*>(tqr + (sep ? 128 : 64) + 32 * b + 16 * h) = make_uint4(d[0], d[1], d[2], d[3]);
               }
             }
             if (valid) {
-              sf[b] = (uint8_t)(e + 127 + (BR == BR_MXINT ? 4 : 0));
-              if (BR == BR_MXINT) sf[(sep ? 512 : 2) + b] = (uint8_t)(e + 127);
+              sf[b] = (uint8_t)(e + 127 + (FPB ? 0 : 4));
+              if (!FPB) sf[(sep ? 512 : 2) + b] = (uint8_t)(e + 127);
+            }
+            if constexpr (FPB) {
+              // Floating-point elements round in steps of up to a fourteenth of the block's maximum, so a sum that lands on the
+              // other side of a tie can show in Y.  What is too close to call on the tensor core's sum - the block's
+              // exponent, an element of the largest binade - is decided on the sum in its defining order, at the end by
+              // all warps (a launch of 8192 rows and rank 64 meets one every few times; settled on the spot, the code around
+              // it cost 3-6 us in every launch, and one warp alone takes 4-12 us for an element).  Where the list is full the tensor core's sum stands.
+              const float dev = amax * p.dev;
+              const TieTest<SIX> tie(inv, dev);
+              const bool edge = ((__float_as_uint(amax + dev) ^ __float_as_uint(amax - dev)) >> 23) != 0;
+              bool close = edge;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) close |= tie(t[j]) | tie(t2[j]);
+              if (valid && close) {
+                uint32_t which = 0;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) which |= (tie(t[j]) ? 1u << j : 0u) | (tie(t2[j]) ? 0x10000u << j : 0u);
+                const int n = atomicAdd(&unsettled[0].x, 1) + 1;
+                if (n < MAX_UNSETTLED) unsettled[n] = make_int4(m, b, edge ? -1 : (int)which, e);
+              }
             }
           }
         }
@@ -579,12 +747,12 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_tempty(tc & 1));
     }
-  } else if (warp >= FIRST_QWARP && qw < nq) {
+  } else if (warp >= FIRST_QWARP && qw < nq * p.teams) {
     // ------------------------------------------------------------------ quantizer
     // This lane: 16-byte vector lc of rows ra and ra + 2 of the tile, of both 64-value boxes of a stage.  The four rows of
     // one access have both values of bit 2, so that the 64-byte halves they write to an operand slab do not meet in the
     // same banks.
-    const int rg = qw % RG, sx = qw / RG, lr = lane >> 3, lc = lane & 7;
+    const int team = qw / nq, rg = (qw - team * nq) % RG, sx = (qw - team * nq) / RG, lr = lane >> 3, lc = lane & 7;
     const int ra = 8 * rg + (lr & 1) + 2 * (lr & 2);
     const uint32_t sw = (uint32_t)(ra & 7), hstep = (uint32_t)(TR * 128);               // from a box to the next
     const uint32_t xo = base + (uint32_t)(sx * TR * 256 + ra * 128);                    // row ra of this warp's first box
@@ -597,8 +765,9 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const uint32_t so = base + (uint32_t)(sm.off_slots + sm.off_sfa + sx * sm.a_ps * 512 + 16 * (sr & 31) + 4 * (sr >> 5));
     const size_t qs = MAIN == MAIN_MXINT8 ? (size_t)2 * p.Kpad : (size_t)p.Kpad;        // bytes per row of qx8
     grid_dependency_wait();        // from here on the activation record is written
-    int xs = 0, slot = 0;
-    uint32_t xpar = 0, epar = 1, tc = 0, buf = 0;
+    Ring xr{0, 0u}, er{0, 1u};     // X slot and operand slot of the current tile's (walk's) first chunk
+    uint32_t tc = 0, buf = 0;
+    int c0 = team;                 // this team's first chunk of the tile: chunks go round the teams without regard to tiles
     bool ok = true;
     for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x, ++tc) {
       const int ma = tile * TR + ra, ms = tile * TR + sr;
@@ -609,12 +778,15 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       __half2 hm = __float2half2_rn(0.f);                        // maxima of rows ra, ra + 2
       // One walk over the tile.  MAINP: main codes and scales; BRP: the branch's operand; FREE: the X slots are handed back.
       auto walk = [&](auto MAINP, auto BRP, const bool free_x) {
-        for (int c = 0, st = sx; c < p.nchunks; ++c, st += spc) {
+        Ring x = xr, e = er;
+        x.step(c0, p.xslots);
+        e.step(c0, p.slots);
+        for (int c = c0, st = c0 * spc + sx; c < p.nchunks; c += p.teams, st += p.teams * spc) {
           const bool live = st < p.nst;
-          if (!mbar_wait_warp(bar_xfull(xs), xpar, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
+          if (!mbar_wait_warp(bar_xfull(x.at), x.par, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
           uint4 a[2], b[2];
           if (live) {
-            const uint32_t at = (uint32_t)(xs * sm.xslot);
+            const uint32_t at = (uint32_t)(x.at * sm.xslot);
             a[0] = lds_v4(xo_a + at); b[0] = lds_v4(xo_b + at);
             a[1] = lds_v4(xo_a + at + hstep); b[1] = lds_v4(xo_b + at + hstep);
           }
@@ -630,26 +802,27 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
                 bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
                 if constexpr (SINT) bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 4));
                 if constexpr (BR == BR_INT) hm = __hmax2(hm, bm);
-                const float m0 = __low2float(bm), m1 = __high2float(bm);
                 if constexpr (SINT) {
-                  const Sint4Scale s0 = sint4_scale(m0), s1 = sint4_scale(m1);
-                  wa[h] = sint4_codes8(a[h], s0); wb[h] = sint4_codes8(b[h], s1);
+                  const Sint4Scale sc(bm);
+                  wa[h] = sint4_codes8(a[h], sc.inv[0], sc.coarse); wb[h] = sint4_codes8(b[h], sc.inv[1], sc.coarse);
                   const int g = 2 * st + h;
-                  if (vs && g < p.G) p.sx[(size_t)g * p.Mpad + ms] = lc ? s1.s : s0.s;
+                  if (vs && g < p.G) p.sx[(size_t)g * p.Mpad + ms] = lc ? sc.s[1] : sc.s[0];
                 } else {
-                  int e0, e1;
-                  if constexpr (MAIN == MAIN_MXINT4) {
-                    e0 = mxint4_exponent(m0); e1 = mxint4_exponent(m1);
-                    wa[h] = mxint4_codes8(a[h], e0); wb[h] = mxint4_codes8(b[h], e1);
-                  } else if constexpr (MAIN == MAIN_MXFP) {
-                    const bool six = p.act6 != 0;
-                    e0 = mxfp8_exponent(m0, six); e1 = mxfp8_exponent(m1, six);
-                    wa[h] = mxfp_codes8(a[h], e0, six); wb[h] = mxfp_codes8(b[h], e1, six);
+                  constexpr int TOP = MAIN == MAIN_MXINT4 ? 2 : MAIN == MAIN_MXINT8 ? 6 : 8;
+                  constexpr int UP = MAIN == MAIN_MXINT4 ? 0xFF : MAIN == MAIN_MXINT8 ? 0x0F : 0;
+                  const PairScale<TOP, UP> ps(as_u32(bm));
+                  uint32_t bytes = ps.bytes;
+                  if (MAIN != MAIN_MXFP6 && ps.ok) {
+                    const __half2 i0 = as_half2(__byte_perm(ps.inv, 0, 0x1010)), i1 = as_half2(__byte_perm(ps.inv, 0, 0x3232));
+                    if constexpr (MAIN == MAIN_MXFP) { wa[h] = mxfp8_codes8(a[h], i0); wb[h] = mxfp8_codes8(b[h], i1); }
+                    else if constexpr (MAIN == MAIN_MXINT4) { wa[h] = mxint4_codes8(a[h], i0); wb[h] = mxint4_codes8(b[h], i1); }
+                    else if constexpr (MAIN == MAIN_MXINT8) { mxint8_codes8(a[h], i0, wa[h], da[h]); mxint8_codes8(b[h], i1, wb[h], db[h]); }
                   } else {
-                    e0 = mxint8_exponent(m0); e1 = mxint8_exponent(m1);
-                    mxint8_codes8(a[h], e0, wa[h], da[h]); mxint8_codes8(b[h], e1, wb[h], db[h]);
+                    const RareCodes rc = rare_codes<MAIN>(a[h], b[h], bm);
+                    wa[h] = rc.wa; wb[h] = rc.wb; da[h] = rc.da; db[h] = rc.db;
+                    bytes = rc.bytes;
                   }
-                  own |= ((uint32_t)(e0 + 127) | ((uint32_t)(e1 + 127) << 16)) << (8 * h);
+                  own |= bytes << (8 * h);
                 }
               }
               if constexpr (!SINT) {
@@ -684,8 +857,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
                 for (int h = 0; h < 2; ++h) { ca[h] = branch_codes8(a[h], sb_a, inv_a); cb[h] = branch_codes8(b[h], sb_b, inv_b); }
               }
             }
-            if (!mbar_wait_warp(bar_empty(slot), epar, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
-            const uint32_t at = (uint32_t)(slot * sm.slot);
+            if (!mbar_wait_warp(bar_empty(e.at), e.par, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
+            const uint32_t at = (uint32_t)(e.at * sm.slot);
             if (live) {
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
@@ -721,22 +894,21 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           // slot is refilled.)
           __syncwarp();
           if (lane == 0) {
-            if (decltype(BRP)::value) mbar_arrive(bar_afull(slot));
-            if (free_x) mbar_arrive(bar_xempty(xs));
+            if (decltype(BRP)::value) mbar_arrive(bar_afull(e.at));
+            if (free_x) mbar_arrive(bar_xempty(x.at));
           }
-          if (++xs == p.xslots) { xs = 0; xpar ^= 1; }
-          if (decltype(BRP)::value && ++slot == p.slots) { slot = 0; epar ^= 1; }
+          x.step(p.teams, p.xslots);
+          e.step(p.teams, p.slots);
         }
+        if (free_x) xr.step(p.nchunks, p.xslots);                // (kept slots are walked again)
+        if (decltype(BRP)::value) er.step(p.nchunks, p.slots);
         return true;
       };
       using Yes = std::true_type;
       using No = std::false_type;
       if constexpr (BR == BR_INT) {
-        const int xs0 = xs;
-        const uint32_t xpar0 = xpar;
         ok = walk(Yes(), No(), p.refetch != 0);
         if (!ok) break;
-        if (!p.refetch) { xs = xs0; xpar = xpar0; }              // the second walk reads the same slots
         // ---- the rows' maxima and scales: non-negative halves order like their bit patterns
         hm = __hmax2(hm, __shfl_xor_sync(0xffffffffu, hm, 4));
         int* mx = rowmax + buf * 64;
@@ -748,12 +920,12 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const float rm_a = __half2float(__ushort_as_half((unsigned short)mx[ra]));
         const float rm_b = __half2float(__ushort_as_half((unsigned short)mx[ra + 2]));
         const uint32_t after = buf == 0 ? 2 : buf - 1;           // two tiles on: every warp is past its last use
-        if (sx == 0 && lc < 2) rowmax[after * 64 + sr] = 0;
+        if (team == 0 && sx == 0 && lc < 2) rowmax[after * 64 + sr] = 0;
         buf = buf == 2 ? 0 : buf + 1;
         sb_a = rm_a == 0.f ? 1.f : __fdiv_rn(rm_a, p.qm);
         sb_b = rm_b == 0.f ? 1.f : __fdiv_rn(rm_b, p.qm);
         inv_a = __frcp_rn(sb_a); inv_b = __frcp_rn(sb_b);
-        if (sx == 0) {                                           // a4 reads the scale: its previous tile of this parity must be done
+        if (team == 0 && sx == 0) {                              // a4 reads the scale: its previous tile of this parity must be done
           ok = mbar_wait_warp(bar_tempty(tc & 1), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_QUANT);
           if (!ok) break;
           if (lc < 2) row_sb[(tc & 1) * 64 + sr] = lc ? sb_b : sb_a;
@@ -763,47 +935,61 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       } else {
         ok = walk(Yes(), std::integral_constant<bool, BR != BR_NONE>(), true);
       }
+      c0 = (c0 + p.teams - p.nchunks % p.teams) % p.teams;
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  if constexpr (BR == BR_MXFP) {
+    for (int w = 0; w < 2; ++w) {
+      const int4* unsettled = reinterpret_cast<const int4*>(smem + sm.off_l1) + w * MAX_UNSETTLED;
+      const int n = min(unsettled[0].x, MAX_UNSETTLED - 1);
+      for (int i = 1; i <= n; ++i)
+        settle_block<MAIN == MAIN_MXFP6>(p, unsettled[i], reinterpret_cast<float*>(smem + sm.off_l1 + 2 * MAX_UNSETTLED * 16));
+    }
+  }
   if (BR != BR_NONE && warp == 2) {
     tc_fence_after();
     tmem_dealloc(__shfl_sync(0xffffffffu, *tmem_slot, 0), (uint32_t)p.tmem_cols);
   }
 }
 
-// How a launch is cut.  Cost model in chunk times of a full complement of warps: a CTA's tiles times (its chunks, twice
-// where a tile is walked twice, plus what starting and finishing a tile costs); among equals the higher tile, which reads
-// the first factor less often.
+// How a launch is cut.  Cost model in rounds, a round being one chunk for every team: a CTA's tiles times (its rounds,
+// twice where a tile is walked twice, plus what starting and finishing a tile costs).
+// A team may only run ahead of the others as far as one-bit phases tell its slots apart: there are at least as many operand
+// slots as teams, and X slots for two rounds.
 bool plan_cut(int br, QuantParams& p, int sms) {
   const int walks = br == BR_INT ? 2 : 1, room = 227 * 1024 - 1024;
   double best = 1e30;
   QuantParams out = p;
   for (int groups = 8; groups >= 1; --groups) {
     if (g_lq_quant_warps > 0 && groups != std::min(8, g_lq_quant_warps)) continue;
-    for (int stages = std::min(QWARPS / groups, p.nst); stages >= 1; --stages) {
+    for (int stages = 1; stages <= std::min(QWARPS / groups, p.nst); ++stages) {
       if (g_lq_quant_ctas > 0 && stages != g_lq_quant_ctas) continue;
       QuantParams c = p;
       c.groups = groups; c.stages = stages;
       c.ntiles = lq_ceil_div(p.M, 8 * groups);
       c.nchunks = lq_ceil_div(p.nst, stages);
-      c.xslots = 0;
-      // operand slots first, then as many chunks of X as fit; an integer branch would rather hold a whole tile of X
-      const int want = br == BR_INT ? c.nchunks : 4;
-      for (int slots = br == BR_NONE ? 1 : MAX_SLOTS; slots >= (br == BR_NONE ? 1 : 2) && c.xslots < want; --slots) {
-        const QuantSmem s = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, slots, 0);
-        const int fit = std::min(MAX_XSLOTS, (room - s.total) / s.xslot);
-        if (fit > c.xslots && fit >= 2) { c.xslots = fit; c.slots = slots; }
+      for (c.teams = std::min(std::min(QWARPS / (groups * stages), c.nchunks), MAX_SLOTS); c.teams >= 1; --c.teams) {
+        c.xslots = 0;
+        // operand slots first, then as many chunks of X as fit; an integer branch would rather hold a whole tile of X
+        const int want = br == BR_INT ? c.nchunks : 2 * c.teams + 2, least = std::max(2, 2 * c.teams - 1);
+        for (int slots = br == BR_NONE ? 1 : MAX_SLOTS; slots >= (br == BR_NONE ? 1 : std::max(2, c.teams)) && c.xslots < want; --slots) {
+          const QuantSmem s = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, slots, 0);
+          const int fit = std::min(MAX_XSLOTS, (room - s.total) / s.xslot);
+          if (fit > c.xslots && fit >= least) { c.xslots = fit; c.slots = slots; }
+        }
+        if (c.xslots == 0) continue;
+        c.xslots = std::min(c.xslots, std::max(least, 2 * c.nchunks));
+        c.refetch = br == BR_INT && c.xslots < c.nchunks;
+        c.smem = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, c.slots, c.xslots).total + 1024;
+        const int warps = groups * stages * c.teams;
+        const double round = 0.4 + 0.6 * warps / QWARPS;
+        const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + 1.0) + 3.0;
+        if (cost < best - 1e-9) { best = cost; out = c; }
+        break;
       }
-      if (c.xslots < 2) continue;
-      c.xslots = std::min(c.xslots, 2 * c.nchunks);
-      c.refetch = br == BR_INT && c.xslots < c.nchunks;
-      c.smem = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, c.slots, c.xslots).total + 1024;
-      const double chunk = 0.4 + 0.6 * groups * stages / QWARPS;
-      const double cost = lq_ceil_div(c.ntiles, sms) * (c.nchunks * walks * chunk + 1.0) + 3.0;
-      if (cost < best) { best = cost; out = c; }
     }
   }
   p = out;
@@ -821,6 +1007,16 @@ cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, i
     attr_set[dev & 63] = true;
   }
   if (!plan_cut(BR, p, sms)) return cudaErrorInvalidConfiguration;
+  // Floating-point branches: a tile's stages alternate over up to four accumulators, which are added in fp32 at the end
+  // (each costs a4 a trip to tensor memory per 16 columns: not more than 128 columns of them).  Tensor memory holds two
+  // such sets - one where every CTA has a single tile - and the scale bytes' columns.
+  const int cols = p.rn * p.bplanes, extra = BR == BR_MXFP || BR == BR_MXINT ? 16 : 0;
+  p.sets = p.ntiles <= sms ? 1 : 2;
+  p.nacc = BR == BR_INT ? 1 : BR == BR_F16 || cols <= 32 ? 4 : cols <= 64 ? 2 : 1;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < p.sets * p.nacc * cols + extra) p.tmem_cols *= 2;
+  // what the chains of fp32 sums and the bits of the products make of the deviation from the defining order
+  p.dev *= (0.3f + (float)p.K / (1000.f * p.nacc)) * 0x1p-22f;
   CUtensorMap tmX;
   if (lq_make_tmap_bytes(&tmX, const_cast<void*>(X), (uint64_t)p.M, (uint64_t)p.K * 2, (uint32_t)(8 * p.groups)) != LQ_OK)
     return cudaErrorInvalidValue;
@@ -839,25 +1035,21 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   p.nst = L->Kpad / LQ_KSTAGE;
   p.qx8 = A->d_qx8; p.sx = A->d_sx; p.sfa = A->d_sfa;
   p.qb = g_lq_store_qb ? A->d_qb : nullptr;
-  p.sXb = A->d_sXb; p.sL1 = L->d_sL1; p.sfl1 = L->d_sfl1;
+  p.sXb = A->d_sXb; p.sL1 = L->d_sL1; p.l1c = L->d_L1c; p.sfl1 = L->d_sfl1;
   p.sft = A->d_sft; p.tq = A->d_tq; p.sT = A->d_sT;
   p.r = L->r; p.rn = lq_l1_rows(L);
   p.bplanes = lq_l1_planes(L);
   p.tq_stride = A->tq_stride;
-  // Floating-point branches: a tile's stages alternate over two to four accumulators, which are added in fp32 at the end;
-  // tensor memory holds two such sets and the scale bytes' columns.
-  p.nacc = L->integer_branch ? 1 : p.rn <= 48 ? 4 : p.rn <= 112 ? 2 : 1;
-  if (L->f16_branch && p.rn > 48) p.nacc = 4;
-  p.tmem_cols = 32;
-  while (p.tmem_cols < 2 * p.nacc * p.rn + ((L->mxfp || L->a8) ? 16 : 0)) p.tmem_cols *= 2;
-  p.act6 = (L->mxfp && L->cfg.act_fmt == LQ_ACT_MXFP6) ? 1 : 0;
+  p.dev = L->cfg.branch == LQ_BRANCH_MXFP8 ? 1.f : L->cfg.branch == LQ_BRANCH_MXFP6 ? 0.5f : 0.2f;
   p.qm = abits > 0 ? (float)((1 << (abits - 1)) - 1) : 0.f;
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device) != cudaSuccess) return LQ_ERR_CUDA;
   cudaError_t e;
-  if (L->mxfp) e = L->r > 0 ? launch_quant<MAIN_MXFP, BR_MXFP>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXFP, BR_NONE>(X, L->tmL1, p, sms, st);
+  if (L->mxfp && L->cfg.act_fmt == LQ_ACT_MXFP6)
+    e = L->r > 0 ? launch_quant<MAIN_MXFP6, BR_MXFP>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXFP6, BR_NONE>(X, L->tmL1, p, sms, st);
+  else if (L->mxfp) e = L->r > 0 ? launch_quant<MAIN_MXFP, BR_MXFP>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXFP, BR_NONE>(X, L->tmL1, p, sms, st);
   else if (L->a8) e = L->r > 0 ? launch_quant<MAIN_MXINT8, BR_MXINT>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXINT8, BR_NONE>(X, L->tmL1, p, sms, st);
   else if (L->mx)
     e = L->f16_branch ? launch_quant<MAIN_MXINT4, BR_F16>(X, L->tmL1, p, sms, st)
