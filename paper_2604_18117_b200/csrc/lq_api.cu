@@ -415,10 +415,12 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
   const int K = L->K, N = L->N, r = L->r, G = L->G, Kpad = L->Kpad, Npad = L->Npad, Gpad = L->Gpad, rn = lq_l1_rows(L);
   lq_status st;
   try {
+    std::vector<int> wrow(Npad), srow(Npad);                     // places of column n in the weight operand and the vectors
+    for (int n = 0; n < Npad; ++n) { wrow[n] = L->mx ? n : lq_col_slot(n); srow[n] = L->mx ? n : lq_colscale_slot(n); }
     std::vector<uint8_t> w8((size_t)Npad * Kpad, lq_encode_code_host(0, L->main_kind));
     for (int k = 0; k < K; ++k)
       for (int n = 0; n < N; ++n)
-        w8[(size_t)n * Kpad + k] = L->mxfp ? L->Wq8h[(size_t)k * N + n] : lq_encode_code_host(L->Wq[(size_t)k * N + n], L->main_kind);
+        w8[(size_t)wrow[n] * Kpad + k] = L->mxfp ? L->Wq8h[(size_t)k * N + n] : lq_encode_code_host(L->Wq[(size_t)k * N + n], L->main_kind);
     if ((st = upload(&L->d_Wq8, w8)) != LQ_OK) return st;
     if (L->mx) {
       // E8M0 bytes (exponent + 127) in the layout the block-scaled MMA reads from tensor memory; 127 = 2^0 for padding
@@ -433,11 +435,11 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
     } else {
       std::vector<float> swf((size_t)Gpad * Npad, 0.f);
       for (int g = 0; g < G; ++g)
-        for (int n = 0; n < N; ++n) swf[(size_t)g * Npad + n] = h2f(L->sw[(size_t)g * N + n]);
+        for (int n = 0; n < N; ++n) swf[(size_t)g * Npad + srow[n]] = h2f(L->sw[(size_t)g * N + n]);
       if ((st = upload(&L->d_sw, swf)) != LQ_OK) return st;
     }
     std::vector<float> bias((size_t)Npad, 0.f);
-    if (L->has_bias) for (int n = 0; n < N; ++n) bias[n] = h2f(L->bias[n]);
+    if (L->has_bias) for (int n = 0; n < N; ++n) bias[srow[n]] = h2f(L->bias[n]);
     if ((st = upload(&L->d_bias, bias)) != LQ_OK) return st;
     std::vector<float> s1(LQ_MAX_RANK, 1.f), s2((size_t)Npad, 1.f);
     std::vector<uint8_t> l2c((size_t)Npad * LQ_RCONT, 0);
@@ -447,9 +449,9 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
         for (int j = 0; j < r; ++j) l1c[(size_t)j * Kpad + k] = (uint8_t)L->L1q[(size_t)k * r + j];
       if ((st = upload(&L->d_L1c, l1c)) != LQ_OK) return st;
       for (int j = 0; j < r; ++j) s1[j] = L->sL1[j];
-      for (int n = 0; n < N; ++n) s2[n] = L->sL2[n];
+      for (int n = 0; n < N; ++n) s2[srow[n]] = L->sL2[n];
       for (int j = 0; j < r; ++j)
-        for (int n = 0; n < N; ++n) l2c[(size_t)n * LQ_RCONT + j] = (uint8_t)L->L2q[(size_t)j * N + n];
+        for (int n = 0; n < N; ++n) l2c[(size_t)wrow[n] * LQ_RCONT + j] = (uint8_t)L->L2q[(size_t)j * N + n];
     } else if ((L->mxfp || L->a8) && r > 0) {
       // The first factor's elements as E4M3 bytes (8-bit integer codes: a plane of hi digits, then one of lo digits) and its
       // E8M0 scale bytes along K, one chunk of (at most) 128 rows x 4 blocks per stage
@@ -523,7 +525,7 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
       if ((st = upload(&L->d_L1c, l1c)) != LQ_OK) return st;
       uint16_t* c16 = (uint16_t*)l2c.data();
       for (int j = 0; j < r; ++j)
-        for (int n = 0; n < N; ++n) c16[(size_t)n * (LQ_RCONT / 2) + j] = L->L2h[(size_t)j * N + n];
+        for (int n = 0; n < N; ++n) c16[(size_t)wrow[n] * (LQ_RCONT / 2) + j] = L->L2h[(size_t)j * N + n];
     }
     if ((st = upload(&L->d_sL1, s1)) != LQ_OK) return st;
     if ((st = upload(&L->d_sL2, s2)) != LQ_OK) return st;
@@ -760,7 +762,7 @@ extern "C" lq_status lq_act_export(const lq_act* A, int8_t* qx, uint16_t* sx, in
       CUDA_OK(cudaMemcpy(h.data(), A->d_sx, h.size() * sizeof(float), cudaMemcpyDeviceToHost));
       for (int m = 0; m < M; ++m)
         for (int g = 0; g < G; ++g) {
-          __half v = __float2half_rn(h[(size_t)g * Mp + m]);   // exact: the value is an fp16 number
+          __half v = __float2half_rn(h[(size_t)g * Mp + lq_row_slot(m)]);   // exact: the value is an fp16 number
           sx[(size_t)m * G + g] = __half_raw(v).x;
         }
     }
@@ -800,7 +802,11 @@ extern "C" lq_status lq_act_export(const lq_act* A, int8_t* qx, uint16_t* sx, in
       const int nbR = lq_ceil_div(r, LQ_MX_BLOCK);
       for (int m = 0; m < M; ++m)
         for (int c = 0; c < nbR; ++c) sT[(size_t)m * nbR + c] = (float)((int)h[lq_sf_offset(m, c, 128)] - 127);
-    } else if (sT && r > 0) CUDA_OK(cudaMemcpy(sT, A->d_sT, M * sizeof(float), cudaMemcpyDeviceToHost));
+    } else if (sT && r > 0) {
+      std::vector<float> h(Mp);
+      CUDA_OK(cudaMemcpy(h.data(), A->d_sT, Mp * sizeof(float), cudaMemcpyDeviceToHost));
+      for (int m = 0; m < M; ++m) sT[m] = h[A->mx ? m : lq_row_slot(m)];
+    }
   } catch (const std::bad_alloc&) { return LQ_ERR_ALLOC; }
   return LQ_OK;
 }

@@ -7,25 +7,29 @@
 // scale per block of 64 values on BOTH operands, so every 64-deep partial product needs its
 // own rank-1 scale before it may be summed.)
 //
-// Shape of the kernel (persistent, one CTA per SM, warp-specialised, 18 warps):
-//   warp 0      TMA producer: operand tiles (two groups = 128 bytes of K per stage row) and
-//               the two groups' scale vectors, all signalled on the stage's "full" barrier
-//   warp 1      owns tensor memory; issues tcgen05.mma: each group of 64 codes is two K=32
-//               MMAs into a FRESH 128 x 128 accumulator.  The (up to) two groups of an operand
-//               stage fill one PAIR of accumulators that is handed over with one commit; two
-//               pairs alternate, so the issuer works a stage ahead of the drain.  The loop is
-//               warp-uniform (operands live in uniform registers) and one elected lane issues
-//   warps 2-17  drain: each warp owns 32 rows x 32 columns of the tile.  A group's accumulator
-//               slice is fetched as two tcgen05.ld.16x256b (256 bits per lane and access), ONE
-//               wait, and the accumulator is handed back at once; the next group's halves are
-//               requested as the registers of the current one are consumed, so the fetch runs
-//               under the arithmetic: acc += P * (sx * sw), packed f32x2, fp32 registers.  After
-//               the last group: bias is already in (it is the start value), convert, exchange
-//               inside each quad so that a lane holds 16 contiguous bytes of a row, store
-// The per-group arithmetic is the bound: 2 fp32 operations per output and group on 128 lanes
-// per SM, against 8192 MACs per clock on the tensor pipe - 256 clocks of drain for 128 clocks
-// of tensor work per 128 x 128 x 64 block.  Work is cut in 128 x 128 tiles; every CTA takes a
-// contiguous, balanced run of them, row block major.
+// Shape of the kernel (persistent, one CTA per SM, warp-specialised, 12 warps):
+//   warp 0      TMA producer: operand tiles (two groups = 128 bytes of K per stage row), the two groups' scale vectors and,
+//               with a tile's first stage, the bias, all signalled on the stage's "full" barrier
+//   warp 1      owns tensor memory; issues tcgen05.mma: each group of 64 codes is two K=32 MMAs into a FRESH 128 x 128
+//               accumulator.  A stage's two groups fill one PAIR of accumulators, each as soon as the drain has read it out,
+//               and are handed over with one commit; two pairs alternate
+//   warps 4-11  drain: each warp owns 32 rows x 64 columns of the tile.  A group's slice is four tcgen05.ld.16x256b.x4; a
+//               whole group is in flight into one register buffer while the one before is consumed from the other:
+//               acc += P * (sx * sw), packed f32x2, fp32 registers.  An accumulator goes back as soon as it sits in
+//               registers.  The next tile's first group is requested before the epilogue
+// What bounds it: the FP32 pipe's operand delivery, and the hand-shakes around it.  Per group and scheduler 64 packed
+// products (two operands: 2 clocks each, measured) and 64 packed FMAs (three: 4 clocks) are 384 clocks, the tensor pipe
+// needs 128; the kernel takes 530.  So everything that is not arithmetic is kept out of the drain's instruction stream: two
+// wide warps per scheduler instead of four narrow ones, no wait or arrival for the scale vectors (they live in a ring deep
+// enough that the accumulators' hand-shakes imply theirs), one wait per stage, 216 registers per drain thread, partly
+// taken over from the other four warps (setmaxnreg).  M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 85 / 96 us with sixteen
+// narrow warps, 80 / 89 with one commit per group, 75.5 / 80 now.  (Scalar FMAs, 3 clocks for two, lose what they gain to
+// their issue slots: 89 / 101 us.)
+// Orders of rows and columns (lq_internal.h) are chosen for the drain's fragments: the columns of the tile are permuted in
+// the weight operand so that a lane's 16 columns of a row are neighbours in Y - the epilogue converts and stores, no
+// exchange - and the scale vectors are permuted so that a lane's come in one (rows) and four (columns) 16-byte loads
+// without bank conflicts.
+// Work is cut in 128 x 128 tiles; every CTA takes a contiguous, balanced run of them, row block major.
 // The 4-bit codes ride in E4M3 operands (integers up to 7 are exact, fp32 accumulation of
 // |sum| <= 3136 is exact); the branch's 8-bit codes use kind::i8 (exact int32), the fp16
 // reference branch kind::f16.
@@ -51,28 +55,30 @@ using namespace lqdev;
 
 constexpr int UNIT = LQ_BN;                        // 128 output columns per tile
 constexpr int NSTAGE = 4;                          // operand ring depth (a power of two: ring positions are masks)
-constexpr int NTBUF = 2;                           // ring of accumulator PAIRS in tensor memory: a pair = the (up to) two groups of one operand stage, 2 x 128 columns
+constexpr int NPAIR = 2;                           // ring of accumulator pairs in tensor memory, a stage's two groups: 2 x 2 x 128 columns
 constexpr int TCOLS = 128;                         // columns per accumulator
 constexpr int STAGE_A_BYTES = LQ_BM * LQ_KSTAGE;   // 16 KB
 constexpr int STAGE_B_BYTES = UNIT * LQ_KSTAGE;    // 16 KB
 constexpr int STAGE_BYTES = STAGE_A_BYTES + STAGE_B_BYTES;
 constexpr int SC_GROUP_FLOATS = LQ_BM + UNIT;      // sx[128] then sw[128]
-constexpr int SC_STAGE_BYTES = 2 * SC_GROUP_FLOATS * 4;   // two groups
-constexpr int NUM_DRAIN_WARPS = 16;
-constexpr int FIRST_DRAIN_WARP = 2;
+constexpr int SC_STAGE_BYTES = (2 * SC_GROUP_FLOATS + UNIT) * 4;   // two groups, bias[128] (a tile's first stage)
+constexpr int SC_RING = 8;                         // slots of the scale ring
+constexpr int NUM_DRAIN_WARPS = 8;
+constexpr int FIRST_DRAIN_WARP = 4;                // the first warpgroup: TMA, MMA, two idle warps
 constexpr int GEMM_THREADS = (FIRST_DRAIN_WARP + NUM_DRAIN_WARPS) * 32;
-constexpr int WCOLS = 32;                          // columns per drain warp
+constexpr int WCOLS = 64;                          // columns per drain warp
+// 12 warps are launched with 168 registers a thread (64512 in all); 128 x 56 + 256 x 216 = 62464
+constexpr int LEAN_REGS = 56, DRAIN_REGS = 216;
 constexpr int SMEM_BAR_BYTES = 256;
-constexpr int SMEM_BYTES = 1024 /*alignment slack*/ + NSTAGE * STAGE_BYTES + NSTAGE * SC_STAGE_BYTES + SMEM_BAR_BYTES;
+constexpr int SMEM_BYTES = 1024 /*alignment slack*/ + NSTAGE * STAGE_BYTES + SC_RING * SC_STAGE_BYTES + SMEM_BAR_BYTES;
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 static_assert(STAGE_BYTES % 1024 == 0, "stages must keep the 1024-byte alignment of the swizzled tiles");
-static_assert((NSTAGE & (NSTAGE - 1)) == 0 && (NTBUF & (NTBUF - 1)) == 0, "ring sizes must be powers of two");
+static_assert((NSTAGE & (NSTAGE - 1)) == 0 && (NPAIR & (NPAIR - 1)) == 0, "ring sizes must be powers of two");
 
 struct GemmParams {
-  int M, N, Mpad, Npad, G;
-  int n_stages_main;      // ceil(G / 2)
-  int branch_mmas;        // 0: no branch; else MMAs of the branch stage (32 bytes of r each)
-  int branch_f16;         // branch operands are halves (kind::f16) instead of int8 (kind::i8)
+  int M, N, Mpad, Npad;
+  int n_stages_main;      // Kpad / 128 (an odd last group's partner has zero codes and scales)
+  int branch_mmas;        // MMAs of the branch stage (32 bytes of r each)
   int tiles_m, units_n;
   const float* sx;        // [Gpad][Mpad]
   const float* sw;        // [Gpad][Npad]
@@ -84,43 +90,55 @@ struct GemmParams {
   int32_t* status;
 };
 
-// One accumulator slice of 16 rows x 32 columns in the layout of tcgen05.ld.16x256b (the accumulator-fragment layout
-// of mma.sync m16n8: with g = lane / 4 and t = lane % 4, registers 4j .. 4j+3 hold row g, columns 8j + 2t and
-// 8j + 2t + 1, then row g + 8, the same columns): acc += P * (sx * sw).  This shape moves 256 bits per lane and access;
-// the one-row-per-thread shape (32x32b) moves 32 and was measured at 60-80 bytes per clock and SM, which capped the
-// whole kernel.  INT: the accumulator holds int32 (kind::i8); |P| < 2^22, so adding 1.5 * 2^23 in the integer domain
-// and subtracting it in fp32 converts exactly without the conversion pipe.
+// One group's slice of a drain warp, two accumulator slices of 16 rows x 64 columns in the layout of tcgen05.ld.16x256b
+// (the accumulator-fragment layout of mma.sync m16n8: with g = lane / 4 and t = lane % 4, registers 4j .. 4j+3 of a
+// slice hold row g, columns 8j + 2t and 8j + 2t + 1, then row g + 8, the same columns): acc += P * (sx * sw).
+// INT: the accumulator holds int32 (kind::i8); |P| < 2^22, so adding 1.5 * 2^23 in the integer domain and subtracting it
+// in fp32 converts exactly without the conversion pipe.
+typedef uint32_t Frag[16];                            // 16 rows x 32 columns
 template <bool INT>
-__device__ __forceinline__ void drain_frag(const uint32_t (&v)[16], float2* acc, float sx_lo, float sx_hi, const float2 (&sw)[4]) {
-  const float2 sl = make_float2(sx_lo, sx_lo), sh = make_float2(sx_hi, sx_hi);
+__device__ __forceinline__ float2 fragment_pair(uint32_t a, uint32_t b) {
+  if constexpr (INT)
+    return make_float2(__int_as_float((int)a + 0x4B400000) - 12582912.0f, __int_as_float((int)b + 0x4B400000) - 12582912.0f);
+  else
+    return make_float2(__uint_as_float(a), __uint_as_float(b));
+}
+struct Scales {                                       // a lane's four row scales and 16 column scales of a group
+  float4 sx, sw[4];
+};
+__device__ __forceinline__ Scales load_scales(const float* sc, int row_at, int col_at) {
+  Scales v;
+  v.sx = *reinterpret_cast<const float4*>(sc + row_at);                     // rows g, g + 8, g + 16, g + 24
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float2 p0, p1;
-    if constexpr (INT) {
-      p0 = make_float2(__int_as_float((int)v[4 * j + 0] + 0x4B400000) - 12582912.0f,
-                       __int_as_float((int)v[4 * j + 1] + 0x4B400000) - 12582912.0f);
-      p1 = make_float2(__int_as_float((int)v[4 * j + 2] + 0x4B400000) - 12582912.0f,
-                       __int_as_float((int)v[4 * j + 3] + 0x4B400000) - 12582912.0f);
-    } else {
-      p0 = make_float2(__uint_as_float(v[4 * j + 0]), __uint_as_float(v[4 * j + 1]));
-      p1 = make_float2(__uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+  for (int k = 0; k < 4; ++k) v.sw[k] = *reinterpret_cast<const float4*>(sc + LQ_BM + col_at + 16 * k);
+  return v;
+}
+template <bool INT>
+__device__ __forceinline__ void drain_group(const Frag (&v)[4], float2 (&acc)[2][16], const Scales& sc) {
+  const float4 sx = sc.sx;
+  const float2 s0 = make_float2(sx.x, sx.x), s1 = make_float2(sx.y, sx.y), s2 = make_float2(sx.z, sx.z), s3 = make_float2(sx.w, sx.w);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float4 w = sc.sw[k];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int j = 2 * k + e, c = j >> 2, q = 4 * (j & 3);
+      const float2 sw = e ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
+      acc[0][2 * j] = __ffma2_rn(fragment_pair<INT>(v[2 * c][q], v[2 * c][q + 1]), __fmul2_rn(s0, sw), acc[0][2 * j]);
+      acc[0][2 * j + 1] = __ffma2_rn(fragment_pair<INT>(v[2 * c][q + 2], v[2 * c][q + 3]), __fmul2_rn(s1, sw), acc[0][2 * j + 1]);
+      acc[1][2 * j] = __ffma2_rn(fragment_pair<INT>(v[2 * c + 1][q], v[2 * c + 1][q + 1]), __fmul2_rn(s2, sw), acc[1][2 * j]);
+      acc[1][2 * j + 1] = __ffma2_rn(fragment_pair<INT>(v[2 * c + 1][q + 2], v[2 * c + 1][q + 3]), __fmul2_rn(s3, sw), acc[1][2 * j + 1]);
     }
-    acc[2 * j + 0] = __ffma2_rn(p0, __fmul2_rn(sl, sw[j]), acc[2 * j + 0]);
-    acc[2 * j + 1] = __ffma2_rn(p1, __fmul2_rn(sh, sw[j]), acc[2 * j + 1]);
   }
 }
-
-// 4 x 4 transpose across the four lanes of a quad: afterwards v[s] of lane t is what v[t] of lane s was.
-__device__ __forceinline__ void quad_transpose(uint32_t (&v)[4], int t) {
-  const bool hi2 = (t & 2) != 0, hi1 = (t & 1) != 0;
-  uint32_t y0 = __shfl_xor_sync(0xffffffffu, hi2 ? v[0] : v[2], 2);
-  uint32_t y1 = __shfl_xor_sync(0xffffffffu, hi2 ? v[1] : v[3], 2);
-  if (hi2) { v[0] = y0; v[1] = y1; } else { v[2] = y0; v[3] = y1; }
-  y0 = __shfl_xor_sync(0xffffffffu, hi1 ? v[0] : v[1], 1);
-  y1 = __shfl_xor_sync(0xffffffffu, hi1 ? v[2] : v[3], 1);
-  if (hi1) { v[0] = y0; v[2] = y1; } else { v[1] = y0; v[3] = y1; }
+__device__ __forceinline__ void fetch_group(uint32_t taddr, Frag (&v)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) tmem_ld_16x256b_x4(taddr + ((uint32_t)(16 * (i & 1)) << 16) + 32 * (i >> 1), v[i]);
 }
 
+enum { BRANCH_NONE = 0, BRANCH_I8 = 1, BRANCH_F16 = 2 };
+
+template <int BRANCH>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
@@ -131,22 +149,21 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const uint32_t sm_stage = base;
   const uint32_t sm_sc = base + NSTAGE * STAGE_BYTES;
   const float* sc_ptr = reinterpret_cast<const float*>(smem + NSTAGE * STAGE_BYTES);
-  const uint32_t sm_bar = sm_sc + NSTAGE * SC_STAGE_BYTES;
-  uint8_t* bar_ptr = smem + NSTAGE * STAGE_BYTES + NSTAGE * SC_STAGE_BYTES;
+  const uint32_t sm_bar = sm_sc + SC_RING * SC_STAGE_BYTES;
+  uint8_t* bar_ptr = smem + NSTAGE * STAGE_BYTES + SC_RING * SC_STAGE_BYTES;
   // barrier map (8 bytes each)
   auto bar_full = [&](int s) { return sm_bar + 8u * (uint32_t)s; };                        // operands + scales landed
   auto bar_empty = [&](int s) { return sm_bar + 8u * (uint32_t)(NSTAGE + s); };           // MMAs of the stage retired
-  auto bar_sempty = [&](int s) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + s); };      // drain done with the scales
-  auto bar_tfull = [&](int b) { return sm_bar + 8u * (uint32_t)(3 * NSTAGE + b); };
-  auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(3 * NSTAGE + NTBUF + b); };
-  constexpr int NBAR = 3 * NSTAGE + 2 * NTBUF;
+  auto bar_tfull = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + b); };
+  auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + NPAIR + b); };
+  constexpr int NBAR = 2 * NSTAGE + 3 * NPAIR;
   static_assert(NBAR * 8 + 16 <= SMEM_BAR_BYTES, "barrier area too small");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + NBAR * 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + NBAR * 8 + 8);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // provably warp-uniform
   const int lane = threadIdx.x & 31;
-  const int stages_per_tile = p.n_stages_main + (p.branch_mmas > 0 ? 1 : 0);
+  const int stages_per_tile = p.n_stages_main + (BRANCH != BRANCH_NONE ? 1 : 0);
   // this CTA's contiguous run of 128 x 128 tiles, row block major
   const long long units = (long long)p.tiles_m * p.units_n;
   const int u_begin = (int)((units * blockIdx.x) / gridDim.x);
@@ -156,9 +173,9 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int s = 0; s < NSTAGE; ++s) {
       mbar_init(bar_full(s), 1);
       mbar_init(bar_empty(s), 1);
-      mbar_init(bar_sempty(s), NUM_DRAIN_WARPS);
     }
-    for (int b = 0; b < NTBUF; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), NUM_DRAIN_WARPS); }
+    for (int b = 0; b < NPAIR; ++b) mbar_init(bar_tfull(b), 1);
+    for (int b = 0; b < 2 * NPAIR; ++b) mbar_init(bar_tempty(b), NUM_DRAIN_WARPS);
     *abort_flag = 0;
     mbar_init_fence();
   }
@@ -174,234 +191,218 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     : warp == FIRST_DRAIN_WARP + NUM_DRAIN_WARPS - 1 ? (int)TL_DRAIN_LAST : -1)
                  : -1);
 
-  if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer
-    uint32_t it = 0, armed = 0;
-    bool ok = true;
-    for (int u = u_begin; u < u_end && ok; ++u) {
-      const int mb = u / p.units_n, nu = u - mb * p.units_n;
-      const int m0 = mb * LQ_BM, n0 = nu * UNIT;
-      for (int s = 0; s < stages_per_tile && ok; ++s, ++it) {
-        const int st = it & (NSTAGE - 1);
-        const uint32_t par = ((it / NSTAGE) & 1) ^ 1;
-        ok = mbar_wait_warp(bar_empty(st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
-        if (!ok) break;
-        ok = mbar_wait_warp(bar_sempty(st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
-        if (!ok) break;
-        LQ_TL(EV_P_SLOT_FREE, s);
-        const uint32_t a_dst = sm_stage + st * STAGE_BYTES, b_dst = a_dst + STAGE_A_BYTES;
-        const uint32_t sc_dst = sm_sc + st * SC_STAGE_BYTES;
-        const uint32_t full = bar_full(st);
-        const bool is_main = s < p.n_stages_main;
-        const int ngroups = is_main ? ((2 * s + 1 < p.G) ? 2 : 1) : 1;
-        const uint32_t tx = STAGE_BYTES + ngroups * SC_GROUP_FLOATS * 4;
-        if (elect_one()) {
-          mbar_expect_tx(full, tx);
-          if (is_main) {
-            tma_load_2d(a_dst, &tmA, s * LQ_KSTAGE, m0, full);
-            tma_load_2d(b_dst, &tmB, s * LQ_KSTAGE, n0, full);
-            for (int q = 0; q < ngroups; ++q) {
-              const size_t g = (size_t)(2 * s + q);
-              bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4, p.sx + g * p.Mpad + m0, LQ_BM * 4, full);
-              bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4 + LQ_BM * 4, p.sw + g * p.Npad + n0, UNIT * 4, full);
-            }
-          } else {
-            tma_load_2d(a_dst, &tmT, 0, m0, full);
-            tma_load_2d(b_dst, &tmL2, 0, n0, full);
-            bulk_load(sc_dst, p.sT + m0, LQ_BM * 4, full);
-            bulk_load(sc_dst + LQ_BM * 4, p.sL2 + n0, UNIT * 4, full);
-          }
-        }
-        __syncwarp();
-        ++armed;
-        LQ_TL(EV_P_ISSUED, s);
-      }
-    }
-    if (!ok && lane == 0) {
-      // aborting: give the copies already issued a bounded time to land before the CTA's shared memory goes away
-      const uint32_t n = armed < (uint32_t)NSTAGE ? armed : (uint32_t)NSTAGE;
-      for (uint32_t i = 1; i <= n; ++i) {
-        const uint32_t j = armed - i;
-        mbar_settle(bar_full(j % NSTAGE), (j / NSTAGE) & 1);
-      }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    uint32_t it = 0;
-    bool ok = true;
-    const uint32_t shape = idesc_shape(UNIT);
-    for (int u = u_begin; u < u_end && ok; ++u) {
-      for (int s = 0; s < stages_per_tile && ok; ++s, ++it) {
-        const int st = it & (NSTAGE - 1);
-        ok = mbar_wait_warp(bar_full(st), (it / NSTAGE) & 1, abort_flag, p.status, LQ_STAGE_MMA);
-        if (!ok) break;
-        tc_fence_after();
-        LQ_TL(EV_M_STAGE_FULL, s);
-        const uint32_t a_addr = sm_stage + st * STAGE_BYTES, b_addr = a_addr + STAGE_A_BYTES;
-        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(b_addr);
-        const bool is_main = s < p.n_stages_main;
-        const int ngroups = is_main ? ((2 * s + 1 < p.G) ? 2 : 1) : 1;
-        // the stage's (up to) two groups go to the two accumulators of one pair; ONE commit hands the pair over
-        const int pb = it & (NTBUF - 1);
-        ok = mbar_wait_warp(bar_tempty(pb), ((it / NTBUF) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
-        if (!ok) break;
-        tc_fence_after();
-        LQ_TL(EV_M_ACC_FREE, s);
-        const uint32_t d = tmem_base + pb * (2 * TCOLS);
-        if (elect_one()) {
-          if (is_main) {
-            for (int q = 0; q < ngroups; ++q) {
-              const uint64_t off = (uint64_t)((q * 64) >> 4);
-              tc_mma<TC_F8>(d + q * TCOLS, adesc + off, bdesc + off, IDESC_F8 | shape, 0u);
-              tc_mma<TC_F8>(d + q * TCOLS, adesc + off + 2, bdesc + off + 2, IDESC_F8 | shape, 1u);
-            }
-          } else {
-            for (int j = 0; j < p.branch_mmas; ++j) {
-              const uint64_t off = (uint64_t)((j * 32) >> 4);
-              if (p.branch_f16) tc_mma<TC_F16>(d, adesc + off, bdesc + off, IDESC_F16 | shape, (uint32_t)j);
-              else tc_mma<TC_I8>(d, adesc + off, bdesc + off, IDESC_I8 | shape, (uint32_t)j);
+  if (warp < FIRST_DRAIN_WARP) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(LEAN_REGS));
+    if (warp == 0) {
+      // ------------------------------------------------------------------ TMA producer
+      uint32_t it = 0, armed = 0;
+      bool ok = true;
+      for (int u = u_begin; u < u_end && ok; ++u) {
+        const int mb = u / p.units_n, nu = u - mb * p.units_n;
+        const int m0 = mb * LQ_BM, n0 = nu * UNIT;
+        for (int s = 0; s < stages_per_tile && ok; ++s, ++it) {
+          const int st = it & (NSTAGE - 1);
+          const uint32_t par = ((it / NSTAGE) & 1) ^ 1;
+          ok = mbar_wait_warp(bar_empty(st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
+          if (!ok) break;
+          // (Nothing says that the drain is done with the slot's old scale vectors, eight stages back, and nothing has to: the
+          // MMAs that have just retired, four stages back, had to wait for the accumulators of six stages back to be in the
+          // drain's registers, and by then it had used up the scales of the stages before.)
+          LQ_TL(EV_P_SLOT_FREE, s);
+          const uint32_t a_dst = sm_stage + st * STAGE_BYTES, b_dst = a_dst + STAGE_A_BYTES;
+          const uint32_t sc_dst = sm_sc + (it & (SC_RING - 1)) * SC_STAGE_BYTES;
+          const uint32_t full = bar_full(st);
+          const bool is_main = s < p.n_stages_main;
+          const int ngroups = is_main ? 2 : 1;
+          const uint32_t tx = STAGE_BYTES + ngroups * SC_GROUP_FLOATS * 4 + (s == 0 ? UNIT * 4 : 0);
+          if (elect_one()) {
+            mbar_expect_tx(full, tx);
+            if (s == 0) bulk_load(sc_dst + 2 * SC_GROUP_FLOATS * 4, p.bias + n0, UNIT * 4, full);
+            if (is_main) {
+              tma_load_2d(a_dst, &tmA, s * LQ_KSTAGE, m0, full);
+              tma_load_2d(b_dst, &tmB, s * LQ_KSTAGE, n0, full);
+              for (int q = 0; q < ngroups; ++q) {
+                const size_t g = (size_t)(2 * s + q);
+                bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4, p.sx + g * p.Mpad + m0, LQ_BM * 4, full);
+                bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4 + LQ_BM * 4, p.sw + g * p.Npad + n0, UNIT * 4, full);
+              }
+            } else {
+              tma_load_2d(a_dst, &tmT, 0, m0, full);
+              tma_load_2d(b_dst, &tmL2, 0, n0, full);
+              bulk_load(sc_dst, p.sT + m0, LQ_BM * 4, full);
+              bulk_load(sc_dst + LQ_BM * 4, p.sL2 + n0, UNIT * 4, full);
             }
           }
-          tc_commit(bar_tfull(pb));
-          tc_commit(bar_empty(st));
+          __syncwarp();
+          ++armed;
+          LQ_TL(EV_P_ISSUED, s);
         }
-        __syncwarp();
-        LQ_TL(EV_M_ISSUED, s);
+      }
+      if (!ok && lane == 0) {
+        // aborting: give the copies already issued a bounded time to land before the CTA's shared memory goes away
+        const uint32_t n = armed < (uint32_t)NSTAGE ? armed : (uint32_t)NSTAGE;
+        for (uint32_t i = 1; i <= n; ++i) {
+          const uint32_t j = armed - i;
+          mbar_settle(bar_full(j % NSTAGE), (j / NSTAGE) & 1);
+        }
+      }
+    } else if (warp == 1) {
+      // ------------------------------------------------------------------ MMA issuer
+      uint32_t it = 0;
+      bool ok = true;
+      const uint32_t shape = idesc_shape(UNIT);
+      for (int u = u_begin; u < u_end && ok; ++u) {
+        for (int s = 0; s < stages_per_tile && ok; ++s, ++it) {
+          const int st = it & (NSTAGE - 1);
+          ok = mbar_wait_warp(bar_full(st), (it / NSTAGE) & 1, abort_flag, p.status, LQ_STAGE_MMA);
+          if (!ok) break;
+          tc_fence_after();
+          LQ_TL(EV_M_STAGE_FULL, s);
+          const uint32_t a_addr = sm_stage + st * STAGE_BYTES, b_addr = a_addr + STAGE_A_BYTES;
+          const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(b_addr);
+          const bool is_main = s < p.n_stages_main;
+          // The stage's groups to the accumulators of one pair, each as soon as the drain has read it out; one commit
+          const int ngroups = is_main ? 2 : 1, pair = it & (NPAIR - 1);
+          for (int q = 0; q < ngroups && ok; ++q) {
+            ok = mbar_wait_warp(bar_tempty(2 * pair + q), ((it / NPAIR) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
+            if (!ok) break;
+            tc_fence_after();
+            LQ_TL(EV_M_ACC_FREE, s);
+            const uint32_t d = tmem_base + (2 * pair + q) * TCOLS;
+            if (elect_one()) {
+              if (is_main) {
+                const uint64_t off = (uint64_t)((q * 64) >> 4);
+                tc_mma<TC_F8>(d, adesc + off, bdesc + off, IDESC_F8 | shape, 0u);
+                tc_mma<TC_F8>(d, adesc + off + 2, bdesc + off + 2, IDESC_F8 | shape, 1u);
+              } else {
+                for (int j = 0; j < p.branch_mmas; ++j) {
+                  const uint64_t off = (uint64_t)((j * 32) >> 4);
+                  if (BRANCH == BRANCH_F16) tc_mma<TC_F16>(d, adesc + off, bdesc + off, IDESC_F16 | shape, (uint32_t)j);
+                  else tc_mma<TC_I8>(d, adesc + off, bdesc + off, IDESC_I8 | shape, (uint32_t)j);
+                }
+              }
+            }
+            __syncwarp();
+          }
+          if (!ok) break;
+          if (elect_one()) {
+            tc_commit(bar_tfull(pair));
+            tc_commit(bar_empty(st));
+          }
+          __syncwarp();
+          LQ_TL(EV_M_ISSUED, s);
+        }
       }
     }
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(DRAIN_REGS));
     // ------------------------------------------------------------------ drain + epilogue
     const int quad = warp & 3;                          // tensor-memory lanes 32*quad .. 32*quad+31
-    const int cgi = (warp - FIRST_DRAIN_WARP) >> 2;     // which quarter of the tile's columns
-    const int coff = cgi * WCOLS;
+    const int coff = ((warp - FIRST_DRAIN_WARP) >> 2) * WCOLS;   // which half of the tile's columns
     const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)coff;
-    const int fg = lane >> 2, ft = lane & 3;            // fragment coordinates: rows fg + 8 i, column pair ft
-    uint32_t it = 0;
+    const int fg = lane >> 2, ft = lane & 3;            // fragment coordinates
+    const int row_at = 32 * quad + 4 * fg, col_at = coff + 4 * ft;    // this lane's places in the scale vectors
+    uint32_t it = 0;                                    // operand stages since the kernel began: ring positions it & (NPAIR-1),
+                                                        // it & (SC_RING-1)
     bool ok = true;
+    Frag va[4], vb[4];                                  // two groups: one being consumed, one being fetched
+    auto pair_at = [&](uint32_t i) { return tlane + (i & (NPAIR - 1)) * (2 * TCOLS); };
+    // Requests stage i's first group once its pair is complete (its scale vectors landed before its MMAs were issued).  The
+    // request is made whatever the wait says, and even where no stage is left (it reads some accumulator, nothing looks at
+    // it): a conditional one would have the compiler keep the fragments twice.
+    auto open_stage = [&](uint32_t i, bool exists) {
+      if (exists) ok = mbar_wait_inline(bar_tfull(i & (NPAIR - 1)), (i / NPAIR) & 1, abort_flag, p.status, LQ_STAGE_DRAIN) && ok;
+      tc_fence_after();
+      fetch_group(pair_at(i), va);
+    };
+    auto landed = [&](uint32_t i, int q) {              // the stage's group q is in registers: its accumulator goes back
+      tmem_ld_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_tempty(2 * (i & (NPAIR - 1)) + q));
+    };
+    auto scales_at = [&](uint32_t i, int q) {
+      return load_scales(sc_ptr + (i & (SC_RING - 1)) * (SC_STAGE_BYTES / 4) + q * SC_GROUP_FLOATS, row_at, col_at);
+    };
+    open_stage(0, u_begin < u_end);
     for (int u = u_begin; u < u_end && ok; ++u) {
       const int mb = u / p.units_n, nu = u - mb * p.units_n;
       const int m0 = mb * LQ_BM, n0 = nu * UNIT;
       LQ_TL(EV_TILE, 0);
-      // this thread's 4 rows x 8 columns: acc[8 h + 2 j + i] = rows 16 h + fg + 8 i, columns 8 j + 2 ft, + 1; starts from the bias
-      float2 acc[16];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 bv = __ldg(reinterpret_cast<const float2*>(p.bias + n0 + coff + 8 * j + 2 * ft));
-        acc[2 * j] = bv; acc[2 * j + 1] = bv; acc[8 + 2 * j] = bv; acc[8 + 2 * j + 1] = bv;
-      }
-      // Groups g = 0 .. G-1 come two per operand stage, then the branch has a stage of its own.  `it` counts operand
-      // stages since the kernel began: stage ring position it & (NSTAGE-1), accumulator pair it & (NTBUF-1).  All
-      // hand-shakes are per stage: the scale vectors and the accumulator pair are awaited once, the pair is handed back
-      // when its last group sits in registers.  The group being consumed sits in (vlo, vhi): rows 0-15 and 16-31 of
-      // this warp's quarter, 32 columns each; the next group's halves are requested as soon as a half is consumed.
-      uint32_t vlo[16], vhi[16];
-      // waits for stage `IT_`'s scale vectors and accumulator pair
-#define LQ_AWAIT_STAGE(IT_)                                                                                              \
-      {                                                                                                                  \
-        const uint32_t i_ = (IT_);                                                                                       \
-        ok = mbar_wait(bar_full(i_ & (NSTAGE - 1)), (i_ / NSTAGE) & 1, abort_flag, p.status, LQ_STAGE_DRAIN);            \
-        if (ok) ok = mbar_wait(bar_tfull(i_ & (NTBUF - 1)), (i_ / NTBUF) & 1, abort_flag, p.status, LQ_STAGE_DRAIN);     \
-        tc_fence_after();                                                                                                \
-      }
-      // one group: arithmetic on (vlo, vhi) with the scales at SCG_; the next group's halves (if HAS_NEXT_) are at TNEXT_
-#define LQ_DRAIN_GROUP(SCG_, IS_INT_, HAS_NEXT_, TNEXT_)                                                                 \
-      {                                                                                                                  \
-        const float* sxp_ = (SCG_) + quad * 32 + fg;                                                                     \
-        const float* swp_ = (SCG_) + LQ_BM + coff + 2 * ft;                                                              \
-        const float sx0 = sxp_[0], sx1 = sxp_[8], sx2 = sxp_[16], sx3 = sxp_[24];                                        \
-        float2 sw2[4];                                                                                                   \
-        _Pragma("unroll") for (int j_ = 0; j_ < 4; ++j_) sw2[j_] = *reinterpret_cast<const float2*>(swp_ + 8 * j_);      \
-        if (IS_INT_) drain_frag<true>(vlo, &acc[0], sx0, sx1, sw2);                                                      \
-        else drain_frag<false>(vlo, &acc[0], sx0, sx1, sw2);                                                             \
-        if (HAS_NEXT_) tmem_ld_16x256b_x4((TNEXT_), vlo);                                                                \
-        if (IS_INT_) drain_frag<true>(vhi, &acc[8], sx2, sx3, sw2);                                                      \
-        else drain_frag<false>(vhi, &acc[8], sx2, sx3, sw2);                                                             \
-        if (HAS_NEXT_) tmem_ld_16x256b_x4((TNEXT_) + (16u << 16), vhi);                                                  \
-      }
-      LQ_AWAIT_STAGE(it)
-      if (!ok) break;
+      // this thread's 4 rows x 16 columns: acc[h][2 j + i] = rows 16 h + fg + 8 i, columns 16 ft + 2 j, + 1; from the bias
+      float2 acc[2][16];
       {
-        const uint32_t t0_ = tlane + (it & (NTBUF - 1)) * (2 * TCOLS);
-        tmem_ld_16x256b_x4(t0_, vlo);
-        tmem_ld_16x256b_x4(t0_ + (16u << 16), vhi);
+        const float* bias = sc_ptr + (it & (SC_RING - 1)) * (SC_STAGE_BYTES / 4) + 2 * SC_GROUP_FLOATS + col_at;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 v = *reinterpret_cast<const float4*>(bias + 16 * k);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            acc[0][4 * k + i] = acc[1][4 * k + i] = make_float2(v.x, v.y);
+            acc[0][4 * k + 2 + i] = acc[1][4 * k + 2 + i] = make_float2(v.z, v.w);
+          }
+        }
       }
-      for (int s = 0; s < stages_per_tile && ok; ++s, ++it) {
-        const bool is_main = s < p.n_stages_main;
-        const bool two = is_main && (2 * s + 1 < p.G);
-        const bool is_int = !is_main && p.branch_f16 == 0;
-        const bool last_stage = s + 1 == stages_per_tile;
-        const int st = it & (NSTAGE - 1);
-        const float* scg = sc_ptr + st * (SC_STAGE_BYTES / 4);
-        const uint32_t tpair = tlane + (it & (NTBUF - 1)) * (2 * TCOLS);
-        const uint32_t tpair_next = tlane + ((it + 1) & (NTBUF - 1)) * (2 * TCOLS);
+      const bool last_tile = u + 1 == u_end;
+      for (int s = 0; s < p.n_stages_main && ok; ++s, ++it) {
+        const bool more = s + 1 < stages_per_tile || !last_tile;
         LQ_TL(EV_D_OPEN, s);
-        if (two) {
-          tmem_ld_wait();                               // the stage's first group is in registers
-          LQ_TL(EV_D_WAITED, s);
-          LQ_DRAIN_GROUP(scg, false, true, tpair + TCOLS)
-          LQ_TL(EV_D_HALF, s);
-        }
-        tmem_ld_wait();                                 // the stage's last group is in registers:
-        tc_fence_before();                              // the accumulator pair goes back to the MMA warp
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_tempty(it & (NTBUF - 1)));
+        Scales sc = scales_at(it, 0);
+        landed(it, 0);
+        LQ_TL(EV_D_WAITED, s);
+        fetch_group(pair_at(it) + TCOLS, vb);
+        drain_group<false>(va, acc, sc);
+        LQ_TL(EV_D_HALF, s);
+        sc = scales_at(it, 1);
+        landed(it, 1);
         LQ_TL(EV_D_LOADED, s);
-        if (!last_stage) LQ_AWAIT_STAGE(it + 1)
+        open_stage(it + 1, more);
         LQ_TL(EV_D_ACC_FULL, s);
-        {
-          const float* scg2 = scg + (two ? SC_GROUP_FLOATS : 0);
-          const bool has_next = !last_stage && ok;
-          LQ_DRAIN_GROUP(scg2, is_int, has_next, tpair_next)
-        }
+        drain_group<false>(vb, acc, sc);
         LQ_TL(EV_D_DONE, s);
-        __syncwarp();                                   // done with this stage's scale vectors
-        if (lane == 0) mbar_arrive(bar_sempty(st));
+        ok = __all_sync(0xffffffffu, ok);
       }
-#undef LQ_DRAIN_GROUP
-#undef LQ_AWAIT_STAGE
+      if (!ok) break;
+      if constexpr (BRANCH != BRANCH_NONE) {
+        const Scales sc = scales_at(it, 0);
+        landed(it, 0);
+        if (lane == 0) mbar_arrive(bar_tempty(2 * (it & (NPAIR - 1)) + 1));   // not used by this stage
+        drain_group<BRANCH == BRANCH_I8>(va, acc, sc);
+        ++it;
+        open_stage(it, !last_tile);
+        ok = __all_sync(0xffffffffu, ok);
+      }
       if (!ok) break;
       LQ_TL(EV_D_EPI_BEGIN, 0);
-      // epilogue straight from registers: rows m0 + 32 quad + 16 h + fg (+ 8), columns n0 + coff + 8 j + 2 ft (+ 1)
-      const int row_w = m0 + quad * 32;
-      if (p.out_f32) {
-        float* Y = reinterpret_cast<float*>(p.Y);
+      // epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad
+      const int c = n0 + coff + 16 * ft;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int r_lo = row_w + 16 * h + fg, r_hi = r_lo + 8;
+      for (int h = 0; h < 2; ++h)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int c = n0 + coff + 8 * j + 2 * ft;                  // four lanes write the 32 bytes of one row's sector
-            if (c < p.N) {
-              if (r_lo < p.M) *reinterpret_cast<float2*>(Y + (size_t)r_lo * p.N + c) = acc[8 * h + 2 * j];
-              if (r_hi < p.M) *reinterpret_cast<float2*>(Y + (size_t)r_hi * p.N + c) = acc[8 * h + 2 * j + 1];
+        for (int i = 0; i < 2; ++i) {
+          const int r = m0 + 32 * quad + 16 * h + 8 * i + fg;
+          if (r >= p.M) continue;
+          if (p.out_f32) {
+            float* Y = reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (c + 8 * (k >> 1) < p.N)
+                *reinterpret_cast<float4*>(Y + 4 * k) = make_float4(acc[h][4 * k + i].x, acc[h][4 * k + i].y, acc[h][4 * k + 2 + i].x, acc[h][4 * k + 2 + i].y);
+          } else {
+            __half* Y = reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c;
+            uint32_t w[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const __half2 q = __floats2half2_rn(acc[h][2 * j + i].x, acc[h][2 * j + i].y);
+              w[j] = *reinterpret_cast<const uint32_t*>(&q);
             }
+            if (c < p.N) *reinterpret_cast<uint4*>(Y) = make_uint4(w[0], w[1], w[2], w[3]);
+            if (c + 8 < p.N) *reinterpret_cast<uint4*>(Y + 8) = make_uint4(w[4], w[5], w[6], w[7]);
           }
         }
-      } else {
-        __half* Y = reinterpret_cast<__half*>(p.Y);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          // pack to fp16, then exchange inside the quad: lane ft ends up with columns 8 ft .. 8 ft + 7 of both rows
-          uint32_t lo[4], hi[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const __half2 l2 = __floats2half2_rn(acc[8 * h + 2 * j].x, acc[8 * h + 2 * j].y);
-            const __half2 h2 = __floats2half2_rn(acc[8 * h + 2 * j + 1].x, acc[8 * h + 2 * j + 1].y);
-            lo[j] = *reinterpret_cast<const uint32_t*>(&l2);
-            hi[j] = *reinterpret_cast<const uint32_t*>(&h2);
-          }
-          quad_transpose(lo, ft);
-          quad_transpose(hi, ft);
-          const int c = n0 + coff + 8 * ft;                            // 16 contiguous bytes of a row per lane
-          const int r_lo = row_w + 16 * h + fg, r_hi = r_lo + 8;
-          if (c < p.N) {
-            if (r_lo < p.M) *reinterpret_cast<uint4*>(Y + (size_t)r_lo * p.N + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            if (r_hi < p.M) *reinterpret_cast<uint4*>(Y + (size_t)r_hi * p.N + c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          }
-        }
-      }
       LQ_TL(EV_D_EPI_END, 0);
     }
+    tmem_ld_wait();                                     // the last request
   }
 
   // ---------------------------------------------------------------------- teardown
@@ -439,9 +440,8 @@ lq_status lq_launch_wait_probe(int device, cudaStream_t st) {
 
 lq_status lq_gemm_prepare(int device) {
   if (cudaSetDevice(device) != cudaSuccess) return LQ_ERR_CUDA;
-  if (lq_note_cuda(cudaFuncSetAttribute(lq_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) !=
-      cudaSuccess)
-    return LQ_ERR_CUDA;
+  for (auto* kernel : {lq_gemm_kernel<BRANCH_NONE>, lq_gemm_kernel<BRANCH_I8>, lq_gemm_kernel<BRANCH_F16>})
+    if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return LQ_ERR_CUDA;
   return LQ_OK;
 }
 
@@ -449,9 +449,8 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   if (cudaSetDevice(A->device) != cudaSuccess) return LQ_ERR_CUDA;
   if (L->main_kind != LQ_KIND_E4M3) return LQ_ERR_UNSUPPORTED;
   GemmParams p;
-  p.M = A->M; p.N = L->N; p.Mpad = A->Mpad; p.Npad = L->Npad; p.G = L->G;
-  p.n_stages_main = lq_ceil_div(L->G, 2);
-  p.branch_f16 = L->f16_branch ? 1 : 0;
+  p.M = A->M; p.N = L->N; p.Mpad = A->Mpad; p.Npad = L->Npad;
+  p.n_stages_main = L->Kpad / LQ_KSTAGE;
   p.branch_mmas = L->r == 0 ? 0 : (L->f16_branch ? lq_ceil_div(L->r, 16) : lq_ceil_div(L->r, 32));
   p.tiles_m = lq_ceil_div(A->M, LQ_BM);
   p.units_n = L->Npad / UNIT;
@@ -464,6 +463,7 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   int ctas = g_lq_gemm_ctas > 0 ? g_lq_gemm_ctas : sms;
   const long long units = (long long)p.tiles_m * p.units_n;
   if (ctas > units) ctas = (int)units;
-  const cudaError_t e = lq_launch(lq_gemm_kernel, ctas, GEMM_THREADS, SMEM_BYTES, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
+  auto* kernel = L->r == 0 ? lq_gemm_kernel<BRANCH_NONE> : L->f16_branch ? lq_gemm_kernel<BRANCH_F16> : lq_gemm_kernel<BRANCH_I8>;
+  const cudaError_t e = lq_launch(kernel, ctas, GEMM_THREADS, SMEM_BYTES, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -37,6 +37,15 @@ static inline size_t lq_sfb_offset(int n, int kb, int Npad) {
   return ((size_t)(kb / 4) * (Npad / 128) + n / 128) * 512 + 16 * (n % 32) + 4 * ((n % 128) / 32) + kb % 4;
 }
 
+// Orders the SINT4 GEMM's operands are laid out in, for the accumulator fragments its drain lanes hold (rows g, g + 8, g + 16,
+// g + 24 of 32; columns 8 j + 2 t + {0, 1} of 64):
+//   place of row m in the row-scale vectors: a lane's four are neighbours
+__host__ __device__ static inline int lq_row_slot(int m) { return (m & ~31) | ((m & 7) << 2) | ((m >> 3) & 3); }
+//   row of the weight operand that carries output column n: a lane's 16 columns are neighbours in the output
+static inline int lq_col_slot(int n) { return (n & ~63) | (((n >> 1) & 7) << 3) | (((n >> 4) & 3) << 1) | (n & 1); }
+//   place of column n in the column-scale vectors and the bias: a lane's come in four 16-byte loads, neighbours across lanes
+static inline int lq_colscale_slot(int n) { return (n & ~63) | (((n >> 2) & 3) << 4) | (((n >> 4) & 3) << 2) | (n & 3); }
+
 static inline bool lq_branch_is_mxfp(int branch) {
   return branch == LQ_BRANCH_MXFP8 || branch == LQ_BRANCH_MXFP6 || branch == LQ_BRANCH_MXFP4;
 }
@@ -83,14 +92,15 @@ struct lq_layer {
   // device copy, operand layouts
   int device;
   int main_kind;               // LQ_KIND_*: byte encoding of the 4-bit codes in the MMA operands
-  uint8_t* d_Wq8;              // [Npad][Kpad] bytes, K contiguous (B operand, K-major)
-  float* d_sw;                 // [Gpad][Npad] fp32 (exact images of the fp16 scales)
+  uint8_t* d_Wq8;              // [Npad][Kpad] bytes, K contiguous (B operand, K-major; SINT4: rows in lq_col_slot order)
+  float* d_sw;                 // [Gpad][Npad] fp32 (exact images of the fp16 scales), in lq_colscale_slot order
   uint8_t* d_L1c;              // [planes * rn][Kpad] bytes (W16A16: [rn][Kpad] halves), K contiguous: first factor as the B operand of
                                // the down-projection; rn = lq_l1_rows; MXINT8 factors: the hi digits' rows, then the lo digits'
   uint8_t* d_sfl1;             // MX branches: E8M0 bytes of L1's block scales, [Kpad/128][512] in the tensor-memory layout (row = row of d_L1c)
   float* d_sL1;                // [LQ_MAX_RANK]
   uint8_t* d_L2c;              // [Npad][LQ_RCONT] bytes: int8 codes (or up to 64 halves) of column n, r contiguous
-  float* d_sL2;                // [Npad]  (ones for W16A16)
+  float* d_sL2;                // [Npad]  (ones for W16A16); SINT4: d_L2c in lq_col_slot order, d_sL2 and d_bias in
+                               // lq_colscale_slot order
   float* d_bias;               // [Npad]  (zeros without bias)
   uint8_t* d_sfl2;             // mxfp: E8M0 bytes of L2's block scales, [1][Npad/128][512] in the tensor-memory layout
   uint8_t* d_sfb;              // MXINT4: E8M0 bytes of the weight scales, [Kpad/128][Npad/128][512] in the 32 x 16-byte
@@ -112,11 +122,11 @@ struct lq_act {
   int M_max, Mpad, device, main_kind;
   int M;                       // rows of the last lq_quantize_act
   uint8_t* d_qx8;              // [Mpad][Kpad] operand bytes of the 4-bit codes (A operand, K-major)
-  float* d_sx;                 // [Gpad][Mpad] fp32 images of the fp16 scales
+  float* d_sx;                 // [Gpad][Mpad] fp32 images of the fp16 scales, in lq_row_slot order
   int8_t* d_qb;                // [Mpad][Kpad] branch activation codes
   float* d_sXb;                // [Mpad]
   uint8_t* d_tq;               // [Mpad][LQ_RCONT] bytes: int8 codes (or halves) of T, r contiguous
-  float* d_sT;                 // [Mpad] (ones for W16A16)
+  float* d_sT;                 // [Mpad] (ones for W16A16); SINT4: in lq_row_slot order
   void* d_Xstage;              // lazily allocated staging for lq_linear_forward_host
   void* d_Ystage;
   size_t ystage_bytes;

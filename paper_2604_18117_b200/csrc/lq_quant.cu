@@ -642,7 +642,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(t[j]));
           }
           const float st = amax == 0.f ? 1.f : __fdiv_rn(amax, p.qm);
-          if (valid) p.sT[m] = st;
+          if (valid) p.sT[SINT ? lq_row_slot(m) : m] = st;
           // The quotient t / st as in branch_codes8.  A power of two keeps its steps in binary32's normal range; the quotient
           // stays what it is (what underflows is far below half a code).
           const float k = st < 1e-20f ? 0x1p64f : st > 1e20f ? 0x1p-64f : 1.f, ns = -st * k, y = __frcp_rn(st * k);
@@ -661,7 +661,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           // zeros up to the next multiple of 32, where the up-projection's K ends
           if ((p.rn & 16) && valid) *reinterpret_cast<uint4*>(tqr + p.rn) = make_uint4(0, 0, 0, 0);
         } else if constexpr (BR == BR_F16) {
-          if (valid) p.sT[m] = 1.f;
+          if (valid) p.sT[SINT ? lq_row_slot(m) : m] = 1.f;
 #pragma unroll 1
           for (int c = 0; c < p.rn; c += 16) {
             fetch(c, t);
@@ -806,7 +806,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
                   const Sint4Scale sc(bm);
                   wa[h] = sint4_codes8(a[h], sc.inv[0], sc.coarse); wb[h] = sint4_codes8(b[h], sc.inv[1], sc.coarse);
                   const int g = 2 * st + h;
-                  if (vs && g < p.G) p.sx[(size_t)g * p.Mpad + ms] = lc ? sc.s[1] : sc.s[0];
+                  if (vs && g < p.G) p.sx[(size_t)g * p.Mpad + lq_row_slot(ms)] = lc ? sc.s[1] : sc.s[0];
                 } else {
                   constexpr int TOP = MAIN == MAIN_MXINT4 ? 2 : MAIN == MAIN_MXINT8 ? 6 : 8;
                   constexpr int UP = MAIN == MAIN_MXINT4 ? 0xFF : MAIN == MAIN_MXINT8 ? 0x0F : 0;
