@@ -272,6 +272,8 @@ lq_status lq_selftest_wait_timeout(int device, void* cuda_stream);
  *   "store_qb"     1: lq_quantize_act also writes the branch activation codes to HBM so that lq_act_export can
  *                  return them (parity tests); 0 (default): they stay on chip
  *   "gemm_ctas"    CTAs of the GEMM kernels; 0 (default) = one per SM
+ *   "gemm_width"   columns of the MX GEMM's tiles: 64, 128, 160, 192 or 224 (with an integer branch at most 160, without one
+ *                  not 160; a forward that cannot have the width returns INVALID_ARG); 0 (default) = chosen by the library
  *   "quant_warps", "quant_ctas"   how the quantizer kernel is cut: row groups of 8 per tile (at most 8 count) and 128-value
  *                  stages of K per chunk; 0 = chosen by the library
  *   "overlap"      1 (default): kernels are launched with programmatic stream serialization - a kernel's CTAs may take

@@ -3,6 +3,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <new>
 
@@ -10,6 +11,7 @@
 
 int g_lq_main_kind = LQ_KIND_E4M3;
 int g_lq_gemm_ctas = 0;
+int g_lq_gemm_width = 0;
 int g_lq_store_qb = 0;
 int g_lq_quant_warps = 0;
 int g_lq_quant_ctas = 0;
@@ -73,6 +75,11 @@ extern "C" lq_status lq_set_option(const char* name, int32_t value) {
   if (!strcmp(name, "overlap")) {
     if (value != 0 && value != 1) return LQ_ERR_INVALID_ARG;
     g_lq_overlap = value;
+    return LQ_OK;
+  }
+  if (!strcmp(name, "gemm_width")) {
+    if (value != 0 && std::find(LQ_MX_WIDTHS, LQ_MX_WIDTHS + LQ_MX_NWIDTHS, value) == LQ_MX_WIDTHS + LQ_MX_NWIDTHS) return LQ_ERR_INVALID_ARG;
+    g_lq_gemm_width = value;
     return LQ_OK;
   }
   if (!strcmp(name, "gemm_ctas")) {
@@ -143,8 +150,8 @@ lq_layer* lq_layer_new(const lq_config* cfg) {
   L->device = -1;
   L->main_kind = g_lq_main_kind;
   L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1c = nullptr; L->d_sL1 = nullptr;
-  L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfb = nullptr;
-  L->d_sfl1 = nullptr; L->d_sfl2 = nullptr;
+  L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfl1 = nullptr;
+  for (int i = 0; i < LQ_MX_NWIDTHS; ++i) L->d_sfbw[i] = L->d_sfl2w[i] = nullptr;
   return L;
 }
 
@@ -389,11 +396,14 @@ static void layer_free_device(lq_layer* L) {
   if (L->device < 0) return;
   cudaSetDevice(L->device);
   cudaFree(L->d_Wq8); cudaFree(L->d_sw); cudaFree(L->d_L1c); cudaFree(L->d_sL1);
-  cudaFree(L->d_L2c); cudaFree(L->d_sL2); cudaFree(L->d_bias); cudaFree(L->d_sfb);
-  cudaFree(L->d_sfl1); cudaFree(L->d_sfl2);
-  L->d_sfl1 = nullptr; L->d_sfl2 = nullptr;
+  cudaFree(L->d_L2c); cudaFree(L->d_sL2); cudaFree(L->d_bias); cudaFree(L->d_sfl1);
+  L->d_sfl1 = nullptr;
+  for (int i = 0; i < LQ_MX_NWIDTHS; ++i) {
+    cudaFree(L->d_sfbw[i]); cudaFree(L->d_sfl2w[i]);
+    L->d_sfbw[i] = L->d_sfl2w[i] = nullptr;
+  }
   L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1c = nullptr; L->d_sL1 = nullptr;
-  L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfb = nullptr;
+  L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr;
   L->device = -1;
 }
 
@@ -416,22 +426,28 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
   lq_status st;
   try {
     std::vector<int> wrow(Npad), srow(Npad);                     // places of column n in the weight operand and the vectors
-    for (int n = 0; n < Npad; ++n) { wrow[n] = L->mx ? n : lq_col_slot(n); srow[n] = L->mx ? n : lq_colscale_slot(n); }
+    for (int n = 0; n < Npad; ++n) { wrow[n] = L->mx ? lq_col32_slot(n) : lq_col_slot(n); srow[n] = L->mx ? n : lq_colscale_slot(n); }
     std::vector<uint8_t> w8((size_t)Npad * Kpad, lq_encode_code_host(0, L->main_kind));
     for (int k = 0; k < K; ++k)
       for (int n = 0; n < N; ++n)
         w8[(size_t)wrow[n] * Kpad + k] = L->mxfp ? L->Wq8h[(size_t)k * N + n] : lq_encode_code_host(L->Wq[(size_t)k * N + n], L->main_kind);
     if ((st = upload(&L->d_Wq8, w8)) != LQ_OK) return st;
     if (L->mx) {
-      // E8M0 bytes (exponent + 127) in the layout the block-scaled MMA reads from tensor memory; 127 = 2^0 for padding
-      std::vector<uint8_t> sfb((size_t)(Npad / 128) * (Kpad / 128) * 512, 127);
-      for (int g = 0; g < G; ++g)
-        for (int n = 0; n < N; ++n) {
-          int x = 0;
-          frexpf(h2f(L->sw[(size_t)g * N + n]), &x);              // 2^e = 0.5 * 2^(e+1)
-          sfb[lq_sfb_offset(n, g, Npad)] = (uint8_t)(x - 1 + 127);
-        }
-      if ((st = upload(&L->d_sfb, sfb)) != LQ_OK) return st;
+      // E8M0 bytes (exponent + 127) in the layout the block-scaled MMA reads from tensor memory, by tile width; 127 = 2^0 for padding
+      std::vector<uint8_t> e8((size_t)G * N);
+      for (size_t i = 0; i < e8.size(); ++i) {
+        int x = 0;
+        frexpf(h2f(L->sw[i]), &x);                                // 2^e = 0.5 * 2^(e+1)
+        e8[i] = (uint8_t)(x - 1 + 127);
+      }
+      for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
+        const int width = LQ_MX_WIDTHS[wi], tiles = lq_ceil_div(N, width);
+        if (!lq_mx_width_used(width, L->integer_branch)) continue;
+        std::vector<uint8_t> sfb((size_t)(Kpad / 128) * tiles * lq_ceil_div(width, 128) * 512, 127);
+        for (int g = 0; g < G; ++g)
+          for (int n = 0; n < N; ++n) sfb[lq_sfb_offset(wrow[n], g, width, tiles)] = e8[(size_t)g * N + n];
+        if ((st = upload(&L->d_sfbw[wi], sfb)) != LQ_OK) return st;
+      }
     } else {
       std::vector<float> swf((size_t)Gpad * Npad, 0.f);
       for (int g = 0; g < G; ++g)
@@ -475,18 +491,18 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
         }
       if ((st = upload(&L->d_L1c, l1c)) != LQ_OK) return st;
       if ((st = upload(&L->d_sfl1, sfl1)) != LQ_OK) return st;
-      // E8M0 bytes of L2's block scales along the rank, one 128-byte-of-rank stage: [1][Npad/128][512]
-      std::vector<uint8_t> sfl2((size_t)(Npad / 128) * 512, 127);
+      // E8M0 bytes of L2's block scales along the rank, four K blocks (one 128-byte-of-rank stage) per column
+      std::vector<uint8_t> e2((size_t)4 * N, 127);
       if (L->a8 && L->cfg.branch == LQ_BRANCH_MXINT4) {
         // 4-bit codes are their own lo digit: one plane, K blocks in order (the intermediate brings its two planes as two
         // stages against this one)
         for (int j = 0; j < r; ++j)
-          for (int n = 0; n < N; ++n) l2c[(size_t)n * LQ_RCONT + j] = lq_digit_e4m3(L->L2q[(size_t)j * N + n]);
+          for (int n = 0; n < N; ++n) l2c[(size_t)wrow[n] * LQ_RCONT + j] = lq_digit_e4m3(L->L2q[(size_t)j * N + n]);
         for (int c = 0; c < lq_ceil_div(r, 32); ++c)
           for (int n = 0; n < N; ++n) {
             int e = 0;
             pow2_exponent(L->s2b[(size_t)c * N + n], &e);
-            sfl2[lq_sfb_offset(n, c, Npad)] = (uint8_t)(e + 127);
+            e2[(size_t)c * N + n] = (uint8_t)(e + 127);
           }
       } else if (L->a8) {
         // two digit planes, code = 16 hi + lo: hi digits of rank index j at byte j, lo digits at byte 64 + j (rank <= 64);
@@ -496,27 +512,34 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
           for (int n = 0; n < N; ++n) {
             int hi, lo;
             lq_split_digits(L->L2q[(size_t)j * N + n], &hi, &lo);
-            l2c[(size_t)n * LQ_RCONT + j] = lq_digit_e4m3(hi);
-            l2c[(size_t)n * LQ_RCONT + 64 + j] = lq_digit_e4m3(lo);
+            l2c[(size_t)wrow[n] * LQ_RCONT + j] = lq_digit_e4m3(hi);
+            l2c[(size_t)wrow[n] * LQ_RCONT + 64 + j] = lq_digit_e4m3(lo);
           }
         for (int c = 0; c < lq_ceil_div(r, 32); ++c)
           for (int n = 0; n < N; ++n) {
             int e = 0;
             pow2_exponent(L->s2b[(size_t)c * N + n], &e);
-            sfl2[lq_sfb_offset(n, c, Npad)] = (uint8_t)(e + 4 + 127);
-            sfl2[lq_sfb_offset(n, 2 + c, Npad)] = (uint8_t)(e + 127);
+            e2[(size_t)c * N + n] = (uint8_t)(e + 4 + 127);
+            e2[(size_t)(2 + c) * N + n] = (uint8_t)(e + 127);
           }
       } else {
         for (int j = 0; j < r; ++j)
-          for (int n = 0; n < N; ++n) l2c[(size_t)n * LQ_RCONT + j] = L->L2e[(size_t)j * N + n];
+          for (int n = 0; n < N; ++n) l2c[(size_t)wrow[n] * LQ_RCONT + j] = L->L2e[(size_t)j * N + n];
         for (int c = 0; c < lq_ceil_div(r, 32); ++c)
           for (int n = 0; n < N; ++n) {
             int e = 0;
             pow2_exponent(L->s2b[(size_t)c * N + n], &e);
-            sfl2[lq_sfb_offset(n, c, Npad)] = (uint8_t)(e + 127);
+            e2[(size_t)c * N + n] = (uint8_t)(e + 127);
           }
       }
-      if ((st = upload(&L->d_sfl2, sfl2)) != LQ_OK) return st;
+      for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
+        const int width = LQ_MX_WIDTHS[wi], tiles = lq_ceil_div(N, width);
+        if (!lq_mx_width_used(width, false)) continue;
+        std::vector<uint8_t> sfl2((size_t)tiles * lq_ceil_div(width, 128) * 512, 127);
+        for (int c = 0; c < 4; ++c)
+          for (int n = 0; n < N; ++n) sfl2[lq_sfb_offset(wrow[n], c, width, tiles)] = e2[(size_t)c * N + n];
+        if ((st = upload(&L->d_sfl2w[wi], sfl2)) != LQ_OK) return st;
+      }
     } else if (L->f16_branch) {
       std::vector<uint8_t> l1c((size_t)rn * Kpad * 2, 0);
       uint16_t* h = (uint16_t*)l1c.data();
@@ -532,7 +555,11 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
     if ((st = upload(&L->d_L2c, l2c)) != LQ_OK) return st;
   } catch (const std::bad_alloc&) { return LQ_ERR_ALLOC; }
   if ((st = lq_make_tmap_bytes(&L->tmB, L->d_Wq8, Npad, Kpad, LQ_BN)) != LQ_OK) return st;
-  if ((st = lq_make_tmap_bytes(&L->tmB2, L->d_Wq8, Npad, Kpad, 2 * LQ_BN)) != LQ_OK) return st;
+  for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
+    if (!L->d_sfbw[wi]) continue;
+    if ((st = lq_make_tmap_bytes(&L->tmBw[wi], L->d_Wq8, Npad, Kpad, (uint32_t)LQ_MX_WIDTHS[wi])) != LQ_OK) return st;
+    if ((st = lq_make_tmap_bytes(&L->tmL2w[wi], L->d_L2c, Npad, LQ_RCONT, (uint32_t)LQ_MX_WIDTHS[wi])) != LQ_OK) return st;
+  }
   if (r > 0 && (st = lq_make_tmap_bytes(&L->tmL1, L->d_L1c, (uint64_t)rn * lq_l1_planes(L), (uint64_t)Kpad * (L->f16_branch ? 2 : 1),
                                         (uint32_t)(rn * lq_l1_planes(L)))) != LQ_OK) return st;
   if ((st = lq_make_tmap_bytes(&L->tmL2, L->d_L2c, Npad, LQ_RCONT, LQ_BN)) != LQ_OK) return st;

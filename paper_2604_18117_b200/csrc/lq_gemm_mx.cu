@@ -8,30 +8,32 @@
 // accumulator and nothing has to be drained per block.  The 4-bit codes ride in E4M3 operands as in the SINT4
 // kernel.  Products q q' 2^(e+e') are exact in fp32; their sum is rounded by the tensor core's fp32 accumulation.
 //
-// Shape of the kernel (persistent, one CTA per SM, 18 warps):
-//   warp 0      TMA producer: per stage 128 bytes of K of A (128 rows) and B (256 rows, one box) plus the stage's scale
-//               bytes (512 B per 128 rows: four K blocks, already in the 32 x 16-byte layout tensor memory wants);
-//               per tile one more stage with the branch operands (tq, L2q) and the vectors sT, sL2, bias for the drain
+// Shape of the kernel (persistent, one CTA per SM, warp-specialised, 18 warps): tiles of 128 rows x W columns, W chosen by
+// the launcher (pick_width).
+//   warp 0      TMA producer: per stage 128 bytes of K of A (128 rows) and B (W rows) plus the stage's scale bytes (512 B per
+//               128 rows: four K blocks, already in the 32 x 16-byte layout tensor memory wants); per tile one or two more
+//               stages with the branch operands (tq, L2q) and the vectors sT, sL2, bias for the drain.  Weights do not depend
+//               on earlier kernels: the first ring's worth is requested before the grid dependency is waited for
 //   warp 1      owns tensor memory; per stage: tcgen05.cp of the scale bytes into tensor-memory columns, then four
-//               K = 32 block-scaled MMAs (N = 256) into the tile's accumulator; after the last stage the low-rank
-//               branch's up-projection U = tq L2q (kind::i8, exact int32; its fp32 scales cannot be applied by the
-//               tensor core) into a second accumulator, then ONE hand-over of both to the drain
-//   warps 2-17  drain: tcgen05.ld the main accumulator (mma.sync fragment layout, 16x256b) straight into registers and
-//               release it - the next tile's main loop starts - then read the branch accumulator,
-//               y = main + sT sL2 U + bias, release that too, convert; a 4 x 4 exchange inside each quad gives
-//               every lane 16 contiguous bytes of one row, so each store instruction writes whole 32-byte sectors
-//               straight from registers.
-// Tensor memory has 512 columns: main accumulator [0, 256), branch accumulator [256, 512).  The 12 scale-factor
-// columns of a stage (one slot: the tensor pipe executes one thread's tcgen05 copies and MMAs in issue order) alias the
-// first 16 columns of the branch accumulator: they are live only while the tile's block-scaled MMAs run, the branch
-// accumulator only from the branch MMA (issued after them) until the drain has read it.  The four drain warps that own
-// those 16 columns read them together with the main accumulator, before the hand-over; the rest of the branch
-// accumulator is read afterwards, under the next tile's main loop, and is needed again only by that tile's branch MMA.
+//               K = 32 block-scaled MMAs into the tile's accumulator; after the last stage the low-rank branch's
+//               up-projection: MX and fp16 branches onto the same accumulator, integer branches (U = tq L2q, kind::i8, exact
+//               int32; fp32 scales that the tensor core cannot apply) into an accumulator of their own
+//   warps 2-17  drain, 32 rows x 32 columns at a time: y = main + sT sL2 U + bias, convert, store.  The columns of a block
+//               of 32 are permuted in the weight operand (lq_col32_slot) so that a lane's eight are neighbours in Y: 16
+//               bytes of a row, no exchange
+// Two accumulators alternate (with an integer branch: two and the branch's), so a tile's output leaves under the next tile's
+// main loop: 2 W (3 W) columns and 12 for the scale factors of a stage (one slot: the tensor pipe executes one thread's
+// tcgen05 copies and MMAs in issue order).  A single 256-column accumulator spent a third of a short-K launch on the
+// hand-over and the stores behind it (M = 8192, K x N = 1152 x 3456, MXFP rank 64: 36.4 us, 28 without the stores).
+// What bounds it: operand delivery from the L2 (W = 256: 48 KB a stage; 70-78 bytes per clock and SM with all SMs at it),
+// the tensor pipe close behind (2 W clocks a stage).
 // What was measured on the way here (PixArt block, four GEMMs): the branch on mma.sync in the drain warps took tensor
 // time from the main loop; TMA stores of the output (32 boxes of 2 KB, or 8 of 8 KB, per tile) cost 15 % against
-// plain stores - they share the TMA unit with the operand loads; a fourth ring stage gained 3 %.
+// plain stores - they share the TMA unit with the operand loads.
 // Every wait is bounded as in lq_gemm.cu.
 #include <cuda_fp16.h>
+
+#include <algorithm>
 
 #include "lq_device.cuh"
 
@@ -49,28 +51,23 @@ namespace {
 
 using namespace lqdev;
 
-constexpr int UNIT = LQ_BN;                        // 128 output columns
-constexpr int NSTAGE = 4;                          // operand ring depth
+constexpr int MAX_STAGES = 8;
 constexpr int STAGE_A_BYTES = LQ_BM * LQ_KSTAGE;   // 16 KB
-constexpr int STAGE_B_BYTES = 2 * UNIT * LQ_KSTAGE;   // 32 KB (one 256-row box, or one 128-row box for a narrow tile)
-constexpr int STAGE_BYTES = STAGE_A_BYTES + STAGE_B_BYTES;
+constexpr int MAX_W = 224;                         // columns of the widest tile
 constexpr int SF_BYTES = 512;                      // scale bytes of 128 rows x 4 K blocks
-constexpr int STAGE_SF_BYTES = 3 * SF_BYTES;       // SFA, then SFB of both halves
-constexpr int SC_FLOATS = LQ_BM + 4 * UNIT;        // per tile: sT[128], sL2[256], bias[256]
+constexpr int STAGE_SF_BYTES = 3 * SF_BYTES;       // SFA, then SFB of up to 256 columns
+constexpr int SC_FLOATS = LQ_BM + 2 * MAX_W;       // per tile: sT[128], sL2[W], bias[W]
 constexpr int NUM_DRAIN_WARPS = 16;
 constexpr int FIRST_DRAIN_WARP = 2;
 constexpr int GEMM_THREADS = (FIRST_DRAIN_WARP + NUM_DRAIN_WARPS) * 32;
 constexpr int SMEM_BAR_BYTES = 256;
-constexpr int SMEM_BYTES = 1024 /*alignment slack*/ + NSTAGE * STAGE_BYTES + NSTAGE * STAGE_SF_BYTES + 2 * SC_FLOATS * 4 +
-                           SMEM_BAR_BYTES;
-static_assert(SMEM_BYTES <= 232448, "shared memory budget");
-static_assert(STAGE_BYTES % 1024 == 0, "stages must keep the 1024-byte alignment of the swizzled tiles");
-// tensor-memory columns: main accumulator [0, 256), branch accumulator [256, 512); 4 columns of A scales and 8 of B
-// scales alias the start of the branch accumulator (disjoint lifetimes, see the top of the file)
-constexpr int TM_BR = 256, TM_SFA = 256, TM_SFB = TM_SFA + 4, TM_SF_ALIASED = 16;
+constexpr int FIXED_SMEM = 1024 /*alignment slack*/ + 2 * SC_FLOATS * 4 + SMEM_BAR_BYTES;
+constexpr int MAX_SMEM = 227 * 1024;
+// tensor-memory columns: accumulators at 0 and W, the branch's at 2 W; 4 columns of A scales and 8 of B scales
+constexpr int TM_SFA = 496, TM_SFB = TM_SFA + 4;
 
 struct MxParams {
-  int M, N, Mpad, Npad;
+  int M, N, Npad;
   int k_stages;           // stages of A per tile: Kpad / 128, times two when 8-bit activation codes come as two digit planes
   int branch_steps;       // 0: no branch; else MMAs of the branch stage (32 bytes of r each)
   int branch_f16;         // the branch operands are halves (W16A16 reference branch): no scales, summed by the tensor core
@@ -80,15 +77,13 @@ struct MxParams {
                           // (plane of T, plane of L2) pair of the same rank block is one MMA.  3: the same codes with 4-bit
                           // factors (one plane) and rank up to 128: two stages like mode 1, one per plane of T
   const uint8_t* sft;     // branch_mx: E8M0 bytes of T's block scales, [Mpad/128][512]
-  const uint8_t* sfl2;    // branch_mx: E8M0 bytes of L2's block scales, [Npad/128][512]
-  int tiles_m, units_n;
-  int by_units;           // how the CTAs share the work: 0 whole tiles, 1 128-column units
+  const uint8_t* sfl2;    // branch_mx: E8M0 bytes of L2's block scales, [tiles_n][sf_chunks][512]
+  int tiles_m, tiles_n;
+  int width, stages;      // W, operand ring depth
   int b_wrap;             // Kpad / 128: stage s reads B (and its scales) at stage s mod b_wrap - the planes share the weights
-                          // (kept in what was the padding before the next pointer: this kernel sits at its register
-                          // cap, and moving its other parameters changed the allocation ptxas found - 50 % more spill
-                          // traffic and 15 % longer launches)
   const uint8_t* sfa;     // [Mpad/128][k_stages][512]
-  const uint8_t* sfb;     // [k_stages][Npad/128][512]: the scale bytes of two neighbouring 128-column units are contiguous
+  const uint8_t* sfb;     // [Kpad/128][tiles_n][sf_chunks][512]
+  int sf_chunks;          // ceil(W / 128)
   const float* sT;        // [Mpad]
   const float* sL2;       // [Npad]
   const float* bias;      // [Npad]
@@ -97,29 +92,51 @@ struct MxParams {
   int32_t* status;
 };
 
-// 4 x 4 transpose across the four lanes of a quad: afterwards v[s] of lane t is what v[t] of lane s was.
-__device__ __forceinline__ void quad_transpose(uint32_t (&v)[4], int t) {
-  const bool hi2 = (t & 2) != 0, hi1 = (t & 1) != 0;
-  uint32_t y0 = __shfl_xor_sync(0xffffffffu, hi2 ? v[0] : v[2], 2);
-  uint32_t y1 = __shfl_xor_sync(0xffffffffu, hi2 ? v[1] : v[3], 2);
-  if (hi2) { v[0] = y0; v[1] = y1; } else { v[2] = y0; v[3] = y1; }
-  y0 = __shfl_xor_sync(0xffffffffu, hi1 ? v[0] : v[1], 1);
-  y1 = __shfl_xor_sync(0xffffffffu, hi1 ? v[2] : v[3], 1);
-  if (hi1) { v[0] = y0; v[2] = y1; } else { v[1] = y0; v[3] = y1; }
+// A stage's instructions under one election, predicated instead of branched around: the control flow of the issuing warps
+// stays uniform and their addresses and descriptors in uniform registers.  (Inside an `if` of one lane every operand
+// is moved there instruction by instruction: 320-370 clocks for the MMA warp's stage and 270 for the producer's.)
+//   main stage of the MMA warp: scale bytes to tensor memory, four K = 32 MMAs, the stage's return
+__device__ __forceinline__ void issue_main_stage(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint64_t sfa, uint64_t sfb, uint32_t two,
+                                                 uint32_t accumulate, uint32_t empty) {
+  asm volatile(
+      "{\n\t.reg .pred P, Q, T, A;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "setp.ne.and.b32 Q, %12, 0, P;\n\t"
+      "setp.ne.b32 A, %13, 0;\n\t"
+      "setp.eq.b32 T, 0, 0;\n\t"
+      "@P tcgen05.cp.cta_group::1.32x128b.warpx4 [%14], %9;\n\t"
+      "@P tcgen05.cp.cta_group::1.32x128b.warpx4 [%15], %10;\n\t"
+      "@Q tcgen05.cp.cta_group::1.32x128b.warpx4 [%16], %11;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %1, %5, %17, [%14], [%15], A;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %2, %6, %18, [%14], [%15], T;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %3, %7, %19, [%14], [%15], T;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %4, %8, %20, [%14], [%15], T;\n\t"
+      "@P tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%21];\n\t}"
+      ::"r"(d), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "l"(sfa), "l"(sfb),
+      "l"(sfb + (SF_BYTES >> 4)), "r"(two), "r"(accumulate), "r"((uint32_t)TM_SFA), "r"((uint32_t)TM_SFB), "r"((uint32_t)(TM_SFB + 4)),
+      "r"(idesc), "r"(idesc | idesc_mx_ids(1)), "r"(idesc | idesc_mx_ids(2)), "r"(idesc | idesc_mx_ids(3)), "r"(empty)
+      : "memory");
 }
-// y = main + U sT sL2 + bias for one n8 fragment (registers: row g columns 2t, 2t+1, then row g + 8 the same columns).
-// U is an exact int32 with |U| < 2^22: converted exactly with the 1.5 * 2^23 trick.
-__device__ __forceinline__ void combine_fragment(float (&a)[4], const uint32_t* u, bool has_branch, float st_lo, float st_hi,
-                                                 float2 sl, float2 bv) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float y = a[i] + ((i & 1) ? bv.y : bv.x);
-    if (has_branch) {
-      const float uf = __int_as_float((int)u[i] + 0x4B400000) - 12582912.0f;
-      y = fmaf(uf, ((i >> 1) ? st_hi : st_lo) * ((i & 1) ? sl.y : sl.x), y);
-    }
-    a[i] = y;
-  }
+//   main stage of the producer: the weights' half (which announces the whole stage) and the activations' half
+__device__ __forceinline__ void load_weights_stage(uint32_t full, uint32_t tx, uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t sf_dst,
+                                                   const uint8_t* sf, uint32_t sf_bytes) {
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "@P mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+      "@P cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5}], [%0];\n\t"
+      "@P cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%6], [%7], %8, [%0];\n\t}"
+      ::"r"(full), "r"(tx), "r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(sf_dst), "l"(reinterpret_cast<uint64_t>(sf)), "r"(sf_bytes)
+      : "memory");
+}
+__device__ __forceinline__ void load_acts_stage(uint32_t full, uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t sf_dst, const uint8_t* sf) {
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "@P cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%1], [%2, {%3, %4}], [%0];\n\t"
+      "@P cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%5], [%6], %7, [%0];\n\t}"
+      ::"r"(full), "r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(sf_dst), "l"(reinterpret_cast<uint64_t>(sf)), "r"((uint32_t)SF_BYTES)
+      : "memory");
 }
 
 // BRANCH_ACC: the layer has an integer branch with fp32 scales, whose product needs an accumulator of its own.  The
@@ -127,19 +144,19 @@ __device__ __forceinline__ void combine_fragment(float (&a)[4], const uint32_t* 
 template <bool BRANCH_ACC>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                  const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmT,
-                  const __grid_constant__ CUtensorMap tmL2, const MxParams p) {
+                  const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
+                  const __grid_constant__ MxParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base - smem_u32(smem_raw));
-  constexpr int OFF_SF = NSTAGE * STAGE_BYTES;
-  constexpr int OFF_SC = OFF_SF + NSTAGE * STAGE_SF_BYTES;
-  constexpr int OFF_BAR = OFF_SC + 2 * SC_FLOATS * 4;
-  const uint32_t sm_stage = base, sm_sf = base + OFF_SF, sm_sc = base + OFF_SC, sm_bar = base + OFF_BAR;
-  const float* sc_ptr = reinterpret_cast<const float*>(smem + OFF_SC);
-  uint8_t* bar_ptr = smem + OFF_BAR;
+  const int W = p.width, NST = p.stages;
+  const uint32_t stage_bytes = STAGE_A_BYTES + (uint32_t)W * LQ_KSTAGE, b_bytes = (uint32_t)W * LQ_KSTAGE;
+  const uint32_t off_sf = (uint32_t)NST * stage_bytes, off_sc = off_sf + NST * STAGE_SF_BYTES, off_bar = off_sc + 2 * SC_FLOATS * 4;
+  const uint32_t sm_stage = base, sm_sf = base + off_sf, sm_sc = base + off_sc, sm_bar = base + off_bar;
+  const float* sc_ptr = reinterpret_cast<const float*>(smem + off_sc);
+  uint8_t* bar_ptr = smem + off_bar;
   // barrier map (8 bytes each)
-  constexpr int B_FULL = 0, B_EMPTY = NSTAGE, B_TFULL = 2 * NSTAGE, B_TEMPTY = B_TFULL + 1, B_RFULL = B_TEMPTY + 1,
+  constexpr int B_FULL = 0, B_EMPTY = MAX_STAGES, B_TFULL = 2 * MAX_STAGES, B_TEMPTY = B_TFULL + 2, B_RFULL = B_TEMPTY + 2,
                 B_REMPTY = B_RFULL + 2, B_BEMPTY = B_REMPTY + 2, NBAR = B_BEMPTY + 1;
   auto bar = [&](int idx) { return sm_bar + 8u * (uint32_t)idx; };
   static_assert(NBAR * 8 + 16 <= SMEM_BAR_BYTES, "barrier area too small");
@@ -149,48 +166,30 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // provably warp-uniform
   const int lane = threadIdx.x & 31;
   const bool has_branch = p.branch_steps > 0;
-  const int nbst = p.branch_mx == 3 ? 2 : 1;              // stages of the branch per tile
-  // An fp16 branch has no scales: its product is accumulated onto the main accumulator by the tensor core and the drain
-  // sees no branch at all.  An integer branch needs its fp32 scales applied per element: second accumulator.
-  constexpr bool branch_acc = BRANCH_ACC;                 // = has_branch && !p.branch_f16 && !p.branch_mx, decided by the host
-  // Each CTA takes a contiguous, equal share of the work and walks it as 256-wide tiles (128-wide where a row block or
-  // the share ends).  A 128-wide tile costs nearly as much as a 256-wide one (a stage's time is set by its hand-shakes
-  // and instruction count, not its MMA width).  by_units = 0 shares whole tiles - row blocks cut into 256-wide tiles
-  // plus at most one 128-wide one - which avoids needless narrow tiles; by_units = 1 shares 128-column units, which
-  // balances better when a CTA gets only two or three tiles and the row blocks have an odd number of units.
-  const int tiles_n = (p.units_n + 1) >> 1;
-  const long long work = (long long)p.tiles_m * (p.by_units ? p.units_n : tiles_n);
+  const int nbst = !has_branch ? 0 : p.branch_mx == 3 ? 2 : 1;             // stages of the branch per tile
+  // this CTA's contiguous run of tiles, row block major
+  const long long work = (long long)p.tiles_m * p.tiles_n;
   const int w_begin = (int)((work * blockIdx.x) / gridDim.x);
   const int w_end = (int)((work * (blockIdx.x + 1)) / gridDim.x);
-  // position w -> row block, first unit and width of the tile that starts there
-  auto tile_at = [&](int w, int& mb, int& nu, int& width) {
-    if (p.by_units) {
-      mb = w / p.units_n; nu = w - mb * p.units_n;
-      width = (nu + 1 < p.units_n && w + 1 < w_end) ? 2 : 1;
-      return w + width;
-    }
-    mb = w / tiles_n; nu = 2 * (w - mb * tiles_n);
-    width = (nu + 1 < p.units_n) ? 2 : 1;
-    return w + 1;
-  };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NSTAGE; ++s) { mbar_init(bar(B_FULL + s), 1); mbar_init(bar(B_EMPTY + s), 1); }
-    mbar_init(bar(B_TFULL), 1);
-    mbar_init(bar(B_TEMPTY), NUM_DRAIN_WARPS);
-    for (int b = 0; b < 2; ++b) { mbar_init(bar(B_RFULL + b), 1); mbar_init(bar(B_REMPTY + b), NUM_DRAIN_WARPS); }
+    for (int s = 0; s < NST; ++s) { mbar_init(bar(B_FULL + s), 1); mbar_init(bar(B_EMPTY + s), 1); }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(bar(B_TFULL + b), 1); mbar_init(bar(B_TEMPTY + b), NUM_DRAIN_WARPS);
+      mbar_init(bar(B_RFULL + b), 1); mbar_init(bar(B_REMPTY + b), NUM_DRAIN_WARPS);
+    }
     mbar_init(bar(B_BEMPTY), NUM_DRAIN_WARPS);
     *abort_flag = 0;
     mbar_init_fence();
   }
-  if (warp == 1) {
-    tmem_alloc(smem_u32(tmem_slot), 512);
-  }
+  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
   tc_fence_before();
   __syncthreads();
-  grid_dependency_sync();        // set-up done; from here on global memory written by earlier kernels is read
   tc_fence_after();
-  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  grid_launch_dependents();
+  // All 512 columns are this CTA's, so they start at 0: a constant, where a value read back would have to be moved into
+  // uniform registers for every instruction that names a column.
+  constexpr uint32_t tmem_base = 0;
 
   LQ_TL_DECL((blockIdx.x == 0 && lane == 0)
                  ? (warp == 0 ? (int)TL_PRODUCER : warp == 1 ? (int)TL_MMA : warp == FIRST_DRAIN_WARP ? (int)TL_DRAIN_FIRST
@@ -199,289 +198,251 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    uint32_t it = 0, tc = 0, rarmed = 0;
+    uint32_t tc = 0, rarmed = 0, par = 1;              // parity of the ring slot's "empty" barrier
+    int st = 0, armed = 0;                             // ring slot; stages announced (up to the ring's depth)
     bool ok = true;
-    for (int w = w_begin, w_next; w < w_end && ok; w = w_next, ++tc) {
-      int mb, nu, width;
-      w_next = tile_at(w, mb, nu, width);
-      const int m0 = mb * LQ_BM, n0 = nu * UNIT;
-      const uint8_t* sfa = p.sfa + (size_t)mb * p.k_stages * SF_BYTES;
-      const uint8_t* sfb = p.sfb + (size_t)nu * SF_BYTES;
+    const uint32_t sfb_bytes = (uint32_t)p.sf_chunks * SF_BYTES;
+    auto load_b = [&](int st, int s, int nu) {         // the weights' half of main stage s; announces the whole stage
+      const uint32_t dst = sm_stage + st * stage_bytes + STAGE_A_BYTES, full = bar(B_FULL + st);
+      const int sb = s >= p.b_wrap ? s - p.b_wrap : s; // the lo digits' plane runs over the same weights
+      load_weights_stage(full, stage_bytes + SF_BYTES + sfb_bytes, dst, &tmB, sb * LQ_KSTAGE, nu * W, sm_sf + st * STAGE_SF_BYTES + SF_BYTES,
+                         p.sfb + ((size_t)sb * p.tiles_n + nu) * sfb_bytes, sfb_bytes);
+    };
+    auto load_a = [&](int st, int s, int mb) {
+      const uint32_t full = bar(B_FULL + st);
+      load_acts_stage(full, sm_stage + st * stage_bytes, &tmA, s * LQ_KSTAGE, mb * LQ_BM, sm_sf + st * STAGE_SF_BYTES,
+                      p.sfa + ((size_t)mb * p.k_stages + s) * SF_BYTES);
+    };
+    auto advance = [&]() {
+      ++armed;
+      if (++st == NST) { st = 0; par ^= 1; }
+    };
+    int early = 0;                                     // stages of the first tile whose weights were requested ahead
+    if (w_begin < w_end) {
+      early = min(NST, p.k_stages);
+      for (int s = 0; s < early; ++s) load_b(s, s, w_begin % p.tiles_n);
+    }
+    grid_dependency_wait();
+    for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
+      const int mb = w / p.tiles_n, nu = w - mb * p.tiles_n;
+      const int m0 = mb * LQ_BM, n0 = nu * W;
+      for (int s = 0; s < p.k_stages; ++s) {
+        const bool ahead = tc == 0 && s < early;
+        if (!ahead) {
+          ok = mbar_wait_warp(bar(B_EMPTY + st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
+          if (!ok) break;
+        }
+        LQ_TL(EV_P_SLOT_FREE, s);
+        if (!ahead) load_b(st, s, nu);
+        load_a(st, s, mb);
+        advance();
+        LQ_TL(EV_P_ISSUED, s);
+      }
+      // the branch operands: the containers of tq (128 rows) and L2q (W rows), r contiguous; mode 3 brings the two
+      // digit planes of tq as two stages against the same L2q
+      for (int bs = 0; bs < nbst && ok; ++bs) {
+        ok = mbar_wait_warp(bar(B_EMPTY + st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
+        if (!ok) break;
+        const uint32_t a_dst = sm_stage + st * stage_bytes;
+        const uint32_t full = bar(B_FULL + st);
+        if (elect_one()) {
+          mbar_expect_tx(full, stage_bytes + (p.branch_mx ? SF_BYTES + sfb_bytes : 0));
+          tma_load_2d(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
+          tma_load_2d(a_dst + STAGE_A_BYTES, &tmL2, 0, n0, full);
+          if (p.branch_mx) {   // the block scales of T (rows) and of L2 (columns) along the rank
+            const uint32_t sf_dst = sm_sf + st * STAGE_SF_BYTES;
+            bulk_load(sf_dst, p.sft + ((size_t)mb * nbst + bs) * SF_BYTES, SF_BYTES, full);
+            bulk_load(sf_dst + SF_BYTES, p.sfl2 + (size_t)nu * sfb_bytes, sfb_bytes, full);
+          }
+        }
+        __syncwarp();
+        advance();
+      }
+      if (!ok) break;
       {   // the tile's scale vectors and bias, for the drain
         const int rb = tc & 1;
         ok = mbar_wait_warp(bar(B_REMPTY + rb), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_PRODUCER);
         if (!ok) break;
         if (elect_one()) {
-          const uint32_t rfull = bar(B_RFULL + rb), dst = sm_sc + rb * SC_FLOATS * 4;
-          mbar_expect_tx(rfull, (LQ_BM + 2 * width * UNIT) * 4);
+          const uint32_t rfull = bar(B_RFULL + rb), dst = sm_sc + rb * SC_FLOATS * 4, cb = (uint32_t)min(W, p.Npad - n0) * 4;
+          mbar_expect_tx(rfull, LQ_BM * 4 + 2 * cb);
           bulk_load(dst, p.sT + m0, LQ_BM * 4, rfull);
-          bulk_load(dst + LQ_BM * 4, p.sL2 + n0, width * UNIT * 4, rfull);
-          bulk_load(dst + (LQ_BM + 2 * UNIT) * 4, p.bias + n0, width * UNIT * 4, rfull);
+          bulk_load(dst + LQ_BM * 4, p.sL2 + n0, cb, rfull);
+          bulk_load(dst + (LQ_BM + MAX_W) * 4, p.bias + n0, cb, rfull);
         }
         __syncwarp();
         ++rarmed;
       }
-      for (int s = 0; s < p.k_stages && ok; ++s, ++it) {
-        const int st = it % NSTAGE;
-        ok = mbar_wait_warp(bar(B_EMPTY + st), ((it / NSTAGE) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_PRODUCER);
-        if (!ok) break;
-        LQ_TL(EV_P_SLOT_FREE, s);
-        const uint32_t a_dst = sm_stage + st * STAGE_BYTES, b_dst = a_dst + STAGE_A_BYTES, sf_dst = sm_sf + st * STAGE_SF_BYTES;
-        const uint32_t full = bar(B_FULL + st);
-        if (elect_one()) {
-          mbar_expect_tx(full, STAGE_A_BYTES + width * (UNIT * LQ_KSTAGE) + (1 + width) * SF_BYTES);
-          const int sb = s >= p.b_wrap ? s - p.b_wrap : s;       // the lo digits' plane runs over the same weights
-          tma_load_2d(a_dst, &tmA, s * LQ_KSTAGE, m0, full);
-          if (width == 2) tma_load_2d(b_dst, &tmB2, sb * LQ_KSTAGE, n0, full);
-          else tma_load_2d(b_dst, &tmB, sb * LQ_KSTAGE, n0, full);
-          bulk_load(sf_dst, sfa + (size_t)s * SF_BYTES, SF_BYTES, full);
-          bulk_load(sf_dst + SF_BYTES, sfb + (size_t)sb * p.units_n * SF_BYTES, width * SF_BYTES, full);
-        }
-        __syncwarp();
-        LQ_TL(EV_P_ISSUED, s);
-      }
-      // the branch operands: the containers of tq (128 rows) and L2q (256 rows), r contiguous; mode 3 brings the two
-      // digit planes of tq as two stages against the same L2q
-      for (int bs = 0; bs < nbst && has_branch && ok; ++bs) {
-        const int st = it % NSTAGE;
-        ok = mbar_wait_warp(bar(B_EMPTY + st), ((it / NSTAGE) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_PRODUCER);
-        if (!ok) break;
-        const uint32_t a_dst = sm_stage + st * STAGE_BYTES, b_dst = a_dst + STAGE_A_BYTES;
-        const uint32_t full = bar(B_FULL + st);
-        if (elect_one()) {
-          mbar_expect_tx(full, STAGE_A_BYTES + width * (UNIT * LQ_KSTAGE) + (p.branch_mx ? (1 + width) * SF_BYTES : 0));
-          tma_load_2d(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
-          tma_load_2d(b_dst, &tmL2, 0, n0, full);
-          if (width == 2) tma_load_2d(b_dst + UNIT * LQ_KSTAGE, &tmL2, 0, n0 + UNIT, full);
-          if (p.branch_mx) {   // the block scales of T (rows) and of L2 (columns) along the rank
-            const uint32_t sf_dst = sm_sf + st * STAGE_SF_BYTES;
-            bulk_load(sf_dst, p.sft + ((size_t)mb * nbst + bs) * SF_BYTES, SF_BYTES, full);
-            bulk_load(sf_dst + SF_BYTES, p.sfl2 + (size_t)nu * SF_BYTES, width * SF_BYTES, full);
-          }
-        }
-        __syncwarp();
-        ++it;
-      }
     }
     if (!ok && lane == 0) {
       // aborting: give the copies already issued a bounded time to land before the CTA's shared memory goes away
-      // (`it` stages have been armed; the last NSTAGE of them may still be in flight)
-      const uint32_t n = it < (uint32_t)NSTAGE ? it : (uint32_t)NSTAGE;
-      for (uint32_t i = 1; i <= n; ++i) {
-        const uint32_t j = it - i;
-        mbar_settle(bar(B_FULL + (int)(j % NSTAGE)), (j / NSTAGE) & 1);
+      for (int i = max(min(armed, NST), early); i > 0; --i) {
+        if (--st < 0) { st = NST - 1; par ^= 1; }
+        mbar_settle(bar(B_FULL + st), par ^ 1);
       }
-      for (uint32_t i = 1; i <= (rarmed < 2u ? rarmed : 2u); ++i) {     // and the tiles' scale vectors
+      for (uint32_t i = 1; i <= min(rarmed, 2u); ++i) {                 // and the tiles' scale vectors
         const uint32_t j = rarmed - i;
         mbar_settle(bar(B_RFULL + (int)(j & 1)), (j >> 1) & 1);
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    uint32_t it = 0, tc = 0;
+    uint32_t tc = 0, par = 0;
+    int st = 0;                                        // ring slot and its parity
     bool ok = true;
-    for (int w = w_begin, w_next; w < w_end && ok; w = w_next, ++tc) {
-      int mb, nu, width;
-      w_next = tile_at(w, mb, nu, width);
-      const int ncols = width * UNIT;
-      // the accumulator is free once the drain has read the previous tile out of it
-      ok = mbar_wait_warp(bar(B_TEMPTY), (tc & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
+    const uint32_t tsfa = tmem_base + TM_SFA, tsfb = tmem_base + TM_SFB;
+    auto copy_scales = [&](int st) {
+      const uint32_t sf = sm_sf + st * STAGE_SF_BYTES;
+      tc_cp_sf(tsfa, make_smem_desc_plain(sf, 16, 128));
+      tc_cp_sf(tsfb, make_smem_desc_plain(sf + SF_BYTES, 16, 128));
+      if (p.sf_chunks == 2) tc_cp_sf(tsfb + 4, make_smem_desc_plain(sf + 2 * SF_BYTES, 16, 128));
+    };
+    for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
+      const int buf = tc & 1;
+      const uint32_t d = tmem_base + (uint32_t)(buf * W);
+      // the accumulator is free once the drain has read the tile before last out of it
+      ok = mbar_wait_warp(bar(B_TEMPTY + buf), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
       if (!ok) break;
       tc_fence_after();
       LQ_TL(EV_M_ACC_FREE, 0);
-      for (int s = 0; s < p.k_stages && ok; ++s, ++it) {
-        const int st = it % NSTAGE;
-        ok = mbar_wait_warp(bar(B_FULL + st), (it / NSTAGE) & 1, abort_flag, p.status, LQ_STAGE_MMA);
+      for (int s = 0; s < p.k_stages; ++s) {
+        ok = mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA);
         if (!ok) break;
         tc_fence_after();
         LQ_TL(EV_M_STAGE_FULL, s);
-        const uint32_t a_addr = sm_stage + st * STAGE_BYTES, b_addr = a_addr + STAGE_A_BYTES, sf_addr = sm_sf + st * STAGE_SF_BYTES;
-        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(b_addr);
-        const uint32_t tsfa = tmem_base + TM_SFA, tsfb = tmem_base + TM_SFB;
-        if (elect_one()) {
-          tc_cp_sf(tsfa, make_smem_desc_plain(sf_addr, 16, 128));
-          tc_cp_sf(tsfb, make_smem_desc_plain(sf_addr + SF_BYTES, 16, 128));
-          if (width == 2) tc_cp_sf(tsfb + 4, make_smem_desc_plain(sf_addr + 2 * SF_BYTES, 16, 128));
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            tc_mma_mx(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc_mx(ncols, j), tsfa, tsfb, (uint32_t)(s | j));
-          tc_commit(bar(B_EMPTY + st));
-        }
-        __syncwarp();
+        const uint32_t a_addr = sm_stage + st * stage_bytes;
+        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + STAGE_A_BYTES);
+        const uint32_t sf = sm_sf + st * STAGE_SF_BYTES;
+        issue_main_stage(d, adesc, bdesc, idesc_mx(W, 0), make_smem_desc_plain(sf, 16, 128), make_smem_desc_plain(sf + SF_BYTES, 16, 128),
+                         (uint32_t)(p.sf_chunks == 2), (uint32_t)s, bar(B_EMPTY + st));
+        if (++st == NST) { st = 0; par ^= 1; }
         LQ_TL(EV_M_ISSUED, s);
       }
-      if (!ok) break;
-      for (int bs = 0; bs < nbst && has_branch; ++bs) {
-        const int st = it % NSTAGE;
-        ok = mbar_wait_warp(bar(B_FULL + st), (it / NSTAGE) & 1, abort_flag, p.status, LQ_STAGE_MMA);
+      for (int bs = 0; bs < nbst && ok; ++bs) {
+        ok = mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA);
         if (!ok) break;
-        if (branch_acc) {
+        if (BRANCH_ACC) {
           // the drain has read the previous tile's branch accumulator (long ago: it does that under this tile's main loop)
           ok = mbar_wait_warp(bar(B_BEMPTY), (tc & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
           if (!ok) break;
         }
         tc_fence_after();
-        const uint32_t a_addr = sm_stage + st * STAGE_BYTES, b_addr = a_addr + STAGE_A_BYTES;
-        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(b_addr);
+        const uint32_t a_addr = sm_stage + st * stage_bytes;
+        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + STAGE_A_BYTES);
         if (elect_one()) {
           if (p.branch_mx) {
-            const uint32_t sf_addr = sm_sf + st * STAGE_SF_BYTES, tsfa = tmem_base + TM_SFA, tsfb = tmem_base + TM_SFB;
-            tc_cp_sf(tsfa, make_smem_desc_plain(sf_addr, 16, 128));
-            tc_cp_sf(tsfb, make_smem_desc_plain(sf_addr + SF_BYTES, 16, 128));
-            if (width == 2) tc_cp_sf(tsfb + 4, make_smem_desc_plain(sf_addr + 2 * SF_BYTES, 16, 128));
+            copy_scales(st);
             if (p.branch_mx == 2) {
               for (int c = 0; c < p.branch_steps; ++c)
                 for (int q = 0; q < 4; ++q) {
                   const int ja = c + 2 * (q >> 1), jb = c + 2 * (q & 1);   // K block of T's plane, of L2's plane
-                  tc_mma_mx(tmem_base, adesc + 2 * ja, bdesc + 2 * jb, idesc_mx2(ncols, ja, jb), tsfa, tsfb, 1u);
+                  tc_mma_mx(d, adesc + 2 * ja, bdesc + 2 * jb, idesc_mx2(W, ja, jb), tsfa, tsfb, 1u);
                 }
             } else {
               for (int j = 0; j < p.branch_steps; ++j)
-                tc_mma_mx(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc_mx(ncols, j), tsfa, tsfb, 1u);
+                tc_mma_mx(d, adesc + 2 * j, bdesc + 2 * j, idesc_mx(W, j), tsfa, tsfb, 1u);
             }
           } else {
             for (int j = 0; j < p.branch_steps; ++j) {
-              if (branch_acc) tc_mma<TC_I8>(tmem_base + TM_BR, adesc + 2 * j, bdesc + 2 * j, IDESC_I8 | idesc_shape(ncols), (uint32_t)j);
-              else tc_mma<TC_F16>(tmem_base, adesc + 2 * j, bdesc + 2 * j, IDESC_F16 | idesc_shape(ncols), 1u);   // 16 halves each
+              if (BRANCH_ACC) tc_mma<TC_I8>(tmem_base + 2 * W, adesc + 2 * j, bdesc + 2 * j, IDESC_I8 | idesc_shape(W), (uint32_t)j);
+              else tc_mma<TC_F16>(d, adesc + 2 * j, bdesc + 2 * j, IDESC_F16 | idesc_shape(W), 1u);   // 16 halves each
             }
           }
           tc_commit(bar(B_EMPTY + st));
         }
         __syncwarp();
-        ++it;
+        if (++st == NST) { st = 0; par ^= 1; }
       }
       if (!ok) break;
-      if (elect_one()) tc_commit(bar(B_TFULL));
+      if (elect_one()) tc_commit(bar(B_TFULL + buf));
       __syncwarp();
       LQ_TL(EV_TILE, 0);
     }
   } else {
     // ------------------------------------------------------------------ drain + epilogue
     const int quad = warp & 3;                          // tensor-memory lanes 32*quad .. 32*quad+31
-    const int cgi = (warp - FIRST_DRAIN_WARP) >> 2;     // which 32 columns of each 128-column half
-    const int g = lane >> 2, t = lane & 3;              // fragment coordinates: rows g and g + 8, column pair t
-    const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(cgi * 32);
+    const int cgi = (warp - FIRST_DRAIN_WARP) >> 2;     // blocks of 32 columns cgi, cgi + 4
+    const int g = lane >> 2, t = lane & 3;              // fragment coordinates: rows g + 8 i, eight columns from 8 t
+    const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16);
+    const int blocks = W >> 5;
     uint32_t tc = 0;
     bool ok = true;
-    for (int w = w_begin, w_next; w < w_end && ok; w = w_next, ++tc) {
-      int mb, nu, width;
-      w_next = tile_at(w, mb, nu, width);
-      const int m0 = mb * LQ_BM, n0 = nu * UNIT;
-      const int rl = quad * 32 + g;                     // this thread's rows inside the tile: rl + 16 mt and + 8
-      const int cl = cgi * 32;                          // this warp's columns inside a half: cl + 8 nt + ...
-      const int rb = tc & 1;
-      float acc[2][2][4][4];                            // [half][m16 tile][n8 tile][fragment register]
-      uint32_t w0[2][8];                                // cgi == 0: the branch columns that the scale factors alias
+    grid_dependency_wait();                             // Y may be what an earlier kernel still reads
+    for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
+      const int mb = w / p.tiles_n, nu = w - mb * p.tiles_n;
+      const int buf = tc & 1;
       LQ_TL(EV_D_OPEN, 0);
-      ok = mbar_wait_idle(bar(B_TFULL), tc & 1, abort_flag, p.status, LQ_STAGE_DRAIN);
+      ok = mbar_wait_warp(bar(B_TFULL + buf), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN) &&
+           mbar_wait_warp(bar(B_RFULL + buf), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN);
       if (!ok) break;
       tc_fence_after();
       LQ_TL(EV_D_ACC_FULL, 0);
-      // hand-over: every load is issued before the one wait; the main accumulator lands in the registers it stays in
+      const float* sc = sc_ptr + buf * SC_FLOATS;
+      const int row0 = quad * 32 + g;                   // this thread's rows inside the tile: row0 + 8 i
+#pragma unroll 1
+      for (int b = cgi; b < blocks; b += 4) {
+        uint32_t v[2][16], u[BRANCH_ACC ? 2 : 1][16];
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (h < width) {
+        for (int h = 0; h < 2; ++h) tmem_ld_16x256b_x4(tlane + ((uint32_t)(16 * h) << 16) + buf * W + 32 * b, v[h]);
+        if constexpr (BRANCH_ACC) {
 #pragma unroll
-          for (int mt = 0; mt < 2; ++mt)
-            tmem_ld_16x256b_x4(tlane + ((uint32_t)(16 * mt) << 16) + h * UNIT, reinterpret_cast<uint32_t(&)[16]>(acc[h][mt]));
+          for (int h = 0; h < 2; ++h) tmem_ld_16x256b_x4(tlane + ((uint32_t)(16 * h) << 16) + 2 * W + 32 * b, u[h]);
         }
-      if (branch_acc && cgi == 0) {
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) tmem_ld_16x256b_x2(tlane + ((uint32_t)(16 * mt) << 16) + TM_BR, w0[mt]);
-      }
-      tmem_ld_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_TEMPTY));
-      LQ_TL(EV_D_LOADED, 0);
-      // y = main + U sT sL2 + bias, under the next tile's main loop (the tensor core has already applied the block
-      // scales to main)
-      ok = mbar_wait(bar(B_RFULL + rb), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN);
-      if (!ok) break;
-      {
-        const float* sc = sc_ptr + rb * SC_FLOATS;
-        const float* sc_l2 = sc + LQ_BM + cl + 2 * t;
-        const float* sc_b = sc + LQ_BM + 2 * UNIT + cl + 2 * t;
-        if (branch_acc && cgi == 0) {                  // the early-read columns first: their registers are free again
-#pragma unroll
-          for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-              combine_fragment(acc[0][mt][nt], &w0[mt][4 * nt], true, sc[rl + 16 * mt], sc[rl + 16 * mt + 8],
-                               *reinterpret_cast<const float2*>(sc_l2 + nt * 8), *reinterpret_cast<const float2*>(sc_b + nt * 8));
+        const float* cb = sc + LQ_BM + MAX_W + 32 * b + 8 * t;
+        const float4 b0 = *reinterpret_cast<const float4*>(cb), b1 = *reinterpret_cast<const float4*>(cb + 4);
+        const float bias[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        float sl[8];
+        if constexpr (BRANCH_ACC) {
+          const float4 l0 = *reinterpret_cast<const float4*>(cb - MAX_W), l1 = *reinterpret_cast<const float4*>(cb - MAX_W + 4);
+          sl[0] = l0.x; sl[1] = l0.y; sl[2] = l0.z; sl[3] = l0.w; sl[4] = l1.x; sl[5] = l1.y; sl[6] = l1.z; sl[7] = l1.w;
         }
+        tmem_ld_wait();
+        if (b + 4 >= blocks) {                          // this warp's last block: the accumulators go back
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(bar(B_TEMPTY + buf));
+            if (BRANCH_ACC) mbar_arrive(bar(B_BEMPTY));
+          }
+          LQ_TL(EV_D_LOADED, 0);
+        }
+        const int c = nu * W + 32 * b + 8 * t;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h < width) {
+        for (int i = 0; i < 4; ++i) {
+          // fragment registers 4 j .. 4 j + 3: row g, columns 2 j, 2 j + 1 of this lane's eight, then row g + 8 the same columns.
+          // U is an exact int32 with |U| < 2^22: converted exactly with the 1.5 * 2^23 trick
+          const int h = i >> 1, q = 2 * (i & 1), r = mb * LQ_BM + row0 + 8 * i;
+          float y[8];
+          const float st = BRANCH_ACC ? sc[row0 + 8 * i] : 0.f;
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-              uint32_t w[16];
-              const bool early = branch_acc && cgi == 0 && h == 0;       // fragments 0 and 1 are done already
-              if (branch_acc) {
-                const uint32_t ta = tlane + ((uint32_t)(16 * mt) << 16) + TM_BR + h * UNIT;
-                if (early) tmem_ld_16x256b_x2(ta + TM_SF_ALIASED, reinterpret_cast<uint32_t(&)[8]>(w[8]));
-                else tmem_ld_16x256b_x4(ta, w);
-                tmem_ld_wait();
+          for (int j = 0; j < 8; ++j) {
+            y[j] = __uint_as_float(v[h][4 * (j >> 1) + q + (j & 1)]) + bias[j];
+            if constexpr (BRANCH_ACC)
+              y[j] = fmaf(__int_as_float((int)u[h][4 * (j >> 1) + q + (j & 1)] + 0x4B400000) - 12582912.0f, st * sl[j], y[j]);
+          }
+          if (r < p.M && c < p.N) {
+            if (p.out_f32) {
+              float4* Y = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c);
+              Y[0] = make_float4(y[0], y[1], y[2], y[3]);
+              Y[1] = make_float4(y[4], y[5], y[6], y[7]);
+            } else {
+              uint32_t o[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const __half2 x = __floats2half2_rn(y[2 * j], y[2 * j + 1]);
+                o[j] = *reinterpret_cast<const uint32_t*>(&x);
               }
-              const float st_lo = sc[rl + 16 * mt], st_hi = sc[rl + 16 * mt + 8];
-#pragma unroll
-              for (int nt = 0; nt < 4; ++nt) {
-                if (nt < 2 && early) continue;
-                combine_fragment(acc[h][mt][nt], &w[4 * nt], branch_acc, st_lo, st_hi,
-                                 *reinterpret_cast<const float2*>(sc_l2 + h * UNIT + nt * 8),
-                                 *reinterpret_cast<const float2*>(sc_b + h * UNIT + nt * 8));
-              }
+              *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c) = make_uint4(o[0], o[1], o[2], o[3]);
             }
           }
         }
       }
-      tc_fence_before();
       __syncwarp();
-      if (lane == 0) { mbar_arrive(bar(B_BEMPTY)); mbar_arrive(bar(B_REMPTY + rb)); }
-      LQ_TL(EV_D_DONE, 0);
-      // epilogue
-      const int row_w = m0 + quad * 32;                 // first row of this group's part
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h < width) {
-          if (p.out_f32) {
-            float* Y = reinterpret_cast<float*>(p.Y);
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-              const int r_lo = row_w + g + 16 * mt, r_hi = r_lo + 8;
-#pragma unroll
-              for (int nt = 0; nt < 4; ++nt) {
-                const int c = n0 + h * UNIT + cl + nt * 8 + 2 * t;
-                if (c < p.N) {
-                  if (r_lo < p.M) *reinterpret_cast<float2*>(Y + (size_t)r_lo * p.N + c) = make_float2(acc[h][mt][nt][0], acc[h][mt][nt][1]);
-                  if (r_hi < p.M) *reinterpret_cast<float2*>(Y + (size_t)r_hi * p.N + c) = make_float2(acc[h][mt][nt][2], acc[h][mt][nt][3]);
-                }
-              }
-            }
-          } else {
-            __half* Y = reinterpret_cast<__half*>(p.Y);
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-              // pack to fp16, then exchange inside the quad: lane t ends up with columns 8 t .. 8 t + 7 of both rows
-              uint32_t lo[4], hi[4];
-#pragma unroll
-              for (int nt = 0; nt < 4; ++nt) {
-                const __half2 l2 = __floats2half2_rn(acc[h][mt][nt][0], acc[h][mt][nt][1]);
-                const __half2 h2 = __floats2half2_rn(acc[h][mt][nt][2], acc[h][mt][nt][3]);
-                lo[nt] = *reinterpret_cast<const uint32_t*>(&l2);
-                hi[nt] = *reinterpret_cast<const uint32_t*>(&h2);
-              }
-              quad_transpose(lo, t);
-              quad_transpose(hi, t);
-              // each lane owns 16 contiguous bytes of a row: a store instruction writes whole 32-byte sectors
-              const int c = n0 + h * UNIT + cl + 8 * t;
-              const int r_lo = row_w + g + 16 * mt, r_hi = r_lo + 8;
-              if (c < p.N) {
-                if (r_lo < p.M) *reinterpret_cast<uint4*>(Y + (size_t)r_lo * p.N + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                if (r_hi < p.M) *reinterpret_cast<uint4*>(Y + (size_t)r_hi * p.N + c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-              }
-            }
-          }
+      if (lane == 0) {
+        mbar_arrive(bar(B_REMPTY + buf));
+        if (cgi >= blocks) {                            // a tile narrower than 128 columns has nothing for this warp
+          mbar_arrive(bar(B_TEMPTY + buf));
+          if (BRANCH_ACC) mbar_arrive(bar(B_BEMPTY));
         }
       }
       LQ_TL(EV_D_EPI_END, 0);
@@ -497,15 +458,39 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   }
 }
 
+// Ring depth that fits beside the fixed part.
+int ring_stages(int width) {
+  return std::min(MAX_STAGES, (MAX_SMEM - FIXED_SMEM) / (STAGE_A_BYTES + width * LQ_KSTAGE + STAGE_SF_BYTES));
+}
+int smem_bytes(int width) {
+  return FIXED_SMEM + ring_stages(width) * (STAGE_A_BYTES + width * LQ_KSTAGE + STAGE_SF_BYTES);
+}
+
+// Index (LQ_MX_WIDTHS) of the tile width for a launch.  Model, in clocks: a stage takes the longer of its MMAs (2 W) and its
+// operands' way from the L2 (70 bytes per clock and SM); a tile the longer of its stages and the drain of the tile before; a
+// launch the tiles of the CTA with the most, plus the last drain and the filling of the ring.
+int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas) {
+  int best = -1;
+  double best_cost = 1e30;
+  for (int i = 0; i < LQ_MX_NWIDTHS; ++i) {
+    if (!L->d_sfbw[i]) continue;
+    const int w = LQ_MX_WIDTHS[i];
+    if (g_lq_gemm_width > 0 && w != g_lq_gemm_width) continue;
+    const long long tiles = (long long)tiles_m * lq_ceil_div(L->N, w);
+    const double stage = std::max(2.0 * w, (STAGE_A_BYTES + w * LQ_KSTAGE) / 70.0);
+    const double drain = 600.0 + 1200.0 * lq_ceil_div(w, 128);
+    const double cost = (double)((tiles + ctas - 1) / ctas) * std::max(stages * stage, drain) + drain + 4.0 * stage;
+    if (cost < best_cost) { best_cost = cost; best = i; }
+  }
+  return best;
+}
+
 }  // namespace
 
 lq_status lq_gemm_mx_prepare(int device) {
   if (cudaSetDevice(device) != cudaSuccess) return LQ_ERR_CUDA;
-  if (lq_note_cuda(cudaFuncSetAttribute(lq_gemm_mx_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) !=
-          cudaSuccess ||
-      lq_note_cuda(cudaFuncSetAttribute(lq_gemm_mx_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) !=
-      cudaSuccess)
-    return LQ_ERR_CUDA;
+  for (auto* kernel : {lq_gemm_mx_kernel<false>, lq_gemm_mx_kernel<true>})
+    if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM)) != cudaSuccess) return LQ_ERR_CUDA;
   return LQ_OK;
 }
 
@@ -513,29 +498,28 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   if (cudaSetDevice(A->device) != cudaSuccess) return LQ_ERR_CUDA;
   if (!L->mx || !A->mx) return LQ_ERR_UNSUPPORTED;
   MxParams p;
-  p.M = A->M; p.N = L->N; p.Mpad = A->Mpad; p.Npad = L->Npad;
+  p.M = A->M; p.N = L->N; p.Npad = L->Npad;
   p.b_wrap = L->Kpad / LQ_KSTAGE;
   p.k_stages = p.b_wrap * A->planes;
   p.branch_f16 = L->f16_branch ? 1 : 0;
   p.branch_mx = L->r == 0 ? 0 : L->mxfp ? 1 : !L->a8 ? 0 : L->cfg.branch == LQ_BRANCH_MXINT4 ? 3 : 2;
-  p.sft = A->d_sft; p.sfl2 = L->d_sfl2;
   p.branch_steps = L->r == 0 ? 0 : lq_ceil_div(L->r, L->f16_branch ? 16 : 32);   // a8: rank blocks of 32 (at most two)
   p.tiles_m = lq_ceil_div(A->M, LQ_BM);
-  p.units_n = L->Npad / UNIT;
-  p.sfa = A->d_sfa; p.sfb = L->d_sfb; p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
-  p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device) != cudaSuccess) return LQ_ERR_CUDA;
   int ctas = g_lq_gemm_ctas > 0 ? g_lq_gemm_ctas : sms;
-  const long long tiles = (long long)p.tiles_m * ((p.units_n + 1) / 2);
+  const int wi = pick_width(L, p.tiles_m, p.k_stages + (L->r > 0), ctas);
+  if (wi < 0) return LQ_ERR_INVALID_ARG;
+  p.width = LQ_MX_WIDTHS[wi]; p.stages = ring_stages(p.width); p.sf_chunks = lq_ceil_div(p.width, 128);
+  p.tiles_n = lq_ceil_div(L->N, p.width);
+  p.sfa = A->d_sfa; p.sfb = L->d_sfbw[wi]; p.sft = A->d_sft; p.sfl2 = L->d_sfl2w[wi];
+  p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
+  p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
+  const long long tiles = (long long)p.tiles_m * p.tiles_n;
   if (ctas > tiles) ctas = (int)tiles;
-  p.by_units = (p.units_n & 1) && tiles < 4ll * ctas;
-  cudaError_t launched;
-  if (p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx)
-    launched = lq_launch(lq_gemm_mx_kernel<true>, ctas, GEMM_THREADS, SMEM_BYTES, st, A->tmA, L->tmB, L->tmB2, A->tmT, L->tmL2, p);
-  else
-    launched = lq_launch(lq_gemm_mx_kernel<false>, ctas, GEMM_THREADS, SMEM_BYTES, st, A->tmA, L->tmB, L->tmB2, A->tmT, L->tmL2, p);
-  return lq_note_cuda(launched != cudaSuccess ? launched : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
+  auto* kernel = p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx ? lq_gemm_mx_kernel<true> : lq_gemm_mx_kernel<false>;
+  const cudaError_t e = lq_launch(kernel, ctas, GEMM_THREADS, (size_t)smem_bytes(p.width), st, A->tmA, L->tmBw[wi], A->tmT, L->tmL2w[wi], p);
+  return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

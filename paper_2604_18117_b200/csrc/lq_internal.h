@@ -32,17 +32,25 @@ static inline size_t lq_sf_offset(int i, int kb, int Kpad) {
   return ((size_t)(i / 128) * (Kpad / 128) + kb / 4) * 512 + 16 * (i % 32) + 4 * ((i % 128) / 32) + kb % 4;
 }
 
-// the same for the weight scales, whose chunks are ordered [kb/4][tile] so that neighbouring column tiles are contiguous
-static inline size_t lq_sfb_offset(int n, int kb, int Npad) {
-  return ((size_t)(kb / 4) * (Npad / 128) + n / 128) * 512 + 16 * (n % 32) + 4 * ((n % 128) / 32) + kb % 4;
+// Tile widths the MX GEMM is launched with.  Layers with an integer branch, whose product needs a third accumulator in tensor
+// memory, go up to 160 columns, the others up to 224.
+constexpr int LQ_MX_WIDTHS[] = {64, 128, 160, 192, 224};
+constexpr int LQ_MX_NWIDTHS = 5;
+static inline bool lq_mx_width_used(int width, bool branch_acc) { return branch_acc ? width <= 160 : width != 160; }
+// the same for the weight scales of operand row n when the columns are cut in `tiles` tiles of `width`: chunks [kb/4][tile][half]
+static inline size_t lq_sfb_offset(int n, int kb, int width, int tiles) {
+  const int i = n % width, chunks = lq_ceil_div(width, 128);
+  return (((size_t)(kb / 4) * tiles + n / width) * chunks + i / 128) * 512 + 16 * (i % 32) + 4 * ((i % 128) / 32) + kb % 4;
 }
 
-// Orders the SINT4 GEMM's operands are laid out in, for the accumulator fragments its drain lanes hold (rows g, g + 8, g + 16,
+// Orders the GEMMs' operands are laid out in, for the accumulator fragments its drain lanes hold (rows g, g + 8, g + 16,
 // g + 24 of 32; columns 8 j + 2 t + {0, 1} of 64):
 //   place of row m in the row-scale vectors: a lane's four are neighbours
 __host__ __device__ static inline int lq_row_slot(int m) { return (m & ~31) | ((m & 7) << 2) | ((m >> 3) & 3); }
 //   row of the weight operand that carries output column n: a lane's 16 columns are neighbours in the output
 static inline int lq_col_slot(int n) { return (n & ~63) | (((n >> 1) & 7) << 3) | (((n >> 4) & 3) << 1) | (n & 1); }
+//   the same for the MX GEMM, whose lanes hold eight columns of 32
+static inline int lq_col32_slot(int n) { return (n & ~31) | (((n >> 1) & 3) << 3) | (((n >> 3) & 3) << 1) | (n & 1); }
 //   place of column n in the column-scale vectors and the bias: a lane's come in four 16-byte loads, neighbours across lanes
 static inline int lq_colscale_slot(int n) { return (n & ~63) | (((n >> 2) & 3) << 4) | (((n >> 4) & 3) << 2) | (n & 3); }
 
@@ -92,21 +100,22 @@ struct lq_layer {
   // device copy, operand layouts
   int device;
   int main_kind;               // LQ_KIND_*: byte encoding of the 4-bit codes in the MMA operands
-  uint8_t* d_Wq8;              // [Npad][Kpad] bytes, K contiguous (B operand, K-major; SINT4: rows in lq_col_slot order)
+  uint8_t* d_Wq8;              // [Npad][Kpad] bytes, K contiguous (B operand, K-major; rows in lq_col_slot order, MX: lq_col32_slot)
   float* d_sw;                 // [Gpad][Npad] fp32 (exact images of the fp16 scales), in lq_colscale_slot order
   uint8_t* d_L1c;              // [planes * rn][Kpad] bytes (W16A16: [rn][Kpad] halves), K contiguous: first factor as the B operand of
                                // the down-projection; rn = lq_l1_rows; MXINT8 factors: the hi digits' rows, then the lo digits'
   uint8_t* d_sfl1;             // MX branches: E8M0 bytes of L1's block scales, [Kpad/128][512] in the tensor-memory layout (row = row of d_L1c)
   float* d_sL1;                // [LQ_MAX_RANK]
   uint8_t* d_L2c;              // [Npad][LQ_RCONT] bytes: int8 codes (or up to 64 halves) of column n, r contiguous
-  float* d_sL2;                // [Npad]  (ones for W16A16); SINT4: d_L2c in lq_col_slot order, d_sL2 and d_bias in
+  float* d_sL2;                // [Npad]  (ones for W16A16); d_L2c in d_Wq8's row order; SINT4: d_sL2 and d_bias in
                                // lq_colscale_slot order
   float* d_bias;               // [Npad]  (zeros without bias)
-  uint8_t* d_sfl2;             // mxfp: E8M0 bytes of L2's block scales, [1][Npad/128][512] in the tensor-memory layout
-  uint8_t* d_sfb;              // MXINT4: E8M0 bytes of the weight scales, [Kpad/128][Npad/128][512] in the 32 x 16-byte
-                               // layout tensor memory wants (byte 16*(n%32) + 4*((n%128)/32) + block%4)
+  // MX, one per tile width in use (LQ_MX_WIDTHS):
+  uint8_t* d_sfbw[LQ_MX_NWIDTHS];   // E8M0 bytes of the weight scales, [Kpad/128][tiles][ceil(width/128)][512] in the 32 x 16-byte
+                                    // layout tensor memory wants (byte 16*(i%32) + 4*((i%128)/32) + block%4)
+  uint8_t* d_sfl2w[LQ_MX_NWIDTHS];  // MX branches: the same for L2's block scales along the rank, [tiles][ceil(width/128)][512]
+  CUtensorMap tmBw[LQ_MX_NWIDTHS], tmL2w[LQ_MX_NWIDTHS];   // over d_Wq8 and d_L2c, box [width][128B], 128B swizzle
   CUtensorMap tmB;             // over d_Wq8, box [LQ_BN][128B], 128B swizzle
-  CUtensorMap tmB2;            // over d_Wq8, box [2 LQ_BN][128B]: both halves of a 256-column tile in one copy
   CUtensorMap tmL1;            // over d_L1c, box [all rows][128B], 128B swizzle
   CUtensorMap tmL2;            // over d_L2c, box [LQ_BN][128B], 128B swizzle
 };
@@ -168,6 +177,7 @@ static inline uint8_t lq_encode_code_host(int q, int kind) {
 
 extern int g_lq_main_kind;   // option "main_kind"
 extern int g_lq_gemm_ctas;   // option "gemm_ctas" (0 = one per SM)
+extern int g_lq_gemm_width;  // option "gemm_width": tile width of the MX GEMM, 0 = chosen by the launcher
 extern int g_lq_quant_warps, g_lq_quant_ctas;   // options "quant_warps", "quant_ctas": the quantizer's row groups per tile and stages per chunk, 0 = chosen by the launcher
 extern int g_lq_overlap;     // option "overlap": launch kernels with programmatic stream serialization
 extern int g_lq_store_qb;    // option "store_qb": also write the branch activation codes to HBM (parity export)
