@@ -12,6 +12,7 @@
 int g_lq_main_kind = LQ_KIND_E4M3;
 int g_lq_gemm_ctas = 0;
 int g_lq_gemm_width = 0;
+int g_lq_gemm_pair = 1;
 int g_lq_store_qb = 0;
 int g_lq_quant_warps = 0;
 int g_lq_quant_ctas = 0;
@@ -80,6 +81,11 @@ extern "C" lq_status lq_set_option(const char* name, int32_t value) {
   if (!strcmp(name, "gemm_width")) {
     if (value != 0 && std::find(LQ_MX_WIDTHS, LQ_MX_WIDTHS + LQ_MX_NWIDTHS, value) == LQ_MX_WIDTHS + LQ_MX_NWIDTHS) return LQ_ERR_INVALID_ARG;
     g_lq_gemm_width = value;
+    return LQ_OK;
+  }
+  if (!strcmp(name, "gemm_pair")) {
+    if (value != 0 && value != 1) return LQ_ERR_INVALID_ARG;
+    g_lq_gemm_pair = value;
     return LQ_OK;
   }
   if (!strcmp(name, "gemm_ctas")) {
@@ -557,8 +563,11 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
   if ((st = lq_make_tmap_bytes(&L->tmB, L->d_Wq8, Npad, Kpad, LQ_BN)) != LQ_OK) return st;
   for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
     if (!L->d_sfbw[wi]) continue;
-    if ((st = lq_make_tmap_bytes(&L->tmBw[wi], L->d_Wq8, Npad, Kpad, (uint32_t)LQ_MX_WIDTHS[wi])) != LQ_OK) return st;
-    if ((st = lq_make_tmap_bytes(&L->tmL2w[wi], L->d_L2c, Npad, LQ_RCONT, (uint32_t)LQ_MX_WIDTHS[wi])) != LQ_OK) return st;
+    const uint32_t width = (uint32_t)LQ_MX_WIDTHS[wi];
+    if ((st = lq_make_tmap_bytes(&L->tmBw[wi], L->d_Wq8, Npad, Kpad, width)) != LQ_OK) return st;
+    if ((st = lq_make_tmap_bytes(&L->tmL2w[wi], L->d_L2c, Npad, LQ_RCONT, width)) != LQ_OK) return st;
+    if ((st = lq_make_tmap_bytes(&L->tmBp[wi], L->d_Wq8, Npad, Kpad, width / 2)) != LQ_OK) return st;
+    if ((st = lq_make_tmap_bytes(&L->tmL2p[wi], L->d_L2c, Npad, LQ_RCONT, width / 2)) != LQ_OK) return st;
   }
   if (r > 0 && (st = lq_make_tmap_bytes(&L->tmL1, L->d_L1c, (uint64_t)rn * lq_l1_planes(L), (uint64_t)Kpad * (L->f16_branch ? 2 : 1),
                                         (uint32_t)(rn * lq_l1_planes(L)))) != LQ_OK) return st;

@@ -60,7 +60,7 @@ constexpr int SC_FLOATS = LQ_BM + 2 * MAX_W;       // per tile: sT[128], sL2[W],
 constexpr int NUM_DRAIN_WARPS = 16;
 constexpr int FIRST_DRAIN_WARP = 2;
 constexpr int GEMM_THREADS = (FIRST_DRAIN_WARP + NUM_DRAIN_WARPS) * 32;
-constexpr int SMEM_BAR_BYTES = 256;
+constexpr int SMEM_BAR_BYTES = 320;
 constexpr int FIXED_SMEM = 1024 /*alignment slack*/ + 2 * SC_FLOATS * 4 + SMEM_BAR_BYTES;
 constexpr int MAX_SMEM = 227 * 1024;
 // tensor-memory columns: accumulators at 0 and W, the branch's at 2 W; 4 columns of A scales and 8 of B scales
@@ -96,7 +96,7 @@ struct MxParams {
 // stays uniform and their addresses and descriptors in uniform registers.  (Inside an `if` of one lane every operand
 // is moved there instruction by instruction: 320-370 clocks for the MMA warp's stage and 270 for the producer's.)
 //   main stage of the MMA warp: scale bytes to tensor memory, four K = 32 MMAs, the stage's return
-__device__ __forceinline__ void issue_main_stage(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint64_t sfa, uint64_t sfb, uint32_t two,
+__device__ __forceinline__ void issue_main_stage_one(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint64_t sfa, uint64_t sfb, uint32_t two,
                                                  uint32_t accumulate, uint32_t empty) {
   asm volatile(
       "{\n\t.reg .pred P, Q, T, A;\n\t"
@@ -115,6 +115,27 @@ __device__ __forceinline__ void issue_main_stage(uint32_t d, uint64_t a, uint64_
       ::"r"(d), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "l"(sfa), "l"(sfb),
       "l"(sfb + (SF_BYTES >> 4)), "r"(two), "r"(accumulate), "r"((uint32_t)TM_SFA), "r"((uint32_t)TM_SFB), "r"((uint32_t)(TM_SFB + 4)),
       "r"(idesc), "r"(idesc | idesc_mx_ids(1)), "r"(idesc | idesc_mx_ids(2)), "r"(idesc | idesc_mx_ids(3)), "r"(empty)
+      : "memory");
+}
+__device__ __forceinline__ void issue_main_stage_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint64_t sfa, uint64_t sfb, uint32_t two,
+                                                 uint32_t accumulate, uint32_t empty) {
+  asm volatile(
+      "{\n\t.reg .pred P, Q, T, A;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "setp.ne.and.b32 Q, %12, 0, P;\n\t"
+      "setp.ne.b32 A, %13, 0;\n\t"
+      "setp.eq.b32 T, 0, 0;\n\t"
+      "@P tcgen05.cp.cta_group::2.32x128b.warpx4 [%14], %9;\n\t"
+      "@P tcgen05.cp.cta_group::2.32x128b.warpx4 [%15], %10;\n\t"
+      "@Q tcgen05.cp.cta_group::2.32x128b.warpx4 [%16], %11;\n\t"
+      "@P tcgen05.mma.cta_group::2.kind::mxf8f6f4.block_scale [%0], %1, %5, %17, [%14], [%15], A;\n\t"
+      "@P tcgen05.mma.cta_group::2.kind::mxf8f6f4.block_scale [%0], %2, %6, %18, [%14], [%15], T;\n\t"
+      "@P tcgen05.mma.cta_group::2.kind::mxf8f6f4.block_scale [%0], %3, %7, %19, [%14], [%15], T;\n\t"
+      "@P tcgen05.mma.cta_group::2.kind::mxf8f6f4.block_scale [%0], %4, %8, %20, [%14], [%15], T;\n\t"
+      "@P tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%21], %22;\n\t}"
+      ::"r"(d), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "l"(sfa), "l"(sfb),
+      "l"(sfb + (SF_BYTES >> 4)), "r"(two), "r"(accumulate), "r"((uint32_t)TM_SFA), "r"((uint32_t)TM_SFB), "r"((uint32_t)(TM_SFB + 4)),
+      "r"(idesc), "r"(idesc | idesc_mx_ids(1)), "r"(idesc | idesc_mx_ids(2)), "r"(idesc | idesc_mx_ids(3)), "r"(empty), "h"((uint16_t)3)
       : "memory");
 }
 //   main stage of the producer: the weights' half (which announces the whole stage) and the activations' half
@@ -141,7 +162,9 @@ __device__ __forceinline__ void load_acts_stage(uint32_t full, uint32_t dst, con
 
 // BRANCH_ACC: the layer has an integer branch with fp32 scales, whose product needs an accumulator of its own.  The
 // other instance (no branch, fp16 branch, MX branches) carries none of that code or its registers.
-template <bool BRANCH_ACC>
+// PAIR: two CTAs of a cluster work on 256 rows x W columns (cta_group::2): each stages its own 128 rows of A and half of the
+// tile's columns of B, and each SM's tensor core reads B from both.
+template <bool BRANCH_ACC, bool PAIR>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
@@ -150,14 +173,17 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base - smem_u32(smem_raw));
   const int W = p.width, NST = p.stages;
-  const uint32_t stage_bytes = STAGE_A_BYTES + (uint32_t)W * LQ_KSTAGE, b_bytes = (uint32_t)W * LQ_KSTAGE;
+  constexpr int CTAS = PAIR ? 2 : 1;
+  const int BW = W / CTAS;                                // columns of B in this CTA's shared memory
+  const uint32_t rank = PAIR ? blockIdx.x & 1 : 0;
+  const uint32_t stage_bytes = STAGE_A_BYTES + (uint32_t)BW * LQ_KSTAGE;
   const uint32_t off_sf = (uint32_t)NST * stage_bytes, off_sc = off_sf + NST * STAGE_SF_BYTES, off_bar = off_sc + 2 * SC_FLOATS * 4;
   const uint32_t sm_stage = base, sm_sf = base + off_sf, sm_sc = base + off_sc, sm_bar = base + off_bar;
   const float* sc_ptr = reinterpret_cast<const float*>(smem + off_sc);
   uint8_t* bar_ptr = smem + off_bar;
   // barrier map (8 bytes each)
   constexpr int B_FULL = 0, B_EMPTY = MAX_STAGES, B_TFULL = 2 * MAX_STAGES, B_TEMPTY = B_TFULL + 2, B_RFULL = B_TEMPTY + 2,
-                B_REMPTY = B_RFULL + 2, B_BEMPTY = B_REMPTY + 2, NBAR = B_BEMPTY + 1;
+                B_REMPTY = B_RFULL + 2, B_BEMPTY = B_REMPTY + 2, B_PFULL = B_BEMPTY + 1, NBAR = B_PFULL + MAX_STAGES;
   auto bar = [&](int idx) { return sm_bar + 8u * (uint32_t)idx; };
   static_assert(NBAR * 8 + 16 <= SMEM_BAR_BYTES, "barrier area too small");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + NBAR * 8);
@@ -167,24 +193,29 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int lane = threadIdx.x & 31;
   const bool has_branch = p.branch_steps > 0;
   const int nbst = !has_branch ? 0 : p.branch_mx == 3 ? 2 : 1;             // stages of the branch per tile
-  // this CTA's contiguous run of tiles, row block major
-  const long long work = (long long)p.tiles_m * p.tiles_n;
-  const int w_begin = (int)((work * blockIdx.x) / gridDim.x);
-  const int w_end = (int)((work * (blockIdx.x + 1)) / gridDim.x);
+  // this CTA's (pair's) contiguous run of tiles, row block major
+  const int unit = (int)blockIdx.x / CTAS, units = (int)gridDim.x / CTAS;
+  const long long work = (long long)((p.tiles_m + CTAS - 1) / CTAS) * p.tiles_n;
+  const int w_begin = (int)((work * unit) / units);
+  const int w_end = (int)((work * (unit + 1)) / units);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NST; ++s) { mbar_init(bar(B_FULL + s), 1); mbar_init(bar(B_EMPTY + s), 1); }
+    for (int s = 0; s < NST; ++s) { mbar_init(bar(B_FULL + s), 1); mbar_init(bar(B_EMPTY + s), 1); mbar_init(bar(B_PFULL + s), 1); }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(bar(B_TFULL + b), 1); mbar_init(bar(B_TEMPTY + b), NUM_DRAIN_WARPS);
+      mbar_init(bar(B_TFULL + b), 1); mbar_init(bar(B_TEMPTY + b), CTAS * NUM_DRAIN_WARPS);
       mbar_init(bar(B_RFULL + b), 1); mbar_init(bar(B_REMPTY + b), NUM_DRAIN_WARPS);
     }
-    mbar_init(bar(B_BEMPTY), NUM_DRAIN_WARPS);
+    mbar_init(bar(B_BEMPTY), CTAS * NUM_DRAIN_WARPS);
     *abort_flag = 0;
     mbar_init_fence();
   }
-  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
+  if (warp == 1) {
+    if (PAIR) tmem_alloc_pair(smem_u32(tmem_slot), 512);
+    else tmem_alloc(smem_u32(tmem_slot), 512);
+  }
   tc_fence_before();
-  __syncthreads();
+  if (PAIR) cluster_sync();
+  else __syncthreads();
   tc_fence_after();
   grid_launch_dependents();
   // All 512 columns are this CTA's, so they start at 0: a constant, where a value read back would have to be moved into
@@ -205,13 +236,13 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     auto load_b = [&](int st, int s, int nu) {         // the weights' half of main stage s; announces the whole stage
       const uint32_t dst = sm_stage + st * stage_bytes + STAGE_A_BYTES, full = bar(B_FULL + st);
       const int sb = s >= p.b_wrap ? s - p.b_wrap : s; // the lo digits' plane runs over the same weights
-      load_weights_stage(full, stage_bytes + SF_BYTES + sfb_bytes, dst, &tmB, sb * LQ_KSTAGE, nu * W, sm_sf + st * STAGE_SF_BYTES + SF_BYTES,
+      load_weights_stage(full, stage_bytes + SF_BYTES + sfb_bytes, dst, &tmB, sb * LQ_KSTAGE, nu * W + (int)rank * BW, sm_sf + st * STAGE_SF_BYTES + SF_BYTES,
                          p.sfb + ((size_t)sb * p.tiles_n + nu) * sfb_bytes, sfb_bytes);
     };
     auto load_a = [&](int st, int s, int mb) {
       const uint32_t full = bar(B_FULL + st);
       load_acts_stage(full, sm_stage + st * stage_bytes, &tmA, s * LQ_KSTAGE, mb * LQ_BM, sm_sf + st * STAGE_SF_BYTES,
-                      p.sfa + ((size_t)mb * p.k_stages + s) * SF_BYTES);
+                      p.sfa + ((size_t)min(mb, p.tiles_m - 1) * p.k_stages + s) * SF_BYTES);
     };
     auto advance = [&]() {
       ++armed;
@@ -224,8 +255,8 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     }
     grid_dependency_wait();
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
-      const int mb = w / p.tiles_n, nu = w - mb * p.tiles_n;
-      const int m0 = mb * LQ_BM, n0 = nu * W;
+      const int mp = w / p.tiles_n, nu = w - mp * p.tiles_n, mb = mp * CTAS + (int)rank;   // (a pair's second block may not exist)
+      const int m0 = mb * LQ_BM, n0 = nu * W, mc = min(mb, p.tiles_m - 1);
       for (int s = 0; s < p.k_stages; ++s) {
         const bool ahead = tc == 0 && s < early;
         if (!ahead) {
@@ -248,10 +279,10 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (elect_one()) {
           mbar_expect_tx(full, stage_bytes + (p.branch_mx ? SF_BYTES + sfb_bytes : 0));
           tma_load_2d(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
-          tma_load_2d(a_dst + STAGE_A_BYTES, &tmL2, 0, n0, full);
+          tma_load_2d(a_dst + STAGE_A_BYTES, &tmL2, 0, n0 + (int)rank * BW, full);
           if (p.branch_mx) {   // the block scales of T (rows) and of L2 (columns) along the rank
             const uint32_t sf_dst = sm_sf + st * STAGE_SF_BYTES;
-            bulk_load(sf_dst, p.sft + ((size_t)mb * nbst + bs) * SF_BYTES, SF_BYTES, full);
+            bulk_load(sf_dst, p.sft + ((size_t)mc * nbst + bs) * SF_BYTES, SF_BYTES, full);
             bulk_load(sf_dst + SF_BYTES, p.sfl2 + (size_t)nu * sfb_bytes, sfb_bytes, full);
           }
         }
@@ -266,7 +297,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (elect_one()) {
           const uint32_t rfull = bar(B_RFULL + rb), dst = sm_sc + rb * SC_FLOATS * 4, cb = (uint32_t)min(W, p.Npad - n0) * 4;
           mbar_expect_tx(rfull, LQ_BM * 4 + 2 * cb);
-          bulk_load(dst, p.sT + m0, LQ_BM * 4, rfull);
+          bulk_load(dst, p.sT + mc * LQ_BM, LQ_BM * 4, rfull);
           bulk_load(dst + LQ_BM * 4, p.sL2 + n0, cb, rfull);
           bulk_load(dst + (LQ_BM + MAX_W) * 4, p.bias + n0, cb, rfull);
         }
@@ -285,6 +316,18 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         mbar_settle(bar(B_RFULL + (int)(j & 1)), (j >> 1) & 1);
       }
     }
+  } else if (warp == 1 && rank != 0) {
+    // ------------------------------------------------------------------ the pair's second CTA: tells the first which stages
+    // have landed here
+    const int total = (w_end - w_begin) * (p.k_stages + nbst);
+    int st = 0;
+    uint32_t par = 0;
+    for (int i = 0; i < total; ++i) {
+      if (!mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA)) break;
+      if (lane == 0) peer_arrive(peer_smem(bar(B_PFULL + st), 0));
+      __syncwarp();
+      if (++st == NST) { st = 0; par ^= 1; }
+    }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     uint32_t tc = 0, par = 0;
@@ -293,9 +336,26 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const uint32_t tsfa = tmem_base + TM_SFA, tsfb = tmem_base + TM_SFB;
     auto copy_scales = [&](int st) {
       const uint32_t sf = sm_sf + st * STAGE_SF_BYTES;
-      tc_cp_sf(tsfa, make_smem_desc_plain(sf, 16, 128));
-      tc_cp_sf(tsfb, make_smem_desc_plain(sf + SF_BYTES, 16, 128));
-      if (p.sf_chunks == 2) tc_cp_sf(tsfb + 4, make_smem_desc_plain(sf + 2 * SF_BYTES, 16, 128));
+      auto cp = [&](uint32_t to, uint32_t from) {
+        if (PAIR) tc_cp_sf_pair(to, make_smem_desc_plain(from, 16, 128));
+        else tc_cp_sf(to, make_smem_desc_plain(from, 16, 128));
+      };
+      cp(tsfa, sf);
+      cp(tsfb, sf + SF_BYTES);
+      if (p.sf_chunks == 2) cp(tsfb + 4, sf + 2 * SF_BYTES);
+    };
+    auto mma_mx = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
+      if (PAIR) tc_mma_mx_pair(d, a, b, idesc, tsfa, tsfb, 1u);
+      else tc_mma_mx(d, a, b, idesc, tsfa, tsfb, 1u);
+    };
+    auto commit = [&](uint32_t b) {
+      if (PAIR) tc_commit_pair(b);
+      else tc_commit(b);
+    };
+    constexpr uint32_t ROWS256 = PAIR ? (uint32_t)(LQ_BM >> 4) << 24 : 0;    // added to a 128-row descriptor's M field: 256
+    auto stage_full = [&]() {
+      return mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA) &&
+             (!PAIR || mbar_wait_warp(bar(B_PFULL + st), par, abort_flag, p.status, LQ_STAGE_MMA));
     };
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
       const int buf = tc & 1;
@@ -306,20 +366,21 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       tc_fence_after();
       LQ_TL(EV_M_ACC_FREE, 0);
       for (int s = 0; s < p.k_stages; ++s) {
-        ok = mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA);
+        ok = stage_full();
         if (!ok) break;
         tc_fence_after();
         LQ_TL(EV_M_STAGE_FULL, s);
         const uint32_t a_addr = sm_stage + st * stage_bytes;
         const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + STAGE_A_BYTES);
         const uint32_t sf = sm_sf + st * STAGE_SF_BYTES;
-        issue_main_stage(d, adesc, bdesc, idesc_mx(W, 0), make_smem_desc_plain(sf, 16, 128), make_smem_desc_plain(sf + SF_BYTES, 16, 128),
-                         (uint32_t)(p.sf_chunks == 2), (uint32_t)s, bar(B_EMPTY + st));
+        auto issue = PAIR ? issue_main_stage_pair : issue_main_stage_one;
+        issue(d, adesc, bdesc, idesc_mx(W, 0) + ROWS256, make_smem_desc_plain(sf, 16, 128), make_smem_desc_plain(sf + SF_BYTES, 16, 128),
+              (uint32_t)(p.sf_chunks == 2), (uint32_t)s, bar(B_EMPTY + st));
         if (++st == NST) { st = 0; par ^= 1; }
         LQ_TL(EV_M_ISSUED, s);
       }
       for (int bs = 0; bs < nbst && ok; ++bs) {
-        ok = mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA);
+        ok = stage_full();
         if (!ok) break;
         if (BRANCH_ACC) {
           // the drain has read the previous tile's branch accumulator (long ago: it does that under this tile's main loop)
@@ -336,25 +397,27 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               for (int c = 0; c < p.branch_steps; ++c)
                 for (int q = 0; q < 4; ++q) {
                   const int ja = c + 2 * (q >> 1), jb = c + 2 * (q & 1);   // K block of T's plane, of L2's plane
-                  tc_mma_mx(d, adesc + 2 * ja, bdesc + 2 * jb, idesc_mx2(W, ja, jb), tsfa, tsfb, 1u);
+                  mma_mx(d, adesc + 2 * ja, bdesc + 2 * jb, idesc_mx2(W, ja, jb) + ROWS256);
                 }
             } else {
               for (int j = 0; j < p.branch_steps; ++j)
-                tc_mma_mx(d, adesc + 2 * j, bdesc + 2 * j, idesc_mx(W, j), tsfa, tsfb, 1u);
+                mma_mx(d, adesc + 2 * j, bdesc + 2 * j, idesc_mx(W, j) + ROWS256);
             }
           } else {
             for (int j = 0; j < p.branch_steps; ++j) {
-              if (BRANCH_ACC) tc_mma<TC_I8>(tmem_base + 2 * W, adesc + 2 * j, bdesc + 2 * j, IDESC_I8 | idesc_shape(W), (uint32_t)j);
-              else tc_mma<TC_F16>(d, adesc + 2 * j, bdesc + 2 * j, IDESC_F16 | idesc_shape(W), 1u);   // 16 halves each
+              constexpr int KIND = BRANCH_ACC ? TC_I8 : TC_F16;                // (16 halves each)
+              const uint32_t to = BRANCH_ACC ? tmem_base + 2 * W : d, idesc = (BRANCH_ACC ? IDESC_I8 : IDESC_F16) + idesc_shape(W) + ROWS256;
+              if (PAIR) tc_mma_pair<KIND>(to, adesc + 2 * j, bdesc + 2 * j, idesc, BRANCH_ACC ? (uint32_t)j : 1u);
+              else tc_mma<KIND>(to, adesc + 2 * j, bdesc + 2 * j, idesc, BRANCH_ACC ? (uint32_t)j : 1u);
             }
           }
-          tc_commit(bar(B_EMPTY + st));
+          commit(bar(B_EMPTY + st));
         }
         __syncwarp();
         if (++st == NST) { st = 0; par ^= 1; }
       }
       if (!ok) break;
-      if (elect_one()) tc_commit(bar(B_TFULL + buf));
+      if (elect_one()) commit(bar(B_TFULL + buf));
       __syncwarp();
       LQ_TL(EV_TILE, 0);
     }
@@ -365,11 +428,15 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const int g = lane >> 2, t = lane & 3;              // fragment coordinates: rows g + 8 i, eight columns from 8 t
     const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16);
     const int blocks = W >> 5;
+    auto give_back = [&](uint32_t b) {                  // to the issuer, which sits in the pair's first CTA
+      if (PAIR) peer_arrive(peer_smem(b, 0));
+      else mbar_arrive(b);
+    };
     uint32_t tc = 0;
     bool ok = true;
     grid_dependency_wait();                             // Y may be what an earlier kernel still reads
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
-      const int mb = w / p.tiles_n, nu = w - mb * p.tiles_n;
+      const int mp = w / p.tiles_n, nu = w - mp * p.tiles_n, mb = mp * CTAS + (int)rank;
       const int buf = tc & 1;
       LQ_TL(EV_D_OPEN, 0);
       ok = mbar_wait_warp(bar(B_TFULL + buf), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN) &&
@@ -401,8 +468,8 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           tc_fence_before();
           __syncwarp();
           if (lane == 0) {
-            mbar_arrive(bar(B_TEMPTY + buf));
-            if (BRANCH_ACC) mbar_arrive(bar(B_BEMPTY));
+            give_back(bar(B_TEMPTY + buf));
+            if (BRANCH_ACC) give_back(bar(B_BEMPTY));
           }
           LQ_TL(EV_D_LOADED, 0);
         }
@@ -441,8 +508,8 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       if (lane == 0) {
         mbar_arrive(bar(B_REMPTY + buf));
         if (cgi >= blocks) {                            // a tile narrower than 128 columns has nothing for this warp
-          mbar_arrive(bar(B_TEMPTY + buf));
-          if (BRANCH_ACC) mbar_arrive(bar(B_BEMPTY));
+          give_back(bar(B_TEMPTY + buf));
+          if (BRANCH_ACC) give_back(bar(B_BEMPTY));
         }
       }
       LQ_TL(EV_D_EPI_END, 0);
@@ -451,35 +518,38 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
   // ---------------------------------------------------------------------- teardown
   tc_fence_before();
-  __syncthreads();
+  if (PAIR) cluster_sync();      // the peer's MMAs and arrivals reach into this CTA's shared memory until here
+  else __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 512);
+    if (PAIR) tmem_dealloc_pair(tmem_base, 512);
+    else tmem_dealloc(tmem_base, 512);
   }
 }
 
 // Ring depth that fits beside the fixed part.
-int ring_stages(int width) {
-  return std::min(MAX_STAGES, (MAX_SMEM - FIXED_SMEM) / (STAGE_A_BYTES + width * LQ_KSTAGE + STAGE_SF_BYTES));
+int ring_stages(int bw) {      // bw: columns of B per CTA
+  return std::min(MAX_STAGES, (MAX_SMEM - FIXED_SMEM) / (STAGE_A_BYTES + bw * LQ_KSTAGE + STAGE_SF_BYTES));
 }
-int smem_bytes(int width) {
-  return FIXED_SMEM + ring_stages(width) * (STAGE_A_BYTES + width * LQ_KSTAGE + STAGE_SF_BYTES);
+int smem_bytes(int bw) {
+  return FIXED_SMEM + ring_stages(bw) * (STAGE_A_BYTES + bw * LQ_KSTAGE + STAGE_SF_BYTES);
 }
 
 // Index (LQ_MX_WIDTHS) of the tile width for a launch.  Model, in clocks: a stage takes the longer of its MMAs (2 W) and its
 // operands' way from the L2 (70 bytes per clock and SM); a tile the longer of its stages and the drain of the tile before; a
 // launch the tiles of the CTA with the most, plus the last drain and the filling of the ring.
-int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas) {
+int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas, bool pair) {
   int best = -1;
   double best_cost = 1e30;
   for (int i = 0; i < LQ_MX_NWIDTHS; ++i) {
     if (!L->d_sfbw[i]) continue;
     const int w = LQ_MX_WIDTHS[i];
     if (g_lq_gemm_width > 0 && w != g_lq_gemm_width) continue;
-    const long long tiles = (long long)tiles_m * lq_ceil_div(L->N, w);
-    const double stage = std::max(2.0 * w, (STAGE_A_BYTES + w * LQ_KSTAGE) / 70.0);
+    const int c = pair ? 2 : 1, units = ctas / c;
+    const long long tiles = (long long)lq_ceil_div(tiles_m, c) * lq_ceil_div(L->N, w);
+    const double stage = std::max(2.0 * w, (STAGE_A_BYTES + w / c * LQ_KSTAGE) / 70.0);
     const double drain = 600.0 + 1200.0 * lq_ceil_div(w, 128);
-    const double cost = (double)((tiles + ctas - 1) / ctas) * std::max(stages * stage, drain) + drain + 4.0 * stage;
+    const double cost = (double)((tiles + units - 1) / units) * std::max(stages * stage, drain) + drain + 4.0 * stage;
     if (cost < best_cost) { best_cost = cost; best = i; }
   }
   return best;
@@ -489,7 +559,7 @@ int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas) {
 
 lq_status lq_gemm_mx_prepare(int device) {
   if (cudaSetDevice(device) != cudaSuccess) return LQ_ERR_CUDA;
-  for (auto* kernel : {lq_gemm_mx_kernel<false>, lq_gemm_mx_kernel<true>})
+  for (auto* kernel : {lq_gemm_mx_kernel<false, false>, lq_gemm_mx_kernel<true, false>, lq_gemm_mx_kernel<false, true>, lq_gemm_mx_kernel<true, true>})
     if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM)) != cudaSuccess) return LQ_ERR_CUDA;
   return LQ_OK;
 }
@@ -510,16 +580,23 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device) != cudaSuccess) return LQ_ERR_CUDA;
   int ctas = g_lq_gemm_ctas > 0 ? g_lq_gemm_ctas : sms;
-  const int wi = pick_width(L, p.tiles_m, p.k_stages + (L->r > 0), ctas);
+  // Pairs from 256 rows on; below, a pair's second CTA would have nothing to do.
+  const bool pair = p.tiles_m > 1 && ctas > 1 && g_lq_gemm_pair;
+  const int wi = pick_width(L, p.tiles_m, p.k_stages + (L->r > 0), ctas, pair);
   if (wi < 0) return LQ_ERR_INVALID_ARG;
-  p.width = LQ_MX_WIDTHS[wi]; p.stages = ring_stages(p.width); p.sf_chunks = lq_ceil_div(p.width, 128);
+  p.width = LQ_MX_WIDTHS[wi]; p.stages = ring_stages(pair ? p.width / 2 : p.width); p.sf_chunks = lq_ceil_div(p.width, 128);
   p.tiles_n = lq_ceil_div(L->N, p.width);
   p.sfa = A->d_sfa; p.sfb = L->d_sfbw[wi]; p.sft = A->d_sft; p.sfl2 = L->d_sfl2w[wi];
   p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
   p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
-  const long long tiles = (long long)p.tiles_m * p.tiles_n;
-  if (ctas > tiles) ctas = (int)tiles;
-  auto* kernel = p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx ? lq_gemm_mx_kernel<true> : lq_gemm_mx_kernel<false>;
-  const cudaError_t e = lq_launch(kernel, ctas, GEMM_THREADS, (size_t)smem_bytes(p.width), st, A->tmA, L->tmBw[wi], A->tmT, L->tmL2w[wi], p);
+  const int c = pair ? 2 : 1;
+  const long long tiles = (long long)lq_ceil_div(p.tiles_m, c) * p.tiles_n;
+  ctas = c * (int)std::min<long long>(ctas / c, tiles);
+  const bool acc = p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx;
+  auto* kernel = acc ? (pair ? lq_gemm_mx_kernel<true, true> : lq_gemm_mx_kernel<true, false>)
+                     : (pair ? lq_gemm_mx_kernel<false, true> : lq_gemm_mx_kernel<false, false>);
+  const CUtensorMap& tmB = pair ? L->tmBp[wi] : L->tmBw[wi];
+  const CUtensorMap& tmL2 = pair ? L->tmL2p[wi] : L->tmL2w[wi];
+  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, (size_t)smem_bytes(p.width / c), st, A->tmA, tmB, A->tmT, tmL2, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -115,6 +115,7 @@ struct lq_layer {
                                     // layout tensor memory wants (byte 16*(i%32) + 4*((i%128)/32) + block%4)
   uint8_t* d_sfl2w[LQ_MX_NWIDTHS];  // MX branches: the same for L2's block scales along the rank, [tiles][ceil(width/128)][512]
   CUtensorMap tmBw[LQ_MX_NWIDTHS], tmL2w[LQ_MX_NWIDTHS];   // over d_Wq8 and d_L2c, box [width][128B], 128B swizzle
+  CUtensorMap tmBp[LQ_MX_NWIDTHS], tmL2p[LQ_MX_NWIDTHS];   // the same with half the width, for a pair of CTAs
   CUtensorMap tmB;             // over d_Wq8, box [LQ_BN][128B], 128B swizzle
   CUtensorMap tmL1;            // over d_L1c, box [all rows][128B], 128B swizzle
   CUtensorMap tmL2;            // over d_L2c, box [LQ_BN][128B], 128B swizzle
@@ -177,6 +178,7 @@ static inline uint8_t lq_encode_code_host(int q, int kind) {
 
 extern int g_lq_main_kind;   // option "main_kind"
 extern int g_lq_gemm_ctas;   // option "gemm_ctas" (0 = one per SM)
+extern int g_lq_gemm_pair;   // option "gemm_pair": 1 = pairs of CTAs share an MX GEMM's tile where there are enough rows
 extern int g_lq_gemm_width;  // option "gemm_width": tile width of the MX GEMM, 0 = chosen by the launcher
 extern int g_lq_quant_warps, g_lq_quant_ctas;   // options "quant_warps", "quant_ctas": the quantizer's row groups per tile and stages per chunk, 0 = chosen by the launcher
 extern int g_lq_overlap;     // option "overlap": launch kernels with programmatic stream serialization
