@@ -274,6 +274,7 @@ lq_status lq_selftest_wait_timeout(int device, void* cuda_stream);
  *   "gemm_ctas"    CTAs of the GEMM kernels; 0 (default) = one per SM
  *   "gemm_width"   columns of the MX GEMM's tiles: 64, 128, 160, 192 or 224 (with an integer branch at most 160, without one
  *                  not 160; a forward that cannot have the width returns INVALID_ARG); 0 (default) = chosen by the library
+ *   "gemm_split"   1, 2, 4, 8: so many CTAs share a tile of the SINT4 GEMM where they fit; 0 (default): chosen by the launcher
  *   "gemm_pair"    1 (default): from 256 rows on, pairs of CTAs share an MX GEMM's tile; 0: never
  *   "quant_warps", "quant_ctas"   how the quantizer kernel is cut: row groups of 8 per tile (at most 8 count) and 128-value
  *                  stages of K per chunk; 0 = chosen by the library

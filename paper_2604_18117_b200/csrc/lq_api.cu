@@ -13,6 +13,7 @@ int g_lq_main_kind = LQ_KIND_E4M3;
 int g_lq_gemm_ctas = 0;
 int g_lq_gemm_width = 0;
 int g_lq_gemm_pair = 1;
+int g_lq_gemm_split = 0;
 int g_lq_store_qb = 0;
 int g_lq_quant_warps = 0;
 int g_lq_quant_ctas = 0;
@@ -86,6 +87,11 @@ extern "C" lq_status lq_set_option(const char* name, int32_t value) {
   if (!strcmp(name, "gemm_pair")) {
     if (value != 0 && value != 1) return LQ_ERR_INVALID_ARG;
     g_lq_gemm_pair = value;
+    return LQ_OK;
+  }
+  if (!strcmp(name, "gemm_split")) {
+    if (value < 0 || value > 8 || (value & (value - 1)) != 0) return LQ_ERR_INVALID_ARG;
+    g_lq_gemm_split = value;
     return LQ_OK;
   }
   if (!strcmp(name, "gemm_ctas")) {
@@ -649,7 +655,7 @@ extern "C" lq_status lq_quantize_act(const lq_layer* L, const void* X, int32_t M
   if (!act_matches(L, A)) return LQ_ERR_INVALID_ARG;
   if (M <= 0 || M > A->M_max) return LQ_ERR_INVALID_ARG;
   if (((uintptr_t)X & 15) != 0) return LQ_ERR_INVALID_ARG;
-  A->M = M;
+  A->M = A->M_call = M;
   return lq_launch_quantize(L, X, M, A, (cudaStream_t)stream);
 }
 
@@ -709,7 +715,7 @@ static lq_status forward_host(const lq_layer* L, lq_act* A, const void* Xh, int3
     CUDA_OK(cudaStreamWaitEvent(st, A->ev_x[c], 0));
     // a view of the activation record that starts at row m0 (m0 is a multiple of the row tile)
     lq_act V = *A;
-    V.M = Mc; V.M_max = Mc;
+    V.M = Mc; V.M_max = Mc; V.M_call = M;
     V.d_qx8 = A->d_qx8 + (size_t)m0 * A->Kpad * A->planes;
     V.d_qb = A->d_qb + (size_t)m0 * A->Kpad;
     V.d_sx = A->d_sx + m0;                                     // [Gpad][Mpad]: the row stride stays Mpad
@@ -727,7 +733,7 @@ static lq_status forward_host(const lq_layer* L, lq_act* A, const void* Xh, int3
     CUDA_OK(cudaStreamWaitEvent(A->s_d2h, A->ev_y[c], 0));
     CUDA_OK(cudaMemcpyAsync((uint8_t*)Yh + (size_t)m0 * A->N * esz, yd, (size_t)Mc * A->N * esz, cudaMemcpyDeviceToHost, A->s_d2h));
   }
-  A->M = M;
+  A->M = A->M_call = M;
   CUDA_OK(cudaEventRecord(A->ev_end, A->s_d2h));
   CUDA_OK(cudaStreamWaitEvent(st, A->ev_end, 0));              // the caller's stream is done when Y has arrived
   if (wait) CUDA_OK(cudaStreamSynchronize(st));

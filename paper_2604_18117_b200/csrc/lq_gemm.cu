@@ -37,6 +37,9 @@
 // raises a CTA-wide abort flag and all roles leave through the common teardown.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "lq_device.cuh"
 
 #ifdef LQ_TIMELINE
@@ -80,6 +83,7 @@ struct GemmParams {
   int n_stages_main;      // Kpad / 128 (an odd last group's partner has zero codes and scales)
   int branch_mmas;        // MMAs of the branch stage (32 bytes of r each)
   int tiles_m, units_n;
+  int split;              // CTAs (of a cluster) that share a tile's stages
   const float* sx;        // [Gpad][Mpad]
   const float* sw;        // [Gpad][Npad]
   const float* sT;        // [Mpad]
@@ -138,7 +142,9 @@ __device__ __forceinline__ void fetch_group(uint32_t taddr, Frag (&v)[4]) {
 
 enum { BRANCH_NONE = 0, BRANCH_I8 = 1, BRANCH_F16 = 2 };
 
-template <int BRANCH>
+// SPLIT: the CTAs of a cluster share one tile, each with a part of the stages (K and the branch); their partial sums meet in
+// distributed shared memory.
+template <int BRANCH, bool SPLIT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
@@ -164,10 +170,14 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // provably warp-uniform
   const int lane = threadIdx.x & 31;
   const int stages_per_tile = p.n_stages_main + (BRANCH != BRANCH_NONE ? 1 : 0);
-  // this CTA's contiguous run of 128 x 128 tiles, row block major
+  // this CTA's contiguous run of 128 x 128 tiles, row block major (SPLIT: its cluster's only one)
   const long long units = (long long)p.tiles_m * p.units_n;
-  const int u_begin = (int)((units * blockIdx.x) / gridDim.x);
-  const int u_end = (int)((units * (blockIdx.x + 1)) / gridDim.x);
+  const int u_begin = SPLIT ? (int)blockIdx.x / p.split : (int)((units * blockIdx.x) / gridDim.x);
+  const int u_end = SPLIT ? u_begin + 1 : (int)((units * (blockIdx.x + 1)) / gridDim.x);
+  // and of a tile's stages
+  const int part = SPLIT ? (int)blockIdx.x % p.split : 0;
+  const int s_begin = SPLIT ? stages_per_tile * part / p.split : 0;
+  const int s_end = SPLIT ? stages_per_tile * (part + 1) / p.split : stages_per_tile;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSTAGE; ++s) {
@@ -182,9 +192,13 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
   tc_fence_before();
   __syncthreads();
-  grid_dependency_sync();        // set-up done; from here on global memory written by earlier kernels is read
+  grid_launch_dependents();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+
+  // SPLIT: where a drain thread's partial sums lie for the other CTAs, items of four neighbouring columns
+  auto partial_at = [&](int item, int thread) { return sm_stage + (uint32_t)(item * NUM_DRAIN_WARPS * 32 + thread) * 16; };
+  bool drained = false;
 
   LQ_TL_DECL((blockIdx.x == 0 && lane == 0)
                  ? (warp == 0 ? (int)TL_PRODUCER : warp == 1 ? (int)TL_MMA : warp == FIRST_DRAIN_WARP ? (int)TL_DRAIN_FIRST
@@ -197,47 +211,63 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // ------------------------------------------------------------------ TMA producer
       uint32_t it = 0, armed = 0;
       bool ok = true;
+      // The weights' half of a stage (with the announcement of all of it) and the activations' half.
+      auto load_weights = [&](uint32_t i, int s, int n0) {
+        const int st = i & (NSTAGE - 1);
+        const uint32_t b_dst = sm_stage + st * STAGE_BYTES + STAGE_A_BYTES, sc_dst = sm_sc + (i & (SC_RING - 1)) * SC_STAGE_BYTES;
+        const uint32_t full = bar_full(st);
+        const bool is_main = s < p.n_stages_main;
+        if (elect_one()) {
+          mbar_expect_tx(full, STAGE_BYTES + (is_main ? 2 : 1) * SC_GROUP_FLOATS * 4 + (s == s_begin ? UNIT * 4 : 0));
+          if (s == s_begin) bulk_load(sc_dst + 2 * SC_GROUP_FLOATS * 4, p.bias + n0, UNIT * 4, full);
+          if (is_main) {
+            tma_load_2d(b_dst, &tmB, s * LQ_KSTAGE, n0, full);
+            for (int q = 0; q < 2; ++q)
+              bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4 + LQ_BM * 4, p.sw + (size_t)(2 * s + q) * p.Npad + n0, UNIT * 4, full);
+          } else {
+            tma_load_2d(b_dst, &tmL2, 0, n0, full);
+            bulk_load(sc_dst + LQ_BM * 4, p.sL2 + n0, UNIT * 4, full);
+          }
+        }
+        __syncwarp();
+      };
+      auto load_acts = [&](uint32_t i, int s, int m0) {
+        const int st = i & (NSTAGE - 1);
+        const uint32_t a_dst = sm_stage + st * STAGE_BYTES, sc_dst = sm_sc + (i & (SC_RING - 1)) * SC_STAGE_BYTES, full = bar_full(st);
+        if (elect_one()) {
+          if (s < p.n_stages_main) {
+            tma_load_2d(a_dst, &tmA, s * LQ_KSTAGE, m0, full);
+            for (int q = 0; q < 2; ++q)
+              bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4, p.sx + (size_t)(2 * s + q) * p.Mpad + m0, LQ_BM * 4, full);
+          } else {
+            tma_load_2d(a_dst, &tmT, 0, m0, full);
+            bulk_load(sc_dst, p.sT + m0, LQ_BM * 4, full);
+          }
+        }
+        __syncwarp();
+      };
+      // Weights do not depend on earlier kernels: the first ring's worth is requested before they are waited for.
+      const uint32_t early = u_begin < u_end ? (uint32_t)min(NSTAGE, s_end - s_begin) : 0;
+      for (uint32_t i = 0; i < early; ++i) load_weights(i, s_begin + (int)i, (u_begin % p.units_n) * UNIT);
+      grid_dependency_wait();
       for (int u = u_begin; u < u_end && ok; ++u) {
         const int mb = u / p.units_n, nu = u - mb * p.units_n;
-        const int m0 = mb * LQ_BM, n0 = nu * UNIT;
-        for (int s = 0; s < stages_per_tile && ok; ++s, ++it) {
-          const int st = it & (NSTAGE - 1);
-          const uint32_t par = ((it / NSTAGE) & 1) ^ 1;
-          ok = mbar_wait_warp(bar_empty(st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
-          if (!ok) break;
-          // (Nothing says that the drain is done with the slot's old scale vectors, eight stages back, and nothing has to: the
-          // MMAs that have just retired, four stages back, had to wait for the accumulators of six stages back to be in the
-          // drain's registers, and by then it had used up the scales of the stages before.)
-          LQ_TL(EV_P_SLOT_FREE, s);
-          const uint32_t a_dst = sm_stage + st * STAGE_BYTES, b_dst = a_dst + STAGE_A_BYTES;
-          const uint32_t sc_dst = sm_sc + (it & (SC_RING - 1)) * SC_STAGE_BYTES;
-          const uint32_t full = bar_full(st);
-          const bool is_main = s < p.n_stages_main;
-          const int ngroups = is_main ? 2 : 1;
-          const uint32_t tx = STAGE_BYTES + ngroups * SC_GROUP_FLOATS * 4 + (s == 0 ? UNIT * 4 : 0);
-          if (elect_one()) {
-            mbar_expect_tx(full, tx);
-            if (s == 0) bulk_load(sc_dst + 2 * SC_GROUP_FLOATS * 4, p.bias + n0, UNIT * 4, full);
-            if (is_main) {
-              tma_load_2d(a_dst, &tmA, s * LQ_KSTAGE, m0, full);
-              tma_load_2d(b_dst, &tmB, s * LQ_KSTAGE, n0, full);
-              for (int q = 0; q < ngroups; ++q) {
-                const size_t g = (size_t)(2 * s + q);
-                bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4, p.sx + g * p.Mpad + m0, LQ_BM * 4, full);
-                bulk_load(sc_dst + q * SC_GROUP_FLOATS * 4 + LQ_BM * 4, p.sw + g * p.Npad + n0, UNIT * 4, full);
-              }
-            } else {
-              tma_load_2d(a_dst, &tmT, 0, m0, full);
-              tma_load_2d(b_dst, &tmL2, 0, n0, full);
-              bulk_load(sc_dst, p.sT + m0, LQ_BM * 4, full);
-              bulk_load(sc_dst + LQ_BM * 4, p.sL2 + n0, UNIT * 4, full);
-            }
+        for (int s = s_begin; s < s_end && ok; ++s, ++it) {
+          if (it >= early) {
+            ok = mbar_wait_warp(bar_empty(it & (NSTAGE - 1)), ((it / NSTAGE) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_PRODUCER);
+            if (!ok) break;
+            // (Nothing says that the drain is done with the slot's old scale vectors, eight stages back, and nothing has to: the
+            // MMAs that have just retired, four stages back, had to wait for the accumulators of six stages back to be in the
+            // drain's registers, and by then it had used up the scales of the stages before.)
+            LQ_TL(EV_P_SLOT_FREE, s);
+            load_weights(it, s, nu * UNIT);
           }
-          __syncwarp();
+          load_acts(it, s, mb * LQ_BM);
           ++armed;
           LQ_TL(EV_P_ISSUED, s);
         }
       }
+      armed = armed > early ? armed : early;
       if (!ok && lane == 0) {
         // aborting: give the copies already issued a bounded time to land before the CTA's shared memory goes away
         const uint32_t n = armed < (uint32_t)NSTAGE ? armed : (uint32_t)NSTAGE;
@@ -252,7 +282,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       bool ok = true;
       const uint32_t shape = idesc_shape(UNIT);
       for (int u = u_begin; u < u_end && ok; ++u) {
-        for (int s = 0; s < stages_per_tile && ok; ++s, ++it) {
+        for (int s = s_begin; s < s_end && ok; ++s, ++it) {
           const int st = it & (NSTAGE - 1);
           ok = mbar_wait_warp(bar_full(st), (it / NSTAGE) & 1, abort_flag, p.status, LQ_STAGE_MMA);
           if (!ok) break;
@@ -324,6 +354,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     auto scales_at = [&](uint32_t i, int q) {
       return load_scales(sc_ptr + (i & (SC_RING - 1)) * (SC_STAGE_BYTES / 4) + q * SC_GROUP_FLOATS, row_at, col_at);
     };
+    grid_dependency_wait();                             // Y may be what an earlier kernel still reads
     open_stage(0, u_begin < u_end);
     for (int u = u_begin; u < u_end && ok; ++u) {
       const int mb = u / p.units_n, nu = u - mb * p.units_n;
@@ -341,11 +372,16 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             acc[0][4 * k + i] = acc[1][4 * k + i] = make_float2(v.x, v.y);
             acc[0][4 * k + 2 + i] = acc[1][4 * k + 2 + i] = make_float2(v.z, v.w);
           }
+          if (SPLIT && part != 0) {
+#pragma unroll
+            for (int j = 4 * k; j < 4 * k + 4; ++j) acc[0][j] = acc[1][j] = make_float2(0.f, 0.f);
+          }
         }
       }
       const bool last_tile = u + 1 == u_end;
-      for (int s = 0; s < p.n_stages_main && ok; ++s, ++it) {
-        const bool more = s + 1 < stages_per_tile || !last_tile;
+      const int s_main = SPLIT ? min(s_end, p.n_stages_main) : p.n_stages_main;
+      for (int s = s_begin; s < s_main && ok; ++s, ++it) {
+        const bool more = s + 1 < s_end || !last_tile;
         LQ_TL(EV_D_OPEN, s);
         Scales sc = scales_at(it, 0);
         landed(it, 0);
@@ -363,7 +399,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         ok = __all_sync(0xffffffffu, ok);
       }
       if (!ok) break;
-      if constexpr (BRANCH != BRANCH_NONE) {
+      if (BRANCH != BRANCH_NONE && (!SPLIT || s_end > p.n_stages_main)) {
         const Scales sc = scales_at(it, 0);
         landed(it, 0);
         if (lane == 0) mbar_arrive(bar_tempty(2 * (it & (NPAIR - 1)) + 1));   // not used by this stage
@@ -374,35 +410,84 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!ok) break;
       LQ_TL(EV_D_EPI_BEGIN, 0);
-      // epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad
-      const int c = n0 + coff + 16 * ft;
+      if constexpr (SPLIT) {
+        // the partial sums to shared memory (the operands' place: every MMA has retired), items of four neighbouring columns
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const int r = m0 + 32 * quad + 16 * h + 8 * i + fg;
-          if (r >= p.M) continue;
-          if (p.out_f32) {
-            float* Y = reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c;
+          for (int i = 0; i < 2; ++i)
+            if (m0 + 32 * quad + 16 * h + 8 * i + fg < p.M) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              if (c + 8 * (k >> 1) < p.N)
-                *reinterpret_cast<float4*>(Y + 4 * k) = make_float4(acc[h][4 * k + i].x, acc[h][4 * k + i].y, acc[h][4 * k + 2 + i].x, acc[h][4 * k + 2 + i].y);
-          } else {
-            __half* Y = reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c;
-            uint32_t w[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const __half2 q = __floats2half2_rn(acc[h][2 * j + i].x, acc[h][2 * j + i].y);
-              w[j] = *reinterpret_cast<const uint32_t*>(&q);
+              for (int k = 0; k < 4; ++k)
+                sts_v4(partial_at(4 * (2 * h + i) + k, (int)threadIdx.x - 32 * FIRST_DRAIN_WARP),
+                       make_uint4(__float_as_uint(acc[h][4 * k + i].x), __float_as_uint(acc[h][4 * k + i].y),
+                                  __float_as_uint(acc[h][4 * k + 2 + i].x), __float_as_uint(acc[h][4 * k + 2 + i].y)));
             }
-            if (c < p.N) *reinterpret_cast<uint4*>(Y) = make_uint4(w[0], w[1], w[2], w[3]);
-            if (c + 8 < p.N) *reinterpret_cast<uint4*>(Y + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+      } else {
+        // epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad
+        const int c = n0 + coff + 16 * ft;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int r = m0 + 32 * quad + 16 * h + 8 * i + fg;
+            if (r >= p.M) continue;
+            if (p.out_f32) {
+              float* Y = reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c;
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                if (c + 8 * (k >> 1) < p.N)
+                  *reinterpret_cast<float4*>(Y + 4 * k) = make_float4(acc[h][4 * k + i].x, acc[h][4 * k + i].y, acc[h][4 * k + 2 + i].x, acc[h][4 * k + 2 + i].y);
+            } else {
+              __half* Y = reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c;
+              uint32_t w[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const __half2 q = __floats2half2_rn(acc[h][2 * j + i].x, acc[h][2 * j + i].y);
+                w[j] = *reinterpret_cast<const uint32_t*>(&q);
+              }
+              if (c < p.N) *reinterpret_cast<uint4*>(Y) = make_uint4(w[0], w[1], w[2], w[3]);
+              if (c + 8 < p.N) *reinterpret_cast<uint4*>(Y + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+            }
           }
-        }
+      }
       LQ_TL(EV_D_EPI_END, 0);
     }
     tmem_ld_wait();                                     // the last request
+    drained = ok;
+  }
+  if constexpr (SPLIT) {
+    // Every CTA of the cluster adds up a part of the items, in the order of the stages, and stores them.
+    __syncwarp();
+    cluster_sync();
+    if (drained) {
+      const int at = (int)threadIdx.x - 32 * FIRST_DRAIN_WARP, mb = u_begin / p.units_n, nu = u_begin - mb * p.units_n, n = 16 / p.split;
+      const int row = mb * LQ_BM + 32 * (warp & 3) + (lane >> 2), col = nu * UNIT + ((warp - FIRST_DRAIN_WARP) >> 2) * WCOLS + 16 * (lane & 3);
+      for (int j = part * n; j < (part + 1) * n; j += 2) {       // two items: eight columns
+        const int r = row + 8 * (j >> 2), c = col + 4 * (j & 3);
+        if (r >= p.M || c >= p.N) continue;
+        float y[8] = {};
+#pragma unroll 4
+        for (int k = 0; k < p.split; ++k) {
+          const float4 a = lds_peer_v4(peer_smem(partial_at(j, at), k)), b = lds_peer_v4(peer_smem(partial_at(j + 1, at), k));
+          y[0] += a.x; y[1] += a.y; y[2] += a.z; y[3] += a.w; y[4] += b.x; y[5] += b.y; y[6] += b.z; y[7] += b.w;
+        }
+        if (p.out_f32) {
+          float4* Y = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c);
+          Y[0] = make_float4(y[0], y[1], y[2], y[3]);
+          Y[1] = make_float4(y[4], y[5], y[6], y[7]);
+        } else {
+          uint32_t w[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const __half2 q = __floats2half2_rn(y[2 * i], y[2 * i + 1]);
+            w[i] = *reinterpret_cast<const uint32_t*>(&q);
+          }
+          *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+    }
+    cluster_sync();                                     // nobody's shared memory goes away while another CTA reads it
   }
 
   // ---------------------------------------------------------------------- teardown
@@ -428,6 +513,24 @@ __global__ void lq_wait_probe_kernel(int32_t* status, long long limit) {
   mbar_wait_slow(bar, 0, &abort_word, status, LQ_STAGE_TEARDOWN, limit);
 }
 
+// CTAs per tile of a launch of few tiles (1, 2, 4 or 8).  A tile's stages are one serial chain, 0.52 us each, so while SMs are idle
+// they may as well share it; a cluster's launch and its two rendezvous cost 1.9 us, the exchange up to 0.15 us per CTA that is
+// read (M = 1, K x N = 1152 x 1152: 7.9 us alone, 5.4 by eight; M = 128, 8192 x 1152: 38 and 11.7; M = 256, 4608 x 1152: 23.2
+// and 11.4 by four).  The hardware places a cluster's CTAs next to each other, so fewer fit than there are SMs; a second
+// round of them would cost more than it gives.
+int g_clusters[64][3];                                // how many clusters of 2, 4, 8 the device holds at once
+int pick_split(int device, int M, long long units, int stages, int ctas) {
+  int best = 1;
+  double best_cost = 0.52 * stages;
+  for (int i = 0, split = 2; i < 3; ++i, split *= 2) {
+    if (split > ctas || split > stages || units > std::min(g_clusters[device & 63][i], ctas / split)) break;
+    if (g_lq_gemm_split > 0 && split != g_lq_gemm_split) continue;
+    const double cost = g_lq_gemm_split > 0 ? 0 : 0.52 * lq_ceil_div(stages, split) + 1.9 + 0.15 * split * std::min(M, LQ_BM) / LQ_BM;
+    if (cost < best_cost) { best_cost = cost; best = split; }
+  }
+  return best;
+}
+
 }  // namespace
 
 lq_status lq_launch_wait_probe(int device, cudaStream_t st) {
@@ -440,8 +543,18 @@ lq_status lq_launch_wait_probe(int device, cudaStream_t st) {
 
 lq_status lq_gemm_prepare(int device) {
   if (cudaSetDevice(device) != cudaSuccess) return LQ_ERR_CUDA;
-  for (auto* kernel : {lq_gemm_kernel<BRANCH_NONE>, lq_gemm_kernel<BRANCH_I8>, lq_gemm_kernel<BRANCH_F16>})
+  for (auto* kernel : {lq_gemm_kernel<BRANCH_NONE, false>, lq_gemm_kernel<BRANCH_I8, false>, lq_gemm_kernel<BRANCH_F16, false>,
+                       lq_gemm_kernel<BRANCH_NONE, true>, lq_gemm_kernel<BRANCH_I8, true>, lq_gemm_kernel<BRANCH_F16, true>})
     if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return LQ_ERR_CUDA;
+  for (int i = 0; i < 3; ++i) {
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2u << i; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    lc.gridDim = dim3(2u << i); lc.blockDim = dim3(GEMM_THREADS); lc.dynamicSmemBytes = SMEM_BYTES; lc.attrs = at; lc.numAttrs = 1;
+    if (lq_note_cuda(cudaOccupancyMaxActiveClusters(&g_clusters[device & 63][i], lq_gemm_kernel<BRANCH_I8, true>, &lc)) != cudaSuccess)
+      return LQ_ERR_CUDA;
+  }
   return LQ_OK;
 }
 
@@ -462,8 +575,14 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device) != cudaSuccess) return LQ_ERR_CUDA;
   int ctas = g_lq_gemm_ctas > 0 ? g_lq_gemm_ctas : sms;
   const long long units = (long long)p.tiles_m * p.units_n;
-  if (ctas > units) ctas = (int)units;
-  auto* kernel = L->r == 0 ? lq_gemm_kernel<BRANCH_NONE> : L->f16_branch ? lq_gemm_kernel<BRANCH_F16> : lq_gemm_kernel<BRANCH_I8>;
-  const cudaError_t e = lq_launch(kernel, ctas, GEMM_THREADS, SMEM_BYTES, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
+  // (by the whole call's rows, so that a row's sums are the same in every chunk of it)
+  p.split = pick_split(A->device, A->M_call, (long long)lq_ceil_div(A->M_call, LQ_BM) * p.units_n, p.n_stages_main + (L->r > 0), ctas);
+  ctas = (int)std::min<long long>(ctas, units * p.split);
+  auto kernel = [&](auto split) {
+    constexpr bool S = decltype(split)::value;
+    return L->r == 0 ? lq_gemm_kernel<BRANCH_NONE, S> : L->f16_branch ? lq_gemm_kernel<BRANCH_F16, S> : lq_gemm_kernel<BRANCH_I8, S>;
+  };
+  const cudaError_t e = lq_launch_cluster(p.split > 1 ? kernel(std::true_type()) : kernel(std::false_type()), ctas, GEMM_THREADS, p.split,
+                                          SMEM_BYTES, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -131,6 +131,7 @@ struct lq_act {
   uint8_t* d_sfa;              // MX: E8M0 bytes of the activation scales, [Mpad/128][Kpad/128][512], same layout
   int M_max, Mpad, device, main_kind;
   int M;                       // rows of the last lq_quantize_act
+  int M_call;                  // rows of the caller's call (more than M in a chunk of one): what the order of a sum may depend on
   uint8_t* d_qx8;              // [Mpad][Kpad] operand bytes of the 4-bit codes (A operand, K-major)
   float* d_sx;                 // [Gpad][Mpad] fp32 images of the fp16 scales, in lq_row_slot order
   int8_t* d_qb;                // [Mpad][Kpad] branch activation codes
@@ -179,6 +180,7 @@ static inline uint8_t lq_encode_code_host(int q, int kind) {
 extern int g_lq_main_kind;   // option "main_kind"
 extern int g_lq_gemm_ctas;   // option "gemm_ctas" (0 = one per SM)
 extern int g_lq_gemm_pair;   // option "gemm_pair": 1 = pairs of CTAs share an MX GEMM's tile where there are enough rows
+extern int g_lq_gemm_split;  // option "gemm_split": CTAs that share a tile of the SINT4 GEMM where there is room for them, 0 = chosen by the launcher
 extern int g_lq_gemm_width;  // option "gemm_width": tile width of the MX GEMM, 0 = chosen by the launcher
 extern int g_lq_quant_warps, g_lq_quant_ctas;   // options "quant_warps", "quant_ctas": the quantizer's row groups per tile and stages per chunk, 0 = chosen by the launcher
 extern int g_lq_overlap;     // option "overlap": launch kernels with programmatic stream serialization

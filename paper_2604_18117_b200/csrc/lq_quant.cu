@@ -67,7 +67,6 @@ enum { MAIN_SINT4 = 0, MAIN_MXINT4 = 1, MAIN_MXFP = 2, MAIN_MXINT8 = 3, MAIN_MXF
 
 struct QuantParams {
   int M, K, Kpad, Mpad;
-  int G;                // SINT4: groups of 64 that hold data
   int nst;              // Kpad / 128 stages of K
   int groups, stages;   // RG row groups of 8 per tile, SX stages of K per chunk
   int teams;            // teams of RG * SX quantizer warps: they take the chunks in turn
@@ -805,8 +804,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
                 if constexpr (SINT) {
                   const Sint4Scale sc(bm);
                   wa[h] = sint4_codes8(a[h], sc.inv[0], sc.coarse); wb[h] = sint4_codes8(b[h], sc.inv[1], sc.coarse);
-                  const int g = 2 * st + h;
-                  if (vs && g < p.G) p.sx[(size_t)g * p.Mpad + lq_row_slot(ms)] = lc ? sc.s[1] : sc.s[0];
+                  if (vs) p.sx[(size_t)(2 * st + h) * p.Mpad + lq_row_slot(ms)] = lc ? sc.s[1] : sc.s[0];   // (of a padding group, too)
                 } else {
                   constexpr int TOP = MAIN == MAIN_MXINT4 ? 2 : MAIN == MAIN_MXINT8 ? 6 : 8;
                   constexpr int UP = MAIN == MAIN_MXINT4 ? 0xFF : MAIN == MAIN_MXINT8 ? 0x0F : 0;
@@ -1031,7 +1029,7 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   if (A->main_kind != LQ_KIND_E4M3) return LQ_ERR_UNSUPPORTED;
   const int abits = lq_branch_abits(L->cfg.branch);
   QuantParams p;
-  p.M = M; p.K = L->K; p.Kpad = L->Kpad; p.Mpad = A->Mpad; p.G = L->G;
+  p.M = M; p.K = L->K; p.Kpad = L->Kpad; p.Mpad = A->Mpad;
   p.nst = L->Kpad / LQ_KSTAGE;
   p.qx8 = A->d_qx8; p.sx = A->d_sx; p.sfa = A->d_sfa;
   p.qb = g_lq_store_qb ? A->d_qb : nullptr;

@@ -1,0 +1,94 @@
+"""GPU parity of the kernels' cuts at the edges of their tiles: CTAs that share a tile of the SINT4 GEMM, the MX GEMM's tile
+widths alone and in pairs of CTAs, and the quantizer's row tiles and K chunks."""
+import numpy as np
+import pytest
+
+from paper_2604_18117_b200 import binding as B
+from tests import test_gpu_mxfp as MXFP
+from tests import test_gpu_mxint4 as MXINT4
+from tests import test_gpu_mxint8 as MXINT8
+from tests import test_gpu_parity as SINT4
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def option():
+    used = []
+
+    def set_option(name, value, default=0):
+        used.append((name, default))
+        B.lq_set_option(name, value)
+
+    yield set_option
+    for name, default in used:
+        B.lq_set_option(name, default)
+
+
+def _x(rng, M, K):
+    X = rng.standard_normal((M, K)).astype(np.float16)
+    X[:, rng.choice(K, max(1, K // 50), replace=False)] *= 20
+    return X
+
+
+@pytest.mark.parametrize("split", [0, 1, 2, 4, 8])
+@pytest.mark.parametrize("M,K,N,r,branch", [(1, 1152, 136, 32, "w8a8"), (129, 1088, 72, 0, "none"), (127, 8192, 8, 24, "w16a16"),
+                                            (128, 512, 200, 16, "w4a8")])
+def test_sint4_tiles_shared_by_a_cluster(option, split, M, K, N, r, branch):
+    """One row, one short of and beyond a tile of rows, columns of less than a vector's neighbours, an odd number of groups, fewer
+    stages than CTAs, a part that is the branch alone."""
+    option("gemm_split", split)
+    rng = np.random.default_rng(split + M)
+    SINT4._check(SINT4._random_layer(rng, K, N, r, branch), _x(rng, M, K),
+                 tol32=SINT4.TOL_F32 * (5 if branch == "w16a16" else 1))
+
+
+@pytest.mark.parametrize("pair", [0, 1])
+@pytest.mark.parametrize("width", [64, 128, 160, 192, 224])
+@pytest.mark.parametrize("main,branch,r", [("mxint4", "none", 0), ("mxint4", "w8a8", 32), ("mxint4", "w16a16", 24), ("mxfp4", "mxfp8", 64),
+                                           ("mxint8", "mxint8", 64), ("mxint8", "mxint4", 128)])
+def test_mx_tile_widths_alone_and_in_pairs(option, main, branch, r, width, pair):
+    """Three row blocks (a pair's second one is missing), the last of them one row; a last tile of eight columns; K beyond the ring."""
+    if (width == 160) != (branch == "w8a8") and width >= 160:
+        pytest.skip("layers with an integer branch have the widths up to 160, the others all but 160")
+    option("gemm_width", width)
+    option("gemm_pair", pair, default=1)
+    rng = np.random.default_rng(width + pair)
+    M, K, N = 257, 1184, 2 * width + 8
+    mod = {"mxint4": MXINT4, "mxfp4": MXFP, "mxint8": MXINT8}[main]
+    layer = mod._mx_layer(rng, K, N, r, branch) if main == "mxint4" else mod._layer(rng, K, N, r, branch)
+    mod._check(layer, _x(rng, M, K))
+
+
+@pytest.mark.parametrize("groups,stages", [(1, 1), (8, 1), (3, 4), (5, 3), (0, 0)])
+@pytest.mark.parametrize("M,K", [(1, 32), (63, 1160), (200, 8192)])
+def test_quantizer_cuts(option, groups, stages, M, K):
+    """Row tiles of 8 to 64 rows and chunks of one to four stages, on one row, one short of a tile and several tiles; less than a
+    stage, a ragged last stage, and the longest K (an integer branch streams the tile twice)."""
+    if stages > -(-K // 128):
+        pytest.skip("a chunk is at most all of K")
+    option("quant_warps", groups)
+    option("quant_ctas", stages)
+    rng = np.random.default_rng(M)
+    X = _x(rng, M, K)
+    SINT4._check(SINT4._random_layer(rng, K, 40, 32, "w8a8"), X)
+    MXFP._check(MXFP._layer(rng, K, 40, 33, "mxfp8"), X)
+    MXINT8._check(MXINT8._layer(rng, K, 40, 40, "mxint8"), X)
+
+
+def test_static_calls_of_different_layers_share_the_scratch():
+    """What an earlier call of another layer left in the padding of the shared record is not read."""
+    from oracle import lq_oracle as O
+    from tests.helpers import import_oracle_layer, rel_fro
+    import torch
+
+    rng = np.random.default_rng(5)
+    for M, K, N, r, branch in ((256, 2048, 264, 64, "w16a16"), (130, 72, 40, 8, "w8a8"), (3, 328, 136, 24, "w16a16"), (3, 328, 8, 0, "none")):
+        layer, X = SINT4._random_layer(rng, K, N, r, branch), _x(rng, M, K)
+        h, _ = import_oracle_layer(layer)
+        B.lq_layer_to_device(h, 0)
+        x, y = torch.from_numpy(X).cuda(), torch.empty(M, N, device="cuda")
+        B.lq_linear_forward_static(h, x.data_ptr(), M, y.data_ptr(), B.OUT_F32, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        B.lq_layer_free(h)
+        assert rel_fro(y.cpu().numpy(), O.forward(X, layer)["Y"]) <= SINT4.TOL_F32 * (10 if branch == "w16a16" else 1)
