@@ -440,24 +440,34 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
     std::vector<int> wrow(Npad), srow(Npad);                     // places of column n in the weight operand and the vectors
     for (int n = 0; n < Npad; ++n) { wrow[n] = L->mx ? lq_col32_slot(n) : lq_col_slot(n); srow[n] = L->mx ? n : lq_colscale_slot(n); }
     std::vector<uint8_t> w8((size_t)Npad * Kpad, lq_encode_code_host(0, L->main_kind));
-    for (int k = 0; k < K; ++k)
-      for (int n = 0; n < N; ++n)
-        w8[(size_t)wrow[n] * Kpad + k] = L->mxfp ? L->Wq8h[(size_t)k * N + n] : lq_encode_code_host(L->Wq[(size_t)k * N + n], L->main_kind);
+    uint8_t code_byte[16] = {};                                       // operand byte of each 4-bit code
+    for (int q = -7; q <= 7; ++q) code_byte[q & 15] = lq_encode_code_host(q, L->main_kind);
+    // transposed in blocks that stay in the cache (K x N = 1152 x 4608: the whole upload 9.9 ms row by row, 5.2 so)
+    for (int k0 = 0; k0 < K; k0 += 64)
+      for (int n0 = 0; n0 < N; n0 += 64)
+        for (int n = n0; n < std::min(n0 + 64, N); ++n) {
+          uint8_t* row = &w8[(size_t)wrow[n] * Kpad];
+          for (int k = k0; k < std::min(k0 + 64, K); ++k)
+            row[k] = L->mxfp ? L->Wq8h[(size_t)k * N + n] : code_byte[L->Wq[(size_t)k * N + n] & 15];
+        }
     if ((st = upload(&L->d_Wq8, w8)) != LQ_OK) return st;
     if (L->mx) {
       // E8M0 bytes (exponent + 127) in the layout the block-scaled MMA reads from tensor memory, by tile width; 127 = 2^0 for padding
-      std::vector<uint8_t> e8((size_t)G * N);
-      for (size_t i = 0; i < e8.size(); ++i) {
-        int x = 0;
-        frexpf(h2f(L->sw[i]), &x);                                // 2^e = 0.5 * 2^(e+1)
-        e8[i] = (uint8_t)(x - 1 + 127);
-      }
+      std::vector<uint32_t> e8((size_t)(Kpad / 128) * N, 0x7F7F7F7Fu);   // a stage's four bytes of a column
+      for (int g = 0; g < G; ++g)
+        for (int n = 0; n < N; ++n) {
+          int x = 0;
+          frexpf(h2f(L->sw[(size_t)g * N + n]), &x);              // 2^e = 0.5 * 2^(e+1)
+          reinterpret_cast<uint8_t*>(&e8[(size_t)(g / 4) * N + n])[g % 4] = (uint8_t)(x - 1 + 127);
+        }
       for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
         const int width = LQ_MX_WIDTHS[wi], tiles = lq_ceil_div(N, width);
         if (!lq_mx_width_used(width, L->integer_branch)) continue;
         std::vector<uint8_t> sfb((size_t)(Kpad / 128) * tiles * lq_ceil_div(width, 128) * 512, 127);
-        for (int g = 0; g < G; ++g)
-          for (int n = 0; n < N; ++n) sfb[lq_sfb_offset(wrow[n], g, width, tiles)] = e8[(size_t)g * N + n];
+        for (int n = 0; n < N; ++n) {
+          const size_t at = lq_sfb_offset(wrow[n], 0, width, tiles), step = (size_t)tiles * lq_ceil_div(width, 128) * 512;
+          for (int s = 0; s < Kpad / 128; ++s) memcpy(&sfb[at + s * step], &e8[(size_t)s * N + n], 4);
+        }
         if ((st = upload(&L->d_sfbw[wi], sfb)) != LQ_OK) return st;
       }
     } else {
