@@ -435,6 +435,56 @@ __device__ __noinline__ void settle_block(const QuantParams& p, int4 what, float
   if ((which >> lane) & 1) p.tq[(size_t)m * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, mine * inv);
 }
 
+// A stage's MMAs under one election, predicated instead of branched around (inside an `if` of one lane every operand is moved to
+// uniform registers one by one, 300 clocks a stage: with a few rows that was what a long K waited for).
+template <int KIND>
+__device__ __forceinline__ void issue_four(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  if constexpr (KIND == TC_I8) {
+    asm volatile(
+        "{\n\t.reg .pred P, T, A;\n\t"
+        "elect.sync _|P, 0xffffffff;\n\t"
+        "setp.ne.b32 A, %10, 0;\n\t"
+        "setp.eq.b32 T, 0, 0;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %5, %9, A;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::i8 [%0], %2, %6, %9, T;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::i8 [%0], %3, %7, %9, T;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::i8 [%0], %4, %8, %9, T;\n\t}"
+        ::"r"(d), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "r"(idesc), "r"(accumulate)
+        : "memory");
+  } else {
+    asm volatile(
+        "{\n\t.reg .pred P, T, A;\n\t"
+        "elect.sync _|P, 0xffffffff;\n\t"
+        "setp.ne.b32 A, %10, 0;\n\t"
+        "setp.eq.b32 T, 0, 0;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %9, A;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %6, %9, T;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::f16 [%0], %3, %7, %9, T;\n\t"
+        "@P tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %8, %9, T;\n\t}"
+        ::"r"(d), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "r"(idesc), "r"(accumulate)
+        : "memory");
+  }
+}
+//   block-scaled: scale bytes of the activations' plane and, where asked for, of the first factor, then the MMAs
+__device__ __forceinline__ void issue_four_mx(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate, uint64_t sfa, uint64_t sfb,
+                                              uint32_t copy_b, uint32_t tsfa, uint32_t tsfb) {
+  asm volatile(
+      "{\n\t.reg .pred P, Q, T, A;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "setp.ne.and.b32 Q, %18, 0, P;\n\t"
+      "setp.ne.b32 A, %13, 0;\n\t"
+      "setp.eq.b32 T, 0, 0;\n\t"
+      "@P tcgen05.cp.cta_group::1.32x128b.warpx4 [%14], %16;\n\t"
+      "@Q tcgen05.cp.cta_group::1.32x128b.warpx4 [%15], %17;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %1, %5, %9, [%14], [%15], A;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %2, %6, %10, [%14], [%15], T;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %3, %7, %11, [%14], [%15], T;\n\t"
+      "@P tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale [%0], %4, %8, %12, [%14], [%15], T;\n\t}"
+      ::"r"(d), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "r"(idesc), "r"(idesc | idesc_mx_ids(1)),
+      "r"(idesc | idesc_mx_ids(2)), "r"(idesc | idesc_mx_ids(3)), "r"(accumulate), "r"(tsfa), "r"(tsfb), "l"(sfa), "l"(sfb), "r"(copy_b)
+      : "memory");
+}
+
 template <int MAIN, int BR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmL1,
@@ -559,34 +609,28 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         const uint32_t at = base + (uint32_t)(sm.off_slots + slot * sm.slot);
-        if (elect_one()) {
-          for (int s = 0; s < ns; ++s) {
-            const int gs = c * spc + s;                          // stage of K: the accumulators take turns
-            const uint32_t d = set + (uint32_t)((gs & (p.nacc - 1)) * cols), more = gs >= p.nacc;
-            const uint32_t a = at + s * sm.a_ps * sm.a_unit, bw = at + sm.off_b + s * sm.b_ps * sm.b_unit;
-            if constexpr (BR == BR_INT) {
-              const uint64_t ad = make_smem_desc(a), bd = make_smem_desc(bw);
+#pragma unroll 1
+        for (int s = 0; s < ns; ++s) {
+          const int gs = c * spc + s;                            // stage of K: the accumulators take turns
+          const uint32_t d = set + (uint32_t)((gs & (p.nacc - 1)) * cols), more = gs >= p.nacc;
+          const uint32_t a = at + s * sm.a_ps * sm.a_unit, bw = at + sm.off_b + s * sm.b_ps * sm.b_unit;
+          if constexpr (BR == BR_INT) {
+            issue_four<TC_I8>(d, make_smem_desc(a), make_smem_desc(bw), IDESC_I8 | shape, more);
+          } else if constexpr (BR == BR_F16) {
+            issue_four<TC_F16>(d, make_smem_desc(a), make_smem_desc(bw), IDESC_F16 | shape, more);
+            issue_four<TC_F16>(d, make_smem_desc(a + sm.a_unit), make_smem_desc(bw + sm.b_unit), IDESC_F16 | shape, 1u);
+          } else {
+            // scale bytes into tensor memory (one slot: the tensor pipe executes these copies and MMAs in issue order), the
+            // activations' digit planes one after the other
+            constexpr int ap = BR == BR_MXINT ? 2 : 1;
+            const uint64_t sfb = make_smem_desc_plain(at + sm.off_sfb + s * 512, 16, 128);
 #pragma unroll
-              for (int j = 0; j < 4; ++j) tc_mma<TC_I8>(d, ad + 2 * j, bd + 2 * j, IDESC_I8 | shape, more | (uint32_t)j);
-            } else if constexpr (BR == BR_F16) {
-#pragma unroll
-              for (int j = 0; j < 8; ++j)
-                tc_mma<TC_F16>(d, make_smem_desc(a + (j >> 2) * sm.a_unit) + 2 * (j & 3), make_smem_desc(bw + (j >> 2) * sm.b_unit) + 2 * (j & 3),
-                               IDESC_F16 | shape, more | (uint32_t)j);
-            } else {
-              // scale bytes into tensor memory (one slot: the tensor pipe executes these copies and MMAs in issue order),
-              // then the activations' digit planes one after the other
-              const int ap = BR == BR_MXINT ? 2 : 1;
-              for (int u = 0; u < ap; ++u) tc_cp_sf(tsf + 4 * u, make_smem_desc_plain(at + sm.off_sfa + (s * ap + u) * 512, 16, 128));
-              tc_cp_sf(tsf + 8, make_smem_desc_plain(at + sm.off_sfb + s * 512, 16, 128));
-              for (int u = 0; u < ap; ++u) {
-                const uint64_t ad = make_smem_desc(a + u * sm.a_unit), bd = make_smem_desc(bw);
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  tc_mma_mx(d, ad + 2 * j, bd + 2 * j, idesc_mx(cols, j), tsf + 4 * u, tsf + 8, more | (uint32_t)(j | u));
-              }
-            }
+            for (int u = 0; u < ap; ++u)
+              issue_four_mx(d, make_smem_desc(a + u * sm.a_unit), make_smem_desc(bw), idesc_mx(cols, 0), more | (uint32_t)u,
+                            make_smem_desc_plain(at + sm.off_sfa + (s * ap + u) * 512, 16, 128), sfb, (uint32_t)(u == 0), tsf + 4 * u, tsf + 8);
           }
+        }
+        if (elect_one()) {
           tc_commit(bar_empty(slot));
           if (c + 1 == p.nchunks) tc_commit(bar_tfull(tc & 1));
         }
