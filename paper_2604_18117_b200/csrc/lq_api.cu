@@ -366,6 +366,20 @@ lq_status lq_make_tmap_bytes(CUtensorMap* tm, void* base, uint64_t rows, uint64_
   return r == CUDA_SUCCESS ? LQ_OK : LQ_ERR_CUDA;
 }
 
+// The same for packed elements of 4 or 6 bits: 16 of them land in 16 bytes of shared memory, data first and then a gap, as the
+// MMA reads operands of less than eight bits.
+static lq_status make_tmap_packed(CUtensorMap* tm, void* base, uint64_t rows, uint64_t row_elems, int bits, uint32_t box_rows) {
+  encode_tiled_fn fn = get_encode_fn();
+  if (!fn) return LQ_ERR_CUDA;
+  cuuint64_t dims[2] = {row_elems, rows};
+  cuuint64_t strides[1] = {row_elems / 8 * bits};
+  cuuint32_t box[2] = {128, box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = fn(tm, bits == 4 ? CU_TENSOR_MAP_DATA_TYPE_16U4_ALIGN16B : CU_TENSOR_MAP_DATA_TYPE_16U6_ALIGN16B, 2, base, dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? LQ_OK : LQ_ERR_CUDA;
+}
+
 // ---- device status word ------------------------------------------------------------------
 static int32_t* g_status[64] = {nullptr};
 static std::mutex g_status_mu;
@@ -439,17 +453,22 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
   try {
     std::vector<int> wrow(Npad), srow(Npad);                     // places of column n in the weight operand and the vectors
     for (int n = 0; n < Npad; ++n) { wrow[n] = L->mx ? lq_col32_slot(n) : lq_col_slot(n); srow[n] = L->mx ? n : lq_colscale_slot(n); }
-    std::vector<uint8_t> w8((size_t)Npad * Kpad, lq_encode_code_host(0, L->main_kind));
-    uint8_t code_byte[16] = {};                                       // operand byte of each 4-bit code
-    for (int q = -7; q <= 7; ++q) code_byte[q & 15] = lq_encode_code_host(q, L->main_kind);
-    // transposed in blocks that stay in the cache (K x N = 1152 x 4608: the whole upload 9.9 ms row by row, 5.2 so)
+    const int bits = L->mx ? lq_mx_weight_bits(L) : 8, row_bytes = Kpad / 8 * bits;
+    std::vector<uint8_t> w8((size_t)Npad * row_bytes, L->mx ? 0 : lq_encode_code_host(0, L->main_kind));
+    uint8_t code[256] = {};                                      // operand element of each code's (mxfp: e4m3) byte
+    if (L->mxfp) for (int i = 0; i < 16; ++i) code[e2m1_to_e4m3((uint8_t)i)] = (uint8_t)i;
+    else for (int q = -7; q <= 7; ++q) code[(uint8_t)(int8_t)q] = L->mx ? lq_code_e2m3(q) : lq_encode_code_host(q, L->main_kind);
+    const uint8_t* src = L->mxfp ? L->Wq8h.data() : reinterpret_cast<const uint8_t*>(L->Wq.data());
+    // transposed in blocks that stay in the cache (K x N = 1152 x 4608: the whole upload 9.9 ms row by row, 5.2 so), four elements
+    // at a time
     for (int k0 = 0; k0 < K; k0 += 64)
       for (int n0 = 0; n0 < N; n0 += 64)
-        for (int n = n0; n < std::min(n0 + 64, N); ++n) {
-          uint8_t* row = &w8[(size_t)wrow[n] * Kpad];
-          for (int k = k0; k < std::min(k0 + 64, K); ++k)
-            row[k] = L->mxfp ? L->Wq8h[(size_t)k * N + n] : code_byte[L->Wq[(size_t)k * N + n] & 15];
-        }
+        for (int n = n0; n < std::min(n0 + 64, N); ++n)
+          for (int k = k0; k < std::min(k0 + 64, K); k += 4) {
+            uint32_t v = 0;
+            for (int i = 0; i < std::min(4, K - k); ++i) v |= (uint32_t)code[src[(size_t)(k + i) * N + n]] << (bits * i);
+            memcpy(&w8[(size_t)wrow[n] * row_bytes + k / 4 * (bits / 2)], &v, bits / 2);
+          }
     if ((st = upload(&L->d_Wq8, w8)) != LQ_OK) return st;
     if (L->mx) {
       // E8M0 bytes (exponent + 127) in the layout the block-scaled MMA reads from tensor memory, by tile width; 127 = 2^0 for padding
@@ -576,13 +595,13 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
     if ((st = upload(&L->d_sL2, s2)) != LQ_OK) return st;
     if ((st = upload(&L->d_L2c, l2c)) != LQ_OK) return st;
   } catch (const std::bad_alloc&) { return LQ_ERR_ALLOC; }
-  if ((st = lq_make_tmap_bytes(&L->tmB, L->d_Wq8, Npad, Kpad, LQ_BN)) != LQ_OK) return st;
+  if (!L->mx && (st = lq_make_tmap_bytes(&L->tmB, L->d_Wq8, Npad, Kpad, LQ_BN)) != LQ_OK) return st;
   for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
     if (!L->d_sfbw[wi]) continue;
     const uint32_t width = (uint32_t)LQ_MX_WIDTHS[wi];
-    if ((st = lq_make_tmap_bytes(&L->tmBw[wi], L->d_Wq8, Npad, Kpad, width)) != LQ_OK) return st;
+    if ((st = make_tmap_packed(&L->tmBw[wi], L->d_Wq8, Npad, Kpad, lq_mx_weight_bits(L), width)) != LQ_OK) return st;
     if ((st = lq_make_tmap_bytes(&L->tmL2w[wi], L->d_L2c, Npad, LQ_RCONT, width)) != LQ_OK) return st;
-    if ((st = lq_make_tmap_bytes(&L->tmBp[wi], L->d_Wq8, Npad, Kpad, width / 2)) != LQ_OK) return st;
+    if ((st = make_tmap_packed(&L->tmBp[wi], L->d_Wq8, Npad, Kpad, lq_mx_weight_bits(L), width / 2)) != LQ_OK) return st;
     if ((st = lq_make_tmap_bytes(&L->tmL2p[wi], L->d_L2c, Npad, LQ_RCONT, width / 2)) != LQ_OK) return st;
   }
   if (r > 0 && (st = lq_make_tmap_bytes(&L->tmL1, L->d_L1c, (uint64_t)rn * lq_l1_planes(L), (uint64_t)Kpad * (L->f16_branch ? 2 : 1),

@@ -326,6 +326,7 @@ constexpr uint32_t IDESC_F16 = (1u << 4) | (0u << 7) | (0u << 10);   // F16 x F1
 __device__ __forceinline__ constexpr uint32_t idesc_mx2(int n, int a_sf_id, int b_sf_id) {
   return ((uint32_t)b_sf_id << 4) | ((uint32_t)(n >> 3) << 17) | (1u << 23) | ((uint32_t)(LQ_BM >> 4) << 24) | ((uint32_t)a_sf_id << 29);
 }
+constexpr uint32_t IDESC_MX_B_E2M1 = 5u << 10, IDESC_MX_B_E2M3 = 3u << 10;   // added: the B operand is E2M1, E2M3
 __device__ __forceinline__ constexpr uint32_t idesc_mx_ids(int sf_id) { return ((uint32_t)sf_id << 4) | ((uint32_t)sf_id << 29); }   // the scale-byte ids alone
 __device__ __forceinline__ constexpr uint32_t idesc_mx(int n, int sf_id) { return idesc_mx2(n, sf_id, sf_id); }
 

@@ -5,8 +5,8 @@
 //
 // Here the tensor core applies the scales itself: tcgen05.mma kind::mxf8f6f4.block_scale takes one E8M0 scale
 // per operand row and 32-deep K block from tensor memory, so ALL blocks of a tile accumulate into ONE fp32
-// accumulator and nothing has to be drained per block.  The 4-bit codes ride in E4M3 operands as in the SINT4
-// kernel.  Products q q' 2^(e+e') are exact in fp32; their sum is rounded by the tensor core's fp32 accumulation.
+// accumulator and nothing has to be drained per block.  The activations' codes ride in E4M3 operands as in the SINT4
+// kernel, the weights' in packed E2M3 ones (MXFP4: E2M1).  Products q q' 2^(e+e') are exact in fp32; their sum is rounded by the tensor core's fp32 accumulation.
 //
 // Shape of the kernel (persistent, one CTA per SM, warp-specialised, 18 warps): tiles of 128 rows x W columns, W chosen by
 // the launcher (pick_width).
@@ -25,8 +25,12 @@
 // main loop: 2 W (3 W) columns and 12 for the scale factors of a stage (one slot: the tensor pipe executes one thread's
 // tcgen05 copies and MMAs in issue order).  A single 256-column accumulator spent a third of a short-K launch on the
 // hand-over and the stores behind it (M = 8192, K x N = 1152 x 3456, MXFP rank 64: 36.4 us, 28 without the stores).
-// What bounds it: operand delivery from the L2 (W = 256: 48 KB a stage; 70-78 bytes per clock and SM with all SMs at it),
-// the tensor pipe close behind (2 W clocks a stage).
+// What bounds it: power.  The tensor pipe needs 2 W clocks a stage and the L2 delivers 70-78 bytes per clock and SM with all SMs
+// at it, which at W = 192 and pairs comes to about the same; a stage takes 440 clocks of 384, at the 1.45-1.5 GHz that the
+// power cap leaves (1.82 GHz with narrow tiles that keep the pipe waiting).  So bytes not moved count twice: pairs stage half
+// the weights each, and the weights stay packed up to shared memory, 4 bits as e2m1 (MXFP4) or 6 as e2m3 (integer codes),
+// where TMA spreads them out.  M = 8192, MXFP: 1152 x 3456 30.6 -> 29.4 us, 2240 x 6720 95.3 -> 91.1, 5600 x 2240 79.4 ->
+// 75.5; integer codes 33.8 -> 33.4 and 51.3 -> 50.5.
 // What was measured on the way here (PixArt block, four GEMMs): the branch on mma.sync in the drain warps took tensor
 // time from the main loop; TMA stores of the output (32 boxes of 2 KB, or 8 of 8 KB, per tile) cost 15 % against
 // plain stores - they share the TMA unit with the operand loads.
@@ -80,6 +84,8 @@ struct MxParams {
   const uint8_t* sfl2;    // branch_mx: E8M0 bytes of L2's block scales, [tiles_n][sf_chunks][512]
   int tiles_m, tiles_n;
   int width, stages;      // W, operand ring depth
+  int b_row;              // bytes of a weight row that a stage copies
+  uint32_t b_format;      // format field of the weights in the instruction descriptor
   int b_wrap;             // Kpad / 128: stage s reads B (and its scales) at stage s mod b_wrap - the planes share the weights
   const uint8_t* sfa;     // [Mpad/128][k_stages][512]
   const uint8_t* sfb;     // [Kpad/128][tiles_n][sf_chunks][512]
@@ -236,7 +242,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     auto load_b = [&](int st, int s, int nu) {         // the weights' half of main stage s; announces the whole stage
       const uint32_t dst = sm_stage + st * stage_bytes + STAGE_A_BYTES, full = bar(B_FULL + st);
       const int sb = s >= p.b_wrap ? s - p.b_wrap : s; // the lo digits' plane runs over the same weights
-      load_weights_stage(full, stage_bytes + SF_BYTES + sfb_bytes, dst, &tmB, sb * LQ_KSTAGE, nu * W + (int)rank * BW, sm_sf + st * STAGE_SF_BYTES + SF_BYTES,
+      load_weights_stage(full, STAGE_A_BYTES + (uint32_t)BW * p.b_row + SF_BYTES + sfb_bytes, dst, &tmB, sb * LQ_KSTAGE, nu * W + (int)rank * BW, sm_sf + st * STAGE_SF_BYTES + SF_BYTES,
                          p.sfb + ((size_t)sb * p.tiles_n + nu) * sfb_bytes, sfb_bytes);
     };
     auto load_a = [&](int st, int s, int mb) {
@@ -374,7 +380,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + STAGE_A_BYTES);
         const uint32_t sf = sm_sf + st * STAGE_SF_BYTES;
         auto issue = PAIR ? issue_main_stage_pair : issue_main_stage_one;
-        issue(d, adesc, bdesc, idesc_mx(W, 0) + ROWS256, make_smem_desc_plain(sf, 16, 128), make_smem_desc_plain(sf + SF_BYTES, 16, 128),
+        issue(d, adesc, bdesc, (idesc_mx(W, 0) | p.b_format) + ROWS256, make_smem_desc_plain(sf, 16, 128), make_smem_desc_plain(sf + SF_BYTES, 16, 128),
               (uint32_t)(p.sf_chunks == 2), (uint32_t)s, bar(B_EMPTY + st));
         if (++st == NST) { st = 0; par ^= 1; }
         LQ_TL(EV_M_ISSUED, s);
@@ -535,9 +541,11 @@ int smem_bytes(int bw) {
   return FIXED_SMEM + ring_stages(bw) * (STAGE_A_BYTES + bw * LQ_KSTAGE + STAGE_SF_BYTES);
 }
 
-// Index (LQ_MX_WIDTHS) of the tile width for a launch.  Model, in clocks: a stage takes the longer of its MMAs (2 W) and its
-// operands' way from the L2 (70 bytes per clock and SM); a tile the longer of its stages and the drain of the tile before; a
-// launch the tiles of the CTA with the most, plus the last drain and the filling of the ring.
+// Index (LQ_MX_WIDTHS) of the tile width for a launch.  Model, in clocks: a stage takes the longest of its MMAs (2 W, and 40 where
+// one stage's meet the next's), its operands' way from the L2 (70 bytes per clock and SM) and its hand-shakes (350: what a
+// stage of 64 columns takes); a tile the longer of its stages and the drain of the tile before; a launch the tiles of the CTA
+// with the most, plus the last drain and the filling of the ring.  Measured, M = 8192, K x N = 4608 x 1152, W = 64 / 128 / 192 /
+// 224: 58 / 37.9 / 35.3 / 38.0 us; 1152 x 3456: 52.5 / 34.2 / 30.3 / 30.0; 2240 x 2240: 61 / 39.6 / 36.3 / 35.0.
 int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas, bool pair) {
   int best = -1;
   double best_cost = 1e30;
@@ -547,7 +555,7 @@ int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas, bool pair) 
     if (g_lq_gemm_width > 0 && w != g_lq_gemm_width) continue;
     const int c = pair ? 2 : 1, units = ctas / c;
     const long long tiles = (long long)lq_ceil_div(tiles_m, c) * lq_ceil_div(L->N, w);
-    const double stage = std::max(2.0 * w, (STAGE_A_BYTES + w / c * LQ_KSTAGE) / 70.0);
+    const double stage = std::max({2.0 * w + 40.0, 350.0, (STAGE_A_BYTES + w / c * LQ_KSTAGE / 8 * lq_mx_weight_bits(L)) / 70.0});
     const double drain = 600.0 + 1200.0 * lq_ceil_div(w, 128);
     const double cost = (double)((tiles + units - 1) / units) * std::max(stages * stage, drain) + drain + 4.0 * stage;
     if (cost < best_cost) { best_cost = cost; best = i; }
@@ -586,6 +594,7 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   if (wi < 0) return LQ_ERR_INVALID_ARG;
   p.width = LQ_MX_WIDTHS[wi]; p.stages = ring_stages(pair ? p.width / 2 : p.width); p.sf_chunks = lq_ceil_div(p.width, 128);
   p.tiles_n = lq_ceil_div(L->N, p.width);
+  p.b_row = LQ_KSTAGE / 8 * lq_mx_weight_bits(L); p.b_format = L->mxfp ? IDESC_MX_B_E2M1 : IDESC_MX_B_E2M3;
   p.sfa = A->d_sfa; p.sfb = L->d_sfbw[wi]; p.sft = A->d_sft; p.sfl2 = L->d_sfl2w[wi];
   p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
   p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;

@@ -100,7 +100,7 @@ struct lq_layer {
   // device copy, operand layouts
   int device;
   int main_kind;               // LQ_KIND_*: byte encoding of the 4-bit codes in the MMA operands
-  uint8_t* d_Wq8;              // [Npad][Kpad] bytes, K contiguous (B operand, K-major; rows in lq_col_slot order, MX: lq_col32_slot)
+  uint8_t* d_Wq8;              // MX: packed, [Npad][Kpad] e2m1 (mxfp) or e2m3 elements; SINT4: [Npad][Kpad] e4m3 bytes, K contiguous (B operand, K-major; rows in lq_col_slot order, MX: lq_col32_slot)
   float* d_sw;                 // [Gpad][Npad] fp32 (exact images of the fp16 scales), in lq_colscale_slot order
   uint8_t* d_L1c;              // [planes * rn][Kpad] bytes (W16A16: [rn][Kpad] halves), K contiguous: first factor as the B operand of
                                // the down-projection; rn = lq_l1_rows; MXINT8 factors: the hi digits' rows, then the lo digits'
@@ -175,6 +175,14 @@ static inline uint8_t lq_encode_code_host(int q, int kind) {
   static const uint8_t mag[8] = {0x00, 0x38, 0x40, 0x44, 0x48, 0x4A, 0x4C, 0x4E};  // E4M3 of 0..7
   int a = q < 0 ? -q : q;
   return (uint8_t)(mag[a] | (q < 0 ? 0x80 : 0));
+}
+
+// bits of a packed weight element of the MX GEMM: MXFP4 as e2m1, the 4-bit integer codes as e2m3 (the narrowest type that has them)
+static inline int lq_mx_weight_bits(const lq_layer* L) { return L->mxfp ? 4 : 6; }
+// E2M3 of an integer in [-7, 7] (bias 1, three mantissa bits)
+static inline uint8_t lq_code_e2m3(int q) {
+  static const uint8_t mag[8] = {0, 8, 16, 20, 24, 26, 28, 30};
+  return (uint8_t)((q < 0 ? 0x20 : 0) | mag[q < 0 ? -q : q]);
 }
 
 extern int g_lq_main_kind;   // option "main_kind"
