@@ -48,31 +48,23 @@
 #include <type_traits>
 
 #include "lq_device.cuh"
+#include "lq_quant_cut.h"
 
 namespace {
 
 using namespace lqdev;
+using namespace lqcut;
 
-constexpr int QWARPS = 15;             // quantizer warps (at most; teams of RG * SX): 20 warps are the most that leave 96 registers each
 constexpr int FIRST_QWARP = 5;         // warps 0-1 a4, 2 MMA, 3 X, 4 first factor
 constexpr int NTHREADS = (FIRST_QWARP + QWARPS) * 32;
-constexpr int MAX_SLOTS = 4;           // chunk slots of the branch's operands
-constexpr int MAX_UNSETTLED = 32;      // list of a4's rows to look at again, per warp
-constexpr int MAX_XSLOTS = 12;         // chunk slots of X
 constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer (ties to even)
-enum { BR_NONE = 0, BR_INT = 1, BR_F16 = 2, BR_MXFP = 3, BR_MXINT = 4 };
 // MXFP: MXFP8e4 activation codes for an MXFP4 weight; MXINT8: MXINT8 activation codes for an MXINT4 weight, stored as
 // two E4M3 digit planes (code = 16 hi + lo); MXFP6: MXFP6e2 activation codes, stored as the E4M3 bytes of the same values
 enum { MAIN_SINT4 = 0, MAIN_MXINT4 = 1, MAIN_MXFP = 2, MAIN_MXINT8 = 3, MAIN_MXFP6 = 4 };
 
-struct QuantParams {
+struct QuantParams : QuantCut {
   int M, K, Kpad, Mpad;
   int nst;              // Kpad / 128 stages of K
-  int groups, stages;   // RG row groups of 8 per tile, SX stages of K per chunk
-  int teams;            // teams of RG * SX quantizer warps: they take the chunks in turn
-  int ntiles, nchunks;  // tiles of the launch, chunks of a tile
-  int slots, xslots;    // chunk slots of the branch's operands and of X
-  int refetch;          // integer branch: the X ring is smaller than a tile, which is streamed twice
   uint8_t* qx8;         // [Mpad][Kpad] (MXINT8: [Mpad][2 Kpad], the hi digits' plane then the lo digits')
   float* sx;            // [Gpad][Mpad]
   uint8_t* sfa;         // MX: E8M0 scale bytes [Mpad/128][Kpad/128][512] (MXINT8: [Mpad/128][2 Kpad/128][512], by plane)
@@ -90,42 +82,10 @@ struct QuantParams {
   int nacc, sets;       // accumulators a tile's stages alternate over (floating-point branches: shorter chains of fp32 sums),
                         // sets of them (2: the next tile's MMAs run under a4)
   int tmem_cols;        // power of two
-  int smem;             // dynamic shared memory of the launch
   float dev;            // MXFP: how far a sum of the tensor core may be from the one in defining order, over its block's maximum
   float qm;             // largest branch activation code
   int32_t* status;
 };
-
-// Shared memory, from a 1024-byte aligned base; the same arithmetic on the host (size) and in the kernel.  First the X ring,
-// then the slots: a slot holds a chunk's operand slabs (128 bytes of K wide, a_ps and b_ps of them per stage) and scale bytes.
-struct QuantSmem {
-  int xslot, a_unit, a_ps, b_unit, b_ps;
-  int off_b, off_sfa, off_sfb, slot;            // within a slot
-  int off_slots, off_l1, off_max, off_sb, off_bar, total;
-};
-__host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, int bplanes, int slots, int xslots) {
-  QuantSmem s{};
-  const bool mx = br == BR_MXFP || br == BR_MXINT;
-  s.xslot = tr * 256 * st;                      // st: stages of K per chunk
-  s.a_unit = tr * 128; s.b_unit = rn * bplanes * 128;
-  s.a_ps = br == BR_NONE ? 0 : (br == BR_F16 || br == BR_MXINT) ? 2 : 1;
-  s.b_ps = br == BR_NONE ? 0 : br == BR_F16 ? 2 : 1;
-  s.off_b = st * s.a_ps * s.a_unit;
-  s.off_sfa = s.off_b + st * s.b_ps * s.b_unit;
-  s.off_sfb = s.off_sfa + (mx ? st * s.a_ps * 512 : 0);
-  s.slot = s.off_sfb + (mx ? st * s.b_ps * 512 : 0);
-  s.slot = (s.slot + 1023) & ~1023;
-  s.off_slots = xslots * s.xslot;
-  s.off_l1 = s.off_slots + (br == BR_NONE ? 0 : slots) * s.slot;
-  s.off_max = s.off_l1 + (br == BR_MXFP ? 2 * MAX_UNSETTLED * 16 + 256 * 4 : LQ_MAX_RANK * 4);   // sL1; MXFP: list, scratch
-  // row maxima of three tiles in rotation, row scales of two
-  s.off_sb = s.off_max + 3 * 64 * 4;
-  s.off_bar = s.off_sb + 2 * 64 * 4;
-  s.total = s.off_bar + 8 * (2 * MAX_XSLOTS + 3 * MAX_SLOTS + 5) + 16;
-  // the 128-row MMA reads past the last slab of a shorter tile
-  if (br != BR_NONE && s.total < s.off_l1 + 128 * 128) s.total = s.off_l1 + 128 * 128;
-  return s;
-}
 
 // Position in a ring of n slots and the parity its barriers have there.
 struct Ring {
@@ -997,47 +957,6 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   }
 }
 
-// How a launch is cut.  Cost model in rounds, a round being one chunk for every team: a CTA's tiles times (its rounds,
-// twice where a tile is walked twice, plus what starting and finishing a tile costs).
-// A team may only run ahead of the others as far as one-bit phases tell its slots apart: there are at least as many operand
-// slots as teams, and X slots for two rounds.
-bool plan_cut(int br, QuantParams& p, int sms) {
-  const int walks = br == BR_INT ? 2 : 1, room = 227 * 1024 - 1024;
-  double best = 1e30;
-  QuantParams out = p;
-  for (int groups = 8; groups >= 1; --groups) {
-    if (g_lq_quant_warps > 0 && groups != std::min(8, g_lq_quant_warps)) continue;
-    for (int stages = 1; stages <= std::min(QWARPS / groups, p.nst); ++stages) {
-      if (g_lq_quant_ctas > 0 && stages != g_lq_quant_ctas) continue;
-      QuantParams c = p;
-      c.groups = groups; c.stages = stages;
-      c.ntiles = lq_ceil_div(p.M, 8 * groups);
-      c.nchunks = lq_ceil_div(p.nst, stages);
-      for (c.teams = std::min(std::min(QWARPS / (groups * stages), c.nchunks), MAX_SLOTS); c.teams >= 1; --c.teams) {
-        c.xslots = 0;
-        // operand slots first, then as many chunks of X as fit; an integer branch would rather hold a whole tile of X
-        const int want = br == BR_INT ? c.nchunks : 2 * c.teams + 2, least = std::max(2, 2 * c.teams - 1);
-        for (int slots = br == BR_NONE ? 1 : MAX_SLOTS; slots >= (br == BR_NONE ? 1 : std::max(2, c.teams)) && c.xslots < want; --slots) {
-          const QuantSmem s = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, slots, 0);
-          const int fit = std::min(MAX_XSLOTS, (room - s.total) / s.xslot);
-          if (fit > c.xslots && fit >= least) { c.xslots = fit; c.slots = slots; }
-        }
-        if (c.xslots == 0) continue;
-        c.xslots = std::min(c.xslots, std::max(least, 2 * c.nchunks));
-        c.refetch = br == BR_INT && c.xslots < c.nchunks;
-        c.smem = quant_smem(br, 8 * groups, stages, p.rn, p.bplanes, c.slots, c.xslots).total + 1024;
-        const int warps = groups * stages * c.teams;
-        const double round = 0.4 + 0.6 * warps / QWARPS;
-        const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + 1.0) + 3.0;
-        if (cost < best - 1e-9) { best = cost; out = c; }
-        break;
-      }
-    }
-  }
-  p = out;
-  return best < 1e30;
-}
-
 template <int MAIN, int BR>
 cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, int sms, cudaStream_t st) {
   static bool attr_set[64] = {false};
@@ -1048,7 +967,7 @@ cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, i
     if (e != cudaSuccess) return e;
     attr_set[dev & 63] = true;
   }
-  if (!plan_cut(BR, p, sms)) return cudaErrorInvalidConfiguration;
+  if (!plan_cut(BR, p.M, p.nst, p.rn, p.bplanes, sms, g_lq_quant_warps, g_lq_quant_ctas, p)) return cudaErrorInvalidConfiguration;
   // Floating-point branches: a tile's stages alternate over up to four accumulators, which are added in fp32 at the end
   // (each costs a4 a trip to tensor memory per 16 columns: not more than 128 columns of them).  Tensor memory holds two
   // such sets - one where every CTA has a single tile - and the scale bytes' columns.

@@ -1,0 +1,108 @@
+// How a launch of the quantizer kernel is cut: rows per tile, stages of K per chunk, teams of warps, ring slots, shared memory.
+// Host arithmetic only (and the shared-memory map, which the kernel uses too), apart from the kernel so that a test can compile it
+// by itself.  Internal: not part of the C ABI.
+#pragma once
+
+#include <algorithm>
+
+#include "lq_internal.h"
+
+namespace lqcut {
+
+constexpr int QWARPS = 15;             // quantizer warps (at most; teams of RG * SX): 20 warps are the most that leave 96 registers each
+constexpr int MAX_SLOTS = 4;           // chunk slots of the branch's operands
+constexpr int MAX_UNSETTLED = 32;      // list of a4's rows to look at again, per warp
+constexpr int MAX_XSLOTS = 12;         // chunk slots of X
+enum { BR_NONE = 0, BR_INT = 1, BR_F16 = 2, BR_MXFP = 3, BR_MXINT = 4 };
+
+struct QuantCut {
+  int groups, stages;   // RG row groups of 8 per tile, SX stages of K per chunk
+  int teams;            // teams of RG * SX quantizer warps: they take the chunks in turn
+  int ntiles, nchunks;  // tiles of the launch, chunks of a tile
+  int slots, xslots;    // chunk slots of the branch's operands and of X
+  int refetch;          // integer branch: the X ring is smaller than a tile, which is streamed twice
+  int smem;             // dynamic shared memory of the launch
+};
+
+// Shared memory, from a 1024-byte aligned base; the same arithmetic on the host (size) and in the kernel.  First the X ring,
+// then the slots: a slot holds a chunk's operand slabs (128 bytes of K wide, a_ps and b_ps of them per stage) and scale bytes.
+struct QuantSmem {
+  int xslot, a_unit, a_ps, b_unit, b_ps;
+  int off_b, off_sfa, off_sfb, slot;            // within a slot
+  int off_slots, off_l1, off_max, off_sb, off_bar, total;
+};
+__host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, int bplanes, int slots, int xslots) {
+  QuantSmem s{};
+  const bool mx = br == BR_MXFP || br == BR_MXINT;
+  s.xslot = tr * 256 * st;                      // st: stages of K per chunk
+  s.a_unit = tr * 128; s.b_unit = rn * bplanes * 128;
+  s.a_ps = br == BR_NONE ? 0 : (br == BR_F16 || br == BR_MXINT) ? 2 : 1;
+  s.b_ps = br == BR_NONE ? 0 : br == BR_F16 ? 2 : 1;
+  s.off_b = st * s.a_ps * s.a_unit;
+  s.off_sfa = s.off_b + st * s.b_ps * s.b_unit;
+  s.off_sfb = s.off_sfa + (mx ? st * s.a_ps * 512 : 0);
+  s.slot = s.off_sfb + (mx ? st * s.b_ps * 512 : 0);
+  s.slot = (s.slot + 1023) & ~1023;
+  s.off_slots = xslots * s.xslot;
+  s.off_l1 = s.off_slots + (br == BR_NONE ? 0 : slots) * s.slot;
+  s.off_max = s.off_l1 + (br == BR_MXFP ? 2 * MAX_UNSETTLED * 16 + 256 * 4 : LQ_MAX_RANK * 4);   // sL1; MXFP: list, scratch
+  // row maxima of three tiles in rotation, row scales of two
+  s.off_sb = s.off_max + 3 * 64 * 4;
+  s.off_bar = s.off_sb + 2 * 64 * 4;
+  s.total = s.off_bar + 8 * (2 * MAX_XSLOTS + 3 * MAX_SLOTS + 5) + 16;
+  // the 128-row MMA reads past the last slab of a shorter tile
+  if (br != BR_NONE && s.total < s.off_l1 + 128 * 128) s.total = s.off_l1 + 128 * 128;
+  return s;
+}
+
+// Cost model in rounds, a round being one chunk for every team: a CTA's tiles times (its rounds,
+// twice where a tile is walked twice, plus what starting and finishing a tile costs).
+//
+// Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
+// one: the chunk that was in the slot before has to be known to have landed (X) or to have been multiplied (operands).
+//   operands  MMAs retire in order, and a team waits for the slots of its own chunks, so as many slots as teams are enough
+//   X         copies land in any order.  A team has seen its own earlier chunks land, so the ring holds a multiple of the teams
+//             and the chunk before was its own - unless the chunk before is known to have landed for another reason: an
+//             integer branch's ring holds a whole tile (the teams meet between the two walks, having seen all of it), or the ring is
+//             as long as the teams and the operand slots together (the slot that the team waited for last was free, so every
+//             chunk up to the one before had been multiplied).
+inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int force_groups, int force_stages, QuantCut& out) {
+  const int walks = br == BR_INT ? 2 : 1, room = 227 * 1024 - 1024;
+  double best = 1e30;
+  for (int groups = 8; groups >= 1; --groups) {
+    if (force_groups > 0 && groups != std::min(8, force_groups)) continue;
+    for (int stages = 1; stages <= std::min(QWARPS / groups, nst); ++stages) {
+      if (force_stages > 0 && stages != force_stages) continue;
+      QuantCut c{};
+      c.groups = groups; c.stages = stages;
+      c.ntiles = lq_ceil_div(M, 8 * groups);
+      c.nchunks = lq_ceil_div(nst, stages);
+      for (c.teams = std::min(std::min(QWARPS / (groups * stages), c.nchunks), MAX_SLOTS); c.teams >= 1; --c.teams) {
+        c.xslots = 0;
+        // operand slots first, then as many chunks of X as fit; an integer branch would rather hold a whole tile of X
+        const int want = br == BR_INT ? c.nchunks : 2 * c.teams + 2;
+        for (int slots = br == BR_NONE ? 1 : MAX_SLOTS; slots >= (br == BR_NONE ? 1 : std::max(2, c.teams)) && c.xslots < want; --slots) {
+          const QuantSmem s = quant_smem(br, 8 * groups, stages, rn, bplanes, slots, 0);
+          int fit = std::min(MAX_XSLOTS, (room - s.total) / s.xslot);
+          const bool whole = br == BR_INT && fit >= c.nchunks, behind = br != BR_NONE && br != BR_INT && fit >= c.teams + slots;
+          if (!whole && !behind) fit -= fit % c.teams;
+          if (fit > c.xslots && fit >= std::max(2, 2 * c.teams - (whole ? 1 : 0))) { c.xslots = fit; c.slots = slots; }
+        }
+        if (c.xslots == 0) continue;
+        // no more than two tiles of X (whole turns of the teams, for the reason above)
+        const int two = br == BR_INT && c.xslots >= c.nchunks ? std::max(2 * c.teams - 1, 2 * c.nchunks) : lq_round_up(2 * c.nchunks, c.teams);
+        c.xslots = std::min(c.xslots, std::max(2, two));
+        c.refetch = br == BR_INT && c.xslots < c.nchunks;
+        c.smem = quant_smem(br, 8 * groups, stages, rn, bplanes, c.slots, c.xslots).total + 1024;
+        const int warps = groups * stages * c.teams;
+        const double round = 0.4 + 0.6 * warps / QWARPS;
+        const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + 1.0) + 3.0;
+        if (cost < best - 1e-9) { best = cost; out = c; }
+        break;
+      }
+    }
+  }
+  return best < 1e30;
+}
+
+}  // namespace lqcut
