@@ -26,15 +26,26 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// CLUSTER: the barrier's arrivals come from another CTA of the cluster, too, and what they hand over is acquired at that scope.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
+  if constexpr (CLUSTER)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
   return ok != 0;
 }
 
@@ -54,11 +65,12 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
 
 // Bounded wait.  Returns false when the CTA is aborting or the deadline passed (then it raises the abort flag
 // and records who gave up in the device status word {code, stage}).
+template <bool CLUSTER = false>
 static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                             int role, long long limit = WAIT_LIMIT_CYCLES) {
   const long long t0 = clock64();
   for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
     if ((it & 0xFF) == 0) {
       if (*abort_flag) return false;
       if (clock64() - t0 > limit) {
@@ -69,10 +81,11 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity
     }
   }
 }
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                           int role) {
-  if (mbar_try_wait(bar, parity)) return true;
-  return mbar_wait_slow(bar, parity, abort_flag, status, role);
+  if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
+  return mbar_wait_slow<CLUSTER>(bar, parity, abort_flag, status, role);
 }
 // The same wait without a call on its slow path: for a warp whose registers are full of data, where a call would save and
 // restore them all.
@@ -92,9 +105,10 @@ __device__ __forceinline__ bool mbar_wait_inline(uint32_t bar, uint32_t parity, 
   }
 }
 // The same wait for a whole warp whose control flow must stay provably uniform.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                                int role) {
-  const bool ok = mbar_wait(bar, parity, abort_flag, status, role);
+  const bool ok = mbar_wait<CLUSTER>(bar, parity, abort_flag, status, role);
   return __all_sync(0xffffffffu, ok);
 }
 // Abort path only: gives a transaction that is still in flight on `bar` a bounded time to land, so that no
@@ -123,10 +137,15 @@ __device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
   return a;
 }
-// Relaxed: what is handed over is not generic memory (operands that a bulk copy has completed, tensor memory that
-// tcgen05.wait::ld has emptied).  As a release the arrival waits for the thread's stores to be performed, over a thousand
-// clocks where it sits in a loop.
+// Arrival on a barrier of another CTA.  What was observed to be in this CTA's shared memory before it is visible to the waiter
+// (which acquires at cluster scope).
 __device__ __forceinline__ void peer_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// The same where no memory is handed over but tensor memory that tcgen05.wait::ld has emptied, ordered by the tcgen05 fences on
+// both sides: relaxed.  As a release the arrival waits for the thread's earlier stores - a drain warp's stores of Y - to be
+// performed, over a thousand clocks.
+__device__ __forceinline__ void peer_arrive_tmem(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ float4 lds_peer_v4(uint32_t a) {

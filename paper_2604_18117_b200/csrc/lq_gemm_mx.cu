@@ -361,13 +361,13 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     constexpr uint32_t ROWS256 = PAIR ? (uint32_t)(LQ_BM >> 4) << 24 : 0;    // added to a 128-row descriptor's M field: 256
     auto stage_full = [&]() {
       return mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA) &&
-             (!PAIR || mbar_wait_warp(bar(B_PFULL + st), par, abort_flag, p.status, LQ_STAGE_MMA));
+             (!PAIR || mbar_wait_warp<PAIR>(bar(B_PFULL + st), par, abort_flag, p.status, LQ_STAGE_MMA));
     };
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
       const int buf = tc & 1;
       const uint32_t d = tmem_base + (uint32_t)(buf * W);
       // the accumulator is free once the drain has read the tile before last out of it
-      ok = mbar_wait_warp(bar(B_TEMPTY + buf), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
+      ok = mbar_wait_warp<PAIR>(bar(B_TEMPTY + buf), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
       if (!ok) break;
       tc_fence_after();
       LQ_TL(EV_M_ACC_FREE, 0);
@@ -390,7 +390,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (!ok) break;
         if (BRANCH_ACC) {
           // the drain has read the previous tile's branch accumulator (long ago: it does that under this tile's main loop)
-          ok = mbar_wait_warp(bar(B_BEMPTY), (tc & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
+          ok = mbar_wait_warp<PAIR>(bar(B_BEMPTY), (tc & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
           if (!ok) break;
         }
         tc_fence_after();
@@ -435,7 +435,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16);
     const int blocks = W >> 5;
     auto give_back = [&](uint32_t b) {                  // to the issuer, which sits in the pair's first CTA
-      if (PAIR) peer_arrive(peer_smem(b, 0));
+      if (PAIR) peer_arrive_tmem(peer_smem(b, 0));
       else mbar_arrive(b);
     };
     uint32_t tc = 0;

@@ -92,3 +92,35 @@ def test_static_calls_of_different_layers_share_the_scratch():
         torch.cuda.synchronize()
         B.lq_layer_free(h)
         assert rel_fro(y.cpu().numpy(), O.forward(X, layer)["Y"]) <= SINT4.TOL_F32 * (10 if branch == "w16a16" else 1)
+
+
+@pytest.mark.parametrize("main,branch,r", [("mxint4", "w8a8", 32), ("mxfp4", "mxfp8", 64)])
+def test_pairs_of_ctas_give_the_bits_of_single_ones_every_time(option, main, branch, r):
+    """Long K and several tiles per pair, so that stages keep changing hands between the two CTAs: the output is that of single
+    CTAs, call after call."""
+    import torch
+    from tests.helpers import import_oracle_layer, import_oracle_mxfp_layer
+
+    rng = np.random.default_rng(11)
+    M, K, N = 2100, 4096, 1160
+    layer = MXINT4._mx_layer(rng, K, N, r, branch) if main == "mxint4" else MXFP._layer(rng, K, N, r, branch)
+    h, _ = (import_oracle_layer if main == "mxint4" else import_oracle_mxfp_layer)(layer)
+    B.lq_layer_to_device(h, 0)
+    act = B.lq_act_create(h, M, 0)
+    x, st = torch.from_numpy(_x(rng, M, K)).cuda(), torch.cuda.current_stream().cuda_stream
+    B.lq_quantize_act(h, x.data_ptr(), M, act, st)
+
+    def forward():
+        y = torch.full((M, N), float("nan"), device="cuda")
+        B.lq_linear_forward(h, act, y.data_ptr(), B.OUT_F32, st)
+        return y
+
+    option("gemm_pair", 0, default=1)
+    alone = forward()
+    option("gemm_pair", 1, default=1)
+    pairs = [forward() for _ in range(20)]
+    torch.cuda.synchronize()
+    assert B.lq_get_device_status(0)[0] == 0
+    assert all(torch.equal(alone, y) for y in pairs)
+    B.lq_act_free(act)
+    B.lq_layer_free(h)
