@@ -129,6 +129,7 @@ __device__ __forceinline__ void grid_dependency_sync() {
 
 // ---- thread-block clusters: rendezvous, and barriers of a peer CTA ---------------------------
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();      // the barrier's aligned form wants the warp's lanes together, whatever branches lie behind them
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

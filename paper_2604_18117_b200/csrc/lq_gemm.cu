@@ -458,7 +458,6 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
   if constexpr (SPLIT) {
     // Every CTA of the cluster adds up a part of the items, in the order of the stages, and stores them.
-    __syncwarp();
     cluster_sync();
     if (drained) {
       const int at = (int)threadIdx.x - 32 * FIRST_DRAIN_WARP, mb = u_begin / p.units_n, nu = u_begin - mb * p.units_n, n = 16 / p.split;
