@@ -649,13 +649,16 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           // The quotient t / st as in branch_codes8.  A power of two keeps its steps in binary32's normal range; the quotient
           // stays what it is (what underflows is far below half a code).
           const float k = st < 1e-20f ? 0x1p64f : st > 1e20f ? 0x1p-64f : 1.f, ns = -st * k, y = __frcp_rn(st * k);
+          const bool coarse = st < 0x1p-126f;                  // a subnormal scale: amax / st may be up to half again as large as qm
 #pragma unroll 1
           for (int c = 0; c < p.rn; c += 16) {
             scaled(c);
             uint32_t w[4];
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              const float x = t[j] * k, q0 = __fmul_rn(x, y), q = __fmaf_rn(__fmaf_rn(q0, ns, x), y, q0);
+              const float x = t[j] * k, q0 = __fmul_rn(x, y);
+              float q = __fmaf_rn(__fmaf_rn(q0, ns, x), y, q0);
+              if (coarse) q = fminf(fmaxf(q, -p.qm), p.qm);
               const uint32_t code = __float_as_uint(__fadd_rn(q, MAGIC)) & 0xFFu;
               w[j >> 2] = (j & 3) == 0 ? code : w[j >> 2] | (code << (8 * (j & 3)));
             }

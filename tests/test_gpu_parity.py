@@ -286,3 +286,24 @@ def test_overlapped_launches_keep_stream_order():
         B.lq_set_option("overlap", 1)
         B.lq_act_free(a1); B.lq_act_free(a2)
         B.lq_layer_free(h1); B.lq_layer_free(h2)
+
+
+@pytest.mark.parametrize("branch", ["w8a8", "w6a6", "w4a8"])
+@pytest.mark.parametrize("mx", [False, True])
+def test_intermediate_under_a_subnormal_scale_is_clamped(branch, mx):
+    """First-factor scales so small that the intermediate's own scale max|t| / qmax rounds to a subnormal number: t / scale reaches
+    up to one and a half times qmax (here 1.496 steps of 2^-149 rounded to one), and the codes are clamped there."""
+    from tests.test_gpu_mxint4 import _mx_layer
+    rng = np.random.default_rng(6)
+    M, K, N, r = 9, 64, 8, 8
+    layer = _mx_layer(rng, K, N, r, branch) if mx else _random_layer(rng, K, N, r, branch)
+    qm = O.qmax(O.BRANCH_BITS[branch][1])
+    X = np.zeros((M, K), np.float16)
+    X[:, 0], X[:, 1] = qm, np.arange(M) * qm // (2 * M)
+    X[:, 2] = 1
+    layer["L1q"][:] = 0
+    layer["L1q"][:2], layer["L1q"][2, 1] = 1, 1               # t = qm + 0 .. qm / 2 (+ 1) steps
+    layer["sL1"][:] = np.float32(2.0 ** -149)
+    ref = O.forward(X, layer)
+    assert np.abs(ref["tq"]).max() == qm and np.unique(ref["sT"]).tolist() == [2.0 ** -149]
+    assert_codes_equal(gpu_forward(layer, X)[1], ref, branch)
