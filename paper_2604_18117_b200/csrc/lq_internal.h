@@ -137,7 +137,7 @@ struct lq_act {
   int8_t* d_qb;                // [Mpad][Kpad] branch activation codes
   float* d_sXb;                // [Mpad]
   uint8_t* d_tq;               // [Mpad][LQ_RCONT] bytes: int8 codes (or halves) of T, r contiguous
-  float* d_sT;                 // [Mpad] (ones for W16A16); SINT4: in lq_row_slot order
+  float* d_sT;                 // [Mpad] (ones for W16A16); SINT4: in lq_row_slot order; MXFP: the quantizer's bits of near blocks
   void* d_Xstage;              // lazily allocated staging for lq_linear_forward_host
   void* d_Ystage;
   size_t ystage_bytes;

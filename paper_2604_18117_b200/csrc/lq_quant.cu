@@ -72,6 +72,7 @@ struct QuantParams : QuantCut {
   float* sXb;           // [Mpad]
   const float* sL1;     // [LQ_MAX_RANK]
   const uint8_t* l1c;   // MXFP: the first factor's elements, [rn][Kpad] (the MMA reads them through tmL1)
+  uint32_t* near;       // MXFP: [Mpad], bit b: block b of the row's intermediate is near a tie
   const uint8_t* sfl1;  // MX branches: E8M0 bytes of the first factor's block scales, [Kpad/128][512]
   uint8_t* sft;         // MX branches: E8M0 bytes of the rank-r intermediate's block scales, [Mpad/128][512 or 1024]
   uint8_t* tq;          // [Mpad][tq_stride]
@@ -82,7 +83,7 @@ struct QuantParams : QuantCut {
   int nacc, sets;       // accumulators a tile's stages alternate over (floating-point branches: shorter chains of fp32 sums),
                         // sets of them (2: the next tile's MMAs run under a4)
   int tmem_cols;        // power of two
-  float dev;            // MXFP: how far a sum of the tensor core may be from the one in defining order, over its block's maximum
+  float dev;            // MXFP: how far a sum of the tensor core is taken to be from the one in settle_tiles' order, over its block's maximum
   float qm;             // largest branch activation code
   int32_t* status;
 };
@@ -308,91 +309,133 @@ __device__ __forceinline__ uint2 branch_codes8(const uint4& v, float sb, float i
   return b;
 }
 
-// One element of T = deq(Q(X)) deq(Q2(L1)) with the sum in its defining order (whole warp; every lane gets it): a partial sum
-// of 32 products per block on mma.sync, fp32 additions of the scaled partial sums in nine interleaved chains (box g of 64
-// values belongs to chain g mod 9, its second block first), the chains added in order.  The tensor core's own order differs
-// from it by less than 2^-22.2 of the block's maximum in 999 of 1000 elements at K = 1152, 2^-20.6 at K = 4608 with
-// one-sided inputs.  Eight blocks per MMA: row i of A and column i of B hold block i, so the products wanted are on the
-// diagonal.
-__device__ __forceinline__ void mma_e4m3_16832(float (&c)[4], uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k32.row.col.f32.e4m3.e4m3.f32 {%0,%1,%2,%3}, {%4,%5,%6,%5}, {%7,%8}, {%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(0), "r"(a2), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ uint2 ld_volatile_v2(const uint8_t* p) {
-  uint2 v;
-  asm volatile("ld.volatile.global.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
-  return v;
-}
-// The partial sums of one element, scaled, into `part`: warp w of the block takes blocks 8 w .. 8 w + 7 and so on.
-__device__ __noinline__ void canonical_parts(const uint8_t* qx, const uint8_t* sfx, const uint8_t* l1, const uint8_t* sfl, int blocks, float* part) {
-  const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-#pragma unroll 1
-  for (int b0 = 8 * (int)(threadIdx.x >> 5); b0 < blocks; b0 += 8 * (NTHREADS / 32)) {
-    const int b = b0 + gid;                                      // (blocks is a multiple of 4)
-    uint2 a = make_uint2(0, 0), w = a;
-    float s = 0.f;
-    if (b < blocks) {
-      a = ld_volatile_v2(qx + 32 * b + 8 * tig);
-      w = *reinterpret_cast<const uint2*>(l1 + 32 * b + 8 * tig);
-      const uint32_t ea = *reinterpret_cast<const volatile uint8_t*>(sfx + (b >> 2) * 512 + (b & 3)), el = sfl[(b >> 2) * 512 + (b & 3)];
-      s = __uint_as_float(ea << 23) * __uint_as_float(el << 23);
-    }
-    float c[4] = {0.f, 0.f, 0.f, 0.f};
-    mma_e4m3_16832(c, a.x, a.y, w.x, w.y);
-    if (tig == (gid >> 1) && b < blocks) part[b] = ((gid & 1) ? c[1] : c[0]) * s;
-  }
-}
-// Their sum (whole warp; every lane gets it).
-__device__ __forceinline__ float canonical_sum(const float* part, int blocks) {
-  const int lane = threadIdx.x & 31;
-  float chain = 0.f, v = 0.f;
-  if (lane < 9)
-    for (int b = 2 * lane; b < blocks; b += 18) chain = __fadd_rn(part[b], __fadd_rn(part[b + 1], chain));
-  for (int c = 0; c < 9; ++c) v += __shfl_sync(0xffffffffu, chain, c);
-  return v;
-}
-// Whether an element may change its code within the deviation: elements of the largest binade (steps of 32 in e4m3, 1/2 in
-// e2m3) whose distance to the nearest code is within the deviation of half a step.
+// Near ties of the MXFP intermediate T = deq(Q(X)) deq(Q2(L1)).  Floating-point elements round in steps of up to a fourteenth of the
+// block's maximum, so a sum that lands on the other side of a tie shows in Y.  Blocks of T that are too close to call on the
+// tensor core's sum - the block's exponent, an element of the largest binade - are settled on the sum in one fixed order
+// instead: a partial sum of 32 products per block of K on mma.sync, fp32 additions of the scaled partial sums in nine
+// interleaved chains (box g of 64 values belongs to chain g mod 9, its second block first), the chains added in order.  Which blocks
+// are settled is decided for each by itself, so a row's codes do not depend on the rows around it.
+// "Too close" is measured, not a bound: the tensor core's sum differs from the other by less than 2^-22.2 of the block's
+// maximum in 999 of 1000 elements at K = 1152, 2^-20.6 at K = 4608 with one-sided inputs.  An element beyond that keeps the code of the
+// tensor core's sum, which is as near to the exact one.
 template <bool SIX>
 struct TieTest {
   float k, limit;
   __device__ __forceinline__ TieTest(float inv, float dev) : k(inv * (SIX ? 2.f : 0.03125f)), limit(0.5f - dev * k) {}
+  // elements of the largest binade (steps of 32 in e4m3, 1/2 in e2m3) whose distance to the nearest code is within the deviation of
+  // half a step
   __device__ __forceinline__ bool operator()(float x) const {
     const float u = fabsf(x) * k;
     return u > 7.5f && fabsf(u - __fadd_rn(__fadd_rn(u, MAGIC), -MAGIC)) > limit;
   }
 };
-// Elements `what.z` of block `what.y` of row `what.x` of the rank-r intermediate again, from the sums in defining order (all
-// threads of the CTA); with all of them asked for, the block's exponent too.
+__device__ __forceinline__ void mma_e4m3_16832(float (&c)[4], const uint2& a0, const uint2& a1, const uint2& b) {
+  asm("mma.sync.aligned.m16n8k32.row.col.f32.e4m3.e4m3.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0.x), "r"(a1.x), "r"(a0.y), "r"(a1.y), "r"(b.x), "r"(b.y));
+}
+__device__ __forceinline__ float e8m0(uint32_t byte) { return __uint_as_float((byte & 0xFFu) << 23); }
+__device__ __forceinline__ size_t sf_row(int m) { return 16 * (m & 31) + 4 * ((m & 127) >> 5); }
+
+// All near blocks of the CTA's tiles (all threads of the CTA, after its last tile), in rounds of up to sixteen rows for each block of
+// the rank: warp 9 h + c sums chain c of sixteen of the 32 elements, then a warp adds a row's chains and quantizes them as a4 does.
+// (What this kernel has written itself is read through the L2.)  What bounds it is the tag stage of the L1: eight rows or columns
+// to a load.  A launch of 8192 rows and rank 64 meets a near block every few times and is 1.6 us longer then at K = 1152, 4.7 us at
+// K = 4608 (9.8 and 26.8 us without); with one value per row, where most blocks are exact ties, 6.9 and 18 us, against 740
+// when element after element was summed by the whole CTA.
+constexpr int SETTLE_ROWS = 16;
+struct SettleList {
+  int met[2];            // whether a4's two warps met near blocks
+  int n[4];              // rows of the round, by block
+  int row[4][SETTLE_ROWS];
+};
+static_assert(sizeof(SettleList) <= LQ_MAX_RANK * 4, "the list lies where other branches keep sL1");
 template <bool SIX>
-__device__ __noinline__ void settle_block(const QuantParams& p, int4 what, float* part) {
-  const int lane = threadIdx.x & 31, m = what.x, b = what.y;
-  const uint32_t which = (uint32_t)what.z;
-  const size_t sf_row = 16 * (m & 31) + 4 * ((m & 127) >> 5);
-  float mine = 0.f;
-  for (uint32_t todo = which; todo != 0; todo &= todo - 1) {
-    const int j = __ffs(todo) - 1, col = 32 * b + j;
-    if (col >= p.r) break;
-    canonical_parts(p.qx8 + (size_t)m * p.Kpad, p.sfa + (size_t)(m >> 7) * (p.Kpad >> 7) * 512 + sf_row, p.l1c + (size_t)col * p.Kpad,
-                    p.sfl1 + 16 * (col & 31) + 4 * (col >> 5), p.Kpad / 32, part);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      const float v = canonical_sum(part, p.Kpad / 32);
-      if (lane == j) mine = v;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x >= 32) return;
-  int e = what.w;
-  if (which == 0xFFFFFFFFu) {
-    float amax = fabsf(mine);
+__device__ __forceinline__ void settle_tiles(const QuantParams& p, float* part, SettleList& list) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3, TR = 8 * p.groups;
+  const int half = warp / SETTLE_CHAINS, chain = warp - half * SETTLE_CHAINS, boxes = p.Kpad / 64;
+  const int rows = (p.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x * TR;   // of this CTA
+#pragma unroll 1
+  for (int r0 = 0; r0 < rows; r0 += NTHREADS) {
+    const int at_row = r0 + (int)threadIdx.x, m = ((int)blockIdx.x + at_row / TR * (int)gridDim.x) * TR + at_row % TR;
+    uint32_t pending = at_row < rows && m < p.M ? __ldcg(p.near + m) : 0;
+#pragma unroll 1
+    while (__syncthreads_or(pending != 0)) {
+      if (threadIdx.x < 4) list.n[threadIdx.x] = 0;
+      __syncthreads();
+      for (uint32_t todo = pending; todo != 0; todo &= todo - 1) {
+        const int b = __ffs(todo) - 1, n = atomicAdd(&list.n[b], 1);
+        if (n < SETTLE_ROWS) { list.row[b][n] = m; pending &= ~(1u << b); }
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int b = 0; 32 * b < p.rn; ++b) {
+        const int n = min(list.n[b], SETTLE_ROWS);
+        if (n == 0) continue;
+        if (half < 2) {
+          // rows gid and gid + 8 of the round (beyond its end: the first one again), columns 16 half + 8 t + gid of the block
+          const int m0 = list.row[b][gid < n ? gid : 0], m1 = list.row[b][gid + 8 < n ? gid + 8 : 0];
+          const uint8_t* x0 = p.qx8 + (size_t)m0 * p.Kpad + 8 * tig;
+          const uint8_t* x1 = p.qx8 + (size_t)m1 * p.Kpad + 8 * tig;
+          const uint8_t* s0 = p.sfa + (size_t)(m0 >> 7) * (p.Kpad >> 7) * 512 + sf_row(m0);
+          const uint8_t* s1 = p.sfa + (size_t)(m1 >> 7) * (p.Kpad >> 7) * 512 + sf_row(m1);
+          const int c0 = 32 * b + 16 * half;                     // (the rank rounded up to 16 may end in the middle of the block)
+          const bool live = c0 < p.rn;
+          const uint8_t* w = p.l1c + (size_t)(c0 + gid) * p.Kpad + 8 * tig;
+          const uint8_t* sl = p.sfl1 + sf_row(c0 + 2 * tig);
+          float acc[2][4] = {};
+          if (live) {
+#pragma unroll 1
+            for (int g = chain; g < boxes; g += SETTLE_CHAINS) {
+              const int at = (g >> 1) * 512 + 2 * (g & 1);       // the box's two scale bytes
+              const uint32_t e0 = __ldcg(reinterpret_cast<const uint16_t*>(s0 + at)), e1 = n > 8 ? __ldcg(reinterpret_cast<const uint16_t*>(s1 + at)) : 0;
+              uint2 a0[2], a1[2], wt[2][2];
+              uint32_t el[2][2];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    e = mxfp_exponent<SIX>(amax);
-    if (lane == 0) p.sft[(size_t)(m >> 7) * 512 + sf_row + b] = (uint8_t)(e + 127);
+              for (int h = 0; h < 2; ++h) {
+                a0[h] = __ldcg(reinterpret_cast<const uint2*>(x0 + 64 * g + 32 * h));
+                a1[h] = n > 8 ? __ldcg(reinterpret_cast<const uint2*>(x1 + 64 * g + 32 * h)) : make_uint2(0, 0);
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                  wt[t][h] = __ldg(reinterpret_cast<const uint2*>(w + (size_t)(8 * t) * p.Kpad + 64 * g + 32 * h));
+                  el[t][h] = __ldg(reinterpret_cast<const uint16_t*>(sl + at + 128 * t + 16 * h));   // columns 2 tig + h
+                }
+              }
+#pragma unroll
+              for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int h = 1; h >= 0; --h) {
+                  float f[4] = {0.f, 0.f, 0.f, 0.f};
+                  mma_e4m3_16832(f, a0[h], a1[h], wt[t][h]);
+                  const float r0 = e8m0(e0 >> (8 * h)), r1 = e8m0(e1 >> (8 * h)), ca = e8m0(el[t][0] >> (8 * h)), cb = e8m0(el[t][1] >> (8 * h));
+                  acc[t][0] = __fadd_rn(f[0] * (r0 * ca), acc[t][0]); acc[t][1] = __fadd_rn(f[1] * (r0 * cb), acc[t][1]);
+                  acc[t][2] = __fadd_rn(f[2] * (r1 * ca), acc[t][2]); acc[t][3] = __fadd_rn(f[3] * (r1 * cb), acc[t][3]);
+                }
+            }
+          }
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            float* to = part + (chain * SETTLE_ROWS + gid) * 32 + 16 * half + 8 * t + 2 * tig;
+            to[0] = acc[t][0]; to[1] = acc[t][1];
+            to[8 * 32] = acc[t][2]; to[8 * 32 + 1] = acc[t][3];
+          }
+        }
+        __syncthreads();
+        if (warp < n) {
+          const int mr = list.row[b][warp];
+          float v = 0.f;
+          for (int c = 0; c < SETTLE_CHAINS; ++c) v = __fadd_rn(v, part[(c * SETTLE_ROWS + warp) * 32 + lane]);
+          float amax = fabsf(v);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+          const int e = mxfp_exponent<SIX>(amax);
+          const float inv = e == -127 ? 0.f : pow2f_n(-e);
+          p.tq[(size_t)mr * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, v * inv);
+          if (lane == 0) p.sft[(size_t)(mr >> 7) * 512 + sf_row(mr) + b] = (uint8_t)(e + 127);
+        }
+        __syncthreads();
+      }
+    }
   }
-  const float inv = e == -127 ? 0.f : pow2f_n(-e);
-  if ((which >> lane) & 1) p.tq[(size_t)m * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, mine * inv);
 }
 
 // A stage's MMAs under one election, predicated instead of branched around (inside an `if` of one lane every operand is moved to
@@ -604,8 +647,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0) + ((uint32_t)(32 * warp) << 16);
     const int nacc = min(p.nacc, p.nst), row = 32 * warp + lane;
     uint32_t tc = 0;
-    int4* unsettled = reinterpret_cast<int4*>(smem + sm.off_l1) + warp * MAX_UNSETTLED;   // MXFP: (row, block, elements, exponent) from 1 on
-    if (BR == BR_MXFP && lane == 0) unsettled[0].x = 0;
+    SettleList* const settle = reinterpret_cast<SettleList*>(smem + sm.off_l1);
+    if (BR == BR_MXFP && lane == 0) settle->met[warp] = 0;
     __syncwarp();
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++tc) {
       const int m = tile * TR + row;
@@ -686,6 +729,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           // 2 + c of one chunk; a container per plane: 128 bytes on, slot c of the next chunk
           const bool sep = p.tq_stride != LQ_RCONT;
           uint8_t* const sf = p.sft + (size_t)(m >> 7) * (!FPB && sep ? 1024 : 512) + 16 * (m & 31) + 4 * ((m & 127) >> 5);
+          [[maybe_unused]] uint32_t near = 0;                    // MXFP: the row's blocks to be settled at the end
 #pragma unroll 1
           for (int b = 0; 32 * b < p.rn; ++b) {
             float t2[16];
@@ -727,25 +771,17 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
               if (!FPB) sf[(sep ? 512 : 2) + b] = (uint8_t)(e + 127);
             }
             if constexpr (FPB) {
-              // Floating-point elements round in steps of up to a fourteenth of the block's maximum, so a sum that lands on the
-              // other side of a tie can show in Y.  What is too close to call on the tensor core's sum - the block's
-              // exponent, an element of the largest binade - is decided on the sum in its defining order, at the end by
-              // all warps (a launch of 8192 rows and rank 64 meets one every few times; settled on the spot, the code around
-              // it cost 3-6 us in every launch, and one warp alone takes 4-12 us for an element).  Where the list is full the tensor core's sum stands.
               const float dev = amax * p.dev;
               const TieTest<SIX> tie(inv, dev);
-              const bool edge = ((__float_as_uint(amax + dev) ^ __float_as_uint(amax - dev)) >> 23) != 0;
-              bool close = edge;
+              bool close = ((__float_as_uint(amax + dev) ^ __float_as_uint(amax - dev)) >> 23) != 0;
 #pragma unroll
               for (int j = 0; j < 16; ++j) close |= tie(t[j]) | tie(t2[j]);
-              if (valid && close) {
-                uint32_t which = 0;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) which |= (tie(t[j]) ? 1u << j : 0u) | (tie(t2[j]) ? 0x10000u << j : 0u);
-                const int n = atomicAdd(&unsettled[0].x, 1) + 1;
-                if (n < MAX_UNSETTLED) unsettled[n] = make_int4(m, b, edge ? -1 : (int)which, e);
-              }
+              near |= (uint32_t)close << b;
             }
+          }
+          if (FPB && valid) {
+            p.near[m] = near;
+            if (near != 0) settle->met[warp] = 1;
           }
         }
       }
@@ -947,12 +983,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   if constexpr (BR == BR_MXFP) {
-    for (int w = 0; w < 2; ++w) {
-      const int4* unsettled = reinterpret_cast<const int4*>(smem + sm.off_l1) + w * MAX_UNSETTLED;
-      const int n = min(unsettled[0].x, MAX_UNSETTLED - 1);
-      for (int i = 1; i <= n; ++i)
-        settle_block<MAIN == MAIN_MXFP6>(p, unsettled[i], reinterpret_cast<float*>(smem + sm.off_l1 + 2 * MAX_UNSETTLED * 16));
-    }
+    SettleList& list = *reinterpret_cast<SettleList*>(smem + sm.off_l1);
+    if ((list.met[0] | list.met[1]) != 0 && !*abort_flag) settle_tiles<MAIN == MAIN_MXFP6>(p, reinterpret_cast<float*>(smem), list);
   }
   if (BR != BR_NONE && warp == 2) {
     tc_fence_after();
@@ -979,7 +1011,7 @@ cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, i
   p.nacc = BR == BR_INT ? 1 : BR == BR_F16 || cols <= 32 ? 4 : cols <= 64 ? 2 : 1;
   p.tmem_cols = 32;
   while (p.tmem_cols < p.sets * p.nacc * cols + extra) p.tmem_cols *= 2;
-  // what the chains of fp32 sums and the bits of the products make of the deviation from the defining order
+  // what the chains of fp32 sums and the bits of the products make of that deviation
   p.dev *= (0.3f + (float)p.K / (1000.f * p.nacc)) * 0x1p-22f;
   CUtensorMap tmX;
   if (lq_make_tmap_bytes(&tmX, const_cast<void*>(X), (uint64_t)p.M, (uint64_t)p.K * 2, (uint32_t)(8 * p.groups)) != LQ_OK)
@@ -1000,7 +1032,7 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   p.qx8 = A->d_qx8; p.sx = A->d_sx; p.sfa = A->d_sfa;
   p.qb = g_lq_store_qb ? A->d_qb : nullptr;
   p.sXb = A->d_sXb; p.sL1 = L->d_sL1; p.l1c = L->d_L1c; p.sfl1 = L->d_sfl1;
-  p.sft = A->d_sft; p.tq = A->d_tq; p.sT = A->d_sT;
+  p.sft = A->d_sft; p.tq = A->d_tq; p.sT = A->d_sT; p.near = reinterpret_cast<uint32_t*>(A->d_sT);   // (an MXFP row has no scale of its own)
   p.r = L->r; p.rn = lq_l1_rows(L);
   p.bplanes = lq_l1_planes(L);
   p.tq_stride = A->tq_stride;

@@ -11,7 +11,8 @@ namespace lqcut {
 
 constexpr int QWARPS = 15;             // quantizer warps (at most; teams of RG * SX): 20 warps are the most that leave 96 registers each
 constexpr int MAX_SLOTS = 4;           // chunk slots of the branch's operands
-constexpr int MAX_UNSETTLED = 32;      // list of a4's rows to look at again, per warp
+constexpr int SETTLE_CHAINS = 9;       // MXFP: chains of the sum that near ties are settled on
+constexpr int SETTLE_BYTES = SETTLE_CHAINS * 16 * 32 * 4;   // their partial sums for sixteen rows, where the rings were
 constexpr int MAX_XSLOTS = 12;         // chunk slots of X
 enum { BR_NONE = 0, BR_INT = 1, BR_F16 = 2, BR_MXFP = 3, BR_MXINT = 4 };
 
@@ -45,7 +46,8 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
   s.slot = (s.slot + 1023) & ~1023;
   s.off_slots = xslots * s.xslot;
   s.off_l1 = s.off_slots + (br == BR_NONE ? 0 : slots) * s.slot;
-  s.off_max = s.off_l1 + (br == BR_MXFP ? 2 * MAX_UNSETTLED * 16 + 256 * 4 : LQ_MAX_RANK * 4);   // sL1; MXFP: list, scratch
+  if (br == BR_MXFP && s.off_l1 < SETTLE_BYTES) s.off_l1 = SETTLE_BYTES;
+  s.off_max = s.off_l1 + LQ_MAX_RANK * 4;       // sL1; MXFP: settle_tiles' list
   // row maxima of three tiles in rotation, row scales of two
   s.off_sb = s.off_max + 3 * 64 * 4;
   s.off_bar = s.off_sb + 2 * 64 * 4;

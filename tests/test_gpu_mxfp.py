@@ -152,3 +152,46 @@ def test_mxfp_host_entry_point_pipelines_row_chunks():
     finally:
         B.lq_act_free(act)
         B.lq_layer_free(h)
+
+
+@pytest.mark.parametrize("act", ["e4m3", "e2m3"])
+def test_near_ties_of_the_intermediate_do_not_depend_on_the_rows_around(act):
+    """Rows whose intermediate is a tie of its element format (272 between 256 and 288, of which 256 is even) plus sixteen terms of a
+    sixteenth of an ulp, which one order of the sum adds up and another rounds away.  Whatever the order, all rows must get the same
+    code: in tiles that are full of such rows, among other rows, and in the row chunks of the host entry point."""
+    import torch
+    from tests.helpers import import_oracle_mxfp_layer
+    rng = np.random.default_rng(12)
+    M, K, N, r = 8192, 1152, 8, 64
+    layer = _layer(rng, K, N, r, "mxfp8", bias=False)
+    layer["act"] = act
+    L1, row = np.zeros((K, r)), np.zeros(K)
+    row[32:34], L1[32:34, 0] = (16, 1), 16
+    tiny = [64 * box + 32 * h for box in (2, 3, 6, 7, 10, 11, 14, 15) for h in (0, 1)]
+    row[tiny], L1[tiny, 0] = 2.0 ** -10, 2.0 ** -9
+    L1[:, 40] = -L1[:, 0]
+    layer["L1v"], layer["e1"] = F.q_columns(L1, "e4m3")
+    assert np.array_equal(F.deq_columns(layer["L1v"], layer["e1"]), L1)
+    X = np.where(rng.random((M, 1)) < 0.9, row, rng.standard_normal((M, K))).astype(np.float16)
+    X[:256] = row
+    same = (X == row.astype(np.float16)).all(axis=1)
+    h, cfg = import_oracle_mxfp_layer(layer)
+    B.lq_layer_to_device(h, 0)
+    a = B.lq_act_create(h, M, 0)
+    st = torch.cuda.current_stream().cuda_stream
+    try:
+        x = torch.from_numpy(X).cuda()
+        B.lq_quantize_act(h, x.data_ptr(), M, a, st)
+        ex = B.lq_act_export(a, M, cfg, st)
+        tq, sT = ex["tq"].copy(), ex["sT"].copy()
+        t = F.deq_mxfp(B.e4m3_decode(tq), sT.astype(np.int16))
+        assert np.unique(t[same][:, 0]).tolist() == [256.0] and np.unique(t[same][:, 40]).tolist() == [-256.0]
+        assert (t[same][:, [j for j in range(r) if j not in (0, 40)]] == 0).all()
+        Xp, Yp = torch.from_numpy(X).pin_memory(), torch.empty(M, N, dtype=torch.float16).pin_memory()
+        B.lq_linear_forward_host(h, a, Xp.data_ptr(), M, Yp.data_ptr(), B.OUT_F16, st)
+        ex = B.lq_act_export(a, M, cfg, st)
+        assert np.array_equal(ex["tq"], tq) and np.array_equal(ex["sT"], sT)
+        assert B.lq_get_device_status(0)[0] == 0
+    finally:
+        B.lq_act_free(a)
+        B.lq_layer_free(h)
