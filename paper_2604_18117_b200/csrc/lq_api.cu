@@ -380,6 +380,19 @@ static lq_status make_tmap_packed(CUtensorMap* tm, void* base, uint64_t rows, ui
   return r == CUDA_SUCCESS ? LQ_OK : LQ_ERR_CUDA;
 }
 
+// Scale bytes: rows of 512, box of `box_rows` whole rows, as they lie in memory.
+static lq_status make_tmap_scales(CUtensorMap* tm, void* base, uint64_t rows, uint32_t box_rows) {
+  encode_tiled_fn fn = get_encode_fn();
+  if (!fn) return LQ_ERR_CUDA;
+  cuuint64_t dims[2] = {128, rows};
+  cuuint64_t strides[1] = {512};
+  cuuint32_t box[2] = {128, box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? LQ_OK : LQ_ERR_CUDA;
+}
+
 // ---- device status word ------------------------------------------------------------------
 static int32_t* g_status[64] = {nullptr};
 static std::mutex g_status_mu;
@@ -603,6 +616,9 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
     if ((st = lq_make_tmap_bytes(&L->tmL2w[wi], L->d_L2c, Npad, LQ_RCONT, width)) != LQ_OK) return st;
     if ((st = make_tmap_packed(&L->tmBp[wi], L->d_Wq8, Npad, Kpad, lq_mx_weight_bits(L), width / 2)) != LQ_OK) return st;
     if ((st = lq_make_tmap_bytes(&L->tmL2p[wi], L->d_L2c, Npad, LQ_RCONT, width / 2)) != LQ_OK) return st;
+    const uint32_t chunks = (uint32_t)lq_ceil_div((int)width, 128), tile_rows = (uint32_t)lq_ceil_div(N, (int)width) * chunks;
+    if ((st = make_tmap_scales(&L->tmSfb[wi], L->d_sfbw[wi], (uint64_t)(Kpad / 128) * tile_rows, chunks)) != LQ_OK) return st;
+    if (L->d_sfl2w[wi] && (st = make_tmap_scales(&L->tmSfl2[wi], L->d_sfl2w[wi], tile_rows, chunks)) != LQ_OK) return st;
   }
   if (r > 0 && (st = lq_make_tmap_bytes(&L->tmL1, L->d_L1c, (uint64_t)rn * lq_l1_planes(L), (uint64_t)Kpad * (L->f16_branch ? 2 : 1),
                                         (uint32_t)(rn * lq_l1_planes(L)))) != LQ_OK) return st;
@@ -655,6 +671,8 @@ extern "C" lq_status lq_act_create(const lq_layer* L, int32_t M_max, int device,
   lq_status st;
   if ((st = lq_make_tmap_bytes(&A->tmA, A->d_qx8, Mp, Kx, LQ_BM)) != LQ_OK) { lq_act_free(A); return st; }
   if ((st = lq_make_tmap_bytes(&A->tmT, A->d_tq, Mp, (uint64_t)A->tq_stride, LQ_BM)) != LQ_OK) { lq_act_free(A); return st; }
+  if (A->mx && (st = make_tmap_scales(&A->tmSfa, A->d_sfa, (Mp / 128) * (Kx / 128), 1)) != LQ_OK) { lq_act_free(A); return st; }
+  if (A->d_sft && (st = make_tmap_scales(&A->tmSft, A->d_sft, (Mp / 128) * (A->tq_stride / LQ_RCONT), 1)) != LQ_OK) { lq_act_free(A); return st; }
   if (cudaDeviceSynchronize() != cudaSuccess) { lq_act_free(A); return LQ_ERR_CUDA; }
   *out = A;
   return LQ_OK;
@@ -744,7 +762,7 @@ static lq_status forward_host(const lq_layer* L, lq_act* A, const void* Xh, int3
     CUDA_OK(cudaStreamWaitEvent(st, A->ev_x[c], 0));
     // a view of the activation record that starts at row m0 (m0 is a multiple of the row tile)
     lq_act V = *A;
-    V.M = Mc; V.M_max = Mc; V.M_call = M;
+    V.M = Mc; V.M_max = Mc; V.M_call = M; V.block0 = m0 / 128;
     V.d_qx8 = A->d_qx8 + (size_t)m0 * A->Kpad * A->planes;
     V.d_qb = A->d_qb + (size_t)m0 * A->Kpad;
     V.d_sx = A->d_sx + m0;                                     // [Gpad][Mpad]: the row stride stays Mpad

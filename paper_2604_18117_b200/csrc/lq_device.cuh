@@ -26,14 +26,14 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// CLUSTER: the barrier's arrivals come from another CTA of the cluster, too, and what they hand over is acquired at that scope.
+// CLUSTER: arrivals come from another CTA of the cluster, too, and hand over tensor memory (peer_arrive).
 template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   if constexpr (CLUSTER)
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.b32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(bar), "r"(parity)
@@ -138,15 +138,10 @@ __device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
   return a;
 }
-// Arrival on a barrier of another CTA.  What was observed to be in this CTA's shared memory before it is visible to the waiter
-// (which acquires at cluster scope).
+// Arrival on a barrier of another CTA that hands over tensor memory and nothing else: tcgen05.wait::ld has emptied it, and the tcgen05
+// fences on both sides order the accesses to it, so arrival and wait may be relaxed.  (As a release the arrival waits for the
+// thread's earlier stores - a drain warp's stores of Y - to be performed, over a thousand clocks.)
 __device__ __forceinline__ void peer_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// The same where no memory is handed over but tensor memory that tcgen05.wait::ld has emptied, ordered by the tcgen05 fences on
-// both sides: relaxed.  As a release the arrival waits for the thread's earlier stores - a drain warp's stores of Y - to be
-// performed, over a thousand clocks.
-__device__ __forceinline__ void peer_arrive_tmem(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ float4 lds_peer_v4(uint32_t a) {
@@ -177,11 +172,15 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 // ---- bulk copies (TMA): every copy goes to the issuing CTA only -----------------------------
+#define LQ_TMA_2D "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+// of a pair of CTAs: the barrier may be the other CTA's
+#define LQ_TMA_2D_PAIR "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+template <bool PAIR = false>
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
+  if constexpr (PAIR)
+    asm volatile(LQ_TMA_2D_PAIR " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar) : "memory");
+  else
+    asm volatile(LQ_TMA_2D " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),

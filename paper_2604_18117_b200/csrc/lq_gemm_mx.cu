@@ -80,16 +80,15 @@ struct MxParams {
                           // both sides - the stage's four K blocks are (hi, 0), (hi, 1), (lo, 0), (lo, 1) and every
                           // (plane of T, plane of L2) pair of the same rank block is one MMA.  3: the same codes with 4-bit
                           // factors (one plane) and rank up to 128: two stages like mode 1, one per plane of T
-  const uint8_t* sft;     // branch_mx: E8M0 bytes of T's block scales, [Mpad/128][512]
-  const uint8_t* sfl2;    // branch_mx: E8M0 bytes of L2's block scales, [tiles_n][sf_chunks][512]
   int tiles_m, tiles_n;
   int width, stages;      // W, operand ring depth
   int b_row;              // bytes of a weight row that a stage copies
   uint32_t b_format;      // format field of the weights in the instruction descriptor
   int b_wrap;             // Kpad / 128: stage s reads B (and its scales) at stage s mod b_wrap - the planes share the weights
-  const uint8_t* sfa;     // [Mpad/128][k_stages][512]
-  const uint8_t* sfb;     // [Kpad/128][tiles_n][sf_chunks][512]
+  // scale bytes, rows of 512: tmSfa [Mpad/128][k_stages], tmSfb [Kpad/128][tiles_n][sf_chunks]; branch_mx: tmSft [Mpad/128][1 or 2] (of T),
+  // tmSfl2 [tiles_n][sf_chunks] (of L2)
   int sf_chunks;          // ceil(W / 128)
+  int block0;             // first row block of the launch in tmSfa and tmSft
   const float* sT;        // [Mpad]
   const float* sL2;       // [Npad]
   const float* bias;      // [Npad]
@@ -144,36 +143,50 @@ __device__ __forceinline__ void issue_main_stage_pair(uint32_t d, uint64_t a, ui
       "r"(idesc), "r"(idesc | idesc_mx_ids(1)), "r"(idesc | idesc_mx_ids(2)), "r"(idesc | idesc_mx_ids(3)), "r"(empty), "h"((uint16_t)3)
       : "memory");
 }
-//   main stage of the producer: the weights' half (which announces the whole stage) and the activations' half
-__device__ __forceinline__ void load_weights_stage(uint32_t full, uint32_t tx, uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t sf_dst,
-                                                   const uint8_t* sf, uint32_t sf_bytes) {
-  asm volatile(
-      "{\n\t.reg .pred P;\n\t"
-      "elect.sync _|P, 0xffffffff;\n\t"
-      "@P mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
-      "@P cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%2], [%3, {%4, %5}], [%0];\n\t"
-      "@P cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%6], [%7], %8, [%0];\n\t}"
-      ::"r"(full), "r"(tx), "r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(sf_dst), "l"(reinterpret_cast<uint64_t>(sf)), "r"(sf_bytes)
-      : "memory");
+//   main stage of the producer: the weights' half, which announces the whole stage (tx bytes; 0: the pair's other CTA does) on
+//   `own`, and the activations' half.  Copies complete on `full`.
+#define LQ_LOAD_WEIGHTS(TMA)                                     \
+  "{\n\t.reg .pred P, Q;\n\t"                                    \
+  "elect.sync _|P, 0xffffffff;\n\t"                             \
+  "setp.ne.and.b32 Q, %1, 0, P;\n\t"                            \
+  "@Q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t" \
+  "@P " TMA " [%3], [%4, {%5, %6}], [%2];\n\t"                  \
+  "@P " TMA " [%7], [%8, {%9, %10}], [%2];\n\t}"
+template <bool PAIR>
+__device__ __forceinline__ void load_weights_stage(uint32_t own, uint32_t tx, uint32_t full, uint32_t dst, const CUtensorMap* tm, int x, int y,
+                                                   uint32_t sf_dst, const CUtensorMap* tm_sf, int sf_row) {
+  const uint64_t t = reinterpret_cast<uint64_t>(tm), ts = reinterpret_cast<uint64_t>(tm_sf);
+  if constexpr (PAIR)
+    asm volatile(LQ_LOAD_WEIGHTS(LQ_TMA_2D_PAIR) ::"r"(own), "r"(tx), "r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0), "r"(sf_row) : "memory");
+  else
+    asm volatile(LQ_LOAD_WEIGHTS(LQ_TMA_2D) ::"r"(own), "r"(tx), "r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0), "r"(sf_row) : "memory");
 }
-__device__ __forceinline__ void load_acts_stage(uint32_t full, uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t sf_dst, const uint8_t* sf) {
-  asm volatile(
-      "{\n\t.reg .pred P;\n\t"
-      "elect.sync _|P, 0xffffffff;\n\t"
-      "@P cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%1], [%2, {%3, %4}], [%0];\n\t"
-      "@P cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%5], [%6], %7, [%0];\n\t}"
-      ::"r"(full), "r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(sf_dst), "l"(reinterpret_cast<uint64_t>(sf)), "r"((uint32_t)SF_BYTES)
-      : "memory");
+#define LQ_LOAD_ACTS(TMA)                        \
+  "{\n\t.reg .pred P;\n\t"                       \
+  "elect.sync _|P, 0xffffffff;\n\t"             \
+  "@P " TMA " [%1], [%2, {%3, %4}], [%0];\n\t"  \
+  "@P " TMA " [%5], [%6, {%7, %8}], [%0];\n\t}"
+template <bool PAIR>
+__device__ __forceinline__ void load_acts_stage(uint32_t full, uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t sf_dst, const CUtensorMap* tm_sf,
+                                                int sf_row) {
+  const uint64_t t = reinterpret_cast<uint64_t>(tm), ts = reinterpret_cast<uint64_t>(tm_sf);
+  if constexpr (PAIR)
+    asm volatile(LQ_LOAD_ACTS(LQ_TMA_2D_PAIR) ::"r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0), "r"(sf_row) : "memory");
+  else
+    asm volatile(LQ_LOAD_ACTS(LQ_TMA_2D) ::"r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0), "r"(sf_row) : "memory");
 }
 
 // BRANCH_ACC: the layer has an integer branch with fp32 scales, whose product needs an accumulator of its own.  The
 // other instance (no branch, fp16 branch, MX branches) carries none of that code or its registers.
 // PAIR: two CTAs of a cluster work on 256 rows x W columns (cta_group::2): each stages its own 128 rows of A and half of the
-// tile's columns of B, and each SM's tensor core reads B from both.
+// tile's columns of B, and each SM's tensor core reads B from both.  Both CTAs' copies complete on the first one's barrier, whose
+// CTA issues the MMAs for both.
 template <bool BRANCH_ACC, bool PAIR>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
+                  const __grid_constant__ CUtensorMap tmSfa, const __grid_constant__ CUtensorMap tmSfb,
+                  const __grid_constant__ CUtensorMap tmSft, const __grid_constant__ CUtensorMap tmSfl2,
                   const __grid_constant__ MxParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -189,7 +202,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   uint8_t* bar_ptr = smem + off_bar;
   // barrier map (8 bytes each)
   constexpr int B_FULL = 0, B_EMPTY = MAX_STAGES, B_TFULL = 2 * MAX_STAGES, B_TEMPTY = B_TFULL + 2, B_RFULL = B_TEMPTY + 2,
-                B_REMPTY = B_RFULL + 2, B_BEMPTY = B_REMPTY + 2, B_PFULL = B_BEMPTY + 1, NBAR = B_PFULL + MAX_STAGES;
+                B_REMPTY = B_RFULL + 2, B_BEMPTY = B_REMPTY + 2, NBAR = B_BEMPTY + 1;
   auto bar = [&](int idx) { return sm_bar + 8u * (uint32_t)idx; };
   static_assert(NBAR * 8 + 16 <= SMEM_BAR_BYTES, "barrier area too small");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + NBAR * 8);
@@ -206,7 +219,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int w_end = (int)((work * (unit + 1)) / units);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NST; ++s) { mbar_init(bar(B_FULL + s), 1); mbar_init(bar(B_EMPTY + s), 1); mbar_init(bar(B_PFULL + s), 1); }
+    for (int s = 0; s < NST; ++s) { mbar_init(bar(B_FULL + s), 1); mbar_init(bar(B_EMPTY + s), 1); }
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar(B_TFULL + b), 1); mbar_init(bar(B_TEMPTY + b), CTAS * NUM_DRAIN_WARPS);
       mbar_init(bar(B_RFULL + b), 1); mbar_init(bar(B_REMPTY + b), NUM_DRAIN_WARPS);
@@ -239,16 +252,19 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     int st = 0, armed = 0;                             // ring slot; stages announced (up to the ring's depth)
     bool ok = true;
     const uint32_t sfb_bytes = (uint32_t)p.sf_chunks * SF_BYTES;
+    const uint32_t first_bar = PAIR ? peer_smem(sm_bar, 0) : sm_bar;   // where the pair's copies complete
+    auto full_bar = [&](int st) { return first_bar + 8u * (uint32_t)(B_FULL + st); };
+    const uint32_t arm = rank == 0 ? CTAS : 0;         // CTAs whose bytes this one announces
+    const int block_last = p.tiles_m - 1;
     auto load_b = [&](int st, int s, int nu) {         // the weights' half of main stage s; announces the whole stage
-      const uint32_t dst = sm_stage + st * stage_bytes + STAGE_A_BYTES, full = bar(B_FULL + st);
       const int sb = s >= p.b_wrap ? s - p.b_wrap : s; // the lo digits' plane runs over the same weights
-      load_weights_stage(full, STAGE_A_BYTES + (uint32_t)BW * p.b_row + SF_BYTES + sfb_bytes, dst, &tmB, sb * LQ_KSTAGE, nu * W + (int)rank * BW, sm_sf + st * STAGE_SF_BYTES + SF_BYTES,
-                         p.sfb + ((size_t)sb * p.tiles_n + nu) * sfb_bytes, sfb_bytes);
+      load_weights_stage<PAIR>(bar(B_FULL + st), arm * (STAGE_A_BYTES + (uint32_t)BW * p.b_row + SF_BYTES + sfb_bytes), full_bar(st),
+                               sm_stage + st * stage_bytes + STAGE_A_BYTES, &tmB, sb * LQ_KSTAGE, nu * W + (int)rank * BW,
+                               sm_sf + st * STAGE_SF_BYTES + SF_BYTES, &tmSfb, (sb * p.tiles_n + nu) * p.sf_chunks);
     };
     auto load_a = [&](int st, int s, int mb) {
-      const uint32_t full = bar(B_FULL + st);
-      load_acts_stage(full, sm_stage + st * stage_bytes, &tmA, s * LQ_KSTAGE, mb * LQ_BM, sm_sf + st * STAGE_SF_BYTES,
-                      p.sfa + ((size_t)min(mb, p.tiles_m - 1) * p.k_stages + s) * SF_BYTES);
+      load_acts_stage<PAIR>(full_bar(st), sm_stage + st * stage_bytes, &tmA, s * LQ_KSTAGE, mb * LQ_BM, sm_sf + st * STAGE_SF_BYTES, &tmSfa,
+                            (p.block0 + min(mb, block_last)) * p.k_stages + s);
     };
     auto advance = [&]() {
       ++armed;
@@ -262,7 +278,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     grid_dependency_wait();
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
       const int mp = w / p.tiles_n, nu = w - mp * p.tiles_n, mb = mp * CTAS + (int)rank;   // (a pair's second block may not exist)
-      const int m0 = mb * LQ_BM, n0 = nu * W, mc = min(mb, p.tiles_m - 1);
+      const int m0 = mb * LQ_BM, n0 = nu * W, mc = min(mb, block_last);
       for (int s = 0; s < p.k_stages; ++s) {
         const bool ahead = tc == 0 && s < early;
         if (!ahead) {
@@ -280,16 +296,15 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       for (int bs = 0; bs < nbst && ok; ++bs) {
         ok = mbar_wait_warp(bar(B_EMPTY + st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
         if (!ok) break;
-        const uint32_t a_dst = sm_stage + st * stage_bytes;
-        const uint32_t full = bar(B_FULL + st);
+        const uint32_t a_dst = sm_stage + st * stage_bytes, full = full_bar(st);
         if (elect_one()) {
-          mbar_expect_tx(full, stage_bytes + (p.branch_mx ? SF_BYTES + sfb_bytes : 0));
-          tma_load_2d(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
-          tma_load_2d(a_dst + STAGE_A_BYTES, &tmL2, 0, n0 + (int)rank * BW, full);
+          if (arm != 0) mbar_expect_tx(bar(B_FULL + st), arm * (stage_bytes + (p.branch_mx ? SF_BYTES + sfb_bytes : 0)));
+          tma_load_2d<PAIR>(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
+          tma_load_2d<PAIR>(a_dst + STAGE_A_BYTES, &tmL2, 0, n0 + (int)rank * BW, full);
           if (p.branch_mx) {   // the block scales of T (rows) and of L2 (columns) along the rank
             const uint32_t sf_dst = sm_sf + st * STAGE_SF_BYTES;
-            bulk_load(sf_dst, p.sft + ((size_t)mc * nbst + bs) * SF_BYTES, SF_BYTES, full);
-            bulk_load(sf_dst + SF_BYTES, p.sfl2 + (size_t)nu * sfb_bytes, sfb_bytes, full);
+            tma_load_2d<PAIR>(sf_dst, &tmSft, 0, (p.block0 + mc) * nbst + bs, full);
+            tma_load_2d<PAIR>(sf_dst + SF_BYTES, &tmSfl2, 0, nu * p.sf_chunks, full);
           }
         }
         __syncwarp();
@@ -313,7 +328,9 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     }
     if (!ok && lane == 0) {
       // aborting: give the copies already issued a bounded time to land before the CTA's shared memory goes away
-      for (int i = max(min(armed, NST), early); i > 0; --i) {
+      // (the pair's second CTA cannot see its own: a barrier of its that nothing completes gives them that time)
+      if (rank != 0) mbar_settle(bar(B_FULL), 0);
+      for (int i = rank != 0 ? 0 : max(min(armed, NST), early); i > 0; --i) {
         if (--st < 0) { st = NST - 1; par ^= 1; }
         mbar_settle(bar(B_FULL + st), par ^ 1);
       }
@@ -323,17 +340,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       }
     }
   } else if (warp == 1 && rank != 0) {
-    // ------------------------------------------------------------------ the pair's second CTA: tells the first which stages
-    // have landed here
-    const int total = (w_end - w_begin) * (p.k_stages + nbst);
-    int st = 0;
-    uint32_t par = 0;
-    for (int i = 0; i < total; ++i) {
-      if (!mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA)) break;
-      if (lane == 0) peer_arrive(peer_smem(bar(B_PFULL + st), 0));
-      __syncwarp();
-      if (++st == NST) { st = 0; par ^= 1; }
-    }
+    // the pair's first CTA issues for both
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     uint32_t tc = 0, par = 0;
@@ -359,10 +366,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       else tc_commit(b);
     };
     constexpr uint32_t ROWS256 = PAIR ? (uint32_t)(LQ_BM >> 4) << 24 : 0;    // added to a 128-row descriptor's M field: 256
-    auto stage_full = [&]() {
-      return mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA) &&
-             (!PAIR || mbar_wait_warp<PAIR>(bar(B_PFULL + st), par, abort_flag, p.status, LQ_STAGE_MMA));
-    };
+    auto stage_full = [&]() { return mbar_wait_warp(bar(B_FULL + st), par, abort_flag, p.status, LQ_STAGE_MMA); };
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
       const int buf = tc & 1;
       const uint32_t d = tmem_base + (uint32_t)(buf * W);
@@ -435,7 +439,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16);
     const int blocks = W >> 5;
     auto give_back = [&](uint32_t b) {                  // to the issuer, which sits in the pair's first CTA
-      if (PAIR) peer_arrive_tmem(peer_smem(b, 0));
+      if (PAIR) peer_arrive(peer_smem(b, 0));
       else mbar_arrive(b);
     };
     uint32_t tc = 0;
@@ -595,7 +599,7 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   p.width = LQ_MX_WIDTHS[wi]; p.stages = ring_stages(pair ? p.width / 2 : p.width); p.sf_chunks = lq_ceil_div(p.width, 128);
   p.tiles_n = lq_ceil_div(L->N, p.width);
   p.b_row = LQ_KSTAGE / 8 * lq_mx_weight_bits(L); p.b_format = L->mxfp ? IDESC_MX_B_E2M1 : IDESC_MX_B_E2M3;
-  p.sfa = A->d_sfa; p.sfb = L->d_sfbw[wi]; p.sft = A->d_sft; p.sfl2 = L->d_sfl2w[wi];
+  p.block0 = A->block0;
   p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
   p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
   const int c = pair ? 2 : 1;
@@ -606,6 +610,7 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
                      : (pair ? lq_gemm_mx_kernel<false, true> : lq_gemm_mx_kernel<false, false>);
   const CUtensorMap& tmB = pair ? L->tmBp[wi] : L->tmBw[wi];
   const CUtensorMap& tmL2 = pair ? L->tmL2p[wi] : L->tmL2w[wi];
-  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, (size_t)smem_bytes(p.width / c), st, A->tmA, tmB, A->tmT, tmL2, p);
+  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, (size_t)smem_bytes(p.width / c), st, A->tmA, tmB, A->tmT, tmL2,
+                                          A->tmSfa, L->tmSfb[wi], A->tmSft, L->tmSfl2[wi], p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -116,6 +116,7 @@ struct lq_layer {
   uint8_t* d_sfl2w[LQ_MX_NWIDTHS];  // MX branches: the same for L2's block scales along the rank, [tiles][ceil(width/128)][512]
   CUtensorMap tmBw[LQ_MX_NWIDTHS], tmL2w[LQ_MX_NWIDTHS];   // over d_Wq8 and d_L2c, box [width][128B], 128B swizzle
   CUtensorMap tmBp[LQ_MX_NWIDTHS], tmL2p[LQ_MX_NWIDTHS];   // the same with half the width, for a pair of CTAs
+  CUtensorMap tmSfb[LQ_MX_NWIDTHS], tmSfl2[LQ_MX_NWIDTHS]; // over d_sfbw and d_sfl2w, rows of 512 bytes, box [ceil(width/128)] rows
   CUtensorMap tmB;             // over d_Wq8, box [LQ_BN][128B], 128B swizzle
   CUtensorMap tmL1;            // over d_L1c, box [all rows][128B], 128B swizzle
   CUtensorMap tmL2;            // over d_L2c, box [LQ_BN][128B], 128B swizzle
@@ -146,6 +147,8 @@ struct lq_act {
   bool pipe_ready;
   CUtensorMap tmA;             // over d_qx8, box [LQ_BM][128B], 128B swizzle
   CUtensorMap tmT;             // over d_tq,  box [LQ_BM][128B], 128B swizzle
+  CUtensorMap tmSfa, tmSft;    // MX: over all of d_sfa and d_sft, one row of 512 bytes
+  int block0;                  // a view's first row / 128 (tmA and tmT begin there, tmSfa and tmSft at the record's first row)
 };
 
 // remembers the last failing CUDA runtime code (per host thread) for lq_last_cuda_error(); returns its argument
