@@ -1,5 +1,6 @@
 // Handles, import/export, device upload and the host-side plumbing of the C ABI.
 #include <cuda_fp16.h>
+#include <cuda_fp8.h>
 #include <math.h>
 #include <string.h>
 
@@ -160,6 +161,7 @@ lq_layer* lq_layer_new(const lq_config* cfg) {
   L->f16_branch = L->r > 0 && L->cfg.branch == LQ_BRANCH_W16A16;
   L->has_bias = false;
   L->device = -1;
+  L->l1_shift = 0;
   L->main_kind = g_lq_main_kind;
   L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1c = nullptr; L->d_sL1 = nullptr;
   L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfl1 = nullptr;
@@ -536,10 +538,30 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
           if (planes == 2) { lq_split_digits(lo, &hi, &lo); dst[plane] = lq_digit_e4m3(lo); lo = hi; }
           *dst = lq_digit_e4m3(lo);
         }
+      // The scales may be any power of two that fp32 has; E8M0 ends at 2^-127, and so do the tensor core's sums.  A factor with
+      // scales near that is carried 2^l1_shift larger, up to 2^80, where sums are still far from overflowing.
+      std::vector<int> e1((size_t)lq_ceil_div(K, 32) * r);
+      int lowest = 0, highest = -200;
       for (int b = 0; b < lq_ceil_div(K, 32); ++b)
         for (int j = 0; j < r; ++j) {
-          int e = 0;
+          int& e = e1[(size_t)b * r + j];
           pow2_exponent(L->s1b[(size_t)b * r + j], &e);
+          bool zero = true;
+          for (int k = 32 * b; k < std::min(K, 32 * b + 32); ++k)
+            zero &= L->a8 ? L->L1q[(size_t)k * r + j] == 0 : (L->L1e[(size_t)k * r + j] & 0x7F) == 0;
+          if (zero) { e = 0; continue; }                                // any scale does
+          lowest = std::min(lowest, e); highest = std::max(highest, e);
+        }
+      L->l1_shift = lowest >= -100 ? 0 : std::max(0, std::min(-100 - lowest, 80 - highest));
+      for (int b = 0; b < lq_ceil_div(K, 32); ++b)
+        for (int j = 0; j < r; ++j) {
+          int e = e1[(size_t)b * r + j] + L->l1_shift;
+          // (What is below even so stands beside scales 2^180 times as large: its elements are rounded to the lowest scale.)
+          for (; e < -126; ++e)
+            for (int k = 32 * b; k < std::min(K, 32 * b + 32); ++k) {
+              uint8_t& v = l1c[(size_t)j * Kpad + k];
+              v = __nv_cvt_float_to_fp8(0.5f * __half2float(__half(__nv_cvt_fp8_to_halfraw(v, __NV_E4M3))), __NV_SATFINITE, __NV_E4M3);
+            }
           sfl1[lq_sf_offset(j, b, Kpad)] = (uint8_t)(e + 127 + (planes == 2 ? 4 : 0));
           if (planes == 2) sfl1[lq_sf_offset(rn + j, b, Kpad)] = (uint8_t)(e + 127);
         }

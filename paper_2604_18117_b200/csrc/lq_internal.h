@@ -105,6 +105,7 @@ struct lq_layer {
   uint8_t* d_L1c;              // [planes * rn][Kpad] bytes (W16A16: [rn][Kpad] halves), K contiguous: first factor as the B operand of
                                // the down-projection; rn = lq_l1_rows; MXINT8 factors: the hi digits' rows, then the lo digits'
   uint8_t* d_sfl1;             // MX branches: E8M0 bytes of L1's block scales, [Kpad/128][512] in the tensor-memory layout (row = row of d_L1c)
+  int l1_shift;                // the scales in d_sfl1 are 2^l1_shift times the factor's; the quantizer takes that off the intermediate again
   float* d_sL1;                // [LQ_MAX_RANK]
   uint8_t* d_L2c;              // [Npad][LQ_RCONT] bytes: int8 codes (or up to 64 halves) of column n, r contiguous
   float* d_sL2;                // [Npad]  (ones for W16A16); d_L2c in d_Wq8's row order; SINT4: d_sL2 and d_bias in

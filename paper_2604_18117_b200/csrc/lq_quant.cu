@@ -43,6 +43,7 @@
 //             are scaled up (exactly) first, a rare branch.  MXFP8e4: products below 2^-14 may lose bits, far below half of e4m3's
 //             smallest step 2^-9.
 #include <cuda_fp16.h>
+#include <math.h>
 
 #include <algorithm>
 #include <type_traits>
@@ -84,6 +85,7 @@ struct QuantParams : QuantCut {
                         // sets of them (2: the next tile's MMAs run under a4)
   int tmem_cols;        // power of two
   float dev;            // MXFP: how far a sum of the tensor core is taken to be from the one in settle_tiles' order, over its block's maximum
+  float unit;           // MX branches: the intermediate over the tensor core's sums (a power of two, 1 but for tiny first factors)
   float qm;             // largest branch activation code
   int32_t* status;
 };
@@ -427,8 +429,8 @@ __device__ __forceinline__ void settle_tiles(const QuantParams& p, float* part, 
           float amax = fabsf(v);
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-          const int e = mxfp_exponent<SIX>(amax);
-          const float inv = e == -127 ? 0.f : pow2f_n(-e);
+          const int e = mxfp_exponent<SIX>(amax * p.unit);
+          const float inv = e == -127 ? 0.f : pow2f_n(-e) * p.unit;
           p.tq[(size_t)mr * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, v * inv);
           if (lane == 0) p.sft[(size_t)(mr >> 7) * 512 + sf_row(mr) + b] = (uint8_t)(e + 127);
         }
@@ -742,8 +744,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             float amax = 0.f;
 #pragma unroll
             for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fmaxf(fabsf(t[j]), fabsf(t2[j])));
-            const int e = FPB ? mxfp_exponent<SIX>(amax) : mxint8_exponent(amax);
-            const float inv = e == -127 ? 0.f : pow2f_n(-e);
+            const int e = FPB ? mxfp_exponent<SIX>(amax * p.unit) : mxint8_exponent(amax * p.unit);
+            const float inv = e == -127 ? 0.f : pow2f_n(-e) * p.unit;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               const float (&x)[16] = h ? t2 : t;
@@ -1037,6 +1039,7 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   p.bplanes = lq_l1_planes(L);
   p.tq_stride = A->tq_stride;
   p.dev = L->cfg.branch == LQ_BRANCH_MXFP8 ? 1.f : L->cfg.branch == LQ_BRANCH_MXFP6 ? 0.5f : 0.2f;
+  p.unit = ldexpf(1.f, -L->l1_shift);
   p.qm = abits > 0 ? (float)((1 << (abits - 1)) - 1) : 0.f;
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;

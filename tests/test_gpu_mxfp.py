@@ -195,3 +195,28 @@ def test_near_ties_of_the_intermediate_do_not_depend_on_the_rows_around(act):
     finally:
         B.lq_act_free(a)
         B.lq_layer_free(h)
+
+
+@pytest.mark.parametrize("act", ["e4m3", "e2m3"])
+def test_first_factor_scales_beyond_the_scale_bytes(act):
+    """First-factor block scales of 2^-131 and around, which fp32 has and a scale byte has not; the second factor's make up for it."""
+    rng = np.random.default_rng(13)
+    layer = _layer(rng, 1152, 136, 64, "mxfp8")
+    layer["act"] = act
+    layer["e1"], layer["e2"] = (layer["e1"] - 120).astype(np.int16), (layer["e2"] + 115).astype(np.int16)
+    assert layer["e1"].max() < -127 and layer["e2"].max() <= 127
+    _check(layer, (rng.standard_normal((70, 1152)) * 256).astype(np.float16))
+
+
+def test_first_factor_scales_that_span_all_of_fp32():
+    """One block of the first factor at 2^100, the others at 2^-149: their elements round to the lowest scale byte's; the intermediate of
+    rows that are zero in the first block is zero, as it is below the smallest value that its format has."""
+    rng = np.random.default_rng(14)
+    layer = _layer(rng, 128, 40, 32, "mxfp8")
+    layer["e1"][:] = -149
+    layer["e1"][0], layer["e2"] = 100, (layer["e2"] - 100).astype(np.int16)
+    X = rng.standard_normal((40, 128)).astype(np.float16)
+    X[20:] *= np.float16(0.01)
+    X[20:, :32] = 0
+    assert (F.forward(X, layer)["tq"][20:] == 0).all()
+    _check(layer, X)

@@ -179,3 +179,12 @@ def test_mxint8_edge_shapes(M, K, N, r, branch):
     rng = np.random.default_rng(M + K)
     X = (rng.standard_normal((M, K)) * rng.choice([0.01, 1.0, 30.0])).astype(np.float16)
     _check(_layer(rng, K, N, r, branch, bias=(N % 16 == 0)), X)
+
+
+def test_first_factor_scales_at_the_bottom_of_their_range():
+    """Block scales down to 2^-120 under small activations: the products lie below 2^-126, the intermediate does not."""
+    rng = np.random.default_rng(15)
+    layer = _layer(rng, 1152, 136, 64, "mxint8")
+    layer["e1"], layer["e2"] = (layer["e1"] - 109).astype(np.int16), (layer["e2"] + 109).astype(np.int16)
+    assert -120 <= layer["e1"].min() < -112 and layer["e2"].max() <= 120
+    _check(layer, (rng.standard_normal((70, 1152)) * 2.0 ** -9).astype(np.float16))
