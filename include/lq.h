@@ -277,7 +277,8 @@ lq_status lq_selftest_wait_timeout(int device, void* cuda_stream);
  *   "gemm_split"   1, 2, 4, 8: so many CTAs share a tile of the SINT4 GEMM where they fit; 0 (default): chosen by the launcher
  *   "gemm_pair"    1 (default): from 256 rows on, pairs of CTAs share an MX GEMM's tile; 0: never
  *   "quant_warps", "quant_ctas"   how the quantizer kernel is cut: row groups of 8 per tile (at most 8 count) and 128-value
- *                  stages of K per chunk; 0 = chosen by the library
+ *                  stages of K per chunk; 0 = chosen by the library.  What a launch cannot have (more than 15 groups times stages,
+ *                  more stages than K has) becomes the largest that it can, stages first
  *   "overlap"      1 (default): kernels are launched with programmatic stream serialization - a kernel's CTAs may take
  *                  their SMs and set up while the previous kernel on the stream drains, and wait (in the kernel) for
  *                  that kernel's completion before touching global memory; 0: plain launches

@@ -1004,7 +1004,7 @@ cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, i
     if (e != cudaSuccess) return e;
     attr_set[dev & 63] = true;
   }
-  if (!plan_cut(BR, p.M, p.nst, p.rn, p.bplanes, sms, g_lq_quant_warps, g_lq_quant_ctas, p)) return cudaErrorInvalidConfiguration;
+  if (!plan_cut_as_asked(BR, p.M, p.nst, p.rn, p.bplanes, sms, g_lq_quant_warps, g_lq_quant_ctas, p)) return cudaErrorInvalidConfiguration;
   // Floating-point branches: a tile's stages alternate over up to four accumulators, which are added in fp32 at the end
   // (each costs a4 a trip to tensor memory per 16 columns: not more than 128 columns of them).  Tensor memory holds two
   // such sets - one where every CTA has a single tile - and the scale bytes' columns.

@@ -72,7 +72,7 @@ inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int f
   const int walks = br == BR_INT ? 2 : 1, room = 227 * 1024 - 1024;
   double best = 1e30;
   for (int groups = 8; groups >= 1; --groups) {
-    if (force_groups > 0 && groups != std::min(8, force_groups)) continue;
+    if (force_groups > 0 && groups != force_groups) continue;
     for (int stages = 1; stages <= std::min(QWARPS / groups, nst); ++stages) {
       if (force_stages > 0 && stages != force_stages) continue;
       QuantCut c{};
@@ -105,6 +105,19 @@ inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int f
     }
   }
   return best < 1e30;
+}
+
+// The same under the options (0: free): what a launch cannot have - more warps than there are, more stages than K has, more shared
+// memory than there is - becomes the largest that it can, stages first.
+inline bool plan_cut_as_asked(int br, int M, int nst, int rn, int bplanes, int sms, int groups, int stages, QuantCut& out) {
+  for (int g = std::min(8, groups);; --g) {
+    for (int s = std::min(stages, nst);; --s) {
+      if (plan_cut(br, M, nst, rn, bplanes, sms, g, s, out)) return true;
+      if (s <= 1) break;
+    }
+    if (g <= 1) break;
+  }
+  return plan_cut(br, M, nst, rn, bplanes, sms, 0, 0, out);
 }
 
 }  // namespace lqcut

@@ -14,7 +14,7 @@ SOURCE = """
 #include "lq_quant_cut.h"
 extern "C" int cut(int br, int M, int nst, int rn, int planes, int groups, int stages, int* out) {
   lqcut::QuantCut c{};
-  if (!lqcut::plan_cut(br, M, nst, rn, planes, 148, groups, stages, c)) return 0;
+  if (!lqcut::plan_cut_as_asked(br, M, nst, rn, planes, 148, groups, stages, c)) return 0;
   const int v[] = {c.groups, c.stages, c.teams, c.ntiles, c.nchunks, c.slots, c.xslots, c.refetch, c.smem};
   for (int i = 0; i < 9; ++i) out[i] = v[i];
   return 1;
@@ -121,4 +121,20 @@ def test_every_layer_has_a_cut_and_no_phase_is_mistaken_for_another(cut):
         assert c["smem"] <= 227 * 1024 and c["teams"] * c["groups"] * c["stages"] <= 15 and c["xslots"] <= 12 and c["slots"] <= 4
         seen.setdefault((br, c["teams"], c["nchunks"], c["slots"], c["xslots"], c["refetch"]), c)
     wrong = [(key, m) for key, c in seen.items() if (m := _mistaken(key[0], c)) is not None]
+    assert not wrong, wrong[:5]
+
+
+def test_every_value_of_the_options_gives_a_cut(cut):
+    """What lq_set_option takes for "quant_warps" and "quant_ctas" never refuses a launch; a cut that a launch can have is the one asked
+    for, and none mistakes a phase."""
+    seen = {}
+    for (br, rn, planes), M, nst in itertools.product(_layers(), (1, 300, 8192), (1, 3, 9, 44)):
+        for groups, stages in itertools.product(range(10), range(5)):
+            c = cut(br, M, nst, rn, planes, groups, stages)
+            assert c is not None and c["smem"] <= 227 * 1024, (br, rn, planes, M, nst, groups, stages)
+            g = min(groups, 8)
+            if br == NONE and g * stages <= 15 and stages <= nst:
+                assert (g or c["groups"], stages or c["stages"]) == (c["groups"], c["stages"])
+            seen.setdefault((br, c["teams"], c["nchunks"], c["slots"], c["xslots"], c["refetch"]), c)
+    wrong = [(key, m) for key, c in seen.items() if (m := _mistaken(key[0], c, tiles=2)) is not None]
     assert not wrong, wrong[:5]
