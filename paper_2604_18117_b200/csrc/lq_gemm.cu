@@ -38,6 +38,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "lq_device.cuh"
@@ -545,6 +546,11 @@ lq_status lq_gemm_prepare(int device) {
   for (auto* kernel : {lq_gemm_kernel<BRANCH_NONE, false>, lq_gemm_kernel<BRANCH_I8, false>, lq_gemm_kernel<BRANCH_F16, false>,
                        lq_gemm_kernel<BRANCH_NONE, true>, lq_gemm_kernel<BRANCH_I8, true>, lq_gemm_kernel<BRANCH_F16, true>})
     if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return LQ_ERR_CUDA;
+  // once per device: launches of other threads read g_clusters without the lock, each after its own layer's upload came through here
+  static std::mutex mu;
+  static bool done[64] = {false};
+  std::lock_guard<std::mutex> lk(mu);
+  if (done[device & 63]) return LQ_OK;
   for (int i = 0; i < 3; ++i) {
     cudaLaunchConfig_t lc = {};
     cudaLaunchAttribute at[1];
@@ -554,6 +560,7 @@ lq_status lq_gemm_prepare(int device) {
     if (lq_note_cuda(cudaOccupancyMaxActiveClusters(&g_clusters[device & 63][i], lq_gemm_kernel<BRANCH_I8, true>, &lc)) != cudaSuccess)
       return LQ_ERR_CUDA;
   }
+  done[device & 63] = true;
   return LQ_OK;
 }
 

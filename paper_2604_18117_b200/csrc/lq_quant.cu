@@ -46,6 +46,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "lq_device.cuh"
@@ -996,7 +997,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 
 template <int MAIN, int BR>
 cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, int sms, cudaStream_t st) {
-  static bool attr_set[64] = {false};
+  static std::atomic<bool> attr_set[64];   // (set by several threads at once it does no harm)
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_set[dev & 63]) {

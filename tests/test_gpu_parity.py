@@ -307,3 +307,43 @@ def test_intermediate_under_a_subnormal_scale_is_clamped(branch, mx):
     ref = O.forward(X, layer)
     assert np.abs(ref["tq"]).max() == qm and np.unique(ref["sT"]).tolist() == [2.0 ** -149]
     assert_codes_equal(gpu_forward(layer, X)[1], ref, branch)
+
+
+def test_layers_uploaded_and_run_from_several_threads():
+    """Distinct handles from distinct threads, uploads among launches: each thread's outputs are those of the same calls made alone."""
+    import threading
+    import torch
+    from tests.helpers import import_oracle_layer
+    rng = np.random.default_rng(21)
+    jobs = [(_random_layer(rng, K, N, 16, "w8a8"), rng.standard_normal((M, K)).astype(np.float16))
+            for M, K, N in ((3, 1152, 136), (128, 2048, 264), (300, 512, 72), (1, 4096, 1160))]
+
+    def run(layer, X, out):
+        torch.cuda.set_device(0)
+        stream = torch.cuda.Stream()
+        for _ in range(10):
+            h, _cfg = import_oracle_layer(layer)
+            B.lq_layer_to_device(h, 0)
+            act = B.lq_act_create(h, X.shape[0], 0)
+            with torch.cuda.stream(stream):
+                x = torch.from_numpy(X).cuda()
+                y = torch.empty(X.shape[0], layer["N"], device="cuda")
+                B.lq_quantize_act(h, x.data_ptr(), X.shape[0], act, stream.cuda_stream)
+                B.lq_linear_forward(h, act, y.data_ptr(), B.OUT_F32, stream.cuda_stream)
+                stream.synchronize()
+            out.append(y.cpu().numpy())
+            B.lq_act_free(act)
+            B.lq_layer_free(h)
+
+    alone = [[] for _ in jobs]
+    for job, out in zip(jobs, alone):
+        run(*job, out)
+    together = [[] for _ in jobs]
+    threads = [threading.Thread(target=run, args=(*job, out)) for job, out in zip(jobs, together)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for a, b in zip(alone, together):
+        assert len(a) == len(b) == 10
+        assert all(np.array_equal(a[0], y) for y in a + b)
