@@ -190,6 +190,9 @@ lq_status lq_quantize_act(const lq_layer* layer, const void* X_f16_dev, int32_t 
  * epilogue only adds the branch and the bias.
  *   act    result of lq_quantize_act for this layer
  *   Y_dev  [M][N] row-major, half or float per `dtype`, device, 16-byte aligned
+ * A row's codes and scales depend on that row alone.  So does its Y for the MX formats; for SINT4 the fp32 sum over
+ * the groups may be cut in two to eight parts where M is small, so Y of the same row may differ by rounding (some 1e-7
+ * of the sum of the terms' magnitudes) between calls of different M - not between the row chunks of one host call.
  * Asynchronous on `cuda_stream`. */
 lq_status lq_linear_forward(const lq_layer* layer, const lq_act* act, void* Y_dev,
                             lq_out_dtype dtype, void* cuda_stream);
@@ -236,9 +239,10 @@ lq_status lq_linear_forward_host_async(const lq_layer* layer, lq_act* act, const
  * (8 MiB holds e.g. M = 256 at any supported K, or M = 1024 at K = 2240).
  * The first call on each device looks up the array's device address (one-time set-up, done
  * with that device current); make that first call before starting any stream capture.
- * All calls share the one array, which keeps the previous call's contents: each call first
- * clears the part it uses (on `cuda_stream`), and two calls that overlap on the GPU - other
- * streams, other threads - race on it; serialise them.  Asynchronous on `cuda_stream`. */
+ * All calls share the one array, which keeps the previous call's contents: a call writes all of
+ * the record that it reads, so nothing is cleared in between.  Two calls that overlap on the
+ * GPU - other streams, other threads - race on the array; serialise them.  Asynchronous on
+ * `cuda_stream`. */
 #define LQ_STATIC_SCRATCH_BYTES (8u << 20)
 lq_status lq_linear_forward_static(const lq_layer* layer, const void* X_f16_dev, int32_t M, void* Y_dev,
                                    lq_out_dtype dtype, void* cuda_stream);
