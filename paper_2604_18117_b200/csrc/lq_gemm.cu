@@ -339,8 +339,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     Frag va[4], vb[4];                                  // two groups: one being consumed, one being fetched
     auto pair_at = [&](uint32_t i) { return tlane + (i & (NPAIR - 1)) * (2 * TCOLS); };
     // Requests stage i's first group once its pair is complete (its scale vectors landed before its MMAs were issued).  The
-    // request is made whatever the wait says, and even where no stage is left (it reads some accumulator, nothing looks at
-    // it): a conditional one would have the compiler keep the fragments twice.
+    // request is made whatever the wait says, and even where no stage is left (it reads some accumulator, nothing looks at it).
     auto open_stage = [&](uint32_t i, bool exists) {
       if (exists) ok = mbar_wait_inline(bar_tfull(i & (NPAIR - 1)), (i / NPAIR) & 1, abort_flag, p.status, LQ_STAGE_DRAIN) && ok;
       tc_fence_after();

@@ -97,9 +97,9 @@ struct MxParams {
   int32_t* status;
 };
 
-// A stage's instructions under one election, predicated instead of branched around: the control flow of the issuing warps
-// stays uniform and their addresses and descriptors in uniform registers.  (Inside an `if` of one lane every operand
-// is moved there instruction by instruction: 320-370 clocks for the MMA warp's stage and 270 for the producer's.)
+// A stage's instructions under one election, predicated instead of branched around: the control flow of the issuing warps stays
+// uniform.  (With an `if` of one lane around them, stamps gave 320-370 clocks for the MMA warp's stage and 270 for the producer's;
+// the MMAs of a stage take 2 W.)
 //   main stage of the MMA warp: scale bytes to tensor memory, four K = 32 MMAs, the stage's return
 __device__ __forceinline__ void issue_main_stage_one(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint64_t sfa, uint64_t sfb, uint32_t two,
                                                  uint32_t accumulate, uint32_t empty) {
@@ -237,8 +237,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   else __syncthreads();
   tc_fence_after();
   grid_launch_dependents();
-  // All 512 columns are this CTA's, so they start at 0: a constant, where a value read back would have to be moved into
-  // uniform registers for every instruction that names a column.
+  // All 512 columns are this CTA's, so they start at 0.
   constexpr uint32_t tmem_base = 0;
 
   LQ_TL_DECL((blockIdx.x == 0 && lane == 0)

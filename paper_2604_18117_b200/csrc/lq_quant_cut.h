@@ -58,7 +58,8 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 }
 
 // Cost model in rounds, a round being one chunk for every team: a CTA's tiles times (its rounds,
-// twice where a tile is walked twice, plus what starting and finishing a tile costs).
+// twice where a tile is walked twice, plus what starting and finishing a tile costs).  It prices rounds only: not the second stream of X
+// where an integer branch's tile is larger than the ring (140 MB read for 75 at M = 8192, K = 4608), nor what overlaps between tiles.
 //
 // Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
 // one: the chunk that was in the slot before has to be known to have landed (X) or to have been multiplied (operands).
