@@ -164,7 +164,7 @@ lq_layer* lq_layer_new(const lq_config* cfg) {
   L->l1_shift = 0;
   L->main_kind = g_lq_main_kind;
   L->d_Wq8 = nullptr; L->d_sw = nullptr; L->d_L1c = nullptr; L->d_sL1 = nullptr;
-  L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfl1 = nullptr;
+  L->d_L2c = nullptr; L->d_sL2 = nullptr; L->d_bias = nullptr; L->d_sfl1 = nullptr; L->d_maps = nullptr;
   for (int i = 0; i < LQ_MX_NWIDTHS; ++i) L->d_sfbw[i] = L->d_sfl2w[i] = nullptr;
   return L;
 }
@@ -437,8 +437,8 @@ static void layer_free_device(lq_layer* L) {
   if (L->device < 0) return;
   cudaSetDevice(L->device);
   cudaFree(L->d_Wq8); cudaFree(L->d_sw); cudaFree(L->d_L1c); cudaFree(L->d_sL1);
-  cudaFree(L->d_L2c); cudaFree(L->d_sL2); cudaFree(L->d_bias); cudaFree(L->d_sfl1);
-  L->d_sfl1 = nullptr;
+  cudaFree(L->d_L2c); cudaFree(L->d_sL2); cudaFree(L->d_bias); cudaFree(L->d_sfl1); cudaFree(L->d_maps);
+  L->d_sfl1 = nullptr; L->d_maps = nullptr;
   for (int i = 0; i < LQ_MX_NWIDTHS; ++i) {
     cudaFree(L->d_sfbw[i]); cudaFree(L->d_sfl2w[i]);
     L->d_sfbw[i] = L->d_sfl2w[i] = nullptr;
@@ -631,16 +631,20 @@ extern "C" lq_status lq_layer_to_device(lq_layer* L, int device) {
     if ((st = upload(&L->d_L2c, l2c)) != LQ_OK) return st;
   } catch (const std::bad_alloc&) { return LQ_ERR_ALLOC; }
   if (!L->mx && (st = lq_make_tmap_bytes(&L->tmB, L->d_Wq8, Npad, Kpad, LQ_BN)) != LQ_OK) return st;
-  for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
-    if (!L->d_sfbw[wi]) continue;
-    const uint32_t width = (uint32_t)LQ_MX_WIDTHS[wi];
-    if ((st = make_tmap_packed(&L->tmBw[wi], L->d_Wq8, Npad, Kpad, lq_mx_weight_bits(L), width)) != LQ_OK) return st;
-    if ((st = lq_make_tmap_bytes(&L->tmL2w[wi], L->d_L2c, Npad, LQ_RCONT, width)) != LQ_OK) return st;
-    if ((st = make_tmap_packed(&L->tmBp[wi], L->d_Wq8, Npad, Kpad, lq_mx_weight_bits(L), width / 2)) != LQ_OK) return st;
-    if ((st = lq_make_tmap_bytes(&L->tmL2p[wi], L->d_L2c, Npad, LQ_RCONT, width / 2)) != LQ_OK) return st;
-    const uint32_t chunks = (uint32_t)lq_ceil_div((int)width, 128), tile_rows = (uint32_t)lq_ceil_div(N, (int)width) * chunks;
-    if ((st = make_tmap_scales(&L->tmSfb[wi], L->d_sfbw[wi], (uint64_t)(Kpad / 128) * tile_rows, chunks)) != LQ_OK) return st;
-    if (L->d_sfl2w[wi] && (st = make_tmap_scales(&L->tmSfl2[wi], L->d_sfl2w[wi], tile_rows, chunks)) != LQ_OK) return st;
+  if (L->mx) {
+    std::vector<LqMxMaps> maps(2 * LQ_MX_NWIDTHS);
+    for (int wi = 0; wi < LQ_MX_NWIDTHS; ++wi) {
+      if (!L->d_sfbw[wi]) continue;
+      const uint32_t width = (uint32_t)LQ_MX_WIDTHS[wi], chunks = (width + 127) / 128, tile_rows = (uint32_t)lq_ceil_div(N, (int)width) * chunks;
+      for (uint32_t c = 1; c <= 2; ++c) {
+        LqMxMaps& m = maps[2 * wi + c - 1];
+        if ((st = make_tmap_packed(&m.b, L->d_Wq8, Npad, Kpad, lq_mx_weight_bits(L), width / c)) != LQ_OK) return st;
+        if ((st = lq_make_tmap_bytes(&m.l2, L->d_L2c, Npad, LQ_RCONT, width / c)) != LQ_OK) return st;
+        if ((st = make_tmap_scales(&m.sfb, L->d_sfbw[wi], (uint64_t)(Kpad / 128) * tile_rows, chunks)) != LQ_OK) return st;
+        if (L->d_sfl2w[wi] && (st = make_tmap_scales(&m.sfl2, L->d_sfl2w[wi], tile_rows, chunks)) != LQ_OK) return st;
+      }
+    }
+    if ((st = upload(&L->d_maps, maps)) != LQ_OK) return st;
   }
   if (r > 0 && (st = lq_make_tmap_bytes(&L->tmL1, L->d_L1c, (uint64_t)rn * lq_l1_planes(L), (uint64_t)Kpad * (L->f16_branch ? 2 : 1),
                                         (uint32_t)(rn * lq_l1_planes(L)))) != LQ_OK) return st;

@@ -85,8 +85,8 @@ struct MxParams {
   int b_row;              // bytes of a weight row that a stage copies
   uint32_t b_format;      // format field of the weights in the instruction descriptor
   int b_wrap;             // Kpad / 128: stage s reads B (and its scales) at stage s mod b_wrap - the planes share the weights
-  // scale bytes, rows of 512: tmSfa [Mpad/128][k_stages], tmSfb [Kpad/128][tiles_n][sf_chunks]; branch_mx: tmSft [Mpad/128][1 or 2] (of T),
-  // tmSfl2 [tiles_n][sf_chunks] (of L2)
+  const LqMxMaps* maps;   // of the layer, for this width; its scale bytes are rows of 512: sfb [Kpad/128][tiles_n][sf_chunks], sfl2 (branch_mx)
+                          // [tiles_n][sf_chunks].  The activations': tmSfa [Mpad/128][k_stages], tmSft (branch_mx) [Mpad/128][1 or 2]
   int sf_chunks;          // ceil(W / 128)
   int block0;             // first row block of the launch in tmSfa and tmSft
   const float* sT;        // [Mpad]
@@ -183,10 +183,8 @@ __device__ __forceinline__ void load_acts_stage(uint32_t full, uint32_t dst, con
 // CTA issues the MMAs for both.
 template <bool BRANCH_ACC, bool PAIR>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
-lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                  const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
-                  const __grid_constant__ CUtensorMap tmSfa, const __grid_constant__ CUtensorMap tmSfb,
-                  const __grid_constant__ CUtensorMap tmSft, const __grid_constant__ CUtensorMap tmSfl2,
+lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmT,
+                  const __grid_constant__ CUtensorMap tmSfa, const __grid_constant__ CUtensorMap tmSft,
                   const __grid_constant__ MxParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -258,8 +256,8 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     auto load_b = [&](int st, int s, int nu) {         // the weights' half of main stage s; announces the whole stage
       const int sb = s >= p.b_wrap ? s - p.b_wrap : s; // the lo digits' plane runs over the same weights
       load_weights_stage<PAIR>(bar(B_FULL + st), arm * (STAGE_A_BYTES + (uint32_t)BW * p.b_row + SF_BYTES + sfb_bytes), full_bar(st),
-                               sm_stage + st * stage_bytes + STAGE_A_BYTES, &tmB, sb * LQ_KSTAGE, nu * W + (int)rank * BW,
-                               sm_sf + st * STAGE_SF_BYTES + SF_BYTES, &tmSfb, (sb * p.tiles_n + nu) * p.sf_chunks);
+                               sm_stage + st * stage_bytes + STAGE_A_BYTES, &p.maps->b, sb * LQ_KSTAGE, nu * W + (int)rank * BW,
+                               sm_sf + st * STAGE_SF_BYTES + SF_BYTES, &p.maps->sfb, (sb * p.tiles_n + nu) * p.sf_chunks);
     };
     auto load_a = [&](int st, int s, int mb) {
       load_acts_stage<PAIR>(full_bar(st), sm_stage + st * stage_bytes, &tmA, s * LQ_KSTAGE, mb * LQ_BM, sm_sf + st * STAGE_SF_BYTES, &tmSfa,
@@ -299,11 +297,11 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (elect_one()) {
           if (arm != 0) mbar_expect_tx(bar(B_FULL + st), arm * (stage_bytes + (p.branch_mx ? SF_BYTES + sfb_bytes : 0)));
           tma_load_2d<PAIR>(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
-          tma_load_2d<PAIR>(a_dst + STAGE_A_BYTES, &tmL2, 0, n0 + (int)rank * BW, full);
+          tma_load_2d<PAIR>(a_dst + STAGE_A_BYTES, &p.maps->l2, 0, n0 + (int)rank * BW, full);
           if (p.branch_mx) {   // the block scales of T (rows) and of L2 (columns) along the rank
             const uint32_t sf_dst = sm_sf + st * STAGE_SF_BYTES;
             tma_load_2d<PAIR>(sf_dst, &tmSft, 0, (p.block0 + mc) * nbst + bs, full);
-            tma_load_2d<PAIR>(sf_dst + SF_BYTES, &tmSfl2, 0, nu * p.sf_chunks, full);
+            tma_load_2d<PAIR>(sf_dst + SF_BYTES, &p.maps->sfl2, 0, nu * p.sf_chunks, full);
           }
         }
         __syncwarp();
@@ -607,9 +605,7 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   const bool acc = p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx;
   auto* kernel = acc ? (pair ? lq_gemm_mx_kernel<true, true> : lq_gemm_mx_kernel<true, false>)
                      : (pair ? lq_gemm_mx_kernel<false, true> : lq_gemm_mx_kernel<false, false>);
-  const CUtensorMap& tmB = pair ? L->tmBp[wi] : L->tmBw[wi];
-  const CUtensorMap& tmL2 = pair ? L->tmL2p[wi] : L->tmL2w[wi];
-  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, (size_t)smem_bytes(p.width / c), st, A->tmA, tmB, A->tmT, tmL2,
-                                          A->tmSfa, L->tmSfb[wi], A->tmSft, L->tmSfl2[wi], p);
+  p.maps = L->d_maps + 2 * wi + c - 1;
+  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, (size_t)smem_bytes(p.width / c), st, A->tmA, A->tmT, A->tmSfa, A->tmSft, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }
