@@ -140,7 +140,7 @@ struct lq_act {
   int M_call;                  // rows of the caller's call (more than M in a chunk of one): what the order of a sum may depend on
   uint8_t* d_qx8;              // [Mpad][Kpad] operand bytes of the 4-bit codes (A operand, K-major)
   float* d_sx;                 // [Gpad][Mpad] fp32 images of the fp16 scales, in lq_row_slot order
-  int8_t* d_qb;                // [Mpad][Kpad] branch activation codes
+  int8_t* d_qb;                // [Mpad][Kpad] branch activation codes; MXFP: the quantizer's near elements
   float* d_sXb;                // [Mpad]
   uint8_t* d_tq;               // [Mpad][LQ_RCONT] bytes: int8 codes (or halves) of T, r contiguous
   float* d_sT;                 // [Mpad] (ones for W16A16); SINT4: in lq_row_slot order; MXFP: the quantizer's bits of near blocks

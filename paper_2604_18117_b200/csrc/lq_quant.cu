@@ -75,6 +75,7 @@ struct QuantParams : QuantCut {
   const float* sL1;     // [LQ_MAX_RANK]
   const uint8_t* l1c;   // MXFP: the first factor's elements, [rn][Kpad] (the MMA reads them through tmL1)
   uint32_t* near;       // MXFP: [Mpad], bit b: block b of the row's intermediate is near a tie
+  uint32_t* near_which; // MXFP: [Mpad][4], where so: its elements
   const uint8_t* sfl1;  // MX branches: E8M0 bytes of the first factor's block scales, [Kpad/128][512]
   uint8_t* sft;         // MX branches: E8M0 bytes of the rank-r intermediate's block scales, [Mpad/128][512 or 1024]
   uint8_t* tq;          // [Mpad][tq_stride]
@@ -316,8 +317,8 @@ __device__ __forceinline__ uint2 branch_codes8(const uint4& v, float sb, float i
 // block's maximum, so a sum that lands on the other side of a tie shows in Y.  Blocks of T that are too close to call on the
 // tensor core's sum - the block's exponent, an element of the largest binade - are settled on the sum in one fixed order
 // instead: a partial sum of 32 products per block of K on mma.sync, fp32 additions of the scaled partial sums in nine
-// interleaved chains (box g of 64 values belongs to chain g mod 9, its second block first), the chains added in order.  Which blocks
-// are settled is decided for each by itself, so a row's codes do not depend on the rows around it.
+// interleaved chains (box g of 64 values belongs to chain g mod 9, its second block first), the chains added in order.  What
+// is settled is decided for each element by itself, so a row's codes do not depend on the rows around it.
 // "Too close" is measured, not a bound: the tensor core's sum differs from the other by less than 2^-22.2 of the block's
 // maximum in 999 of 1000 elements at K = 1152, 2^-20.6 at K = 4608 with one-sided inputs.  An element beyond that keeps the code of the
 // tensor core's sum, which is as near to the exact one.
@@ -339,19 +340,78 @@ __device__ __forceinline__ void mma_e4m3_16832(float (&c)[4], const uint2& a0, c
 __device__ __forceinline__ float e8m0(uint32_t byte) { return __uint_as_float((byte & 0xFFu) << 23); }
 __device__ __forceinline__ size_t sf_row(int m) { return 16 * (m & 31) + 4 * ((m & 127) >> 5); }
 
-// All near blocks of the CTA's tiles (all threads of the CTA, after its last tile), in rounds of up to sixteen rows for each block of
-// the rank: warp 9 h + c sums chain c of sixteen of the 32 elements, then a warp adds a row's chains and quantizes them as a4 does.
-// (What this kernel has written itself is read through the L2.)  What bounds it is the tag stage of the L1: eight rows or columns
-// to a load.  A launch of 8192 rows and rank 64 meets a near block every few times and is 1.6 us longer then at K = 1152, 4.7 us at
-// K = 4608 (9.8 and 26.8 us without); with one value per row, where most blocks are exact ties, 6.9 and 18 us, against 740
-// when element after element was summed by the whole CTA.
-constexpr int SETTLE_ROWS = 16;
+// Settled are the elements that are near a tie, or with the exponent in doubt all of the block's: a few of a CTA one after the other,
+// more by tiles.  Both sum in the same order, so which of the two it is shows in the time only.  A launch of 8192 rows and rank 64
+// meets an element every few times at K = 1152 and most times at K = 4608; us at K = 4608 without / with one: 27.0 / 26.7 - it is gone
+// in the launch's end - against 31.8 by tiles.  An element takes about 0.4 us, a round by tiles 1.6 us at K = 1152 and 4.7 us at K =
+// 4608, hence the line between them.  One value per row, where most blocks are exact ties: 18.6 and 48 us by tiles, 610 and
+// 815 element by element.
+constexpr int SETTLE_ROWS = 16, SETTLE_ENTRIES = 18;
+__device__ __forceinline__ int settle_few(int K) { return 2 + K / 512; }   // 18 at most: never all of a block's 32
 struct SettleList {
-  int met[2];            // whether a4's two warps met near blocks
-  int n[4];              // rows of the round, by block
-  int row[4][SETTLE_ROWS];
+  int entries, elements;           // near blocks and elements that the CTA met
+  union {
+    int4 entry[SETTLE_ENTRIES];    // (row, block, elements, exponent)
+    struct {
+      int n[4];                    // rows of a round, by block
+      int row[4][SETTLE_ROWS];
+    };
+  };
 };
 static_assert(sizeof(SettleList) <= LQ_MAX_RANK * 4, "the list lies where other branches keep sL1");
+
+// One element after the other (all threads of the CTA, after its last tile).  Eight blocks of K per MMA: row i of A and column i of B
+// hold block i, so the products wanted are on the diagonal, and loads are contiguous.
+// (What this kernel has written itself is read through the L2, here and below.)
+template <bool SIX>
+__device__ __forceinline__ void settle_elements(const QuantParams& p, float* part, const SettleList& list) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3, blocks = p.Kpad / 32, n = list.entries;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    const int4 what = list.entry[i];
+    const int m = what.x, b = what.y;
+    const uint8_t* qx = p.qx8 + (size_t)m * p.Kpad;
+    const uint8_t* sfx = p.sfa + (size_t)(m >> 7) * (p.Kpad >> 7) * 512 + sf_row(m);
+    float mine = 0.f;
+#pragma unroll 1
+    for (uint32_t todo = (uint32_t)what.z; todo != 0; todo &= todo - 1) {
+      const int j = __ffs(todo) - 1, col = 32 * b + j;
+      if (col >= p.r) break;
+      const uint8_t *l1 = p.l1c + (size_t)col * p.Kpad, *sfl = p.sfl1 + sf_row(col);
+#pragma unroll 1
+      for (int b0 = 8 * warp; b0 < blocks; b0 += 8 * (NTHREADS / 32)) {
+        const int k = b0 + gid;                                  // (blocks is a multiple of 4)
+        uint2 a = make_uint2(0, 0), w = a;
+        float sc = 0.f;
+        if (k < blocks) {
+          a = __ldcg(reinterpret_cast<const uint2*>(qx + 32 * k + 8 * tig));
+          w = __ldg(reinterpret_cast<const uint2*>(l1 + 32 * k + 8 * tig));
+          sc = e8m0(__ldcg(sfx + (k >> 2) * 512 + (k & 3))) * e8m0(__ldg(sfl + (k >> 2) * 512 + (k & 3)));
+        }
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_e4m3_16832(c, a, make_uint2(0, 0), w);
+        if (tig == (gid >> 1) && k < blocks) part[k] = ((gid & 1) ? c[1] : c[0]) * sc;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        float chain = 0.f, v = 0.f;
+        if (lane < SETTLE_CHAINS)
+          for (int k = 2 * lane; k < blocks; k += 2 * SETTLE_CHAINS) chain = __fadd_rn(part[k], __fadd_rn(part[k + 1], chain));
+        for (int c = 0; c < SETTLE_CHAINS; ++c) v = __fadd_rn(v, __shfl_sync(0xffffffffu, chain, c));
+        if (lane == j) mine = v;
+      }
+      __syncthreads();
+    }
+    if (warp == 0) {
+      const float inv = what.w == -127 ? 0.f : pow2f_n(-what.w) * p.unit;
+      if (((uint32_t)what.z >> lane) & 1) p.tq[(size_t)m * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, mine * inv);
+    }
+  }
+}
+
+// By tiles: all near blocks of the CTA in rounds of up to sixteen rows for each block of the rank: warp 9 h + c sums chain c of sixteen
+// of the 32 elements, then a warp adds a row's chains and quantizes them as a4 does.  What bounds it is the tag stage of the L1:
+// eight rows or columns to a load.
 template <bool SIX>
 __device__ __forceinline__ void settle_tiles(const QuantParams& p, float* part, SettleList& list) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3, TR = 8 * p.groups;
@@ -430,10 +490,13 @@ __device__ __forceinline__ void settle_tiles(const QuantParams& p, float* part, 
           float amax = fabsf(v);
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-          const int e = mxfp_exponent<SIX>(amax * p.unit);
+          const uint32_t which = __ldcg(p.near_which + 4 * (size_t)mr + b);
+          uint8_t* const sf = p.sft + (size_t)(mr >> 7) * 512 + sf_row(mr) + b;
+          const int e = which == 0xFFFFFFFFu ? mxfp_exponent<SIX>(amax * p.unit) : (int)__ldcg(sf) - 127;
           const float inv = e == -127 ? 0.f : pow2f_n(-e) * p.unit;
-          p.tq[(size_t)mr * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, v * inv);
-          if (lane == 0) p.sft[(size_t)(mr >> 7) * 512 + sf_row(mr) + b] = (uint8_t)(e + 127);
+          __syncwarp();
+          if ((which >> lane) & 1) p.tq[(size_t)mr * p.tq_stride + 32 * b + lane] = (uint8_t)mxfp_pair<SIX>(0.f, v * inv);
+          if (lane == 0) *sf = (uint8_t)(e + 127);
         }
         __syncthreads();
       }
@@ -527,6 +590,10 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
     *abort_flag = 0;
     mbar_init_fence();
+  }
+  if (BR == BR_MXFP && threadIdx.x == 0) {
+    SettleList* settle = reinterpret_cast<SettleList*>(smem + sm.off_l1);
+    settle->entries = settle->elements = 0;
   }
   if constexpr (BR == BR_INT) {
     if (threadIdx.x < 3 * 64) rowmax[threadIdx.x] = 0;
@@ -651,8 +718,6 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const int nacc = min(p.nacc, p.nst), row = 32 * warp + lane;
     uint32_t tc = 0;
     SettleList* const settle = reinterpret_cast<SettleList*>(smem + sm.off_l1);
-    if (BR == BR_MXFP && lane == 0) settle->met[warp] = 0;
-    __syncwarp();
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++tc) {
       const int m = tile * TR + row;
       const bool valid = row < TR && m < p.M;
@@ -776,16 +841,24 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             if constexpr (FPB) {
               const float dev = amax * p.dev;
               const TieTest<SIX> tie(inv, dev);
-              bool close = ((__float_as_uint(amax + dev) ^ __float_as_uint(amax - dev)) >> 23) != 0;
+              const bool edge = ((__float_as_uint(amax + dev) ^ __float_as_uint(amax - dev)) >> 23) != 0;
+              bool close = edge;
 #pragma unroll
               for (int j = 0; j < 16; ++j) close |= tie(t[j]) | tie(t2[j]);
-              near |= (uint32_t)close << b;
+              if (close && valid) {
+                uint32_t which = 0;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) which |= (tie(t[j]) ? 1u << j : 0u) | (tie(t2[j]) ? 0x10000u << j : 0u);
+                if (edge) which = 0xFFFFFFFFu;
+                near |= 1u << b;
+                p.near_which[4 * (size_t)m + b] = which;
+                atomicAdd(&settle->elements, __popc(which));
+                const int n = atomicAdd(&settle->entries, 1);
+                if (n < SETTLE_ENTRIES) settle->entry[n] = make_int4(m, b, (int)which, e);
+              }
             }
           }
-          if (FPB && valid) {
-            p.near[m] = near;
-            if (near != 0) settle->met[warp] = 1;
-          }
+          if (FPB && valid) p.near[m] = near;
         }
       }
       tc_fence_before();
@@ -987,7 +1060,11 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   __syncthreads();
   if constexpr (BR == BR_MXFP) {
     SettleList& list = *reinterpret_cast<SettleList*>(smem + sm.off_l1);
-    if ((list.met[0] | list.met[1]) != 0 && !*abort_flag) settle_tiles<MAIN == MAIN_MXFP6>(p, reinterpret_cast<float*>(smem), list);
+    float* part = reinterpret_cast<float*>(smem);
+    if (list.elements != 0 && !*abort_flag) {
+      if (list.elements <= settle_few(p.K)) settle_elements<MAIN == MAIN_MXFP6>(p, part, list);
+      else settle_tiles<MAIN == MAIN_MXFP6>(p, part, list);
+    }
   }
   if (BR != BR_NONE && warp == 2) {
     tc_fence_after();
@@ -1035,7 +1112,8 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   p.qx8 = A->d_qx8; p.sx = A->d_sx; p.sfa = A->d_sfa;
   p.qb = g_lq_store_qb ? A->d_qb : nullptr;
   p.sXb = A->d_sXb; p.sL1 = L->d_sL1; p.l1c = L->d_L1c; p.sfl1 = L->d_sfl1;
-  p.sft = A->d_sft; p.tq = A->d_tq; p.sT = A->d_sT; p.near = reinterpret_cast<uint32_t*>(A->d_sT);   // (an MXFP row has no scale of its own)
+  p.sft = A->d_sft; p.tq = A->d_tq; p.sT = A->d_sT; 
+  p.near = reinterpret_cast<uint32_t*>(A->d_sT); p.near_which = reinterpret_cast<uint32_t*>(A->d_qb);   // (an MXFP row has neither a scale nor branch codes of its own)
   p.r = L->r; p.rn = lq_l1_rows(L);
   p.bplanes = lq_l1_planes(L);
   p.tq_stride = A->tq_stride;

@@ -155,10 +155,12 @@ def test_mxfp_host_entry_point_pipelines_row_chunks():
 
 
 @pytest.mark.parametrize("act", ["e4m3", "e2m3"])
-def test_near_ties_of_the_intermediate_do_not_depend_on_the_rows_around(act):
+@pytest.mark.parametrize("what", ["element", "exponent"])
+def test_near_ties_of_the_intermediate_do_not_depend_on_the_rows_around(what, act):
     """Rows whose intermediate is a tie of its element format (272 between 256 and 288, of which 256 is even) plus sixteen terms of a
-    sixteenth of an ulp, which one order of the sum adds up and another rounds away.  Whatever the order, all rows must get the same
-    code: in tiles that are full of such rows, among other rows, and in the row chunks of the host entry point."""
+    sixteenth of an ulp, which one order of the sum adds up and another rounds away; and rows of 256, where the block's exponent changes,
+    less sixteen such terms.  Whatever the order, all rows must get the same codes: in tiles that are full of such rows, among
+    other rows, in the row chunks of the host entry point, and alone."""
     import torch
     from tests.helpers import import_oracle_mxfp_layer
     rng = np.random.default_rng(12)
@@ -166,9 +168,9 @@ def test_near_ties_of_the_intermediate_do_not_depend_on_the_rows_around(act):
     layer = _layer(rng, K, N, r, "mxfp8", bias=False)
     layer["act"] = act
     L1, row = np.zeros((K, r)), np.zeros(K)
-    row[32:34], L1[32:34, 0] = (16, 1), 16
+    row[32:34], L1[32:34, 0] = (16, 1 if what == "element" else 0), 16
     tiny = [64 * box + 32 * h for box in (2, 3, 6, 7, 10, 11, 14, 15) for h in (0, 1)]
-    row[tiny], L1[tiny, 0] = 2.0 ** -10, 2.0 ** -9
+    row[tiny], L1[tiny, 0] = 2.0 ** -10, 2.0 ** -9 if what == "element" else -2.0 ** -10
     L1[:, 40] = -L1[:, 0]
     layer["L1v"], layer["e1"] = F.q_columns(L1, "e4m3")
     assert np.array_equal(F.deq_columns(layer["L1v"], layer["e1"]), L1)
@@ -181,9 +183,13 @@ def test_near_ties_of_the_intermediate_do_not_depend_on_the_rows_around(act):
     st = torch.cuda.current_stream().cuda_stream
     try:
         x = torch.from_numpy(X).cuda()
-        B.lq_quantize_act(h, x.data_ptr(), M, a, st)
-        ex = B.lq_act_export(a, M, cfg, st)
-        tq, sT = ex["tq"].copy(), ex["sT"].copy()
+        tq = sT = None
+        for rows in (M, 1, 3, 40):
+            B.lq_quantize_act(h, x.data_ptr(), rows, a, st)
+            ex = B.lq_act_export(a, rows, cfg, st)
+            if rows == M:
+                tq, sT = ex["tq"].copy(), ex["sT"].copy()
+            assert np.array_equal(ex["tq"], tq[:rows]) and np.array_equal(ex["sT"], sT[:rows]), rows
         t = F.deq_mxfp(B.e4m3_decode(tq), sT.astype(np.int16))
         assert np.unique(t[same][:, 0]).tolist() == [256.0] and np.unique(t[same][:, 40]).tolist() == [-256.0]
         assert (t[same][:, [j for j in range(r) if j not in (0, 40)]] == 0).all()
