@@ -118,6 +118,10 @@ __device__ __forceinline__ Scales load_scales(const float* sc, int row_at, int c
   for (int k = 0; k < 4; ++k) v.sw[k] = *reinterpret_cast<const float4*>(sc + LQ_BM + col_at + 16 * k);
   return v;
 }
+// Two orders of the same products.  The codes' sums have 12 bits and the fp16 scales 11, so P sx and sx sw are exact alike and every FMA
+// rounds the same number; P sx leaves an FMA with an operand (sw) that four rows in a row share, which costs the register file
+// less (us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 79.2 / 86.4 -> 76.4 / 82.4).  The integer branch's scales have 24 bits, its sums up
+// to 22: there sx sw is rounded first.
 template <bool INT>
 __device__ __forceinline__ void drain_group(const Frag (&v)[4], float2 (&acc)[2][16], const Scales& sc) {
   const float4 sx = sc.sx;
@@ -129,10 +133,16 @@ __device__ __forceinline__ void drain_group(const Frag (&v)[4], float2 (&acc)[2]
     for (int e = 0; e < 2; ++e) {
       const int j = 2 * k + e, c = j >> 2, q = 4 * (j & 3);
       const float2 sw = e ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
-      acc[0][2 * j] = __ffma2_rn(fragment_pair<INT>(v[2 * c][q], v[2 * c][q + 1]), __fmul2_rn(s0, sw), acc[0][2 * j]);
-      acc[0][2 * j + 1] = __ffma2_rn(fragment_pair<INT>(v[2 * c][q + 2], v[2 * c][q + 3]), __fmul2_rn(s1, sw), acc[0][2 * j + 1]);
-      acc[1][2 * j] = __ffma2_rn(fragment_pair<INT>(v[2 * c + 1][q], v[2 * c + 1][q + 1]), __fmul2_rn(s2, sw), acc[1][2 * j]);
-      acc[1][2 * j + 1] = __ffma2_rn(fragment_pair<INT>(v[2 * c + 1][q + 2], v[2 * c + 1][q + 3]), __fmul2_rn(s3, sw), acc[1][2 * j + 1]);
+      const float2 p0 = fragment_pair<INT>(v[2 * c][q], v[2 * c][q + 1]), p1 = fragment_pair<INT>(v[2 * c][q + 2], v[2 * c][q + 3]);
+      const float2 p2 = fragment_pair<INT>(v[2 * c + 1][q], v[2 * c + 1][q + 1]), p3 = fragment_pair<INT>(v[2 * c + 1][q + 2], v[2 * c + 1][q + 3]);
+      float2 &a0 = acc[0][2 * j], &a1 = acc[0][2 * j + 1], &a2 = acc[1][2 * j], &a3 = acc[1][2 * j + 1];
+      if constexpr (INT) {
+        a0 = __ffma2_rn(p0, __fmul2_rn(s0, sw), a0); a1 = __ffma2_rn(p1, __fmul2_rn(s1, sw), a1);
+        a2 = __ffma2_rn(p2, __fmul2_rn(s2, sw), a2); a3 = __ffma2_rn(p3, __fmul2_rn(s3, sw), a3);
+      } else {
+        const float2 t0 = __fmul2_rn(p0, s0), t1 = __fmul2_rn(p1, s1), t2 = __fmul2_rn(p2, s2), t3 = __fmul2_rn(p3, s3);
+        a0 = __ffma2_rn(t0, sw, a0); a1 = __ffma2_rn(t1, sw, a1); a2 = __ffma2_rn(t2, sw, a2); a3 = __ffma2_rn(t3, sw, a3);
+      }
     }
   }
 }
