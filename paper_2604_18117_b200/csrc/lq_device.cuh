@@ -143,6 +143,20 @@ __device__ __forceinline__ void sts_v2(uint32_t a, const uint2& v) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
 }
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+// 32 bytes (of an address that is a multiple of 32) to global memory: a whole sector in one request
+__device__ __forceinline__ void stg_v8(void* p, const uint32_t (&w)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]),
+               "r"(w[6]), "r"(w[7]) : "memory");
+}
+// the same of an address that is a multiple of 32 or (wide = 0) only of 16
+__device__ __forceinline__ void stg_32(void* p, const uint32_t (&w)[8], int wide) {
+  if (wide) {
+    stg_v8(p, w);
+  } else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
 // generic-proxy writes to shared memory become visible to the asynchronous proxy (MMA operands, tensor-memory copies)
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 

@@ -92,6 +92,7 @@ struct GemmParams {
   const float* bias;      // [Npad]
   void* Y;
   int out_f32;
+  int wide;               // Y and its rows begin on 32-byte boundaries
   int32_t* status;
 };
 
@@ -434,7 +435,9 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                   __float_as_uint(acc[h][4 * k + 2 + i].x), __float_as_uint(acc[h][4 * k + 2 + i].y)));
             }
       } else {
-        // epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad
+        // Epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad.  Two lanes' stores of 16
+        // bytes never meet in a 32-byte sector here, so each would write half of one; where all of Y's rows are whole sectors a lane
+        // stores 32 bytes at once (us, M = 8192, K x N = 1152 x 3456: 79.3 -> 73.4).
         const int c = n0 + coff + 16 * ft;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
@@ -445,9 +448,15 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (p.out_f32) {
               float* Y = reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c;
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                if (c + 8 * (k >> 1) < p.N)
-                  *reinterpret_cast<float4*>(Y + 4 * k) = make_float4(acc[h][4 * k + i].x, acc[h][4 * k + i].y, acc[h][4 * k + 2 + i].x, acc[h][4 * k + 2 + i].y);
+              for (int k = 0; k < 2; ++k) {
+                uint32_t w[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                  w[2 * j] = __float_as_uint(acc[h][8 * k + 2 * j + i].x);
+                  w[2 * j + 1] = __float_as_uint(acc[h][8 * k + 2 * j + i].y);
+                }
+                if (c + 8 * k < p.N) stg_32(Y + 8 * k, w, p.wide);
+              }
             } else {
               __half* Y = reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c;
               uint32_t w[8];
@@ -456,8 +465,12 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const __half2 q = __floats2half2_rn(acc[h][2 * j + i].x, acc[h][2 * j + i].y);
                 w[j] = *reinterpret_cast<const uint32_t*>(&q);
               }
-              if (c < p.N) *reinterpret_cast<uint4*>(Y) = make_uint4(w[0], w[1], w[2], w[3]);
-              if (c + 8 < p.N) *reinterpret_cast<uint4*>(Y + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+              if (p.wide) {                               // (N is then a multiple of 16)
+                if (c < p.N) stg_v8(Y, w);
+              } else {
+                if (c < p.N) *reinterpret_cast<uint4*>(Y) = make_uint4(w[0], w[1], w[2], w[3]);
+                if (c + 8 < p.N) *reinterpret_cast<uint4*>(Y + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+              }
             }
           }
       }
@@ -584,6 +597,7 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   p.units_n = L->Npad / UNIT;
   p.sx = A->d_sx; p.sw = L->d_sw; p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
   p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
+  p.wide = lq_rows_of_sectors(Y, L->N, dt);
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;
   int sms = 0;

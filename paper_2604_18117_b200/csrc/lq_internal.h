@@ -177,6 +177,11 @@ static inline int lq_l1_planes(const lq_layer* L) { return L->a8 && L->cfg.branc
 // TMA descriptor (lq_api.cu): 2-D byte tensor [rows][row_bytes], box [box_rows][128 bytes], 128-byte swizzle.
 lq_status lq_make_tmap_bytes(CUtensorMap* tm, void* base, uint64_t rows, uint64_t row_bytes, uint32_t box_rows);
 
+// whether every row of Y begins on a 32-byte boundary (callers promise 16 bytes, and N a multiple of 8)
+static inline int lq_rows_of_sectors(const void* Y, int N, lq_out_dtype dt) {
+  return (((uintptr_t)Y | (uintptr_t)N * (dt == LQ_OUT_F32 ? 4 : 2)) & 31) == 0;
+}
+
 // byte an MMA operand carries for a 4-bit code q in [-7, 7]
 static inline uint8_t lq_encode_code_host(int q, int kind) {
   if (kind == LQ_KIND_I8) return (uint8_t)(int8_t)q;
