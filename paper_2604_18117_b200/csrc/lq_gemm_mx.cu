@@ -94,6 +94,7 @@ struct MxParams {
   const float* bias;      // [Npad]
   void* Y;
   int out_f32;
+  int wide;               // Y and its rows begin on 32-byte boundaries
   int32_t* status;
 };
 
@@ -495,10 +496,11 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               y[j] = fmaf(__int_as_float((int)u[h][4 * (j >> 1) + q + (j & 1)] + 0x4B400000) - 12582912.0f, st * sl[j], y[j]);
           }
           if (r < p.M && c < p.N) {
-            if (p.out_f32) {
-              float4* Y = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c);
-              Y[0] = make_float4(y[0], y[1], y[2], y[3]);
-              Y[1] = make_float4(y[4], y[5], y[6], y[7]);
+            if (p.out_f32) {                                // (whole sectors; us, M = 1365, 1160 x 2312: 11.3 by 16 bytes, 9.2 so)
+              uint32_t o[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) o[j] = __float_as_uint(y[j]);
+              stg_32(reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c, o, p.wide);
             } else {
               uint32_t o[4];
 #pragma unroll
@@ -598,7 +600,7 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   p.b_row = LQ_KSTAGE / 8 * lq_mx_weight_bits(L); p.b_format = L->mxfp ? IDESC_MX_B_E2M1 : IDESC_MX_B_E2M3;
   p.block0 = A->block0;
   p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
-  p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
+  p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0; p.wide = lq_rows_of_sectors(Y, L->N, dt);
   const int c = pair ? 2 : 1;
   const long long tiles = (long long)lq_ceil_div(p.tiles_m, c) * p.tiles_n;
   ctas = c * (int)std::min<long long>(ctas / c, tiles);

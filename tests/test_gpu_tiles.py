@@ -123,3 +123,35 @@ def test_pairs_of_ctas_give_the_bits_of_single_ones_every_time(option, main, bra
     assert all(torch.equal(alone, y) for y in pairs)
     B.lq_act_free(act)
     B.lq_layer_free(h)
+
+
+@pytest.mark.parametrize("main,branch,r", [("sint4", "w8a8", 32), ("mxint4", "w8a8", 32), ("mxfp4", "mxfp8", 64)])
+@pytest.mark.parametrize("N", [8, 72, 208])
+def test_outputs_that_begin_between_sectors(option, main, branch, r, N):
+    """Rows of Y that begin on 16-byte boundaries only, by their length or by Y's own place, hold the bits of those that begin on
+    32-byte ones, and nothing beside them is written."""
+    import torch
+    from tests.helpers import import_oracle_layer, import_oracle_mxfp_layer
+
+    option("gemm_split", 1)                                       # (tiles shared by a cluster are stored by 16 bytes)
+    rng = np.random.default_rng(N)
+    M, K = 131, 200
+    layer = {"sint4": SINT4._random_layer, "mxint4": MXINT4._mx_layer, "mxfp4": MXFP._layer}[main](rng, K, N, r, branch)
+    h, _ = (import_oracle_mxfp_layer if main == "mxfp4" else import_oracle_layer)(layer)
+    B.lq_layer_to_device(h, 0)
+    act = B.lq_act_create(h, M, 0)
+    x, st = torch.from_numpy(_x(rng, M, K)).cuda(), torch.cuda.current_stream().cuda_stream
+    B.lq_quantize_act(h, x.data_ptr(), M, act, st)
+    for dtype, out in ((torch.float16, B.OUT_F16), (torch.float32, B.OUT_F32)):
+        size, got = 16 // torch.empty(0, dtype=dtype).element_size(), []      # elements of 16 bytes
+        for at in (2 * size, 3 * size):
+            y = torch.full((M * N + 6 * size,), 7.0, dtype=dtype, device="cuda")
+            assert y.data_ptr() % 32 == 0
+            B.lq_linear_forward(h, act, y.data_ptr() + 16 * at // size, out, st)
+            got.append(y[at:at + M * N])
+            assert bool((y[:at] == 7).all()) and bool((y[at + M * N:] == 7).all())
+        assert torch.equal(got[0], got[1])
+        assert float(got[0].float().std()) > 0
+    assert B.lq_get_device_status(0)[0] == 0
+    B.lq_act_free(act)
+    B.lq_layer_free(h)
