@@ -11,9 +11,12 @@
 //   warp 3      TMA producer of X: a box is TR rows x 64 values; a ring of up to twelve chunks is always in flight, across
 //               tiles too
 //   warps 5-19  quantizer: teams of RG x SX warps take the chunks in turn; in a chunk each warp has one piece, 8 rows x one
-//               stage.  Eight lanes own 64 values of a row, a 16-byte vector each, and every lane has vectors of two rows: a
-//               block of 32 is four lanes, its maximum two shuffles, and loads, stores and shared-memory accesses all move
-//               whole rows of a box.  (A first version loaded X into registers from global memory, half rows per
+//               stage.  A lane owns 16 neighbouring values of two rows, two 16-byte vectors of X each: they share a block and its
+//               scale, a block of 32 is two lanes, its maximum one shuffle, and a lane's codes are one 16-byte store, to global and
+//               to shared memory.  (With a vector of each half of the stage to a lane, four lanes to a block, every scale was worked
+//               out twice as often and stores were of 8 bytes; us, M = 8192, K = 1152 / 4608: SINT4 11.8 / 34.6 -> 11.3 / 32.8, MXINT4 x 8 12.7 /
+//               36.1 -> 12.0 / 33.6.)
+//               Loads and stores move whole rows of a box.  (A first version loaded X into registers from global memory, half rows per
 //               instruction: the tag stage of the L1 was what bounded it, at 40 lookups a piece, and its unrolled ring
 //               cost a microsecond of instruction misses.)  The branch's operand goes to shared memory in the layout
 //               the MMA reads (K-major, 128-byte swizzle).  More warps (28 at 64 registers) were no faster, twelve were
@@ -279,6 +282,7 @@ struct Sint4Scale {
     coarse = (bits & 0xFFFFu) < 0x0400u || bits < 0x04000000u;
   }
 };
+__device__ __forceinline__ uint4 vec16(const uint2 (&v)[2]) { return make_uint4(v[0].x, v[0].y, v[1].x, v[1].y); }
 __device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
 __device__ __forceinline__ uint2 sint4_codes8(const uint4& v, float rcp, bool coarse) {
   const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
@@ -867,19 +871,20 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
   } else if (warp >= FIRST_QWARP && qw < nq * p.teams) {
     // ------------------------------------------------------------------ quantizer
-    // This lane: 16-byte vector lc of rows ra and ra + 2 of the tile, of both 64-value boxes of a stage.  The four rows of
-    // one access have both values of bit 2, so that the 64-byte halves they write to an operand slab do not meet in the
-    // same banks.
-    const int team = qw / nq, rg = (qw - team * nq) % RG, sx = (qw - team * nq) / RG, lr = lane >> 3, lc = lane & 7;
-    const int ra = 8 * rg + (lr & 1) + 2 * (lr & 2);
-    const uint32_t sw = (uint32_t)(ra & 7), hstep = (uint32_t)(TR * 128);               // from a box to the next
-    const uint32_t xo = base + (uint32_t)(sx * TR * 256 + ra * 128);                    // row ra of this warp's first box
-    const uint32_t xo_a = xo + ((lc ^ sw) << 4), xo_b = xo + 256 + ((lc ^ sw ^ 2) << 4);
-    // this lane's eight codes in an operand slab (rows of 128 bytes, 16-byte pieces exchanged by row mod 8); the second box's
-    // are at the address with bit 6 flipped
-    const uint32_t ao = base + (uint32_t)(sm.off_slots + sx * sm.a_ps * sm.a_unit + ra * 128 + 8 * (lc & 1));
-    const uint32_t ao_a = ao + (((lc >> 1) ^ sw) << 4), ao_b = ao + 256 + (((lc >> 1) ^ sw ^ 2) << 4);
-    const int sr = ra + 2 * (lc & 1);                                                   // lanes 0 and 1 of a row store its scale bytes
+    // This lane: 16 neighbouring values (a piece pair pp of a box) of rows ra and ra + 2 of the tile.  They share a block, so its scale
+    // is worked out once, and their codes are one 16-byte vector of a row.  The two rows that eight lanes in a row read or write
+    // together differ in bits 0 and 2: even pieces of X and the four pieces of an operand slab's half fall in different banks.
+    const int team = qw / nq, rg = (qw - team * nq) % RG, sx = (qw - team * nq) / RG, pp = lane & 3, box = (lane >> 3) & 1;
+    const int ra = 8 * rg + (((lane >> 2) & 1) * 5 ^ (lane >> 4));
+    const uint32_t sw = (uint32_t)(ra & 7);
+    // X: the pair's first piece (the second is at the address with bit 4 flipped), a box is TR rows of 128 bytes
+    const uint32_t xo = base + (uint32_t)(sx * TR * 256 + box * TR * 128 + ra * 128);
+    const uint32_t xo_a = xo + (((2 * pp) ^ sw) << 4), xo_b = xo + 256 + (((2 * pp) ^ sw ^ 2) << 4);
+    // this lane's 16 codes in an operand slab (rows of 128 bytes, 16-byte pieces exchanged by row mod 8)
+    const uint32_t ao = base + (uint32_t)(sm.off_slots + sx * sm.a_ps * sm.a_unit + ra * 128);
+    const uint32_t ao_a = ao + (((4 * box + pp) ^ sw) << 4), ao_b = ao + 256 + (((4 * box + pp) ^ sw ^ 2) << 4);
+    const int sr = ra + 2 * box;                                                        // the row whose scale bytes (maximum, scale) this lane has where
+    const bool first = pp == 0;                                                         // it is its box's first
     const uint32_t so = base + (uint32_t)(sm.off_slots + sm.off_sfa + sx * sm.a_ps * 512 + 16 * (sr & 31) + 4 * (sr >> 5));
     const size_t qs = MAIN == MAIN_MXINT8 ? (size_t)2 * p.Kpad : (size_t)p.Kpad;        // bytes per row of qx8
     grid_dependency_wait();        // from here on the activation record is written
@@ -889,8 +894,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     bool ok = true;
     for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x, ++tc) {
       const int ma = tile * TR + ra, ms = tile * TR + sr;
-      const bool va = ma < p.M, vb = ma + 2 < p.M, vs = lc < 2 && ms < p.M;
-      uint8_t* const qa = p.qx8 + (size_t)ma * qs + sx * 128 + 8 * lc;
+      const bool va = ma < p.M, vb = ma + 2 < p.M, vs = first && ms < p.M;
+      uint8_t* const qa = p.qx8 + (size_t)ma * qs + sx * 128 + 64 * box + 16 * pp;
       uint8_t* const sfr = SINT ? nullptr : p.sfa + ((size_t)(ms >> 7) * (qs >> 7) + sx) * 512 + 16 * (ms & 31) + 4 * ((ms & 127) >> 5);
       float sb_a = 1.f, sb_b = 1.f, inv_a = 1.f, inv_b = 1.f;
       __half2 hm = __float2half2_rn(0.f);                        // maxima of rows ra, ra + 2
@@ -906,46 +911,50 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           if (live) {
             const uint32_t at = (uint32_t)(x.at * sm.xslot);
             a[0] = lds_v4(xo_a + at); b[0] = lds_v4(xo_b + at);
-            a[1] = lds_v4(xo_a + at + hstep); b[1] = lds_v4(xo_b + at + hstep);
+            a[1] = lds_v4((xo_a + at) ^ 16); b[1] = lds_v4((xo_b + at) ^ 16);
           }
           uint2 wa[2], wb[2], da[2], db[2];                      // main codes of the two rows (MXINT8: hi digits; d: lo digits)
           uint32_t four = 0;                                     // the stage's scale bytes of row sr (lanes 0 and 1 of a row)
           if constexpr (decltype(MAINP)::value) {
             if (live) {
-              [[maybe_unused]] uint32_t own = 0;
+              __half2 bm = __halves2half2(__hmax(absmax8(a[0]), absmax8(a[1])), __hmax(absmax8(b[0]), absmax8(b[1])));
+              bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
+              if constexpr (SINT) bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
+              if constexpr (BR == BR_INT) hm = __hmax2(hm, bm);
+              if constexpr (SINT) {
+                const Sint4Scale sc(bm);
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                __half2 bm = __halves2half2(absmax8(a[h]), absmax8(b[h]));
-                bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
-                bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
-                if constexpr (SINT) bm = __hmax2(bm, __shfl_xor_sync(0xffffffffu, bm, 4));
-                if constexpr (BR == BR_INT) hm = __hmax2(hm, bm);
-                if constexpr (SINT) {
-                  const Sint4Scale sc(bm);
+                for (int h = 0; h < 2; ++h) {
                   wa[h] = sint4_codes8(a[h], sc.inv[0], sc.coarse); wb[h] = sint4_codes8(b[h], sc.inv[1], sc.coarse);
-                  if (vs) p.sx[(size_t)(2 * st + h) * p.Mpad + lq_row_slot(ms)] = lc ? sc.s[1] : sc.s[0];   // (of a padding group, too)
-                } else {
-                  constexpr int TOP = MAIN == MAIN_MXINT4 ? 2 : MAIN == MAIN_MXINT8 ? 6 : 8;
-                  constexpr int UP = MAIN == MAIN_MXINT4 ? 0xFF : MAIN == MAIN_MXINT8 ? 0x0F : 0;
-                  const PairScale<TOP, UP> ps(as_u32(bm));
-                  uint32_t bytes = ps.bytes;
-                  if (MAIN != MAIN_MXFP6 && ps.ok) {
-                    const __half2 i0 = as_half2(__byte_perm(ps.inv, 0, 0x1010)), i1 = as_half2(__byte_perm(ps.inv, 0, 0x3232));
+                }
+                // (of a padding group, too)
+                if (pp < 2 && ma + 2 * pp < p.M) p.sx[(size_t)(2 * st + box) * p.Mpad + lq_row_slot(ma + 2 * pp)] = pp ? sc.s[1] : sc.s[0];
+              } else {
+                constexpr int TOP = MAIN == MAIN_MXINT4 ? 2 : MAIN == MAIN_MXINT8 ? 6 : 8;
+                constexpr int UP = MAIN == MAIN_MXINT4 ? 0xFF : MAIN == MAIN_MXINT8 ? 0x0F : 0;
+                const PairScale<TOP, UP> ps(as_u32(bm));
+                uint32_t own = ps.bytes;                         // this block's bytes: row ra's and, 16 bits on, row ra + 2's
+                if (MAIN != MAIN_MXFP6 && ps.ok) {
+                  const __half2 i0 = as_half2(__byte_perm(ps.inv, 0, 0x1010)), i1 = as_half2(__byte_perm(ps.inv, 0, 0x3232));
+#pragma unroll
+                  for (int h = 0; h < 2; ++h) {
                     if constexpr (MAIN == MAIN_MXFP) { wa[h] = mxfp8_codes8(a[h], i0); wb[h] = mxfp8_codes8(b[h], i1); }
                     else if constexpr (MAIN == MAIN_MXINT4) { wa[h] = mxint4_codes8(a[h], i0); wb[h] = mxint4_codes8(b[h], i1); }
                     else if constexpr (MAIN == MAIN_MXINT8) { mxint8_codes8(a[h], i0, wa[h], da[h]); mxint8_codes8(b[h], i1, wb[h], db[h]); }
-                  } else {
+                  }
+                } else {
+#pragma unroll
+                  for (int h = 0; h < 2; ++h) {
                     const RareCodes rc = rare_codes<MAIN>(a[h], b[h], bm);
                     wa[h] = rc.wa; wb[h] = rc.wb; da[h] = rc.da; db[h] = rc.db;
-                    bytes = rc.bytes;
+                    own = rc.bytes;
                   }
-                  own |= bytes << (8 * h);
                 }
-              }
-              if constexpr (!SINT) {
-                // a row's four bytes are with two lanes, a block pair apart: lane 0 collects row ra's, lane 1 row ra + 2's
-                const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 4);
-                four = __byte_perm(own, other, lc ? 0x7362 : 0x5140);
+                // a row's four bytes are with four lanes: the box's two blocks, then the boxes; box 0 collects row ra's, box 1 row ra + 2's
+                const uint32_t next = __shfl_xor_sync(0xffffffffu, own, 2);
+                const uint32_t both = __byte_perm(pp & 2 ? next : own, pp & 2 ? own : next, 0x6240);
+                const uint32_t other = __shfl_xor_sync(0xffffffffu, both, 8);
+                four = box ? __byte_perm(other, both, 0x7632) : __byte_perm(both, other, 0x5410);
                 if (vs) {
                   uint8_t* sf = sfr + (size_t)c * spc * 512;     // (the hi digits weigh 16 times as much)
                   *reinterpret_cast<uint32_t*>(sf) = MAIN == MAIN_MXINT8 ? four + 0x04040404u : four;
@@ -953,16 +962,13 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
                 }
               }
               uint8_t* const q = qa + c * spc * 128;
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                if (va) {
-                  *reinterpret_cast<uint2*>(q + 64 * h) = wa[h];
-                  if (MAIN == MAIN_MXINT8) *reinterpret_cast<uint2*>(q + p.Kpad + 64 * h) = da[h];
-                }
-                if (vb) {
-                  *reinterpret_cast<uint2*>(q + 2 * qs + 64 * h) = wb[h];
-                  if (MAIN == MAIN_MXINT8) *reinterpret_cast<uint2*>(q + 2 * qs + p.Kpad + 64 * h) = db[h];
-                }
+              if (va) {
+                *reinterpret_cast<uint4*>(q) = vec16(wa);
+                if (MAIN == MAIN_MXINT8) *reinterpret_cast<uint4*>(q + p.Kpad) = vec16(da);
+              }
+              if (vb) {
+                *reinterpret_cast<uint4*>(q + 2 * qs) = vec16(wb);
+                if (MAIN == MAIN_MXINT8) *reinterpret_cast<uint4*>(q + 2 * qs + p.Kpad) = vec16(db);
               }
             }
           }
@@ -977,29 +983,27 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             if (!mbar_wait_warp(bar_empty(e.at), e.par, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
             const uint32_t at = (uint32_t)(e.at * sm.slot);
             if (live) {
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                if constexpr (BR == BR_INT) {
-                  sts_v2((ao_a + at) ^ (64 * h), ca[h]);
-                  sts_v2((ao_b + at) ^ (64 * h), cb[h]);
-                  if (p.qb != nullptr) {
-                    int8_t* o = p.qb + (qa - p.qx8) + c * spc * 128 + 64 * h;
-                    if (va) *reinterpret_cast<uint2*>(o) = ca[h];
-                    if (vb) *reinterpret_cast<uint2*>(o + 2 * qs) = cb[h];
-                  }
-                } else if constexpr (BR == BR_F16) {             // a slab per box: 64 halves, laid out as in the X ring
-                  sts_v4(xo_a + sm.off_slots + at + h * hstep, a[h]);
-                  sts_v4(xo_b + sm.off_slots + at + h * hstep, b[h]);
-                } else {
-                  sts_v2((ao_a + at) ^ (64 * h), wa[h]);
-                  sts_v2((ao_b + at) ^ (64 * h), wb[h]);
-                  if constexpr (BR == BR_MXINT) {
-                    sts_v2(((ao_a + at) ^ (64 * h)) + sm.a_unit, da[h]);
-                    sts_v2(((ao_b + at) ^ (64 * h)) + sm.a_unit, db[h]);
-                  }
+              if constexpr (BR == BR_INT) {
+                sts_v4(ao_a + at, vec16(ca));
+                sts_v4(ao_b + at, vec16(cb));
+                if (p.qb != nullptr) {
+                  int8_t* o = p.qb + (qa - p.qx8) + c * spc * 128;
+                  if (va) *reinterpret_cast<uint4*>(o) = vec16(ca);
+                  if (vb) *reinterpret_cast<uint4*>(o + 2 * qs) = vec16(cb);
+                }
+              } else if constexpr (BR == BR_F16) {               // a slab per box: 64 halves, laid out as in the X ring
+                const uint32_t to = (uint32_t)sm.off_slots + at;
+                sts_v4(xo_a + to, a[0]); sts_v4((xo_a + to) ^ 16, a[1]);
+                sts_v4(xo_b + to, b[0]); sts_v4((xo_b + to) ^ 16, b[1]);
+              } else {
+                sts_v4(ao_a + at, vec16(wa));
+                sts_v4(ao_b + at, vec16(wb));
+                if constexpr (BR == BR_MXINT) {
+                  sts_v4(ao_a + at + sm.a_unit, vec16(da));
+                  sts_v4(ao_b + at + sm.a_unit, vec16(db));
                 }
               }
-              if (MXB && lc < 2) {
+              if (MXB && first) {
                 sts_u32(so + at, BR == BR_MXINT ? four + 0x04040404u : four);
                 if (BR == BR_MXINT) sts_u32(so + at + 512, four);
               }
@@ -1027,9 +1031,10 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         ok = walk(Yes(), No(), p.refetch != 0);
         if (!ok) break;
         // ---- the rows' maxima and scales: non-negative halves order like their bit patterns
-        hm = __hmax2(hm, __shfl_xor_sync(0xffffffffu, hm, 4));
+        if constexpr (!SINT) hm = __hmax2(hm, __shfl_xor_sync(0xffffffffu, hm, 2));
+        hm = __hmax2(hm, __shfl_xor_sync(0xffffffffu, hm, 8));
         int* mx = rowmax + buf * 64;
-        if (lc < 2) atomicMax(&mx[sr], (int)__half_as_ushort(lc ? __high2half(hm) : __low2half(hm)));
+        if (first) atomicMax(&mx[sr], (int)__half_as_ushort(box ? __high2half(hm) : __low2half(hm)));
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_sync);
         ok = mbar_wait_warp(bar_sync, tc & 1, abort_flag, p.status, LQ_STAGE_QUANT);
@@ -1037,7 +1042,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const float rm_a = __half2float(__ushort_as_half((unsigned short)mx[ra]));
         const float rm_b = __half2float(__ushort_as_half((unsigned short)mx[ra + 2]));
         const uint32_t after = buf == 0 ? 2 : buf - 1;           // two tiles on: every warp is past its last use
-        if (team == 0 && sx == 0 && lc < 2) rowmax[after * 64 + sr] = 0;
+        if (team == 0 && sx == 0 && first) rowmax[after * 64 + sr] = 0;
         buf = buf == 2 ? 0 : buf + 1;
         sb_a = rm_a == 0.f ? 1.f : __fdiv_rn(rm_a, p.qm);
         sb_b = rm_b == 0.f ? 1.f : __fdiv_rn(rm_b, p.qm);
@@ -1045,8 +1050,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (team == 0 && sx == 0) {                              // a4 reads the scale: its previous tile of this parity must be done
           ok = mbar_wait_warp(bar_tempty(tc & 1), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_QUANT);
           if (!ok) break;
-          if (lc < 2) row_sb[(tc & 1) * 64 + sr] = lc ? sb_b : sb_a;
-          if (vs) p.sXb[ms] = lc ? sb_b : sb_a;
+          if (first) row_sb[(tc & 1) * 64 + sr] = box ? sb_b : sb_a;
+          if (vs) p.sXb[ms] = box ? sb_b : sb_a;
         }
         ok = walk(No(), Yes(), true);
       } else {
