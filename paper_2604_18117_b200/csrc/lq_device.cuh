@@ -148,9 +148,10 @@ __device__ __forceinline__ void stg_v8(void* p, const uint32_t (&w)[8]) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]),
                "r"(w[6]), "r"(w[7]) : "memory");
 }
-// the same of an address that is a multiple of 32 or (wide = 0) only of 16
-__device__ __forceinline__ void stg_32(void* p, const uint32_t (&w)[8], int wide) {
-  if (wide) {
+// the same of an address that is a multiple of 32 (SECTORS) or only of 16
+template <bool SECTORS>
+__device__ __forceinline__ void stg_32(void* p, const uint32_t (&w)[8]) {
+  if constexpr (SECTORS) {
     stg_v8(p, w);
   } else {
     reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);

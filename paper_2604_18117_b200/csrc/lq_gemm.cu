@@ -17,14 +17,17 @@
 //               whole group is in flight into one register buffer while the one before is consumed from the other:
 //               acc += P * (sx * sw), packed f32x2, fp32 registers.  An accumulator goes back as soon as it sits in
 //               registers.  The next tile's first group is requested before the epilogue
-// What bounds it: the FP32 pipe's operand delivery, and the hand-shakes around it.  Per group and scheduler 64 packed
-// products (two operands: 2 clocks each, measured) and 64 packed FMAs (three: 4 clocks) are 384 clocks, the tensor pipe
-// needs 128; the kernel takes 530.  So everything that is not arithmetic is kept out of the drain's instruction stream: two
+// What bounds it: the FP32 pipe's operand delivery and the drain's other instructions.  Per group and scheduler 64 packed products
+// (2.0 to 2.6 clocks each, measured) and 64 packed FMAs (2.75 with an operand shared by neighbours, 3.9 with three of their own) are about 320
+// clocks, the tensor pipe needs 128; the same loop over tensor memory without any hand-shake takes 400, 100 of them for the scales' way
+// from shared memory, the kernel takes 440.  So everything that is not arithmetic is kept out of the drain's instruction stream: two
 // wide warps per scheduler instead of four narrow ones, no wait or arrival for the scale vectors (they live in a ring deep
-// enough that the accumulators' hand-shakes imply theirs), one wait per stage, 216 registers per drain thread, partly
+// enough that the accumulators' hand-shakes imply theirs), one wait per stage, 224 registers per drain thread, partly
 // taken over from the other four warps (setmaxnreg).  M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 85 / 96 us with sixteen
-// narrow warps, 80 / 89 with one commit per group, 75.5 / 80 now.  (Scalar FMAs, 3 clocks for two, lose what they gain to
-// their issue slots: 89 / 101 us.)
+// narrow warps, 80 / 89 with one commit per group, 79 / 86 before P sx was taken first, sectors were stored whole, the issuer lost its
+// branches and the drain got its last eight registers.  Scalar FMAs lose their issue slots (94 - 104 us for 79); scales of
+// the next group loaded where this one's were used last, 302 clocks a group by itself, made the kernel slower (73.6 for 68.8: registers); two column
+// halves as pipelines of their own, each with an issuer, 67.9 for 66.5.
 // Orders of rows and columns (lq_internal.h) are chosen for the drain's fragments: the columns of the tile are permuted in
 // the weight operand so that a lane's 16 columns of a row are neighbours in Y - the epilogue converts and stores, no
 // exchange - and the scale vectors are permuted so that a lane's come in one (rows) and four (columns) 16-byte loads
@@ -71,8 +74,9 @@ constexpr int NUM_DRAIN_WARPS = 8;
 constexpr int FIRST_DRAIN_WARP = 4;                // the first warpgroup: TMA, MMA, two idle warps
 constexpr int GEMM_THREADS = (FIRST_DRAIN_WARP + NUM_DRAIN_WARPS) * 32;
 constexpr int WCOLS = 64;                          // columns per drain warp
-// 12 warps are launched with 168 registers a thread (64512 in all); 128 x 56 + 256 x 216 = 62464
-constexpr int LEAN_REGS = 56, DRAIN_REGS = 216;
+// 12 warps are launched with 168 registers a thread: 384 x 168 = 64512 = 128 x 56 + 256 x 224.  (216 for the drain: 64.6 / 73.1 us at the sizes
+// above for 62.7 / 69.6; 232 and 40: 64.1 / 71.5, the producer spills)
+constexpr int LEAN_REGS = 56, DRAIN_REGS = 224;
 constexpr int SMEM_BAR_BYTES = 256;
 constexpr int SMEM_BYTES = 1024 /*alignment slack*/ + NSTAGE * STAGE_BYTES + SC_RING * SC_STAGE_BYTES + SMEM_BAR_BYTES;
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
@@ -92,7 +96,6 @@ struct GemmParams {
   const float* bias;      // [Npad]
   void* Y;
   int out_f32;
-  int wide;               // Y and its rows begin on 32-byte boundaries
   int32_t* status;
 };
 
@@ -112,12 +115,10 @@ __device__ __forceinline__ float2 fragment_pair(uint32_t a, uint32_t b) {
 struct Scales {                                       // a lane's four row scales and 16 column scales of a group
   float4 sx, sw[4];
 };
-__device__ __forceinline__ Scales load_scales(const float* sc, int row_at, int col_at) {
-  Scales v;
-  v.sx = *reinterpret_cast<const float4*>(sc + row_at);                     // rows g, g + 8, g + 16, g + 24
+__device__ __forceinline__ void load_scales(Scales& v, uint32_t sx_at, uint32_t sw_at) {
+  v.sx = *reinterpret_cast<const float4*>(__cvta_shared_to_generic(sx_at));           // rows g, g + 8, g + 16, g + 24
 #pragma unroll
-  for (int k = 0; k < 4; ++k) v.sw[k] = *reinterpret_cast<const float4*>(sc + LQ_BM + col_at + 16 * k);
-  return v;
+  for (int k = 0; k < 4; ++k) v.sw[k] = *reinterpret_cast<const float4*>(__cvta_shared_to_generic(sw_at + 64 * k));
 }
 // Two orders of the same products.  The codes' sums have 12 bits and the fp16 scales 11, so P sx and sx sw are exact alike and every FMA
 // rounds the same number; P sx leaves an FMA with an operand (sw) that four rows in a row share, which costs the register file
@@ -153,38 +154,39 @@ __device__ __forceinline__ void fetch_group(uint32_t taddr, Frag (&v)[4]) {
 }
 
 // A group's two MMAs under one election, predicated instead of branched around: the control flow of the issuing warp stays uniform.
-// (Against an `if` of one lane around them and around the commits, us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 68.9 / 78.5 -> 64.6 /
-// 73.2: a stage's way through the issuer, 1.2 k clocks, was as long as the drain's.)
+// (An `if` of one lane around them and around the commits, with a loop over the groups: a stage's way through the issuer, 1.2 k clocks,
+// was as long as the drain's.  us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 70.5 / 80.0 -> 64.7 / 71.3.)
+#define LQ_GROUP_MMAS                                                   \
+  "{\n\t.reg .pred P, T, F;\n\t"                                       \
+  "elect.sync _|P, 0xffffffff;\n\t"                                    \
+  "setp.eq.b32 T, 0, 0;\n\t"                                           \
+  "setp.ne.b32 F, 0, 0;\n\t"                                           \
+  "@P tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %3, %5, F;\n\t"  \
+  "@P tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %2, %4, %5, T;\n\t"
 __device__ __forceinline__ void issue_group(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred P, T, F;\n\t"
-      "elect.sync _|P, 0xffffffff;\n\t"
-      "setp.eq.b32 T, 0, 0;\n\t"
-      "setp.ne.b32 F, 0, 0;\n\t"
-      "@P tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %3, %5, F;\n\t"
-      "@P tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %2, %4, %5, T;\n\t}"
-      ::"r"(d), "l"(a), "l"(a + 2), "l"(b), "l"(b + 2), "r"(idesc)
-      : "memory");
+  asm volatile(LQ_GROUP_MMAS "}" ::"r"(d), "l"(a), "l"(a + 2), "l"(b), "l"(b + 2), "r"(idesc) : "memory");
 }
-__device__ __forceinline__ void issue_commits(uint32_t first, uint32_t second) {
-  asm volatile(
-      "{\n\t.reg .pred P;\n\t"
-      "elect.sync _|P, 0xffffffff;\n\t"
-      "@P tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t"
-      "@P tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}"
-      ::"r"(first), "r"(second)
-      : "memory");
+// a stage's last group: and the commits
+__device__ __forceinline__ void issue_group(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t bar_group, uint32_t bar_stage) {
+  asm volatile(LQ_GROUP_MMAS
+               "@P tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t"
+               "@P tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n\t}"
+               ::"r"(d), "l"(a), "l"(a + 2), "l"(b), "l"(b + 2), "r"(idesc), "r"(bar_group), "r"(bar_stage)
+               : "memory");
 }
 
 enum { BRANCH_NONE = 0, BRANCH_I8 = 1, BRANCH_F16 = 2 };
+enum { TILE_WHOLE = 0, TILE_SECTORS = 1, TILE_SPLIT = 2 };
 
-// SPLIT: the CTAs of a cluster share one tile, each with a part of the stages (K and the branch); their partial sums meet in
-// distributed shared memory.
-template <int BRANCH, bool SPLIT>
+// TILE_SPLIT: the CTAs of a cluster share one tile, each with a part of the stages (K and the branch); their partial sums meet in
+// distributed shared memory.  TILE_SECTORS: every row of Y begins on a 32-byte boundary.  (An instance of its own: with both kinds of
+// stores in one epilogue the drain's registers were worse allocated: 63.6 / 69.4 us for 62.3 / 69.0, M = 8192, K x N = 1152 x 3456 / 4608 x 1152.)
+template <int BRANCH, int TILE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
                const GemmParams p) {
+  constexpr bool SPLIT = TILE == TILE_SPLIT, SECTORS = TILE == TILE_SECTORS;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base - smem_u32(smem_raw));
@@ -326,28 +328,31 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           LQ_TL(EV_M_STAGE_FULL, s);
           const uint32_t a_addr = sm_stage + st * STAGE_BYTES, b_addr = a_addr + STAGE_A_BYTES;
           const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(b_addr);
-          const bool is_main = s < p.n_stages_main;
           // The stage's groups to the accumulators of one pair, each as soon as the drain has read it out; one commit
-          const int ngroups = is_main ? 2 : 1, pair = it & (NPAIR - 1);
-          for (int q = 0; q < ngroups && ok; ++q) {
-            ok = mbar_wait_warp(bar_tempty(2 * pair + q), ((it / NPAIR) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
+          const int pair = it & (NPAIR - 1);
+          const uint32_t d = tmem_base + 2 * pair * TCOLS, par = ((it / NPAIR) & 1) ^ 1;
+          ok = mbar_wait_warp(bar_tempty(2 * pair), par, abort_flag, p.status, LQ_STAGE_MMA);
+          if (!ok) break;
+          tc_fence_after();
+          LQ_TL(EV_M_ACC_FREE, s);
+          if (s < p.n_stages_main) {
+            issue_group(d, adesc, bdesc, IDESC_F8 | shape);
+            ok = mbar_wait_warp(bar_tempty(2 * pair + 1), par, abort_flag, p.status, LQ_STAGE_MMA);
             if (!ok) break;
             tc_fence_after();
             LQ_TL(EV_M_ACC_FREE, s);
-            const uint32_t d = tmem_base + (2 * pair + q) * TCOLS;
-            if (is_main) {
-              issue_group(d, adesc + 4 * q, bdesc + 4 * q, IDESC_F8 | shape);
-            } else {
-              if (elect_one())
-                for (int j = 0; j < p.branch_mmas; ++j) {
-                  if (BRANCH == BRANCH_F16) tc_mma<TC_F16>(d, adesc + 2 * j, bdesc + 2 * j, IDESC_F16 | shape, (uint32_t)j);
-                  else tc_mma<TC_I8>(d, adesc + 2 * j, bdesc + 2 * j, IDESC_I8 | shape, (uint32_t)j);
-                }
-              __syncwarp();
+            issue_group(d + TCOLS, adesc + 4, bdesc + 4, IDESC_F8 | shape, bar_tfull(pair), bar_empty(st));
+          } else {
+            if (elect_one()) {
+              for (int j = 0; j < p.branch_mmas; ++j) {
+                if (BRANCH == BRANCH_F16) tc_mma<TC_F16>(d, adesc + 2 * j, bdesc + 2 * j, IDESC_F16 | shape, (uint32_t)j);
+                else tc_mma<TC_I8>(d, adesc + 2 * j, bdesc + 2 * j, IDESC_I8 | shape, (uint32_t)j);
+              }
+              tc_commit(bar_tfull(pair));
+              tc_commit(bar_empty(st));
             }
+            __syncwarp();
           }
-          if (!ok) break;
-          issue_commits(bar_tfull(pair), bar_empty(st));
           LQ_TL(EV_M_ISSUED, s);
         }
       }
@@ -378,8 +383,10 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_tempty(2 * (i & (NPAIR - 1)) + q));
     };
-    auto scales_at = [&](uint32_t i, int q) {
-      return load_scales(sc_ptr + (i & (SC_RING - 1)) * (SC_STAGE_BYTES / 4) + q * SC_GROUP_FLOATS, row_at, col_at);
+    Scales sc;
+    auto load_scales_of = [&](uint32_t i, int q) {
+      const uint32_t at = sm_sc + (i & (SC_RING - 1)) * SC_STAGE_BYTES + q * SC_GROUP_FLOATS * 4;
+      load_scales(sc, at + row_at * 4, at + (LQ_BM + col_at) * 4);
     };
     grid_dependency_wait();                             // Y may be what an earlier kernel still reads
     open_stage(0, u_begin < u_end);
@@ -410,13 +417,13 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int s = s_begin; s < s_main && ok; ++s, ++it) {
         const bool more = s + 1 < s_end || !last_tile;
         LQ_TL(EV_D_OPEN, s);
-        Scales sc = scales_at(it, 0);
+        load_scales_of(it, 0);
         landed(it, 0);
         LQ_TL(EV_D_WAITED, s);
         fetch_group(pair_at(it) + TCOLS, vb);
         drain_group<false>(va, acc, sc);
         LQ_TL(EV_D_HALF, s);
-        sc = scales_at(it, 1);
+        load_scales_of(it, 1);
         landed(it, 1);
         LQ_TL(EV_D_LOADED, s);
         open_stage(it + 1, more);
@@ -427,7 +434,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!ok) break;
       if (BRANCH != BRANCH_NONE && (!SPLIT || s_end > p.n_stages_main)) {
-        const Scales sc = scales_at(it, 0);
+        load_scales_of(it, 0);
         landed(it, 0);
         if (lane == 0) mbar_arrive(bar_tempty(2 * (it & (NPAIR - 1)) + 1));   // not used by this stage
         drain_group<BRANCH == BRANCH_I8>(va, acc, sc);
@@ -471,7 +478,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                   w[2 * j] = __float_as_uint(acc[h][8 * k + 2 * j + i].x);
                   w[2 * j + 1] = __float_as_uint(acc[h][8 * k + 2 * j + i].y);
                 }
-                if (c + 8 * k < p.N) stg_32(Y + 8 * k, w, p.wide);
+                if (c + 8 * k < p.N) stg_32<SECTORS>(Y + 8 * k, w);
               }
             } else {
               __half* Y = reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c;
@@ -481,7 +488,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const __half2 q = __floats2half2_rn(acc[h][2 * j + i].x, acc[h][2 * j + i].y);
                 w[j] = *reinterpret_cast<const uint32_t*>(&q);
               }
-              if (p.wide) {                               // (N is then a multiple of 16)
+              if constexpr (SECTORS) {                      // (N is then a multiple of 16)
                 if (c < p.N) stg_v8(Y, w);
               } else {
                 if (c < p.N) *reinterpret_cast<uint4*>(Y) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -581,8 +588,9 @@ lq_status lq_launch_wait_probe(int device, cudaStream_t st) {
 
 lq_status lq_gemm_prepare(int device) {
   if (cudaSetDevice(device) != cudaSuccess) return LQ_ERR_CUDA;
-  for (auto* kernel : {lq_gemm_kernel<BRANCH_NONE, false>, lq_gemm_kernel<BRANCH_I8, false>, lq_gemm_kernel<BRANCH_F16, false>,
-                       lq_gemm_kernel<BRANCH_NONE, true>, lq_gemm_kernel<BRANCH_I8, true>, lq_gemm_kernel<BRANCH_F16, true>})
+  for (auto* kernel : {lq_gemm_kernel<BRANCH_NONE, TILE_WHOLE>, lq_gemm_kernel<BRANCH_I8, TILE_WHOLE>, lq_gemm_kernel<BRANCH_F16, TILE_WHOLE>,
+                       lq_gemm_kernel<BRANCH_NONE, TILE_SECTORS>, lq_gemm_kernel<BRANCH_I8, TILE_SECTORS>, lq_gemm_kernel<BRANCH_F16, TILE_SECTORS>,
+                       lq_gemm_kernel<BRANCH_NONE, TILE_SPLIT>, lq_gemm_kernel<BRANCH_I8, TILE_SPLIT>, lq_gemm_kernel<BRANCH_F16, TILE_SPLIT>})
     if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return LQ_ERR_CUDA;
   // once per device: launches of other threads read g_clusters without the lock, each after its own layer's upload came through here
   static std::mutex mu;
@@ -595,7 +603,7 @@ lq_status lq_gemm_prepare(int device) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2u << i; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     lc.gridDim = dim3(2u << i); lc.blockDim = dim3(GEMM_THREADS); lc.dynamicSmemBytes = SMEM_BYTES; lc.attrs = at; lc.numAttrs = 1;
-    if (lq_note_cuda(cudaOccupancyMaxActiveClusters(&g_clusters[device & 63][i], lq_gemm_kernel<BRANCH_I8, true>, &lc)) != cudaSuccess)
+    if (lq_note_cuda(cudaOccupancyMaxActiveClusters(&g_clusters[device & 63][i], lq_gemm_kernel<BRANCH_I8, TILE_SPLIT>, &lc)) != cudaSuccess)
       return LQ_ERR_CUDA;
   }
   done[device & 63] = true;
@@ -613,7 +621,6 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   p.units_n = L->Npad / UNIT;
   p.sx = A->d_sx; p.sw = L->d_sw; p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
   p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
-  p.wide = lq_rows_of_sectors(Y, L->N, dt);
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;
   int sms = 0;
@@ -623,11 +630,12 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   // (by the whole call's rows, so that a row's sums are the same in every chunk of it)
   p.split = pick_split(A->device, A->M_call, (long long)lq_ceil_div(A->M_call, LQ_BM) * p.units_n, p.n_stages_main + (L->r > 0), ctas);
   ctas = (int)std::min<long long>(ctas, units * p.split);
-  auto kernel = [&](auto split) {
-    constexpr bool S = decltype(split)::value;
-    return L->r == 0 ? lq_gemm_kernel<BRANCH_NONE, S> : L->f16_branch ? lq_gemm_kernel<BRANCH_F16, S> : lq_gemm_kernel<BRANCH_I8, S>;
+  auto kernel = [&](auto tile) {
+    constexpr int T = decltype(tile)::value;
+    return L->r == 0 ? lq_gemm_kernel<BRANCH_NONE, T> : L->f16_branch ? lq_gemm_kernel<BRANCH_F16, T> : lq_gemm_kernel<BRANCH_I8, T>;
   };
-  const cudaError_t e = lq_launch_cluster(p.split > 1 ? kernel(std::true_type()) : kernel(std::false_type()), ctas, GEMM_THREADS, p.split,
-                                          SMEM_BYTES, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
+  auto* k = p.split > 1 ? kernel(std::integral_constant<int, TILE_SPLIT>())
+                        : lq_rows_of_sectors(Y, L->N, dt) ? kernel(std::integral_constant<int, TILE_SECTORS>()) : kernel(std::integral_constant<int, TILE_WHOLE>());
+  const cudaError_t e = lq_launch_cluster(k, ctas, GEMM_THREADS, p.split, SMEM_BYTES, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -500,7 +500,9 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               uint32_t o[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) o[j] = __float_as_uint(y[j]);
-              stg_32(reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c, o, p.wide);
+              float* Y = reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c;
+              if (p.wide) stg_32<true>(Y, o);
+              else stg_32<false>(Y, o);
             } else {
               uint32_t o[4];
 #pragma unroll
