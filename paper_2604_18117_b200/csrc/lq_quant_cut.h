@@ -60,11 +60,14 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 // Cost model in rounds, a round being one chunk for every team: a CTA's tiles times (its rounds,
 // twice where a tile is walked twice, plus three for starting and finishing a tile).  It prices rounds only: not the second stream of X
 // where an integer branch's tile is larger than the ring (140 MB read for 75 at M = 8192, K = 4608), nor what overlaps between tiles.
-// Of cuts with the same rounds the one with the longer chunks (up to four stages) and so the fewer teams is taken, where a slot's
-// operands are small enough (integer branches, MXFP up to rank 64) to leave the ring its depth; the others lose up to 5 % by it.
-// Timed over every cut of up to four stages, eight formats, K from 264 to 8192 and M from 1 to 32768: with one round for a tile instead of three
-// and no word on chunks 150 of 464 sizes had another cut, 7 % slower in the mean (us, M = 32768, SINT4 rank 32, K = 1152 / 4608: 39.1 -> 37.1, 129.7
-// -> 116.3; M = 4096, MXINT4, K = 4608: 22.1 -> 18.7; M = 8192, MXFP rank 64, K = 4608: 25.4 -> 23.9).
+// Of cuts with the same rounds the one with the most warps and then the longer chunks (up to four stages) is taken, where a slot's
+// operands are small enough (integer branches, MXFP up to rank 64; the others lose up to 5 % by it) and K has the eight stages that fill
+// two such chunks.  Two exceptions of an integer branch, whose ring the long chunks shrink: a ring of two chunks (from five row groups on; us,
+// M = 17600, rank 128, K = 1280 / 1664, chunks of 1 and of 3 stages: 27.6 and 31.2 / 33.4 and 37.6), and chunks of two
+// stages where K has an odd number of them (M = 32768, rank 32, K = 1408, chunks of 1 and of 2 stages: 41.1 and 42.7; above rank 48 and from
+// 1536 on, or from 24 stages on, they are the faster ones all the same).  Elsewhere they may even make a tile too large for the ring: M = 32768, K = 1536, rank 64,
+// X streamed once by chunks of 1 and twice by chunks of 2: 49.1 and 45.8.
+// Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold).
 //
 // Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
 // one: the chunk that was in the slot before has to be known to have landed (X) or to have been multiplied (operands).
@@ -104,9 +107,10 @@ inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int f
         c.smem = quant_smem(br, 8 * groups, stages, rn, bplanes, c.slots, c.xslots).total + 1024;
         const int warps = groups * stages * c.teams;
         const double round = 0.4 + 0.6 * warps / QWARPS;
-        const bool longer = br == BR_INT || (br == BR_MXFP && rn <= 64);
+        const bool shallow = c.xslots < 3 && groups > 4, uneven = stages == 2 && nst % 2 != 0 && nst < 24 && (rn <= 48 || nst < 12);
+        const bool longer = nst >= 8 && stages <= 4 && (br == BR_INT ? !shallow && !uneven : br == BR_MXFP && rn <= 64);
         const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + 3.0) + 3.0 -
-                            (longer && nst >= 8 && stages <= 4 ? 1e-3 * stages : 0.0);
+                            (longer ? 1e-3 * (warps + stages) : 0.0);
         if (cost < best - 1e-9) { best = cost; out = c; }
         break;
       }

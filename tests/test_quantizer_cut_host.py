@@ -138,3 +138,32 @@ def test_every_value_of_the_options_gives_a_cut(cut):
             seen.setdefault((br, c["teams"], c["nchunks"], c["slots"], c["xslots"], c["refetch"]), c)
     wrong = [(key, m) for key, c in seen.items() if (m := _mistaken(key[0], c, tiles=2)) is not None]
     assert not wrong, wrong[:5]
+
+
+def _rounds(br, c):
+    """A launch in rounds (one chunk for every team) of so many warps: what the cost model compares."""
+    return -(-c["ntiles"] // 148) * -(-c["nchunks"] // c["teams"]), c["groups"] * c["stages"] * c["teams"]
+
+
+def test_long_chunks_leave_an_integer_branch_its_ring(cut):
+    """A cut that is taken for its longer chunks alone has no ring of two large chunks, and it gives up a ring that would hold the whole
+    tile (so that X is streamed twice) only for chunks that K fills, or where the factors are wide and K is long."""
+    for rn, M, nst in itertools.product(range(16, 129, 16), (1, 1000, 4096, 8192, 16384, 17600, 32768), range(8, 65)):
+        c = cut(INT, M, nst, rn)
+        equal = [a for g, s in itertools.product(range(1, 9), range(1, 5)) if (a := cut(INT, M, nst, rn, 1, g, s))["groups"] == c["groups"]
+                 and a["stages"] == s < c["stages"] and _rounds(INT, a) == _rounds(INT, c)]
+        if c["stages"] <= 4 and equal:
+            assert c["xslots"] >= 3 or c["groups"] <= 4, (rn, M, nst, c)
+            if c["refetch"] and not all(a["refetch"] for a in equal):
+                assert c["stages"] > 2 or nst % 2 == 0 or (rn > 48 and nst >= 12), (rn, M, nst, c)
+
+
+# (branch kind, rows, stages of K, columns of the first factor) -> row groups and stages of the cut timed as the fastest there
+TIMED = [((INT, 8192, 11, 32), (7, 1)), ((INT, 32768, 11, 32), (7, 1)), ((INT, 32768, 12, 64), (7, 2)), ((INT, 8192, 9, 96), (7, 1)), ((INT, 17600, 10, 128), (5, 1)),
+         ((INT, 17600, 13, 128), (5, 1)), ((INT, 1365, 44, 32), (2, 7)), ((INT, 2048, 8, 48), (2, 4)), ((INT, 4096, 18, 48), (4, 3)), ((INT, 3000, 13, 128), (3, 4))]
+
+
+@pytest.mark.parametrize("size,best", TIMED)
+def test_cuts_that_were_timed_as_the_fastest(cut, size, best):
+    c = cut(*size)
+    assert (c["groups"], c["stages"]) == best
