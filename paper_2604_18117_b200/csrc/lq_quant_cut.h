@@ -67,6 +67,9 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 // stages where K has an odd number of them (M = 32768, rank 32, K = 1408, chunks of 1 and of 2 stages: 41.1 and 42.7; above rank 48 and from
 // 1536 on, or from 24 stages on, they are the faster ones all the same).  Elsewhere they may even make a tile too large for the ring: M = 32768, K = 1536, rank 64,
 // X streamed once by chunks of 1 and twice by chunks of 2: 49.1 and 45.8.
+// Eight row groups leave room for one team of eight warps with nothing to run beside its waits: a tenth more a round (SINT4 rank 32, M = 17600, K = 640 / 896:
+// 16.2 / 19.0 us by 5 groups, 17.4 / 21.6 by 8).  With the widest factors, which every tile fetches anew, their fewer tiles make up for it (rank 128, K = 384: 18.5
+// and 15.8).
 // Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold).
 //
 // Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
@@ -106,7 +109,7 @@ inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int f
         c.refetch = br == BR_INT && c.xslots < c.nchunks;
         c.smem = quant_smem(br, 8 * groups, stages, rn, bplanes, c.slots, c.xslots).total + 1024;
         const int warps = groups * stages * c.teams;
-        const double round = 0.4 + 0.6 * warps / QWARPS;
+        const double round = 0.4 + 0.6 * warps / QWARPS + (groups == 8 && rn <= 96 ? 0.1 : 0.0);
         const bool shallow = c.xslots < 3 && groups > 4, uneven = stages == 2 && nst % 2 != 0 && nst < 24 && (rn <= 48 || nst < 12);
         const bool longer = nst >= 8 && stages <= 4 && (br == BR_INT ? !shallow && !uneven : br == BR_MXFP && rn <= 64);
         const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + 3.0) + 3.0 -
