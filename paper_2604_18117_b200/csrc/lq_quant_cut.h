@@ -58,7 +58,8 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 }
 
 // Cost model in rounds, a round being one chunk for every team: a CTA's tiles times (its rounds,
-// twice where a tile is walked twice, plus three for starting and finishing a tile).  It prices rounds only: not the second stream of X
+// twice where a tile is walked twice, plus three for starting and finishing a tile, or one without a branch: no factor, sums or re-quantization wait there,
+// and with three M = 22000, K = 1152 took 17.7 / 13.7 us, caches cold / warm, for 16.5 / 13.1).  It prices rounds only: not the second stream of X
 // where an integer branch's tile is larger than the ring (140 MB read for 75 at M = 8192, K = 4608), nor what overlaps between tiles.
 // Of cuts with the same rounds the one with the most warps and then the longer chunks (up to four stages) is taken, where a slot's
 // operands are small enough (integer branches, MXFP up to rank 64; the others lose up to 5 % by it) and K has the eight stages that fill
@@ -70,7 +71,9 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 // Eight row groups leave room for one team of eight warps with nothing to run beside its waits: a tenth more a round (SINT4 rank 32, M = 17600, K = 640 / 896:
 // 16.2 / 19.0 us by 5 groups, 17.4 / 21.6 by 8).  With the widest factors, which every tile fetches anew, their fewer tiles make up for it (rank 128, K = 384: 18.5
 // and 15.8).
-// Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold).
+// Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold): with one
+// round for every tile and no word on chunks and eight groups 3842 of them had another cut, 6.3 % slower in the mean; 90 were more than 1.5 % faster with it, by 9 % at most
+// (26 by more than 4 %: factors of up to 32 columns at K above 5000, tiles of 40 or 48 rows for 24 or 16, and a few of seven or eight groups).
 //
 // Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
 // one: the chunk that was in the slot before has to be known to have landed (X) or to have been multiplied (operands).
@@ -82,6 +85,7 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 //             chunk up to the one before had been multiplied).
 inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int force_groups, int force_stages, QuantCut& out) {
   const int walks = br == BR_INT ? 2 : 1, room = 227 * 1024 - 1024;
+  const double per_tile = br == BR_NONE ? 1.0 : 3.0;
   double best = 1e30;
   for (int groups = 8; groups >= 1; --groups) {
     if (force_groups > 0 && groups != force_groups) continue;
@@ -112,7 +116,7 @@ inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int f
         const double round = 0.4 + 0.6 * warps / QWARPS + (groups == 8 && rn <= 96 ? 0.1 : 0.0);
         const bool shallow = c.xslots < 3 && groups > 4, uneven = stages == 2 && nst % 2 != 0 && nst < 24 && (rn <= 48 || nst < 12);
         const bool longer = nst >= 8 && stages <= 4 && (br == BR_INT ? !shallow && !uneven : br == BR_MXFP && rn <= 64);
-        const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + 3.0) + 3.0 -
+        const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + per_tile) + 3.0 -
                             (longer ? 1e-3 * (warps + stages) : 0.0);
         if (cost < best - 1e-9) { best = cost; out = c; }
         break;
