@@ -63,17 +63,19 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 // where an integer branch's tile is larger than the ring (140 MB read for 75 at M = 8192, K = 4608), nor what overlaps between tiles.
 // Of cuts with the same rounds the one with the most warps and then the longer chunks (up to four stages) is taken, where a slot's
 // operands are small enough (integer branches, MXFP up to rank 64; the others lose up to 5 % by it) and K has the eight stages that fill
-// two such chunks.  Two exceptions of an integer branch, whose ring the long chunks shrink: a ring of two chunks (from five row groups on; us,
+// two such chunks.  Exceptions.  An integer branch, whose ring the long chunks shrink: a ring of two chunks (from five row groups on; us,
 // M = 17600, rank 128, K = 1280 / 1664, chunks of 1 and of 3 stages: 27.6 and 31.2 / 33.4 and 37.6), and chunks of two
 // stages where K has an odd number of them (M = 32768, rank 32, K = 1408, chunks of 1 and of 2 stages: 41.1 and 42.7; above rank 48 and from
 // 1536 on, or from 24 stages on, they are the faster ones all the same).  Elsewhere they may even make a tile too large for the ring: M = 32768, K = 1536, rank 64,
 // X streamed once by chunks of 1 and twice by chunks of 2: 49.1 and 45.8.
+// MXFP: chunks of two of an odd number below twelve where a CTA has one tile, whose first chunk nothing covers (rank 64, M = 8192, K = 1152, caches cold: 11.16
+// by chunks of 1, 11.43 of 2).
 // Eight row groups leave room for one team of eight warps with nothing to run beside its waits: a tenth more a round (SINT4 rank 32, M = 17600, K = 640 / 896:
 // 16.2 / 19.0 us by 5 groups, 17.4 / 21.6 by 8).  With the widest factors, which every tile fetches anew, their fewer tiles make up for it (rank 128, K = 384: 18.5
 // and 15.8).
-// Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold): with one
-// round for every tile and no word on chunks and eight groups 3842 of them had another cut, 6.3 % slower in the mean; 90 were more than 1.5 % faster with it, by 9 % at most
-// (26 by more than 4 %: factors of up to 32 columns at K above 5000, tiles of 40 or 48 rows for 24 or 16, and a few of seven or eight groups).
+// Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold): by one
+// round for every tile and none of these rules 3824 of them get another cut, which is 6.3 % slower in the mean; 84 get one that is more than 1.5 % faster, 9 % at
+// most (26 more than 4 %: factors of up to 32 columns at K above 5000, tiles of 16 or 24 rows instead of 40 or 48, and a few instead of seven or eight groups).
 //
 // Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
 // one: the chunk that was in the slot before has to be known to have landed (X) or to have been multiplied (operands).
@@ -114,8 +116,8 @@ inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int f
         c.smem = quant_smem(br, 8 * groups, stages, rn, bplanes, c.slots, c.xslots).total + 1024;
         const int warps = groups * stages * c.teams;
         const double round = 0.4 + 0.6 * warps / QWARPS + (groups == 8 && rn <= 96 ? 0.1 : 0.0);
-        const bool shallow = c.xslots < 3 && groups > 4, uneven = stages == 2 && nst % 2 != 0 && nst < 24 && (rn <= 48 || nst < 12);
-        const bool longer = nst >= 8 && stages <= 4 && (br == BR_INT ? !shallow && !uneven : br == BR_MXFP && rn <= 64);
+        const bool shallow = c.xslots < 3 && groups > 4, uneven = stages == 2 && nst % 2 != 0 && (br == BR_INT ? nst < 24 && (rn <= 48 || nst < 12) : nst < 12 && c.ntiles <= sms);
+        const bool longer = nst >= 8 && stages <= 4 && !uneven && (br == BR_INT ? !shallow : br == BR_MXFP && rn <= 64);
         const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + per_tile) + 3.0 -
                             (longer ? 1e-3 * (warps + stages) : 0.0);
         if (cost < best - 1e-9) { best = cost; out = c; }

@@ -162,6 +162,7 @@ def test_long_chunks_leave_an_integer_branch_its_ring(cut):
 TIMED = [((INT, 8192, 11, 32), (7, 1)), ((INT, 32768, 11, 32), (7, 1)), ((INT, 32768, 12, 64), (7, 2)), ((INT, 8192, 9, 96), (7, 1)), ((INT, 17600, 10, 128), (5, 1)),
          ((INT, 17600, 13, 128), (5, 1)), ((INT, 1365, 44, 32), (2, 7)), ((INT, 2048, 8, 48), (2, 4)), ((INT, 4096, 18, 48), (4, 3)), ((INT, 3000, 13, 128), (3, 4)),
          ((INT, 17600, 7, 32), (5, 1)), ((INT, 17600, 5, 32), (5, 1)), ((INT, 26000, 7, 96), (6, 1)), ((INT, 17600, 3, 128), (8, 1)),
+         ((MXFP, 8192, 9, 64), (7, 1)), ((MXFP, 7000, 11, 32), (6, 1)), ((MXFP, 16384, 9, 64), (7, 2)),
          ((NONE, 22000, 9, 16), (5, 1)), ((NONE, 17600, 8, 16), (5, 1)), ((NONE, 26000, 12, 16), (5, 1))]
 
 
