@@ -618,9 +618,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     uint32_t par = 1, issued = 0;
     bool ok = true;
     const int walks = BR == BR_INT && p.refetch ? 2 : 1;
-    // X read for the last time is the first to leave the L2, before the codes, which the GEMM comes for next (us a block, M = 8192, other
-    // inputs each time: MXINT4 198.9 -> 193.7, MXFP4 170.0 -> 167.3, MXINT4 x 8 274.5 -> 272.4, SINT4 344.7 -> 343.2)
-    const uint64_t last_read = l2_evict_first(), read_again = l2_evict_normal();
+    const uint64_t policy = p.drop_x ? l2_evict_first() : l2_evict_normal();       // (x_leaves_first)
     for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x)
       for (int w = 0; w < walks && ok; ++w)
         for (int c = 0; c < p.nchunks; ++c) {
@@ -630,8 +628,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             const int nb = 2 * min(spc, p.nst - c * spc);
             mbar_expect_tx(bar_xfull(xs), (uint32_t)(nb * TR * 128));
             for (int b = 0; b < nb; ++b)
-              tma_load_2d_hint(base + (uint32_t)(xs * sm.xslot + b * TR * 128), &tmX, (2 * c * spc + b) * 128, tile * TR, bar_xfull(xs),
-                               w + 1 == walks ? last_read : read_again);
+              tma_load_2d_hint(base + (uint32_t)(xs * sm.xslot + b * TR * 128), &tmX, (2 * c * spc + b) * 128, tile * TR, bar_xfull(xs), policy);
           }
           __syncwarp();
           ++issued;
@@ -1092,6 +1089,7 @@ cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, i
     attr_set[dev & 63] = true;
   }
   if (!plan_cut_as_asked(BR, p.M, p.nst, p.rn, p.bplanes, sms, g_lq_quant_warps, g_lq_quant_ctas, p)) return cudaErrorInvalidConfiguration;
+  p.drop_x = x_leaves_first(p, MAIN == MAIN_MXINT8, (double)p.M * (2.0 * p.K + p.Kpad));
   // Floating-point branches: a tile's stages alternate over up to four accumulators, which are added in fp32 at the end
   // (each costs a4 a trip to tensor memory per 16 columns: not more than 128 columns of them).  Tensor memory holds two
   // such sets - one where every CTA has a single tile - and the scale bytes' columns.

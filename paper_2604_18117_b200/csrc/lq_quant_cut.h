@@ -23,6 +23,7 @@ struct QuantCut {
   int slots, xslots;    // chunk slots of the branch's operands and of X
   int refetch;          // integer branch: the X ring is smaller than a tile, which is streamed twice
   int smem;             // dynamic shared memory of the launch
+  int drop_x;           // X is the first to leave the L2 (x_leaves_first)
 };
 
 // Shared memory, from a 1024-byte aligned base; the same arithmetic on the host (size) and in the kernel.  First the X ring,
@@ -74,7 +75,7 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 // 16.2 / 19.0 us by 5 groups, 17.4 / 21.6 by 8).  With the widest factors, which every tile fetches anew, their fewer tiles make up for it (rank 128, K = 384: 18.5
 // and 15.8).
 // Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold): by one
-// round for every tile and none of these rules 3824 of them get another cut, which is 6.3 % slower in the mean; 84 get one that is more than 1.5 % faster, 9 % at
+// round for every tile and none of these rules 3830 of them get another cut, which is 6.4 % slower in the mean; 84 get one that is more than 1.5 % faster, 9 % at
 // most (26 more than 4 %: factors of up to 32 columns at K above 5000, tiles of 16 or 24 rows instead of 40 or 48, and a few instead of seven or eight groups).
 //
 // Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
@@ -139,6 +140,20 @@ inline bool plan_cut_as_asked(int br, int M, int nst, int rn, int bplanes, int s
     if (g <= 1) break;
   }
   return plan_cut(br, M, nst, rn, bplanes, sms, 0, 0, out);
+}
+
+// Whether X is the first to leave the L2 (126 MB), before the codes, which the GEMM comes for next.  The launch cannot know whether somebody reads X
+// again - another layer, a residual sum - so it is so only where X and the codes (bytes) are too large to stay all the same, and then it costs nobody anything; nor
+// where an integer branch streams X twice itself.  Timed with and without over X and codes of 36 to 240 MB, K from 640 to 4608, four formats: quantizer and GEMM alone,
+// two layers in turn on one X, both quantizers first, X just written, X read again behind the GEMM.  Rank 32 / 64, K = 1152, N = 1152:
+//   X and codes   MXINT4: one layer, two, quantizers first, read again   MXFP4
+//     28 MB       0.972  1.010  1.019  1.014                             0.987  1.017  1.028  1.014   not taken (M = 8192)
+//     72 MB       0.986  0.986  0.984  0.988                             0.973  0.975  0.973  0.997   not taken (K = 4608: 0.981  0.997  1.005  0.996)
+//    125 MB       0.983  0.980  0.984  0.983                             0.986  0.987  0.982  0.982
+//    200 MB       0.996  0.982  1.001  0.997                             0.994  1.002  1.003  0.996   not taken (K = 4608: 0.981  0.989  1.008  0.994)
+// MXINT8's codes (two planes) are as large as X: both quantizers first lost 1.0 to 1.7 % at K = 4608, one layer won 1 to 2 %; it is left out.
+inline bool x_leaves_first(const QuantCut& c, bool two_planes, double x_and_codes) {
+  return !c.refetch && !two_planes && x_and_codes > 80e6 && x_and_codes < 160e6;
 }
 
 }  // namespace lqcut

@@ -19,6 +19,11 @@ extern "C" int cut(int br, int M, int nst, int rn, int planes, int groups, int s
   for (int i = 0; i < 9; ++i) out[i] = v[i];
   return 1;
 }
+extern "C" int leaves_first(int refetch, int two_planes, double bytes) {
+  lqcut::QuantCut c{};
+  c.refetch = refetch;
+  return lqcut::x_leaves_first(c, two_planes != 0, bytes);
+}
 """
 
 
@@ -32,10 +37,13 @@ def cut(tmp_path_factory):
                    check=True)
     lib = ctypes.CDLL(str(d / "cut.so"))
 
+    lib.leaves_first.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_double]
+
     def get(br, M, nst, rn, planes=1, groups=0, stages=0):
         out = (ctypes.c_int * 9)()
         return dict(zip(FIELDS, out)) if lib.cut(br, M, nst, rn, planes, groups, stages, out) else None
 
+    get.leaves_first = lambda c, M, K, planes=1: bool(lib.leaves_first(c["refetch"], planes == 2, M * (2.0 * K + planes * -(-K // 128) * 128)))
     return get
 
 
@@ -170,3 +178,12 @@ TIMED = [((INT, 8192, 11, 32), (7, 1)), ((INT, 32768, 11, 32), (7, 1)), ((INT, 3
 def test_cuts_that_were_timed_as_the_fastest(cut, size, best):
     c = cut(*size)
     assert (c["groups"], c["stages"]) == best
+
+
+@pytest.mark.parametrize("br,rn,planes,M,K,first", [
+    (INT, 32, 1, 8192, 1152, False), (INT, 32, 1, 16384, 1152, False), (INT, 32, 1, 32768, 1152, True), (INT, 32, 1, 8192, 4608, False),
+    (MXFP, 64, 1, 8192, 1152, False), (MXFP, 64, 1, 4096, 4608, False), (MXFP, 64, 1, 8192, 4608, True), (MXFP, 64, 1, 32768, 4608, False),
+    (MXINT, 64, 2, 8192, 4608, False)])
+def test_x_leaves_the_l2_first_only_where_it_would_not_stay(cut, br, rn, planes, M, K, first):
+    """What another layer or a residual sum may read again is not marked as read for the last time where the L2 could keep it."""
+    assert cut.leaves_first(cut(br, M, -(-K // 128), rn), M, K, planes) == first
