@@ -76,7 +76,10 @@ constexpr int GEMM_THREADS = (FIRST_DRAIN_WARP + NUM_DRAIN_WARPS) * 32;
 constexpr int WCOLS = 64;                          // columns per drain warp
 // 12 warps are launched with 168 registers a thread: 384 x 168 = 64512 = 128 x 56 + 256 x 224.  (216 for the drain: 64.6 / 73.1 us at the sizes
 // above for 62.7 / 69.6; 232 and 40: 64.1 / 71.5, the producer spills)
-constexpr int LEAN_REGS = 56, DRAIN_REGS = 224;
+constexpr int LAUNCH_REGS = 65536 / GEMM_THREADS & ~7, LEAN_REGS = 56, DRAIN_REGS = 224;
+// setmaxnreg takes from what the CTA was launched with and would wait for ever for more: the only wait without a limit, so its sum is
+// checked here and every instance's own count in lq_gemm_prepare
+static_assert(FIRST_DRAIN_WARP * 32 * LEAN_REGS + NUM_DRAIN_WARPS * 32 * DRAIN_REGS <= GEMM_THREADS * LAUNCH_REGS, "registers of the split");
 constexpr int SMEM_BAR_BYTES = 256;
 constexpr int SMEM_BYTES = 1024 /*alignment slack*/ + NSTAGE * STAGE_BYTES + SC_RING * SC_STAGE_BYTES + SMEM_BAR_BYTES;
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
@@ -590,8 +593,12 @@ lq_status lq_gemm_prepare(int device) {
   if (cudaSetDevice(device) != cudaSuccess) return LQ_ERR_CUDA;
   for (auto* kernel : {lq_gemm_kernel<BRANCH_NONE, TILE_WHOLE>, lq_gemm_kernel<BRANCH_I8, TILE_WHOLE>, lq_gemm_kernel<BRANCH_F16, TILE_WHOLE>,
                        lq_gemm_kernel<BRANCH_NONE, TILE_SECTORS>, lq_gemm_kernel<BRANCH_I8, TILE_SECTORS>, lq_gemm_kernel<BRANCH_F16, TILE_SECTORS>,
-                       lq_gemm_kernel<BRANCH_NONE, TILE_SPLIT>, lq_gemm_kernel<BRANCH_I8, TILE_SPLIT>, lq_gemm_kernel<BRANCH_F16, TILE_SPLIT>})
+                       lq_gemm_kernel<BRANCH_NONE, TILE_SPLIT>, lq_gemm_kernel<BRANCH_I8, TILE_SPLIT>, lq_gemm_kernel<BRANCH_F16, TILE_SPLIT>}) {
+    cudaFuncAttributes at;
+    if (lq_note_cuda(cudaFuncGetAttributes(&at, kernel)) != cudaSuccess) return LQ_ERR_CUDA;
+    if (at.numRegs < LAUNCH_REGS) return LQ_ERR_UNSUPPORTED;
     if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return LQ_ERR_CUDA;
+  }
   // once per device: launches of other threads read g_clusters without the lock, each after its own layer's upload came through here
   static std::mutex mu;
   static bool done[64] = {false};
