@@ -15,7 +15,7 @@
 //               and are handed over with one commit; two pairs alternate
 //   warps 4-11  drain: each warp owns 32 rows x 64 columns of the tile.  A group's slice is four tcgen05.ld.16x256b.x4; a
 //               whole group is in flight into one register buffer while the one before is consumed from the other:
-//               acc += P * (sx * sw), packed f32x2, fp32 registers.  An accumulator goes back as soon as it sits in
+//               acc += (P * sx) * sw, packed f32x2, fp32 registers (the integer branch's stage: P * (sx * sw)).  An accumulator goes back as soon as it sits in
 //               registers.  The next tile's first group is requested before the epilogue
 // What bounds it: the FP32 pipe's operand delivery and the drain's other instructions.  Per group and scheduler 64 packed products
 // (2.0 to 2.6 clocks each, measured) and 64 packed FMAs (2.75 with an operand shared by neighbours, 3.9 with three of their own) are about 320
@@ -24,8 +24,10 @@
 // wide warps per scheduler instead of four narrow ones, no wait or arrival for the scale vectors (they live in a ring deep
 // enough that the accumulators' hand-shakes imply theirs), one wait per stage, 224 registers per drain thread, partly
 // taken over from the other four warps (setmaxnreg).  M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 85 / 96 us with sixteen
-// narrow warps, 80 / 89 with one commit per group, 79 / 86 before P sx was taken first, sectors were stored whole, the issuer lost its
-// branches and the drain got its last eight registers.  Scalar FMAs lose their issue slots (94 - 104 us for 79); scales of
+// narrow warps, 80 / 89 with one commit per group; then, timed in turn with other inputs each time, 81.1 / 88.3, 78.0 / 84.0 with P sx first,
+// 72.4 / 81.6 with sectors stored whole, 70.1 / 78.1 with a stage's commits under one election, 64.5 / 70.9 with the issuer written out and the
+// drain's last eight registers.  At K = 1152 a tile's end is a fifth of the launch: of 11.4 k clocks a tile 1.0 k are the branch's group, 0.8 k the stores, 0.5 k
+// the way to the next tile's first stage.  Scalar FMAs lose their issue slots (94 - 104 us for 79); scales of
 // the next group loaded where this one's were used last, 302 clocks a group by itself, made the kernel slower (73.6 for 68.8: registers); two column
 // halves as pipelines of their own, each with an issuer, 67.9 for 66.5.
 // Orders of rows and columns (lq_internal.h) are chosen for the drain's fragments: the columns of the tile are permuted in
@@ -104,7 +106,7 @@ struct GemmParams {
 
 // One group's slice of a drain warp, two accumulator slices of 16 rows x 64 columns in the layout of tcgen05.ld.16x256b
 // (the accumulator-fragment layout of mma.sync m16n8: with g = lane / 4 and t = lane % 4, registers 4j .. 4j+3 of a
-// slice hold row g, columns 8j + 2t and 8j + 2t + 1, then row g + 8, the same columns): acc += P * (sx * sw).
+// slice hold row g, columns 8j + 2t and 8j + 2t + 1, then row g + 8, the same columns), times its scales, added to the accumulators.
 // INT: the accumulator holds int32 (kind::i8); |P| < 2^22, so adding 1.5 * 2^23 in the integer domain and subtracting it
 // in fp32 converts exactly without the conversion pipe.
 typedef uint32_t Frag[16];                            // 16 rows x 32 columns
@@ -125,7 +127,7 @@ __device__ __forceinline__ void load_scales(Scales& v, uint32_t sx_at, uint32_t 
 }
 // Two orders of the same products.  The codes' sums have 12 bits and the fp16 scales 11, so P sx and sx sw are exact alike and every FMA
 // rounds the same number; P sx leaves an FMA with an operand (sw) that four rows in a row share, which costs the register file
-// less (us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 79.2 / 86.4 -> 76.4 / 82.4).  The integer branch's scales have 24 bits, its sums up
+// less (us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 81.1 / 88.3 -> 78.0 / 84.0).  The integer branch's scales have 24 bits, its sums up
 // to 22: there sx sw is rounded first.
 template <bool INT>
 __device__ __forceinline__ void drain_group(const Frag (&v)[4], float2 (&acc)[2][16], const Scales& sc) {
@@ -158,7 +160,7 @@ __device__ __forceinline__ void fetch_group(uint32_t taddr, Frag (&v)[4]) {
 
 // A group's two MMAs under one election, predicated instead of branched around: the control flow of the issuing warp stays uniform.
 // (An `if` of one lane around them and around the commits, with a loop over the groups: a stage's way through the issuer, 1.2 k clocks,
-// was as long as the drain's.  us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 70.5 / 80.0 -> 64.7 / 71.3.)
+// was as long as the drain's.  us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 72.4 / 81.6 -> 64.5 / 70.9, with the drain's eight registers.)
 #define LQ_GROUP_MMAS                                                   \
   "{\n\t.reg .pred P, T, F;\n\t"                                       \
   "elect.sync _|P, 0xffffffff;\n\t"                                    \
@@ -463,7 +465,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       } else {
         // Epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad.  Two lanes' stores of 16
         // bytes never meet in a 32-byte sector here, so each would write half of one; where all of Y's rows are whole sectors a lane
-        // stores 32 bytes at once (us, M = 8192, K x N = 1152 x 3456: 79.3 -> 73.4).
+        // stores 32 bytes at once (us, M = 8192, K x N = 1152 x 3456: 78.0 -> 72.4).
         const int c = n0 + coff + 16 * ft;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
@@ -561,11 +563,14 @@ __global__ void lq_wait_probe_kernel(int32_t* status, long long limit) {
   mbar_wait_slow(bar, 0, &abort_word, status, LQ_STAGE_TEARDOWN, limit);
 }
 
-// CTAs per tile of a launch of few tiles (1, 2, 4 or 8).  A tile's stages are one serial chain, 0.52 us each, so while SMs are idle
-// they may as well share it; a cluster's launch and its two rendezvous cost 1.9 us, the exchange up to 0.15 us per CTA that is
-// read (M = 1, K x N = 1152 x 1152: 7.9 us alone, 5.4 by eight; M = 128, 8192 x 1152: 38 and 11.7; M = 256, 4608 x 1152: 23.2
-// and 11.4 by four).  The hardware places a cluster's CTAs next to each other, so fewer fit than there are SMs; a second
-// round of them would cost more than it gives.
+// CTAs per tile of a launch of few tiles (1, 2, 4 or 8).  A tile's stages are one serial chain, so while SMs are idle they may as well share
+// it; a cluster's launch, its two rendezvous and the exchange cost the rest (us now, alone and shared: M = 1, K x N = 1152 x 1152: 6.9 and 5.4 by
+// eight; M = 128, 8192 x 1152: 30.8 and 11.4 by eight; M = 256, 4608 x 1152: 18.9 and 11.0 by four).  The hardware places a cluster's CTAs next to each
+// other, so fewer fit than there are SMs; a second round of them would cost more than it gives.  The prices are those of the drain as it was, 0.52 us a stage and
+// 1.9 + 0.15 per CTA that is read; now a stage takes 0.43, a cluster 2.0 and, with full tiles, 0.55 + 0.26 per CTA more.  By those 34 of 40 sizes timed (K from 384 to 8192, M from
+// 1 to 512) are cut as here and 6, all of ten stages, would not be shared (M = 128, 1152 x 4608: 8.3 by two, 7.5 alone).  The line stays
+// where it was: shared sums are the shorter chains, and further from the exact sum is what those rows would be (that size, fp32 output: relative error
+// 6.0e-8 by two, 7.4e-8 alone).
 int g_clusters[64][3];                                // how many clusters of 2, 4, 8 the device holds at once
 int pick_split(int device, int M, long long units, int stages, int ctas) {
   int best = 1;

@@ -14,8 +14,8 @@
 //               stage.  A lane owns 16 neighbouring values of two rows, two 16-byte vectors of X each: they share a block and its
 //               scale, a block of 32 is two lanes, its maximum one shuffle, and a lane's codes are one 16-byte store, to global and
 //               to shared memory.  (With a vector of each half of the stage to a lane, four lanes to a block, every scale was worked
-//               out twice as often and stores were of 8 bytes; us, M = 8192, K = 1152 / 4608: SINT4 11.8 / 34.6 -> 11.3 / 32.8, MXINT4 x 8 12.7 /
-//               36.1 -> 11.1 / 33.6.)
+//               out twice as often and stores were of 8 bytes; us, timed in turn, M = 8192, K = 1152 / 4608, X cold: SINT4 13.8 / 37.4 -> 13.4 / 36.2,
+//               MXINT4 x 8 13.5 / 37.6 -> 12.9 / 34.2, MXFP4 11.1 / 28.4 -> 11.1 / 28.6; X in the L2: 12.1 / 35.0 -> 11.5 / 32.6, 12.5 / 37.7 -> 11.4 / 34.2.)
 //               Loads and stores move whole rows of a box.  (A first version loaded X into registers from global memory, half rows per
 //               instruction: the tag stage of the L1 was what bounded it, at 40 lookups a piece, and its unrolled ring
 //               cost a microsecond of instruction misses.)  The branch's operand goes to shared memory in the layout
@@ -915,7 +915,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             a[1] = lds_v4((xo_a + at) ^ 16); b[1] = lds_v4((xo_b + at) ^ 16);
           }
           uint2 wa[2], wb[2], da[2], db[2];                      // main codes of the two rows (MXINT8: hi digits; d: lo digits)
-          uint32_t four = 0;                                     // the stage's scale bytes of row sr (lanes 0 and 1 of a row)
+          uint32_t four = 0;                                     // the stage's scale bytes of row sr (a box's first lane has them)
           if constexpr (decltype(MAINP)::value) {
             if (live) {
               __half2 bm = __halves2half2(__hmax(absmax8(a[0]), absmax8(a[1])), __hmax(absmax8(b[0]), absmax8(b[1])));
