@@ -613,12 +613,12 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int qw = warp - FIRST_QWARP;
   if (warp == 3) {
     // ------------------------------------------------------------------ TMA producer: X
+    const uint64_t policy = p.drop_x ? l2_evict_first() : l2_evict_normal();       // (x_leaves_first; behind the wait it cost MXFP 0.2 us a launch)
     grid_dependency_wait();
     int xs = 0;
     uint32_t par = 1, issued = 0;
     bool ok = true;
     const int walks = BR == BR_INT && p.refetch ? 2 : 1;
-    const uint64_t policy = p.drop_x ? l2_evict_first() : l2_evict_normal();       // (x_leaves_first)
     for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x)
       for (int w = 0; w < walks && ok; ++w)
         for (int c = 0; c < p.nchunks; ++c) {
