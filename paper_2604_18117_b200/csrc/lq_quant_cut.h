@@ -64,7 +64,7 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 // where an integer branch's tile is larger than the ring (140 MB read for 75 at M = 8192, K = 4608), nor what overlaps between tiles.
 // Of cuts with the same rounds the one with the most warps and then the longer chunks (up to four stages) is taken, where a slot's
 // operands are small enough (integer branches, MXFP up to rank 64; the others lose up to 5 % by it) and K has the eight stages that fill
-// two such chunks.  Exceptions.  An integer branch, whose ring the long chunks shrink: a ring of two chunks (from five row groups on; us,
+// two such chunks (without that limit 44 more of the timed sizes are over 1.5 % slower than by short ones).  Exceptions.  An integer branch, whose ring the long chunks shrink: a ring of two chunks (from five row groups on; us,
 // M = 17600, rank 128, K = 1280 / 1664, chunks of 1 and of 3 stages: 27.6 and 31.2 / 33.4 and 37.6), and chunks of two
 // stages where K has an odd number of them (M = 32768, rank 32, K = 1408, chunks of 1 and of 2 stages: 41.1 and 42.7; above rank 48 and from
 // 1536 on, or from 24 stages on, they are the faster ones all the same).  Elsewhere they may even make a tile too large for the ring: M = 32768, K = 1536, rank 64,
