@@ -117,7 +117,8 @@ inline bool plan_cut(int br, int M, int nst, int rn, int bplanes, int sms, int f
         c.smem = quant_smem(br, 8 * groups, stages, rn, bplanes, c.slots, c.xslots).total + 1024;
         const int warps = groups * stages * c.teams;
         const double round = 0.4 + 0.6 * warps / QWARPS + (groups == 8 && rn <= 96 ? 0.1 : 0.0);
-        const bool shallow = c.xslots < 3 && groups > 4, uneven = stages == 2 && nst % 2 != 0 && (br == BR_INT ? nst < 24 && (rn <= 48 || nst < 12) : nst < 12 && c.ntiles <= sms);
+        const bool shallow = c.xslots < 3 && groups > 4;
+        const bool uneven = stages == 2 && nst % 2 != 0 && (br == BR_INT ? nst < 24 && (rn <= 48 || nst < 12) : nst < 12 && c.ntiles <= sms);
         const bool longer = nst >= 8 && stages <= 4 && !uneven && (br == BR_INT ? !shallow : br == BR_MXFP && rn <= 64);
         const double cost = lq_ceil_div(c.ntiles, sms) * (lq_ceil_div(c.nchunks, c.teams) * walks * round + per_tile) + 3.0 -
                             (longer ? 1e-3 * (warps + stages) : 0.0);
