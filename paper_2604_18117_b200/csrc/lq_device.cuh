@@ -26,11 +26,21 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// CLUSTER: arrivals come from another CTA of the cluster, too, and hand over tensor memory (peer_arrive).
-template <bool CLUSTER = false>
+// SCOPE: whose arrivals the wait is for.  PEER_TMEM: another CTA's of the cluster, too, which hand over tensor memory (peer_arrive).
+// PEER_DATA: copies of other CTAs into this one's shared memory (peer_copy), which the wait makes visible.
+enum { OWN_CTA = 0, PEER_TMEM = 1, PEER_DATA = 2 };
+template <int SCOPE = OWN_CTA>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
-  if constexpr (CLUSTER)
+  if constexpr (SCOPE == PEER_DATA)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+  else if constexpr (SCOPE == PEER_TMEM)
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
@@ -51,12 +61,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 
 // Bounded wait.  Returns false when the CTA is aborting or the deadline passed (then it raises the abort flag
 // and records who gave up in the device status word {code, stage}).
-template <bool CLUSTER = false>
+template <int SCOPE = OWN_CTA>
 static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                             int role, long long limit = WAIT_LIMIT_CYCLES) {
   const long long t0 = clock64();
   for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
+    if (mbar_try_wait<SCOPE>(bar, parity)) return true;
     if ((it & 0xFF) == 0) {
       if (*abort_flag) return false;
       if (clock64() - t0 > limit) {
@@ -67,11 +77,11 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity
     }
   }
 }
-template <bool CLUSTER = false>
+template <int SCOPE = OWN_CTA>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                           int role) {
-  if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
-  return mbar_wait_slow<CLUSTER>(bar, parity, abort_flag, status, role);
+  if (mbar_try_wait<SCOPE>(bar, parity)) return true;
+  return mbar_wait_slow<SCOPE>(bar, parity, abort_flag, status, role);
 }
 // The same wait without a call on its slow path: for a warp whose registers are full of data.
 __device__ __forceinline__ bool mbar_wait_inline(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int role) {
@@ -90,10 +100,10 @@ __device__ __forceinline__ bool mbar_wait_inline(uint32_t bar, uint32_t parity, 
   }
 }
 // The same wait for a whole warp: all lanes go on, or none.
-template <bool CLUSTER = false>
+template <int SCOPE = OWN_CTA>
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                                int role) {
-  const bool ok = mbar_wait<CLUSTER>(bar, parity, abort_flag, status, role);
+  const bool ok = mbar_wait<SCOPE>(bar, parity, abort_flag, status, role);
   return __all_sync(0xffffffffu, ok);
 }
 // Abort path only: gives a transaction that is still in flight on `bar` a bounded time to land, so that no
@@ -109,10 +119,17 @@ __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddep
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- thread-block clusters: rendezvous, and barriers of a peer CTA ---------------------------
-__device__ __forceinline__ void cluster_sync() {
+__device__ __forceinline__ void cluster_arrive() {
   __syncwarp();      // the barrier's aligned form wants the warp's lanes together, whatever branches lie behind them
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
   uint32_t a;
@@ -125,10 +142,10 @@ __device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void peer_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ float4 lds_peer_v4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-  return v;
+// Copies shared memory (16-byte multiples) to another CTA's, counted on a barrier of that CTA when it is there.
+__device__ __forceinline__ void peer_copy(uint32_t peer_dst, uint32_t src, uint32_t bytes, uint32_t peer_bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(peer_dst), "r"(src), "r"(bytes),
+               "r"(peer_bar) : "memory");
 }
 // ---- shared memory by 32-bit address ---------------------------------------------------------
 __device__ __forceinline__ uint4 lds_v4(uint32_t a) {

@@ -84,7 +84,10 @@ constexpr int LAUNCH_REGS = 65536 / GEMM_THREADS & ~7, LEAN_REGS = 56, DRAIN_REG
 static_assert(FIRST_DRAIN_WARP * 32 * LEAN_REGS + NUM_DRAIN_WARPS * 32 * DRAIN_REGS <= GEMM_THREADS * LAUNCH_REGS, "registers of the split");
 constexpr int SMEM_BAR_BYTES = 256;
 constexpr int SMEM_BYTES = 1024 /*alignment slack*/ + NSTAGE * STAGE_BYTES + SC_RING * SC_STAGE_BYTES + SMEM_BAR_BYTES;
-static_assert(SMEM_BYTES <= 232448, "shared memory budget");
+// TILE_SPLIT: and the cluster's partial sums of this CTA's part of the tile
+constexpr int GATHER_ITEMS = 16;                   // of a drain thread's 4 rows x 16 columns, four neighbouring columns each
+constexpr int GATHER_BYTES = GATHER_ITEMS * NUM_DRAIN_WARPS * 32 * 16;
+static_assert(SMEM_BYTES + GATHER_BYTES <= 232448, "shared memory budget");
 static_assert(STAGE_BYTES % 1024 == 0, "stages must keep the 1024-byte alignment of the swizzled tiles");
 static_assert((NSTAGE & (NSTAGE - 1)) == 0 && (NPAIR & (NPAIR - 1)) == 0, "ring sizes must be powers of two");
 
@@ -101,6 +104,7 @@ struct GemmParams {
   const float* bias;      // [Npad]
   void* Y;
   int out_f32;
+  int wide;               // TILE_SPLIT: Y and its rows begin on 32-byte boundaries
   int32_t* status;
 };
 
@@ -183,8 +187,11 @@ __device__ __forceinline__ void issue_group(uint32_t d, uint64_t a, uint64_t b, 
 enum { BRANCH_NONE = 0, BRANCH_I8 = 1, BRANCH_F16 = 2 };
 enum { TILE_WHOLE = 0, TILE_SECTORS = 1, TILE_SPLIT = 2 };
 
-// TILE_SPLIT: the CTAs of a cluster share one tile, each with a part of the stages (K and the branch); their partial sums meet in
-// distributed shared memory.  TILE_SECTORS: every row of Y begins on a 32-byte boundary.  (An instance of its own: with both kinds of
+// TILE_SPLIT: the CTAs of a cluster share one tile, each with a part of the stages (K and the branch).  Every CTA adds up a part of the tile: the others
+// copy their partial sums of it into its shared memory, and it waits for the bytes.  What bounds it is that one trip.  (Rendezvous, loads of all parts from
+// the others' shared memory and a second rendezvous before leaving: us, M x K x N by two, four, eight CTAs, 120 x 1152 x 4608 8.40 -> 7.57, 256 x 4608 x 1152 11.05 -> 10.27,
+// 1 x 1152 x 1152 5.46 -> 4.80, 120 x 8192 x 1152 11.26 -> 9.83.  Stores of 16 bytes by every thread instead of copies from a staging place: 4.60 with one row, but
+// 8.90 with 128; both, by the number of rows: 4.68 and 7.8.)  TILE_SECTORS: every row of Y begins on a 32-byte boundary.  (An instance of its own: with both kinds of
 // stores in one epilogue the drain's registers were worse allocated: 63.6 / 69.4 us for 62.3 / 69.0, M = 8192, K x N = 1152 x 3456 / 4608 x 1152.)
 template <int BRANCH, int TILE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
@@ -205,7 +212,8 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto bar_empty = [&](int s) { return sm_bar + 8u * (uint32_t)(NSTAGE + s); };           // MMAs of the stage retired
   auto bar_tfull = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + b); };
   auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + NPAIR + b); };
-  constexpr int NBAR = 2 * NSTAGE + 3 * NPAIR;
+  [[maybe_unused]] const uint32_t bar_gather = sm_bar + 8u * (uint32_t)(2 * NSTAGE + 3 * NPAIR);
+  constexpr int NBAR = 2 * NSTAGE + 3 * NPAIR + 1;
   static_assert(NBAR * 8 + 16 <= SMEM_BAR_BYTES, "barrier area too small");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + NBAR * 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + NBAR * 8 + 8);
@@ -230,17 +238,29 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int b = 0; b < NPAIR; ++b) mbar_init(bar_tfull(b), 1);
     for (int b = 0; b < 2 * NPAIR; ++b) mbar_init(bar_tempty(b), NUM_DRAIN_WARPS);
     *abort_flag = 0;
+    if constexpr (SPLIT) mbar_init(bar_gather, 1);
     mbar_init_fence();
+    if constexpr (SPLIT) {
+      // what the cluster's other CTAs will copy here: of this part's items those of eight rows that exist, by two warps (column halves) each
+      int items = 0;
+      for (int j = part * GATHER_ITEMS / p.split; j < (part + 1) * GATHER_ITEMS / p.split; ++j)
+        for (int q = 0; q < 4; ++q) items += (u_begin / p.units_n) * LQ_BM + 32 * q + 8 * (j >> 2) < p.M;
+      mbar_expect_tx(bar_gather, (uint32_t)((p.split - 1) * 2 * items * 512));
+    }
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
   tc_fence_before();
   __syncthreads();
+  if constexpr (SPLIT) cluster_arrive();
   grid_launch_dependents();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-  // SPLIT: where a drain thread's partial sums lie for the other CTAs, items of four neighbouring columns
-  auto partial_at = [&](int item, int thread) { return sm_stage + (uint32_t)(item * NUM_DRAIN_WARPS * 32 + thread) * 16; };
+  // SPLIT: the place of a drain warp's items (n_items of 32 lanes x 16 bytes, then the next warp's) that CTA `from` of the cluster has
+  // summed for this one; and where this CTA's own sums wait, by the part that they are for (the operands' place: every MMA has retired)
+  [[maybe_unused]] const int n_items = SPLIT ? GATHER_ITEMS / p.split : 0;
+  auto items_at = [&](uint32_t area, int block, int dwarp) { return area + (uint32_t)((block * NUM_DRAIN_WARPS + dwarp) * n_items) * 512; };
+  [[maybe_unused]] const uint32_t sm_gather = sm_bar + SMEM_BAR_BYTES;
   bool drained = false;
 
   LQ_TL_DECL((blockIdx.x == 0 && lane == 0)
@@ -393,6 +413,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const uint32_t at = sm_sc + (i & (SC_RING - 1)) * SC_STAGE_BYTES + q * SC_GROUP_FLOATS * 4;
       load_scales(sc, at + row_at * 4, at + (LQ_BM + col_at) * 4);
     };
+    if constexpr (SPLIT) cluster_wait();                // the other CTAs' barriers are set up
     grid_dependency_wait();                             // Y may be what an earlier kernel still reads
     open_stage(0, u_begin < u_end);
     for (int u = u_begin; u < u_end && ok; ++u) {
@@ -450,18 +471,28 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (!ok) break;
       LQ_TL(EV_D_EPI_BEGIN, 0);
       if constexpr (SPLIT) {
-        // the partial sums to shared memory (the operands' place: every MMA has retired), items of four neighbouring columns
+        // the partial sums to the CTAs that add them up
+        const int dwarp = warp - FIRST_DRAIN_WARP, row0 = m0 + 32 * quad;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-          for (int i = 0; i < 2; ++i)
-            if (m0 + 32 * quad + 16 * h + 8 * i + fg < p.M) {
+          for (int i = 0; i < 2; ++i) {
+            if (row0 + 8 * (2 * h + i) >= p.M) break;
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                sts_v4(partial_at(4 * (2 * h + i) + k, (int)threadIdx.x - 32 * FIRST_DRAIN_WARP),
-                       make_uint4(__float_as_uint(acc[h][4 * k + i].x), __float_as_uint(acc[h][4 * k + i].y),
-                                  __float_as_uint(acc[h][4 * k + 2 + i].x), __float_as_uint(acc[h][4 * k + 2 + i].y)));
+            for (int k = 0; k < 4; ++k) {
+              const int item = 4 * (2 * h + i) + k, to = item * p.split / GATHER_ITEMS;
+              sts_v4(items_at(sm_stage, to, dwarp) + (uint32_t)((item - to * n_items) * 512 + lane * 16),
+                     make_uint4(__float_as_uint(acc[h][4 * k + i].x), __float_as_uint(acc[h][4 * k + i].y),
+                                __float_as_uint(acc[h][4 * k + 2 + i].x), __float_as_uint(acc[h][4 * k + 2 + i].y)));
             }
+          }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane < p.split && lane != part) {            // a lane for each other CTA: the items that have a row
+          int n = 0;
+          for (int j = lane * n_items; j < (lane + 1) * n_items; ++j) n += row0 + 8 * (j >> 2) < p.M;
+          if (n > 0) peer_copy(peer_smem(items_at(sm_gather, part, dwarp), lane), items_at(sm_stage, lane, dwarp), (uint32_t)n * 512, peer_smem(bar_gather, lane));
+        }
       } else {
         // Epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad.  Two lanes' stores of 16
         // bytes never meet in a 32-byte sector here, so each would write half of one; where all of Y's rows are whole sectors a lane
@@ -508,36 +539,41 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     drained = ok;
   }
   if constexpr (SPLIT) {
-    // Every CTA of the cluster adds up a part of the items, in the order of the stages, and stores them.
-    cluster_sync();
-    if (drained) {
-      const int at = (int)threadIdx.x - 32 * FIRST_DRAIN_WARP, mb = u_begin / p.units_n, nu = u_begin - mb * p.units_n, n = 16 / p.split;
+    // Every CTA of the cluster adds up its items, in the order of the stages, and stores them.
+    if (warp < FIRST_DRAIN_WARP) cluster_wait();
+    if (drained && mbar_wait_warp<PEER_DATA>(bar_gather, 0, abort_flag, p.status, LQ_STAGE_DRAIN)) {
+      const int dwarp = warp - FIRST_DRAIN_WARP, mb = u_begin / p.units_n, nu = u_begin - mb * p.units_n;
       const int row = mb * LQ_BM + 32 * (warp & 3) + (lane >> 2), col = nu * UNIT + ((warp - FIRST_DRAIN_WARP) >> 2) * WCOLS + 16 * (lane & 3);
-      for (int j = part * n; j < (part + 1) * n; j += 2) {       // two items: eight columns
-        const int r = row + 8 * (j >> 2), c = col + 4 * (j & 3);
+#pragma unroll 2
+      for (int i = 0; i < n_items; i += 2) {                     // two items: eight columns
+        const int j = part * n_items + i, r = row + 8 * (j >> 2), c = col + 4 * (j & 3);
         if (r >= p.M || c >= p.N) continue;
         float y[8] = {};
 #pragma unroll 4
         for (int k = 0; k < p.split; ++k) {
-          const float4 a = lds_peer_v4(peer_smem(partial_at(j, at), k)), b = lds_peer_v4(peer_smem(partial_at(j + 1, at), k));
-          y[0] += a.x; y[1] += a.y; y[2] += a.z; y[3] += a.w; y[4] += b.x; y[5] += b.y; y[6] += b.z; y[7] += b.w;
+          const uint32_t from = (k == part ? items_at(sm_stage, part, dwarp) : items_at(sm_gather, k, dwarp)) + (uint32_t)(i * 512 + lane * 16);
+          const uint4 a = lds_v4(from), b = lds_v4(from + 512);
+          y[0] += __uint_as_float(a.x); y[1] += __uint_as_float(a.y); y[2] += __uint_as_float(a.z); y[3] += __uint_as_float(a.w);
+          y[4] += __uint_as_float(b.x); y[5] += __uint_as_float(b.y); y[6] += __uint_as_float(b.z); y[7] += __uint_as_float(b.w);
         }
         if (p.out_f32) {
-          float4* Y = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c);
-          Y[0] = make_float4(y[0], y[1], y[2], y[3]);
-          Y[1] = make_float4(y[4], y[5], y[6], y[7]);
+          uint32_t w[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) w[k] = __float_as_uint(y[k]);
+          float* Y = reinterpret_cast<float*>(p.Y) + (size_t)r * p.N + c;
+          if (p.wide) stg_32<true>(Y, w);
+          else stg_32<false>(Y, w);
         } else {
           uint32_t w[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const __half2 q = __floats2half2_rn(y[2 * i], y[2 * i + 1]);
-            w[i] = *reinterpret_cast<const uint32_t*>(&q);
+          for (int k = 0; k < 4; ++k) {
+            const __half2 q = __floats2half2_rn(y[2 * k], y[2 * k + 1]);
+            w[k] = *reinterpret_cast<const uint32_t*>(&q);
           }
           *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(p.Y) + (size_t)r * p.N + c) = make_uint4(w[0], w[1], w[2], w[3]);
         }
       }
     }
-    cluster_sync();                                     // nobody's shared memory goes away while another CTA reads it
   }
 
   // ---------------------------------------------------------------------- teardown
@@ -547,6 +583,9 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
   }
+  // SPLIT: all that this CTA was to be sent is here, so it may leave.  Where a wait has run out it stays until the others have left or
+  // stay, too: they may still be storing to it.
+  if (SPLIT && *abort_flag) cluster_sync();
 }
 
 // Self-test of the bounded wait: one warp waits on a barrier that nothing ever arrives on.
@@ -564,13 +603,13 @@ __global__ void lq_wait_probe_kernel(int32_t* status, long long limit) {
 }
 
 // CTAs per tile of a launch of few tiles (1, 2, 4 or 8).  A tile's stages are one serial chain, so while SMs are idle they may as well share
-// it; a cluster's launch, its two rendezvous and the exchange cost the rest (us now, alone and shared: M = 1, K x N = 1152 x 1152: 6.9 and 5.4 by
-// eight; M = 128, 8192 x 1152: 30.8 and 11.4 by eight; M = 256, 4608 x 1152: 18.9 and 11.0 by four).  The hardware places a cluster's CTAs next to each
-// other, so fewer fit than there are SMs; a second round of them would cost more than it gives.  The prices are those of the drain as it was, 0.52 us a stage and
-// 1.9 + 0.15 per CTA that is read; now a stage takes 0.43, a cluster 2.0 and, with full tiles, 0.55 + 0.26 per CTA more.  By those 34 of 40 sizes timed (K from 384 to 8192, M from
-// 1 to 512) are cut as here and 6, all of ten stages, would not be shared (M = 128, 1152 x 4608: 8.3 by two, 7.5 alone).  The line stays
-// where it was: shared sums are the shorter chains, and further from the exact sum is what those rows would be (that size, fp32 output: relative error
-// 6.0e-8 by two, 7.4e-8 alone).
+// it; a cluster's launch and the exchange cost the rest (us, alone and shared: M = 1, K x N = 1152 x 1152: 7.0 and 4.8 by
+// eight; M = 120, 8192 x 1152: 30.8 and 9.8 by eight; M = 256, 4608 x 1152: 18.9 and 10.3 by four).  The hardware places a cluster's CTAs next to each
+// other, so fewer fit than there are SMs; a second round of them would cost more than it gives.  Prices: the exchange 1.62 us, with full tiles 0.6 + 0.08
+// per CTA more; a stage 0.52, as the drain once took it - 0.44 now, by which a few sizes of ten stages would not be shared any more (M = 120,
+// 1152 x 4608: 7.57 by two, 7.50 alone; M = 256: 8.90 and 7.71).  But shared sums are the shorter chains, and further from the exact sum is what those rows would
+// be (M = 128, fp32 output: relative error 6.0e-8 by two, 7.4e-8 alone): with these prices no size is shared by fewer CTAs than while the exchange took longer,
+// and tiles of six stages are shared, too (M = 1, 640 x 1152: 4.9 by four, 5.3 alone; up to 60 rows).
 int g_clusters[64][3];                                // how many clusters of 2, 4, 8 the device holds at once
 int pick_split(int device, int M, long long units, int stages, int ctas) {
   int best = 1;
@@ -578,7 +617,7 @@ int pick_split(int device, int M, long long units, int stages, int ctas) {
   for (int i = 0, split = 2; i < 3; ++i, split *= 2) {
     if (split > ctas || split > stages || units > std::min(g_clusters[device & 63][i], ctas / split)) break;
     if (g_lq_gemm_split > 0 && split != g_lq_gemm_split) continue;
-    const double cost = g_lq_gemm_split > 0 ? 0 : 0.52 * lq_ceil_div(stages, split) + 1.9 + 0.15 * split * std::min(M, LQ_BM) / LQ_BM;
+    const double cost = g_lq_gemm_split > 0 ? 0 : 0.52 * lq_ceil_div(stages, split) + 1.62 + (0.6 + 0.08 * split) * std::min(M, LQ_BM) / LQ_BM;
     if (cost < best_cost) { best_cost = cost; best = split; }
   }
   return best;
@@ -602,7 +641,7 @@ lq_status lq_gemm_prepare(int device) {
     cudaFuncAttributes at;
     if (lq_note_cuda(cudaFuncGetAttributes(&at, kernel)) != cudaSuccess) return LQ_ERR_CUDA;
     if (at.numRegs < LAUNCH_REGS) return LQ_ERR_UNSUPPORTED;
-    if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return LQ_ERR_CUDA;
+    if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES + GATHER_BYTES)) != cudaSuccess) return LQ_ERR_CUDA;
   }
   // once per device: launches of other threads read g_clusters without the lock, each after its own layer's upload came through here
   static std::mutex mu;
@@ -614,7 +653,7 @@ lq_status lq_gemm_prepare(int device) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2u << i; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    lc.gridDim = dim3(2u << i); lc.blockDim = dim3(GEMM_THREADS); lc.dynamicSmemBytes = SMEM_BYTES; lc.attrs = at; lc.numAttrs = 1;
+    lc.gridDim = dim3(2u << i); lc.blockDim = dim3(GEMM_THREADS); lc.dynamicSmemBytes = SMEM_BYTES + GATHER_BYTES; lc.attrs = at; lc.numAttrs = 1;
     if (lq_note_cuda(cudaOccupancyMaxActiveClusters(&g_clusters[device & 63][i], lq_gemm_kernel<BRANCH_I8, TILE_SPLIT>, &lc)) != cudaSuccess)
       return LQ_ERR_CUDA;
   }
@@ -632,7 +671,7 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   p.tiles_m = lq_ceil_div(A->M, LQ_BM);
   p.units_n = L->Npad / UNIT;
   p.sx = A->d_sx; p.sw = L->d_sw; p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
-  p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0;
+  p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0; p.wide = lq_rows_of_sectors(Y, L->N, dt);
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;
   int sms = 0;
@@ -648,6 +687,6 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   };
   auto* k = p.split > 1 ? kernel(std::integral_constant<int, TILE_SPLIT>())
                         : lq_rows_of_sectors(Y, L->N, dt) ? kernel(std::integral_constant<int, TILE_SECTORS>()) : kernel(std::integral_constant<int, TILE_WHOLE>());
-  const cudaError_t e = lq_launch_cluster(k, ctas, GEMM_THREADS, p.split, SMEM_BYTES, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
+  const cudaError_t e = lq_launch_cluster(k, ctas, GEMM_THREADS, p.split, SMEM_BYTES + (p.split > 1 ? GATHER_BYTES : 0), st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }
