@@ -39,8 +39,11 @@
 //   SINT4     x and s are 11-bit numbers, so x / s is either exactly k + 1/2 or at least 2^-14 away from it.  The product
 //             with a reciprocal that is an ulp or two off is within 2^-19 of the quotient; adding 192 rounds it to a multiple of 2^-16, which restores
 //             exact ties and moves nothing else across one; a second addition then rounds to the integer, ties to even.
-//   branch    x / sb from the correctly rounded reciprocal by one FMA correction step, which yields the correctly
-//             rounded binary32 quotient; 1.5 * 2^23 rounds it to the nearest even integer.
+//   branch    x / sb is within 2^-23 of qm x / max, which is either exactly k + 1/2 or at least 2^-19 away from it (11-bit numbers, qm of 5
+//             or 7 bits); so one FMA with 1.5 * 2^23 and a reciprocal good to 2^-21 rounds like the quotient everywhere but on such
+//             ties.  As qm is prime they are at x = +-max / 2, for which the reciprocal is taken on the side that gives the quotient's code
+//             (BranchScale), or the maximum's significand is a multiple of qm: such rows go by the correctly rounded
+//             quotient, from the reciprocal by one FMA correction step.
 //   MX        x * 2^-e is exact, and the fp16 pipe does it two values at a time: one fma with 1.5 * 2^10 rounds x * 2^-e to
 //             the nearest even integer without an intermediate rounding; blocks so small that 2^-e is no fp16 number
 //             are scaled up (exactly) first, a rare branch.  MXFP8e4: products below 2^-14 may lose bits, far below half of e4m3's
@@ -91,7 +94,8 @@ struct QuantParams : QuantCut {
   int tmem_cols;        // power of two
   float dev;            // MXFP: how far a sum of the tensor core is taken to be from the one in settle_tiles' order, over its block's maximum
   float unit;           // MX branches: the intermediate over the tensor core's sums (a power of two, 1 but for tiny first factors)
-  float qm;             // largest branch activation code
+  float qm, rqm;        // largest branch activation code, 1 over it
+  float near_tie;       // half an ulp of qm / 2
   int32_t* status;
 };
 
@@ -298,23 +302,52 @@ __device__ __forceinline__ uint2 sint4_codes8(const uint4& v, float rcp, bool co
                     f32x2_to_e4m3x2(q[2].y, q[2].x) | (f32x2_to_e4m3x2(q[3].y, q[3].x) << 16));
 }
 
-// Branch codes of eight values under the row's scale sb, invb = fl32(1/sb): q0 = fl32(x invb) is within one ulp of x / sb,
-// r = x - sb q0 is exact in an FMA, and fl32(q0 + r invb) is then the correctly rounded quotient (Markstein's correction
-// step); |x| / sb <= qm (1 + 2^-23), so it never leaves [-qm, qm].  The low byte of (code + MAGIC)'s bit pattern is the code.
-__device__ __forceinline__ uint2 branch_codes8(const uint4& v, float sb, float invb) {
-  const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
-  const float2 y = splat(invb), ns = splat(-sb), magic = splat(MAGIC);
+// Scale of a row's branch codes (its maximum over qm, 1 for a row of zeros) and the reciprocal that codes are formed with (see the top).
+struct BranchScale {
+  float sb, rcp, inv;    // rcp: fl32(1 / sb), inv: the same or a few ulps beside it
+  bool exact;            // this row's codes need the quotient: ties elsewhere, or a maximum that is no number
+  // rqm: fl32(1 / qm); near: half an ulp of qm / 2
+  __device__ __forceinline__ BranchScale(uint32_t max_bits, float qm, float rqm, float near) {
+    const float rm = __half2float(__ushort_as_half((unsigned short)max_bits));
+    sb = rm == 0.f ? 1.f : __fdiv_rn(rm, qm);
+    inv = rcp = __frcp_rn(sb);
+    const float a = (float)((max_bits & 0x3FFu) | (max_bits < 0x400u ? 0u : 0x400u));       // significand of the maximum
+    exact = max_bits >= 0x7C00u || (a != 0.f && __fmul_rn(rintf(__fmul_rn(a, rqm)), qm) == a);
+    // The code of max / 2 is rint(fl32(max / 2 / sb)).  The quotient is within 2^-23 of qm / 2, which is half of an odd number plus one:
+    // ties go up, and what is no more than half an ulp below is a tie.  (max / 2 - sb qm / 2 is exact, half of the division's remainder.)
+    const bool up = __fmaf_rn(sb, -0.5f * qm, 0.5f * rm) >= -near * sb;
+    if ((__fmaf_rn(0.5f * rm, rcp, -0.5f * qm) >= 0.f) != up) inv = __uint_as_float(__float_as_uint(rcp) + (up ? 4u : -4u));
+  }
+};
+// Branch codes of eight values: the low byte of the code + MAGIC is the code.
+__device__ __forceinline__ uint2 low_bytes8(const float2 (&q)[4]) {
   uint32_t t[8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { t[2 * i] = __float_as_uint(q[i].x); t[2 * i + 1] = __float_as_uint(q[i].y); }
+  return make_uint2(__byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410),
+                    __byte_perm(__byte_perm(t[4], t[5], 0x0040), __byte_perm(t[6], t[7], 0x0040), 0x5410));
+}
+__device__ __forceinline__ uint2 branch_codes8(const uint4& v, float inv) {
+  const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
+  const float2 y = splat(inv), magic = splat(MAGIC);
+  float2 q[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) q[i] = __ffma2_rn(x[i], y, magic);
+  return low_bytes8(q);
+}
+// The same by the quotient, inv = fl32(1 / sb): q0 = fl32(x inv) is within one ulp of x / sb, r = x - sb q0 is exact in an FMA, and
+// fl32(q0 + r inv) is then the correctly rounded quotient (Markstein's correction step); |x| / sb <= qm (1 + 2^-23), so it never
+// leaves [-qm, qm].
+__device__ __forceinline__ uint2 branch_codes8_exact(const uint4& v, float sb, float inv) {
+  const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
+  const float2 y = splat(inv), ns = splat(-sb), magic = splat(MAGIC);
+  float2 q[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const float2 q0 = __fmul2_rn(x[i], y);
-    const float2 q1 = __fadd2_rn(__ffma2_rn(__ffma2_rn(q0, ns, x[i]), y, q0), magic);
-    t[2 * i] = __float_as_uint(q1.x); t[2 * i + 1] = __float_as_uint(q1.y);
+    q[i] = __fadd2_rn(__ffma2_rn(__ffma2_rn(q0, ns, x[i]), y, q0), magic);
   }
-  uint2 b;
-  b.x = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
-  b.y = __byte_perm(__byte_perm(t[4], t[5], 0x0040), __byte_perm(t[6], t[7], 0x0040), 0x5410);
-  return b;
+  return low_bytes8(q);
 }
 
 // Near ties of the MXFP intermediate T = deq(Q(X)) deq(Q2(L1)).  Floating-point elements round in steps of up to a fourteenth of the
@@ -898,7 +931,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       const bool va = ma < p.M, vb = ma + 2 < p.M, vs = first && ms < p.M;
       uint8_t* const qa = p.qx8 + (size_t)ma * qs + sx * 128 + 64 * box + 16 * pp;
       uint8_t* const sfr = SINT ? nullptr : p.sfa + ((size_t)(ms >> 7) * (qs >> 7) + sx) * 512 + 16 * (ms & 31) + 4 * ((ms & 127) >> 5);
-      float sb_a = 1.f, sb_b = 1.f, inv_a = 1.f, inv_b = 1.f;
+      float sb_a = 1.f, sb_b = 1.f, inv_a = 1.f, inv_b = 1.f;     // integer branch: scales of rows ra, ra + 2
+      bool exact = false;                                        // (of any of the warp's rows)
       __half2 hm = __float2half2_rn(0.f);                        // maxima of rows ra, ra + 2
       // One walk over the tile.  MAINP: main codes and scales; BRP: the branch's operand; FREE: the X slots are handed back.
       auto walk = [&](auto MAINP, auto BRP, const bool free_x) {
@@ -976,9 +1010,12 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           if constexpr (decltype(BRP)::value) {
             [[maybe_unused]] uint2 ca[2], cb[2];
             if constexpr (BR == BR_INT) {
-              if (live) {
+              if (live && !exact) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) { ca[h] = branch_codes8(a[h], sb_a, inv_a); cb[h] = branch_codes8(b[h], sb_b, inv_b); }
+                for (int h = 0; h < 2; ++h) { ca[h] = branch_codes8(a[h], inv_a); cb[h] = branch_codes8(b[h], inv_b); }
+              } else if (live) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) { ca[h] = branch_codes8_exact(a[h], sb_a, inv_a); cb[h] = branch_codes8_exact(b[h], sb_b, inv_b); }
               }
             }
             if (!mbar_wait_warp(bar_empty(e.at), e.par, abort_flag, p.status, LQ_STAGE_QUANT)) return false;
@@ -1040,19 +1077,23 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (lane == 0) mbar_arrive(bar_sync);
         ok = mbar_wait_warp(bar_sync, tc & 1, abort_flag, p.status, LQ_STAGE_QUANT);
         if (!ok) break;
-        const float rm_a = __half2float(__ushort_as_half((unsigned short)mx[ra]));
-        const float rm_b = __half2float(__ushort_as_half((unsigned short)mx[ra + 2]));
+        // eight lanes have the same two rows: one half works out row ra's scale, the other row ra + 2's
+        const BranchScale mine((uint32_t)mx[sr], p.qm, p.rqm, p.near_tie);
+        {
+          exact = __any_sync(0xffffffffu, mine.exact);
+          const float own = exact ? mine.rcp : mine.inv;
+          const float sb = __shfl_xor_sync(0xffffffffu, mine.sb, 8), inv = __shfl_xor_sync(0xffffffffu, own, 8);
+          sb_a = box ? sb : mine.sb; sb_b = box ? mine.sb : sb;
+          inv_a = box ? inv : own; inv_b = box ? own : inv;
+        }
         const uint32_t after = buf == 0 ? 2 : buf - 1;           // two tiles on: every warp is past its last use
         if (team == 0 && sx == 0 && first) rowmax[after * 64 + sr] = 0;
         buf = buf == 2 ? 0 : buf + 1;
-        sb_a = rm_a == 0.f ? 1.f : __fdiv_rn(rm_a, p.qm);
-        sb_b = rm_b == 0.f ? 1.f : __fdiv_rn(rm_b, p.qm);
-        inv_a = __frcp_rn(sb_a); inv_b = __frcp_rn(sb_b);
         if (team == 0 && sx == 0) {                              // a4 reads the scale: its previous tile of this parity must be done
           ok = mbar_wait_warp(bar_tempty(tc & 1), ((tc >> 1) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_QUANT);
           if (!ok) break;
-          if (first) row_sb[(tc & 1) * 64 + sr] = box ? sb_b : sb_a;
-          if (vs) p.sXb[ms] = box ? sb_b : sb_a;
+          if (first) row_sb[(tc & 1) * 64 + sr] = mine.sb;
+          if (vs) p.sXb[ms] = mine.sb;
         }
         ok = walk(No(), Yes(), true);
       } else {
@@ -1127,6 +1168,8 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   p.dev = L->cfg.branch == LQ_BRANCH_MXFP8 ? 1.f : L->cfg.branch == LQ_BRANCH_MXFP6 ? 0.5f : 0.2f;
   p.unit = ldexpf(1.f, -L->l1_shift);
   p.qm = abits > 0 ? (float)((1 << (abits - 1)) - 1) : 0.f;
+  p.rqm = 1.f / p.qm;
+  p.near_tie = abits > 0 ? ldexpf(1.f, abits - 27) : 0.f;
   p.status = lq_device_status_ptr(A->device);
   if (!p.status) return LQ_ERR_CUDA;
   int sms = 0;

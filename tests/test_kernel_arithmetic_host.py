@@ -3,6 +3,7 @@ relies on, against the plain definition (Appendix A.3: SINT4, fp16 scale, RTN)."
 from fractions import Fraction
 
 import numpy as np
+import pytest
 
 from oracle import lq_oracle as O
 
@@ -65,3 +66,33 @@ def test_fma_corrected_quotient_is_the_correctly_rounded_division():
         assert q1 == _rn32(a / b), (float(a), float(b))
         ties += (2 * a / b).denominator == 1 and (a / b).denominator == 2
     assert ties > 100
+
+
+@pytest.mark.parametrize("qm", [127, 31])
+def test_one_fma_with_a_chosen_reciprocal_gives_the_codes_of_the_quotient(qm):
+    """Branch codes by x -> rint(x inv) (one FMA with 1.5 * 2^23: the product is not rounded before) for every finite fp16 row
+    maximum and, of the values up to it, the two next to every tie (k + 1/2) max / qm and the tie itself: the codes of the definition,
+    rint(fl32(x / sb)).  Values away from ties cannot differ if these do not.  Rows whose maximum's significand is a multiple of qm
+    go another way and are left out."""
+    bits = np.arange(1, 0x7C00, dtype=np.uint32)
+    significand = (bits & 0x3FF) | np.where(bits < 0x400, 0, 0x400)
+    rm = bits[significand % qm != 0].astype(np.uint16).view(np.float16).astype(np.float32)
+    sb = rm / np.float32(qm)
+    rcp = (1.0 / sb.astype(np.float64)).astype(np.float32)
+    near = {127: 2.0 ** -19, 31: 2.0 ** -21}[qm]                                         # half an ulp of qm / 2
+    up = 0.5 * rm.astype(np.float64) - sb.astype(np.float64) * (0.5 * qm) >= -near * sb  # exact: 31 bits
+    assert np.array_equal(up, np.rint((np.float32(0.5) * rm) / sb) == (qm + 1) // 2)
+    above = 0.5 * rm.astype(np.float64) * rcp.astype(np.float64) - 0.5 * qm >= 0          # exact: 35 bits
+    inv = np.where(above == up, rcp.view(np.int32), rcp.view(np.int32) + np.where(up, 4, -4)).astype(np.int32).view(np.float32)
+    assert (above != up).sum() > 1000
+    ties = 0
+    for k in range(qm):
+        t = (k + 0.5) * rm.astype(np.float64) / qm
+        mid = t.astype(np.float16)
+        for step in (-1, 0, 1):
+            x = (mid.view(np.int16) + step).astype(np.int16).view(np.float16).astype(np.float64)
+            x = np.where((x >= 0) & (x <= rm), x, 0.0)
+            code = np.rint((x.astype(np.float32) / sb).astype(np.float64))
+            assert np.array_equal(np.rint(x * inv.astype(np.float64)), code), k
+            ties += (x * 2 * qm == (2 * k + 1) * rm.astype(np.float64)).sum()
+    assert ties > 10000
