@@ -110,6 +110,7 @@ struct Ring {
 
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
 __device__ __forceinline__ uint32_t as_u32(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+__device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float pow2f_n(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }   // -126 <= e <= 127
 
 // two floats -> two E4M3 bytes (hi: first operand, lo: second)
@@ -231,11 +232,12 @@ __device__ __forceinline__ void mxint8_codes8(const uint4& v, __half2 inv, uint2
   hi = make_uint2(f16x4_to_e4m3x4(h[0], h[1]), f16x4_to_e4m3x4(h[2], h[3]));
   lo = make_uint2(f16x4_to_e4m3x4(l[0], l[1]), f16x4_to_e4m3x4(l[2], l[3]));
 }
-// One fp32 value (the rank-r intermediate) under its block's exponent, the same digits.
-__device__ __forceinline__ void mxint8_digits(float x, float inv, float& hi, float& lo) {
-  const float c = __fadd_rn(__fmaf_rn(x, inv, MAGIC), -MAGIC);
-  hi = floorf(__fmul_rn(__fadd_rn(c, 8.f), 0.0625f));
-  lo = __fmaf_rn(hi, -16.f, c);
+// Two fp32 values (of the rank-r intermediate) under their block's exponent, the same digits.
+__device__ __forceinline__ void mxint8_digits(float2 x, float inv, float2& hi, float2& lo) {
+  const float2 up = splat(MAGIC), down = splat(-MAGIC);
+  const float2 c = __fadd2_rn(__ffma2_rn(x, splat(inv), up), down);
+  hi = __fadd2_rn(__fadd2_rn(__ffma2_rn(c, splat(0.0625f), splat(0.015625f)), up), down);
+  lo = __ffma2_rn(hi, splat(-16.f), c);
 }
 
 // Two rows' vectors whose block maxima are out of PairScale's range (MXFP6e2: any): kept out of the main loop's instructions.
@@ -287,7 +289,6 @@ struct Sint4Scale {
   }
 };
 __device__ __forceinline__ uint4 vec16(const uint2 (&v)[2]) { return make_uint4(v[0].x, v[0].y, v[1].x, v[1].y); }
-__device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
 __device__ __forceinline__ uint2 sint4_codes8(const uint4& v, float rcp, bool coarse) {
   const float2 x[4] = {__half22float2(as_half2(v.x)), __half22float2(as_half2(v.y)), __half22float2(as_half2(v.z)), __half22float2(as_half2(v.w))};
   const float2 inv = splat(rcp), c0 = splat(192.f), c1 = splat(MAGIC - 192.f), c2 = splat(-MAGIC);
@@ -368,6 +369,17 @@ struct TieTest {
   __device__ __forceinline__ bool operator()(float x) const {
     const float u = fabsf(x) * k;
     return u > 7.5f && fabsf(u - __fadd_rn(__fadd_rn(u, MAGIC), -MAGIC)) > limit;
+  }
+  // whether one of them is that close to half a step of the largest binade, in whichever binade it is
+  __device__ __forceinline__ bool any(const float (&x)[32]) const {
+    float far[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float2 u = __fmul2_rn(make_float2(x[2 * i], x[2 * i + 1]), splat(k));
+      const float2 d = __ffma2_rn(__fadd2_rn(__fadd2_rn(u, splat(MAGIC)), splat(-MAGIC)), splat(-1.f), u);
+      far[0] = fmaxf(far[0], fabsf(d.x)); far[1] = fmaxf(far[1], fabsf(d.y));
+    }
+    return fmaxf(far[0], far[1]) > limit;
   }
 };
 __device__ __forceinline__ void mma_e4m3_16832(float (&c)[4], const uint2& a0, const uint2& a1, const uint2& b) {
@@ -751,6 +763,10 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
   } else if (BR != BR_NONE && warp < 2) {
     // ------------------------------------------------------------------ a4: lane = row of the tile, straight from tensor memory
+    // One warp's chain of instructions at the end of a launch, a microsecond or two long: 32 columns at a time, two values to an
+    // instruction, a rank of up to 32 read once.  (Sixteen at a time, one by one, the scaled sums worked out for the maximum and again for the codes: us,
+    // M = 1 / 8192, K = 1152, X in the L2, SINT4 rank 32 6.5 / 11.1 -> 5.9 / 10.7, MXFP8 rank 64 6.2 / 9.3 -> 5.5 / 8.5, MXFP4 rank 128 7.7 / 11.6 -> 6.6 / 10.3,
+    // MXINT8 rank 64 7.5 / 11.2 -> 6.9 / 10.5.)
     grid_dependency_wait();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0) + ((uint32_t)(32 * warp) << 16);
     const int nacc = min(p.nacc, p.nst), row = 32 * warp + lane;
@@ -764,68 +780,96 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       tc_fence_after();
       uint8_t* const tqr = p.tq + (size_t)m * p.tq_stride;
       if (32 * warp < TR) {
-        // 16 columns of the row from `col` on: the sum over the accumulators (and the first factor's digit planes)
-        auto fetch = [&](int col, float (&t)[16]) {
-          uint32_t v[16];
-#pragma unroll 1
-          for (int a = 0; a < nacc * p.bplanes; ++a) {
-            tmem_ld_32x16(set + (uint32_t)(a * p.rn + col), v);
+        // 32 columns of the row from `col` on (zeros beyond the rank): the sum over the accumulators (and the first factor's digit planes)
+        auto fetch = [&](int col, float (&t)[32]) {
+          const bool both = col + 16 < p.rn;
+          auto load = [&](int a, uint32_t (&v)[2][16]) {
+            const uint32_t at = set + (uint32_t)(a * p.rn + col);
+            tmem_ld_32x16(at, v[0]);
+            if (both) tmem_ld_32x16(at + 16, v[1]);
             tmem_ld_wait();
+          };
+          uint32_t v[2][16];
+          load(0, v);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float x = BR == BR_INT ? __int2float_rn((int)v[j]) : __uint_as_float(v[j]);
-              t[j] = a == 0 ? x : t[j] + x;
+          for (int j = 0; j < 32; ++j) {
+            const uint32_t w = j < 16 || both ? v[j >> 4][j & 15] : 0u;
+            t[j] = BR == BR_INT ? __int2float_rn((int)w) : __uint_as_float(w);
+          }
+          if constexpr (BR != BR_INT) {
+#pragma unroll 1
+            for (int a = 1; a < nacc * p.bplanes; ++a) {
+              load(a, v);
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                if (j < 16 || both) t[j] += __uint_as_float(v[j >> 4][j & 15]);
             }
           }
         };
-        float t[16];
+        auto pair = [](const float (&t)[32], int i) { return make_float2(t[2 * i], t[2 * i + 1]); };
+        auto largest = [](const float (&t)[32]) {                // of the magnitudes
+          float m[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int j = 0; j < 32; ++j) m[j & 3] = fmaxf(m[j & 3], fabsf(t[j]));
+          return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+        };
+        float t[32];
         if constexpr (BR == BR_INT) {
           const float sr = row_sb[(tc & 1) * 64 + row];
           auto scaled = [&](int c) {                           // t = fl32(fl32(I1) fl32(sXb sL1)); rows beyond the tile hold anything
             fetch(c, t);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) t[j] = valid ? __fmul_rn(t[j], __fmul_rn(sr, sl1[c + j])) : 0.f;
+            for (int i = 0; i < 8; ++i) {
+              const float4 s = *reinterpret_cast<const float4*>(__builtin_assume_aligned(sl1 + c + 4 * i, 16));
+              const float2 u = __fmul2_rn(pair(t, 2 * i), __fmul2_rn(splat(sr), make_float2(s.x, s.y)));
+              const float2 w = __fmul2_rn(pair(t, 2 * i + 1), __fmul2_rn(splat(sr), make_float2(s.z, s.w)));
+              t[4 * i] = u.x; t[4 * i + 1] = u.y; t[4 * i + 2] = w.x; t[4 * i + 3] = w.y;
+            }
           };
           float amax = 0.f;
 #pragma unroll 1
-          for (int c = 0; c < p.rn; c += 16) {
+          for (int c = 0; c < p.rn; c += 32) {
             scaled(c);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(t[j]));
+            amax = fmaxf(amax, largest(t));
           }
           const float st = amax == 0.f ? 1.f : __fdiv_rn(amax, p.qm);
           if (valid) p.sT[SINT ? lq_row_slot(m) : m] = st;
-          // The quotient t / st as in branch_codes8.  A power of two keeps its steps in binary32's normal range; the quotient
+          // The correctly rounded quotient t / st as in branch_codes8_exact.  A power of two keeps its steps in binary32's normal range; the quotient
           // stays what it is (what underflows is far below half a code).
-          const float k = st < 1e-20f ? 0x1p64f : st > 1e20f ? 0x1p-64f : 1.f, ns = -st * k, y = __frcp_rn(st * k);
+          const float k = st < 1e-20f ? 0x1p64f : st > 1e20f ? 0x1p-64f : 1.f;
+          const float2 ns = splat(-st * k), y = splat(__frcp_rn(st * k));
           const bool coarse = st < 0x1p-126f;                  // a subnormal scale: amax / st may be up to half again as large as qm
 #pragma unroll 1
-          for (int c = 0; c < p.rn; c += 16) {
-            scaled(c);
-            uint32_t w[4];
+          for (int c = 0; c < p.rn; c += 32) {
+            if (p.rn > 32) scaled(c);                          // (up to 32 columns are still there)
+            uint32_t w[8];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float x = t[j] * k, q0 = __fmul_rn(x, y);
-              float q = __fmaf_rn(__fmaf_rn(q0, ns, x), y, q0);
-              if (coarse) q = fminf(fmaxf(q, -p.qm), p.qm);
-              const uint32_t code = __float_as_uint(__fadd_rn(q, MAGIC)) & 0xFFu;
-              w[j >> 2] = (j & 3) == 0 ? code : w[j >> 2] | (code << (8 * (j & 3)));
+            for (int i = 0; i < 16; ++i) {
+              const float2 x = __fmul2_rn(pair(t, i), splat(k)), q0 = __fmul2_rn(x, y);
+              float2 q = __ffma2_rn(__ffma2_rn(q0, ns, x), y, q0);
+              if (coarse) q = make_float2(fminf(fmaxf(q.x, -p.qm), p.qm), fminf(fmaxf(q.y, -p.qm), p.qm));
+              q = __fadd2_rn(q, splat(MAGIC));
+              const uint32_t two = __byte_perm(__float_as_uint(q.x), __float_as_uint(q.y), 0x0040);
+              w[i >> 1] = (i & 1) == 0 ? two : __byte_perm(w[i >> 1], two, 0x5410);
             }
-            if (valid) *reinterpret_cast<uint4*>(tqr + c) = make_uint4(w[0], w[1], w[2], w[3]);
+            // (a rank of 16 more than a multiple of 32: zeros up to there, where the up-projection's K ends)
+            if (valid) {
+              *reinterpret_cast<uint4*>(tqr + c) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(tqr + c + 16) = c + 16 < p.rn ? make_uint4(w[4], w[5], w[6], w[7]) : make_uint4(0, 0, 0, 0);
+            }
           }
-          // zeros up to the next multiple of 32, where the up-projection's K ends
-          if ((p.rn & 16) && valid) *reinterpret_cast<uint4*>(tqr + p.rn) = make_uint4(0, 0, 0, 0);
         } else if constexpr (BR == BR_F16) {
           if (valid) p.sT[SINT ? lq_row_slot(m) : m] = 1.f;
 #pragma unroll 1
-          for (int c = 0; c < p.rn; c += 16) {
+          for (int c = 0; c < p.rn; c += 32) {
             fetch(c, t);
-            uint32_t w[8];
+            uint32_t w[16];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) w[j] = as_u32(__floats2half2_rn(t[2 * j], t[2 * j + 1]));
+            for (int j = 0; j < 16; ++j) w[j] = as_u32(__floats2half2_rn(t[2 * j], t[2 * j + 1]));
             if (valid) {
-              *reinterpret_cast<uint4*>(tqr + 2 * c) = make_uint4(w[0], w[1], w[2], w[3]);
-              *reinterpret_cast<uint4*>(tqr + 2 * c + 16) = make_uint4(w[4], w[5], w[6], w[7]);
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (j < 2 || c + 16 < p.rn) *reinterpret_cast<uint4*>(tqr + 2 * c + 16 * j) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
             }
           }
         } else {
@@ -838,32 +882,25 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           [[maybe_unused]] uint32_t near = 0;                    // MXFP: the row's blocks to be settled at the end
 #pragma unroll 1
           for (int b = 0; 32 * b < p.rn; ++b) {
-            float t2[16];
             fetch(32 * b, t);
-            if (32 * b + 16 < p.rn) fetch(32 * b + 16, t2);
-            else {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) t2[j] = 0.f;
-            }
-            float amax = 0.f;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fmaxf(fabsf(t[j]), fabsf(t2[j])));
+            const float amax = largest(t);
             const int e = FPB ? mxfp_exponent<SIX>(amax * p.unit) : mxint8_exponent(amax * p.unit);
             const float inv = e == -127 ? 0.f : pow2f_n(-e) * p.unit;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-              const float (&x)[16] = h ? t2 : t;
               uint32_t w[4], d[4];
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
+                const float2 x0 = pair(t, 8 * h + 2 * j), x1 = pair(t, 8 * h + 2 * j + 1);
                 if constexpr (!FPB) {
-                  float hi[4], lo[4];
-#pragma unroll
-                  for (int i = 0; i < 4; ++i) mxint8_digits(x[4 * j + i], inv, hi[i], lo[i]);
-                  w[j] = f32x2_to_e4m3x2(hi[1], hi[0]) | (f32x2_to_e4m3x2(hi[3], hi[2]) << 16);
-                  d[j] = f32x2_to_e4m3x2(lo[1], lo[0]) | (f32x2_to_e4m3x2(lo[3], lo[2]) << 16);
+                  float2 hi0, lo0, hi1, lo1;
+                  mxint8_digits(x0, inv, hi0, lo0);
+                  mxint8_digits(x1, inv, hi1, lo1);
+                  w[j] = f32x2_to_e4m3x2(hi0.y, hi0.x) | (f32x2_to_e4m3x2(hi1.y, hi1.x) << 16);
+                  d[j] = f32x2_to_e4m3x2(lo0.y, lo0.x) | (f32x2_to_e4m3x2(lo1.y, lo1.x) << 16);
                 } else {
-                  w[j] = mxfp_pair<SIX>(x[4 * j + 1] * inv, x[4 * j] * inv) | (mxfp_pair<SIX>(x[4 * j + 3] * inv, x[4 * j + 2] * inv) << 16);
+                  const float2 y0 = __fmul2_rn(x0, splat(inv)), y1 = __fmul2_rn(x1, splat(inv));
+                  w[j] = mxfp_pair<SIX>(y0.y, y0.x) | (mxfp_pair<SIX>(y1.y, y1.x) << 16);
                   d[j] = 0;
                 }
               }
@@ -880,19 +917,19 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
               const float dev = amax * p.dev;
               const TieTest<SIX> tie(inv, dev);
               const bool edge = ((__float_as_uint(amax + dev) ^ __float_as_uint(amax - dev)) >> 23) != 0;
-              bool close = edge;
-#pragma unroll
-              for (int j = 0; j < 16; ++j) close |= tie(t[j]) | tie(t2[j]);
-              if (close && valid) {
+              // (any binade at first: few lanes go on to ask which elements)
+              if ((edge || tie.any(t)) && valid) {
                 uint32_t which = 0;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) which |= (tie(t[j]) ? 1u << j : 0u) | (tie(t2[j]) ? 0x10000u << j : 0u);
+                for (int j = 0; j < 32; ++j) which |= tie(t[j]) ? 1u << j : 0u;
                 if (edge) which = 0xFFFFFFFFu;
-                near |= 1u << b;
-                p.near_which[4 * (size_t)m + b] = which;
-                atomicAdd(&settle->elements, __popc(which));
-                const int n = atomicAdd(&settle->entries, 1);
-                if (n < SETTLE_ENTRIES) settle->entry[n] = make_int4(m, b, (int)which, e);
+                if (which != 0) {
+                  near |= 1u << b;
+                  p.near_which[4 * (size_t)m + b] = which;
+                  atomicAdd(&settle->elements, __popc(which));
+                  const int n = atomicAdd(&settle->entries, 1);
+                  if (n < SETTLE_ENTRIES) settle->entry[n] = make_int4(m, b, (int)which, e);
+                }
               }
             }
           }
