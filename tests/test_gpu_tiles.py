@@ -155,3 +155,26 @@ def test_outputs_that_begin_between_sectors(option, main, branch, r, N):
     assert B.lq_get_device_status(0)[0] == 0
     B.lq_act_free(act)
     B.lq_layer_free(h)
+
+
+@pytest.mark.parametrize("M,K,N", [(2047, 40, 24), (2048, 40, 24), (2049, 40, 24), (2305, 3200, 24), (2300, 40, 3800)])
+def test_row_chunks_of_a_call_from_host_memory(M, K, N):
+    """Around the number of rows from which chunks differ in size, few bytes and many, row counts beside a tile: the bits of the call on device
+    memory, and nothing beside them."""
+    import torch
+    from tests.helpers import import_oracle_layer
+
+    rng = np.random.default_rng(M)
+    h, _ = import_oracle_layer(MXINT4._mx_layer(rng, K, N, 16, "w8a8"))
+    B.lq_layer_to_device(h, 0)
+    act, st = B.lq_act_create(h, M, 0), torch.cuda.current_stream().cuda_stream
+    x = torch.from_numpy(_x(rng, M, K)).pin_memory()
+    y, ref = torch.full((M + 1, N), float("nan")).pin_memory(), torch.empty(M, N, device="cuda")
+    B.lq_linear_forward_host(h, act, x.data_ptr(), M, y.data_ptr(), B.OUT_F32, st)
+    xd = x.cuda()
+    B.lq_quantize_act(h, xd.data_ptr(), M, act, st)
+    B.lq_linear_forward(h, act, ref.data_ptr(), B.OUT_F32, st)
+    assert torch.equal(y[:M], ref.cpu()) and bool(y[M].isnan().all())
+    assert B.lq_get_device_status(0)[0] == 0
+    B.lq_act_free(act)
+    B.lq_layer_free(h)
