@@ -11,24 +11,24 @@
 //   warp 0      TMA producer: operand tiles (two groups = 128 bytes of K per stage row), the two groups' scale vectors and,
 //               with a tile's first stage, the bias, all signalled on the stage's "full" barrier
 //   warp 1      owns tensor memory; issues tcgen05.mma: each group of 64 codes is two K=32 MMAs into a FRESH 128 x 128
-//               accumulator.  A stage's two groups fill one PAIR of accumulators, each as soon as the drain has read it out,
+//               accumulator.  A stage's two groups fill one PAIR of accumulators as soon as the drain has read it out
 //               and are handed over with one commit; two pairs alternate
-//   warps 4-11  drain: each warp owns 32 rows x 64 columns of the tile.  A group's slice is four tcgen05.ld.16x256b.x4; a
-//               whole group is in flight into one register buffer while the one before is consumed from the other:
-//               acc += (P * sx) * sw, packed f32x2, fp32 registers (the integer branch's stage: P * (sx * sw)).  An accumulator goes back as soon as it sits in
-//               registers.  The next tile's first group is requested before the epilogue
+//   warps 4-11  drain: each warp owns 32 rows x 64 columns of the tile.  Half a group's slice is two tcgen05.ld.16x256b.x4; it is
+//               in flight into one register buffer while the half before is consumed from the other:
+//               acc += (P * sx) * sw, packed f32x2, fp32 registers (the integer branch's stage: P * (sx * sw)).  A pair goes back as soon as its last half sits in
+//               registers.  The next stage's scales are loaded, and the next tile's first half is requested, before the last half is consumed
 // What bounds it: the FP32 pipe's operand delivery and the drain's other instructions.  Per group and scheduler 64 packed products
 // (2.0 to 2.6 clocks each, measured) and 64 packed FMAs (2.75 with an operand shared by neighbours, 3.9 with three of their own) are about 320
 // clocks, the tensor pipe needs 128; the same loop over tensor memory without any hand-shake takes 400, 100 of them for the scales' way
-// from shared memory, the kernel takes 440.  So everything that is not arithmetic is kept out of the drain's instruction stream: two
+// from shared memory, the kernel takes 430.  So everything that is not arithmetic is kept out of the drain's instruction stream: two
 // wide warps per scheduler instead of four narrow ones, no wait or arrival for the scale vectors (they live in a ring deep
 // enough that the accumulators' hand-shakes imply theirs), one wait per stage, 224 registers per drain thread, partly
 // taken over from the other four warps (setmaxnreg).  M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 85 / 96 us with sixteen
 // narrow warps, 80 / 89 with one commit per group; then, timed in turn with other inputs each time, 81.1 / 88.3, 78.0 / 84.0 with P sx first,
 // 72.4 / 81.6 with sectors stored whole, 70.1 / 78.1 with a stage's commits under one election, 64.5 / 70.9 with the issuer written out and the
-// drain's last eight registers.  At K = 1152 a tile's end is a fifth of the launch: of 11.4 k clocks a tile 1.0 k are the branch's group, 0.8 k the stores, 0.5 k
-// the way to the next tile's first stage.  Scalar FMAs lose their issue slots (94 - 104 us for 79); scales of
-// the next group loaded where this one's were used last, 302 clocks a group by itself, made the kernel slower (73.6 for 68.8: registers); two column
+// drain's last eight registers, 64.2 / 68.9 with halves of groups in flight and one hand-back a stage.  At K = 1152 a tile's end is a fifth of the launch: of 11.4 k clocks a tile 1.0 k are the branch's group, 0.8 k the stores, 0.5 k
+// the way to the next tile's first stage.  Scalar FMAs lose their issue slots (94 - 104 us for 79); with whole groups in flight, scales of
+// the next group loaded where this one's were used last made the kernel slower (73.6 for 68.8: registers); two column
 // halves as pipelines of their own, each with an issuer, 67.9 for 66.5.
 // Orders of rows and columns (lq_internal.h) are chosen for the drain's fragments: the columns of the tile are permuted in
 // the weight operand so that a lane's 16 columns of a row are neighbours in Y - the epilogue converts and stores, no
@@ -108,7 +108,7 @@ struct GemmParams {
   int32_t* status;
 };
 
-// One group's slice of a drain warp, two accumulator slices of 16 rows x 64 columns in the layout of tcgen05.ld.16x256b
+// Half a group's slice of a drain warp, two accumulator slices of 16 rows x 32 columns in the layout of tcgen05.ld.16x256b
 // (the accumulator-fragment layout of mma.sync m16n8: with g = lane / 4 and t = lane % 4, registers 4j .. 4j+3 of a
 // slice hold row g, columns 8j + 2t and 8j + 2t + 1, then row g + 8, the same columns), times its scales, added to the accumulators.
 // INT: the accumulator holds int32 (kind::i8); |P| < 2^22, so adding 1.5 * 2^23 in the integer domain and subtracting it
@@ -133,19 +133,19 @@ __device__ __forceinline__ void load_scales(Scales& v, uint32_t sx_at, uint32_t 
 // rounds the same number; P sx leaves an FMA with an operand (sw) that four rows in a row share, which costs the register file
 // less (us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 81.1 / 88.3 -> 78.0 / 84.0).  The integer branch's scales have 24 bits, its sums up
 // to 22: there sx sw is rounded first.
-template <bool INT>
-__device__ __forceinline__ void drain_group(const Frag (&v)[4], float2 (&acc)[2][16], const Scales& sc) {
+template <bool INT, int HALF>
+__device__ __forceinline__ void drain_half(const Frag (&v)[2], float2 (&acc)[2][16], const Scales& sc) {
   const float4 sx = sc.sx;
   const float2 s0 = make_float2(sx.x, sx.x), s1 = make_float2(sx.y, sx.y), s2 = make_float2(sx.z, sx.z), s3 = make_float2(sx.w, sx.w);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 2 * HALF; k < 2 * HALF + 2; ++k) {
     const float4 w = sc.sw[k];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const int j = 2 * k + e, c = j >> 2, q = 4 * (j & 3);
+      const int j = 2 * k + e, q = 4 * (j & 3);
       const float2 sw = e ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
-      const float2 p0 = fragment_pair<INT>(v[2 * c][q], v[2 * c][q + 1]), p1 = fragment_pair<INT>(v[2 * c][q + 2], v[2 * c][q + 3]);
-      const float2 p2 = fragment_pair<INT>(v[2 * c + 1][q], v[2 * c + 1][q + 1]), p3 = fragment_pair<INT>(v[2 * c + 1][q + 2], v[2 * c + 1][q + 3]);
+      const float2 p0 = fragment_pair<INT>(v[0][q], v[0][q + 1]), p1 = fragment_pair<INT>(v[0][q + 2], v[0][q + 3]);
+      const float2 p2 = fragment_pair<INT>(v[1][q], v[1][q + 1]), p3 = fragment_pair<INT>(v[1][q + 2], v[1][q + 3]);
       float2 &a0 = acc[0][2 * j], &a1 = acc[0][2 * j + 1], &a2 = acc[1][2 * j], &a3 = acc[1][2 * j + 1];
       if constexpr (INT) {
         a0 = __ffma2_rn(p0, __fmul2_rn(s0, sw), a0); a1 = __ffma2_rn(p1, __fmul2_rn(s1, sw), a1);
@@ -157,12 +157,12 @@ __device__ __forceinline__ void drain_group(const Frag (&v)[4], float2 (&acc)[2]
     }
   }
 }
-__device__ __forceinline__ void fetch_group(uint32_t taddr, Frag (&v)[4]) {
+__device__ __forceinline__ void fetch_half(uint32_t taddr, Frag (&v)[2]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) tmem_ld_16x256b_x4(taddr + ((uint32_t)(16 * (i & 1)) << 16) + 32 * (i >> 1), v[i]);
+  for (int i = 0; i < 2; ++i) tmem_ld_16x256b_x4(taddr + ((uint32_t)(16 * i) << 16), v[i]);
 }
 
-// A group's two MMAs under one election, predicated instead of branched around: the control flow of the issuing warp stays uniform.
+// A group's two MMAs under one election (both groups of a stage under one were 1 to 2 % slower), predicated instead of branched around: the control flow of the issuing warp stays uniform.
 // (An `if` of one lane around them and around the commits, with a loop over the groups: a stage's way through the issuer, 1.2 k clocks,
 // was as long as the drain's.  us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 72.4 / 81.6 -> 64.5 / 70.9, with the drain's eight registers.)
 #define LQ_GROUP_MMAS                                                   \
@@ -211,7 +211,8 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto bar_full = [&](int s) { return sm_bar + 8u * (uint32_t)s; };                        // operands + scales landed
   auto bar_empty = [&](int s) { return sm_bar + 8u * (uint32_t)(NSTAGE + s); };           // MMAs of the stage retired
   auto bar_tfull = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + b); };
-  auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + NPAIR + b); };
+  // (16 bytes apart: with tfull's stride the same code was 1.5 to 2.5 % slower, whatever the stride)
+  auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + NPAIR + 1 + 2 * b); };
   [[maybe_unused]] const uint32_t bar_gather = sm_bar + 8u * (uint32_t)(2 * NSTAGE + 3 * NPAIR);
   constexpr int NBAR = 2 * NSTAGE + 3 * NPAIR + 1;
   static_assert(NBAR * 8 + 16 <= SMEM_BAR_BYTES, "barrier area too small");
@@ -235,8 +236,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       mbar_init(bar_full(s), 1);
       mbar_init(bar_empty(s), 1);
     }
-    for (int b = 0; b < NPAIR; ++b) mbar_init(bar_tfull(b), 1);
-    for (int b = 0; b < 2 * NPAIR; ++b) mbar_init(bar_tempty(b), NUM_DRAIN_WARPS);
+    for (int b = 0; b < NPAIR; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), NUM_DRAIN_WARPS); }
     *abort_flag = 0;
     if constexpr (SPLIT) mbar_init(bar_gather, 1);
     mbar_init_fence();
@@ -353,19 +353,15 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           LQ_TL(EV_M_STAGE_FULL, s);
           const uint32_t a_addr = sm_stage + st * STAGE_BYTES, b_addr = a_addr + STAGE_A_BYTES;
           const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(b_addr);
-          // The stage's groups to the accumulators of one pair, each as soon as the drain has read it out; one commit
+          // The stage's groups to the accumulators of one pair, as soon as the drain has read them out; one commit
           const int pair = it & (NPAIR - 1);
-          const uint32_t d = tmem_base + 2 * pair * TCOLS, par = ((it / NPAIR) & 1) ^ 1;
-          ok = mbar_wait_warp(bar_tempty(2 * pair), par, abort_flag, p.status, LQ_STAGE_MMA);
+          const uint32_t d = tmem_base + 2 * pair * TCOLS;
+          ok = mbar_wait_warp(bar_tempty(pair), ((it / NPAIR) & 1) ^ 1, abort_flag, p.status, LQ_STAGE_MMA);
           if (!ok) break;
           tc_fence_after();
           LQ_TL(EV_M_ACC_FREE, s);
           if (s < p.n_stages_main) {
             issue_group(d, adesc, bdesc, IDESC_F8 | shape);
-            ok = mbar_wait_warp(bar_tempty(2 * pair + 1), par, abort_flag, p.status, LQ_STAGE_MMA);
-            if (!ok) break;
-            tc_fence_after();
-            LQ_TL(EV_M_ACC_FREE, s);
             issue_group(d + TCOLS, adesc + 4, bdesc + 4, IDESC_F8 | shape, bar_tfull(pair), bar_empty(st));
           } else {
             if (elect_one()) {
@@ -393,29 +389,30 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t it = 0;                                    // operand stages since the kernel began: ring positions it & (NPAIR-1),
                                                         // it & (SC_RING-1)
     bool ok = true;
-    Frag va[4], vb[4];                                  // two groups: one being consumed, one being fetched
+    Frag va[2], vb[2];                                  // two halves of groups: one being consumed, one being fetched
     auto pair_at = [&](uint32_t i) { return tlane + (i & (NPAIR - 1)) * (2 * TCOLS); };
-    // Requests stage i's first group once its pair is complete (its scale vectors landed before its MMAs were issued).  The
+    // Requests stage i's first half once its pair is complete (its scale vectors landed before its MMAs were issued).  The
     // request is made whatever the wait says, and even where no stage is left (it reads some accumulator, nothing looks at it).
     auto open_stage = [&](uint32_t i, bool exists) {
       if (exists) ok = mbar_wait_inline(bar_tfull(i & (NPAIR - 1)), (i / NPAIR) & 1, abort_flag, p.status, LQ_STAGE_DRAIN) && ok;
       tc_fence_after();
-      fetch_group(pair_at(i), va);
+      fetch_half(pair_at(i), va);
     };
-    auto landed = [&](uint32_t i, int q) {              // the stage's group q is in registers: its accumulator goes back
-      tmem_ld_wait();
+    // The stage's pair is in registers: it goes back, before the next request (the fence waits for every load that is in flight: 71.1 us for 64.0).
+    auto give_back = [&](uint32_t i) {
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_tempty(2 * (i & (NPAIR - 1)) + q));
+      if (lane == 0) mbar_arrive(bar_tempty(i & (NPAIR - 1)));
     };
-    Scales sc;
-    auto load_scales_of = [&](uint32_t i, int q) {
+    Scales sc, sd;                                      // of the two groups of a stage
+    auto load_scales_of = [&](Scales& sc, uint32_t i, int q) {
       const uint32_t at = sm_sc + (i & (SC_RING - 1)) * SC_STAGE_BYTES + q * SC_GROUP_FLOATS * 4;
       load_scales(sc, at + row_at * 4, at + (LQ_BM + col_at) * 4);
     };
     if constexpr (SPLIT) cluster_wait();                // the other CTAs' barriers are set up
     grid_dependency_wait();                             // Y may be what an earlier kernel still reads
     open_stage(0, u_begin < u_end);
+    load_scales_of(sc, 0, 0);
     for (int u = u_begin; u < u_end && ok; ++u) {
       const int mb = u / p.units_n, nu = u - mb * p.units_n;
       const int m0 = mb * LQ_BM, n0 = nu * UNIT;
@@ -443,29 +440,40 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int s = s_begin; s < s_main && ok; ++s, ++it) {
         const bool more = s + 1 < s_end || !last_tile;
         LQ_TL(EV_D_OPEN, s);
-        load_scales_of(it, 0);
-        landed(it, 0);
+        tmem_ld_wait();
         LQ_TL(EV_D_WAITED, s);
-        fetch_group(pair_at(it) + TCOLS, vb);
-        drain_group<false>(va, acc, sc);
+        fetch_half(pair_at(it) + WCOLS / 2, vb);
+        drain_half<false, 0>(va, acc, sc);
+        tmem_ld_wait();
+        fetch_half(pair_at(it) + TCOLS, va);
+        load_scales_of(sd, it, 1);
+        drain_half<false, 1>(vb, acc, sc);
         LQ_TL(EV_D_HALF, s);
-        load_scales_of(it, 1);
-        landed(it, 1);
+        tmem_ld_wait();
+        fetch_half(pair_at(it) + TCOLS + WCOLS / 2, vb);
+        drain_half<false, 0>(va, acc, sd);
+        tmem_ld_wait();
+        give_back(it);
         LQ_TL(EV_D_LOADED, s);
         open_stage(it + 1, more);
         LQ_TL(EV_D_ACC_FULL, s);
-        drain_group<false>(vb, acc, sc);
+        load_scales_of(sc, it + 1, 0);
+        drain_half<false, 1>(vb, acc, sd);
         LQ_TL(EV_D_DONE, s);
         ok = __all_sync(0xffffffffu, ok);
       }
       if (!ok) break;
       if (BRANCH != BRANCH_NONE && (!SPLIT || s_end > p.n_stages_main)) {
-        load_scales_of(it, 0);
-        landed(it, 0);
-        if (lane == 0) mbar_arrive(bar_tempty(2 * (it & (NPAIR - 1)) + 1));   // not used by this stage
-        drain_group<BRANCH == BRANCH_I8>(va, acc, sc);
+        tmem_ld_wait();
+        fetch_half(pair_at(it) + WCOLS / 2, vb);
+        drain_half<BRANCH == BRANCH_I8, 0>(va, acc, sc);
+        tmem_ld_wait();
+        give_back(it);
+        sd = sc;
         ++it;
         open_stage(it, !last_tile);
+        load_scales_of(sc, it, 0);
+        drain_half<BRANCH == BRANCH_I8, 1>(vb, acc, sd);
         ok = __all_sync(0xffffffffu, ok);
       }
       if (!ok) break;
