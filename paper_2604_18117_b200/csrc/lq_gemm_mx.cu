@@ -31,6 +31,8 @@
 // the weights each, and the weights stay packed up to shared memory, 4 bits as e2m1 (MXFP4) or 6 as e2m3 (integer codes),
 // where TMA spreads them out.  M = 8192, MXFP: 1152 x 3456 30.6 -> 29.4 us, 2240 x 6720 95.3 -> 91.1, 5600 x 2240 79.4 ->
 // 75.5; integer codes 33.8 -> 33.4 and 51.3 -> 50.5.
+// So do the weights that a pair needs for its next tile, too: where K is short enough they stay in shared memory, and the pair goes down its columns
+// (RESIDENT; the launcher has the rule).  5 to 10 % less time where it applies, and about as much under the power cap.
 // What was measured on the way here (PixArt block, four GEMMs): the branch on mma.sync in the drain warps took tensor
 // time from the main loop; TMA stores of the output (32 boxes of 2 KB, or 8 of 8 KB, per tile) cost 15 % against
 // plain stores - they share the TMA unit with the operand loads.
@@ -85,6 +87,7 @@ struct MxParams {
   int b_row;              // bytes of a weight row that a stage copies
   uint32_t b_format;      // format field of the weights in the instruction descriptor
   int b_wrap;             // Kpad / 128: stage s reads B (and its scales) at stage s mod b_wrap - the planes share the weights
+  int b_slots;            // RESIDENT: places of B in shared memory, the branch's last
   const LqMxMaps* maps;   // of the layer, for this width; its scale bytes are rows of 512: sfb [Kpad/128][tiles_n][sf_chunks], sfl2 (branch_mx)
                           // [tiles_n][sf_chunks].  The activations': tmSfa [Mpad/128][k_stages], tmSft (branch_mx) [Mpad/128][1 or 2]
   int sf_chunks;          // ceil(W / 128)
@@ -182,7 +185,9 @@ __device__ __forceinline__ void load_acts_stage(uint32_t full, uint32_t dst, con
 // PAIR: two CTAs of a cluster work on 256 rows x W columns (cta_group::2): each stages its own 128 rows of A and half of the
 // tile's columns of B, and each SM's tensor core reads B from both.  Both CTAs' copies complete on the first one's barrier, whose
 // CTA issues the MMAs for both.
-template <bool BRANCH_ACC, bool PAIR>
+// RESIDENT (pairs): a tile's columns of B - all stages of K, and the branch's - stay in shared memory while the pair goes through its run of tiles
+// column by column; only A comes anew with every tile.
+template <bool BRANCH_ACC, bool PAIR, bool RESIDENT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmT,
                   const __grid_constant__ CUtensorMap tmSfa, const __grid_constant__ CUtensorMap tmSft,
@@ -194,9 +199,14 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   constexpr int CTAS = PAIR ? 2 : 1;
   const int BW = W / CTAS;                                // columns of B in this CTA's shared memory
   const uint32_t rank = PAIR ? blockIdx.x & 1 : 0;
-  const uint32_t stage_bytes = STAGE_A_BYTES + (uint32_t)BW * LQ_KSTAGE;
-  const uint32_t off_sf = (uint32_t)NST * stage_bytes, off_sc = off_sf + NST * STAGE_SF_BYTES, off_bar = off_sc + 2 * SC_FLOATS * 4;
+  const uint32_t b_bytes = (uint32_t)BW * LQ_KSTAGE, stage_bytes = STAGE_A_BYTES + (RESIDENT ? 0 : b_bytes);
+  constexpr uint32_t SF_STAGE = RESIDENT ? SF_BYTES : STAGE_SF_BYTES, SFB_SLOT = STAGE_SF_BYTES - SF_BYTES;
+  const uint32_t off_b = (uint32_t)NST * stage_bytes, off_sf = off_b + (RESIDENT ? p.b_slots * b_bytes : 0u), off_sfb = off_sf + NST * SF_STAGE;
+  const uint32_t off_sc = off_sfb + (RESIDENT ? p.b_slots * SFB_SLOT : 0u), off_bar = off_sc + 2 * SC_FLOATS * 4;
   const uint32_t sm_stage = base, sm_sf = base + off_sf, sm_sc = base + off_sc, sm_bar = base + off_bar;
+  // a stage's B and its scale bytes: in the ring's slot, or RESIDENT in their own
+  auto b_at = [&](int st, int slot) { return RESIDENT ? base + off_b + (uint32_t)slot * b_bytes : sm_stage + (uint32_t)st * stage_bytes + STAGE_A_BYTES; };
+  auto sfb_at = [&](int st, int slot) { return RESIDENT ? base + off_sfb + (uint32_t)slot * SFB_SLOT : sm_sf + (uint32_t)st * SF_STAGE + SF_BYTES; };
   const float* sc_ptr = reinterpret_cast<const float*>(smem + off_sc);
   uint8_t* bar_ptr = smem + off_bar;
   // barrier map (8 bytes each)
@@ -211,9 +221,13 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int lane = threadIdx.x & 31;
   const bool has_branch = p.branch_steps > 0;
   const int nbst = !has_branch ? 0 : p.branch_mx == 3 ? 2 : 1;             // stages of the branch per tile
-  // this CTA's (pair's) contiguous run of tiles, row block major
-  const int unit = (int)blockIdx.x / CTAS, units = (int)gridDim.x / CTAS;
-  const long long work = (long long)((p.tiles_m + CTAS - 1) / CTAS) * p.tiles_n;
+  // this CTA's (pair's) contiguous run of tiles, row block major, RESIDENT column major
+  const int unit = (int)blockIdx.x / CTAS, units = (int)gridDim.x / CTAS, blocks_m = (p.tiles_m + CTAS - 1) / CTAS;
+  auto tile_at = [&](int w, int& mp, int& nu) {
+    if (RESIDENT) { nu = w / blocks_m; mp = w - nu * blocks_m; }
+    else { mp = w / p.tiles_n; nu = w - mp * p.tiles_n; }
+  };
+  const long long work = (long long)blocks_m * p.tiles_n;
   const int w_begin = (int)((work * unit) / units);
   const int w_end = (int)((work * (unit + 1)) / units);
 
@@ -254,14 +268,21 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     auto full_bar = [&](int st) { return first_bar + 8u * (uint32_t)(B_FULL + st); };
     const uint32_t arm = rank == 0 ? CTAS : 0;         // CTAs whose bytes this one announces
     const int block_last = p.tiles_m - 1;
-    auto load_b = [&](int st, int s, int nu) {         // the weights' half of main stage s; announces the whole stage
+    // The weights' half of main stage s; announces the whole stage.  RESIDENT: only where they are not there yet.  (Their place is free: the MMAs that read it
+    // last are at least as many stages back as the ring has slots, and the slot's own wait was for those.)
+    auto load_b = [&](int st, int s, int nu, bool there) {
       const int sb = s >= p.b_wrap ? s - p.b_wrap : s; // the lo digits' plane runs over the same weights
-      load_weights_stage<PAIR>(bar(B_FULL + st), arm * (STAGE_A_BYTES + (uint32_t)BW * p.b_row + SF_BYTES + sfb_bytes), full_bar(st),
-                               sm_stage + st * stage_bytes + STAGE_A_BYTES, &p.maps->b, sb * LQ_KSTAGE, nu * W + (int)rank * BW,
-                               sm_sf + st * STAGE_SF_BYTES + SF_BYTES, &p.maps->sfb, (sb * p.tiles_n + nu) * p.sf_chunks);
+      const uint32_t acts = STAGE_A_BYTES + SF_BYTES;
+      if (RESIDENT && (there || s >= p.b_wrap)) {
+        if (arm != 0 && elect_one()) mbar_expect_tx(bar(B_FULL + st), arm * acts);
+        __syncwarp();
+      } else {
+        load_weights_stage<PAIR>(bar(B_FULL + st), arm * (acts + (uint32_t)BW * p.b_row + sfb_bytes), full_bar(st), b_at(st, sb), &p.maps->b, sb * LQ_KSTAGE,
+                                 nu * W + (int)rank * BW, sfb_at(st, sb), &p.maps->sfb, (sb * p.tiles_n + nu) * p.sf_chunks);
+      }
     };
     auto load_a = [&](int st, int s, int mb) {
-      load_acts_stage<PAIR>(full_bar(st), sm_stage + st * stage_bytes, &tmA, s * LQ_KSTAGE, mb * LQ_BM, sm_sf + st * STAGE_SF_BYTES, &tmSfa,
+      load_acts_stage<PAIR>(full_bar(st), sm_stage + st * stage_bytes, &tmA, s * LQ_KSTAGE, mb * LQ_BM, sm_sf + st * SF_STAGE, &tmSfa,
                             (p.block0 + min(mb, block_last)) * p.k_stages + s);
     };
     auto advance = [&]() {
@@ -269,13 +290,18 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       if (++st == NST) { st = 0; par ^= 1; }
     };
     int early = 0;                                     // stages of the first tile whose weights were requested ahead
+    int mp, nu, nu_there = -1;                         // nu_there: whose weights are resident
     if (w_begin < w_end) {
+      tile_at(w_begin, mp, nu);
       early = min(NST, p.k_stages);
-      for (int s = 0; s < early; ++s) load_b(s, s, w_begin % p.tiles_n);
+      for (int s = 0; s < early; ++s) load_b(s, s, nu, false);
     }
     grid_dependency_wait();
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
-      const int mp = w / p.tiles_n, nu = w - mp * p.tiles_n, mb = mp * CTAS + (int)rank;   // (a pair's second block may not exist)
+      tile_at(w, mp, nu);
+      const int mb = mp * CTAS + (int)rank;            // (a pair's second block may not exist)
+      const bool there = RESIDENT && nu == nu_there;
+      nu_there = nu;
       const int m0 = mb * LQ_BM, n0 = nu * W, mc = min(mb, block_last);
       for (int s = 0; s < p.k_stages; ++s) {
         const bool ahead = tc == 0 && s < early;
@@ -284,7 +310,7 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           if (!ok) break;
         }
         LQ_TL(EV_P_SLOT_FREE, s);
-        if (!ahead) load_b(st, s, nu);
+        if (!ahead) load_b(st, s, nu, there);
         load_a(st, s, mb);
         advance();
         LQ_TL(EV_P_ISSUED, s);
@@ -295,14 +321,14 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         ok = mbar_wait_warp(bar(B_EMPTY + st), par, abort_flag, p.status, LQ_STAGE_PRODUCER);
         if (!ok) break;
         const uint32_t a_dst = sm_stage + st * stage_bytes, full = full_bar(st);
+        const bool fetch = !RESIDENT || (!there && bs == 0);
         if (elect_one()) {
-          if (arm != 0) mbar_expect_tx(bar(B_FULL + st), arm * (stage_bytes + (p.branch_mx ? SF_BYTES + sfb_bytes : 0)));
+          if (arm != 0) mbar_expect_tx(bar(B_FULL + st), arm * (STAGE_A_BYTES + (p.branch_mx ? SF_BYTES : 0) + (fetch ? b_bytes + (p.branch_mx ? sfb_bytes : 0) : 0u)));
           tma_load_2d<PAIR>(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
-          tma_load_2d<PAIR>(a_dst + STAGE_A_BYTES, &p.maps->l2, 0, n0 + (int)rank * BW, full);
+          if (fetch) tma_load_2d<PAIR>(b_at(st, p.b_wrap), &p.maps->l2, 0, n0 + (int)rank * BW, full);
           if (p.branch_mx) {   // the block scales of T (rows) and of L2 (columns) along the rank
-            const uint32_t sf_dst = sm_sf + st * STAGE_SF_BYTES;
-            tma_load_2d<PAIR>(sf_dst, &tmSft, 0, (p.block0 + mc) * nbst + bs, full);
-            tma_load_2d<PAIR>(sf_dst + SF_BYTES, &p.maps->sfl2, 0, nu * p.sf_chunks, full);
+            tma_load_2d<PAIR>(sm_sf + st * SF_STAGE, &tmSft, 0, (p.block0 + mc) * nbst + bs, full);
+            if (fetch) tma_load_2d<PAIR>(sfb_at(st, p.b_wrap), &p.maps->sfl2, 0, nu * p.sf_chunks, full);
           }
         }
         __syncwarp();
@@ -345,15 +371,15 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     int st = 0;                                        // ring slot and its parity
     bool ok = true;
     const uint32_t tsfa = tmem_base + TM_SFA, tsfb = tmem_base + TM_SFB;
-    auto copy_scales = [&](int st) {
-      const uint32_t sf = sm_sf + st * STAGE_SF_BYTES;
+    auto copy_scales = [&](int st, int slot) {
+      const uint32_t sfb = sfb_at(st, slot);
       auto cp = [&](uint32_t to, uint32_t from) {
         if (PAIR) tc_cp_sf_pair(to, make_smem_desc_plain(from, 16, 128));
         else tc_cp_sf(to, make_smem_desc_plain(from, 16, 128));
       };
-      cp(tsfa, sf);
-      cp(tsfb, sf + SF_BYTES);
-      if (p.sf_chunks == 2) cp(tsfb + 4, sf + 2 * SF_BYTES);
+      cp(tsfa, sm_sf + st * SF_STAGE);
+      cp(tsfb, sfb);
+      if (p.sf_chunks == 2) cp(tsfb + 4, sfb + SF_BYTES);
     };
     auto mma_mx = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
       if (PAIR) tc_mma_mx_pair(d, a, b, idesc, tsfa, tsfb, 1u);
@@ -378,11 +404,10 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (!ok) break;
         tc_fence_after();
         LQ_TL(EV_M_STAGE_FULL, s);
-        const uint32_t a_addr = sm_stage + st * stage_bytes;
-        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + STAGE_A_BYTES);
-        const uint32_t sf = sm_sf + st * STAGE_SF_BYTES;
+        const int sb = s >= p.b_wrap ? s - p.b_wrap : s;
+        const uint64_t adesc = make_smem_desc(sm_stage + st * stage_bytes), bdesc = make_smem_desc(b_at(st, sb));
         auto issue = PAIR ? issue_main_stage_pair : issue_main_stage_one;
-        issue(d, adesc, bdesc, (idesc_mx(W, 0) | p.b_format) + ROWS256, make_smem_desc_plain(sf, 16, 128), make_smem_desc_plain(sf + SF_BYTES, 16, 128),
+        issue(d, adesc, bdesc, (idesc_mx(W, 0) | p.b_format) + ROWS256, make_smem_desc_plain(sm_sf + st * SF_STAGE, 16, 128), make_smem_desc_plain(sfb_at(st, sb), 16, 128),
               (uint32_t)(p.sf_chunks == 2), (uint32_t)s, bar(B_EMPTY + st));
         if (++st == NST) { st = 0; par ^= 1; }
         LQ_TL(EV_M_ISSUED, s);
@@ -396,11 +421,10 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           if (!ok) break;
         }
         tc_fence_after();
-        const uint32_t a_addr = sm_stage + st * stage_bytes;
-        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + STAGE_A_BYTES);
+        const uint64_t adesc = make_smem_desc(sm_stage + st * stage_bytes), bdesc = make_smem_desc(b_at(st, p.b_wrap));
         if (elect_one()) {
           if (p.branch_mx) {
-            copy_scales(st);
+            copy_scales(st, p.b_wrap);
             if (p.branch_mx == 2) {
               for (int c = 0; c < p.branch_steps; ++c)
                 for (int q = 0; q < 4; ++q) {
@@ -444,8 +468,9 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     bool ok = true;
     grid_dependency_wait();                             // Y may be what an earlier kernel still reads
     for (int w = w_begin; w < w_end && ok; ++w, ++tc) {
-      const int mp = w / p.tiles_n, nu = w - mp * p.tiles_n, mb = mp * CTAS + (int)rank;
-      const int buf = tc & 1;
+      int mp, nu;
+      tile_at(w, mp, nu);
+      const int mb = mp * CTAS + (int)rank, buf = tc & 1;
       LQ_TL(EV_D_OPEN, 0);
       ok = mbar_wait_warp(bar(B_TFULL + buf), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN) &&
            mbar_wait_warp(bar(B_RFULL + buf), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN);
@@ -545,6 +570,13 @@ int ring_stages(int bw) {      // bw: columns of B per CTA
 int smem_bytes(int bw) {
   return FIXED_SMEM + ring_stages(bw) * (STAGE_A_BYTES + bw * LQ_KSTAGE + STAGE_SF_BYTES);
 }
+// The same with `slots` stages of B resident (negative: they do not fit).
+int resident_smem(int bw, int slots, int stages) {
+  return FIXED_SMEM + slots * (bw * LQ_KSTAGE + STAGE_SF_BYTES - SF_BYTES) + stages * (STAGE_A_BYTES + SF_BYTES);
+}
+int resident_stages(int bw, int slots) {
+  return std::min(MAX_STAGES, (MAX_SMEM - resident_smem(bw, slots, 0)) / (STAGE_A_BYTES + SF_BYTES));
+}
 
 // Index (LQ_MX_WIDTHS) of the tile width for a launch.  Model, in clocks: a stage takes the longest of its MMAs (2 W, and 40 where
 // one stage's meet the next's), its operands' way from the L2 (70 bytes per clock and SM) and its hand-shakes (350: what a
@@ -572,7 +604,8 @@ int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas, bool pair) 
 
 lq_status lq_gemm_mx_prepare(int device) {
   if (cudaSetDevice(device) != cudaSuccess) return LQ_ERR_CUDA;
-  for (auto* kernel : {lq_gemm_mx_kernel<false, false>, lq_gemm_mx_kernel<true, false>, lq_gemm_mx_kernel<false, true>, lq_gemm_mx_kernel<true, true>})
+  for (auto* kernel : {lq_gemm_mx_kernel<false, false, false>, lq_gemm_mx_kernel<true, false, false>, lq_gemm_mx_kernel<false, true, false>,
+                       lq_gemm_mx_kernel<true, true, false>, lq_gemm_mx_kernel<false, true, true>, lq_gemm_mx_kernel<true, true, true>})
     if (lq_note_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM)) != cudaSuccess) return LQ_ERR_CUDA;
   return LQ_OK;
 }
@@ -607,9 +640,20 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   const long long tiles = (long long)lq_ceil_div(p.tiles_m, c) * p.tiles_n;
   ctas = c * (int)std::min<long long>(ctas / c, tiles);
   const bool acc = p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx;
-  auto* kernel = acc ? (pair ? lq_gemm_mx_kernel<true, true> : lq_gemm_mx_kernel<true, false>)
-                     : (pair ? lq_gemm_mx_kernel<false, true> : lq_gemm_mx_kernel<false, false>);
+  size_t smem = (size_t)smem_bytes(p.width / c);
+  // Weights stay where they fit beside four stages of A (K up to 1152 at 224 columns, 1280 at 160), a pair has two tiles or more, and the launch is where it was timed
+  // to pay, us with weights fetched for every tile / kept, MXFP4, MXINT4 with W8A8, MXINT4 x 8: M = 8192, 1152 x 3456 29.0 / 27.5, 32.4 / 31.0, 50.0 / 47.7; 1024 x 4096 32.2 / 29.1,
+  // 35.0 / 33.5, 54.7 / 51.1; 768 x 3072 21.1 / 19.0, 25.5 / 26.3, 32.7 / 30.5; 640 x 8192 45.1 / 46.9, 53.0 / 54.1, 71.9 / 73.7.  Few rows leave little to
+  // keep them for (M = 2048, 1152 x 4608: 13.6 / 13.4, 14.4 / 14.7, 20.2 / 20.0; M = 3000: 16.3 / 15.7, 18.3 / 18.0, 25.8 / 25.3).  Down a column of many rows the pairs
+  // are spread over all of A and Y, row blocks keep them together: M = 16384, 1152 x 1152 24.3 / 23.0, 25.9 / 25.5, 39.9 / 38.0; M = 32768 42.4 / 44.9, 46.7 / 48.3, 73.0 / 78.0.
+  p.b_slots = p.b_wrap + (L->r > 0);
+  const int left = std::min(resident_stages(p.width / c, p.b_slots), p.b_wrap), blocks = lq_ceil_div(p.tiles_m, c);   // (no more stages than K has: load_b)
+  const bool resident = pair && tiles >= 2 * (ctas / 2) && left >= 4 && blocks >= 10 && blocks <= 64 && p.b_wrap >= (acc ? 7 : 6);
+  if (resident) { p.stages = left; smem = (size_t)resident_smem(p.width / c, p.b_slots, left); }
+  auto* kernel = resident ? (acc ? lq_gemm_mx_kernel<true, true, true> : lq_gemm_mx_kernel<false, true, true>)
+                 : acc    ? (pair ? lq_gemm_mx_kernel<true, true, false> : lq_gemm_mx_kernel<true, false, false>)
+                          : (pair ? lq_gemm_mx_kernel<false, true, false> : lq_gemm_mx_kernel<false, false, false>);
   p.maps = L->d_maps + 2 * wi + c - 1;
-  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, (size_t)smem_bytes(p.width / c), st, A->tmA, A->tmT, A->tmSfa, A->tmSft, p);
+  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, smem, st, A->tmA, A->tmT, A->tmSfa, A->tmSft, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

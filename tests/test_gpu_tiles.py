@@ -178,3 +178,39 @@ def test_row_chunks_of_a_call_from_host_memory(M, K, N):
     assert B.lq_get_device_status(0)[0] == 0
     B.lq_act_free(act)
     B.lq_layer_free(h)
+
+
+@pytest.mark.parametrize("ctas", [6, 0])
+@pytest.mark.parametrize("width", [64, 0])
+@pytest.mark.parametrize("main,branch,r,K", [("mxint4", "none", 0, 1152), ("mxint4", "w8a8", 32, 1152), ("mxint4", "w16a16", 24, 1030 + 2), ("mxfp4", "mxfp8", 64, 1400),
+                                             ("mxint8", "mxint8", 64, 1152), ("mxint8", "mxint4", 128, 1160)])
+def test_weights_that_stay_while_a_pair_goes_down_its_columns(option, main, branch, r, K, width, ctas):
+    """Runs of tiles that begin and end within a column, change columns once or more often, a pair without a second row block, a last tile of eight
+    columns, K at and beyond what stays: the bits of single CTAs."""
+    import torch
+    from tests.helpers import import_oracle_layer, import_oracle_mxfp_layer, import_oracle_mxint_layer
+
+    rng = np.random.default_rng(K + width)
+    M, N = 2600, 1160
+    mod = {"mxint4": MXINT4, "mxfp4": MXFP, "mxint8": MXINT8}[main]
+    layer = mod._mx_layer(rng, K, N, r, branch) if main == "mxint4" else mod._layer(rng, K, N, r, branch)
+    h, _ = {"mxint4": import_oracle_layer, "mxfp4": import_oracle_mxfp_layer, "mxint8": import_oracle_mxint_layer}[main](layer)
+    B.lq_layer_to_device(h, 0)
+    act = B.lq_act_create(h, M, 0)
+    x, st = torch.from_numpy(_x(rng, M, K)).cuda(), torch.cuda.current_stream().cuda_stream
+    B.lq_quantize_act(h, x.data_ptr(), M, act, st)
+    option("gemm_width", width)
+
+    def forward(pair, n):
+        option("gemm_pair", pair, default=1)
+        option("gemm_ctas", n)
+        y = torch.full((M, N), float("nan"), device="cuda")
+        B.lq_linear_forward(h, act, y.data_ptr(), B.OUT_F32, st)
+        return y
+
+    alone, pairs = forward(0, 0), forward(1, ctas)
+    torch.cuda.synchronize()
+    assert B.lq_get_device_status(0)[0] == 0
+    assert torch.equal(alone, pairs)
+    B.lq_act_free(act)
+    B.lq_layer_free(h)
