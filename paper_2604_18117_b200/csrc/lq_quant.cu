@@ -304,21 +304,24 @@ __device__ __forceinline__ uint2 sint4_codes8(const uint4& v, float rcp, bool co
                     f32x2_to_e4m3x2(q[2].y, q[2].x) | (f32x2_to_e4m3x2(q[3].y, q[3].x) << 16));
 }
 
-// Scale of a row's branch codes (its maximum over qm, 1 for a row of zeros) and the reciprocal that codes are formed with (see the top).
+// Scale of a row's branch codes (its maximum over qm, 1 for a row of zeros) and the reciprocal that codes are formed with (see the top).  All of
+// a tile's warps wait for it between its two walks, so it is worked out without a division: the maximum over a constant is the correctly rounded quotient after
+// one correction step (checked for every fp16 maximum on the host), and where codes do not need the quotient an approximate reciprocal will do.
 struct BranchScale {
-  float sb, rcp, inv;    // rcp: fl32(1 / sb), inv: the same or a few ulps beside it
+  float sb, inv;
   bool exact;            // this row's codes need the quotient: ties elsewhere, or a maximum that is no number
   // rqm: fl32(1 / qm); near: half an ulp of qm / 2
   __device__ __forceinline__ BranchScale(uint32_t max_bits, float qm, float rqm, float near) {
     const float rm = __half2float(__ushort_as_half((unsigned short)max_bits));
-    sb = rm == 0.f ? 1.f : __fdiv_rn(rm, qm);
-    inv = rcp = __frcp_rn(sb);
+    const float q0 = __fmul_rn(rm, rqm), q1 = __fmaf_rn(__fmaf_rn(q0, -qm, rm), rqm, q0);
+    sb = rm == 0.f ? 1.f : max_bits >= 0x7C00u ? rm : q1;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(sb));
     const float a = (float)((max_bits & 0x3FFu) | (max_bits < 0x400u ? 0u : 0x400u));       // significand of the maximum
     exact = max_bits >= 0x7C00u || (a != 0.f && __fmul_rn(rintf(__fmul_rn(a, rqm)), qm) == a);
     // The code of max / 2 is rint(fl32(max / 2 / sb)).  The quotient is within 2^-23 of qm / 2, which is half of an odd number plus one:
     // ties go up, and what is no more than half an ulp below is a tie.  (max / 2 - sb qm / 2 is exact, half of the division's remainder.)
     const bool up = __fmaf_rn(sb, -0.5f * qm, 0.5f * rm) >= -near * sb;
-    if ((__fmaf_rn(0.5f * rm, rcp, -0.5f * qm) >= 0.f) != up) inv = __uint_as_float(__float_as_uint(rcp) + (up ? 4u : -4u));
+    if ((__fmaf_rn(0.5f * rm, inv, -0.5f * qm) >= 0.f) != up) inv = __uint_as_float(__float_as_uint(inv) + (up ? 4u : -4u));
   }
 };
 // Branch codes of eight values: the low byte of the code + MAGIC is the code.
@@ -1130,7 +1133,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const BranchScale mine((uint32_t)mx[sr], p.qm, p.rqm, p.near_tie);
         {
           exact = __any_sync(0xffffffffu, mine.exact);
-          const float own = exact ? mine.rcp : mine.inv;
+          const float own = exact ? __frcp_rn(mine.sb) : mine.inv;
           const float sb = __shfl_xor_sync(0xffffffffu, mine.sb, 8), inv = __shfl_xor_sync(0xffffffffu, own, 8);
           sb_a = box ? sb : mine.sb; sb_b = box ? mine.sb : sb;
           inv_a = box ? inv : own; inv_b = box ? own : inv;

@@ -69,6 +69,18 @@ def test_fma_corrected_quotient_is_the_correctly_rounded_division():
 
 
 @pytest.mark.parametrize("qm", [127, 31])
+def test_row_scale_without_a_division(qm):
+    """sb = fl32(max / qm) of every finite fp16 maximum from the product with fl32(1 / qm) and one correction step.  (The last FMA is rounded from a sum in 64 bits: a
+    quotient is never nearer than 2^-33 to the middle between two binary32 numbers.)"""
+    rm = np.arange(1, 0x7C00, dtype=np.uint16).view(np.float16).astype(np.float32)
+    rqm = np.float64(np.float32(1) / np.float32(qm))
+    q0 = (rm * rqm).astype(np.float32).astype(np.float64)
+    rest = rm.astype(np.float64) - q0 * qm
+    assert np.array_equal(rest, rest.astype(np.float32))
+    assert np.array_equal((q0 + rest * rqm).astype(np.float32), rm / np.float32(qm))
+
+
+@pytest.mark.parametrize("qm", [127, 31])
 def test_one_fma_with_a_chosen_reciprocal_gives_the_codes_of_the_quotient(qm):
     """Branch codes by x -> rint(x inv) (one FMA with 1.5 * 2^23: the product is not rounded before) for every finite fp16 row
     maximum and, of the values up to it, the two next to every tie (k + 1/2) max / qm and the tie itself: the codes of the definition,
@@ -78,13 +90,16 @@ def test_one_fma_with_a_chosen_reciprocal_gives_the_codes_of_the_quotient(qm):
     significand = (bits & 0x3FF) | np.where(bits < 0x400, 0, 0x400)
     rm = bits[significand % qm != 0].astype(np.uint16).view(np.float16).astype(np.float32)
     sb = rm / np.float32(qm)
-    rcp = (1.0 / sb.astype(np.float64)).astype(np.float32)
+    exact = (1.0 / sb.astype(np.float64)).astype(np.float32)
     near = {127: 2.0 ** -19, 31: 2.0 ** -21}[qm]                                         # half an ulp of qm / 2
     up = 0.5 * rm.astype(np.float64) - sb.astype(np.float64) * (0.5 * qm) >= -near * sb  # exact: 31 bits
     assert np.array_equal(up, np.rint((np.float32(0.5) * rm) / sb) == (qm + 1) // 2)
-    above = 0.5 * rm.astype(np.float64) * rcp.astype(np.float64) - 0.5 * qm >= 0          # exact: 35 bits
-    inv = np.where(above == up, rcp.view(np.int32), rcp.view(np.int32) + np.where(up, 4, -4)).astype(np.int32).view(np.float32)
-    assert (above != up).sum() > 1000
+    codes = []                                                       # of reciprocals up to an ulp and a half off
+    for off in (-1, 0, 1):
+        rcp = (exact.view(np.int32) + off).astype(np.int32).view(np.float32)
+        above = 0.5 * rm.astype(np.float64) * rcp.astype(np.float64) - 0.5 * qm >= 0      # exact: 35 bits
+        codes.append(np.where(above == up, rcp.view(np.int32), rcp.view(np.int32) + np.where(up, 4, -4)).astype(np.int32).view(np.float32))
+        assert (above != up).sum() > 1000
     ties = 0
     for k in range(qm):
         t = (k + 0.5) * rm.astype(np.float64) / qm
@@ -93,6 +108,7 @@ def test_one_fma_with_a_chosen_reciprocal_gives_the_codes_of_the_quotient(qm):
             x = (mid.view(np.int16) + step).astype(np.int16).view(np.float16).astype(np.float64)
             x = np.where((x >= 0) & (x <= rm), x, 0.0)
             code = np.rint((x.astype(np.float32) / sb).astype(np.float64))
-            assert np.array_equal(np.rint(x * inv.astype(np.float64)), code), k
+            for inv in codes:
+                assert np.array_equal(np.rint(x * inv.astype(np.float64)), code), k
             ties += (x * 2 * qm == (2 * k + 1) * rm.astype(np.float64)).sum()
     assert ties > 10000
