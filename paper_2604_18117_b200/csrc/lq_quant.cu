@@ -23,7 +23,7 @@
 //               10-30 % slower
 //   warp 4      TMA producer of the first factor's slabs, one per stage, and their scale bytes.  (The MMA warp fetched them at
 //               first, after the chunk it had just issued: the slabs were late, 24 against 30 us at K = 4608)
-//   warp 2      owns tensor memory, issues the MMAs of a chunk once its slabs are complete.  The MMA is 128 rows high; the rows
+//   warp 2      owns tensor memory, issues the MMAs of a chunk once its slabs are complete.  The MMA is 128 rows high, or 64 (mma_64_rows); the rows
 //               beyond TR read whatever follows in shared memory and their results are never looked at (rows are
 //               independent, and the tensor cores are idle here otherwise)
 //   warps 0-1   a4: lane = row; the rank-r row is read from tensor memory under the next tile's quantization (two
@@ -607,6 +607,11 @@ __device__ __forceinline__ void issue_four_mx(uint32_t d, uint64_t a, uint64_t b
       : "memory");
 }
 
+// What bounds a narrow MMA is its A operand's way from shared memory, so tiles of up to 32 rows use MMAs of 64 (block-scaled ones have no fewer than
+// 128).  Their rows lie in tensor memory sixteen to a quarter of the lanes, and the two warps of a4 reach the first two quarters.  us with 128 rows / 64, X in the L2:
+// W16A16 rank 24, M x K = 1365 x 2312 8.6 / 7.5, 1 x 4608 12.0 / 10.4, 120 x 1152 5.1 / 4.7; W8A8 rank 32 9.1 / 8.7, 11.1 / 10.3, 5.9 / 5.7; rank 128 12.1 / 11.8, 15.0 / 14.6, 8.0 / 7.8.
+__device__ __forceinline__ constexpr bool mma_64_rows(int br, int groups) { return (br == BR_INT || br == BR_F16) && groups <= 4; }
+
 template <int MAIN, int BR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmL1,
@@ -730,7 +735,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const int cols = p.rn * p.bplanes;
-    const uint32_t shape = idesc_shape(cols), tsf = tmem + (uint32_t)(p.sets * p.nacc * cols);
+    const uint32_t shape = idesc_shape(cols) - (mma_64_rows(BR, RG) ? (uint32_t)(64 >> 4) << 24 : 0u), tsf = tmem + (uint32_t)(p.sets * p.nacc * cols);
     bool ok = true;
     uint32_t tc = 0, par = 0;
     int slot = 0;
@@ -782,7 +787,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     if (warp == 0) fetch_ahead();
     grid_dependency_wait();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0) + ((uint32_t)(32 * warp) << 16);
-    const int nacc = min(p.nacc, p.nst), row = 32 * warp + lane;
+    const bool low = mma_64_rows(BR, RG);                // sixteen rows to a warp
+    const int nacc = min(p.nacc, p.nst), row0 = (low ? 16 : 32) * warp, row = low && lane >= 16 ? TR : row0 + lane;
     uint32_t tc = 0;
     SettleList* const settle = reinterpret_cast<SettleList*>(smem + sm.off_l1);
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++tc) {
@@ -792,7 +798,7 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       if (!mbar_wait_warp(bar_tfull(tc & 1), (tc >> 1) & 1, abort_flag, p.status, LQ_STAGE_DRAIN)) break;
       tc_fence_after();
       uint8_t* const tqr = p.tq + (size_t)m * p.tq_stride;
-      if (32 * warp < TR) {
+      if (row0 < TR) {
         // 32 columns of the row from `col` on (zeros beyond the rank): the sum over the accumulators (and the first factor's digit planes)
         auto fetch = [&](int col, float (&t)[32]) {
           const bool both = col + 16 < p.rn;

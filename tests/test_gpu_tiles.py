@@ -214,3 +214,15 @@ def test_weights_that_stay_while_a_pair_goes_down_its_columns(option, main, bran
     assert torch.equal(alone, pairs)
     B.lq_act_free(act)
     B.lq_layer_free(h)
+
+
+@pytest.mark.parametrize("groups", [1, 2, 4, 5])
+@pytest.mark.parametrize("M,r", [(7, 8), (33, 24), (70, 64)])
+def test_row_tiles_on_either_side_of_32_rows(option, groups, M, r):
+    """The down-projection of tiles of up to 32 rows is 64 rows high and lies elsewhere in tensor memory: fp16 and integer factors, ranks of one and more
+    blocks, rows of one warp and of two."""
+    option("quant_warps", groups)
+    rng = np.random.default_rng(M + groups)
+    X = _x(rng, M, 1160)
+    SINT4._check(SINT4._random_layer(rng, 1160, 40, r, "w16a16"), X, tol32=SINT4.TOL_F32 * 5)
+    MXINT4._check(MXINT4._mx_layer(rng, 1160, 40, r, "w6a6"), X)
