@@ -119,9 +119,12 @@ __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddep
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- thread-block clusters: rendezvous, and barriers of a peer CTA ---------------------------
+// HANDS_OVER: what this thread has written before is for the others to read once they have waited.
+template <bool HANDS_OVER = true>
 __device__ __forceinline__ void cluster_arrive() {
   __syncwarp();      // the barrier's aligned form wants the warp's lanes together, whatever branches lie behind them
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  if constexpr (HANDS_OVER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
   __syncwarp();

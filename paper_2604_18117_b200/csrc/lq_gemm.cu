@@ -549,7 +549,10 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if constexpr (SPLIT) {
     // Every CTA of the cluster adds up its items, in the order of the stages, and stores them.
     if (warp < FIRST_DRAIN_WARP) cluster_wait();
-    if (drained && mbar_wait_warp<PEER_DATA>(bar_gather, 0, abort_flag, p.status, LQ_STAGE_DRAIN)) {
+    const bool gathered = drained && mbar_wait_warp<PEER_DATA>(bar_gather, 0, abort_flag, p.status, LQ_STAGE_DRAIN);
+    if (warp >= FIRST_DRAIN_WARP && !gathered) mbar_settle(bar_gather, 0);
+    cluster_arrive<false>();                            // nothing is on its way to this CTA any more
+    if (gathered) {
       const int dwarp = warp - FIRST_DRAIN_WARP, mb = u_begin / p.units_n, nu = u_begin - mb * p.units_n;
       const int row = mb * LQ_BM + 32 * (warp & 3) + (lane >> 2), col = nu * UNIT + ((warp - FIRST_DRAIN_WARP) >> 2) * WCOLS + 16 * (lane & 3);
 #pragma unroll 2
@@ -591,9 +594,11 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
   }
-  // SPLIT: all that this CTA was to be sent is here, so it may leave.  Where a wait has run out it stays until the others have left or
-  // stay, too: they may still be storing to it.
-  if (SPLIT && *abort_flag) cluster_sync();
+  // SPLIT: this CTA's own copies are read from its shared memory, and only who receives them knows when they have landed.  So it stays
+  // until every CTA of the cluster has what it was to be sent, also where a wait has run out.  The stores of Y lie between arriving and
+  // waiting.  (us, leaving at once / staying / staying, with an arrival that releases what was written: M x K x N = 1 x 1152 x 1152
+  // 4.62 / 4.67 / 4.83, 120 x 1152 x 4608 7.43 / 7.52 / 7.66, 120 x 8192 x 1152 9.56 / 9.64 / 9.82.)
+  if constexpr (SPLIT) cluster_wait();
 }
 
 // Self-test of the bounded wait: one warp waits on a barrier that nothing ever arrives on.

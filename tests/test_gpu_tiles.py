@@ -43,6 +43,41 @@ def test_sint4_tiles_shared_by_a_cluster(option, split, M, K, N, r, branch):
                  tol32=SINT4.TOL_F32 * (5 if branch == "w16a16" else 1))
 
 
+@pytest.mark.parametrize("split", [2, 4, 8])
+@pytest.mark.parametrize("M", [1, 9, 25, 128])
+def test_launches_close_behind_a_shared_tile_find_its_sums_as_they_were(option, split, M):
+    """The CTAs of a cluster leave while kernels behind them begin to fill the shared memory that the partial sums were sent from.  Four layers
+    in turn, twenty times, have the bits of each by itself; of the parts of a tile some have no row, or all have."""
+    import torch
+    from tests.helpers import import_oracle_layer
+
+    option("gemm_split", split)
+    rng = np.random.default_rng(split + M)
+    st, linears = torch.cuda.current_stream().cuda_stream, []
+    for K, N, r, branch in ((1152, 1160, 32, "w8a8"), (576, 2048, 0, "none"), (2048, 136, 24, "w16a16"), (1088, 1024, 16, "w4a8")):
+        h, _ = import_oracle_layer(SINT4._random_layer(rng, K, N, r, branch))
+        B.lq_layer_to_device(h, 0)
+        linears.append((h, B.lq_act_create(h, M, 0), torch.from_numpy(_x(rng, M, K)).cuda(), N))
+
+    def forward(h, act, x, N):
+        y = torch.full((M, N), float("nan"), device="cuda")
+        B.lq_quantize_act(h, x.data_ptr(), M, act, st)
+        B.lq_linear_forward(h, act, y.data_ptr(), B.OUT_F32, st)
+        return y
+
+    alone = []
+    for l in linears:
+        alone.append(forward(*l))
+        torch.cuda.synchronize()
+    chain = [forward(*l) for _ in range(20) for l in linears]
+    torch.cuda.synchronize()
+    assert B.lq_get_device_status(0)[0] == 0
+    assert all(torch.equal(y, alone[i % len(linears)]) for i, y in enumerate(chain))
+    for h, act, _, _ in linears:
+        B.lq_act_free(act)
+        B.lq_layer_free(h)
+
+
 @pytest.mark.parametrize("pair", [0, 1])
 @pytest.mark.parametrize("width", [64, 128, 160, 192, 224])
 @pytest.mark.parametrize("main,branch,r", [("mxint4", "none", 0), ("mxint4", "w8a8", 32), ("mxint4", "w16a16", 24), ("mxfp4", "mxfp8", 64),
