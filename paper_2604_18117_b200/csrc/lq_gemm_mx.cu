@@ -32,7 +32,7 @@
 // where TMA spreads them out.  M = 8192, MXFP: 1152 x 3456 30.6 -> 29.4 us, 2240 x 6720 95.3 -> 91.1, 5600 x 2240 79.4 ->
 // 75.5; integer codes 33.8 -> 33.4 and 51.3 -> 50.5.
 // So do the weights that a pair needs for its next tile, too: where K is short enough they stay in shared memory, and the pair goes down its columns
-// (RESIDENT; the launcher has the rule).  5 to 10 % less time where it applies, and about as much under the power cap.
+// (RESIDENT; weights_stay has the rule).  5 to 10 % less time where it applies, and about as much under the power cap.
 // What was measured on the way here (PixArt block, four GEMMs): the branch on mma.sync in the drain warps took tensor
 // time from the main loop; TMA stores of the output (32 boxes of 2 KB, or 8 of 8 KB, per tile) cost 15 % against
 // plain stores - they share the TMA unit with the operand loads.
@@ -42,6 +42,7 @@
 #include <algorithm>
 
 #include "lq_device.cuh"
+#include "lq_gemm_mx_cut.h"
 
 #ifdef LQ_TIMELINE
 // Timeline build only: copies this kernel's stamp lists of the last launch to the host and clears them.
@@ -56,19 +57,11 @@ extern "C" int lq_debug_timeline_mx(unsigned long long* host_out) {
 namespace {
 
 using namespace lqdev;
+using namespace lqmx;
 
-constexpr int MAX_STAGES = 8;
-constexpr int STAGE_A_BYTES = LQ_BM * LQ_KSTAGE;   // 16 KB
-constexpr int MAX_W = 224;                         // columns of the widest tile
-constexpr int SF_BYTES = 512;                      // scale bytes of 128 rows x 4 K blocks
-constexpr int STAGE_SF_BYTES = 3 * SF_BYTES;       // SFA, then SFB of up to 256 columns
-constexpr int SC_FLOATS = LQ_BM + 2 * MAX_W;       // per tile: sT[128], sL2[W], bias[W]
 constexpr int NUM_DRAIN_WARPS = 16;
 constexpr int FIRST_DRAIN_WARP = 2;
 constexpr int GEMM_THREADS = (FIRST_DRAIN_WARP + NUM_DRAIN_WARPS) * 32;
-constexpr int SMEM_BAR_BYTES = 320;
-constexpr int FIXED_SMEM = 1024 /*alignment slack*/ + 2 * SC_FLOATS * 4 + SMEM_BAR_BYTES;
-constexpr int MAX_SMEM = 227 * 1024;
 // tensor-memory columns: accumulators at 0 and W, the branch's at 2 W; 4 columns of A scales and 8 of B scales
 constexpr int TM_SFA = 496, TM_SFB = TM_SFA + 4;
 
@@ -563,43 +556,6 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   }
 }
 
-// Ring depth that fits beside the fixed part.
-int ring_stages(int bw) {      // bw: columns of B per CTA
-  return std::min(MAX_STAGES, (MAX_SMEM - FIXED_SMEM) / (STAGE_A_BYTES + bw * LQ_KSTAGE + STAGE_SF_BYTES));
-}
-int smem_bytes(int bw) {
-  return FIXED_SMEM + ring_stages(bw) * (STAGE_A_BYTES + bw * LQ_KSTAGE + STAGE_SF_BYTES);
-}
-// The same with `slots` stages of B resident (negative: they do not fit).
-int resident_smem(int bw, int slots, int stages) {
-  return FIXED_SMEM + slots * (bw * LQ_KSTAGE + STAGE_SF_BYTES - SF_BYTES) + stages * (STAGE_A_BYTES + SF_BYTES);
-}
-int resident_stages(int bw, int slots) {
-  return std::min(MAX_STAGES, (MAX_SMEM - resident_smem(bw, slots, 0)) / (STAGE_A_BYTES + SF_BYTES));
-}
-
-// Index (LQ_MX_WIDTHS) of the tile width for a launch.  Model, in clocks: a stage takes the longest of its MMAs (2 W, and 40 where
-// one stage's meet the next's), its operands' way from the L2 (70 bytes per clock and SM) and its hand-shakes (350: what a
-// stage of 64 columns takes); a tile the longer of its stages and the drain of the tile before; a launch the tiles of the CTA
-// with the most, plus the last drain and the filling of the ring.  Measured, M = 8192, K x N = 4608 x 1152, W = 64 / 128 / 192 /
-// 224: 58 / 37.9 / 35.3 / 38.0 us; 1152 x 3456: 52.5 / 34.2 / 30.3 / 30.0; 2240 x 2240: 61 / 39.6 / 36.3 / 35.0.
-int pick_width(const lq_layer* L, int tiles_m, int stages, int ctas, bool pair) {
-  int best = -1;
-  double best_cost = 1e30;
-  for (int i = 0; i < LQ_MX_NWIDTHS; ++i) {
-    if (!L->d_sfbw[i]) continue;
-    const int w = LQ_MX_WIDTHS[i];
-    if (g_lq_gemm_width > 0 && w != g_lq_gemm_width) continue;
-    const int c = pair ? 2 : 1, units = ctas / c;
-    const long long tiles = (long long)lq_ceil_div(tiles_m, c) * lq_ceil_div(L->N, w);
-    const double stage = std::max({2.0 * w + 40.0, 350.0, (STAGE_A_BYTES + w / c * LQ_KSTAGE / 8 * lq_mx_weight_bits(L)) / 70.0});
-    const double drain = 600.0 + 1200.0 * lq_ceil_div(w, 128);
-    const double cost = (double)((tiles + units - 1) / units) * std::max(stages * stage, drain) + drain + 4.0 * stage;
-    if (cost < best_cost) { best_cost = cost; best = i; }
-  }
-  return best;
-}
-
 }  // namespace
 
 lq_status lq_gemm_mx_prepare(int device) {
@@ -625,35 +581,20 @@ lq_status lq_launch_gemm_mx(const lq_layer* L, const lq_act* A, void* Y, lq_out_
   if (!p.status) return LQ_ERR_CUDA;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device) != cudaSuccess) return LQ_ERR_CUDA;
-  int ctas = g_lq_gemm_ctas > 0 ? g_lq_gemm_ctas : sms;
-  // Pairs from 256 rows on; below, a pair's second CTA would have nothing to do.
-  const bool pair = p.tiles_m > 1 && ctas > 1 && g_lq_gemm_pair;
-  const int wi = pick_width(L, p.tiles_m, p.k_stages + (L->r > 0), ctas, pair);
-  if (wi < 0) return LQ_ERR_INVALID_ARG;
-  p.width = LQ_MX_WIDTHS[wi]; p.stages = ring_stages(pair ? p.width / 2 : p.width); p.sf_chunks = lq_ceil_div(p.width, 128);
-  p.tiles_n = lq_ceil_div(L->N, p.width);
+  const bool acc = p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx;
+  const MxShape shape = {A->M, L->N, p.b_wrap, A->planes, L->r > 0, acc, lq_mx_weight_bits(L), dt == LQ_OUT_F32 ? 4 : 2};
+  MxCut cut;
+  if (!plan_mx(shape, g_lq_gemm_ctas > 0 ? g_lq_gemm_ctas : sms, g_lq_gemm_width, g_lq_gemm_pair != 0, cut) || !L->d_sfbw[cut.width_index])
+    return LQ_ERR_INVALID_ARG;
+  p.width = cut.width; p.stages = cut.stages; p.b_slots = cut.b_slots; p.tiles_n = cut.tiles_n; p.sf_chunks = lq_ceil_div(p.width, 128);
   p.b_row = LQ_KSTAGE / 8 * lq_mx_weight_bits(L); p.b_format = L->mxfp ? IDESC_MX_B_E2M1 : IDESC_MX_B_E2M3;
   p.block0 = A->block0;
   p.sT = A->d_sT; p.sL2 = L->d_sL2; p.bias = L->d_bias;
   p.Y = Y; p.out_f32 = dt == LQ_OUT_F32 ? 1 : 0; p.wide = lq_rows_of_sectors(Y, L->N, dt);
-  const int c = pair ? 2 : 1;
-  const long long tiles = (long long)lq_ceil_div(p.tiles_m, c) * p.tiles_n;
-  ctas = c * (int)std::min<long long>(ctas / c, tiles);
-  const bool acc = p.branch_steps > 0 && !p.branch_f16 && !p.branch_mx;
-  size_t smem = (size_t)smem_bytes(p.width / c);
-  // Weights stay where they fit beside four stages of A (K up to 1152 at 224 columns, 1280 at 160), a pair has two tiles or more, and the launch is where it was timed
-  // to pay, us with weights fetched for every tile / kept, MXFP4, MXINT4 with W8A8, MXINT4 x 8: M = 8192, 1152 x 3456 29.0 / 27.5, 32.4 / 31.0, 50.0 / 47.7; 1024 x 4096 32.2 / 29.1,
-  // 35.0 / 33.5, 54.7 / 51.1; 768 x 3072 21.1 / 19.0, 25.5 / 26.3, 32.7 / 30.5; 640 x 8192 45.1 / 46.9, 53.0 / 54.1, 71.9 / 73.7.  Few rows leave little to
-  // keep them for (M = 2048, 1152 x 4608: 13.6 / 13.4, 14.4 / 14.7, 20.2 / 20.0; M = 3000: 16.3 / 15.7, 18.3 / 18.0, 25.8 / 25.3).  Down a column of many rows the pairs
-  // are spread over all of A and Y, row blocks keep them together: M = 16384, 1152 x 1152 24.3 / 23.0, 25.9 / 25.5, 39.9 / 38.0; M = 32768 42.4 / 44.9, 46.7 / 48.3, 73.0 / 78.0.
-  p.b_slots = p.b_wrap + (L->r > 0);
-  const int left = std::min(resident_stages(p.width / c, p.b_slots), p.b_wrap), blocks = lq_ceil_div(p.tiles_m, c);   // (no more stages than K has: load_b)
-  const bool resident = pair && tiles >= 2 * (ctas / 2) && left >= 4 && blocks >= 10 && blocks <= 64 && p.b_wrap >= (acc ? 7 : 6);
-  if (resident) { p.stages = left; smem = (size_t)resident_smem(p.width / c, p.b_slots, left); }
-  auto* kernel = resident ? (acc ? lq_gemm_mx_kernel<true, true, true> : lq_gemm_mx_kernel<false, true, true>)
-                 : acc    ? (pair ? lq_gemm_mx_kernel<true, true, false> : lq_gemm_mx_kernel<true, false, false>)
-                          : (pair ? lq_gemm_mx_kernel<false, true, false> : lq_gemm_mx_kernel<false, false, false>);
-  p.maps = L->d_maps + 2 * wi + c - 1;
-  const cudaError_t e = lq_launch_cluster(kernel, ctas, GEMM_THREADS, c, smem, st, A->tmA, A->tmT, A->tmSfa, A->tmSft, p);
+  auto* kernel = cut.resident ? (acc ? lq_gemm_mx_kernel<true, true, true> : lq_gemm_mx_kernel<false, true, true>)
+                 : acc        ? (cut.pair ? lq_gemm_mx_kernel<true, true, false> : lq_gemm_mx_kernel<true, false, false>)
+                              : (cut.pair ? lq_gemm_mx_kernel<false, true, false> : lq_gemm_mx_kernel<false, false, false>);
+  p.maps = L->d_maps + 2 * cut.width_index + cut.pair;
+  const cudaError_t e = lq_launch_cluster(kernel, cut.ctas, GEMM_THREADS, 1 + cut.pair, (size_t)cut.smem, st, A->tmA, A->tmT, A->tmSfa, A->tmSft, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -216,9 +216,10 @@ def test_row_chunks_of_a_call_from_host_memory(M, K, N):
 
 
 @pytest.mark.parametrize("ctas", [6, 0])
-@pytest.mark.parametrize("width", [64, 0])
+@pytest.mark.parametrize("width", [64, 0, 192])
 @pytest.mark.parametrize("main,branch,r,K", [("mxint4", "none", 0, 1152), ("mxint4", "w8a8", 32, 1152), ("mxint4", "w16a16", 24, 1030 + 2), ("mxfp4", "mxfp8", 64, 1400),
-                                             ("mxint8", "mxint8", 64, 1152), ("mxint8", "mxint4", 128, 1160)])
+                                             ("mxfp4", "mxfp8", 64, 1152), ("mxint8", "mxint8", 64, 1152), ("mxint8", "mxint4", 128, 1160),
+                                             ("mxint8", "mxint4", 128, 1152)])
 def test_weights_that_stay_while_a_pair_goes_down_its_columns(option, main, branch, r, K, width, ctas):
     """Runs of tiles that begin and end within a column, change columns once or more often, a pair without a second row block, a last tile of eight
     columns, K at and beyond what stays: the bits of single CTAs."""
@@ -234,7 +235,7 @@ def test_weights_that_stay_while_a_pair_goes_down_its_columns(option, main, bran
     act = B.lq_act_create(h, M, 0)
     x, st = torch.from_numpy(_x(rng, M, K)).cuda(), torch.cuda.current_stream().cuda_stream
     B.lq_quantize_act(h, x.data_ptr(), M, act, st)
-    option("gemm_width", width)
+    option("gemm_width", 160 if width == 192 and branch == "w8a8" else width)
 
     def forward(pair, n):
         option("gemm_pair", pair, default=1)
