@@ -773,7 +773,7 @@ static lq_status forward_host(const lq_layer* L, lq_act* A, const void* Xh, int3
   }
   const size_t esz = dt == LQ_OUT_F32 ? 4 : 2;
   int end[LQ_HOST_CHUNKS];
-  const int nchunk = host_chunks(M, (size_t)M * (A->K * 2 + A->N * esz), end);
+  const int nchunk = host_chunks(M, (size_t)M * A->K * 2, (size_t)M * A->N * esz, end);
   CUDA_OK(cudaEventRecord(A->ev_begin, st));                  // copies start after what the caller queued before
   CUDA_OK(cudaStreamWaitEvent(A->s_h2d, A->ev_begin, 0));
   CUDA_OK(cudaStreamWaitEvent(A->s_d2h, A->ev_begin, 0));

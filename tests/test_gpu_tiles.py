@@ -192,7 +192,7 @@ def test_outputs_that_begin_between_sectors(option, main, branch, r, N):
     B.lq_layer_free(h)
 
 
-@pytest.mark.parametrize("M,K,N", [(2047, 40, 24), (2048, 40, 24), (2049, 40, 24), (2305, 3200, 24), (2300, 40, 3800)])
+@pytest.mark.parametrize("M,K,N", [(2047, 40, 24), (2048, 40, 24), (2049, 40, 24), (2305, 3200, 24), (2300, 40, 3800), (2300, 1152, 1160)])
 def test_row_chunks_of_a_call_from_host_memory(M, K, N):
     """Around the number of rows from which chunks differ in size, few bytes and many, row counts beside a tile: the bits of the call on device
     memory, and nothing beside them."""

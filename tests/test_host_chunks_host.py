@@ -13,10 +13,10 @@ SOURCE = """
 #define LQ_HOST_CHUNKS MOST
 #endif
 #include "lq_host_chunks.h"
-extern "C" int chunks(int M, double bytes, int* out) {
+extern "C" int chunks(int M, double x, double y, int* out) {
   struct { int end[LQ_HOST_CHUNKS], guard[16]; } s;
   for (int& g : s.guard) g = -7;
-  const int n = host_chunks(M, (size_t)bytes, s.end);
+  const int n = host_chunks(M, (size_t)x, (size_t)y, s.end);
   for (int g : s.guard)
     if (g != -7) return -1;
   for (int i = 0; i < n && i < LQ_HOST_CHUNKS; ++i) out[i] = s.end[i];
@@ -34,11 +34,11 @@ def chunks(tmp_path_factory, request):
                     os.path.join(ROOT, "paper_2604_18117_b200", "csrc"), "-I", os.path.join(cuda, "include"), str(d / "chunks.cpp"), "-o",
                     str(d / "chunks.so")], check=True)
     lib = ctypes.CDLL(str(d / "chunks.so"))
-    lib.chunks.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_void_p]
+    lib.chunks.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double, ctypes.c_void_p]
 
-    def get(M, bytes):
+    def get(M, x, y):
         out = (ctypes.c_int * 16)()
-        n = lib.chunks(M, bytes, out)
+        n = lib.chunks(M, x, y, out)
         assert n >= 1, "written beyond the end"
         return list(out)[:n]
 
@@ -46,9 +46,16 @@ def chunks(tmp_path_factory, request):
     return get
 
 
-@pytest.mark.parametrize("bytes", [1e3, 2e7, 1e9])
-def test_chunks_cover_the_rows(chunks, bytes):
+@pytest.mark.parametrize("x,y", [(1e3, 1e3), (7e6, 7e6), (7e6, 14e6), (5e8, 5e8)])
+def test_chunks_cover_the_rows(chunks, x, y):
     for M in [*range(1, 2600), 4096, 5001, 8192, 32768]:
-        end = chunks(M, bytes)
+        end = chunks(M, x, y)
         assert len(end) <= chunks.most and end[-1] == M
         assert all(e % 128 == 0 for e in end[:-1]) and all(a < b for a, b in zip([0, *end], end))
+
+
+# MB of X and Y, the faster number of chunks (timed against each other): more where the way out waits for the way in
+@pytest.mark.parametrize("x,y,n", [(9.4, 9.4, 4), (16.8, 21.0, 5), (8.4, 16.8, 8), (5.9, 14.8, 8), (14.4, 21.5, 8), (3.1, 10.6, 8), (8.4, 33.6, 5),
+                                   (9.4, 37.7, 5), (4.2, 6.3, 4), (33.6, 67.1, 5)])
+def test_the_faster_number_of_chunks(chunks, x, y, n):
+    assert len(chunks(4096, 1e6 * x, 1e6 * y)) == min(n, chunks.most)
