@@ -160,17 +160,12 @@ def test_pairs_of_ctas_give_the_bits_of_single_ones_every_time(option, main, bra
     B.lq_layer_free(h)
 
 
-@pytest.mark.parametrize("main,branch,r", [("sint4", "w8a8", 32), ("mxint4", "w8a8", 32), ("mxfp4", "mxfp8", 64)])
-@pytest.mark.parametrize("N", [8, 72, 208])
-def test_outputs_that_begin_between_sectors(option, main, branch, r, N):
+def _begins_between_sectors(rng, main, branch, r, M, K, N):
     """Rows of Y that begin on 16-byte boundaries only, by their length or by Y's own place, hold the bits of those that begin on
     32-byte ones, and nothing beside them is written."""
     import torch
     from tests.helpers import import_oracle_layer, import_oracle_mxfp_layer
 
-    option("gemm_split", 1)                                       # (tiles shared by a cluster are stored by 16 bytes)
-    rng = np.random.default_rng(N)
-    M, K = 131, 200
     layer = {"sint4": SINT4._random_layer, "mxint4": MXINT4._mx_layer, "mxfp4": MXFP._layer}[main](rng, K, N, r, branch)
     h, _ = (import_oracle_mxfp_layer if main == "mxfp4" else import_oracle_layer)(layer)
     B.lq_layer_to_device(h, 0)
@@ -190,6 +185,22 @@ def test_outputs_that_begin_between_sectors(option, main, branch, r, N):
     assert B.lq_get_device_status(0)[0] == 0
     B.lq_act_free(act)
     B.lq_layer_free(h)
+
+
+@pytest.mark.parametrize("main,branch,r", [("sint4", "w8a8", 32), ("mxint4", "w8a8", 32), ("mxfp4", "mxfp8", 64)])
+@pytest.mark.parametrize("N", [8, 72, 208])
+def test_outputs_that_begin_between_sectors(option, main, branch, r, N):
+    option("gemm_split", 1)                                       # (tiles shared by a cluster have stores of their own)
+    _begins_between_sectors(np.random.default_rng(N), main, branch, r, 131, 200, N)
+
+
+@pytest.mark.parametrize("split", [2, 4, 8])
+@pytest.mark.parametrize("M", [1, 9, 131])
+@pytest.mark.parametrize("N", [8, 72, 208])
+def test_outputs_of_shared_tiles_that_begin_between_sectors(option, split, M, N):
+    """(parts of a tile without rows, with some and with all)"""
+    option("gemm_split", split)
+    _begins_between_sectors(np.random.default_rng(N + M), "sint4", "w8a8", 32, M, 1152, N)
 
 
 @pytest.mark.parametrize("M,K,N", [(2047, 40, 24), (2048, 40, 24), (2049, 40, 24), (2305, 3200, 24), (2300, 40, 3800), (2300, 1152, 1160)])
