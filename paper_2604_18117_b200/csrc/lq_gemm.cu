@@ -15,8 +15,9 @@
 //               and are handed over with one commit; two pairs alternate
 //   warps 4-11  drain: each warp owns 32 rows x 64 columns of the tile.  Half a group's slice is two tcgen05.ld.16x256b.x4; it is
 //               in flight into one register buffer while the half before is consumed from the other:
-//               acc += (P * sx) * sw, packed f32x2, fp32 registers (the integer branch's stage: P * (sx * sw)).  A pair goes back as soon as its last half sits in
-//               registers.  The next stage's scales are loaded, and the next tile's first half is requested, before the last half is consumed
+//               acc += (P * sx) * sw, packed f32x2, fp32 registers (the integer branch's stage: P * (sx * sw)).  A pair goes back as soon
+//               as its last half sits in registers.  The next stage's scales are loaded, and the next tile's first half is requested,
+//               before the last half is consumed
 // What bounds it: the FP32 pipe's operand delivery and the drain's other instructions.  Per group and scheduler 64 packed products
 // (2.0 to 2.6 clocks each, measured) and 64 packed FMAs (2.75 with an operand shared by neighbours, 3.9 with three of their own) are about 320
 // clocks, the tensor pipe needs 128; the same loop over tensor memory without any hand-shake takes 400, 100 of them for the scales' way
@@ -26,10 +27,11 @@
 // taken over from the other four warps (setmaxnreg).  M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 85 / 96 us with sixteen
 // narrow warps, 80 / 89 with one commit per group; then, timed in turn with other inputs each time, 81.1 / 88.3, 78.0 / 84.0 with P sx first,
 // 72.4 / 81.6 with sectors stored whole, 70.1 / 78.1 with a stage's commits under one election, 64.5 / 70.9 with the issuer written out and the
-// drain's last eight registers, 64.2 / 68.9 with halves of groups in flight and one hand-back a stage.  At K = 1152 a tile's end is a fifth of the launch: of 11.4 k clocks a tile 1.0 k are the branch's group, 0.8 k the stores, 0.5 k
-// the way to the next tile's first stage.  Scalar FMAs lose their issue slots (94 - 104 us for 79); with whole groups in flight, scales of
-// the next group loaded where this one's were used last made the kernel slower (73.6 for 68.8: registers); two column
-// halves as pipelines of their own, each with an issuer, 67.9 for 66.5.
+// drain's last eight registers, 64.2 / 68.9 with halves of groups in flight and one hand-back a stage.  At K = 1152 a tile's end is a
+// fifth of the launch: of 11.4 k clocks a tile 1.0 k are the branch's group, 0.8 k the stores, 0.5 k the way to the next tile's first
+// stage.  Scalar FMAs lose their issue slots (94 - 104 us for 79); with whole groups in flight, scales of the next group loaded where
+// this one's were used last made the kernel slower (73.6 for 68.8: registers); two column halves as pipelines of their own, each with an
+// issuer, 67.9 for 66.5.
 // Orders of rows and columns (lq_internal.h) are chosen for the drain's fragments: the columns of the tile are permuted in
 // the weight operand so that a lane's 16 columns of a row are neighbours in Y - the epilogue converts and stores, no
 // exchange - and the scale vectors are permuted so that a lane's come in one (rows) and four (columns) 16-byte loads
@@ -162,9 +164,10 @@ __device__ __forceinline__ void fetch_half(uint32_t taddr, Frag (&v)[2]) {
   for (int i = 0; i < 2; ++i) tmem_ld_16x256b_x4(taddr + ((uint32_t)(16 * i) << 16), v[i]);
 }
 
-// A group's two MMAs under one election (both groups of a stage under one were 1 to 2 % slower), predicated instead of branched around: the control flow of the issuing warp stays uniform.
-// (An `if` of one lane around them and around the commits, with a loop over the groups: a stage's way through the issuer, 1.2 k clocks,
-// was as long as the drain's.  us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152: 72.4 / 81.6 -> 64.5 / 70.9, with the drain's eight registers.)
+// A group's two MMAs under one election (both groups of a stage under one were 1 to 2 % slower), predicated instead of branched around:
+// the control flow of the issuing warp stays uniform.  (An `if` of one lane around them and around the commits, with a loop over the
+// groups: a stage's way through the issuer, 1.2 k clocks, was as long as the drain's.  us, M = 8192, K x N = 1152 x 3456 / 4608 x 1152:
+// 72.4 / 81.6 -> 64.5 / 70.9, with the drain's eight registers.)
 #define LQ_GROUP_MMAS                                                   \
   "{\n\t.reg .pred P, T, F;\n\t"                                       \
   "elect.sync _|P, 0xffffffff;\n\t"                                    \
@@ -187,11 +190,12 @@ __device__ __forceinline__ void issue_group(uint32_t d, uint64_t a, uint64_t b, 
 enum { BRANCH_NONE = 0, BRANCH_I8 = 1, BRANCH_F16 = 2 };
 enum { TILE_WHOLE = 0, TILE_SECTORS = 1, TILE_SPLIT = 2 };
 
-// TILE_SPLIT: the CTAs of a cluster share one tile, each with a part of the stages (K and the branch).  Every CTA adds up a part of the tile: the others
-// copy their partial sums of it into its shared memory, and it waits for the bytes.  What bounds it is that one trip.  (Rendezvous, loads of all parts from
-// the others' shared memory and a second rendezvous before leaving: us, M x K x N by two, four, eight CTAs, 120 x 1152 x 4608 8.40 -> 7.57, 256 x 4608 x 1152 11.05 -> 10.27,
-// 1 x 1152 x 1152 5.46 -> 4.80, 120 x 8192 x 1152 11.26 -> 9.83.  Stores of 16 bytes by every thread instead of copies from a staging place: 4.60 with one row, but
-// 8.90 with 128; both, by the number of rows: 4.68 and 7.8.)  TILE_SECTORS: every row of Y begins on a 32-byte boundary.  (An instance of its own: with both kinds of
+// TILE_SPLIT: the CTAs of a cluster share one tile, each with a part of the stages (K and the branch).  Every CTA adds up a part of the
+// tile: the others copy their partial sums of it into its shared memory, and it waits for the bytes.  What bounds it is that one trip.
+// (Rendezvous, loads of all parts from the others' shared memory and a second rendezvous before leaving: us, M x K x N by two, four,
+// eight CTAs, 120 x 1152 x 4608 8.40 -> 7.57, 256 x 4608 x 1152 11.05 -> 10.27, 1 x 1152 x 1152 5.46 -> 4.80, 120 x 8192 x 1152 11.26 ->
+// 9.83.  Stores of 16 bytes by every thread instead of copies from a staging place: 4.60 with one row, but 8.90 with 128; both, by the
+// number of rows: 4.68 and 7.8.)  TILE_SECTORS: every row of Y begins on a 32-byte boundary.  (An instance of its own: with both kinds of
 // stores in one epilogue the drain's registers were worse allocated: 63.6 / 69.4 us for 62.3 / 69.0, M = 8192, K x N = 1152 x 3456 / 4608 x 1152.)
 template <int BRANCH, int TILE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
@@ -211,7 +215,7 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto bar_full = [&](int s) { return sm_bar + 8u * (uint32_t)s; };                        // operands + scales landed
   auto bar_empty = [&](int s) { return sm_bar + 8u * (uint32_t)(NSTAGE + s); };           // MMAs of the stage retired
   auto bar_tfull = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + b); };
-  // (16 bytes apart: with tfull's stride the same code was 1.5 to 2.5 % slower, whatever the stride)
+  // (16 bytes apart: 8 bytes apart, as they would fit, the same code was 1.5 to 2.5 % slower; what in it is not known)
   auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + NPAIR + 1 + 2 * b); };
   [[maybe_unused]] const uint32_t bar_gather = sm_bar + 8u * (uint32_t)(2 * NSTAGE + 3 * NPAIR);
   constexpr int NBAR = 2 * NSTAGE + 3 * NPAIR + 1;
@@ -499,7 +503,9 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (lane < p.split && lane != part) {            // a lane for each other CTA: the items that have a row
           int n = 0;
           for (int j = lane * n_items; j < (lane + 1) * n_items; ++j) n += row0 + 8 * (j >> 2) < p.M;
-          if (n > 0) peer_copy(peer_smem(items_at(sm_gather, part, dwarp), lane), items_at(sm_stage, lane, dwarp), (uint32_t)n * 512, peer_smem(bar_gather, lane));
+          if (n > 0)
+            peer_copy(peer_smem(items_at(sm_gather, part, dwarp), lane), items_at(sm_stage, lane, dwarp), (uint32_t)n * 512,
+                      peer_smem(bar_gather, lane));
         }
       } else {
         // Epilogue straight from registers: 16 neighbouring columns of four rows per lane, 128 of a row per quad.  Two lanes' stores of 16
@@ -617,20 +623,23 @@ __global__ void lq_wait_probe_kernel(int32_t* status, long long limit) {
 
 // CTAs per tile of a launch of few tiles (1, 2, 4 or 8).  A tile's stages are one serial chain, so while SMs are idle they may as well share
 // it; a cluster's launch and the exchange cost the rest (us, alone and shared: M = 1, K x N = 1152 x 1152: 7.0 and 4.8 by
-// eight; M = 120, 8192 x 1152: 30.8 and 9.8 by eight; M = 256, 4608 x 1152: 18.9 and 10.3 by four).  The hardware places a cluster's CTAs next to each
-// other, so fewer fit than there are SMs; a second round of them would cost more than it gives.  Prices: the exchange 1.62 us, with full tiles 0.6 + 0.08
-// per CTA more; a stage 0.52, as the drain once took it - 0.44 now, by which a few sizes of ten stages would not be shared any more (M = 120,
-// 1152 x 4608: 7.57 by two, 7.50 alone; M = 256: 8.90 and 7.71).  But shared sums are the shorter chains, and further from the exact sum is what those rows would
-// be (M = 128, fp32 output: relative error 6.0e-8 by two, 7.4e-8 alone): with these prices no size is shared by fewer CTAs than while the exchange took longer,
-// and tiles of six stages are shared, too (M = 1, 640 x 1152: 4.9 by four, 5.3 alone; up to 60 rows).
+// eight; M = 120, 8192 x 1152: 30.8 and 9.8 by eight; M = 256, 4608 x 1152: 18.9 and 10.3 by four).  The hardware places a cluster's CTAs
+// next to each other, so fewer fit than there are SMs; a second round of them would cost more than it gives.  Prices, us: a stage 0.44, the
+// exchange 1.62, with full tiles 0.6 + 0.08 per CTA more.
+// A stage of a chain is charged 0.08 us beyond its time, because the sum's error grows with the chain: rows of ten stages are so
+// shared by two where alone would be as fast or faster (M = 120, 1152 x 4608: 7.57 by two, 7.50 alone; M = 256: 8.90 and 7.71), with a relative
+// error of 6.0e-8 instead of 7.4e-8 (M = 128, fp32 output).  Tiles of six stages are shared up to 60 rows (M = 1, 640 x 1152: 4.9 by four,
+// 5.3 alone).
+constexpr double STAGE_US = 0.44, CHAIN_US = 0.08;
 int g_clusters[64][3];                                // how many clusters of 2, 4, 8 the device holds at once
 int pick_split(int device, int M, long long units, int stages, int ctas) {
   int best = 1;
-  double best_cost = 0.52 * stages;
+  double best_cost = (STAGE_US + CHAIN_US) * stages;
   for (int i = 0, split = 2; i < 3; ++i, split *= 2) {
     if (split > ctas || split > stages || units > std::min(g_clusters[device & 63][i], ctas / split)) break;
     if (g_lq_gemm_split > 0 && split != g_lq_gemm_split) continue;
-    const double cost = g_lq_gemm_split > 0 ? 0 : 0.52 * lq_ceil_div(stages, split) + 1.62 + (0.6 + 0.08 * split) * std::min(M, LQ_BM) / LQ_BM;
+    const double exchange = 1.62 + (0.6 + 0.08 * split) * std::min(M, LQ_BM) / LQ_BM;
+    const double cost = g_lq_gemm_split > 0 ? 0 : (STAGE_US + CHAIN_US) * lq_ceil_div(stages, split) + exchange;
     if (cost < best_cost) { best_cost = cost; best = split; }
   }
   return best;
@@ -699,7 +708,9 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
     return L->r == 0 ? lq_gemm_kernel<BRANCH_NONE, T> : L->f16_branch ? lq_gemm_kernel<BRANCH_F16, T> : lq_gemm_kernel<BRANCH_I8, T>;
   };
   auto* k = p.split > 1 ? kernel(std::integral_constant<int, TILE_SPLIT>())
-                        : lq_rows_of_sectors(Y, L->N, dt) ? kernel(std::integral_constant<int, TILE_SECTORS>()) : kernel(std::integral_constant<int, TILE_WHOLE>());
-  const cudaError_t e = lq_launch_cluster(k, ctas, GEMM_THREADS, p.split, SMEM_BYTES + (p.split > 1 ? GATHER_BYTES : 0), st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
+            : lq_rows_of_sectors(Y, L->N, dt) ? kernel(std::integral_constant<int, TILE_SECTORS>())
+                                              : kernel(std::integral_constant<int, TILE_WHOLE>());
+  const size_t smem = SMEM_BYTES + (p.split > 1 ? GATHER_BYTES : 0);
+  const cudaError_t e = lq_launch_cluster(k, ctas, GEMM_THREADS, p.split, smem, st, A->tmA, L->tmB, A->tmT, L->tmL2, p);
   return lq_note_cuda(e != cudaSuccess ? e : cudaGetLastError()) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -6,7 +6,8 @@
 // Here the tensor core applies the scales itself: tcgen05.mma kind::mxf8f6f4.block_scale takes one E8M0 scale
 // per operand row and 32-deep K block from tensor memory, so ALL blocks of a tile accumulate into ONE fp32
 // accumulator and nothing has to be drained per block.  The activations' codes ride in E4M3 operands as in the SINT4
-// kernel, the weights' in packed E2M3 ones (MXFP4: E2M1).  Products q q' 2^(e+e') are exact in fp32; their sum is rounded by the tensor core's fp32 accumulation.
+// kernel, the weights' in packed E2M3 ones (MXFP4: E2M1).  Products q q' 2^(e+e') are exact in fp32; their sum is rounded by the tensor
+// core's fp32 accumulation.
 //
 // Shape of the kernel (persistent, one CTA per SM, warp-specialised, 18 warps): tiles of 128 rows x W columns, W chosen by
 // the launcher (pick_width).
@@ -32,7 +33,7 @@
 // where TMA spreads them out.  M = 8192, MXFP: 1152 x 3456 30.6 -> 29.4 us, 2240 x 6720 95.3 -> 91.1, 5600 x 2240 79.4 ->
 // 75.5; integer codes 33.8 -> 33.4 and 51.3 -> 50.5.
 // So do the weights that a pair needs for its next tile, too: where K is short enough they stay in shared memory, and the pair goes down its columns
-// (RESIDENT; weights_stay has the rule).  5 to 10 % less time where it applies, and about as much under the power cap.
+// (RESIDENT; weights_stay has the rule).  6 % less time on average where it applies, and about as much under the power cap.
 // What was measured on the way here (PixArt block, four GEMMs): the branch on mma.sync in the drain warps took tensor
 // time from the main loop; TMA stores of the output (32 boxes of 2 KB, or 8 of 8 KB, per tile) cost 15 % against
 // plain stores - they share the TMA unit with the operand loads.
@@ -154,9 +155,13 @@ __device__ __forceinline__ void load_weights_stage(uint32_t own, uint32_t tx, ui
                                                    uint32_t sf_dst, const CUtensorMap* tm_sf, int sf_row) {
   const uint64_t t = reinterpret_cast<uint64_t>(tm), ts = reinterpret_cast<uint64_t>(tm_sf);
   if constexpr (PAIR)
-    asm volatile(LQ_LOAD_WEIGHTS(LQ_TMA_2D_PAIR) ::"r"(own), "r"(tx), "r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0), "r"(sf_row) : "memory");
+    asm volatile(LQ_LOAD_WEIGHTS(LQ_TMA_2D_PAIR) ::"r"(own), "r"(tx), "r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0),
+                 "r"(sf_row)
+                 : "memory");
   else
-    asm volatile(LQ_LOAD_WEIGHTS(LQ_TMA_2D) ::"r"(own), "r"(tx), "r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0), "r"(sf_row) : "memory");
+    asm volatile(LQ_LOAD_WEIGHTS(LQ_TMA_2D) ::"r"(own), "r"(tx), "r"(full), "r"(dst), "l"(t), "r"(x), "r"(y), "r"(sf_dst), "l"(ts), "r"(0),
+                 "r"(sf_row)
+                 : "memory");
 }
 #define LQ_LOAD_ACTS(TMA)                        \
   "{\n\t.reg .pred P;\n\t"                       \
@@ -261,8 +266,8 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     auto full_bar = [&](int st) { return first_bar + 8u * (uint32_t)(B_FULL + st); };
     const uint32_t arm = rank == 0 ? CTAS : 0;         // CTAs whose bytes this one announces
     const int block_last = p.tiles_m - 1;
-    // The weights' half of main stage s; announces the whole stage.  RESIDENT: only where they are not there yet.  (Their place is free: the MMAs that read it
-    // last are at least as many stages back as the ring has slots, and the slot's own wait was for those.)
+    // The weights' half of main stage s; announces the whole stage.  RESIDENT: only where they are not there yet.  (Their place is free:
+    // the MMAs that read it last are at least as many stages back as the ring has slots, and the slot's own wait was for those.)
     auto load_b = [&](int st, int s, int nu, bool there) {
       const int sb = s >= p.b_wrap ? s - p.b_wrap : s; // the lo digits' plane runs over the same weights
       const uint32_t acts = STAGE_A_BYTES + SF_BYTES;
@@ -316,7 +321,8 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint32_t a_dst = sm_stage + st * stage_bytes, full = full_bar(st);
         const bool fetch = !RESIDENT || (!there && bs == 0);
         if (elect_one()) {
-          if (arm != 0) mbar_expect_tx(bar(B_FULL + st), arm * (STAGE_A_BYTES + (p.branch_mx ? SF_BYTES : 0) + (fetch ? b_bytes + (p.branch_mx ? sfb_bytes : 0) : 0u)));
+          const uint32_t acts = STAGE_A_BYTES + (p.branch_mx ? SF_BYTES : 0), weights = b_bytes + (p.branch_mx ? sfb_bytes : 0);
+          if (arm != 0) mbar_expect_tx(bar(B_FULL + st), arm * (acts + (fetch ? weights : 0u)));
           tma_load_2d<PAIR>(a_dst, &tmT, bs * LQ_KSTAGE, m0, full);
           if (fetch) tma_load_2d<PAIR>(b_at(st, p.b_wrap), &p.maps->l2, 0, n0 + (int)rank * BW, full);
           if (p.branch_mx) {   // the block scales of T (rows) and of L2 (columns) along the rank
@@ -400,7 +406,8 @@ lq_gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const int sb = s >= p.b_wrap ? s - p.b_wrap : s;
         const uint64_t adesc = make_smem_desc(sm_stage + st * stage_bytes), bdesc = make_smem_desc(b_at(st, sb));
         auto issue = PAIR ? issue_main_stage_pair : issue_main_stage_one;
-        issue(d, adesc, bdesc, (idesc_mx(W, 0) | p.b_format) + ROWS256, make_smem_desc_plain(sm_sf + st * SF_STAGE, 16, 128), make_smem_desc_plain(sfb_at(st, sb), 16, 128),
+        issue(d, adesc, bdesc, (idesc_mx(W, 0) | p.b_format) + ROWS256, make_smem_desc_plain(sm_sf + st * SF_STAGE, 16, 128),
+              make_smem_desc_plain(sfb_at(st, sb), 16, 128),
               (uint32_t)(p.sf_chunks == 2), (uint32_t)s, bar(B_EMPTY + st));
         if (++st == NST) { st = 0; par ^= 1; }
         LQ_TL(EV_M_ISSUED, s);

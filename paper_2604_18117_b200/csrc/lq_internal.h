@@ -106,7 +106,8 @@ struct lq_layer {
   // device copy, operand layouts
   int device;
   int main_kind;               // LQ_KIND_*: byte encoding of the 4-bit codes in the MMA operands
-  uint8_t* d_Wq8;              // MX: packed, [Npad][Kpad] e2m1 (mxfp) or e2m3 elements; SINT4: [Npad][Kpad] e4m3 bytes, K contiguous (B operand, K-major; rows in lq_col_slot order, MX: lq_col32_slot)
+  uint8_t* d_Wq8;              // MX: packed, [Npad][Kpad] e2m1 (mxfp) or e2m3 elements; SINT4: [Npad][Kpad] e4m3 bytes, K contiguous
+                               // (B operand, K-major; rows in lq_col_slot order, MX: lq_col32_slot)
   float* d_sw;                 // [Gpad][Npad] fp32 (exact images of the fp16 scales), in lq_colscale_slot order
   uint8_t* d_L1c;              // [planes * rn][Kpad] bytes (W16A16: [rn][Kpad] halves), K contiguous: first factor as the B operand of
                                // the down-projection; rn = lq_l1_rows; MXINT8 factors: the hi digits' rows, then the lo digits'
@@ -203,7 +204,8 @@ extern int g_lq_gemm_ctas;   // option "gemm_ctas" (0 = one per SM)
 extern int g_lq_gemm_pair;   // option "gemm_pair": 1 = pairs of CTAs share an MX GEMM's tile where there are enough rows
 extern int g_lq_gemm_split;  // option "gemm_split": CTAs that share a tile of the SINT4 GEMM where there is room for them, 0 = chosen by the launcher
 extern int g_lq_gemm_width;  // option "gemm_width": tile width of the MX GEMM, 0 = chosen by the launcher
-extern int g_lq_quant_warps, g_lq_quant_ctas;   // options "quant_warps", "quant_ctas": the quantizer's row groups per tile and stages per chunk, 0 = chosen by the launcher
+// options "quant_warps", "quant_ctas": the quantizer's row groups per tile and stages per chunk, 0 = chosen by the launcher
+extern int g_lq_quant_warps, g_lq_quant_ctas;
 extern int g_lq_overlap;     // option "overlap": launch kernels with programmatic stream serialization
 extern int g_lq_store_qb;    // option "store_qb": also write the branch activation codes to HBM (parity export)
 
@@ -211,7 +213,8 @@ extern int g_lq_store_qb;    // option "store_qb": also write the branch activat
 // Launches `kernel` on `st`.  With the "overlap" option the launch carries programmatic stream serialization: the
 // kernel's CTAs may become resident and run their set-up (barriers, tensor memory) while the previous kernel on the
 // stream is still draining its last tiles; every kernel of this library executes griddepcontrol.wait after that set-up,
-// before it reads or writes global memory, and griddepcontrol.launch_dependents right before it, so that the chain
+// before it reads what an earlier kernel may write or writes global memory (weights, which no kernel writes, and the quantizer's
+// prefetch of X to the L2 come before it), and griddepcontrol.launch_dependents after the set-up, so that the chain
 // quantizer -> GEMM -> next quantizer overlaps its launch gaps and tails.  All kernels here are persistent (the whole
 // grid is resident at once), so a waiting successor never holds an SM that a predecessor CTA still needs.
 template <typename... KArgs, typename... Args>

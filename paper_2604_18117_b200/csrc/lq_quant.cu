@@ -14,11 +14,11 @@
 //               stage.  A lane owns 16 neighbouring values of two rows, two 16-byte vectors of X each: they share a block and its
 //               scale, a block of 32 is two lanes, its maximum one shuffle, and a lane's codes are one 16-byte store, to global and
 //               to shared memory.  (With a vector of each half of the stage to a lane, four lanes to a block, every scale was worked
-//               out twice as often and stores were of 8 bytes; us, timed in turn, M = 8192, K = 1152 / 4608, X cold: SINT4 13.8 / 37.4 -> 13.4 / 36.2,
-//               MXINT4 x 8 13.5 / 37.6 -> 12.9 / 34.2, MXFP4 11.1 / 28.4 -> 11.1 / 28.6; X in the L2: 12.1 / 35.0 -> 11.5 / 32.6, 12.5 / 37.7 -> 11.4 / 34.2.)
-//               Loads and stores move whole rows of a box.  (A first version loaded X into registers from global memory, half rows per
-//               instruction: the tag stage of the L1 was what bounded it, at 40 lookups a piece, and its unrolled ring
-//               cost a microsecond of instruction misses.)  The branch's operand goes to shared memory in the layout
+//               out twice as often and stores were of 8 bytes; us, timed in turn, M = 8192, K = 1152 / 4608, X cold: SINT4 13.8 / 37.4 ->
+//               13.4 / 36.2, MXINT4 x 8 13.5 / 37.6 -> 12.9 / 34.2, MXFP4 11.1 / 28.4 -> 11.1 / 28.6; X in the L2: 12.1 / 35.0 -> 11.5 /
+//               32.6, 12.5 / 37.7 -> 11.4 / 34.2.)  Loads and stores move whole rows of a box.  (A first version loaded X into registers
+//               from global memory, half rows per instruction: the tag stage of the L1 was what bounded it, at 40 lookups a piece, and
+//               its unrolled ring cost a microsecond of instruction misses.)  The branch's operand goes to shared memory in the layout
 //               the MMA reads (K-major, 128-byte swizzle).  More warps (28 at 64 registers) were no faster, twelve were
 //               10-30 % slower
 //   warp 4      TMA producer of the first factor's slabs, one per stage, and their scale bytes.  (The MMA warp fetched them at
@@ -37,8 +37,8 @@
 //   scale     fp16(a / 7) == fp16(a * fl32(1/7)) for every finite fp16 a (checked exhaustively on the host),
 //             because a/7 never comes closer than 2^-15 (relative) to an fp16 midpoint.
 //   SINT4     x and s are 11-bit numbers, so x / s is either exactly k + 1/2 or at least 2^-14 away from it.  The product
-//             with a reciprocal that is an ulp or two off is within 2^-19 of the quotient; adding 192 rounds it to a multiple of 2^-16, which restores
-//             exact ties and moves nothing else across one; a second addition then rounds to the integer, ties to even.
+//             with a reciprocal that is an ulp or two off is within 2^-19 of the quotient; adding 192 rounds it to a multiple of 2^-16,
+//             which restores exact ties and moves nothing else across one; a second addition then rounds to the integer, ties to even.
 //   branch    x / sb is within 2^-23 of qm x / max, which is either exactly k + 1/2 or at least 2^-19 away from it (11-bit numbers, qm of 5
 //             or 7 bits); so one FMA with 1.5 * 2^23 and a reciprocal good to 2^-21 rounds like the quotient everywhere but on such
 //             ties.  As qm is prime they are at x = +-max / 2, for which the reciprocal is taken on the side that gives the quotient's code
@@ -305,8 +305,9 @@ __device__ __forceinline__ uint2 sint4_codes8(const uint4& v, float rcp, bool co
 }
 
 // Scale of a row's branch codes (its maximum over qm, 1 for a row of zeros) and the reciprocal that codes are formed with (see the top).  All of
-// a tile's warps wait for it between its two walks, so it is worked out without a division: the maximum over a constant is the correctly rounded quotient after
-// one correction step (checked for every fp16 maximum on the host), and where codes do not need the quotient an approximate reciprocal will do.
+// a tile's warps wait for it between its two walks, so it is worked out without a division: the maximum over a constant is the correctly
+// rounded quotient after one correction step (checked for every fp16 maximum on the host), and where codes do not need the quotient an
+// approximate reciprocal will do.
 struct BranchScale {
   float sb, inv;
   bool exact;            // this row's codes need the quotient: ties elsewhere, or a maximum that is no number
@@ -608,8 +609,9 @@ __device__ __forceinline__ void issue_four_mx(uint32_t d, uint64_t a, uint64_t b
 }
 
 // What bounds a narrow MMA is its A operand's way from shared memory, so tiles of up to 32 rows use MMAs of 64 (block-scaled ones have no fewer than
-// 128).  Their rows lie in tensor memory sixteen to a quarter of the lanes, and the two warps of a4 reach the first two quarters.  us with 128 rows / 64, X in the L2:
-// W16A16 rank 24, M x K = 1365 x 2312 8.6 / 7.5, 1 x 4608 12.0 / 10.4, 120 x 1152 5.1 / 4.7; W8A8 rank 32 9.1 / 8.7, 11.1 / 10.3, 5.9 / 5.7; rank 128 12.1 / 11.8, 15.0 / 14.6, 8.0 / 7.8.
+// 128).  Their rows lie in tensor memory sixteen to a quarter of the lanes, and the two warps of a4 reach the first two quarters.  us
+// with 128 rows / 64, X in the L2: W16A16 rank 24, M x K = 1365 x 2312 8.6 / 7.5, 1 x 4608 12.0 / 10.4, 120 x 1152 5.1 / 4.7; W8A8 rank
+// 32 9.1 / 8.7, 11.1 / 10.3, 5.9 / 5.7; rank 128 12.1 / 11.8, 15.0 / 14.6, 8.0 / 7.8.
 __device__ __forceinline__ constexpr bool mma_64_rows(int br, int groups) { return (br == BR_INT || br == BR_F16) && groups <= 4; }
 
 template <int MAIN, int BR>
@@ -664,13 +666,14 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   // The tensor-memory columns are taken before a dependent kernel may start and want them.
   grid_launch_dependents();
 
-  // While the kernel before still runs, as much of this CTA's first tile as the X ring holds comes to the L2 (what that kernel writes of it, it writes there).  All CTAs of a
-  // launch ask for their X at once, so the first chunk was there after 1.3 to 2.1 us instead of 0.8; M = 8192, K = 1152 behind a GEMM, from the dependency wait to the
-  // end, us: SINT4 11.0 -> 9.8, MXINT4 10.2 -> 8.9, MXFP4 7.7 -> 6.5; two linears of 1365 rows 34.0 -> 32.3.  (By the X producer's warp, whose loads then queue behind it: 10.6 -> 11.9
-  // where X is in the L2 already.)
+  // While the kernel before still runs, as much of this CTA's first tile as the X ring holds comes to the L2 (what that kernel writes of
+  // it, it writes there).  All CTAs of a launch ask for their X at once, so the first chunk was there after 1.3 to 2.1 us instead of 0.8;
+  // M = 8192, K = 1152 behind a GEMM, from the dependency wait to the end, us: SINT4 11.0 -> 9.8, MXINT4 10.2 -> 8.9, MXFP4 7.7 -> 6.5;
+  // two linears of 1365 rows 34.0 -> 32.3.  (By the X producer's warp, whose loads then queue behind it: 10.6 -> 11.9 where X is in the L2 already.)
   auto fetch_ahead = [&]() {
     if (p.X != nullptr)
-      for (int m = blockIdx.x * TR + lane; m < min(p.M, ((int)blockIdx.x + 1) * TR); m += 32) bulk_prefetch(p.X + (size_t)m * (2 * p.K), (uint32_t)min(2 * p.K, p.xslots * spc * 256));
+      for (int m = blockIdx.x * TR + lane; m < min(p.M, ((int)blockIdx.x + 1) * TR); m += 32)
+        bulk_prefetch(p.X + (size_t)m * (2 * p.K), (uint32_t)min(2 * p.K, p.xslots * spc * 256));
   };
   const int qw = warp - FIRST_QWARP;
   if (warp == 3) {
@@ -781,9 +784,9 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   } else if (BR != BR_NONE && warp < 2) {
     // ------------------------------------------------------------------ a4: lane = row of the tile, straight from tensor memory
     // One warp's chain of instructions at the end of a launch, a microsecond or two long: 32 columns at a time, two values to an
-    // instruction, a rank of up to 32 read once.  (Sixteen at a time, one by one, the scaled sums worked out for the maximum and again for the codes: us,
-    // M = 1 / 8192, K = 1152, X in the L2, SINT4 rank 32 6.5 / 11.1 -> 5.9 / 10.7, MXFP8 rank 64 6.2 / 9.3 -> 5.5 / 8.5, MXFP4 rank 128 7.7 / 11.6 -> 6.6 / 10.3,
-    // MXINT8 rank 64 7.5 / 11.2 -> 6.9 / 10.5.)
+    // instruction, a rank of up to 32 read once.  (Sixteen at a time, one by one, the scaled sums worked out for the maximum and again
+    // for the codes: us, M = 1 / 8192, K = 1152, X in the L2, SINT4 rank 32 6.5 / 11.1 -> 5.9 / 10.7, MXFP8 rank 64 6.2 / 9.3 -> 5.5 /
+    // 8.5, MXFP4 rank 128 7.7 / 11.6 -> 6.6 / 10.3, MXINT8 rank 64 7.5 / 11.2 -> 6.9 / 10.5.)
     if (warp == 0) fetch_ahead();
     grid_dependency_wait();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0) + ((uint32_t)(32 * warp) << 16);
@@ -1177,8 +1180,8 @@ lq_quant_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   }
 }
 
-// The launch's cut.  Working it out takes the calling thread 0.5 to 1.5 us of a launch's 4 to 5, which back-to-back calls of a few rows wait for, so each thread
-// keeps the last ones by everything that they depend on (a call of one row, K = 1152: 4.3 -> 3.8 us).
+// The launch's cut.  Working it out takes the calling thread 0.5 to 1.5 us of a launch's 4 to 5, which back-to-back calls of a few rows
+// wait for, so each thread keeps the last ones by everything that they depend on (a call of one row, K = 1152: 4.3 -> 3.8 us).
 bool cut_of(int br, int M, int nst, int rn, int bplanes, int sms, QuantCut& out) {
   struct Kept { int key[8]; QuantCut cut; };
   static thread_local Kept kept[16];                             // (a key's M is not 0)
@@ -1209,7 +1212,7 @@ cudaError_t launch_quant(const void* X, const CUtensorMap& tm, QuantParams& p, i
   // From 1 MB of X on: less comes in one trip anyway.
   p.X = (size_t)p.M * p.K * 2 >= (1u << 20) ? static_cast<const uint8_t*>(X) : nullptr;
   // Floating-point branches: a tile's stages alternate over up to four accumulators, which are added in fp32 at the end
-  // (each costs a4 a trip to tensor memory per 16 columns: not more than 128 columns of them).  Tensor memory holds two
+  // (each costs a4 a trip to tensor memory per 32 columns: not more than 128 columns of them).  Tensor memory holds two
   // such sets - one where every CTA has a single tile - and the scale bytes' columns.
   const int cols = p.rn * p.bplanes, extra = BR == BR_MXFP || BR == BR_MXINT ? 16 : 0;
   p.sets = p.ntiles <= sms ? 1 : 2;
@@ -1238,7 +1241,8 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   p.qb = g_lq_store_qb ? A->d_qb : nullptr;
   p.sXb = A->d_sXb; p.sL1 = L->d_sL1; p.l1c = L->d_L1c; p.sfl1 = L->d_sfl1;
   p.sft = A->d_sft; p.tq = A->d_tq; p.sT = A->d_sT; 
-  p.near = reinterpret_cast<uint32_t*>(A->d_sT); p.near_which = reinterpret_cast<uint32_t*>(A->d_qb);   // (an MXFP row has neither a scale nor branch codes of its own)
+  // (an MXFP row has neither a scale nor branch codes of its own)
+  p.near = reinterpret_cast<uint32_t*>(A->d_sT); p.near_which = reinterpret_cast<uint32_t*>(A->d_qb);
   p.r = L->r; p.rn = lq_l1_rows(L);
   p.bplanes = lq_l1_planes(L);
   p.tq_stride = A->tq_stride;
@@ -1258,9 +1262,11 @@ lq_status lq_launch_quantize(const lq_layer* L, const void* X, int M, lq_act* A,
   else if (L->a8) e = L->r > 0 ? launch_quant<MAIN_MXINT8, BR_MXINT>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXINT8, BR_NONE>(X, L->tmL1, p, sms, st);
   else if (L->mx)
     e = L->f16_branch ? launch_quant<MAIN_MXINT4, BR_F16>(X, L->tmL1, p, sms, st)
-                      : L->integer_branch ? launch_quant<MAIN_MXINT4, BR_INT>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_MXINT4, BR_NONE>(X, L->tmL1, p, sms, st);
+                      : L->integer_branch ? launch_quant<MAIN_MXINT4, BR_INT>(X, L->tmL1, p, sms, st)
+                                          : launch_quant<MAIN_MXINT4, BR_NONE>(X, L->tmL1, p, sms, st);
   else
     e = L->f16_branch ? launch_quant<MAIN_SINT4, BR_F16>(X, L->tmL1, p, sms, st)
-                      : L->integer_branch ? launch_quant<MAIN_SINT4, BR_INT>(X, L->tmL1, p, sms, st) : launch_quant<MAIN_SINT4, BR_NONE>(X, L->tmL1, p, sms, st);
+                      : L->integer_branch ? launch_quant<MAIN_SINT4, BR_INT>(X, L->tmL1, p, sms, st)
+                                          : launch_quant<MAIN_SINT4, BR_NONE>(X, L->tmL1, p, sms, st);
   return lq_note_cuda(e) == cudaSuccess ? LQ_OK : LQ_ERR_CUDA;
 }

@@ -59,24 +59,27 @@ __host__ __device__ inline QuantSmem quant_smem(int br, int tr, int st, int rn, 
 }
 
 // Cost model in rounds, a round being one chunk for every team: a CTA's tiles times (its rounds,
-// twice where a tile is walked twice, plus three for starting and finishing a tile, or one without a branch: no factor, sums or re-quantization wait there,
-// and with three M = 22000, K = 1152 took 17.7 / 13.7 us, caches cold / warm, for 16.5 / 13.1).  It prices rounds only: not the second stream of X
-// where an integer branch's tile is larger than the ring (140 MB read for 75 at M = 8192, K = 4608), nor what overlaps between tiles.
-// Of cuts with the same rounds the one with the most warps and then the longer chunks (up to four stages) is taken, where a slot's
-// operands are small enough (integer branches, MXFP up to rank 64; the others lose up to 5 % by it) and K has the eight stages that fill
-// two such chunks (without that limit 44 more of the timed sizes are over 1.5 % slower than by short ones).  Exceptions.  An integer branch, whose ring the long chunks shrink: a ring of two chunks (from five row groups on; us,
-// M = 17600, rank 128, K = 1280 / 1664, chunks of 1 and of 3 stages: 27.6 and 31.2 / 33.4 and 37.6), and chunks of two
-// stages where K has an odd number of them (M = 32768, rank 32, K = 1408, chunks of 1 and of 2 stages: 41.1 and 42.7; above rank 48 and from
-// 1536 on, or from 24 stages on, they are the faster ones all the same).  Elsewhere they may even make a tile too large for the ring: M = 32768, K = 1536, rank 64,
-// X streamed once by chunks of 1 and twice by chunks of 2: 49.1 and 45.8.
-// MXFP: chunks of two of an odd number below twelve where a CTA has one tile, whose first chunk nothing covers (rank 64, M = 8192, K = 1152, caches cold: 11.16
-// by chunks of 1, 11.43 of 2).
-// Eight row groups leave room for one team of eight warps with nothing to run beside its waits: a tenth more a round (SINT4 rank 32, M = 17600, K = 640 / 896:
-// 16.2 / 19.0 us by 5 groups, 17.4 / 21.6 by 8).  With the widest factors, which every tile fetches anew, their fewer tiles make up for it (rank 128, K = 384: 18.5
-// and 15.8).
+// twice where a tile is walked twice, plus three for starting and finishing a tile, or one without a branch: no factor, sums or
+// re-quantization wait there, and with three M = 22000, K = 1152 took 17.7 / 13.7 us, caches cold / warm, for 16.5 / 13.1).  It prices
+// rounds only: not the second stream of X where an integer branch's tile is larger than the ring (140 MB read for 75 at M = 8192, K =
+// 4608), nor what overlaps between tiles.  Of cuts with the same rounds the one with the most warps and then the longer chunks (up to four
+// stages) is taken, where a slot's operands are small enough (integer branches, MXFP up to rank 64; the others lose up to 5 % by it) and
+// K has the eight stages that fill two such chunks (without that limit 44 more of the timed sizes are over 1.5 % slower than by short
+// ones).  Exceptions.  An integer branch, whose ring the long chunks shrink: a ring of two chunks (from five row groups on; us, M =
+// 17600, rank 128, K = 1280 / 1664, chunks of 1 and of 3 stages: 27.6 and 31.2 / 33.4 and 37.6), and chunks of two stages where K has an
+// odd number of them (M = 32768, rank 32, K = 1408, chunks of 1 and of 2 stages: 41.1 and 42.7; above rank 48 and from 1536 on, or from
+// 24 stages on, they are the faster ones all the same).  Elsewhere they may even make a tile too large for the ring: M = 32768, K = 1536,
+// rank 64, X streamed once by chunks of 1 and twice by chunks of 2: 49.1 and 45.8.
+// MXFP: chunks of two of an odd number below twelve where a CTA has one tile, whose first chunk nothing covers (rank 64, M = 8192, K = 1152,
+// caches cold: 11.16 by chunks of 1, 11.43 of 2).
+// Eight row groups leave room for one team of eight warps with nothing to run beside its waits: a tenth more a round (SINT4 rank 32, M =
+// 17600, K = 640 / 896: 16.2 / 19.0 us by 5 groups, 17.4 / 21.6 by 8).  With the widest factors, which every tile fetches anew, their
+// fewer tiles make up for it (rank 128, K = 384: 18.5 and 15.8).
 // Timed over the sensible cuts of 11616 sizes (22 formats and ranks, K from 256 to 8192, M from 1 to 32768, caches warm and cold): by one
-// round for every tile and none of these rules 3830 of them get another cut, which is 6.4 % slower in the mean; 84 get one that is more than 1.5 % faster, 9 % at
-// most (26 more than 4 %: factors of up to 32 columns at K above 5000, tiles of 16 or 24 rows instead of 40 or 48, and a few instead of seven or eight groups).
+// round for every tile and none of these rules 3830 of them get another cut, which is 6.4 % slower in the mean; 84 get one that is more
+// than 1.5 % faster, 9 % at most (26 more than 4 %: factors of up to 32 columns at K above 5000, tiles of 16 or 24 rows instead of 40 or
+// 48, and a few instead of seven or eight groups).  All these times are of the kernel before tiles of up to 32 rows had MMAs of 64 rows,
+// branch codes one FMA, and the re-quantization two values to an instruction.
 //
 // Barrier phases have one bit, so a team that waits for a slot must not be able to mistake the phase before last for the last
 // one: the chunk that was in the slot before has to be known to have landed (X) or to have been multiplied (operands).
@@ -144,9 +147,10 @@ inline bool plan_cut_as_asked(int br, int M, int nst, int rn, int bplanes, int s
 }
 
 // Whether X is the first to leave the L2 (126 MB), before the codes, which the GEMM comes for next.  The launch cannot know whether somebody reads X
-// again - another layer, a residual sum - so it is so only where X and the codes (bytes) are too large to stay all the same, and then it costs nobody anything; nor
-// where an integer branch streams X twice itself.  Timed with and without over X and codes of 36 to 240 MB, K from 640 to 4608, four formats: quantizer and GEMM alone,
-// two layers in turn on one X, both quantizers first, X just written, X read again behind the GEMM.  Rank 32 / 64, K = 1152, N = 1152:
+// again - another layer, a residual sum - so it is so only where X and the codes (bytes) are too large to stay all the same, and then it
+// costs nobody anything; nor where an integer branch streams X twice itself.  Timed with and without over X and codes of 36 to 240 MB, K
+// from 640 to 4608, four formats: quantizer and GEMM alone, two layers in turn on one X, both quantizers first, X just written, X read
+// again behind the GEMM.  Rank 32 / 64, K = 1152, N = 1152:
 //   X and codes   MXINT4: one layer, two, quantizers first, read again   MXFP4
 //     28 MB       0.972  1.010  1.019  1.014                             0.987  1.017  1.028  1.014   not taken (M = 8192)
 //     72 MB       0.986  0.986  0.984  0.988                             0.973  0.975  0.973  0.997   not taken (K = 4608: 0.981  0.997  1.005  0.996)
