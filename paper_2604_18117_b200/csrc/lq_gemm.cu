@@ -49,6 +49,7 @@
 #include <type_traits>
 
 #include "lq_device.cuh"
+#include "lq_gemm_cut.h"
 
 #ifdef LQ_TIMELINE
 // Timeline build only: copies the stamp lists of the last launch to the host ([TL_LISTS][TL_CAP] words) and clears them.
@@ -621,29 +622,7 @@ __global__ void lq_wait_probe_kernel(int32_t* status, long long limit) {
   mbar_wait_slow(bar, 0, &abort_word, status, LQ_STAGE_TEARDOWN, limit);
 }
 
-// CTAs per tile of a launch of few tiles (1, 2, 4 or 8).  A tile's stages are one serial chain, so while SMs are idle they may as well share
-// it; a cluster's launch and the exchange cost the rest (us, alone and shared: M = 1, K x N = 1152 x 1152: 7.0 and 4.8 by
-// eight; M = 120, 8192 x 1152: 30.8 and 9.8 by eight; M = 256, 4608 x 1152: 18.9 and 10.3 by four).  The hardware places a cluster's CTAs
-// next to each other, so fewer fit than there are SMs; a second round of them would cost more than it gives.  Prices, us: a stage 0.44, the
-// exchange 1.62, with full tiles 0.6 + 0.08 per CTA more.
-// A stage of a chain is charged 0.08 us beyond its time, because the sum's error grows with the chain: rows of ten stages are so
-// shared by two where alone would be as fast or faster (M = 120, 1152 x 4608: 7.57 by two, 7.50 alone; M = 256: 8.90 and 7.71), with a relative
-// error of 6.0e-8 instead of 7.4e-8 (M = 128, fp32 output).  Tiles of six stages are shared up to 60 rows (M = 1, 640 x 1152: 4.9 by four,
-// 5.3 alone).
-constexpr double STAGE_US = 0.44, CHAIN_US = 0.08;
 int g_clusters[64][3];                                // how many clusters of 2, 4, 8 the device holds at once
-int pick_split(int device, int M, long long units, int stages, int ctas) {
-  int best = 1;
-  double best_cost = (STAGE_US + CHAIN_US) * stages;
-  for (int i = 0, split = 2; i < 3; ++i, split *= 2) {
-    if (split > ctas || split > stages || units > std::min(g_clusters[device & 63][i], ctas / split)) break;
-    if (g_lq_gemm_split > 0 && split != g_lq_gemm_split) continue;
-    const double exchange = 1.62 + (0.6 + 0.08 * split) * std::min(M, LQ_BM) / LQ_BM;
-    const double cost = g_lq_gemm_split > 0 ? 0 : (STAGE_US + CHAIN_US) * lq_ceil_div(stages, split) + exchange;
-    if (cost < best_cost) { best_cost = cost; best = split; }
-  }
-  return best;
-}
 
 }  // namespace
 
@@ -701,7 +680,8 @@ lq_status lq_launch_gemm(const lq_layer* L, const lq_act* A, void* Y, lq_out_dty
   int ctas = g_lq_gemm_ctas > 0 ? g_lq_gemm_ctas : sms;
   const long long units = (long long)p.tiles_m * p.units_n;
   // (by the whole call's rows, so that a row's sums are the same in every chunk of it)
-  p.split = pick_split(A->device, A->M_call, (long long)lq_ceil_div(A->M_call, LQ_BM) * p.units_n, p.n_stages_main + (L->r > 0), ctas);
+  p.split = pick_split(A->M_call, (long long)lq_ceil_div(A->M_call, LQ_BM) * p.units_n, p.n_stages_main + (L->r > 0), ctas,
+                       g_clusters[A->device & 63], g_lq_gemm_split);
   ctas = (int)std::min<long long>(ctas, units * p.split);
   auto kernel = [&](auto tile) {
     constexpr int T = decltype(tile)::value;

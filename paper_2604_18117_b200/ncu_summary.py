@@ -25,7 +25,7 @@ from collections import OrderedDict
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2604_18117_b200", "csrc")
 # source files a GEMM kernel is compiled from: a record made for other sources is stale
-KERNEL_SOURCES = {"lq_gemm_kernel": ("lq_gemm.cu", "lq_device.cuh"), "lq_gemm_mx_kernel": ("lq_gemm_mx.cu", "lq_gemm_mx_cut.h", "lq_device.cuh")}
+KERNEL_SOURCES = {"lq_gemm_kernel": ("lq_gemm.cu", "lq_gemm_cut.h", "lq_device.cuh"), "lq_gemm_mx_kernel": ("lq_gemm_mx.cu", "lq_gemm_mx_cut.h", "lq_device.cuh")}
 
 
 def sources_sha256(kernel: str) -> str:
