@@ -216,8 +216,10 @@ lq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto bar_full = [&](int s) { return sm_bar + 8u * (uint32_t)s; };                        // operands + scales landed
   auto bar_empty = [&](int s) { return sm_bar + 8u * (uint32_t)(NSTAGE + s); };           // MMAs of the stage retired
   auto bar_tfull = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + b); };
-  // (16 bytes apart: 8 bytes apart, as they would fit, the same code was 1.5 to 2.5 % slower; what in it is not known)
-  auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + NPAIR + 1 + 2 * b); };
+  // (With a branch 16 bytes apart: 8 bytes apart, as they fit, the same code is 1.5 to 2.5 % slower, without one 2 to 4 % faster; what in it is
+  // not known.  No branch, us 16 / 8 bytes apart: M = 8192, K x N = 1152 x 3456 / 4608 x 1152 59.0 / 56.8, 69.1 / 66.1, M = 23821, 712 x 6328 251 / 246.)
+  constexpr int EMPTY_AT = BRANCH == BRANCH_NONE ? 0 : 1, EMPTY_STRIDE = BRANCH == BRANCH_NONE ? 1 : 2;
+  auto bar_tempty = [&](int b) { return sm_bar + 8u * (uint32_t)(2 * NSTAGE + NPAIR + EMPTY_AT + EMPTY_STRIDE * b); };
   [[maybe_unused]] const uint32_t bar_gather = sm_bar + 8u * (uint32_t)(2 * NSTAGE + 3 * NPAIR);
   constexpr int NBAR = 2 * NSTAGE + 3 * NPAIR + 1;
   static_assert(NBAR * 8 + 16 <= SMEM_BAR_BYTES, "barrier area too small");
